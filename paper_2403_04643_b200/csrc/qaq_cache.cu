@@ -42,10 +42,11 @@ extern "C" qaq_status qaq_cache_create(const qaq_config* cfg, qaq_cache** out) {
     c->tmax_pad = (int)align_up((size_t)cfg->max_tokens, QAQ_TILE);
     c->ntiles = c->tmax_pad / QAQ_TILE;
     const int D = cfg->head_dim;
-    // worst case per tile: every token at 8 bits or the largest padding of the value groups, plus alignment
-    // padding per tile and a read-ahead margin
-    c->pool_bytes = align_up((size_t)c->ntiles * (size_t)qaqc::v_tile_bytes_max(D) + 16 * (size_t)c->ntiles + 256, 256);
-    if (c->pool_bytes >= ((size_t)1 << 32)) { free(c); return QAQ_ERR_UNSUPPORTED_SHAPE; }
+    // worst case per tile: every token at 8 bits; per tile some room beside that (six tokens' worth) for tiles that
+    // are raised and move, alignment padding, and a read-ahead margin
+    c->pool_bytes = align_up((size_t)c->ntiles * ((size_t)qaqc::tile_bytes_max(D) + 6 * D + 32) + 256, 256);
+    if (c->pool_bytes >= ((size_t)1 << 32) - ((size_t)1 << 26))   // offsets are 32 bits; takers that find no room run past the end for a while
+        { free(c); return QAQ_ERR_UNSUPPORTED_SHAPE; }
     long ocap = cfg->max_outliers_per_bh;
     if (ocap <= 0) {
         double want = 2.0 * cfg->outlier_frac * (double)c->tmax_pad * D + 1024.0;
@@ -58,7 +59,7 @@ extern "C" qaq_status qaq_cache_create(const qaq_config* cfg, qaq_cache** out) {
     const size_t BH = (size_t)c->BH;
     size_t off = 0;
     auto carve = [&](size_t bytes) { size_t o = off; off = align_up(off + bytes, 256); return o; };
-    size_t o_codes[2], o_bits[2], o_mnmx[2], o_toff[2], o_tnb[2], o_tooff[2], o_tocnt[2], o_outl[2], o_pe[2], o_ope[2];
+    size_t o_codes[2], o_bits[2], o_mnmx[2], o_tile[2], o_outl[2], o_pe[2], o_ope[2];
     // three regions: pools that need no initialisation; tables that start at zero; what qaq_cache_reset clears
     // (one contiguous range, one memset)
     for (int x = 0; x < 2; ++x) {
@@ -67,13 +68,10 @@ extern "C" qaq_status qaq_cache_create(const qaq_config* cfg, qaq_cache** out) {
     }
     for (int x = 0; x < 2; ++x) {
         o_mnmx[x] = carve(BH * c->tmax_pad * 4);
-        o_toff[x] = carve(BH * c->ntiles * 4);
-        o_tooff[x] = carve(BH * c->ntiles * 4);
     }
     for (int x = 0; x < 2; ++x) {
-        o_bits[x] = carve(BH * c->tmax_pad);
-        o_tnb[x] = carve(BH * c->ntiles * 4);
-        o_tocnt[x] = carve(BH * c->ntiles * 4);
+        o_bits[x] = carve(BH * c->tmax_pad * 2);
+        o_tile[x] = carve(BH * c->ntiles * 16);
         o_pe[x] = carve(BH * 4);
         o_ope[x] = carve(BH * 4);
     }
@@ -84,12 +82,9 @@ extern "C" qaq_status qaq_cache_create(const qaq_config* cfg, qaq_cache** out) {
     for (int x = 0; x < 2; ++x) {
         TensorStore& t = c->t[x];
         t.codes = (uint8_t*)(base + o_codes[x]);
-        t.bits = (uint8_t*)(base + o_bits[x]);
+        t.bs = (unsigned short*)(base + o_bits[x]);
         t.mnmx = (uint32_t*)(base + o_mnmx[x]);
-        t.tile_off = (uint32_t*)(base + o_toff[x]);
-        t.tile_nbytes = (uint32_t*)(base + o_tnb[x]);
-        t.tile_ooff = (uint32_t*)(base + o_tooff[x]);
-        t.tile_ocnt = (uint32_t*)(base + o_tocnt[x]);
+        t.tile = (uint4*)(base + o_tile[x]);
         t.outl = (uint32_t*)(base + o_outl[x]);
         t.pool_end = (uint32_t*)(base + o_pe[x]);
         t.opool_end = (uint32_t*)(base + o_ope[x]);
@@ -174,7 +169,7 @@ struct StatsDev {
     unsigned long long hist[2][9];
     unsigned long long code_bytes[2];
     unsigned long long outliers[2];
-    unsigned long long stored_bytes[2];   // bytes the tiles occupy (values: with the padding of their groups)
+    unsigned long long stored_bytes[2];   // bytes the tiles occupy (values: at the widths of their groups)
 };
 
 __global__ void stats_kernel(TensorStore tk, TensorStore tv, int T, int tmax_pad, int ntiles, int D, StatsDev* out) {
@@ -187,13 +182,13 @@ __global__ void stats_kernel(TensorStore tk, TensorStore tv, int T, int tmax_pad
     for (int x = 0; x < 2; ++x) {
         const TensorStore& ts = x ? tv : tk;
         for (int t = threadIdx.x; t < T; t += blockDim.x) {
-            int b = ts.bits[(size_t)bh * tmax_pad + t];
+            int b = ts.bs[(size_t)bh * tmax_pad + t] & 0xFF;
             atomicAdd(&sh[x][b > 8 ? 8 : b], 1ULL);
         }
         int nt = (T + QAQ_TILE - 1) / QAQ_TILE;
         for (int i = threadIdx.x; i < nt; i += blockDim.x) {
-            atomicAdd(&so[x], (unsigned long long)ts.tile_ocnt[(size_t)bh * ntiles + i]);
-            atomicAdd(&sb[x], (unsigned long long)ts.tile_nbytes[(size_t)bh * ntiles + i]);
+            atomicAdd(&so[x], (unsigned long long)ts.tile[(size_t)bh * ntiles + i].w);
+            atomicAdd(&sb[x], (unsigned long long)ts.tile[(size_t)bh * ntiles + i].y);
         }
     }
     __syncthreads();
@@ -242,7 +237,7 @@ extern "C" qaq_status qaq_cache_stats(const qaq_cache* cc, qaq_stats* host_out, 
         host_out->outliers[x] = (long)h.outliers[x];
         for (int b = 0; b < 9; ++b) host_out->hist[x][b] = (long)h.hist[x][b];
         bits_total += 8.0 * (double)h.code_bytes[x] + 16.0 * (double)h.outliers[x];
-        resident += (long)h.stored_bytes[x] + 4 * (long)h.outliers[x] + BH * T * 5 + BH * nt * 16;
+        resident += (long)h.stored_bytes[x] + 4 * (long)h.outliers[x] + BH * T * 6 + BH * nt * 16;
     }
     host_out->resident_bytes = resident;
     double orig_bits = 16.0 * 2.0 * (double)BH * (double)T * (double)D;
@@ -260,14 +255,14 @@ __global__ void export_count_kernel(TensorStore ts, int T, int tmax_pad, int D, 
     const int t = tile * QAQ_TILE + threadIdx.x;
     const size_t rowbase = (size_t)bh * (T + 1);
     if (threadIdx.x < QAQ_TILE && t < T) {
-        if (off) off[rowbase + t + 1] = (uint32_t)D * ts.bits[(size_t)bh * tmax_pad + t] / 8;
+        if (off) off[rowbase + t + 1] = (uint32_t)D * (ts.bs[(size_t)bh * tmax_pad + t] & 0xFF) / 8;
     }
 }
 
 __global__ void export_ocount_kernel(TensorStore ts, int T, int ntiles, uint32_t ocap, uint32_t* rowptr) {
     const int bh = blockIdx.y, tile = blockIdx.x;
-    const uint32_t n = ts.tile_ocnt[(size_t)bh * ntiles + tile];
-    const uint32_t o0 = ts.tile_ooff[(size_t)bh * ntiles + tile];
+    const uint32_t n = ts.tile[(size_t)bh * ntiles + tile].w;
+    const uint32_t o0 = ts.tile[(size_t)bh * ntiles + tile].z;
     const uint32_t* e = ts.outl + (size_t)bh * ocap + o0;
     for (uint32_t i = threadIdx.x; i < n; i += blockDim.x) {
         int t = tile * QAQ_TILE + (int)(e[i] >> 24);
@@ -300,21 +295,41 @@ __global__ void export_scan_kernel(uint32_t* a, int T) {
     }
 }
 
+// the code of channel d of the token in `slot`, from the tile as it is stored (w: width of the token's row)
+__device__ uint32_t code_at(const uint8_t* tile, const qaqc::Section& s, int is_v, int D, int slot, int w, int d) {
+    const int p = d >> 5, u = (d >> 3) & 3, cls = (d >> 2) & 1, b = d & 3;
+    uint32_t code = 0;
+    for (int part = 0; part < 2; ++part) {
+        const int pw = part ? w - 4 : (w < 4 ? w : 4);
+        if (pw < 1) continue;
+        const uint8_t* src = tile + (part ? s.high : s.main);
+        const int first = part ? s.start : s.mstart, n = part ? s.n : s.mn;
+        // byte c of the words the channel is in
+        const uint8_t* x = is_v ? src + qaqc::v_unit(D, n, (slot >> 2) - first, 4 * p + b) * 4 * pw + (slot & 3)
+                                : src + (uint32_t)((slot - first) * (D / 32) + p) * 4 * pw + b;
+        uint32_t v = 0;
+        if (pw == 4) v = (x[4 * u] >> (4 * cls)) & 15u;
+        else if (pw == 3) {
+            if (u < 3) v = (x[4 * u] >> (4 * cls)) & 7u;
+            else for (int i = 0; i < 3; ++i) v |= (((uint32_t)x[4 * i] >> (4 * cls + 3)) & 1u) << i;
+        } else if (pw == 2) v = (x[4 * (u >> 1)] >> (4 * cls + 2 * (u & 1))) & 3u;
+        else v = (x[0] >> (4 * cls + u)) & 1u;
+        code |= v << (4 * part);
+    }
+    return code;
+}
 // one canonical byte of a token: byte y of its string (the planes of its pieces, widest first; inside the plane of
-// a w-bit piece channel d = 32p + 4j + i sits in word p*w + j*w/8 at bit 8i + w*(j mod 8/w)), put together from the
-// pieces as the tile stores them
-template <bool IS_V>
-__device__ uint32_t canonical_byte(const uint8_t* tile, const qaqc::TileMasks& tm, const uint32_t (&base)[5], int D, int slot,
-                                   int B, uint32_t y) {
+// a piece of `w` bits channel d = 32p + 4j + i sits in word p*w + j*w/8 at bit 8i + w*(j mod 8/w))
+__device__ uint32_t canonical_byte(const uint8_t* tile, const qaqc::Section& s, int is_v, int D, int slot, int row_w, int B, uint32_t y) {
     for (int c = 0; c < 4; ++c) {
         const int w = 8 >> c;
         if (!(B & w)) continue;
         const uint32_t plen = (uint32_t)D * w / 8;
         if (y >= plen) { y -= plen; continue; }
         const int per = 8 / w, cw = y >> 2, i = y & 3, p = cw / w, rr = cw % w;
-        const int r = qaqc::rank_in(tm, c, slot);
         uint32_t v = 0;
-        for (int mm = 0; mm < per; ++mm) v |= qaqc::piece_at<IS_V>(tile, base, D, c, r, 32 * p + 4 * (rr * per + mm) + i) << (w * mm);
+        for (int mm = 0; mm < per; ++mm)
+            v |= ((code_at(tile, s, is_v, D, slot, row_w, 32 * p + 4 * (rr * per + mm) + i) >> (B & (w - 1))) & ((1u << w) - 1u)) << (w * mm);
         return v;
     }
     return 0;
@@ -325,18 +340,27 @@ __global__ void export_gather_kernel(TensorStore ts, int is_v, int T, int tmax_p
                                      long codes_stride, const uint32_t* rowptr, uint8_t* ch, __half* val, long outl_stride) {
     const int bh = blockIdx.y, tile = blockIdx.x;
     __shared__ uint32_t s_in[QAQ_TILE + 1];
-    __shared__ uint8_t s_b[QAQ_TILE];
-    __shared__ unsigned int s_m[4][2];
+    __shared__ uint8_t s_b[QAQ_TILE], s_slot[QAQ_TILE], s_row[QAQ_TILE];
+    __shared__ qaqc::Section s_tab[9];
     const int t0 = tile * QAQ_TILE;
     if (threadIdx.x < QAQ_TILE) {
         const int t = t0 + threadIdx.x;
-        int B = t < T ? ts.bits[(size_t)bh * tmax_pad + t] : 0;
-        B = B > 8 ? 8 : B;
-        s_b[threadIdx.x] = (uint8_t)B;
-        for (int c = 0; c < 4; ++c) {
-            const unsigned int bal = __ballot_sync(0xFFFFFFFFu, (B & (8 >> c)) != 0);
-            if ((threadIdx.x & 31) == 0) s_m[c][threadIdx.x >> 5] = bal;
-        }
+        const unsigned bs = t < T ? ts.bs[(size_t)bh * tmax_pad + t] : 0u;
+        s_b[threadIdx.x] = (uint8_t)min(bs & 0xFFu, 8u);
+        s_slot[threadIdx.x] = (uint8_t)((bs >> 8) & (QAQ_TILE - 1));
+    }
+    const uint8_t* src = ts.codes + (size_t)bh * pool_bytes + ts.tile[(size_t)bh * ntiles + tile].x;
+    if (threadIdx.x == 0) {
+        int n[9];
+        const uint32_t* h = reinterpret_cast<const uint32_t*>(src);
+        const bool there = ts.tile[(size_t)bh * ntiles + tile].y != 0;
+        qaqc::counts_of(there ? h[0] : 0u, there ? h[1] : 0u, n);
+        const int units = is_v ? D / 8 : D / 32;
+        if (units == 1) qaqc::make_sections<1>(n, s_tab, nullptr);
+        else if (units == 2) qaqc::make_sections<2>(n, s_tab, nullptr);
+        else if (units == 4) qaqc::make_sections<4>(n, s_tab, nullptr);
+        else if (units == 8) qaqc::make_sections<8>(n, s_tab, nullptr);
+        else qaqc::make_sections<16>(n, s_tab, nullptr);
     }
     __syncthreads();
     if (threadIdx.x == 0) {
@@ -346,6 +370,14 @@ __global__ void export_gather_kernel(TensorStore ts, int is_v, int T, int tmax_p
             acc += (uint32_t)D * s_b[k] / 8;
         }
         s_in[QAQ_TILE] = acc;
+    }
+    if (threadIdx.x < QAQ_TILE) {      // width of the row a token is in
+        int w = s_b[threadIdx.x];
+        if (is_v && w) {
+            const int row = s_slot[threadIdx.x] >> 2;
+            for (int k = 8; k >= 1; --k) if (row >= s_tab[k].start && row < s_tab[k].start + s_tab[k].n) w = k;
+        }
+        s_row[threadIdx.x] = (uint8_t)w;
     }
     __syncthreads();
     if (threadIdx.x < QAQ_TILE && t0 + (int)threadIdx.x < T) {
@@ -359,33 +391,17 @@ __global__ void export_gather_kernel(TensorStore ts, int is_v, int T, int tmax_p
         if (step) step[(size_t)bh * T + t] = qaqc::step_of(fmn, fmx, B);
     }
     if (codes && off) {
-        const uint8_t* src = ts.codes + (size_t)bh * pool_bytes + ts.tile_off[(size_t)bh * ntiles + tile];
         uint8_t* dst = codes + (size_t)bh * codes_stride + off[(size_t)bh * (T + 1) + t0];
-        qaqc::TileMasks tm;
-        for (int c = 0; c < 4; ++c) tm.m[c] = (unsigned long long)s_m[c][0] | ((unsigned long long)s_m[c][1] << 32);
-        int n[4];
-        for (int c = 0; c < 4; ++c) n[c] = __popcll(tm.m[c]);
-        uint32_t base[5];
-        {   // section offsets for any head_dim (the templates of the codec header fix it at compile time)
-            uint32_t o = qaqc::QAQ_TILE_HDR;
-            for (int c = 0; c < 4; ++c) {
-                const int w = 8 >> c;
-                base[c] = o;
-                o += is_v ? (uint32_t)((n[c] + 3) >> 2) * (uint32_t)(D * w / 2) : (uint32_t)n[c] * (uint32_t)(D * w / 8);
-            }
-            base[4] = o;
-        }
         for (int k0 = 0; k0 < QAQ_TILE; k0 += 4) {
             const int k = k0 + (threadIdx.x >> 6);
             const uint32_t len = s_in[k + 1] - s_in[k];
             for (uint32_t y = threadIdx.x & 63; y < len; y += 64)
-                dst[s_in[k] + y] = (uint8_t)(is_v ? canonical_byte<true>(src, tm, base, D, k, s_b[k], y)
-                                                  : canonical_byte<false>(src, tm, base, D, k, s_b[k], y));
+                dst[s_in[k] + y] = (uint8_t)canonical_byte(src, s_tab[s_row[k]], is_v, D, s_slot[k], s_row[k], s_b[k], y);
         }
     }
     if (rowptr && (ch || val)) {
-        const uint32_t n = ts.tile_ocnt[(size_t)bh * ntiles + tile];
-        const uint32_t* e = ts.outl + (size_t)bh * ocap + ts.tile_ooff[(size_t)bh * ntiles + tile];
+        const uint32_t n = ts.tile[(size_t)bh * ntiles + tile].w;
+        const uint32_t* e = ts.outl + (size_t)bh * ocap + ts.tile[(size_t)bh * ntiles + tile].z;
         const uint32_t dst0 = rowptr[(size_t)bh * (T + 1) + t0];
         for (uint32_t i = threadIdx.x; i < n; i += blockDim.x) {
             uint32_t v = e[i];

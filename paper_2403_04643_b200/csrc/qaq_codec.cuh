@@ -5,29 +5,31 @@
 // segments): step = (max-min) * 2^-B, code = min(2^B-1, floor((x-min) * (1/step))) in binary32 with separately
 // rounded operations; an outlier's code slot holds 0.
 //
-// Pieces.  A B-bit code is cut into the power-of-two pieces of B's binary representation, widest first, the
-// widest holding the most significant bits (7 = 4+2+1): the piece of width w (w in {8,4,2,1}, present iff B & w)
-// is (code >> (B & (w-1))) & (2^w - 1).
-//
-// Tile layout in the code pool.  A tile (QAQ_TILE consecutive tokens of one (b,h) and tensor) is stored as four
-// sections, one per piece width, in the order 8, 4, 2, 1.  Section w holds the w-bit pieces of the tokens that
-// have one, in token order; the position of a token among them is its rank r_w.
-//   keys:    item r of section w is the plane of that token: head_dim*w/8 bytes; channel d = 32p + 4j + i sits in
-//            little-endian word p*w + j*w/8 of the plane at bit 8i + w*(j mod 8/w)  (after one shift and a
-//            byte-replicated mask a word has one field per byte lane: the operand of dp4a against four channels
-//            of the query).
-//   values:  items are stored in groups of four (the last group of a section is padded with zero bytes):
-//            group G = items 4G..4G+3, head_dim*w/2 bytes, made of 32-bit words whose byte lane i belongs to item
-//            4G+i and whose bit field m (bits w*m .. w*m+w-1 of every byte) is one channel, so that a masked word is
-//            four tokens of one channel, one per byte: the A operand of the integer tensor-core instruction
-//            mma.m16n8k32 with rows = channels and k = tokens.  Channel c sits in word c / (8/w), field
-//            c % (8/w): seen per token, a group interleaves byte by byte the four tokens' rows of packed fields
-//            (consecutive channels, lowest bits first).  The MMA lane with group id g takes the head_dim/8
-//            channels from g*head_dim/8 on as its rows, one vector load per group.
-// The sections are preceded by a header of QAQ_TILE_HDR bytes: the four 64-bit masks "slot t has a piece of width
-// 8, 4, 2, 1" (widths, ranks and section sizes of a tile can be read off them without the per-token metadata).
-// A tile therefore takes the header plus sum_t head_dim*B_t/8 bytes for keys, and that plus the group padding for
-// values.
+// Tile layout in the code pool.  A tile (QAQ_TILE consecutive tokens of one (b,h) and tensor) holds its tokens sorted by
+// width, widest first (ties in token order); the position of a token in that order is its slot, kept with its width in
+// the token's metadata.  Everything of one width is one section, and a section is a list of rows:
+//   keys:    a row is one token.
+//   values:  a row is a group of four consecutive slots, at the width of the widest of them (empty slots are zero).
+// All sections of a tile are cut into the same units, which are what a lane of the decode kernels loads at a time: the
+// registers it hands to the integer tensor-core instruction are one or two instructions away from the loaded words.
+// Nibble words: 32 codes of up to 4 bits are four words v0..v3, eight codes a word, code A(b) of byte b in its low and
+// B(b) in its high nibble, so that (v & mask) and (v & mask << 4) are operand registers (four codes, one per byte).
+// A unit stores them in as many words x as the codes have bits:
+//   4 bits: x_u = v_u     2 bits: x0 = v0 | v1 << 2, x1 = v2 | v3 << 2     1 bit: x0 = v0 | v1 << 1 | v2 << 2 | v3 << 3
+//   3 bits: x_u = v_u (u < 3) plus one bit of every nibble of v3 in the free bit of theirs: bit i of a nibble of v3 is
+//           bit 3 of the same nibble of x_i
+// and codes of 5..8 bits are two units, the low 4 bits (the main part) and the rest (the high part).  The main parts of
+// all rows of 4 bits and more are one list, so the main part of a tile is at most four lists and its high part four more.
+//   keys:    unit p of a row (p < head_dim/32) = the token's channels 32p .. 32p+31; in v_u, byte b is A = channel
+//            32p + 8u + b and B = channel 32p + 8u + 4 + b.
+//   values:  unit 4p + b of a row = byte b of those words for its four tokens: byte i of v_u belongs to slot 4G + i, A and
+//            B as above.  Rows of a list are interleaved by fours (the last m rows of a list by m): unit e of row
+//            4k + t lies at index 16k * head_dim/32 + e * m + t, which makes the loads of a warp contiguous.
+// Storage: a header of QAQ_TILE_HDR bytes (number of rows of every width, byte offsets of the zones below, total), then
+// the parts of the sections ordered by unit size so that every load is aligned: zone 4 (main parts of widths 8 .. 4,
+// 16-byte units; then the high part of width 8), zone 2 (high part of width 6, then width 2; 8-byte units), zone 13 (high
+// part of width 7, width 3, high part of width 5, width 1; 12- and 4-byte units).  A tile of keys takes the header plus
+// sum_t head_dim*B_t/8 bytes; a tile of values that plus what the widest tokens of mixed groups cost the others.
 #pragma once
 #include <cuda_fp16.h>
 #include <stdint.h>
@@ -102,67 +104,16 @@ __device__ __forceinline__ void mask_outliers32(uint32_t (&v)[16], __half2 lo2, 
     }
 }
 
-// ------------------------------------------------------------------------------------------ tile layout
-constexpr int QAQ_TILE_HDR = 32;
-
-// Which slots of a tile have a piece of width 8 >> c (c = 0..3): one 64-bit mask per width.
-struct TileMasks {
-    unsigned long long m[4];
-};
-
-// largest tile: the header, 64 tokens at 8 bits plus the worst padding of the value groups (three items in each of the four
-// sections), rounded up to a multiple of 16 so that images of tiles can sit back to back in shared memory
-__host__ __device__ constexpr int v_tile_bytes_max(int D) {
-    return (QAQ_TILE_HDR + QAQ_TILE_TOKENS * D + 3 * (D * 15 / 8) + 15) / 16 * 16;
-}
-
-// Byte offsets of the four sections inside a tile (base[4] = bytes of the tile).
-template <int D, bool IS_V>
-__device__ __forceinline__ void section_bases(const int (&n)[4], uint32_t (&base)[5]) {
-    uint32_t o = QAQ_TILE_HDR;
-#pragma unroll
-    for (int c = 0; c < 4; ++c) {
-        const int w = 8 >> c;
-        base[c] = o;
-        o += IS_V ? (uint32_t)((n[c] + 3) >> 2) * (uint32_t)(D * w / 2) : (uint32_t)n[c] * (uint32_t)(D * w / 8);
-    }
-    base[4] = o;
-}
-template <int D, bool IS_V>
-__device__ __forceinline__ void section_bases(const TileMasks& tm, uint32_t (&base)[5]) {
-    int n[4];
-#pragma unroll
-    for (int c = 0; c < 4; ++c) n[c] = __popcll(tm.m[c]);
-    section_bases<D, IS_V>(n, base);
-}
-// the header of a tile image (16-byte aligned, shared or global memory)
-__device__ __forceinline__ void write_header(uint8_t* img, const TileMasks& tm, int c) {
-    reinterpret_cast<unsigned long long*>(img)[c] = tm.m[c];
-}
-__device__ __forceinline__ int rank_in(const TileMasks& tm, int c, int slot) {
-    return __popcll(tm.m[c] & ((1ull << slot) - 1ull));
-}
-// The ranks of one slot in the four sections, either taken from the masks when asked for or handed over packed
-// (rank in section c in byte c; a tile has at most 64 items per section).
-struct MaskRanks {
-    const TileMasks& tm;
-    int slot;
-    __device__ __forceinline__ int operator()(int c) const { return rank_in(tm, c, slot); }
-};
-struct PackedRanks {
-    uint32_t rk;
-    __device__ __forceinline__ int operator()(int c) const { return (int)((rk >> (8 * c)) & 0xFFu); }
-};
-
 template <int NW>
-__device__ __forceinline__ void store_words(uint8_t* p, const uint32_t* w) {   // p is min(16, 4*NW)-byte aligned
+__device__ __forceinline__ void store_words(uint8_t* p, const uint32_t* w) {   // aligned to the widest access it takes: 16 bytes for multiples of four words, 8 for two, else 4
     if (NW % 4 == 0) {
 #pragma unroll
         for (int i = 0; i < NW; i += 4) *reinterpret_cast<uint4*>(p + 4 * i) = make_uint4(w[i], w[i + 1], w[i + 2], w[i + 3]);
     } else if (NW == 2) {
         *reinterpret_cast<uint2*>(p) = make_uint2(w[0], w[1]);
     } else {
-        *reinterpret_cast<uint32_t*>(p) = w[0];
+#pragma unroll
+        for (int i = 0; i < NW; ++i) reinterpret_cast<uint32_t*>(p)[i] = w[i];
     }
 }
 template <int NW>
@@ -177,251 +128,219 @@ __device__ __forceinline__ void load_words(const uint8_t* p, uint32_t* w) {
         const uint2 v = *reinterpret_cast<const uint2*>(p);
         w[0] = v.x; w[1] = v.y;
     } else {
-        w[0] = *reinterpret_cast<const uint32_t*>(p);
+#pragma unroll
+        for (int i = 0; i < NW; ++i) w[i] = reinterpret_cast<const uint32_t*>(p)[i];
     }
 }
 
-// The pieces of one thread's 32 channels (block p of the token in `slot`, codes one per byte in creg) written
-// into a tile image (shared or global memory, 16-byte aligned).
-template <int D, bool IS_V, typename Ranks>
-__device__ __forceinline__ void write_pieces(uint8_t* img, const Ranks& rk, const uint32_t (&base)[5], int B, int p,
-                                             const uint32_t (&creg)[8]) {
-    if (!IS_V) {
-        if (B & 8) store_words<8>(img + base[0] + rk(0) * D + p * 32, creg);
-        if (B & 4) {
-            const int sh = B & 3;
-            uint32_t w[4];
+// ------------------------------------------------------------------------------------------ tile layout
+constexpr int QAQ_TILE_HDR = 16;
+
+// largest tile: the header and 64 tokens at 8 bits
+__host__ __device__ constexpr int tile_bytes_max(int D) { return QAQ_TILE_HDR + QAQ_TILE_TOKENS * D; }
+// units per row: keys head_dim/32, values four times that
+template <int D, bool IS_V> constexpr int UNITS = IS_V ? D / 8 : D / 32;
+
+// Where the section of one width lies (byte offsets inside the tile) and which rows of the tile it holds.
+struct alignas(8) Section {
+    uint16_t main, high;     // first byte of the main and of the high part
+    uint8_t start, n;        // first row (in sorted order) and number of rows
+    uint8_t mstart, mn;      // the same for the list of rows the main part is in: all rows of 4 bits and more share one
+};
+
+// Sections of a tile with n[w] rows of width w (U units each): tab[1..8] and, if head is given, the header's four words.
+// Returns the bytes of the tile.
+template <int U>
+__device__ __forceinline__ uint32_t make_sections(const int (&n)[9], Section* tab, uint32_t* head) {
+    const int s7 = n[8], s6 = s7 + n[7], s5 = s6 + n[6], s4 = s5 + n[5], s3 = s4 + n[4], s2 = s3 + n[3], s1 = s2 + n[2];
+    const int h8 = QAQ_TILE_HDR + s3 * U * 16, z2 = h8 + n[8] * U * 16, m2 = z2 + n[6] * U * 8, z13 = m2 + n[2] * U * 8;
+    const int m3 = z13 + n[7] * U * 12, h5 = m3 + n[3] * U * 12, m1 = h5 + n[5] * U * 4, total = m1 + n[1] * U * 4;
+    auto put = [&](int w, int main, int high, int start) {
+        Section s;
+        s.main = (uint16_t)main; s.high = (uint16_t)high; s.start = (uint8_t)start; s.n = (uint8_t)n[w];
+        s.mstart = (uint8_t)(w >= 4 ? 0 : start); s.mn = (uint8_t)(w >= 4 ? s3 : n[w]);
+        tab[w] = s;
+    };
+    put(8, QAQ_TILE_HDR, h8, 0);
+    put(7, QAQ_TILE_HDR, z13, s7);
+    put(6, QAQ_TILE_HDR, z2, s6);
+    put(5, QAQ_TILE_HDR, h5, s5);
+    put(4, QAQ_TILE_HDR, 0, s4);
+    put(3, m3, 0, s3);
+    put(2, m2, 0, s2);
+    put(1, m1, 0, s1);
+    if (head) {
+        head[0] = (uint32_t)(n[1] | (n[2] << 8) | (n[3] << 16) | (n[4] << 24));
+        head[1] = (uint32_t)(n[5] | (n[6] << 8) | (n[7] << 16) | (n[8] << 24));
+        head[2] = (uint32_t)(h8 | (z2 << 16));
+        head[3] = (uint32_t)(z13 | (total << 16));
+    }
+    return (uint32_t)total;
+}
+// the counts of a stored header
+__device__ __forceinline__ void counts_of(uint32_t lo, uint32_t hi, int (&n)[9]) {
+    n[0] = 0;
 #pragma unroll
-            for (int j = 0; j < 4; ++j)     // the odd register goes straight to the high nibbles: one shift by 4 - sh
-                w[j] = ((creg[2 * j] >> sh) & 0x0F0F0F0Fu) | ((creg[2 * j + 1] << (4 - sh)) & 0xF0F0F0F0u);
-            store_words<4>(img + base[1] + rk(1) * (D / 2) + p * 16, w);
-        }
-        if (B & 2) {
-            const int sh = B & 1;
-            uint32_t w[2];
+    for (int w = 1; w <= 4; ++w) { n[w] = (lo >> (8 * w - 8)) & 0xFF; n[w + 4] = (hi >> (8 * w - 8)) & 0xFF; }
+}
+
+// What one warp finds out about a tile from the widths of its 64 slots (lane: slots lane and lane + 32; 0 = empty):
+// the slots' places in the sorted order, the width of the row each one belongs to (values: of its group), the number of
+// rows of every width.  sorted: 64 bytes of shared memory.
+struct Sorted { int slot[2], row_w[2]; };
+template <bool IS_V>
+__device__ __forceinline__ Sorted sort_tile(int lane, int b0, int b1, int (&n)[9], uint8_t* sorted) {
+    const unsigned lt = (1u << lane) - 1u;
+    Sorted r;
+    r.slot[0] = r.slot[1] = 0;
+    int start = 0;
+    n[0] = 0;
 #pragma unroll
-            for (int j = 0; j < 2; ++j) {
-                uint32_t acc = (creg[4 * j] >> sh) & 0x03030303u;
+    for (int w = 8; w >= 1; --w) {
+        const unsigned m0 = __ballot_sync(0xFFFFFFFFu, b0 == w), m1 = __ballot_sync(0xFFFFFFFFu, b1 == w);
+        const int c0 = __popc(m0), c = c0 + __popc(m1);
+        if (b0 == w) r.slot[0] = start + __popc(m0 & lt);
+        if (b1 == w) r.slot[1] = start + c0 + __popc(m1 & lt);
+        n[w] = IS_V ? ((start + c + 3) >> 2) - ((start + 3) >> 2) : c;   // groups whose first slot is in the section
+        start += c;
+    }
+    r.row_w[0] = b0; r.row_w[1] = b1;
+    if (IS_V) {
+        if (b0) sorted[r.slot[0]] = (uint8_t)b0;
+        if (b1) sorted[r.slot[1]] = (uint8_t)b1;
+        __syncwarp();
+        if (b0) r.row_w[0] = sorted[r.slot[0] & ~3];
+        if (b1) r.row_w[1] = sorted[r.slot[1] & ~3];
+    }
+    return r;
+}
+
+constexpr uint32_t NIB = 0x0F0F0F0Fu;
+// (a & m) | (b & ~m)
+__device__ __forceinline__ uint32_t bitsel(uint32_t a, uint32_t b, uint32_t m) { return (a & m) | (b & ~m); }
+
+// The w-bit words of a unit (codes one per byte in creg; bits shift .. shift+3 of them, of which w are in use).
+__device__ __forceinline__ void store_part(uint8_t* dst, int w, int shift, const uint32_t (&creg)[8]) {
+    uint32_t v[4];
 #pragma unroll
-                for (int m = 1; m < 4; ++m) acc |= (creg[4 * j + m] << (2 * m - sh)) & (0x03030303u << (2 * m));
-                w[j] = acc;
-            }
-            store_words<2>(img + base[2] + rk(2) * (D / 4) + p * 8, w);
-        }
-        if (B & 1) {
-            uint32_t acc = 0;
-#pragma unroll
-            for (int m = 0; m < 8; ++m) acc |= (creg[m] & 0x01010101u) << m;
-            *reinterpret_cast<uint32_t*>(img + base[3] + rk(3) * (D / 8) + p * 4) = acc;
-        }
+    for (int u = 0; u < 4; ++u) {
+        const uint32_t a = shift ? creg[2 * u] >> 4 : creg[2 * u], b = shift ? creg[2 * u + 1] : creg[2 * u + 1] << 4;
+        v[u] = bitsel(a, b, NIB);
+    }
+    if (w == 4) {
+        *reinterpret_cast<uint4*>(dst) = make_uint4(v[0], v[1], v[2], v[3]);
+    } else if (w == 3) {
+        uint32_t* x = reinterpret_cast<uint32_t*>(dst);
+        x[0] = v[0] | ((v[3] & 0x11111111u) << 3);
+        x[1] = v[1] | ((v[3] & 0x22222222u) << 2);
+        x[2] = v[2] | ((v[3] & 0x44444444u) << 1);
+    } else if (w == 2) {
+        *reinterpret_cast<uint2*>(dst) = make_uint2(v[0] | (v[1] << 2), v[2] | (v[3] << 2));
     } else {
-        // values: byte lane (rank & 3) of the words of group rank >> 2; channel 32p + 4j + b is byte b of creg[j]
-        if (B & 8) {
-            const int r = rk(0);
-            uint8_t* grp = img + base[0] + (r >> 2) * (D * 4) + (r & 3);
-#pragma unroll
-            for (int j = 0; j < 8; ++j)
-#pragma unroll
-                for (int b = 0; b < 4; ++b) grp[4 * (32 * p + 4 * j + b)] = (uint8_t)(creg[j] >> (8 * b));
-        }
-        if (B & 4) {
-            const int sh = B & 3, r = rk(1);
-            uint8_t* grp = img + base[1] + (r >> 2) * (D * 2) + (r & 3);
-#pragma unroll
-            for (int j = 0; j < 8; ++j) {
-                const uint32_t x = (creg[j] >> sh) & 0x0F0F0F0Fu;
-                const uint32_t y = x | (x >> 4);     // byte 0: channels 4j, 4j+1; byte 2: channels 4j+2, 4j+3
-                grp[4 * (16 * p + 2 * j)] = (uint8_t)y;
-                grp[4 * (16 * p + 2 * j + 1)] = (uint8_t)(y >> 16);
-            }
-        }
-        if (B & 2) {
-            const int sh = B & 1, r = rk(2);
-            uint8_t* grp = img + base[2] + (r >> 2) * D + (r & 3);
-#pragma unroll
-            for (int j = 0; j < 8; ++j) {
-                const uint32_t x = (creg[j] >> sh) & 0x03030303u;
-                const uint32_t z = x | (x >> 6);
-                grp[4 * (8 * p + j)] = (uint8_t)(z | (z >> 12));    // the four 2-bit fields of channels 4j..4j+3
-            }
-        }
-        if (B & 1) {
-            const int r = rk(3);
-            uint8_t* grp = img + base[3] + (r >> 2) * (D / 2) + (r & 3);
-#pragma unroll
-            for (int j = 0; j < 8; j += 2) {
-                const uint32_t n0 = (((creg[j] & 0x01010101u) * 0x01020408u) >> 24) & 15u;
-                const uint32_t n1 = (((creg[j + 1] & 0x01010101u) * 0x01020408u) >> 24) & 15u;
-                grp[4 * (4 * p + j / 2)] = (uint8_t)(n0 | (n1 << 4));
-            }
-        }
+        *reinterpret_cast<uint32_t*>(dst) = v[0] | (v[1] << 1) | (v[2] << 2) | (v[3] << 3);
     }
 }
-
-template <int D, bool IS_V>
-__device__ __forceinline__ void write_pieces(uint8_t* img, const TileMasks& tm, const uint32_t (&base)[5], int slot, int B,
-                                             int p, const uint32_t (&creg)[8]) {
-    write_pieces<D, IS_V>(img, MaskRanks{tm, slot}, base, B, p, creg);
-}
-
-// The inverse: codes of one thread's 32 channels (one per byte) put together from the token's pieces.
-template <int D, bool IS_V>
-__device__ __forceinline__ void read_pieces(const uint8_t* img, const TileMasks& tm, const uint32_t (&base)[5], int slot, int B,
-                                            int p, uint32_t (&creg)[8]) {
+// The nibble words of a unit of w-bit words.  Bits of a nibble beyond the w lowest are undefined.
+template <int W>
+__device__ __forceinline__ void nibble_words(const uint32_t* x, uint32_t (&v)[4]) {
+    if (W == 4) {
 #pragma unroll
-    for (int j = 0; j < 8; ++j) creg[j] = 0;
-    if (!IS_V) {
-        if (B & 8) load_words<8>(img + base[0] + rank_in(tm, 0, slot) * D + p * 32, creg);
-        if (B & 4) {
-            const int sh = B & 3;
-            uint32_t w[4];
-            load_words<4>(img + base[1] + rank_in(tm, 1, slot) * (D / 2) + p * 16, w);
-#pragma unroll
-            for (int j = 0; j < 4; ++j) {
-                creg[2 * j] |= (w[j] & 0x0F0F0F0Fu) << sh;
-                creg[2 * j + 1] |= ((w[j] >> 4) & 0x0F0F0F0Fu) << sh;
-            }
-        }
-        if (B & 2) {
-            const int sh = B & 1;
-            uint32_t w[2];
-            load_words<2>(img + base[2] + rank_in(tm, 2, slot) * (D / 4) + p * 8, w);
-#pragma unroll
-            for (int j = 0; j < 2; ++j)
-#pragma unroll
-                for (int m = 0; m < 4; ++m) creg[4 * j + m] |= ((w[j] >> (2 * m)) & 0x03030303u) << sh;
-        }
-        if (B & 1) {
-            const uint32_t w = *reinterpret_cast<const uint32_t*>(img + base[3] + rank_in(tm, 3, slot) * (D / 8) + p * 4);
-#pragma unroll
-            for (int m = 0; m < 8; ++m) creg[m] |= (w >> m) & 0x01010101u;
-        }
+        for (int u = 0; u < 4; ++u) v[u] = x[u];
+    } else if (W == 3) {
+        v[0] = x[0]; v[1] = x[1]; v[2] = x[2];
+        v[3] = ((x[0] >> 3) & 0x11111111u) | ((x[1] >> 2) & 0x22222222u) | ((x[2] >> 1) & 0x44444444u);
+    } else if (W == 2) {
+        v[0] = x[0]; v[1] = x[0] >> 2; v[2] = x[1]; v[3] = x[1] >> 2;
     } else {
-        if (B & 8) {
-            const int r = rank_in(tm, 0, slot);
-            const uint8_t* grp = img + base[0] + (r >> 2) * (D * 4) + (r & 3);
+        v[0] = x[0]; v[1] = x[0] >> 1; v[2] = x[0] >> 2; v[3] = x[0] >> 3;
+    }
+}
+// the codes (one per byte) of a unit's words, or'd into creg at bit `shift` (0 or 4)
+__device__ __forceinline__ void take_part(const uint32_t (&x)[4], int w, int shift, uint32_t (&creg)[8]) {
+    uint32_t v[4];
+    if (w == 4) nibble_words<4>(x, v);
+    else if (w == 3) nibble_words<3>(x, v);
+    else if (w == 2) nibble_words<2>(x, v);
+    else nibble_words<1>(x, v);
+    const uint32_t m = 0x01010101u * ((1u << w) - 1u);
 #pragma unroll
-            for (int j = 0; j < 8; ++j)
-#pragma unroll
-                for (int b = 0; b < 4; ++b) creg[j] |= (uint32_t)grp[4 * (32 * p + 4 * j + b)] << (8 * b);
-        }
-        if (B & 4) {
-            const int sh = B & 3, r = rank_in(tm, 1, slot);
-            const uint8_t* grp = img + base[1] + (r >> 2) * (D * 2) + (r & 3);
-#pragma unroll
-            for (int j = 0; j < 8; ++j) {
-                const uint32_t b0 = grp[4 * (16 * p + 2 * j)], b1 = grp[4 * (16 * p + 2 * j + 1)];
-                const uint32_t x = (b0 & 15u) | ((b0 >> 4) << 8) | ((b1 & 15u) << 16) | ((b1 >> 4) << 24);
-                creg[j] |= x << sh;
-            }
-        }
-        if (B & 2) {
-            const int sh = B & 1, r = rank_in(tm, 2, slot);
-            const uint8_t* grp = img + base[2] + (r >> 2) * D + (r & 3);
-#pragma unroll
-            for (int j = 0; j < 8; ++j) {
-                const uint32_t b = grp[4 * (8 * p + j)];
-                const uint32_t u = b | (b << 12);
-                creg[j] |= ((u | (u << 6)) & 0x03030303u) << sh;
-            }
-        }
-        if (B & 1) {
-            const int r = rank_in(tm, 3, slot);
-            const uint8_t* grp = img + base[3] + (r >> 2) * (D / 2) + (r & 3);
-#pragma unroll
-            for (int j = 0; j < 8; ++j) {
-                const uint32_t b = ((uint32_t)grp[4 * (4 * p + j / 2)] >> (4 * (j & 1))) & 15u;
-                creg[j] |= (b * 0x00204081u) & 0x01010101u;
-            }
-        }
+    for (int u = 0; u < 4; ++u) {
+        creg[2 * u] |= (v[u] & m) << shift;
+        creg[2 * u + 1] |= ((v[u] >> 4) & m) << shift;
     }
 }
 
-// ------------------------------------------------------------------------------------------ values, fast writer
-// The quantizer builds the values of a tile in two steps so that it never stores single bytes of a word that four
-// tokens share.  Step 1 (write_planes_v): every token writes its row of packed w-bit fields (consecutive channels,
-// lowest bits first) on its own with vector stores: the item of rank r of section c takes the quarter (r & 3) of
-// its group.  Step 2 (group_unit_v): 16 bytes of the final layout, words 4u .. 4u+3 of a group, are the 4x4 byte
-// transpose of word u of the group's four rows.
-template <int D, typename Ranks>
-__device__ __forceinline__ void write_planes_v(uint8_t* img, const Ranks& rk, const uint32_t (&base)[5], int B, int p,
-                                               const uint32_t (&creg)[8]) {
-    if (B & 8) {
-        const int r = rk(0);
-        store_words<8>(img + base[0] + (r >> 2) * (D * 4) + (r & 3) * D + 32 * p, creg);
-    }
-    if (B & 4) {
-        const int sh = B & 3, r = rk(1);
-        uint32_t y[8], w[4];
-#pragma unroll
-        for (int j = 0; j < 8; ++j) {
-            const uint32_t x = (creg[j] >> sh) & 0x0F0F0F0Fu;
-            y[j] = x | (x >> 4);                     // byte 0: channels 4j, 4j+1; byte 2: channels 4j+2, 4j+3
-        }
-#pragma unroll
-        for (int m = 0; m < 4; ++m) w[m] = prmt(y[2 * m], y[2 * m + 1], 0x6420u);
-        store_words<4>(img + base[1] + (r >> 2) * (D * 2) + (r & 3) * (D / 2) + 16 * p, w);
-    }
-    if (B & 2) {
-        const int sh = B & 1, r = rk(2);
-        // the four 2-bit fields of a register gathered into one byte by a multiplication: field b (bit 8b + sh) times
-        // 2^(24 - 6b - sh) lands at bit 24 + 2b, and no other product of a field and a term reaches the top byte
-        const uint32_t msk = 0x03030303u << sh, mul = 0x01041040u >> sh;
-        uint32_t t[8], w[2];
-#pragma unroll
-        for (int j = 0; j < 8; ++j) t[j] = (creg[j] & msk) * mul;
-#pragma unroll
-        for (int k = 0; k < 2; ++k)
-            w[k] = prmt(prmt(t[4 * k], t[4 * k + 1], 0x0073u), prmt(t[4 * k + 2], t[4 * k + 3], 0x0073u), 0x5410u);
-        store_words<2>(img + base[2] + (r >> 2) * D + (r & 3) * (D / 4) + 8 * p, w);
-    }
-    if (B & 1) {
-        const int r = rk(3);
-        // the low bits of a register's four bytes gathered into a nibble by a multiplication (bit 8b times 2^(24 - 7b)
-        // lands at bit 24 + b); odd registers are placed four bits higher, so that a pair fills the top byte
-        uint32_t t[4];
-#pragma unroll
-        for (int k = 0; k < 4; ++k)
-            t[k] = (((creg[2 * k] & 0x01010101u) * 0x01020408u) & 0x0F000000u) | (((creg[2 * k + 1] & 0x01010101u) * 0x10204080u) & 0xF0000000u);
-        const uint32_t w = prmt(prmt(t[0], t[1], 0x0073u), prmt(t[2], t[3], 0x0073u), 0x5410u);
-        *reinterpret_cast<uint32_t*>(img + base[3] + (r >> 2) * (D / 2) + (r & 3) * (D / 8) + 4 * p) = w;
-    }
+// index of unit e of row r (counted from the section's first row) of a section of n rows of values
+__device__ __forceinline__ uint32_t v_unit(int D, int n, int r, int e) {
+    const int k4 = r & ~3, m = n - k4 < 4 ? n - k4 : 4;
+    return (uint32_t)(k4 * (D / 8) + e * m + (r & 3));
 }
 
-// 16 bytes at offset o (a multiple of 16, QAQ_TILE_HDR <= o < base[4]) of the final layout of a values tile, from
-// the rows that write_planes_v left in the image
-template <int D, int C>
-__device__ __forceinline__ uint4 group_unit_c(const uint8_t* img, uint32_t sec, uint32_t rel) {
-    constexpr int W = 8 >> C, GB = D * W / 2;
-    const uint32_t G = rel / GB, u = (rel % GB) >> 4;
-    const uint8_t* grp = img + sec + G * GB + 4 * u;
-    uint32_t in[4];
+// One thread's 32 channels (block p) of a token, codes one per byte, written at its slot into a tile image:
+// keys as they are stored, values token by token (the token's words of a row take the quarter slot & 3 of the row's
+// bytes; group_out turns rows into the stored form).  B: width of the row.
+template <int D>
+__device__ __forceinline__ void write_token(uint8_t* img, const Section& s, bool is_v, int slot, int B, int p, const uint32_t (&creg)[8]) {
+    const int w = B < 4 ? B : 4;
+    store_part(img + s.main + ((slot - (is_v ? 4 * s.mstart : s.mstart)) * (D / 32) + p) * 4 * w, w, 0, creg);
+    if (B > 4) store_part(img + s.high + ((slot - (is_v ? 4 * s.start : s.start)) * (D / 32) + p) * 4 * (B - 4), B - 4, 4, creg);
+}
+
+// Values: one part of unit 4p + b of row r of a section as it is stored, from the words of its four tokens in the image.
+template <int D, int W>
+__device__ __forceinline__ void group_part(const uint8_t* img, uint8_t* dst, uint32_t base, int n, int r, int e) {
+    const uint32_t* src = reinterpret_cast<const uint32_t*>(img + base) + (uint32_t)(4 * r * (D / 32) + (e >> 2)) * W;
+    const uint32_t s01 = 0x0040u + 0x0011u * (uint32_t)(e & 3);     // byte e & 3 of both operands
+    uint32_t y[W];
+    uint32_t x[4][W];
 #pragma unroll
-    for (int i = 0; i < 4; ++i) in[i] = *reinterpret_cast<const uint32_t*>(grp + i * (GB / 4));
-    const uint32_t t0 = prmt(in[0], in[1], 0x5140u), t1 = prmt(in[2], in[3], 0x5140u);
-    const uint32_t t2 = prmt(in[0], in[1], 0x7362u), t3 = prmt(in[2], in[3], 0x7362u);
-    return make_uint4(prmt(t0, t1, 0x5410u), prmt(t0, t1, 0x7632u), prmt(t2, t3, 0x5410u), prmt(t2, t3, 0x7632u));
+    for (int i = 0; i < 4; ++i) load_words<W>(reinterpret_cast<const uint8_t*>(src + i * (D / 32) * W), x[i]);
+#pragma unroll
+    for (int c = 0; c < W; ++c) y[c] = prmt(prmt(x[0][c], x[1][c], s01), prmt(x[2][c], x[3][c], s01), 0x5410u);
+    store_words<W>(dst + base + v_unit(D, n, r, e) * 4 * W, y);
 }
 template <int D>
-__device__ __forceinline__ uint4 group_unit_v(const uint8_t* img, const uint32_t (&base)[5], uint32_t o) {
-    if (o >= base[3]) return group_unit_c<D, 3>(img, base[3], o - base[3]);
-    if (o >= base[2]) return group_unit_c<D, 2>(img, base[2], o - base[2]);
-    if (o >= base[1]) return group_unit_c<D, 1>(img, base[1], o - base[1]);
-    return group_unit_c<D, 0>(img, base[0], o - base[0]);
+__device__ __forceinline__ void group_out(const uint8_t* img, uint8_t* dst, const Section& s, int W, int row, int e) {
+    const int r = row - s.start, n = s.n, rm = row - s.mstart;
+    switch (W) {
+        case 1: group_part<D, 1>(img, dst, s.main, s.mn, rm, e); break;
+        case 2: group_part<D, 2>(img, dst, s.main, s.mn, rm, e); break;
+        case 3: group_part<D, 3>(img, dst, s.main, s.mn, rm, e); break;
+        default:
+            group_part<D, 4>(img, dst, s.main, s.mn, rm, e);
+            if (W == 5) group_part<D, 1>(img, dst, s.high, n, r, e);
+            else if (W == 6) group_part<D, 2>(img, dst, s.high, n, r, e);
+            else if (W == 7) group_part<D, 3>(img, dst, s.high, n, r, e);
+            else if (W == 8) group_part<D, 4>(img, dst, s.high, n, r, e);
+    }
 }
 
-// The w-bit piece (w = 8 >> c) of channel d of the item of rank r in section c (for the canonical export).
-template <bool IS_V>
-__device__ __forceinline__ uint32_t piece_at(const uint8_t* tile, const uint32_t (&base)[5], int D, int c, int r, int d) {
-    const int w = 8 >> c, per = 8 / w;
-    if (!IS_V) {
-        const uint8_t* item = tile + base[c] + (size_t)r * (D * w / 8);
-        const int p = d >> 5, j = (d >> 2) & 7, i = d & 3;
-        const uint32_t word = *reinterpret_cast<const uint32_t*>(item + 4 * (p * w + j * w / 8));
-        return (word >> (8 * i + w * (j & (per - 1)))) & ((1u << w) - 1u);
-    } else {
-        const uint8_t* grp = tile + base[c] + (size_t)(r >> 2) * (D * w / 2);
-        return ((uint32_t)grp[4 * (d / per) + (r & 3)] >> (w * (d & (per - 1)))) & ((1u << w) - 1u);
+// The inverse of write_token (and of group_out) on a stored tile: codes of one thread's 32 channels, one per byte.
+// B: width of the token's row.
+template <int D, bool IS_V>
+__device__ __forceinline__ void read_token(const uint8_t* tile, const Section& s, int slot, int B, int p, uint32_t (&creg)[8]) {
+#pragma unroll
+    for (int j = 0; j < 8; ++j) creg[j] = 0;
+#pragma unroll
+    for (int part = 0; part < 2; ++part) {
+        const int w = part ? B - 4 : (B < 4 ? B : 4);
+        if (w < 1) continue;
+        const uint8_t* src = tile + (part ? s.high : s.main);
+        const int first = part ? s.start : s.mstart, n = part ? s.n : s.mn;
+        uint32_t x[4] = {0, 0, 0, 0};
+        if (!IS_V) {
+            const uint32_t* u = reinterpret_cast<const uint32_t*>(src + (uint32_t)((slot - first) * (D / 32) + p) * 4 * w);
+#pragma unroll
+            for (int c = 0; c < 4; ++c) if (c < w) x[c] = u[c];
+        } else {
+#pragma unroll
+            for (int b = 0; b < 4; ++b) {
+                const uint8_t* u = src + v_unit(D, n, (slot >> 2) - first, 4 * p + b) * 4 * w + (slot & 3);
+#pragma unroll
+                for (int c = 0; c < 4; ++c) if (c < w) x[c] |= (uint32_t)u[4 * c] << (8 * b);
+            }
+        }
+        take_part(x, w, 4 * part, creg);
     }
 }
 

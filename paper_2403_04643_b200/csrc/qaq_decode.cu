@@ -1,7 +1,8 @@
 // S4+S5: decode attention over the packed cache (Section 2.1 / Figure 1 of the paper):
 //   S = Softmax(scale * q Khat^T),  X = S Vhat,  xhat = min + (code + 1/2) * step,
 // outliers restored from the sparse side list, split over the sequence with a
-// log-sum-exp merge of the split partials.
+// log-sum-exp merge of the split partials; one, two or four queries per (b,h) and pass (Section 4.2,
+// "Integration in text generation process": the packed cache is what every query reads).
 //
 // The affine map is factored out of the inner loops so they work on raw codes:
 //   q . Khat_t = step_t * sum_d q_d c_td + (min_t + step_t/2) * sum_d q_d
@@ -9,41 +10,118 @@
 // and a token's outliers add  q_ch * (x - (min_t + step_t/2))  resp.  p_t * (v - ...)
 // because their code slot holds 0.
 //
-// Both sums over codes run on the integer tensor-core instruction mma.sync.m16n8k32 (u8 x s8 -> s32).  A plane
-// word of the cache, after one shift and a byte-replicated mask, holds one w-bit field per byte lane, which is
-// exactly an A-operand register of that instruction (four consecutive k), so a decode step - a GEMV, whose cost
-// here is taking bit fields apart, not multiplying - spends one instruction per 512 code-times-weight products
-// instead of one per four.  The exact integer sums make the result independent of any accumulation order.
-//   q.K:  rows = 16 tokens of a section, k = channels; B = q in 16-bit fixed point per (b,h), split into two
-//         signed byte digits that sit in columns 0 and 1 (q_d ~ qscale * (256 * hi_d + lo_d)).
-//   S.V:  rows = 16 channels, k = 32 tokens of a section (the value pieces of four tokens share a word, one per
-//         byte lane); B = the per-token weights p_t * step_t * 2^shift in 23-bit fixed point with one scale per
-//         tile, three signed byte digits in columns 0..2.  The integer sums of a tile are added to binary32
-//         accumulators once per tile.  The rounded weight of a token is also what the softmax denominator and the
-//         constant part of its values use, so numerator and denominator see the same slightly perturbed probability.
+// Both sums over codes run on the integer tensor-core instruction mma.sync (u8 operands, s32 sums).  The cache stores
+// the codes so that a loaded word is one mask (for some widths a shift) away from an operand register
+// (qaq_codec.cuh), so a decode step - a GEMV, whose cost here is taking bit fields apart, not multiplying - spends one
+// tensor-core instruction per 512 (keys) or 256 (values) code-times-weight products.  The exact integer sums make the
+// result independent of any accumulation order.
+//   q.K:  m16n8k32, rows = 16 tokens of one width, k = channels; B = q in 16-bit fixed point per (b,h), split into two
+//         signed byte digits in two columns per query (q_d ~ qscale * (256 * hi_d + lo_d)).
+//   S.V:  m16n8k16, rows = 16 channels, k = 16 slots of one width; B = the per-token weights p_t * step_t in 28-bit
+//         fixed point, four byte digits in four columns per query.  The sums of consecutive tiles stay in the integer
+//         accumulators while they share the reference of the exponentials and the size of a unit.  The rounded weight
+//         of a token is also what the softmax denominator and the constant part of its values use, so numerator and
+//         denominator see the same slightly perturbed probability.
 //
 // One CTA = one run of consecutive tiles of the flattened (b,h, tile) sequence (runs of equal length, so every SM
 // gets the same amount of work); each warp works through whole tiles (QAQ_TILE tokens) on its own, with its own
-// running max / sum / accumulators and no CTA barrier in the tile loop; warps are merged once at the end.  A tile
-// is stored as sections of equal-width pieces behind a header of four masks (qaq_codec.cuh), so every inner loop
-// runs one extraction routine over the items of one section, and a token finds its items by its rank among the
-// tokens that have a piece of that width (population counts on the masks; no lists are built, the per-token
-// widths are not read).  The packed bytes of the next tile are copied to a per-warp shared-memory buffer with
-// cp.async while the current one is worked on: the keys during the value phase (at the front of the buffer), the
-// values during the key phase (at its back).  The buffer is sized for typical tiles; a tile that does not fit
-// beside its neighbour is read in place from global memory by the same loops.
+// running sums and no CTA barrier in the tile loop; warps are merged once at the end.  Lane l looks after tokens 2l and
+// 2l + 1 of the tile (logit, softmax weight, value weight); the tokens of a tile are stored sorted by width, so the
+// section loops run one extraction routine over full row blocks, write dot products and read weights by slot, and a
+// token finds its own through the slot in its metadata.
+// The packed bytes and the outlier list of a tile come to the warp's shared-memory buffer by bulk copies (one per piece,
+// completion on a transaction barrier): the next keys to the front while the values are worked on, the values to the back
+// while the keys are.  The buffer holds both for typical tiles; what does not fit beside its neighbour is copied later,
+// when the neighbour has been used.
 //
-// Outlier corrections are summed in fixed point with 32-bit integer atomics in shared memory (a high and a low
-// part with fixed scales), so the result does not depend on the order in which lanes arrive.
-#include "qaq_decode_common.cuh"
+// Outlier corrections are summed in fixed point with 32-bit integer atomics in shared memory, so the result does not
+// depend on the order in which lanes arrive.
+//
+// The partials of a (b,h) that was split over several CTAs are merged by the last of these CTAs to finish, in the
+// same launch (see finish_split).
+#include <atomic>
+#include <chrono>
+#include <mutex>
+
+#include "qaq_codec.cuh"
+#include "qaq_internal.cuh"
 
 namespace {
 
-using namespace qaqd;
+using qaqc::Section;
 
-constexpr int DEC_WARPS = 4;
-constexpr int DEC_THREADS = DEC_WARPS * 32;
-constexpr int DEC_CTAS_PER_SM = 4;
+// ------------------------------------------------------------------------------------------ instructions
+// D(16x8, s32) += A(16x32, u8, row) * B(32x8, s8, col).  Lane = 4*g + t holds
+//   a0: row g, k 4t..4t+3   a1: row g+8, k 4t..4t+3   a2: row g, k 16+4t..   a3: row g+8, k 16+4t..   (one k per byte)
+//   b0: k 4t..4t+3, column g   b1: k 16+4t.., column g
+//   d0, d1: row g, columns 2t, 2t+1   d2, d3: row g+8, columns 2t, 2t+1
+__device__ __forceinline__ void mma_k32(int (&d)[4], uint32_t a0, uint32_t a1, uint32_t a2, uint32_t a3, uint32_t b0, uint32_t b1) {
+    asm volatile("mma.sync.aligned.m16n8k32.row.col.s32.u8.s8.s32 {%0,%1,%2,%3}, {%4,%5,%6,%7}, {%8,%9}, {%0,%1,%2,%3};"
+                 : "+r"(d[0]), "+r"(d[1]), "+r"(d[2]), "+r"(d[3])
+                 : "r"(a0), "r"(a1), "r"(a2), "r"(a3), "r"(b0), "r"(b1));
+}
+// D(16x8, s32) += A(16x16, u8, row) * B(16x8, u8, col): a0, a1 and b0 as above
+__device__ __forceinline__ void mma_k16(int (&d)[4], uint32_t a0, uint32_t a1, uint32_t b0) {
+    asm volatile("mma.sync.aligned.m16n8k16.row.col.s32.u8.u8.s32 {%0,%1,%2,%3}, {%4,%5}, {%6}, {%0,%1,%2,%3};"
+                 : "+r"(d[0]), "+r"(d[1]), "+r"(d[2]), "+r"(d[3])
+                 : "r"(a0), "r"(a1), "r"(b0));
+}
+// the same two with a zero third operand
+__device__ __forceinline__ void mma_k32_first(int (&d)[4], uint32_t a0, uint32_t a1, uint32_t a2, uint32_t a3, uint32_t b0, uint32_t b1) {
+    asm volatile("mma.sync.aligned.m16n8k32.row.col.s32.u8.s8.s32 {%0,%1,%2,%3}, {%4,%5,%6,%7}, {%8,%9}, {%10,%10,%10,%10};"
+                 : "=r"(d[0]), "=r"(d[1]), "=r"(d[2]), "=r"(d[3])
+                 : "r"(a0), "r"(a1), "r"(a2), "r"(a3), "r"(b0), "r"(b1), "r"(0));
+}
+__device__ __forceinline__ uint32_t smem_addr(const void* p) { return (uint32_t)__cvta_generic_to_shared(p); }
+// W words from shared memory (aligned to the widest access taken: 16 bytes for four words, 8 for two, else 4)
+template <int W>
+__device__ __forceinline__ void lds_words(uint32_t addr, uint32_t (&x)[W]) {
+    if constexpr (W == 4) asm volatile("ld.shared.v4.u32 {%0,%1,%2,%3}, [%4];" : "=r"(x[0]), "=r"(x[1]), "=r"(x[2]), "=r"(x[3]) : "r"(addr));
+    else if constexpr (W == 2) asm volatile("ld.shared.v2.u32 {%0,%1}, [%2];" : "=r"(x[0]), "=r"(x[1]) : "r"(addr));
+    else {
+#pragma unroll
+        for (int i = 0; i < W; ++i) asm volatile("ld.shared.u32 %0, [%1];" : "=r"(x[i]) : "r"(addr + 4 * i));
+    }
+}
+__device__ __forceinline__ void sts_word(uint32_t addr, int v) { asm volatile("st.shared.u32 [%0], %1;" ::"r"(addr), "r"(v) : "memory"); }
+
+// bulk copies into shared memory, completion on a transaction barrier
+__device__ __forceinline__ void bar_init(uint32_t bar) { asm volatile("mbarrier.init.shared::cta.b64 [%0], 1;" ::"r"(bar) : "memory"); }
+__device__ __forceinline__ void bar_expect(uint32_t bar, uint32_t bytes) {
+    asm volatile("mbarrier.arrive.expect_tx.shared::cta.b64 _, [%0], %1;" ::"r"(bar), "r"(bytes) : "memory");
+}
+__device__ __forceinline__ void bulk_copy(uint32_t dst, const void* src, uint32_t bytes, uint32_t bar) {
+    asm volatile("cp.async.bulk.shared::cluster.global.mbarrier::complete_tx::bytes [%0], [%1], %2, [%3];" ::"r"(dst), "l"(src), "r"(bytes), "r"(bar)
+                 : "memory");
+}
+// false if the phase did not complete within the limit (seconds; a copy takes microseconds)
+__device__ __forceinline__ bool bar_wait(uint32_t bar, uint32_t parity) {
+    uint32_t done = 0;
+#pragma unroll 1
+    for (int i = 0; i < (1 << 22) && !done; ++i)
+        asm volatile("{\n.reg .pred p;\nmbarrier.try_wait.parity.shared::cta.b64 p, [%1], %2;\nselp.u32 %0, 1, 0, p;\n}" : "=r"(done) : "r"(bar), "r"(parity) : "memory");
+    return done != 0;
+}
+__device__ __forceinline__ float warp_max(float x) {
+    float r;
+    asm("redux.sync.max.f32 %0, %1, 0xffffffff;" : "=f"(r) : "f"(x));
+    return r;
+}
+__device__ __forceinline__ float warp_sum(float x) {
+#pragma unroll
+    for (int o = 16; o > 0; o >>= 1) x += __shfl_xor_sync(0xFFFFFFFFu, x, o);
+    return x;
+}
+
+// ------------------------------------------------------------------------------------------ shapes
+// Warps per CTA and CTAs per SM by queries per pass: 16 warps per SM for one query (128 registers each), 12 for four
+// (168 registers: four times the accumulators on the value side).
+template <int NQ> struct Shape {
+    static constexpr int WARPS = NQ == 4 ? 4 : 8, CTAS_PER_SM = NQ == 4 ? 3 : 2, THREADS = 32 * WARPS, SLOTS = 148 * CTAS_PER_SM;
+};
+constexpr int SCORES_FUSED_TOKENS = 8192;          // up to here the CTA that merges a (b,h) normalises its score row too
+constexpr uint32_t LIST_STAGED = 1024;             // outlier entries per tile and tensor that come through shared memory at most; more are read in place
+constexpr uint32_t SMALL_MAX = 0x5800u;            // 128 as binary16: up to here outlier terms are summed in one 32-bit word
 
 struct DecArgs {
     TensorStore k, v;
@@ -53,25 +131,28 @@ struct DecArgs {
     int T;
     const int* d_count;          // counted kernels only: the token count in device memory (T, run and ncta are then derived from it)
     const __half* q;
-    long q_stride, out_stride;   // elements between the rows of consecutive (b,h) in q and in out
+    long q_stride, out_stride;   // elements between the rows of consecutive (b,h) in q and in out (queries of a (b,h) are D apart)
     float scale;
-    float* part;       // [ncta][2][D+3]: accumulators, running max, sum of the weights used, exact sum
-    float* ml;         // [BH][2]   merged (max, sum) for score normalisation
+    float* part;       // [ncta][2][NQ][D+4]: accumulators, reference of the exponentials, sum of the weights used, exact sum
+    unsigned long long* done;    // [BH]: tag of the call | partials that are complete (see finish_split)
+    unsigned long long tag;      // of this call; the low 12 bits are zero
+    float* ml;         // [BH][2]   merged (max, sum) for the normalisation of long score rows, or null
     int BH, run, ncta; // (b,h) count; tiles per CTA of the flattened (b,h, tile) sequence; CTAs
-    float* out;        // [BH][D]
-    float* scores;     // [BH][scores_stride] or null
+    float* out;
+    float* scores;     // [BH][scores_stride] or null (one query only)
     long scores_stride;
+    int* status;       // device status of the cache (a copy that never completed)
 };
 
 // The flattened sequence of BH * ntiles tiles is cut into runs of `run` consecutive tiles, one CTA
-// each: enough CTAs to fill every SM (148 SMs, 4 resident CTAs each) evenly, at least one tile per
-// warp where there are that many, and never more than one (b,h) boundary inside a run.
-constexpr int DEC_SLOTS = 148 * DEC_CTAS_PER_SM;
+// each: enough CTAs to fill every SM evenly, at least one tile per warp where there are that many, and never more than
+// one (b,h) boundary inside a run.
 struct DecPlan { int run, ncta; };
+template <int NQ>
 __host__ __device__ inline DecPlan plan_decode(int BH, int ntiles) {
     const long long total = (long long)BH * ntiles;
-    long long run = (total + DEC_SLOTS - 1) / DEC_SLOTS;
-    const int floor_run = ntiles < DEC_WARPS ? ntiles : DEC_WARPS;
+    long long run = (total + Shape<NQ>::SLOTS - 1) / Shape<NQ>::SLOTS;
+    const int floor_run = ntiles < Shape<NQ>::WARPS ? ntiles : Shape<NQ>::WARPS;
     if (run < floor_run) run = floor_run;
     if (run > ntiles) run = ntiles;
     DecPlan p;
@@ -80,97 +161,323 @@ __host__ __device__ inline DecPlan plan_decode(int BH, int ntiles) {
     return p;
 }
 
-constexpr int OL_STAGED = 96;     // outlier entries per tile and tensor that come through shared memory; more are read in place
-
+// ------------------------------------------------------------------------------------------ shared memory
 // per-warp scratch for the tile a warp is working on
-template <int D>
+template <int D, int NQ>
 struct WarpScratch {
-    static constexpr int STAGE = 72 * D;      // bytes of the staging buffer (9 KB at head_dim 128: four CTAs per SM)
-    alignas(16) uint8_t buf[STAGE];           // keys of a tile from the front, values from the back
+    static constexpr int STAGE = (NQ == 1 ? 86 : 72) * D;      // bytes of the staging buffer; any tile of one tensor fits alone
+    static constexpr int DOTS = QAQ_TILE + 16;                 // the last row block of a list may store up to 15 rows too many
+    static constexpr int WROW = QAQ_TILE + 4;                  // digit rows are spread over the banks
+    static constexpr int VC = NQ < 2 ? 2 : NQ;
+    static_assert(STAGE % 16 == 0 && STAGE >= qaqc::tile_bytes_max(D), "staging buffer");
+    alignas(16) uint8_t buf[STAGE];           // keys (tile, outlier list) from the front, values to the back
     union alignas(16) {                       // the key phase is over (logits taken) before the value weights are written
-        int dotw[4][QAQ_TILE];                // integer q . piece per section and rank
-        uint32_t wts[4][QAQ_TILE / 4][4];     // per section and value group: the three byte digits of the four weights
+        int dot[2][DOTS][NQ];                 // integer q . (low 4 bits of the code), q . (the bits above) by slot
+        uint8_t wts[2][NQ][4][WROW];          // the four byte digits (highest first) of the value weights, and of 16 times them, by slot
     };
-    uint32_t olist[2][OL_STAGED];             // the first outlier entries of the tile's keys / values (copied in with the packed words)
-    float midK[QAQ_TILE];       // min + step/2
-    float midV[QAQ_TILE];
-    float p[QAQ_TILE];          // attention weights of the tile's tokens at the current scale of the running sums
-    int kcorr[2][QAQ_TILE];     // fixed-point sums (high, low part) of the key-outlier corrections per token (zero between tiles)
-    int vcorr[2][D];            // ... of the value-outlier corrections per channel (zero between tiles)
+    union alignas(16) {                       // likewise
+        int kcorr[NQ][2][QAQ_TILE];           // fixed-point sums of the key-outlier corrections per token (second word: the low part)
+        float2 tok[NQ][QAQ_TILE];             // p, p * (min + step/2) of the values
+    };
+    alignas(8) float mid[QAQ_TILE];           // min + step/2 of the keys
+    alignas(16) int vcorr[VC][D];             // fixed-point sums of the value-outlier corrections per channel (zero between uses)
+    alignas(16) float macc[NQ][D];            // weighted sums of the values, as far as they have left the integer accumulators
+    alignas(8) unsigned long long bar[2];     // transaction barriers of the keys and of the values
 };
 
-template <int D>
+template <int D, int NQ>
 struct DecSmem {
-    WarpScratch<D> ws[DEC_WARPS];
-    float qf[D];
-    float macc[DEC_WARPS][D];
-    float mm[DEC_WARPS], ml[DEC_WARPS], mlx[DEC_WARPS];
-    float red[DEC_WARPS], red2[DEC_WARPS];
-    float qscale, qsum;
+    WarpScratch<D, NQ> ws[Shape<NQ>::WARPS];
+    alignas(16) float qf[D][NQ];
+    alignas(16) uint32_t qw[32][D / 16];      // operand words of q per lane: low and high nibbles of its first word, of its second, ...
+    float mm[Shape<NQ>::WARPS][NQ], ml[Shape<NQ>::WARPS][NQ], mlx[Shape<NQ>::WARPS], cs[Shape<NQ>::WARPS][NQ];
+    float red[3 * Shape<NQ>::WARPS];
+    int flag;
 };
 
-// q . piece for the items of one key section: 16 items per instruction row block, lane 4g+t holds the channels
-// 4*(t*NR + r) + i (r < NR = D/16) of items g and g+8
+// ------------------------------------------------------------------------------------------ lists of rows
+// The nibble words of a key row a lane works with: of the four of its unit those of its channels (at head_dim 128 all
+// four, at 64 two, at 32 one, by t).
 template <int D, int W>
-__device__ __forceinline__ void k_section(const uint8_t* sec, int n, int* dots, const uint32_t (&qb)[D / 16], int g, int t) {
-    constexpr int NR = D / 16, ITEM = D * W / 8;
-#pragma unroll 1
-    for (int i0 = 0; i0 < n; i0 += 16) {
-        const int r0 = i0 + g, r1 = r0 + 8;
-        uint32_t x0[NR], x1[NR];
-        fetch_regs<W, NR>(sec + r0 * ITEM, t * NR, r0 < n, x0);
-        fetch_regs<W, NR>(sec + r1 * ITEM, t * NR, r1 < n, x1);
-        int d[4] = {0, 0, 0, 0};
+__device__ __forceinline__ void key_words(uint32_t addr, int t, uint32_t (&v)[D / 32]) {
+    uint32_t x[W], a[4];
+    lds_words<W>(addr, x);
+    qaqc::nibble_words<W>(x, a);
+    if (D == 128) {
 #pragma unroll
-        for (int m = 0; m < NR / 2; ++m) mma_u8s8(d, x0[2 * m], x1[2 * m], x0[2 * m + 1], x1[2 * m + 1], qb[2 * m], qb[2 * m + 1]);
-        if (t == 0) {          // columns 0 and 1: the high and the low digit of q
-            if (r0 < n) dots[r0] = d[0] * 256 + d[1];
-            if (r1 < n) dots[r1] = d[2] * 256 + d[3];
+        for (int u = 0; u < D / 32; ++u) v[u] = a[u];
+    } else if (D == 64) {
+#pragma unroll
+        for (int u = 0; u < D / 32; ++u) v[u] = (t & 1) ? a[2 + u] : a[u];
+    } else {
+        const uint32_t lo = (t & 1) ? a[1] : a[0], hi = (t & 1) ? a[3] : a[2];
+        v[0] = (t & 2) ? hi : lo;
+    }
+}
+
+// q . code for a list of n rows of W-bit codes of the keys: 16 rows per block, lane 4g+t holds the channels of q operand
+// (t, u) of rows g and g+8.  The last block reads past the list (at most 15 rows, inside the warp's scratch) and
+// stores what the next list or nobody writes over it.  A nibble word gives two operand registers: the low nibbles
+// as they are, the high nibbles sixteen times too large, which is taken out of the exact sums.
+template <int D, int W, int NQ>
+__device__ __forceinline__ void k_list(uint32_t addr, int n, uint32_t dots, const uint32_t (&qa)[D / 32], const uint32_t (&qb)[D / 32], int g, int t) {
+    constexpr int P = D / 32;
+    constexpr uint32_t MA = 0x01010101u * ((1u << W) - 1u), MB = MA << 4;
+    addr += (g * P + (t * P >> 2)) * 4 * W;
+    dots += (g * NQ + t) * 4;
+#pragma unroll 1
+    for (; n > 0; n -= 16, addr += 64 * P * W, dots += 64 * NQ) {
+        uint32_t v0[P], v1[P];
+        key_words<D, W>(addr, t, v0);
+        key_words<D, W>(addr + 32 * P * W, t, v1);
+        int s0, s1;
+        if constexpr (P == 1) {
+            int a[4];
+            mma_k32_first(a, v0[0] & MA, v1[0] & MA, (v0[0] >> 4) & MA, (v1[0] >> 4) & MA, qa[0], qb[0]);
+            s0 = a[0] * 256 + a[1];
+            s1 = a[2] * 256 + a[3];
+        } else {
+            int a[4], b[4];
+            mma_k32_first(a, v0[0] & MA, v1[0] & MA, v0[1] & MA, v1[1] & MA, qa[0], qa[1]);
+            mma_k32_first(b, v0[0] & MB, v1[0] & MB, v0[1] & MB, v1[1] & MB, qb[0], qb[1]);
+            if constexpr (P == 4) {
+                mma_k32(a, v0[2] & MA, v1[2] & MA, v0[3] & MA, v1[3] & MA, qa[2], qa[3]);
+                mma_k32(b, v0[2] & MB, v1[2] & MB, v0[3] & MB, v1[3] & MB, qb[2], qb[3]);
+            }
+            s0 = a[0] * 256 + a[1] + ((b[0] * 256 + b[1]) >> 4);
+            s1 = a[2] * 256 + a[3] + ((b[2] * 256 + b[3]) >> 4);
+        }
+        if (t < NQ) { sts_word(dots, s0); sts_word(dots + 32 * NQ, s1); }       // columns 2t, 2t+1: the digits of query t
+    }
+}
+
+// Weighted sums over a list of n rows (groups of four slots) of W-bit codes of the values: 4 rows per instruction, lane
+// 4g+t holds the channels of units g (and g + 8 at head_dim 128) of row t.  wt: the lane's digits at the list's first
+// row, pair of queries by pair (`pair` bytes apart).  Rows past the list are read (inside shared memory) with weight
+// zero.  The sums of the high nibbles come out sixteen times too large.
+template <int D, int W, int NQ>
+__device__ __forceinline__ void v_list(uint32_t addr, int n, uint32_t wt, bool use, int (&acc)[(NQ + 1) / 2][D / 16][4], int g, int t) {
+    constexpr int NH = D == 128 ? 2 : 1, NP = (NQ + 1) / 2, PAIR = 8 * WarpScratch<D, NQ>::WROW;
+    constexpr uint32_t MA = 0x01010101u * ((1u << W) - 1u), MB = MA << 4;
+    const int e = D == 32 ? (g & 3) : g;
+#pragma unroll 1
+    for (; n > 0; n -= 4, addr += (D / 2) * 4 * W, wt += 16) {
+        const int m = min(4, n);
+        uint32_t wgt[NP];
+#pragma unroll
+        for (int pr = 0; pr < NP; ++pr) {
+            uint32_t x[1] = {0};
+            if (use && t < m) lds_words<1>(wt + pr * PAIR, x);
+            wgt[pr] = x[0];
+        }
+        const uint32_t at = addr + (e * m + t) * 4 * W;
+#pragma unroll
+        for (int h = 0; h < NH; ++h) {
+            uint32_t x[W], v[4];
+            lds_words<W>(at + h * 32 * W * m, x);
+            qaqc::nibble_words<W>(x, v);
+            // row block 4h + 2 * nibble + u/2: rows g and g+8 are the channels of words u, u+1
+#pragma unroll
+            for (int pr = 0; pr < NP; ++pr) {
+                if constexpr (D == 32) {
+                    const uint32_t u0 = g >= 4 ? v[2] : v[0], u1 = g >= 4 ? v[3] : v[1];
+                    mma_k16(acc[pr][0], u0 & MA, u1 & MA, wgt[pr]);
+                    mma_k16(acc[pr][1], u0 & MB, u1 & MB, wgt[pr]);
+                } else {
+                    mma_k16(acc[pr][4 * h], v[0] & MA, v[1] & MA, wgt[pr]);
+                    mma_k16(acc[pr][4 * h + 1], v[2] & MA, v[3] & MA, wgt[pr]);
+                    mma_k16(acc[pr][4 * h + 2], v[0] & MB, v[1] & MB, wgt[pr]);
+                    mma_k16(acc[pr][4 * h + 3], v[2] & MB, v[3] & MB, wgt[pr]);
+                }
+            }
         }
     }
 }
 
-// weighted sums over the groups of one value section: 8 groups (32 tokens) per instruction, lane 4g+t holds the
-// channels (D/8)*g + 2*mb + s (rows g + 8s of row block mb) of groups t and t+4
-template <int D, int W>
-__device__ __forceinline__ void v_section(const uint8_t* sec, int ngroups, const uint32_t (*wts)[4], int (&acc)[D / 16][4], int g, int t) {
-    constexpr int NRV = D / 8, GB = D * W / 2;
-#pragma unroll 1
-    for (int g0 = 0; g0 < ngroups; g0 += 8) {
-        const int ga = g0 + t, gb = ga + 4;
-        uint32_t xa[NRV], xb[NRV];
-        fetch_regs<W, NRV>(sec + ga * GB, g * NRV, ga < ngroups, xa);
-        fetch_regs<W, NRV>(sec + gb * GB, g * NRV, gb < ngroups, xb);
-        const uint32_t b0 = (g < 3 && ga < ngroups) ? wts[ga][g] : 0u;
-        const uint32_t b1 = (g < 3 && gb < ngroups) ? wts[gb][g] : 0u;
+// The lists of a tile with U units per row, from its header: pass 0 the main parts (4, 3, 2, 1 bits; rows in slot order),
+// pass 1 the high parts (widths 8, 7, 6, 5; rows in slot order).  o: byte offset, n: rows.
+struct Lists { uint32_t o4, o3, o2, o1; int n4, n3, n2, n1; };
+template <int U>
+__device__ __forceinline__ Lists lists_of(const uint4& h, int pass) {
+    const uint32_t n7 = (h.y >> 16) & 0xFF, n6 = (h.y >> 8) & 0xFF, n5 = h.y & 0xFF, n3 = (h.x >> 16) & 0xFF;
+    const uint32_t z2 = h.z >> 16, z13 = h.w & 0xFFFFu, m3 = z13 + n7 * U * 12, h5 = m3 + n3 * U * 12;
+    Lists l;
+    if (pass == 0) {
+        l.o4 = qaqc::QAQ_TILE_HDR; l.n4 = (int)__dp4a(h.y, 0x01010101u, h.x >> 24);
+        l.o3 = m3; l.n3 = (int)n3;
+        l.o2 = z2 + n6 * U * 8; l.n2 = (int)((h.x >> 8) & 0xFF);
+        l.o1 = h5 + n5 * U * 4; l.n1 = (int)(h.x & 0xFF);
+    } else {
+        l.o4 = h.z & 0xFFFFu; l.n4 = (int)(h.y >> 24);
+        l.o3 = z13; l.n3 = (int)n7;
+        l.o2 = z2; l.n2 = (int)n6;
+        l.o1 = h5; l.n1 = (int)n5;
+    }
+    return l;
+}
+// channel of row g + 8s of value row block mb (blocks of high nibbles: v_high)
+template <int D>
+__device__ __forceinline__ constexpr bool v_high(int mb) { return D == 32 ? mb == 1 : ((mb >> 1) & 1) == 1; }
+template <int D>
+__device__ __forceinline__ int v_channel(int mb, int g, int s) {
+    if (D == 32) return 8 * (2 * (g >> 2) + s) + 4 * mb + (g & 3);
+    const int e = g + 8 * (mb >> 2), u = 2 * (mb & 1) + s;
+    return 32 * (e >> 2) + 8 * u + 4 * ((mb >> 1) & 1) + (e & 3);
+}
+
+// ------------------------------------------------------------------------------------------ outlier sums
+// Outlier terms are summed in fixed point.  Where all values of a tile are small (up to 128) one word is enough: a unit
+// is 2^-22 of a bound on the largest term, so that the 128 terms a token can have (64 per channel) stay inside 32 bits.
+// Otherwise a term is a high part in units of 2^-4 and the exact remainder in units of 2^-28; terms of 2^18 or more (and
+// non-finite ones) are left out.
+constexpr float OC_LIMIT = 262144.0f;
+__device__ __forceinline__ void wide_add(int* hi_cell, int* lo_cell, float tm) {
+    if (fabsf(tm) < OC_LIMIT) {
+        const float hi = rintf(tm * 16.0f);
+        const float rem = fmaf(hi, -0.0625f, tm);              // exact, |rem| <= 2^-5
+        atomicAdd(hi_cell, (int)hi);
+        atomicAdd(lo_cell, __float2int_rn(rem * 268435456.0f));
+    }
+}
+__device__ __forceinline__ float wide_sum(int hi, int lo) { return fmaf((float)lo, 1.0f / 268435456.0f, (float)hi * 0.0625f); }
+// 2^22 over a power of two above x (x > 0, normal), and its inverse
+__device__ __forceinline__ void fixed_unit(float x, float& inv, float& unit) {
+    const int ex = min(max((__float_as_int(x) >> 23) & 0xFF, 40), 240);
+    inv = __int_as_float((254 - ex - 1 + 22) << 23);
+    unit = __int_as_float((ex + 1 - 22) << 23);
+}
+
+// The score row of one (b,h), normalised in place by the whole CTA.
+template <int THREADS>
+__device__ __forceinline__ void normalise_scores(float* row, int T, float M, float LX) {
+    const float inv = LX > 0.f ? 1.0f / LX : 0.f;
+    int t = threadIdx.x;
+    for (; t + 7 * THREADS < T; t += 8 * THREADS) {
+        float x[8];
 #pragma unroll
-        for (int mb = 0; mb < D / 16; ++mb) mma_u8s8(acc[mb], xa[2 * mb], xa[2 * mb + 1], xb[2 * mb], xb[2 * mb + 1], b0, b1);
+        for (int u = 0; u < 8; ++u) x[u] = __ldcg(row + t + u * THREADS);
+#pragma unroll
+        for (int u = 0; u < 8; ++u) row[t + u * THREADS] = __expf(x[u] - M) * inv;
+    }
+    for (; t < T; t += THREADS) row[t] = __expf(__ldcg(row + t) - M) * inv;
+}
+
+// The partial of this CTA's segment is complete (written by all threads).  The CTA that finds all partials of the
+// (b,h) complete merges them (log-sum-exp), in CTA order, so the result does not depend on which one it is.
+//
+// The CTAs are counted in a word of the workspace, which comes uninitialised: the count carries the tag of the call, a
+// number no other call uses, and a word with another tag counts as zero.  The last CTA clears the word, so that a replay
+// of the same launch (a CUDA graph carries the same tag) starts from zero again.
+template <int D, int NQ>
+__device__ void finish_split(const DecArgs& a, DecSmem<D, NQ>& sm, int bh, int ntiles, int run, int T) {
+    using S = Shape<NQ>;
+    const int c_lo = (bh * ntiles) / run, n = ((bh + 1) * ntiles - 1) / run - c_lo + 1;
+    // the CTAs whose runs meet this (b,h); only the first of them can have begun in the (b,h) before (then its second segment)
+    const int first_slot = 2 * c_lo + (c_lo * run < bh * ntiles ? 1 : 0);
+    constexpr int PS = D + 4;
+    auto part = [&](int i, int j) { return a.part + ((size_t)(i == 0 ? first_slot : 2 * (c_lo + i)) * NQ + j) * PS; };
+    const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
+    __syncthreads();
+    if (tid == 0) {
+        asm volatile("fence.acq_rel.gpu;" ::: "memory");
+        unsigned long long cur = *(volatile unsigned long long*)(a.done + bh), next;
+        for (;;) {           // a failed exchange means that another CTA has been counted: at most n rounds
+            next = ((cur ^ a.tag) >> 12) == 0 ? cur + 1 : a.tag + 1;
+            const unsigned long long was = atomicCAS(a.done + bh, cur, next);
+            if (was == cur) break;
+            cur = was;
+        }
+        const bool last = (int)(next & 0xFFF) == n;
+        if (last) a.done[bh] = 0ull;
+        asm volatile("fence.acq_rel.gpu;" ::: "memory");
+        sm.flag = last;
+    }
+    __syncthreads();
+    if (!sm.flag) return;
+    float* s_w = reinterpret_cast<float*>(sm.ws[0].buf);            // [n] <= SLOTS
+    float4* s_x = reinterpret_cast<float4*>(sm.ws[1].buf);          // [THREADS]
+    static_assert(S::SLOTS * sizeof(float) <= sizeof(sm.ws[0].buf) && S::THREADS * sizeof(float4) <= sizeof(sm.ws[1]), "scratch of the merge");
+    for (int j = 0; j < NQ; ++j) {
+        // ---- weights of the partials, sums of the softmax denominators
+        float M = __int_as_float(0xff800000);
+        for (int i = tid; i < n; i += S::THREADS) M = fmaxf(M, __ldcg(part(i, j) + D));
+        M = warp_max(M);
+        if (lane == 0) sm.red[warp] = M;
+        __syncthreads();
+        M = sm.red[0];
+#pragma unroll
+        for (int w = 1; w < S::WARPS; ++w) M = fmaxf(M, sm.red[w]);
+        float L = 0.f, LX = 0.f;
+        for (int i = tid; i < n; i += S::THREADS) {
+            const float4 h = __ldcg(reinterpret_cast<const float4*>(part(i, j) + D));    // reference, sums
+            const float w = h.x == __int_as_float(0xff800000) ? 0.f : __expf(h.x - M);
+            s_w[i] = w;
+            L = fmaf(w, h.y, L);
+            LX = fmaf(w, h.z, LX);
+        }
+        L = warp_sum(L);
+        LX = warp_sum(LX);
+        if (lane == 0) { sm.red[S::WARPS + warp] = L; sm.red[2 * S::WARPS + warp] = LX; }
+        __syncthreads();
+        L = 0.f; LX = 0.f;
+#pragma unroll
+        for (int w = 0; w < S::WARPS; ++w) { L += sm.red[S::WARPS + w]; LX += sm.red[2 * S::WARPS + w]; }
+        // ---- the channels: D/4 threads per partial, four channels each
+        constexpr int CT = D / 4, SH = S::THREADS / CT;
+        const int d4 = tid % CT, sh = tid / CT;
+        float4 x = make_float4(0.f, 0.f, 0.f, 0.f);
+#pragma unroll 4
+        for (int i = sh; i < n; i += SH) {
+            const float w = s_w[i];
+            const float4 v = __ldcg(reinterpret_cast<const float4*>(part(i, j)) + d4);
+            if (w != 0.f) { x.x = fmaf(w, v.x, x.x); x.y = fmaf(w, v.y, x.y); x.z = fmaf(w, v.z, x.z); x.w = fmaf(w, v.w, x.w); }
+        }
+        s_x[tid] = x;
+        __syncthreads();
+        if (tid < D) {
+            float y = 0.f;
+#pragma unroll
+            for (int k = 0; k < SH; ++k) y += reinterpret_cast<const float*>(s_x + k * CT)[tid];
+            a.out[(size_t)bh * a.out_stride + j * D + tid] = L > 0.f ? y / L : 0.f;
+        }
+        if (NQ == 1) {
+            if (a.ml && tid == 0) { a.ml[2 * bh] = M; a.ml[2 * bh + 1] = LX; }
+            if (a.scores && !a.ml) normalise_scores<S::THREADS>(a.scores + (size_t)bh * a.scores_stride, T, M, LX);
+        } else {
+            __syncthreads();
+        }
     }
 }
 
-// One CTA = one run of consecutive tiles, which meets one or two (b,h): the body below runs once
-// per (b,h) segment and leaves one partial per segment.  Every warp works through whole tiles on its
-// own: own running max / sum / accumulators, own staging buffer, no CTA barrier in the loop; the
-// warps are merged once at the end.  Lane l looks after tokens l and l + 32 of the tile (logit, softmax
-// weight, fixed-point value weight); in the section loops lane 4g+t is lane (g, t) of the tensor-core fragments.
+// The body runs once per (b,h) segment of the CTA's run (one or two) and leaves one partial per segment, or the result
+// where a (b,h) is one CTA's alone.  In the section loops lane 4g+t is lane (g, t) of the tensor-core fragments.
 // COUNTED: the token count is read from device memory and the split derived from it here (the grid is then the
 // largest one any count needs; CTAs beyond the split find no tiles and leave).
-template <int D, bool COUNTED>
-__global__ void __launch_bounds__(DEC_THREADS, DEC_CTAS_PER_SM) decode_kernel(const DecArgs a) {
-    constexpr int NR = D / 16;       // key operand registers per lane and item
+template <int D, int NQ, bool COUNTED>
+__global__ void __launch_bounds__(Shape<NQ>::THREADS, Shape<NQ>::CTAS_PER_SM) decode_kernel(const DecArgs a) {
+    using S = Shape<NQ>;
+    using WS = WarpScratch<D, NQ>;
+    constexpr int P = D / 32;        // nibble words of a key row per lane
     constexpr int MB = D / 16;       // 16-channel row blocks of the value side
-    constexpr int HALF = QAQ_TILE / 2;
-    constexpr uint32_t STAGE = WarpScratch<D>::STAGE;
+    constexpr int NP = (NQ + 1) / 2; // pairs of queries that share an instruction on the value side
+    constexpr int CPL = D / 32;      // channels per lane in the outlier sums of the values
+    constexpr uint32_t STAGE = WS::STAGE;
+    const float NEG = __int_as_float(0xff800000);
     extern __shared__ __align__(16) unsigned char smem_raw[];
-    DecSmem<D>& sm = *reinterpret_cast<DecSmem<D>*>(smem_raw);
+    DecSmem<D, NQ>& sm = *reinterpret_cast<DecSmem<D, NQ>*>(smem_raw);
     const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
     const int fg = lane >> 2, ft = lane & 3;
-    const unsigned lt = (1u << lane) - 1u;
-    WarpScratch<D>& ws = sm.ws[warp];
+    WS& ws = sm.ws[warp];
     const int T = COUNTED ? *a.d_count : a.T;
-    if (COUNTED && T < 1) return;
-    const int run = COUNTED ? plan_decode(a.BH, (T + QAQ_TILE - 1) / QAQ_TILE).run : a.run;
+    if (COUNTED && T < 1) {          // nothing cached: zeros
+        for (int bh = blockIdx.x; bh < a.BH; bh += gridDim.x)
+            if (tid < D) a.out[(size_t)bh * a.out_stride + tid] = 0.f;
+        return;
+    }
+    const int run = COUNTED ? plan_decode<NQ>(a.BH, (T + QAQ_TILE - 1) / QAQ_TILE).run : a.run;
 
+    uint32_t phase = 0;          // of the warp's two transaction barriers
+    bool first_seg = true;
 #pragma unroll 1
     for (int seg = 0; seg < 2; ++seg) {
     // this CTA's run of the flattened (b,h, tile) sequence; it touches at most two (b,h).  The block
@@ -183,459 +490,457 @@ __global__ void __launch_bounds__(DEC_THREADS, DEC_CTAS_PER_SM) decode_kernel(co
     const int tile_lo = max(flat_lo, bh * ntiles) - bh * ntiles, tile_hi = min(flat_hi, (bh + 1) * ntiles) - bh * ntiles;
     if (tile_lo >= tile_hi) continue;   // the same for every thread of the CTA
 
-    // ---- q: float copy, fixed-point byte digits per lane
-    float qmax = 0.f, qs = 0.f;
-    for (int d = tid; d < D; d += DEC_THREADS) {
-        const float f = __half2float(a.q[(size_t)bh * a.q_stride + d]);
-        sm.qf[d] = f;
-        qmax = fmaxf(qmax, fabsf(f));
-        qs += f;
-    }
-#pragma unroll
-    for (int o = 16; o > 0; o >>= 1) {
-        qmax = fmaxf(qmax, __shfl_xor_sync(0xFFFFFFFFu, qmax, o));
-        qs += __shfl_xor_sync(0xFFFFFFFFu, qs, o);
-    }
-    if (lane == 0) { sm.red[warp] = qmax; sm.red2[warp] = qs; }
-    for (int d = lane; d < D; d += 32) { ws.vcorr[0][d] = 0; ws.vcorr[1][d] = 0; }
-    for (int i = lane; i < QAQ_TILE; i += 32) { ws.kcorr[0][i] = 0; ws.kcorr[1][i] = 0; }
-    __syncthreads();
-    if (tid == 0) {
-        float m = 0.f, s = 0.f;
-        for (int w = 0; w < DEC_WARPS; ++w) { m = fmaxf(m, sm.red[w]); s += sm.red2[w]; }
-        sm.qscale = m / 32639.0f;        // |q| <= 32639 units: both byte digits of 256 * hi + lo stay signed bytes
-        sm.qsum = s;
-    }
-    __syncthreads();
-    const float qscale = sm.qscale, qsum = sm.qsum;
-    const float qinv = qscale > 0.f ? 1.0f / qscale : 0.f;
-    uint32_t qb[NR];             // column fg of the B operand: the high (fg = 0) or low (fg = 1) digit, zero otherwise
-#pragma unroll
-    for (int r = 0; r < NR; ++r) {
-        uint32_t v = 0;
-#pragma unroll
-        for (int i = 0; i < 4; ++i) {
-            int qi = __float2int_rn(sm.qf[4 * (ft * NR + r) + i] * qinv);
-            qi = max(-32639, min(32639, qi));
-            const int dg = fg == 0 ? ((qi + 128) >> 8) : qi;     // 256 * hi + lo with lo in [-128, 127]
-            v |= (uint32_t)(dg & 0xFF) << (8 * i);
-        }
-        qb[r] = fg < 2 ? v : 0u;
-    }
-
-    float X[MB][2];             // rows fg and fg + 8 of row block mb: this lane's share of the digit columns (summed over ft at the end)
-#pragma unroll
-    for (int mb = 0; mb < MB; ++mb) { X[mb][0] = 0.f; X[mb][1] = 0.f; }
-    // what the accumulator columns of this lane stand for: lane ft = 0 holds the digits 2^16 and 2^8, ft = 1 the units
-    const float dig0 = ft == 0 ? 65536.0f : (ft == 1 ? 1.0f : 0.f), dig1 = ft == 0 ? 256.0f : 0.f;
-    float m_run = __int_as_float(0xff800000), l_run = 0.f, lx_run = 0.f;   // lx: sum of the unperturbed p
-    float c_run = 0.f;       // per-lane part of sum_t p_t * (min_t + step_t/2) of the values
-    float vout[(D + 31) / 32];   // value-outlier corrections of channels lane, lane + 32, ...
-#pragma unroll
-    for (int k = 0; k < (D + 31) / 32; ++k) vout[k] = 0.f;
-
-    const size_t trow = (size_t)bh * a.ntiles_max;
-    const size_t mrow = (size_t)bh * a.tmax_pad;
+    const size_t mrow = (size_t)bh * a.tmax_pad + 2 * lane;
+    const uint4* tabK = a.k.tile + (size_t)bh * a.ntiles_max;
+    const uint4* tabV = a.v.tile + (size_t)bh * a.ntiles_max;
     const uint8_t* poolK = a.k.codes + (size_t)bh * a.pool_bytes;
     const uint8_t* poolV = a.v.codes + (size_t)bh * a.pool_bytes;
     const uint32_t* ogK = a.k.outl + (size_t)bh * a.ocap;
     const uint32_t* ogV = a.v.outl + (size_t)bh * a.ocap;
+    const uint32_t buf = smem_addr(ws.buf), bar = smem_addr(ws.bar);
 
-    // ---- tile metadata in registers: table words in lanes 0..7 (offset and length of the bytes, first entry and
-    //      length of the outlier list; keys in lanes 0..3, values in 4..7), min/max of tokens lane, lane+32.
-    //      Table entries that point outside the pool or the list are not followed (length 0).
-    //      The loads are only issued here; nothing looks at what they return before settle() does, a tile later.
-    struct Meta { uint32_t tb, mm[4]; };
+    // ---- tile metadata in registers: the table words (offset and length of the bytes, first entry and length of the
+    //      outlier list), min/max, widths and slots of tokens 2*lane, 2*lane+1
+    struct Meta { uint4 tk, tv; uint2 mk, mv; uint32_t bk, bv; };
     auto fetch_meta = [&](int tile) {
         Meta m;
-        m.tb = 0; m.mm[0] = m.mm[1] = m.mm[2] = m.mm[3] = 0;
+        m.tk = m.tv = make_uint4(0u, 0u, 0u, 0u); m.mk = m.mv = make_uint2(0u, 0u); m.bk = m.bv = 0;
         if (tile < tile_hi) {
-            if (lane < 8) {
-                const TensorStore& ts = (lane >= 4) ? a.v : a.k;
-                const uint32_t* tab = (lane & 2) ? ((lane & 1) ? ts.tile_ocnt : ts.tile_ooff) : ((lane & 1) ? ts.tile_nbytes : ts.tile_off);
-                m.tb = tab[trow + tile];
-            }
-            const size_t t0 = mrow + (size_t)tile * QAQ_TILE + lane;
-            m.mm[0] = a.k.mnmx[t0]; m.mm[1] = a.k.mnmx[t0 + 32]; m.mm[2] = a.v.mnmx[t0]; m.mm[3] = a.v.mnmx[t0 + 32];
+            m.tk = __ldg(tabK + tile); m.tv = __ldg(tabV + tile);
+            const size_t t0 = mrow + (size_t)tile * QAQ_TILE;
+            m.mk = __ldg(reinterpret_cast<const uint2*>(a.k.mnmx + t0)); m.mv = __ldg(reinterpret_cast<const uint2*>(a.v.mnmx + t0));
+            m.bk = __ldg(reinterpret_cast<const uint32_t*>(a.k.bs + t0)); m.bv = __ldg(reinterpret_cast<const uint32_t*>(a.v.bs + t0));
         }
         return m;
     };
-    // the table words of a tile as they are used: a length becomes 0 where offset and length point outside the pool
-    // or the list (lanes 2k, 2k+1 hold an offset and its length)
-    auto settle = [&](uint32_t tb) -> uint32_t {
-        const uint32_t other = __shfl_xor_sync(0xFFFFFFFFu, tb, 1);
-        const uint32_t first = (lane & 1) ? other : tb, len = (lane & 1) ? tb : other;
-        const bool bad = (lane & 2) ? ((size_t)first + len > a.ocap)
-                                    : ((first & 15u) || len < (uint32_t)qaqc::QAQ_TILE_HDR || (size_t)first + ((len + 15u) & ~15u) > a.pool_bytes);
-        return lane < 8 ? ((lane & 1) ? (bad ? 0u : len) : first) : 0u;
+    // how a tile lies in the buffer: bytes of the tile and of the piece of the outlier list that comes with it (from the
+    // 16-byte boundary before its first entry; what lies behind its last one belongs to the read-ahead margin of the
+    // list's capacity), both multiples of 16
+    struct Lay { uint32_t nb, lb; };
+    auto layout = [&](const uint4& tb) {
+        Lay l;
+        l.nb = (tb.y + 15u) & ~15u;
+        l.lb = tb.w ? (((tb.z & 3u) + min(tb.w, LIST_STAGED)) * 4u + 15u) & ~15u : 0u;
+        l.lb = min(l.lb, STAGE - l.nb);
+        return l;
     };
-    // copies nb bytes (a multiple of 16) of a tile to the staging buffer
-    auto stage = [&](uint8_t* dst, const uint8_t* src, uint32_t nb) {
-        unsigned sa = (unsigned)__cvta_generic_to_shared(dst) + lane * 16;
-        const uint8_t* g = src + lane * 16;
-#pragma unroll 1
-        for (uint32_t o = lane * 16; o < nb; o += 4 * 512, sa += 4 * 512, g += 4 * 512) {      // four copies per round
-#pragma unroll
-            for (int u = 0; u < 4; ++u)
-                if (o + 512u * u < nb) asm volatile("cp.async.cg.shared.global [%0], [%1], 16;\n" ::"r"(sa + 512u * u), "l"(g + 512 * u));
+    auto stage = [&](uint32_t dst, const Lay& l, const uint8_t* pool, const uint32_t* og, const uint4& tb, int x) {
+        if (lane == 0) {
+            bar_expect(bar + 8 * x, l.nb + l.lb);
+            if (l.nb) bulk_copy(dst, pool + tb.x, l.nb, bar + 8 * x);
+            if (l.lb) bulk_copy(dst + l.nb, og + (tb.z & ~3u), l.lb, bar + 8 * x);
         }
     };
-    // the first entries of a tile's outlier list, 4 bytes each, into the warp's scratch (part of the copy group open then)
-    // (lists of whole tiles start on 16-byte boundaries: four entries per copy, reading up to three entries past the
-    // list, which the capacity's read-ahead margin covers; a list that grew with an open tile may start anywhere)
-    auto stage_list = [&](uint32_t* dst, const uint32_t* src, uint32_t cnt) {
-        if (((uintptr_t)src & 15) == 0) {
-            if (lane < OL_STAGED / 4 && 4u * lane < cnt) cp_async<16>(dst + 4 * lane, src + 4 * lane);
-        } else {
-#pragma unroll
-            for (int k = 0; k < OL_STAGED / 32; ++k)
-                if (lane + 32 * k < cnt) {
-                    const unsigned sa = (unsigned)__cvta_generic_to_shared(dst + lane + 32 * k);
-                    asm volatile("cp.async.ca.shared.global [%0], [%1], 4;\n" ::"r"(sa), "l"(src + lane + 32 * k));
-                }
-        }
-    };
+
     int tile = tile_lo + warp;
     Meta cur = fetch_meta(tile);
-    Meta nxt = fetch_meta(tile + DEC_WARPS);
-    cur.tb = settle(cur.tb);
-    // what is staged: bytes (rounded up to 16) of the current keys / values in the buffer, 0 = read in place
-    uint32_t stK = 0, stV = 0;
-    if (tile < tile_hi) {
-        const uint32_t nbK = (__shfl_sync(0xFFFFFFFFu, cur.tb, 1) + 15u) & ~15u, nbV = (__shfl_sync(0xFFFFFFFFu, cur.tb, 5) + 15u) & ~15u;
-        if (nbK <= STAGE) { stK = nbK; stage(ws.buf, poolK + __shfl_sync(0xFFFFFFFFu, cur.tb, 0), nbK); }
-        stage_list(ws.olist[0], ogK + __shfl_sync(0xFFFFFFFFu, cur.tb, 2), __shfl_sync(0xFFFFFFFFu, cur.tb, 3));
-        cp_async_commit();
-        if (stK + nbV <= STAGE) { stV = nbV; stage(ws.buf + STAGE - nbV, poolV + __shfl_sync(0xFFFFFFFFu, cur.tb, 4), nbV); }
-        stage_list(ws.olist[1], ogV + __shfl_sync(0xFFFFFFFFu, cur.tb, 6), __shfl_sync(0xFFFFFFFFu, cur.tb, 7));
-        cp_async_commit();
-    }
+    if (lane == 0 && first_seg) { bar_init(bar); bar_init(bar + 8); asm volatile("fence.proxy.async.shared::cta;" ::: "memory"); }
 
-    for (; tile < tile_hi; tile += DEC_WARPS) {
-        const uint32_t offK = __shfl_sync(0xFFFFFFFFu, cur.tb, 0), nbK = __shfl_sync(0xFFFFFFFFu, cur.tb, 1);
-        const uint32_t ooK = __shfl_sync(0xFFFFFFFFu, cur.tb, 2), ocK = __shfl_sync(0xFFFFFFFFu, cur.tb, 3);
-        const uint32_t offV = __shfl_sync(0xFFFFFFFFu, cur.tb, 4), nbV = __shfl_sync(0xFFFFFFFFu, cur.tb, 5);
-        const uint32_t ooV = __shfl_sync(0xFFFFFFFFu, cur.tb, 6), ocV = __shfl_sync(0xFFFFFFFFu, cur.tb, 7);
-        const bool has_next = tile + DEC_WARPS < tile_hi;
-        const int t0 = tile * QAQ_TILE + lane;              // this lane's tokens: t0 and t0 + 32
-        const bool val0 = t0 < T, val1 = t0 + HALF < T;
-        const uint8_t* tK = stK ? ws.buf : poolK + offK;
-        const uint8_t* tV = stV ? ws.buf + STAGE - stV : poolV + offV;
-        cp_async_wait<1>();     // this tile's keys have landed (its values may still be in flight)
-        __syncwarp();
+    first_seg = false;
 
-        // ---- keys: widths, ranks of this lane's tokens in the sections, section sizes (from the tile's header)
-        int B[2][2];          // [tensor][token]
-        uint32_t rk[2][2];    // rank in section c in byte c
-        int n[2][4];
-        B[0][0] = B[0][1] = B[1][0] = B[1][1] = 0;
-        rk[0][0] = rk[0][1] = rk[1][0] = rk[1][1] = 0;
+    // ---- q: float copies, scales and sums (every warp for itself)
+    float qscale[NQ], qsum[NQ], qtop = 0.f;
 #pragma unroll
-        for (int c = 0; c < 4; ++c) {
-            const uint2 mk = nbK ? *reinterpret_cast<const uint2*>(tK + 8 * c) : make_uint2(0u, 0u);
-            if ((mk.x >> lane) & 1u) B[0][0] |= 8 >> c;
-            if ((mk.y >> lane) & 1u) B[0][1] |= 8 >> c;
-            const int n0 = __popc(mk.x);
-            n[0][c] = n0 + __popc(mk.y);
-            rk[0][0] |= (uint32_t)__popc(mk.x & lt) << (8 * c);
-            rk[0][1] |= (uint32_t)(n0 + __popc(mk.y & lt)) << (8 * c);
+    for (int j = 0; j < NQ; ++j) {
+        float qmax = 0.f, qs = 0.f;
+#pragma unroll
+        for (int i = 0; i < D / 32; ++i) {
+            const float f = __half2float(a.q[(size_t)bh * a.q_stride + j * D + lane + 32 * i]);
+            if (warp == 0) sm.qf[lane + 32 * i][j] = f;
+            qmax = fmaxf(qmax, fabsf(f));
+            qs += f;
         }
-        if (!val0) B[0][0] = 0;
-        if (!val1) B[0][1] = 0;
-        uint32_t kb[5];
-        qaqc::section_bases<D, false>(n[0], kb);
-        // a tile that does not hold the sections its masks ask for is not read: its tokens then count with their
-        // constant parts only
-        const bool okK = kb[4] <= nbK;
-        if (!okK) { n[0][0] = n[0][1] = n[0][2] = n[0][3] = 0; }
+        qmax = warp_max(qmax);
+        qsum[j] = warp_sum(qs);
+        qscale[j] = qmax / 32639.0f;             // |q| <= 32639 units: both byte digits of 256 * hi + lo stay signed bytes
+        qtop = fmaxf(qtop, qmax);
+    }
+    __syncwarp();
+    if (tile < tile_hi) stage(buf, layout(cur.tk), poolK, ogK, cur.tk, 0);
+    for (int i = lane; i < WS::VC * D; i += 32) (&ws.vcorr[0][0])[i] = 0;
+    for (int i = lane; i < NQ * D; i += 32) (&ws.macc[0][0])[i] = 0.f;
+    // ---- operand words of q for all lanes, one or two per thread: nibble word u of lane ln, its low (even r) or high
+    //      nibbles; column ln / 4: the high (even) or low (odd) digit of query ln / 8
+    for (int idx = tid; idx < 32 * 2 * P; idx += S::THREADS) {
+        const int ln = idx / (2 * P), r = idx % (2 * P), lg = ln >> 2, lt = ln & 3, jq = lg >> 1;
+        uint32_t v = 0;
+        if (jq < NQ) {
+            float qsc = qscale[0];
+#pragma unroll
+            for (int j = 1; j < NQ; ++j) if (jq == j) qsc = qscale[j];
+            const float qinv = qsc > 0.f ? 1.0f / qsc : 0.f;
+            // first channel: unit p = lt * P / 4, word (lt * P mod 4) + u of it
+            const int ch = 32 * (lt * P >> 2) + 8 * ((lt * P & 3) + (r >> 1)) + 4 * (r & 1);
+            const uint2 raw = __ldg(reinterpret_cast<const uint2*>(a.q + (size_t)bh * a.q_stride + jq * D + ch));
+#pragma unroll
+            for (int i = 0; i < 4; ++i) {
+                const uint32_t w = i < 2 ? raw.x : raw.y;
+                int qi = __float2int_rn(__half2float(__ushort_as_half((unsigned short)(w >> (16 * (i & 1))))) * qinv);
+                qi = max(-32639, min(32639, qi));
+                const int dg = (lg & 1) == 0 ? ((qi + 128) >> 8) : qi;     // 256 * hi + lo with lo in [-128, 127]
+                v |= (uint32_t)(dg & 0xFF) << (8 * i);
+            }
+        }
+        sm.qw[ln][r] = v;
+    }
+    __syncthreads();
+    uint32_t qa[P], qb[P];
+#pragma unroll
+    for (int u = 0; u < P; ++u) { qa[u] = sm.qw[lane][2 * u]; qb[u] = sm.qw[lane][2 * u + 1]; }
+    // digit rows of the value weights this lane feeds: columns 0..3 of the first query of a pair, 4..7 of the second
+    const bool wuse = NQ > 1 || fg < 4;
+    const uint32_t wrow = smem_addr(&ws.wts[0][NQ > 1 ? fg >> 2 : 0][fg & 3][4 * ft]);
 
-        // ---- per-token scalars of the keys
-        float stepK[2];
+    // The value sums of several tiles stay in integer accumulators (exact) as long as the tiles agree on the reference
+    // of the exponentials and on the size of one fixed-point unit; they are added to ws.macc when one of the two changes.
+    int acc[NP][MB][4];
+#pragma unroll
+    for (int pr = 0; pr < NP; ++pr)
+#pragma unroll
+        for (int mb = 0; mb < MB; ++mb) { acc[pr][mb][0] = 0; acc[pr][mb][1] = 0; acc[pr][mb][2] = 0; acc[pr][mb][3] = 0; }
+    int held = 0;                // tiles in the accumulators: a tile adds less than 2^22 (64 tokens, 255 * 255), 500 of them fit
+    float m_ref[NQ], wunit[NQ];  // exponentials are taken relative to this logit; weight of one fixed-point unit, a power of two
+    float l_run[NQ], c_run[NQ], lx_run = 0.f;       // over this lane's tokens: sum of p, of p * (min + step/2) of the values, of the unperturbed p
+#pragma unroll
+    for (int j = 0; j < NQ; ++j) { m_ref[j] = NEG; wunit[j] = 0.f; l_run[j] = 0.f; c_run[j] = 0.f; }
+    auto flush = [&]() {
+        // digits 2^24, 2^16, 2^8, 1: columns 0..3 (lanes ft = 0, 1) are the first query of a pair, columns 4..7 the second
+        const float d0 = (ft & 1) ? 256.0f : 16777216.0f, d1 = (ft & 1) ? 1.0f : 65536.0f;
+        __syncwarp();
+#pragma unroll
+        for (int pr = 0; pr < NP; ++pr) {
+            float un = wunit[2 * pr];
+            if constexpr (NQ > 1) { if (ft >= 2) un = wunit[2 * pr + 1]; }
+            float* row = ws.macc[NQ > 1 ? 2 * pr + (ft >> 1) : 0];
+#pragma unroll
+            for (int mb = 0; mb < MB; ++mb)
+#pragma unroll
+                for (int s2 = 0; s2 < 2; ++s2) {
+                    float v = fmaf((float)acc[pr][mb][2 * s2], d0, (float)acc[pr][mb][2 * s2 + 1] * d1);
+                    v += __shfl_xor_sync(0xFFFFFFFFu, v, 1);
+                    if ((ft & 1) == 0 && (NQ > 1 || ft == 0)) row[v_channel<D>(mb, fg, s2)] += v * (v_high<D>(mb) ? 0.0625f * un : un);
+                    acc[pr][mb][2 * s2] = 0; acc[pr][mb][2 * s2 + 1] = 0;
+                }
+        }
+        held = 0;
+        __syncwarp();
+    };
+
+#pragma unroll 1
+    for (; tile < tile_hi; tile += S::WARPS) {
+        const Lay lk = layout(cur.tk), lv = layout(cur.tv);
+        const uint32_t tV = buf + STAGE - lv.nb - lv.lb;
+        // the tile before is done with: this tile's values come in behind its keys, if there is room
+        const bool besideV = lk.nb + lk.lb + lv.nb + lv.lb <= STAGE;
+        if (besideV) stage(tV, lv, poolV, ogV, cur.tv, 1);
+        const Meta nxt = fetch_meta(tile + S::WARPS);
+        const bool has_next = tile + S::WARPS < tile_hi;
+        const int t0 = tile * QAQ_TILE + 2 * lane;              // this lane's tokens: t0 and t0 + 1
+        const bool val[2] = {t0 < T, t0 + 1 < T};
+        int B[2];
+        float stepK[2], midK[2];
 #pragma unroll
         for (int j = 0; j < 2; ++j) {
-            const bool v = j ? val1 : val0;
-            const uint32_t mk = cur.mm[j];
-            const float kmn = __half2float(__ushort_as_half((unsigned short)(mk & 0xFFFF)));
-            const float kmx = __half2float(__ushort_as_half((unsigned short)(mk >> 16)));
-            stepK[j] = v ? qaqc::step_of(kmn, kmx, B[0][j]) : 0.f;
-            ws.midK[lane + HALF * j] = v ? fmaf(0.5f, stepK[j], kmn) : 0.f;
+            const uint32_t mm = j ? cur.mk.y : cur.mk.x;
+            B[j] = val[j] ? (int)((cur.bk >> (16 * j)) & 15u) : 0;
+            const float mn = __half2float(__ushort_as_half((unsigned short)(mm & 0xFFFF))), mx = __half2float(__ushort_as_half((unsigned short)(mm >> 16)));
+            stepK[j] = val[j] ? qaqc::step_of(mn, mx, B[j]) : 0.f;
+            midK[j] = val[j] ? fmaf(0.5f, stepK[j], mn) : 0.f;
         }
+        *reinterpret_cast<float2*>(&ws.mid[2 * lane]) = make_float2(midK[0], midK[1]);
+        bool landed = bar_wait(bar, phase & 1u);
         __syncwarp();
 
-        // ---- K: integer dot products per section
-        k_section<D, 8>(tK + kb[0], n[0][0], ws.dotw[0], qb, fg, ft);
-        k_section<D, 4>(tK + kb[1], n[0][1], ws.dotw[1], qb, fg, ft);
-        k_section<D, 2>(tK + kb[2], n[0][2], ws.dotw[2], qb, fg, ft);
-        k_section<D, 1>(tK + kb[3], n[0][3], ws.dotw[3], qb, fg, ft);
-        // key outliers: q_ch * (x - mid) per token
-        auto k_outlier = [&](uint32_t v) {
-            const int tok = (v >> 24) & (QAQ_TILE - 1);
-            const float tm = sm.qf[(v >> 16) & (D - 1)] * (__half2float(__ushort_as_half((unsigned short)(v & 0xFFFF))) - ws.midK[tok]);
-            outlier_add(&ws.kcorr[0][tok], &ws.kcorr[1][tok], tm);
-        };
-#pragma unroll
-        for (int k = 0; k < OL_STAGED / 32; ++k)         // the staged entries: independent chains, side by side
-            if (lane + 32u * k < ocK) k_outlier(ws.olist[0][lane + 32 * k]);
+        // ---- K: integer dot products, list by list
+        {
+            uint4 h = *reinterpret_cast<const uint4*>(ws.buf);
+            if (!cur.tk.y || !landed) h = make_uint4(0u, 0u, 0u, 0u);
 #pragma unroll 1
-        for (uint32_t e = lane + OL_STAGED; e < ocK; e += 32) k_outlier(__ldg(ogK + ooK + e));
+            for (int pass = 0; pass < (h.y ? 2 : 1); ++pass) {
+                const Lists l = lists_of<P>(h, pass);
+                uint32_t dots = smem_addr(&ws.dot[pass][0][0]);
+                k_list<D, 4, NQ>(buf + l.o4, l.n4, dots, qa, qb, fg, ft);
+                dots += l.n4 * 4 * NQ;
+                k_list<D, 3, NQ>(buf + l.o3, l.n3, dots, qa, qb, fg, ft);
+                dots += l.n3 * 4 * NQ;
+                k_list<D, 2, NQ>(buf + l.o2, l.n2, dots, qa, qb, fg, ft);
+                dots += l.n2 * 4 * NQ;
+                k_list<D, 1, NQ>(buf + l.o1, l.n1, dots, qa, qb, fg, ft);
+            }
+        }
+        // ---- key outliers: q_ch * (x - mid) per token
+        float kunit = 0.f;          // > 0: the corrections are one word in this unit; 0: none; < 0: two words
+        if (cur.tk.w && landed) {
+            const uint32_t oc = cur.tk.w, sc = min(min(oc, LIST_STAGED), lk.lb / 4 - (cur.tk.z & 3u));       // entries, of which staged
+            const uint32_t* list = reinterpret_cast<const uint32_t*>(ws.buf + lk.nb) + (cur.tk.z & 3u);
+#pragma unroll
+            for (int i = 0; i < NQ; ++i) *reinterpret_cast<uint4*>(&ws.kcorr[i][0][4 * lane]) = make_uint4(0u, 0u, 0u, 0u);
+            // largest value of the tile: outliers and ranges
+            uint32_t top = max(max(cur.mk.x & 0x7FFFu, (cur.mk.x >> 16) & 0x7FFFu), max(cur.mk.y & 0x7FFFu, (cur.mk.y >> 16) & 0x7FFFu));
+#pragma unroll 4
+            for (uint32_t e = lane; e < sc; e += 32) top = max(top, list[e] & 0x7FFFu);
+            top = sc == oc ? __reduce_max_sync(0xFFFFFFFFu, top) : SMALL_MAX + 1;
+            auto entry = [&](uint32_t v, int& tok, float& dx) {
+                tok = (v >> 24) & (QAQ_TILE - 1);
+                dx = __half2float(__ushort_as_half((unsigned short)(v & 0xFFFF))) - ws.mid[tok];
+                return &sm.qf[(v >> 16) & (D - 1)][0];
+            };
+            __syncwarp();
+            if (top <= SMALL_MAX) {
+                float inv;
+                fixed_unit(qtop * 2.0f * __half2float(__ushort_as_half((unsigned short)top)), inv, kunit);
+#pragma unroll 4
+                for (uint32_t e = lane; e < sc; e += 32) {
+                    int tok; float dx;
+                    const float* qv = entry(list[e], tok, dx);
+                    dx *= inv;
+#pragma unroll
+                    for (int j = 0; j < NQ; ++j) atomicAdd(&ws.kcorr[j][0][tok], __float2int_rn(qv[j] * dx));
+                }
+            } else {
+                kunit = -1.0f;
+#pragma unroll 1
+                for (uint32_t e = lane; e < oc; e += 32) {
+                    int tok; float dx;
+                    const float* qv = entry(e < sc ? list[e] : __ldg(ogK + cur.tk.z + e), tok, dx);
+#pragma unroll
+                    for (int j = 0; j < NQ; ++j) wide_add(&ws.kcorr[j][0][tok], &ws.kcorr[j][1][tok], qv[j] * dx);
+                }
+            }
+        }
+        __syncwarp();
+        // ---- logits of this lane's tokens
+        float lg[NQ][2];
+#pragma unroll
+        for (int i = 0; i < 2; ++i) {
+            const int sl = (cur.bk >> (16 * i + 8)) & (QAQ_TILE - 1);
+#pragma unroll
+            for (int j = 0; j < NQ; ++j) {
+                int dot = B[i] ? ws.dot[0][sl][j] : 0;
+                if (B[i] > 4) dot += ws.dot[1][sl][j] << 4;
+                float kc = 0.f;
+                if (kunit > 0.f) kc = (float)ws.kcorr[j][0][2 * lane + i] * kunit;
+                else if (kunit < 0.f) kc = wide_sum(ws.kcorr[j][0][2 * lane + i], ws.kcorr[j][1][2 * lane + i]);
+                const float qk = fmaf(qscale[j] * stepK[i], (float)dot, fmaf(midK[i], qsum[j], kc));
+                lg[j][i] = val[i] ? a.scale * qk : NEG;
+            }
+            if (NQ == 1 && a.scores && val[i]) a.scores[(size_t)bh * a.scores_stride + t0 + i] = lg[0][i];
+        }
         __syncwarp();
         // ---- the front of the buffer is free: start the copy of the next tile's keys (beside this tile's values)
-        uint32_t stKn = 0;
-        nxt.tb = settle(nxt.tb);       // fetched a tile ago
-        if (has_next) {
-            const uint32_t nb = (__shfl_sync(0xFFFFFFFFu, nxt.tb, 1) + 15u) & ~15u;
-            if (nb + stV <= STAGE) { stKn = nb; stage(ws.buf, poolK + __shfl_sync(0xFFFFFFFFu, nxt.tb, 0), nb); }
-            stage_list(ws.olist[0], ogK + __shfl_sync(0xFFFFFFFFu, nxt.tb, 2), __shfl_sync(0xFFFFFFFFu, nxt.tb, 3));
-        }
-        cp_async_commit();
+        if (!besideV) stage(tV, lv, poolV, ogV, cur.tv, 1);
+        const Lay ln = layout(nxt.tk);
+        const bool besideK = ln.nb + ln.lb + lv.nb + lv.lb <= STAGE;
+        if (has_next && besideK) stage(buf, ln, poolK, ogK, nxt.tk, 0);
 
-        // ---- logits of this lane's tokens; running max / sum
-        float lg[2];
-#pragma unroll
-        for (int j = 0; j < 2; ++j) {
-            int dot = 0;
-#pragma unroll
-            for (int c = 0; c < 4; ++c) {
-                const int w = 8 >> c;
-                if ((B[0][j] & w) && okK) dot += ws.dotw[c][(rk[0][j] >> (8 * c)) & 0xFF] << (B[0][j] & (w - 1));
-            }
-            lg[j] = __int_as_float(0xff800000);
-            const int tk = lane + HALF * j;
-            const int kh = ws.kcorr[0][tk], kl = ws.kcorr[1][tk];
-            if (kh | kl) { ws.kcorr[0][tk] = 0; ws.kcorr[1][tk] = 0; }
-            if (j ? val1 : val0) {
-                const float qk = fmaf(qscale * stepK[j], (float)dot, fmaf(ws.midK[tk], qsum, outlier_sum(kh, kl)));
-                lg[j] = a.scale * qk;
-                if (a.scores) a.scores[(size_t)bh * a.scores_stride + t0 + HALF * j] = lg[j];
-            }
-        }
-        float m = fmaxf(lg[0], lg[1]);
-#pragma unroll
-        for (int o = 16; o > 0; o >>= 1) m = fmaxf(m, __shfl_xor_sync(0xFFFFFFFFu, m, o));
-        const float m_new = fmaxf(m_run, m);
-        const float alpha = __expf(m_run - m_new);   // 0 on the first tile (m_run = -inf)
-        m_run = m_new;
-        if (alpha != 1.0f) {
-#pragma unroll
-            for (int mb = 0; mb < MB; ++mb) { X[mb][0] *= alpha; X[mb][1] *= alpha; }
-            c_run *= alpha;
-#pragma unroll
-            for (int k = 0; k < (D + 31) / 32; ++k) vout[k] *= alpha;
-        }
-        cp_async_wait<1>();     // this tile's values have landed
-        __syncwarp();
-
-        // ---- values: widths, ranks, section sizes; per-token scalars
-#pragma unroll
-        for (int c = 0; c < 4; ++c) {
-            const uint2 mv = nbV ? *reinterpret_cast<const uint2*>(tV + 8 * c) : make_uint2(0u, 0u);
-            if ((mv.x >> lane) & 1u) B[1][0] |= 8 >> c;
-            if ((mv.y >> lane) & 1u) B[1][1] |= 8 >> c;
-            const int n0 = __popc(mv.x);
-            n[1][c] = n0 + __popc(mv.y);
-            rk[1][0] |= (uint32_t)__popc(mv.x & lt) << (8 * c);
-            rk[1][1] |= (uint32_t)(n0 + __popc(mv.y & lt)) << (8 * c);
-        }
-        if (!val0) B[1][0] = 0;
-        if (!val1) B[1][1] = 0;
-        uint32_t vb[5];
-        qaqc::section_bases<D, true>(n[1], vb);
-        const bool okV = vb[4] <= nbV;
-        if (!okV) { n[1][0] = n[1][1] = n[1][2] = n[1][3] = 0; }
+        // ---- p relative to a reference somewhat above the largest logit, which is moved only when a logit exceeds it (so
+        //      p never exceeds 1), and value weights p * step as fixed point of up to 28 bits.  (A token's step falls with
+        //      its width, so next to a 2-bit token an 8-bit token of the same p has a weight 64 times smaller.)  p is
+        //      replaced by what the rounded weight stands for, so that the codes, the constant part and the softmax
+        //      denominator all see the same (slightly perturbed) probability.  The largest weight of every tile takes 21
+        //      bits or more: the unit stays while it takes between 2^21 and 2^28 units, and is set so that it takes 2^24
+        //      to 2^25.
         float stepV[2], midV[2];
 #pragma unroll
-        for (int j = 0; j < 2; ++j) {
-            const bool v = j ? val1 : val0;
-            const uint32_t mv = cur.mm[2 + j];
-            const float vmn = __half2float(__ushort_as_half((unsigned short)(mv & 0xFFFF)));
-            const float vmx = __half2float(__ushort_as_half((unsigned short)(mv >> 16)));
-            stepV[j] = v ? qaqc::step_of(vmn, vmx, B[1][j]) : 0.f;
-            midV[j] = v ? fmaf(0.5f, stepV[j], vmn) : 0.f;
-            ws.midV[lane + HALF * j] = midV[j];
+        for (int i = 0; i < 2; ++i) {
+            const uint32_t mm = i ? cur.mv.y : cur.mv.x;
+            B[i] = val[i] ? (int)((cur.bv >> (16 * i)) & 15u) : 0;
+            const float mn = __half2float(__ushort_as_half((unsigned short)(mm & 0xFFFF))), mx = __half2float(__ushort_as_half((unsigned short)(mm >> 16)));
+            stepV[i] = val[i] ? qaqc::step_of(mn, mx, B[i]) : 0.f;
+            midV[i] = val[i] ? fmaf(0.5f, stepV[i], mn) : 0.f;
         }
-        // ---- value weights p * step * 2^shift as 22-bit fixed point with one scale for the tile (a token's step
-        //      falls with its width, so next to a 2-bit token an 8-bit token of the same p has a weight 64 times
-        //      smaller: 16 bits would leave it about 10).  The weight of the token's lowest piece is rounded once;
-        //      the other pieces use exact multiples of it, and p is replaced by what the rounded weight stands for,
-        //      so that the pieces, the constant part and the softmax denominator all see the same (slightly
-        //      perturbed) probability.
-        float pe[2], wf[2];
-        int top[2];
-        float wmax = 0.f;
+        float alpha[NQ], wnew[NQ];
+        bool wok[NQ], any_w = false, change = held == 500;
 #pragma unroll
-        for (int j = 0; j < 2; ++j) {
-            pe[j] = __expf(lg[j] - m_new);           // 0 for slots beyond T
-            wf[j] = pe[j] * stepV[j];
-            const int Bv = B[1][j];
-            top[j] = Bv ? Bv - (1 << (31 - __clz(Bv))) : 0;      // shift of the widest piece
-            wmax = fmaxf(wmax, wf[j] * __int_as_float((127 + top[j]) << 23));
+        for (int j = 0; j < NQ; ++j) {
+            const float m = warp_max(fmaxf(lg[j][0], lg[j][1]));
+            alpha[j] = 1.0f;
+            if (m > m_ref[j]) {
+                alpha[j] = __expf(m_ref[j] - (m + 3.0f));       // 0 on the first tile
+                m_ref[j] = m + 3.0f;
+                change = true;
+            }
+            lg[j][0] = __expf(lg[j][0] - m_ref[j]);              // from here on: p (0 for slots beyond T)
+            lg[j][1] = __expf(lg[j][1] - m_ref[j]);
+            const float wmax = warp_max(fmaxf(B[0] ? lg[j][0] * stepV[0] : 0.f, B[1] ? lg[j][1] * stepV[1] : 0.f));
+            const int wex = (__float_as_int(wmax) >> 23) & 0xFF;
+            wok[j] = wex > 28 && wex < 255 && cur.tv.y;             // zero, tiny or non-finite weights: the codes add nothing
+            any_w = any_w || wok[j];
+            wnew[j] = wunit[j];
+            if (wok[j] && !(wmax >= 2097152.0f * wunit[j] && wmax < 268435440.0f * wunit[j])) {
+                wnew[j] = __int_as_float((wex - 24) << 23);
+                change = true;
+            }
         }
+        if (change) {
+            if (held) flush();
 #pragma unroll
-        for (int o = 16; o > 0; o >>= 1) wmax = fmaxf(wmax, __shfl_xor_sync(0xFFFFFFFFu, wmax, o));
-        // wmax < 2^(ex-126): one unit = 2^(ex-126-22) keeps every shifted weight at or below 2^22
-        const int wex = (__float_as_int(wmax) >> 23) & 0xFF;
-        const bool wok = wex > 24 && wex < 255 && okV;             // zero, tiny or non-finite weights: the pieces add nothing
-        const float wunit = wok ? __int_as_float((wex - 21) << 23) : 0.f;
-        const float winv = wok ? __int_as_float((254 - (wex - 21)) << 23) : 0.f;
-        float s = 0.f, sx = 0.f;
+            for (int j = 0; j < NQ; ++j) {
+                wunit[j] = wnew[j];
+                if (alpha[j] != 1.0f) {
 #pragma unroll
-        for (int j = 0; j < 2; ++j) {
-            const int Bv = B[1][j];
-            uint32_t iw = (uint32_t)__float2int_rn(wf[j] * winv);
-            iw = min(iw, 0x7F0000u >> top[j]);       // the three balanced byte digits of a shifted weight stay signed bytes
-            float p = pe[j];
-            if (stepV[j] > 0.f && wok) p = __fdividef((float)iw * wunit, stepV[j]);
-            uint8_t* wbytes = reinterpret_cast<uint8_t*>(ws.wts);
-#pragma unroll
-            for (int c = 0; c < 4; ++c) {
-                const int w = 8 >> c;
-                if (Bv & w) {
-                    const uint32_t r = (rk[1][j] >> (8 * c)) & 0xFF, wt = iw << (Bv & (w - 1));
-                    // wt = 65536 * d2 + 256 * d1 + d0 with d1, d0 in [-128, 127]
-                    const uint32_t r1 = (wt + 128u) >> 8, r2 = (r1 + 128u) >> 8;
-                    uint8_t* gp = wbytes + c * (QAQ_TILE / 4) * 16 + (r >> 2) * 16 + (r & 3);
-                    gp[0] = (uint8_t)r2;
-                    gp[4] = (uint8_t)r1;
-                    gp[8] = (uint8_t)wt;
+                    for (int k = 0; k < CPL; ++k) ws.macc[j][lane + 32 * k] *= alpha[j];
+                    c_run[j] *= alpha[j]; l_run[j] *= alpha[j];
+                    if (NQ == 1) lx_run *= alpha[j];
                 }
             }
-            c_run = fmaf(p, midV[j], c_run);
-            s += p; sx += pe[j];
-            ws.p[lane + HALF * j] = p;
         }
 #pragma unroll
-        for (int o = 16; o > 0; o >>= 1) {
-            s += __shfl_xor_sync(0xFFFFFFFFu, s, o);
-            sx += __shfl_xor_sync(0xFFFFFFFFu, sx, o);
+        for (int j = 0; j < NQ; ++j) {
+            const float winv = wok[j] ? __int_as_float((254 << 23) - __float_as_int(wunit[j])) : 0.f;       // 1 / wunit
+            float2 pm[2];
+#pragma unroll
+            for (int i = 0; i < 2; ++i) {
+                const uint32_t iw = __float2uint_rn(lg[j][i] * stepV[i] * winv);
+                float p = lg[j][i];
+                if (stepV[i] > 0.f && wok[j] && B[i]) p = __fdividef((float)iw * wunit[j], stepV[i]);
+                uint8_t* gp = &ws.wts[0][j][0][(cur.bv >> (16 * i + 8)) & (QAQ_TILE - 1)];
+                if (B[i]) {
+                    gp[0] = (uint8_t)(iw >> 24);
+                    gp[WS::WROW] = (uint8_t)(iw >> 16);
+                    gp[2 * WS::WROW] = (uint8_t)(iw >> 8);
+                    gp[3 * WS::WROW] = (uint8_t)iw;
+                }
+                if (B[i] > 4) {                      // 16 times the weight, for the bits above the low four
+                    gp += 4 * NQ * WS::WROW;
+                    gp[0] = (uint8_t)(iw >> 20);
+                    gp[WS::WROW] = (uint8_t)(iw >> 12);
+                    gp[2 * WS::WROW] = (uint8_t)(iw >> 4);
+                    gp[3 * WS::WROW] = (uint8_t)(iw << 4);
+                }
+                pm[i] = make_float2(p, p * midV[i]);
+                c_run[j] += pm[i].y;
+                l_run[j] += p;
+                if (NQ == 1) lx_run += lg[j][i];
+            }
+            *reinterpret_cast<float4*>(&ws.tok[j][2 * lane]) = make_float4(pm[0].x, pm[0].y, pm[1].x, pm[1].y);
         }
-        l_run = l_run * alpha + s;
-        lx_run = lx_run * alpha + sx;
+        landed = bar_wait(bar + 8, phase & 1u) && landed;     // this tile's values are there
         __syncwarp();
 
-        // ---- V: integer weighted sums per section, added to the binary32 accumulators once per tile
-        if (wok) {
-            int acc[MB][4];
-#pragma unroll
-            for (int mb = 0; mb < MB; ++mb) { acc[mb][0] = 0; acc[mb][1] = 0; acc[mb][2] = 0; acc[mb][3] = 0; }
-            v_section<D, 8>(tV + vb[0], (n[1][0] + 3) >> 2, ws.wts[0], acc, fg, ft);
-            v_section<D, 4>(tV + vb[1], (n[1][1] + 3) >> 2, ws.wts[1], acc, fg, ft);
-            v_section<D, 2>(tV + vb[2], (n[1][2] + 3) >> 2, ws.wts[2], acc, fg, ft);
-            v_section<D, 1>(tV + vb[3], (n[1][3] + 3) >> 2, ws.wts[3], acc, fg, ft);
-#pragma unroll
-            for (int mb = 0; mb < MB; ++mb) {
-                X[mb][0] = fmaf(fmaf((float)acc[mb][0], dig0, (float)acc[mb][1] * dig1), wunit, X[mb][0]);
-                X[mb][1] = fmaf(fmaf((float)acc[mb][2], dig0, (float)acc[mb][3] * dig1), wunit, X[mb][1]);
-            }
-        }
-        // value outliers: p_t * (v - mid) per channel
-        auto v_outlier = [&](uint32_t v) {
-            const int tok = (v >> 24) & (QAQ_TILE - 1), ch = (v >> 16) & (D - 1);
-            const float tm = ws.p[tok] * (__half2float(__ushort_as_half((unsigned short)(v & 0xFFFF))) - ws.midV[tok]);
-            outlier_add(&ws.vcorr[0][ch], &ws.vcorr[1][ch], tm);
-        };
-#pragma unroll
-        for (int k = 0; k < OL_STAGED / 32; ++k)
-            if (lane + 32u * k < ocV) v_outlier(ws.olist[1][lane + 32 * k]);
+        // ---- V: integer weighted sums, list by list
+        if (any_w && landed) {
+            const uint4 h = *reinterpret_cast<const uint4*>(ws.buf + STAGE - lv.nb - lv.lb);
 #pragma unroll 1
-        for (uint32_t e = lane + OL_STAGED; e < ocV; e += 32) v_outlier(__ldg(ogV + ooV + e));
-        __syncwarp();
-        if (ocV) {
+            for (int pass = 0; pass < (h.y ? 2 : 1); ++pass) {
+                const Lists l = lists_of<D / 8>(h, pass);
+                uint32_t wt = wrow + pass * 4 * NQ * WS::WROW;
+                v_list<D, 4, NQ>(tV + l.o4, l.n4, wt, wuse, acc, fg, ft);
+                wt += 4 * l.n4;
+                v_list<D, 3, NQ>(tV + l.o3, l.n3, wt, wuse, acc, fg, ft);
+                wt += 4 * l.n3;
+                v_list<D, 2, NQ>(tV + l.o2, l.n2, wt, wuse, acc, fg, ft);
+                wt += 4 * l.n2;
+                v_list<D, 1, NQ>(tV + l.o1, l.n1, wt, wuse, acc, fg, ft);
+            }
+            ++held;
+        }
+        // ---- value outliers: p_t * (v - mid) per channel
+        if (cur.tv.w && landed) {
+            const uint32_t oc = cur.tv.w, sc = min(min(oc, LIST_STAGED), lv.lb / 4 - (cur.tv.z & 3u));
+            const uint32_t* list = reinterpret_cast<const uint32_t*>(ws.buf + STAGE - lv.lb) + (cur.tv.z & 3u);
+            uint32_t top = max(max(cur.mv.x & 0x7FFFu, (cur.mv.x >> 16) & 0x7FFFu), max(cur.mv.y & 0x7FFFu, (cur.mv.y >> 16) & 0x7FFFu));
+#pragma unroll 4
+            for (uint32_t e = lane; e < sc; e += 32) top = max(top, list[e] & 0x7FFFu);
+            top = sc == oc ? __reduce_max_sync(0xFFFFFFFFu, top) : SMALL_MAX + 1;
+            if (top <= SMALL_MAX) {
+                float inv[NQ], unit[NQ];
 #pragma unroll
-            for (int k = 0; k < (D + 31) / 32; ++k) {
-                const int d = lane + 32 * k;
-                if (d < D) {
-                    const int h = ws.vcorr[0][d], l = ws.vcorr[1][d];
-                    if (h | l) { vout[k] += outlier_sum(h, l); ws.vcorr[0][d] = 0; ws.vcorr[1][d] = 0; }
+                for (int j = 0; j < NQ; ++j)
+                    fixed_unit(warp_max(fmaxf(lg[j][0], lg[j][1])) * 2.5f * __half2float(__ushort_as_half((unsigned short)top)), inv[j], unit[j]);
+#pragma unroll 4
+                for (uint32_t e = lane; e < sc; e += 32) {
+                    const uint32_t v = list[e];
+                    const int tk = (v >> 24) & (QAQ_TILE - 1), ch = (v >> 16) & (D - 1);
+                    const float x = __half2float(__ushort_as_half((unsigned short)(v & 0xFFFF)));
+#pragma unroll
+                    for (int j = 0; j < NQ; ++j) {
+                        const float2 pm = ws.tok[j][tk];
+                        atomicAdd(&ws.vcorr[j][ch], __float2int_rn(fmaf(x, pm.x, -pm.y) * inv[j]));
+                    }
+                }
+                __syncwarp();
+#pragma unroll
+                for (int j = 0; j < NQ; ++j)
+#pragma unroll
+                    for (int k = 0; k < CPL; ++k) {
+                        const int d = lane + 32 * k;
+                        ws.macc[j][d] += (float)ws.vcorr[j][d] * unit[j];
+                        ws.vcorr[j][d] = 0;
+                    }
+            } else {
+#pragma unroll 1
+                for (int j = 0; j < NQ; ++j) {
+#pragma unroll 1
+                    for (uint32_t e = lane; e < oc; e += 32) {
+                        const uint32_t v = e < sc ? list[e] : __ldg(ogV + cur.tv.z + e);
+                        const int tk = (v >> 24) & (QAQ_TILE - 1), ch = (v >> 16) & (D - 1);
+                        const float2 pm = ws.tok[j][tk];
+                        wide_add(&ws.vcorr[0][ch], &ws.vcorr[1][ch], fmaf(__half2float(__ushort_as_half((unsigned short)(v & 0xFFFF))), pm.x, -pm.y));
+                    }
+                    __syncwarp();
+#pragma unroll
+                    for (int k = 0; k < CPL; ++k) {
+                        const int d = lane + 32 * k;
+                        ws.macc[j][d] += wide_sum(ws.vcorr[0][d], ws.vcorr[1][d]);
+                        ws.vcorr[0][d] = 0; ws.vcorr[1][d] = 0;
+                    }
+                    __syncwarp();
                 }
             }
         }
         __syncwarp();
-        // ---- the back of the buffer is free: start the copy of the next tile's values (beside its keys)
-        uint32_t stVn = 0;
-        if (has_next) {
-            const uint32_t nb = (__shfl_sync(0xFFFFFFFFu, nxt.tb, 5) + 15u) & ~15u;
-            if (nb + stKn <= STAGE) { stVn = nb; stage(ws.buf + STAGE - nb, poolV + __shfl_sync(0xFFFFFFFFu, nxt.tb, 4), nb); }
-            stage_list(ws.olist[1], ogV + __shfl_sync(0xFFFFFFFFu, nxt.tb, 6), __shfl_sync(0xFFFFFFFFu, nxt.tb, 7));
-        }
-        cp_async_commit();
-        stK = stKn; stV = stVn;
+        if (has_next && !besideK) stage(buf, ln, poolK, ogK, nxt.tk, 0);
+        if (!landed) atomicMax(a.status, (int)QAQ_ERR_CUDA);
+        phase ^= 1u;
         cur = nxt;
-        nxt = fetch_meta(tile + 2 * DEC_WARPS);
     }
-    cp_async_wait<0>();
+    if (held) flush();
 
-    // ---- warp result: the four lanes ft of a group hold the digit columns of the same channels
-    float cs = c_run;
+    // ---- warp result
 #pragma unroll
-    for (int o = 16; o > 0; o >>= 1) cs += __shfl_xor_sync(0xFFFFFFFFu, cs, o);
-#pragma unroll
-    for (int k = 0; k < (D + 31) / 32; ++k)
-        if (lane + 32 * k < D) sm.macc[warp][lane + 32 * k] = vout[k] + cs;
-    __syncwarp();
-#pragma unroll
-    for (int mb = 0; mb < MB; ++mb)
-#pragma unroll
-        for (int s2 = 0; s2 < 2; ++s2) {
-            float v = X[mb][s2];
-            v += __shfl_xor_sync(0xFFFFFFFFu, v, 1);
-            v += __shfl_xor_sync(0xFFFFFFFFu, v, 2);
-            const int ch = (D / 8) * fg + 2 * mb + s2;     // row fg + 8*s2 of row block mb
-            if (ft == 0) sm.macc[warp][ch] += v;
-        }
-    if (lane == 0) { sm.mm[warp] = m_run; sm.ml[warp] = l_run; sm.mlx[warp] = lx_run; }
+    for (int j = 0; j < NQ; ++j) {
+        const float l = warp_sum(l_run[j]), cs = warp_sum(c_run[j]);
+        if (lane == 0) { sm.mm[warp][j] = m_ref[j]; sm.ml[warp][j] = l; sm.cs[warp][j] = cs; }
+    }
+    if (NQ == 1) {
+        const float lx = warp_sum(lx_run);
+        if (lane == 0) sm.mlx[warp] = lx;
+    }
     __syncthreads();
     // ---- merge the warps (log-sum-exp) into this segment's partial
-    float M = __int_as_float(0xff800000);
+    const bool alone = tile_hi - tile_lo == ntiles;        // the whole (b,h) in this CTA: nothing to merge with
+#pragma unroll 1
+    for (int j = 0; j < NQ; ++j) {
+        float M = NEG;
 #pragma unroll
-    for (int w = 0; w < DEC_WARPS; ++w) M = fmaxf(M, sm.mm[w]);
-    float* dst = a.part + (size_t)(2 * cta + seg) * (D + 3);
-    float L = 0.f, LX = 0.f;
-    float wgt[DEC_WARPS];
+        for (int i = 0; i < S::WARPS; ++i) M = fmaxf(M, sm.mm[i][j]);
+        float L = 0.f, LX = 0.f, x = 0.f;
 #pragma unroll
-    for (int w = 0; w < DEC_WARPS; ++w) {
-        wgt[w] = (sm.mm[w] == __int_as_float(0xff800000)) ? 0.f : __expf(sm.mm[w] - M);
-        L = fmaf(wgt[w], sm.ml[w], L);
-        LX = fmaf(wgt[w], sm.mlx[w], LX);
+        for (int i = 0; i < S::WARPS; ++i) {
+            const float wgt = sm.mm[i][j] == NEG ? 0.f : __expf(sm.mm[i][j] - M);
+            L = fmaf(wgt, sm.ml[i][j], L);
+            if (NQ == 1) LX = fmaf(wgt, sm.mlx[i], LX);
+            if (tid < D) x = fmaf(wgt, sm.ws[i].macc[j][tid] + sm.cs[i][j], x);
+        }
+        float* dst = a.part + ((size_t)(2 * cta + seg) * NQ + j) * (D + 4);
+        if (alone) {
+            if (tid < D) a.out[(size_t)bh * a.out_stride + j * D + tid] = L > 0.f ? x / L : 0.f;
+            if (NQ == 1) {
+                if (a.ml && tid == 0) { a.ml[2 * bh] = M; a.ml[2 * bh + 1] = LX; }
+                if (a.scores && !a.ml) normalise_scores<S::THREADS>(a.scores + (size_t)bh * a.scores_stride, T, M, LX);
+            }
+        } else {
+            if (tid < D) __stcg(dst + tid, x);
+            if (tid == 0) __stcg(reinterpret_cast<float4*>(dst + D), make_float4(M, L, LX, 0.f));
+        }
     }
-    for (int d = tid; d < D; d += DEC_THREADS) {
-        float x = 0.f;
-#pragma unroll
-        for (int w = 0; w < DEC_WARPS; ++w) x = fmaf(wgt[w], sm.macc[w][d], x);
-        dst[d] = x;
-    }
-    if (tid == 0) { dst[D] = M; dst[D + 1] = L; dst[D + 2] = LX; }
+    if (!alone) finish_split<D, NQ>(a, sm, bh, ntiles, run, T);
     __syncthreads();   // the shared arrays are reused by the second segment
     }
 }
 
-// log-sum-exp merge of the partials -> X, and (max, sum) for the score row
-template <int D, bool COUNTED>
-__global__ void merge_kernel(const DecArgs a) {
-    const int bh = blockIdx.x, d = threadIdx.x;
-    const int T = COUNTED ? *a.d_count : a.T;
-    if (COUNTED && T < 1) { a.out[(size_t)bh * a.out_stride + d] = 0.f; return; }
-    const int ntiles = (T + QAQ_TILE - 1) / QAQ_TILE;
-    const int run = COUNTED ? plan_decode(a.BH, ntiles).run : a.run;
-    // the CTAs of decode_kernel whose runs meet this (b,h); a CTA's first segment has slot 0
-    const int c_lo = (bh * ntiles) / run, c_hi = ((bh + 1) * ntiles - 1) / run;
-    // only the first of them can have begun in the (b,h) before
-    auto slot = [&](int c) { return a.part + (size_t)(2 * c + (c * run < bh * ntiles ? 1 : 0)) * (D + 3); };
-    float M = __int_as_float(0xff800000);
-    for (int c = c_lo; c <= c_hi; ++c) M = fmaxf(M, slot(c)[D]);
-    float L = 0.f, LX = 0.f, x = 0.f;
-    for (int c = c_lo; c <= c_hi; ++c) {
-        const float* p = slot(c);
-        const float m = p[D];
-        if (m == __int_as_float(0xff800000)) continue;
-        const float w = __expf(m - M);
-        L = fmaf(w, p[D + 1], L);
-        LX = fmaf(w, p[D + 2], LX);
-        x = fmaf(w, p[d], x);
-    }
-    a.out[(size_t)bh * a.out_stride + d] = L > 0.f ? x / L : 0.f;
-    if (d == 0) { a.ml[2 * bh] = M; a.ml[2 * bh + 1] = LX; }
-}
-
+// Score rows too long for one CTA to normalise on the side.
 __global__ void scores_kernel(float* scores, long stride, const float* ml, int T, const int* d_count) {
     const int bh = blockIdx.y;
     if (d_count) T = *d_count;
@@ -647,32 +952,74 @@ __global__ void scores_kernel(float* scores, long stride, const float* ml, int T
     }
 }
 
-// floats of workspace for the partials (two slots per CTA) and the merged (max, sum) pairs
-size_t decode_ws_floats(int BH, int ncta, int D) { return (size_t)2 * ncta * (D + 3) + (size_t)BH * 2; }
+// bytes of workspace: the partials of split (b,h) (two slots per CTA; a grid of more than SLOTS CTAs splits none), the
+// counting words, the merged (max, sum) pairs
+template <int NQ>
+size_t decode_ws_bytes(int BH, int D) {
+    return (size_t)2 * Shape<NQ>::SLOTS * NQ * (D + 4) * sizeof(float) + (size_t)BH * (sizeof(unsigned long long) + 2 * sizeof(float));
+}
 
-template <int D, bool COUNTED = false>
-qaq_status run_decode(const DecArgs& a, int BH, cudaStream_t s) {
-    const size_t smem = sizeof(DecSmem<D>);
+// a number no other call of this process uses (splitmix64 of a counter that starts at the clock), the low 12 bits zero
+unsigned long long call_tag() {
+    static std::atomic<unsigned long long> next{(unsigned long long)std::chrono::steady_clock::now().time_since_epoch().count()};
+    unsigned long long z = next.fetch_add(1, std::memory_order_relaxed) * 0x9E3779B97F4A7C15ull;
+    z = (z ^ (z >> 30)) * 0xBF58476D1CE4E5B9ull;
+    z = (z ^ (z >> 27)) * 0x94D049BB133111EBull;
+    z = (z ^ (z >> 31)) & ~0xFFFull;
+    return z ? z : 0x1000ull;
+}
+
+template <int D, int NQ, bool COUNTED>
+qaq_status launch_decode(const DecArgs& a, cudaStream_t s) {
+    const size_t smem = sizeof(DecSmem<D, NQ>);
+    static_assert(sizeof(DecSmem<D, NQ>) + 1024 <= 227 * 1024 / Shape<NQ>::CTAS_PER_SM, "shared memory of the CTAs of an SM");
     if (smem > 48 * 1024)
-        QAQ_CUDA_TRY(cudaFuncSetAttribute(decode_kernel<D, COUNTED>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem));
-    decode_kernel<D, COUNTED><<<a.ncta, DEC_THREADS, smem, s>>>(a);
-    merge_kernel<D, COUNTED><<<BH, D, 0, s>>>(a);
-    if (a.scores) {
+        QAQ_CUDA_TRY(cudaFuncSetAttribute(decode_kernel<D, NQ, COUNTED>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem));
+    decode_kernel<D, NQ, COUNTED><<<a.ncta, Shape<NQ>::THREADS, smem, s>>>(a);
+    if (NQ == 1 && a.ml) {
         int gx = (a.T + 1023) / 1024;     // counted: a.T holds the capacity
         if (gx > 64) gx = 64;
-        scores_kernel<<<dim3(gx, BH), 256, 0, s>>>(a.scores, a.scores_stride, a.ml, a.T, COUNTED ? a.d_count : nullptr);
+        scores_kernel<<<dim3(gx, a.BH), 256, 0, s>>>(a.scores, a.scores_stride, a.ml, a.T, COUNTED ? a.d_count : nullptr);
     }
     QAQ_CUDA_TRY(cudaGetLastError());
     return QAQ_OK;
+}
+
+// NQ queries per (b,h) (D elements apart inside a row of q and of out; rows of consecutive (b,h) lie q_stride /
+// out_stride elements apart); counted: the token count is taken from device memory
+template <int NQ, bool COUNTED>
+qaq_status decode(const qaq_cache* c, const void* q, long q_stride, float softmax_scale, float* out, long out_stride, float* scores,
+                  long scores_stride, void* ws, cudaStream_t s) {
+    const int D = c->cfg.head_dim, BH = c->BH;
+    DecArgs a;
+    a.k = c->t[0]; a.v = c->t[1]; a.pool_bytes = c->pool_bytes; a.ocap = c->ocap;
+    a.tmax_pad = c->tmax_pad; a.ntiles_max = c->ntiles;
+    a.T = COUNTED ? (int)c->cfg.max_tokens : (int)c->tokens;
+    a.d_count = COUNTED ? qaq_d_count(c) : nullptr;
+    a.q = (const __half*)q; a.q_stride = q_stride; a.scale = softmax_scale;
+    a.out = out; a.out_stride = out_stride; a.scores = scores; a.scores_stride = scores_stride; a.status = c->d_status;
+    const DecPlan plan = plan_decode<NQ>(BH, (a.T + QAQ_TILE - 1) / QAQ_TILE);
+    a.BH = BH;
+    a.run = COUNTED ? 0 : plan.run;
+    a.ncta = COUNTED ? (BH > Shape<NQ>::SLOTS ? BH : Shape<NQ>::SLOTS) : plan.ncta;   // counted: the largest grid any count needs
+    // nothing in the workspace is read before it is written (the counting words: see finish_split)
+    a.part = (float*)ws;
+    a.done = (unsigned long long*)(a.part + (size_t)(BH > Shape<NQ>::SLOTS ? 0 : 2 * Shape<NQ>::SLOTS) * NQ * (D + 4));
+    a.tag = call_tag();
+    a.ml = scores && a.T > SCORES_FUSED_TOKENS ? (float*)(a.done + BH) : nullptr;
+    switch (D) {
+        case 32: return launch_decode<32, NQ, COUNTED>(a, s);
+        case 64: return launch_decode<64, NQ, COUNTED>(a, s);
+        case 128: return launch_decode<128, NQ, COUNTED>(a, s);
+    }
+    return QAQ_ERR_UNSUPPORTED_SHAPE;
 }
 
 }  // namespace
 
 extern "C" qaq_status qaq_decode_workspace_bytes(const qaq_cache* c, size_t* host_out) {
     if (!c || !host_out) return QAQ_ERR_INVALID_ARG;
-    // plan_decode never uses more CTAs than max(DEC_SLOTS, BH), whatever the token count
-    const int ncta_max = c->BH > DEC_SLOTS ? c->BH : DEC_SLOTS;
-    *host_out = decode_ws_floats(c->BH, ncta_max, c->cfg.head_dim) * sizeof(float);
+    *host_out = decode_ws_bytes<1>(c->BH, c->cfg.head_dim);
     return QAQ_OK;
 }
 
@@ -683,47 +1030,40 @@ extern "C" qaq_status qaq_decode_attention(const qaq_cache* c, const void* q, fl
     size_t need = 0;
     qaq_decode_workspace_bytes(c, &need);
     if (ws_bytes < need || ((uintptr_t)ws & 15)) return QAQ_ERR_WORKSPACE;
-    const int D = c->cfg.head_dim, BH = c->BH;
-    DecArgs a;
-    a.k = c->t[0]; a.v = c->t[1]; a.pool_bytes = c->pool_bytes; a.ocap = c->ocap;
-    a.tmax_pad = c->tmax_pad; a.ntiles_max = c->ntiles; a.T = (int)c->tokens;
-    a.q = (const __half*)q; a.scale = softmax_scale; a.q_stride = c->cfg.head_dim; a.out_stride = c->cfg.head_dim;
-    const int ntiles = (a.T + QAQ_TILE - 1) / QAQ_TILE;
-    const DecPlan plan = plan_decode(BH, ntiles);
-    a.BH = BH; a.run = plan.run; a.ncta = plan.ncta;
-    a.part = (float*)ws;
-    a.ml = a.part + (size_t)2 * plan.ncta * (D + 3);
-    a.out = out; a.scores = scores_out; a.scores_stride = a.T; a.d_count = nullptr;
-    cudaStream_t s = (cudaStream_t)stream;
-    switch (D) {
-        case 32: return run_decode<32>(a, BH, s);
-        case 64: return run_decode<64>(a, BH, s);
-        case 128: return run_decode<128>(a, BH, s);
-    }
-    return QAQ_ERR_UNSUPPORTED_SHAPE;
+    return decode<1, false>(c, q, c->cfg.head_dim, softmax_scale, out, c->cfg.head_dim, scores_out, c->tokens, ws, (cudaStream_t)stream);
 }
 
-// One query per (b,h) taken from / written to rows that lie q_stride / out_stride elements apart (used by the
-// batched entry point for the queries that do not fill a pass of their own); ws as for qaq_decode_attention.
-qaq_status qaq_decode_strided(const qaq_cache* c, const void* q, long q_stride, float softmax_scale, float* out, long out_stride,
-                              void* ws, cudaStream_t s) {
-    const int D = c->cfg.head_dim, BH = c->BH;
-    DecArgs a;
-    a.k = c->t[0]; a.v = c->t[1]; a.pool_bytes = c->pool_bytes; a.ocap = c->ocap;
-    a.tmax_pad = c->tmax_pad; a.ntiles_max = c->ntiles; a.T = (int)c->tokens;
-    a.q = (const __half*)q; a.scale = softmax_scale; a.q_stride = q_stride; a.out_stride = out_stride;
-    const int ntiles = (a.T + QAQ_TILE - 1) / QAQ_TILE;
-    const DecPlan plan = plan_decode(BH, ntiles);
-    a.BH = BH; a.run = plan.run; a.ncta = plan.ncta;
-    a.part = (float*)ws;
-    a.ml = a.part + (size_t)2 * plan.ncta * (D + 3);
-    a.out = out; a.scores = nullptr; a.scores_stride = 0; a.d_count = nullptr;
-    switch (D) {
-        case 32: return run_decode<32>(a, BH, s);
-        case 64: return run_decode<64>(a, BH, s);
-        case 128: return run_decode<128>(a, BH, s);
+// ---------------------------------------------------------------------------------------
+// Several queries per (b,h): passes of four, two or one query.
+extern "C" qaq_status qaq_decode_multi_workspace_bytes(const qaq_cache* c, size_t* host_out) {
+    if (!c || !host_out) return QAQ_ERR_INVALID_ARG;
+    const int D = c->cfg.head_dim, BH = c->BH;       // the passes of a call reuse the space
+    const size_t b1 = decode_ws_bytes<1>(BH, D), b2 = decode_ws_bytes<2>(BH, D), b4 = decode_ws_bytes<4>(BH, D);
+    *host_out = b1 > b2 ? (b1 > b4 ? b1 : b4) : (b2 > b4 ? b2 : b4);
+    return QAQ_OK;
+}
+
+extern "C" qaq_status qaq_decode_attention_multi(const qaq_cache* c, const void* q, int n_q, float softmax_scale, float* out,
+                                                 void* ws, size_t ws_bytes, void* stream) {
+    if (!c || !q || !out || !ws || n_q < 1 || n_q > 8) return QAQ_ERR_INVALID_ARG;
+    if (c->tokens < 1) return QAQ_ERR_INVALID_ARG;
+    size_t need = 0;
+    qaq_decode_multi_workspace_bytes(c, &need);
+    if (ws_bytes < need || ((uintptr_t)ws & 15)) return QAQ_ERR_WORKSPACE;
+    const int D = c->cfg.head_dim;
+    const long row = (long)n_q * D;
+    cudaStream_t s = (cudaStream_t)stream;
+    for (int q0 = 0; q0 < n_q;) {
+        const int left = n_q - q0;
+        const __half* qp = (const __half*)q + (size_t)q0 * D;
+        float* op = out + (size_t)q0 * D;
+        qaq_status st;
+        if (left >= 4) { st = decode<4, false>(c, qp, row, softmax_scale, op, row, nullptr, 0, ws, s); q0 += 4; }
+        else if (left >= 2) { st = decode<2, false>(c, qp, row, softmax_scale, op, row, nullptr, 0, ws, s); q0 += 2; }
+        else { st = decode<1, false>(c, qp, row, softmax_scale, op, row, nullptr, 0, ws, s); q0 += 1; }
+        if (st != QAQ_OK) return st;
     }
-    return QAQ_ERR_UNSUPPORTED_SHAPE;
+    return QAQ_OK;
 }
 
 // ---------------------------------------------------------------------------------------
@@ -736,21 +1076,27 @@ qaq_status qaq_decode_strided(const qaq_cache* c, const void* q, long q_stride, 
 #define QAQ_STATIC_SCRATCH_BYTES (4u << 20)
 static __device__ __align__(256) unsigned char g_decode_scratch[QAQ_STATIC_SCRATCH_BYTES];
 
-#include <mutex>
 static std::mutex g_scratch_mutex;
 static void* g_scratch_addr[64];  // device address of g_decode_scratch, per device ordinal
+
+// the documented limit: what two partials per CTA of a split into at most 592 (or one per (b,h)) and a pair of words
+// per (b,h) would take
+static bool static_scratch_fits(int BH, long tokens, int D) {
+    const long ntiles = (tokens + QAQ_TILE - 1) / QAQ_TILE;
+    const long long total = (long long)BH * ntiles, floor_run = ntiles < 4 ? ntiles : 4;
+    long long run = (total + 591) / 592;
+    run = run < floor_run ? floor_run : (run > ntiles ? ntiles : run);
+    const long long ncta = (total + run - 1) / run;
+    return ((size_t)2 * ncta * (D + 3) + (size_t)BH * 2) * sizeof(float) <= QAQ_STATIC_SCRATCH_BYTES;
+}
 
 extern "C" qaq_status qaq_decode_attention_static(const qaq_cache* c, const void* q, float softmax_scale,
                                                   float* out, void* stream) {
     if (!c || !q || !out) return QAQ_ERR_INVALID_ARG;
     if (c->tokens < 1) return QAQ_ERR_INVALID_ARG;
-    const int D = c->cfg.head_dim, BH = c->BH;
-    const int T = (int)c->tokens;
-    const int ntiles = (T + QAQ_TILE - 1) / QAQ_TILE;
-    const DecPlan plan = plan_decode(BH, ntiles);
-    // partials [ncta][2][D+3] followed by the merged (max, sum) pairs [BH][2]
-    const size_t need = decode_ws_floats(BH, plan.ncta, D) * sizeof(float);
-    if (need > QAQ_STATIC_SCRATCH_BYTES) return QAQ_ERR_WORKSPACE;  // shape too large for the built-in scratch
+    const int D = c->cfg.head_dim;
+    if (!static_scratch_fits(c->BH, c->tokens, D)) return QAQ_ERR_WORKSPACE;  // shape too large for the built-in scratch
+    if (decode_ws_bytes<1>(c->BH, D) > QAQ_STATIC_SCRATCH_BYTES) return QAQ_ERR_WORKSPACE;   // never: the limit above is the tighter one
 
     int dev = -1;
     QAQ_CUDA_TRY(cudaGetDevice(&dev));
@@ -770,23 +1116,7 @@ extern "C" qaq_status qaq_decode_attention_static(const qaq_cache* c, const void
         }
         scratch = g_scratch_addr[dev];
     }
-    DecArgs a;
-    a.k = c->t[0]; a.v = c->t[1]; a.pool_bytes = c->pool_bytes; a.ocap = c->ocap;
-    a.tmax_pad = c->tmax_pad; a.ntiles_max = c->ntiles; a.T = T;
-    a.q = (const __half*)q; a.scale = softmax_scale; a.q_stride = c->cfg.head_dim; a.out_stride = c->cfg.head_dim;
-    a.BH = BH; a.run = plan.run; a.ncta = plan.ncta;
-    // Every partial that the merge reads and every (max,sum) pair is written before it is read,
-    // so nothing in the scratch has to be cleared between calls.
-    a.part = (float*)scratch;
-    a.ml = a.part + (size_t)2 * plan.ncta * (D + 3);
-    a.out = out; a.scores = nullptr; a.scores_stride = 0; a.d_count = nullptr;
-    cudaStream_t s = (cudaStream_t)stream;
-    switch (D) {
-        case 32: return run_decode<32>(a, BH, s);
-        case 64: return run_decode<64>(a, BH, s);
-        case 128: return run_decode<128>(a, BH, s);
-    }
-    return QAQ_ERR_UNSUPPORTED_SHAPE;
+    return decode<1, false>(c, q, D, softmax_scale, out, D, nullptr, 0, scratch, (cudaStream_t)stream);
 }
 
 // Decode attention over as many tokens as the device-side count says (qaq_stream_begin / qaq_stream_append): the
@@ -799,21 +1129,5 @@ extern "C" qaq_status qaq_stream_decode(const qaq_cache* c, const void* q, float
     size_t need = 0;
     qaq_decode_workspace_bytes(c, &need);
     if (ws_bytes < need || ((uintptr_t)ws & 15)) return QAQ_ERR_WORKSPACE;
-    const int D = c->cfg.head_dim, BH = c->BH;
-    DecArgs a;
-    a.k = c->t[0]; a.v = c->t[1]; a.pool_bytes = c->pool_bytes; a.ocap = c->ocap;
-    a.tmax_pad = c->tmax_pad; a.ntiles_max = c->ntiles; a.T = (int)c->cfg.max_tokens;
-    a.d_count = qaq_d_count(c);
-    a.q = (const __half*)q; a.scale = softmax_scale; a.q_stride = D; a.out_stride = D;
-    a.BH = BH; a.run = 0; a.ncta = BH > DEC_SLOTS ? BH : DEC_SLOTS;
-    a.part = (float*)ws;
-    a.ml = a.part + (size_t)2 * a.ncta * (D + 3);
-    a.out = out; a.scores = scores_out; a.scores_stride = scores_stride;
-    cudaStream_t s = (cudaStream_t)stream;
-    switch (D) {
-        case 32: return run_decode<32, true>(a, BH, s);
-        case 64: return run_decode<64, true>(a, BH, s);
-        case 128: return run_decode<128, true>(a, BH, s);
-    }
-    return QAQ_ERR_UNSUPPORTED_SHAPE;
+    return decode<1, true>(c, q, c->cfg.head_dim, softmax_scale, out, c->cfg.head_dim, scores_out, scores_stride, ws, (cudaStream_t)stream);
 }

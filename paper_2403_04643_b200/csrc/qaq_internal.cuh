@@ -9,20 +9,17 @@
 #define QAQ_TILE QAQ_TILE_TOKENS
 
 // Device storage of one tensor (K or V) of the cache.  Tokens are grouped in tiles of
-// QAQ_TILE consecutive tokens; a tile's packed codes are contiguous, tokens in order, and
+// QAQ_TILE consecutive tokens; a tile's packed codes are contiguous, sorted by width, and
 // start 16-byte aligned somewhere in the (b,h) pool (tiles are placed by a bump allocator,
-// so their order in memory is not the token order).  Per-token metadata is 5 bytes:
-// the width and the binary16 min and max of the non-outlier entries (step = (max-min)*2^-B
-// is recomputed where needed).  Outliers of a tile are contiguous 32-bit entries
+// so their order in memory is not the token order).  Per-token metadata is 6 bytes: the width, the
+// token's place in the tile (qaq_codec.cuh) and the binary16 min and max of the non-outlier entries
+// (step = (max-min)*2^-B is recomputed where needed).  Outliers of a tile are contiguous 32-bit entries
 //   value(binary16) | channel << 16 | token-in-tile << 24,  sorted by (token, channel).
 struct TensorStore {
     uint8_t* codes;         // [BH][pool_bytes]
-    uint8_t* bits;          // [BH][tmax_pad]
+    unsigned short* bs;     // [BH][tmax_pad]  width | slot << 8
     uint32_t* mnmx;         // [BH][tmax_pad]  half(min) | half(max) << 16
-    uint32_t* tile_off;     // [BH][ntiles]    byte offset of the tile in its pool
-    uint32_t* tile_nbytes;  // [BH][ntiles]
-    uint32_t* tile_ooff;    // [BH][ntiles]    first outlier entry of the tile
-    uint32_t* tile_ocnt;    // [BH][ntiles]
+    uint4* tile;            // [BH][ntiles]    byte offset of the tile in its pool, bytes, first outlier entry, outlier entries
     uint32_t* outl;         // [BH][ocap]
     uint32_t* pool_end;     // [BH] bump pointer, bytes
     uint32_t* opool_end;    // [BH] bump pointer, entries
@@ -60,6 +57,15 @@ extern int g_qaq_last_cuda_error;
 static inline int* qaq_d_count(const qaq_cache* c) { return c->d_status + 1; }
 static inline unsigned* qaq_d_ticket(const qaq_cache* c) { return (unsigned*)(c->d_status + 2); }
 
+#ifdef __CUDACC__
+// Space taken from a pool that turned out not to fit is given back only while nothing has been taken behind it: with a
+// plain subtraction a later taker could be handed space that somebody else holds.  Otherwise it stays taken until
+// qaq_cache_compact or qaq_cache_reset.
+__device__ __forceinline__ void pool_give_back(uint32_t* pool_end, uint32_t base, uint32_t taken) {
+    if (taken) atomicCAS(pool_end, base + taken, base);
+}
+#endif
+
 static inline bool qaq_dim_ok(int D) { return D == 32 || D == 64 || D == 128; }
 
 // launchers implemented in the kernel translation units
@@ -69,6 +75,3 @@ qaq_status qaq_launch_select(const qaq_config* cfg, const qaq_policy* pol, const
 qaq_status qaq_launch_append(qaq_cache* c, const void* K, const void* V, long sb, long sh, long st, int n_new,
                              const uint8_t* bitsK, const uint8_t* bitsV, const qaq_policy* pol, const float* ring,
                              const uint8_t* nvalid, const float* thr, cudaStream_t s);
-// single-query decode on strided query / output rows (qaq_decode.cu); ws: qaq_decode_workspace_bytes bytes
-qaq_status qaq_decode_strided(const qaq_cache* c, const void* q, long q_stride, float softmax_scale, float* out, long out_stride,
-                              void* ws, cudaStream_t s);

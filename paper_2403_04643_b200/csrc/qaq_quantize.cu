@@ -6,11 +6,11 @@
 //   phase 0  attention-window maximum of the score rows (Section 4.2)
 //   phase 1  outlier masks and min/max of the non-outliers in binary16 pair arithmetic
 //            (exact: the inputs are binary16), width from the exponents (Section 4.1)
-//   phase 2  warp 0: which slots have a piece of each width (ballots), section sizes of the tile,
+//   phase 2  warp 0: the tokens sorted by width (ballots), sections and size of the tile,
 //            exclusive scan of the outlier counts, space taken from the (b,h) pools by atomicAdd
-//   phase 3  codes (binary32: one sub, one mul, round down), pieces written into a shared-memory
-//            image of the tile in the section layout of qaq_codec.cuh (values as token-major planes
-//            that the copy-out transposes into groups of four tokens), vector stores; outlier
+//   phase 3  codes (binary32: one sub, one mul, round down), packed words written into a shared-memory
+//            image of the tile in the section layout of qaq_codec.cuh (values token by token, which
+//            the copy-out transposes into rows of four tokens), vector stores; outlier
 //            entries placed by popc ranks
 // A tile that is continued (an append behind a partly filled tile) is built anew: the codes of
 // its old tokens are read back from the pool, the image of old and new tokens replaces it.
@@ -86,11 +86,15 @@ __device__ __forceinline__ void analyze32(uint32_t (&v)[16], __half2 lo2, __half
 
 // space from a (b,h) pool: `whole` tiles take a rounded-up amount in one atomic; a tile that is
 // being continued takes the exact amount and is padded to the unit when it closes.  `taken` is
-// what the pool end moved by (to be given back if the space turns out not to fit).
-__device__ __forceinline__ uint32_t pool_take(uint32_t* pool, uint32_t amount, uint32_t unit_mask, bool whole, bool closes,
+// what the pool end moved by (to be given back if the space turns out not to fit: pool_give_back).
+// full: the pool end already lay beyond the pool when the CTA began; nothing is taken, so that the end cannot run away.
+__device__ __forceinline__ uint32_t pool_take(uint32_t* pool, uint32_t amount, uint32_t unit_mask, bool whole, bool closes, bool full,
                                               uint32_t& taken) {
     uint32_t base;
-    if (whole) {
+    if (full) {
+        taken = 0;
+        base = 0xFFFF0000u;
+    } else if (whole) {
         taken = (amount + unit_mask) & ~unit_mask;
         base = atomicAdd(pool, taken);
     } else {
@@ -108,8 +112,8 @@ __device__ __forceinline__ uint32_t pool_take(uint32_t* pool, uint32_t amount, u
 // One CTA = one tile of 64 tokens of one (b,h); P = D/32 lanes own a token, each lane 32
 // consecutive channels (64 bytes) of K and of V, kept in registers across all phases.
 // Order of work (barriers in brackets): loads, attention window, outlier masks and ranges,
-// widths [A] warp 0 finds the section sizes of the tile, scans the outlier counts and takes pool
-// space with four atomics in flight at once while every warp computes its codes [B] pieces into a
+// widths [A] warp 0 sorts the tile's tokens by width and sizes its sections, warp 1 scans the outlier counts and takes pool
+// space with four atomics in flight at once while every warp computes its codes [B] words into a
 // shared-memory image of the tile [C] the image goes out with 16-byte stores; outlier entries and
 // per-token metadata follow.  Slots below the first new token of a continued tile hold the tile's
 // old tokens: their widths come from the metadata, their codes from the tile as it is stored.
@@ -126,7 +130,7 @@ __global__ void __launch_bounds__(2 * D, XSEL < 0 ? (D == 128 ? 3 : 4) : (D == 1
     constexpr int X0 = XSEL < 0 ? 0 : XSEL, X1 = XSEL < 0 ? 2 : XSEL + 1;
     constexpr int P = D / 32;            // lanes per token
     constexpr int NT = 2 * D;            // threads
-    constexpr int IMG = qaqc::v_tile_bytes_max(D);
+    constexpr int IMG = qaqc::tile_bytes_max(D);
     constexpr bool COUNTED = XSEL < 0 && !SELECT_ONLY;   // the launches that may take the token count from device memory
     const int bh = blockIdx.y;
     const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
@@ -163,9 +167,9 @@ __global__ void __launch_bounds__(2 * D, XSEL < 0 ? (D == 128 ? 3 : 4) : (D == 1
 
     __shared__ uint8_t s_bits[2][QAQ_TILE];   // widths of the tile's slots (0: empty)
     __shared__ uint32_t s_cnt[2][QAQ_TILE];   // outlier counts of the new tokens, then exclusive offsets
-    __shared__ qaqc::TileMasks s_tm[2];
-    __shared__ uint32_t s_rank[2][QAQ_TILE];   // ranks of the slots in the four sections, one per byte
-    __shared__ uint32_t s_sec[2][5];           // byte offsets of the sections
+    __shared__ qaqc::Section s_tab[2][9], s_otab[2][9];   // sections of the tile by width, and of the tile as it was (continued tiles)
+    __shared__ unsigned short s_place[2][QAQ_TILE];       // slot of every token in the sorted order | width of its row << 8
+    __shared__ uint8_t s_sorted[2][QAQ_TILE], s_orow[2][QAQ_TILE / 4];   // width of every slot; width of the stored rows of values
     __shared__ uint32_t s_tot[2], s_base[2], s_obase[2], s_olimit[2], s_otot[2];
     constexpr uint32_t OUT_STAGE = 4 * D;      // outliers of a tile whose (slot, channel) are listed on chip in entry order; more go out one by one
     __shared__ unsigned short s_work[SELECT_ONLY ? 1 : X1 - X0][SELECT_ONLY ? 1 : OUT_STAGE];
@@ -194,7 +198,35 @@ __global__ void __launch_bounds__(2 * D, XSEL < 0 ? (D == 128 ? 3 : 4) : (D == 1
             vv[4 * i] = y.x; vv[4 * i + 1] = y.y; vv[4 * i + 2] = y.z; vv[4 * i + 3] = y.w;
         }
     }
-    // the padding of the value groups has to read as zero
+    uint32_t pool_now = 0;          // in the lanes that take space further down
+    if (!SELECT_ONLY && warp < 2 && (lane >> 1) >= X0 && (lane >> 1) < X1 && (lane & 1) == warp)
+        pool_now = *((warp ? ((lane >> 1) ? a.v : a.k).opool_end : ((lane >> 1) ? a.v : a.k).pool_end) + bh);
+    // a continued tile: its sections as they are stored (warp x for tensor x; used behind the first barrier)
+    if (!SELECT_ONLY && s_lo > 0) {
+#pragma unroll
+        for (int x = X0; x < X1; ++x) {
+            if (warp != x) continue;
+            const TensorStore& ts = x ? a.v : a.k;
+            uint2 h = make_uint2(0u, 0u);
+            if (ts.tile[ti].y) h = *reinterpret_cast<const uint2*>(ts.codes + (size_t)bh * a.pool_bytes + ts.tile[ti].x);
+            int n[9];
+            qaqc::counts_of(h.x, h.y, n);
+            if (lane == 0) {
+                if (x) qaqc::make_sections<qaqc::UNITS<D, true>>(n, s_otab[x], nullptr);
+                else qaqc::make_sections<qaqc::UNITS<D, false>>(n, s_otab[x], nullptr);
+            }
+            if (x && lane < QAQ_TILE / 4) {
+                int w = 0, end = 0;
+#pragma unroll
+                for (int k = 8; k >= 1; --k) {
+                    if (lane >= end && lane < end + n[k]) w = k;
+                    end += n[k];
+                }
+                s_orow[x][lane] = (uint8_t)w;
+            }
+        }
+    }
+    // empty slots of the value groups have to read as zero
     if (!SELECT_ONLY && XSEL != 0) {
         uint4* z = reinterpret_cast<uint4*>(s_img[X1 - X0 - 1]);
         for (int o = tid; o < IMG / 16; o += NT) z[o] = make_uint4(0, 0, 0, 0);
@@ -250,7 +282,7 @@ __global__ void __launch_bounds__(2 * D, XSEL < 0 ? (D == 128 ? 3 : 4) : (D == 1
     }
 
     // ---- widths
-    int Bx[2];
+    int Bx[2], oslot[2] = {0, 0};      // oslot: where an old token lies in the tile as it is stored
 #pragma unroll
     for (int x = X0; x < X1; ++x) {
         int B;
@@ -267,8 +299,9 @@ __global__ void __launch_bounds__(2 * D, XSEL < 0 ? (D == 128 ? 3 : 4) : (D == 1
         }
         Bx[x] = valid ? B : 0;
         if (old) {
-            const int bo = (x ? a.v : a.k).bits[mt];
-            Bx[x] = bo > 8 ? 8 : bo;
+            const uint32_t bs = (x ? a.v : a.k).bs[mt];
+            Bx[x] = min((int)(bs & 0xFFu), 8);
+            oslot[x] = (int)(bs >> 8);
         }
         if (p == 0) {                                   // every slot of the tile is written: empty ones count nothing
             s_bits[x][slot] = (uint8_t)Bx[x];
@@ -279,7 +312,7 @@ __global__ void __launch_bounds__(2 * D, XSEL < 0 ? (D == 128 ? 3 : 4) : (D == 1
     if (SELECT_ONLY) return;
     __syncthreads();   // [A] widths and outlier counts visible
 
-    // ---- warp 0: section masks of the tile, ranks and section offsets, space for the bytes; warp 1: scan of the
+    // ---- warp 0: tokens sorted by width, sections and header of the tile, space for the bytes; warp 1: scan of the
     //      outlier counts, space for the entries (the two halves do not depend on each other; the atomics - lane 2x of
     //      warp 0 and lane 2x + 1 of warp 1 for tensor x - stay in flight while every warp computes its codes)
     const bool starts = (s_lo == 0), closes = (s_hi == QAQ_TILE), whole = starts && closes;
@@ -288,33 +321,26 @@ __global__ void __launch_bounds__(2 * D, XSEL < 0 ? (D == 128 ? 3 : 4) : (D == 1
         uint32_t amount[2];
 #pragma unroll
         for (int x = X0; x < X1; ++x) {
-            const uint32_t b0 = s_bits[x][lane], b1 = s_bits[x][lane + 32];
-            qaqc::TileMasks tm;
-            uint32_t rk0 = 0, rk1 = 0;       // ranks of slots lane and lane + 32
-#pragma unroll
-            for (int c = 0; c < 4; ++c) {
-                const unsigned lo = __ballot_sync(0xFFFFFFFFu, (b0 & (8u >> c)) != 0), hi = __ballot_sync(0xFFFFFFFFu, (b1 & (8u >> c)) != 0);
-                tm.m[c] = (unsigned long long)lo | ((unsigned long long)hi << 32);
-                const unsigned below = (1u << lane) - 1u;
-                rk0 |= (uint32_t)__popc(lo & below) << (8 * c);
-                rk1 |= (uint32_t)(__popc(lo) + __popc(hi & below)) << (8 * c);
-            }
-            s_rank[x][lane] = rk0; s_rank[x][lane + 32] = rk1;
-            uint32_t base[5];
-            if (x == 0) qaqc::section_bases<D, false>(tm, base); else qaqc::section_bases<D, true>(tm, base);
+            const int b0 = s_bits[x][lane], b1 = s_bits[x][lane + 32];
+            int n[9];
+            const qaqc::Sorted so = x ? qaqc::sort_tile<true>(lane, b0, b1, n, s_sorted[x]) : qaqc::sort_tile<false>(lane, b0, b1, n, s_sorted[x]);
+            s_place[x][lane] = (unsigned short)(so.slot[0] | (so.row_w[0] << 8));
+            s_place[x][lane + 32] = (unsigned short)(so.slot[1] | (so.row_w[1] << 8));
+            uint32_t total = 0;
             if (lane == 0) {
-#pragma unroll
-                for (int c = 0; c < 5; ++c) s_sec[x][c] = base[c];
+                uint32_t* head = reinterpret_cast<uint32_t*>(s_img[x - X0]);
+                total = x ? qaqc::make_sections<qaqc::UNITS<D, true>>(n, s_tab[x], head) : qaqc::make_sections<qaqc::UNITS<D, false>>(n, s_tab[x], head);
+                s_tot[x] = total;
             }
+            total = __shfl_sync(0xFFFFFFFFu, total, 0);
             // a continued tile stays where it is and takes only what it grows by behind its end
-            const uint32_t old_nb = starts ? 0u : (x ? a.v : a.k).tile_nbytes[ti];
-            amount[x] = base[4] - old_nb;
-            if (lane == 0) { s_tm[x] = tm; s_tot[x] = base[4]; }
+            const uint32_t old_nb = starts ? 0u : (x ? a.v : a.k).tile[ti].y;
+            amount[x] = total - old_nb;
         }
         if (!(lane & 1) && lane >= 2 * X0 && lane < 2 * X1) {
             const int x = lane >> 1;
             my_amount = x ? amount[1] : amount[0];
-            my_base = pool_take(&(x ? a.v : a.k).pool_end[bh], my_amount, 15u, whole, closes, my_taken);
+            my_base = pool_take(&(x ? a.v : a.k).pool_end[bh], my_amount, 15u, whole, closes, pool_now > a.pool_bytes, my_taken);
         }
     } else if (warp == 1) {
         uint32_t amount[2];
@@ -335,7 +361,7 @@ __global__ void __launch_bounds__(2 * D, XSEL < 0 ? (D == 128 ? 3 : 4) : (D == 1
         if ((lane & 1) && lane >= 2 * X0 && lane < 2 * X1) {
             const int x = lane >> 1;
             my_amount = x ? amount[1] : amount[0];
-            my_base = pool_take(&(x ? a.v : a.k).opool_end[bh], my_amount, 3u, whole, closes, my_taken);
+            my_base = pool_take(&(x ? a.v : a.k).opool_end[bh], my_amount, 3u, whole, closes, pool_now > a.ocap, my_taken);
         }
     }
 
@@ -343,40 +369,28 @@ __global__ void __launch_bounds__(2 * D, XSEL < 0 ? (D == 128 ? 3 : 4) : (D == 1
     uint32_t cregs[2][8];
 #pragma unroll
     for (int x = X0; x < X1; ++x) qaqc::codes32(x ? vv : vk, mnf[x], mxf[x], Bx[x], cregs[x]);
-    __syncthreads();   // [B] section masks visible
-
-    // ---- old tokens of a continued tile: their codes from the tile as it is stored (read before anything is written)
+    // old tokens of a continued tile: their codes from the tile as it is stored (read before anything is written)
     if (!starts) {
 #pragma unroll
         for (int x = X0; x < X1; ++x) {
             if (!old) continue;
             const TensorStore& ts = x ? a.v : a.k;
-            const uint8_t* src = ts.codes + (size_t)bh * a.pool_bytes + ts.tile_off[ti];
-            qaqc::TileMasks om;
-#pragma unroll
-            for (int c = 0; c < 4; ++c) om.m[c] = s_tm[x].m[c] & ((1ull << s_lo) - 1ull);
-            uint32_t ob[5];
-            if (x == 0) { qaqc::section_bases<D, false>(om, ob); qaqc::read_pieces<D, false>(src, om, ob, slot, Bx[x], p, cregs[x]); }
-            else        { qaqc::section_bases<D, true>(om, ob);  qaqc::read_pieces<D, true>(src, om, ob, slot, Bx[x], p, cregs[x]); }
+            const uint8_t* src = ts.codes + (size_t)bh * a.pool_bytes + ts.tile[ti].x;
+            const int w = x ? (int)s_orow[x][(oslot[x] >> 2) & (QAQ_TILE / 4 - 1)] : Bx[x];
+            if (!Bx[x]) continue;                       // never stored (the pool was full)
+            if (x == 0) qaqc::read_token<D, false>(src, s_otab[x][w], oslot[x], w, p, cregs[x]);
+            else        qaqc::read_token<D, true>(src, s_otab[x][w], oslot[x], w, p, cregs[x]);
         }
     }
-    // ---- header and pieces into the shared-memory image of the tile (the values as token-major planes, which the
-    //      copy to global memory turns into groups of four tokens)
-    uint32_t vbase[5] = {0, 0, 0, 0, 0};
+    __syncthreads();   // [B] sections visible
+
+    // ---- packed words into the shared-memory image of the tile (the values token by token: the copy to global memory
+    //      turns them into rows of four tokens)
 #pragma unroll
     for (int x = X0; x < X1; ++x) {
-        if (tid < 4) qaqc::write_header(s_img[x - X0], s_tm[x], tid);
-        const qaqc::PackedRanks rk{s_rank[x][slot & (QAQ_TILE - 1)]};
-        if (x == 0) {
-            uint32_t base[5];
-#pragma unroll
-            for (int c = 0; c < 5; ++c) base[c] = s_sec[x][c];
-            if (valid || old) qaqc::write_pieces<D, false>(s_img[x - X0], rk, base, Bx[x], p, cregs[x]);
-        } else {
-#pragma unroll
-            for (int c = 0; c < 5; ++c) vbase[c] = s_sec[x][c];
-            if (valid || old) qaqc::write_planes_v<D>(s_img[x - X0], rk, vbase, Bx[x], p, cregs[x]);
-        }
+        const uint32_t pl = s_place[x][slot & (QAQ_TILE - 1)];
+        const int w = (int)(pl >> 8);
+        if ((valid || old) && w) qaqc::write_token<D>(s_img[x - X0], s_tab[x][w], x == 1, (int)(pl & 0xFFu), w, p, cregs[x]);
     }
     // ---- where the outliers of the new tokens are: (slot, channel) in (token, channel) order - entries of lanes
     //      p' < p of a token come first - listed in shared memory; their place needs only the scan of the counts.
@@ -415,17 +429,20 @@ __global__ void __launch_bounds__(2 * D, XSEL < 0 ? (D == 128 ? 3 : 4) : (D == 1
         const int x = lane >> 1;
         const TensorStore& ts = x ? a.v : a.k;
         if (mine) {
-            const uint32_t off = starts ? my_base : ts.tile_off[ti];
+            const uint32_t off = starts ? my_base : ts.tile[ti].x;
             fail = (size_t)my_base + my_taken + 16 > a.pool_bytes || (size_t)off + s_tot[x] + 16 > a.pool_bytes;
+            // a continued tile grows into what lies behind it: that has to be the space just taken (an open tile that
+            // re-quantization could not keep the last thing in a full pool cannot grow)
+            if (!starts && my_base != off + ts.tile[ti].y) fail = true;
             s_base[x] = off;
         }
         const bool any_fail = __any_sync(0xFFFFFFFFu, fail);
         if (mine) {
             if (any_fail) {
-                if (my_taken) atomicSub(&ts.pool_end[bh], my_taken);
+                pool_give_back(&ts.pool_end[bh], my_base, my_taken);
             } else {
-                if (starts) ts.tile_off[ti] = my_base;
-                ts.tile_nbytes[ti] = s_tot[x];
+                if (starts) ts.tile[ti].x = my_base;
+                ts.tile[ti].y = s_tot[x];
             }
         }
         if (lane == 0) {
@@ -435,7 +452,7 @@ __global__ void __launch_bounds__(2 * D, XSEL < 0 ? (D == 128 ? 3 : 4) : (D == 1
     } else if (warp == 1) {   // the outlier lists: what fits is known now, the table is written once the byte pools have answered
         if ((lane & 1) && lane >= 2 * X0 && lane < 2 * X1) {
             const int x = lane >> 1;
-            const uint32_t room = my_base + 8 < a.ocap ? a.ocap - 8 - my_base : 0;  // 8 entries of read-ahead margin
+            const uint32_t room = (size_t)my_base + 8 < a.ocap ? a.ocap - 8 - my_base : 0;  // 8 entries of read-ahead margin
             const uint32_t stored = my_amount < room ? my_amount : room;
             if (stored < my_amount) atomicMax(a.status, (int)QAQ_ERR_CAPACITY);
             s_obase[x] = my_base;
@@ -447,11 +464,11 @@ __global__ void __launch_bounds__(2 * D, XSEL < 0 ? (D == 128 ? 3 : 4) : (D == 1
         const int x = lane >> 1;
         const TensorStore& ts = x ? a.v : a.k;
         if (s_skip) {
-            if (my_taken) atomicSub(&ts.opool_end[bh], my_taken);
+            pool_give_back(&ts.opool_end[bh], my_base, my_taken);
         } else {
             const uint32_t stored = s_olimit[x] - s_obase[x];
-            if (starts) { ts.tile_ooff[ti] = my_base; ts.tile_ocnt[ti] = stored; }
-            else ts.tile_ocnt[ti] += stored;
+            if (starts) { ts.tile[ti].z = my_base; ts.tile[ti].w = stored; }
+            else ts.tile[ti].w += stored;
         }
     }
     if (s_skip) { tick(); return; }
@@ -472,11 +489,17 @@ __global__ void __launch_bounds__(2 * D, XSEL < 0 ? (D == 128 ? 3 : 4) : (D == 1
             w_first = s_work[x - X0][tid];
             v_first = __half_as_ushort(X[(size_t)(tile * QAQ_TILE + (int)(w_first >> 8) - t_old) * a.st + (w_first & 0xFFu)]);
         }
-        for (uint32_t o = tid * 16; o < nb; o += NT * 16) {
-            uint4 v;
-            if (x == 0 || o < (uint32_t)qaqc::QAQ_TILE_HDR) v = *reinterpret_cast<const uint4*>(s_img[x - X0] + o);
-            else v = qaqc::group_unit_v<D>(s_img[x - X0], vbase, o);
-            *reinterpret_cast<uint4*>(dst + o) = v;
+        if (x == 0) {
+            for (uint32_t o = tid * 16; o < nb; o += NT * 16)
+                *reinterpret_cast<uint4*>(dst + o) = *reinterpret_cast<const uint4*>(s_img[x - X0] + o);
+        } else {
+            // one unit per thread, the four rows that are interleaved side by side
+            const int row = (tid / (16 * P)) * 4 + (tid & 3), e = (tid >> 2) % (4 * P);
+            if (row < s_tab[x][1].start + s_tab[x][1].n) {
+                const int w = s_sorted[x][4 * row];
+                qaqc::group_out<D>(s_img[x - X0], dst, s_tab[x][w], w, row, e);
+            }
+            if (tid == 0) *reinterpret_cast<uint4*>(dst) = *reinterpret_cast<const uint4*>(s_img[x - X0]);
         }
         // outlier entries: one listed outlier per thread (value read again from the input: the registers hold -inf in
         // its place), stores next to each other; a tile with more outliers than are listed writes the rest one by one
@@ -526,8 +549,8 @@ __global__ void __launch_bounds__(2 * D, XSEL < 0 ? (D == 128 ? 3 : 4) : (D == 1
                 }
             }
         }
+        if ((valid || old) && p == 0) ts.bs[mt] = (unsigned short)(Bx[x] | ((s_place[x][slot & (QAQ_TILE - 1)] & 0xFFu) << 8));
         if (valid && p == 0) {
-            ts.bits[mt] = (uint8_t)Bx[x];
             ts.mnmx[mt] = (uint32_t)__half_as_ushort(__float2half_rn(mnf[x])) | ((uint32_t)__half_as_ushort(__float2half_rn(mxf[x])) << 16);
         }
     }

@@ -14,7 +14,7 @@
 // One CTA = one tile (QAQ_TILE tokens) of one (b,h), both tensors; head_dim/32 lanes own a
 // token, each lane the codes of 32 consecutive channels, one byte per code in 8 registers.
 // All of a tile's old bytes are in registers before the first new byte is written (the new
-// planes are built in a shared-memory image of the tile first), so a tile that does not grow is
+// words are built in a shared-memory image of the tile first), so a tile that does not grow is
 // rewritten in place.  A closed tile that grows takes a new place at the end of its pool (the
 // old bytes stay unused); the open (last, partly filled) tile is handled in a launch of its own
 // after the closed ones and is kept - or made again - the last thing in its pool, so that later
@@ -61,14 +61,13 @@ __device__ __forceinline__ void fresh_codes(const __half* row, float lo, float h
     qaqc::codes32(v, mn, mx, B, creg);
 }
 
-// UP: widths may be raised (the unquantized copy is there).  Either way a tile whose bytes grow - raised widths,
-// or lowered ones that need more padding of the value groups than before - takes a new place at the end of its
-// pool; closed tiles are handled by one launch, the open tile by a launch of its own after it.
+// UP: widths may be raised (the unquantized copy is there).  A tile whose bytes grow takes a new place at the end of
+// its pool; closed tiles are handled by one launch, the open tile by a launch of its own after it.
 template <int D, bool UP>
 __global__ void __launch_bounds__(2 * D) requant_kernel(const RequantArgs a) {
     constexpr int P = D / 32;
     constexpr int NT = 2 * D;
-    constexpr int IMG = qaqc::v_tile_bytes_max(D);
+    constexpr int IMG = qaqc::tile_bytes_max(D);
     const int tile = a.first_tile + blockIdx.x, bh = blockIdx.y;
     const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
     const int slot = tid / P, p = tid % P;
@@ -79,12 +78,14 @@ __global__ void __launch_bounds__(2 * D) requant_kernel(const RequantArgs a) {
     __shared__ float s_part[P][QAQ_TILE];
     __shared__ uint8_t s_nv[QAQ_TILE];
     __shared__ uint8_t s_bo[2][QAQ_TILE], s_bn[2][QAQ_TILE];      // widths before and after
-    __shared__ qaqc::TileMasks s_tmo[2], s_tmn[2];
+    __shared__ qaqc::Section s_otab[2][9], s_tab[2][9];             // sections before and after
+    __shared__ unsigned short s_place[2][QAQ_TILE];                 // new slot | width of its row << 8
+    __shared__ uint8_t s_sorted[2][QAQ_TILE], s_orow[QAQ_TILE / 4]; // new width of every slot; stored width of the rows of values
     __shared__ uint32_t s_tot[2], s_off[2];                        // new bytes of the tile, where they go in the pool
     __shared__ int s_skip[2];
     __shared__ __align__(16) uint8_t s_img[2][IMG];
 
-    // the padding of the value groups has to read as zero
+    // empty slots of the value groups have to read as zero
     for (int o = tid; o < IMG / 16; o += NT) reinterpret_cast<uint4*>(s_img[1])[o] = make_uint4(0, 0, 0, 0);
 
     // ---- attention window of the tile's tokens (value rule); P threads share a token's rows
@@ -104,14 +105,15 @@ __global__ void __launch_bounds__(2 * D) requant_kernel(const RequantArgs a) {
     }
     // ---- current widths and ranges
     const size_t mt = (size_t)bh * a.tmax_pad + tok;
-    int Bo[2] = {0, 0};
+    int Bo[2] = {0, 0}, oslot[2] = {0, 0};
     float rng[2] = {0.f, 0.f}, mnf[2] = {0.f, 0.f}, mxf[2] = {0.f, 0.f};
     if (valid) {
 #pragma unroll
         for (int x = 0; x < 2; ++x) {
             const TensorStore& ts = x ? a.v : a.k;
-            Bo[x] = ts.bits[mt];
-            Bo[x] = Bo[x] > 8 ? 8 : Bo[x];
+            const uint32_t bs = ts.bs[mt];
+            Bo[x] = min((int)(bs & 0xFFu), 8);
+            oslot[x] = (int)((bs >> 8) & (QAQ_TILE - 1));
             const uint32_t mm = ts.mnmx[mt];
             mnf[x] = __half2float(__ushort_as_half((unsigned short)(mm & 0xFFFF)));
             mxf[x] = __half2float(__ushort_as_half((unsigned short)(mm >> 16)));
@@ -155,7 +157,7 @@ __global__ void __launch_bounds__(2 * D) requant_kernel(const RequantArgs a) {
 #pragma unroll
         for (int x = 0; x < 2; ++x) {
             const TensorStore& ts = x ? a.v : a.k;
-            relocate[x] = ts.tile_off[ti0] + ts.tile_nbytes[ti0] != ts.pool_end[bh];
+            relocate[x] = ts.tile[ti0].x + ts.tile[ti0].y != ts.pool_end[bh];
             changed[x] = changed[x] || relocate[x];
         }
     }
@@ -165,23 +167,40 @@ __global__ void __launch_bounds__(2 * D) requant_kernel(const RequantArgs a) {
     if (warp == 0) {
 #pragma unroll
         for (int x = 0; x < 2; ++x) {
-            const uint32_t o0 = s_bo[x][lane], o1 = s_bo[x][lane + 32], n0 = s_bn[x][lane], n1 = s_bn[x][lane + 32];
-            qaqc::TileMasks mo, mn_;
+            {   // the sections as they are stored
+                const TensorStore& ts = x ? a.v : a.k;
+                const size_t ti0 = (size_t)bh * a.ntiles + tile;
+                uint2 h = make_uint2(0u, 0u);
+                if (ts.tile[ti0].y) h = *reinterpret_cast<const uint2*>(ts.codes + (size_t)bh * a.pool_bytes + ts.tile[ti0].x);
+                int n[9];
+                qaqc::counts_of(h.x, h.y, n);
+                if (lane == 0) {
+                    if (x) qaqc::make_sections<qaqc::UNITS<D, true>>(n, s_otab[x], nullptr);
+                    else qaqc::make_sections<qaqc::UNITS<D, false>>(n, s_otab[x], nullptr);
+                }
+                if (x && lane < QAQ_TILE / 4) {
+                    int w = 0, end = 0;
 #pragma unroll
-            for (int c = 0; c < 4; ++c) {
-                mo.m[c] = (unsigned long long)__ballot_sync(0xFFFFFFFFu, (o0 & (8u >> c)) != 0) |
-                          ((unsigned long long)__ballot_sync(0xFFFFFFFFu, (o1 & (8u >> c)) != 0) << 32);
-                mn_.m[c] = (unsigned long long)__ballot_sync(0xFFFFFFFFu, (n0 & (8u >> c)) != 0) |
-                           ((unsigned long long)__ballot_sync(0xFFFFFFFFu, (n1 & (8u >> c)) != 0) << 32);
+                    for (int k = 8; k >= 1; --k) {
+                        if (lane >= end && lane < end + n[k]) w = k;
+                        end += n[k];
+                    }
+                    s_orow[lane] = (uint8_t)w;
+                }
             }
+            int n[9];
+            const int b0 = s_bn[x][lane], b1 = s_bn[x][lane + 32];
+            const qaqc::Sorted so = x ? qaqc::sort_tile<true>(lane, b0, b1, n, s_sorted[x]) : qaqc::sort_tile<false>(lane, b0, b1, n, s_sorted[x]);
+            s_place[x][lane] = (unsigned short)(so.slot[0] | (so.row_w[0] << 8));
+            s_place[x][lane + 32] = (unsigned short)(so.slot[1] | (so.row_w[1] << 8));
             if (lane == 0) {
-                s_tmo[x] = mo; s_tmn[x] = mn_;
-                uint32_t nbase[5];
-                if (x == 0) qaqc::section_bases<D, false>(mn_, nbase); else qaqc::section_bases<D, true>(mn_, nbase);
+                uint32_t* head = reinterpret_cast<uint32_t*>(s_img[x]);
+                const uint32_t nb = x ? qaqc::make_sections<qaqc::UNITS<D, true>>(n, s_tab[x], head)
+                                      : qaqc::make_sections<qaqc::UNITS<D, false>>(n, s_tab[x], head);
                 // where the new tile goes: in place unless it grows
                 const TensorStore& ts = x ? a.v : a.k;
                 const size_t ti0 = (size_t)bh * a.ntiles + tile;
-                const uint32_t nb = nbase[4], off = ts.tile_off[ti0], old_nb = ts.tile_nbytes[ti0];
+                const uint32_t off = ts.tile[ti0].x, old_nb = ts.tile[ti0].y;
                 const uint32_t old_own = open ? old_nb : ((old_nb + 15u) & ~15u);   // closed tiles own a rounded amount
                 uint32_t noff = off;
                 int skip = 0;
@@ -200,9 +219,11 @@ __global__ void __launch_bounds__(2 * D) requant_kernel(const RequantArgs a) {
                         // the end of the pool need not be aligned while a tile is open: take 16 bytes more and align;
                         // space that does not fit is given back
                         const uint32_t take = ((nb + 15u) & ~15u) + 16u;
-                        const uint32_t at = atomicAdd(&ts.pool_end[bh], take);
+                        const bool full = *(volatile uint32_t*)&ts.pool_end[bh] > a.pool_bytes;      // takes nothing: the end must not run away
+                        const uint32_t at = full ? 0u : atomicAdd(&ts.pool_end[bh], take);
                         noff = (at + 15u) & ~15u;
-                        if ((size_t)at + take + 16 > a.pool_bytes) { skip = 1; atomicSub(&ts.pool_end[bh], take); }
+                        if (full) skip = 1;
+                        else if ((size_t)at + take + 16 > a.pool_bytes) { skip = 1; pool_give_back(&ts.pool_end[bh], at, take); }
                     }
                     if (skip) atomicMax(a.status, (int)QAQ_ERR_CAPACITY);
                 }
@@ -221,29 +242,25 @@ __global__ void __launch_bounds__(2 * D) requant_kernel(const RequantArgs a) {
     for (int x = 0; x < 2; ++x) {
         if (!changed[x]) continue;
         const TensorStore& ts = x ? a.v : a.k;
-        if (tid < 4) qaqc::write_header(s_img[x], s_tmn[x], tid);
         uint32_t creg[8];
-        if (valid) {
+        if (valid && Bn[x]) {
             if (UP && Bn[x] > Bo[x]) {
                 // raised: codes from the unquantized row, with the token's stored min / max and the thresholds
                 const __half* row = (x ? a.Vs : a.Ks) + (size_t)(bh / a.H) * a.sb + (size_t)(bh % a.H) * a.sh +
                                     (size_t)tok * a.st + 32 * p;
                 fresh_codes(row, a.thr[(size_t)bh * 4 + 2 * x], a.thr[(size_t)bh * 4 + 2 * x + 1], mnf[x], mxf[x], Bn[x], creg);
             } else {
-                const uint8_t* src = ts.codes + (size_t)bh * a.pool_bytes + ts.tile_off[ti];
-                const qaqc::TileMasks mo = s_tmo[x];
-                uint32_t ob[5];
-                if (x == 0) { qaqc::section_bases<D, false>(mo, ob); qaqc::read_pieces<D, false>(src, mo, ob, slot, Bo[x], p, creg); }
-                else        { qaqc::section_bases<D, true>(mo, ob);  qaqc::read_pieces<D, true>(src, mo, ob, slot, Bo[x], p, creg); }
+                const uint8_t* src = ts.codes + (size_t)bh * a.pool_bytes + ts.tile[ti].x;
+                const int w = x ? (int)s_orow[oslot[x] >> 2] : Bo[x];
+                if (x == 0) qaqc::read_token<D, false>(src, s_otab[x][w], oslot[x], w, p, creg);
+                else        qaqc::read_token<D, true>(src, s_otab[x][w], oslot[x], w, p, creg);
                 const int drop = Bo[x] - Bn[x];
                 const uint32_t keep = 0x01010101u * (0xFFu >> drop);
 #pragma unroll
                 for (int j = 0; j < 8; ++j) creg[j] = (creg[j] >> drop) & keep;
             }
-            const qaqc::TileMasks mn_ = s_tmn[x];
-            uint32_t nbs[5];
-            if (x == 0) { qaqc::section_bases<D, false>(mn_, nbs); qaqc::write_pieces<D, false>(s_img[0], mn_, nbs, slot, Bn[x], p, creg); }
-            else        { qaqc::section_bases<D, true>(mn_, nbs);  qaqc::write_pieces<D, true>(s_img[1], mn_, nbs, slot, Bn[x], p, creg); }
+            const uint32_t pl = s_place[x][slot];
+            qaqc::write_token<D>(s_img[x], s_tab[x][pl >> 8], x == 1, (int)(pl & 0xFFu), (int)(pl >> 8), p, creg);
         }
     }
     __syncthreads();   // every old byte of the tile has been read, the image is complete
@@ -256,16 +273,25 @@ __global__ void __launch_bounds__(2 * D) requant_kernel(const RequantArgs a) {
         const uint32_t off = s_off[x];
         uint8_t* dst = ts.codes + (size_t)bh * a.pool_bytes + off;
         const uint32_t nb = s_tot[x], nb16 = (nb + 15u) & ~15u;
-        for (uint32_t o = tid * 16; o < nb16; o += NT * 16)
-            *reinterpret_cast<uint4*>(dst + o) = *reinterpret_cast<const uint4*>(s_img[x] + o);
-        if (valid && p == 0) ts.bits[mt] = (uint8_t)Bn[x];
+        if (x == 0) {
+            for (uint32_t o = tid * 16; o < nb16; o += NT * 16)
+                *reinterpret_cast<uint4*>(dst + o) = *reinterpret_cast<const uint4*>(s_img[x] + o);
+        } else {
+            const int row = (tid / (16 * P)) * 4 + (tid & 3), e = (tid >> 2) % (4 * P);
+            if (row < s_tab[x][1].start + s_tab[x][1].n) {
+                const int w = s_sorted[x][4 * row];
+                qaqc::group_out<D>(s_img[x], dst, s_tab[x][w], w, row, e);
+            }
+            if (tid == 0) *reinterpret_cast<uint4*>(dst) = *reinterpret_cast<const uint4*>(s_img[x]);
+        }
+        if (valid && p == 0) ts.bs[mt] = (unsigned short)(Bn[x] | ((s_place[x][slot] & 0xFFu) << 8));
         if (tid == 0) {
             // an open tile that is still the last thing in its pool gives back what it no longer needs:
             // appends continue right behind its bytes
-            const uint32_t old_off = ts.tile_off[ti], old_nb = ts.tile_nbytes[ti];
+            const uint32_t old_off = ts.tile[ti].x, old_nb = ts.tile[ti].y;
             if (open && off == old_off && nb < old_nb && old_off + old_nb == ts.pool_end[bh]) ts.pool_end[bh] = off + nb;
-            ts.tile_off[ti] = off;
-            ts.tile_nbytes[ti] = nb;
+            ts.tile[ti].x = off;
+            ts.tile[ti].y = nb;
         }
     }
 }
@@ -369,7 +395,7 @@ __global__ void __launch_bounds__(256) compact_kernel(const CompactArgs a) {
     while (n2 < nt) n2 <<= 1;
     const size_t row = (size_t)bh * a.ntiles;
     for (int i = threadIdx.x; i < n2; i += blockDim.x)
-        s_key[i] = i < nt ? ((unsigned long long)ts.tile_off[row + i] << 32) | (unsigned)i : ~0ull;
+        s_key[i] = i < nt ? ((unsigned long long)ts.tile[row + i].x << 32) | (unsigned)i : ~0ull;
     __syncthreads();
     // bitonic sort by current offset
     for (int k = 2; k <= n2; k <<= 1)
@@ -389,7 +415,7 @@ __global__ void __launch_bounds__(256) compact_kernel(const CompactArgs a) {
     for (int s = 0; s < nt; ++s) {
         const uint32_t src = (uint32_t)(s_key[s] >> 32);
         const int tile = (int)(s_key[s] & 0xFFFFFFFFu);
-        const uint32_t n = ts.tile_nbytes[row + tile];
+        const uint32_t n = ts.tile[row + tile].y;
         const uint32_t n16 = (n + 15u) & ~15u;
         if (src != dst) {                                  // dst < src: tiles before this one only moved down
             for (uint32_t o = 0; o < n16; o += 256 * 16) {
@@ -399,7 +425,7 @@ __global__ void __launch_bounds__(256) compact_kernel(const CompactArgs a) {
                 __syncthreads();
                 if (b < n16) *reinterpret_cast<uint4*>(pool + dst + b) = v;
             }
-            if (threadIdx.x == 0) ts.tile_off[row + tile] = dst;
+            if (threadIdx.x == 0) ts.tile[row + tile].x = dst;
         }
         // closed tiles own a 16-byte rounded amount; the open tile, which is the last one, its exact bytes
         const bool open = tile == a.T / QAQ_TILE && (a.T % QAQ_TILE) != 0;
@@ -409,10 +435,11 @@ __global__ void __launch_bounds__(256) compact_kernel(const CompactArgs a) {
     if (threadIdx.x == 0) ts.pool_end[bh] = dst;
 }
 
-__global__ void pool_use_kernel(TensorStore tk, TensorStore tv, int BH, unsigned int* out) {
+// (a pool end can stand beyond the pool's capacity when takers that found no room could not give their space back)
+__global__ void pool_use_kernel(TensorStore tk, TensorStore tv, int BH, unsigned int cap, unsigned int* out) {
     for (int i = blockIdx.x * blockDim.x + threadIdx.x; i < BH; i += gridDim.x * blockDim.x) {
-        atomicMax(&out[0], tk.pool_end[i]);
-        atomicMax(&out[1], tv.pool_end[i]);
+        atomicMax(&out[0], min(tk.pool_end[i], cap));
+        atomicMax(&out[1], min(tv.pool_end[i], cap));
     }
 }
 
@@ -435,7 +462,7 @@ extern "C" qaq_status qaq_cache_pool_use(const qaq_cache* c, long* host_used, lo
     cudaStream_t s = (cudaStream_t)stream;
     unsigned int* d = (unsigned int*)c->d_status + 2;      // two spare words behind the status word
     QAQ_CUDA_TRY(cudaMemsetAsync(d, 0, 8, s));
-    pool_use_kernel<<<32, 256, 0, s>>>(c->t[0], c->t[1], c->BH, d);
+    pool_use_kernel<<<32, 256, 0, s>>>(c->t[0], c->t[1], c->BH, (unsigned)c->pool_bytes, d);
     QAQ_CUDA_TRY(cudaGetLastError());
     unsigned int h[2] = {0, 0};
     QAQ_CUDA_TRY(cudaMemcpyAsync(h, d, 8, cudaMemcpyDeviceToHost, s));
