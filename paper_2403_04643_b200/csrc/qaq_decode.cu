@@ -19,9 +19,7 @@
 //         signed byte digits in two columns per query (q_d ~ qscale * (256 * hi_d + lo_d)).
 //   S.V:  m16n8k16, rows = 16 channels, k = 16 slots of one width; B = the per-token weights p_t * step_t in 28-bit
 //         fixed point, four byte digits in four columns per query.  The sums of consecutive tiles stay in the integer
-//         accumulators while they share the reference of the exponentials and the size of a unit.  The rounded weight
-//         of a token is also what the softmax denominator and the constant part of its values use, so numerator and
-//         denominator see the same slightly perturbed probability.
+//         accumulators while they share the reference of the exponentials and the size of a unit.
 //
 // One CTA = one run of consecutive tiles of the flattened (b,h, tile) sequence (runs of equal length, so every SM
 // gets the same amount of work); each warp works through whole tiles (QAQ_TILE tokens) on its own, with its own
@@ -133,7 +131,7 @@ struct DecArgs {
     const __half* q;
     long q_stride, out_stride;   // elements between the rows of consecutive (b,h) in q and in out (queries of a (b,h) are D apart)
     float scale;
-    float* part;       // [ncta][2][NQ][D+4]: accumulators, reference of the exponentials, sum of the weights used, exact sum
+    float* part;       // [ncta][2][NQ][D+4]: accumulators, reference of the exponentials, sum of p
     unsigned long long* done;    // [BH]: tag of the call | partials that are complete (see finish_split)
     unsigned long long tag;      // of this call; the low 12 bits are zero
     float* ml;         // [BH][2]   merged (max, sum) for the normalisation of long score rows, or null
@@ -189,9 +187,9 @@ template <int D, int NQ>
 struct DecSmem {
     WarpScratch<D, NQ> ws[Shape<NQ>::WARPS];
     alignas(16) float qf[D][NQ];
-    alignas(16) uint32_t qw[32][D / 16];      // operand words of q per lane: low and high nibbles of its first word, of its second, ...
-    float mm[Shape<NQ>::WARPS][NQ], ml[Shape<NQ>::WARPS][NQ], mlx[Shape<NQ>::WARPS], cs[Shape<NQ>::WARPS][NQ];
-    float red[3 * Shape<NQ>::WARPS];
+    alignas(16) uint32_t qw[2][32][D / 32];   // operand words of q per lane: low nibbles of its words, high nibbles
+    float mm[Shape<NQ>::WARPS][NQ], ml[Shape<NQ>::WARPS][NQ], cs[Shape<NQ>::WARPS][NQ];
+    float red[2 * Shape<NQ>::WARPS];
     int flag;
 };
 
@@ -349,8 +347,8 @@ __device__ __forceinline__ void fixed_unit(float x, float& inv, float& unit) {
 
 // The score row of one (b,h), normalised in place by the whole CTA.
 template <int THREADS>
-__device__ __forceinline__ void normalise_scores(float* row, int T, float M, float LX) {
-    const float inv = LX > 0.f ? 1.0f / LX : 0.f;
+__device__ __forceinline__ void normalise_scores(float* row, int T, float M, float L) {
+    const float inv = L > 0.f ? 1.0f / L : 0.f;
     int t = threadIdx.x;
     for (; t + 7 * THREADS < T; t += 8 * THREADS) {
         float x[8];
@@ -407,21 +405,19 @@ __device__ void finish_split(const DecArgs& a, DecSmem<D, NQ>& sm, int bh, int n
         M = sm.red[0];
 #pragma unroll
         for (int w = 1; w < S::WARPS; ++w) M = fmaxf(M, sm.red[w]);
-        float L = 0.f, LX = 0.f;
+        float L = 0.f;
         for (int i = tid; i < n; i += S::THREADS) {
-            const float4 h = __ldcg(reinterpret_cast<const float4*>(part(i, j) + D));    // reference, sums
+            const float2 h = __ldcg(reinterpret_cast<const float2*>(part(i, j) + D));    // reference, sum
             const float w = h.x == __int_as_float(0xff800000) ? 0.f : __expf(h.x - M);
             s_w[i] = w;
             L = fmaf(w, h.y, L);
-            LX = fmaf(w, h.z, LX);
         }
         L = warp_sum(L);
-        LX = warp_sum(LX);
-        if (lane == 0) { sm.red[S::WARPS + warp] = L; sm.red[2 * S::WARPS + warp] = LX; }
+        if (lane == 0) sm.red[S::WARPS + warp] = L;
         __syncthreads();
-        L = 0.f; LX = 0.f;
+        L = 0.f;
 #pragma unroll
-        for (int w = 0; w < S::WARPS; ++w) { L += sm.red[S::WARPS + w]; LX += sm.red[2 * S::WARPS + w]; }
+        for (int w = 0; w < S::WARPS; ++w) L += sm.red[S::WARPS + w];
         // ---- the channels: D/4 threads per partial, four channels each
         constexpr int CT = D / 4, SH = S::THREADS / CT;
         const int d4 = tid % CT, sh = tid / CT;
@@ -441,8 +437,8 @@ __device__ void finish_split(const DecArgs& a, DecSmem<D, NQ>& sm, int bh, int n
             a.out[(size_t)bh * a.out_stride + j * D + tid] = L > 0.f ? y / L : 0.f;
         }
         if (NQ == 1) {
-            if (a.ml && tid == 0) { a.ml[2 * bh] = M; a.ml[2 * bh + 1] = LX; }
-            if (a.scores && !a.ml) normalise_scores<S::THREADS>(a.scores + (size_t)bh * a.scores_stride, T, M, LX);
+            if (a.ml && tid == 0) { a.ml[2 * bh] = M; a.ml[2 * bh + 1] = L; }
+            if (a.scores && !a.ml) normalise_scores<S::THREADS>(a.scores + (size_t)bh * a.scores_stride, T, M, L);
         } else {
             __syncthreads();
         }
@@ -499,19 +495,19 @@ __global__ void __launch_bounds__(Shape<NQ>::THREADS, Shape<NQ>::CTAS_PER_SM) de
     const uint32_t* ogV = a.v.outl + (size_t)bh * a.ocap;
     const uint32_t buf = smem_addr(ws.buf), bar = smem_addr(ws.bar);
 
-    // ---- tile metadata in registers: the table words (offset and length of the bytes, first entry and length of the
-    //      outlier list), min/max, widths and slots of tokens 2*lane, 2*lane+1
-    struct Meta { uint4 tk, tv; uint2 mk, mv; uint32_t bk, bv; };
-    auto fetch_meta = [&](int tile) {
-        Meta m;
-        m.tk = m.tv = make_uint4(0u, 0u, 0u, 0u); m.mk = m.mv = make_uint2(0u, 0u); m.bk = m.bv = 0;
+    // ---- tile metadata: the table words (offset and length of the bytes, first entry and length of the outlier list),
+    //      min/max, widths and slots of tokens 2*lane, 2*lane+1; fetched as late as their latency allows
+    auto fetch_tab = [&](const uint4* tab, int tile) { return tile < tile_hi ? __ldg(tab + tile) : make_uint4(0u, 0u, 0u, 0u); };
+    struct Toks { uint2 mm; uint32_t b; };      // min | max << 16; width | slot << 8 of two tokens
+    auto fetch_toks = [&](const TensorStore& ts, int tile) {
+        Toks t;
+        t.mm = make_uint2(0u, 0u); t.b = 0;
         if (tile < tile_hi) {
-            m.tk = __ldg(tabK + tile); m.tv = __ldg(tabV + tile);
             const size_t t0 = mrow + (size_t)tile * QAQ_TILE;
-            m.mk = __ldg(reinterpret_cast<const uint2*>(a.k.mnmx + t0)); m.mv = __ldg(reinterpret_cast<const uint2*>(a.v.mnmx + t0));
-            m.bk = __ldg(reinterpret_cast<const uint32_t*>(a.k.bs + t0)); m.bv = __ldg(reinterpret_cast<const uint32_t*>(a.v.bs + t0));
+            t.mm = __ldg(reinterpret_cast<const uint2*>(ts.mnmx + t0));
+            t.b = __ldg(reinterpret_cast<const uint32_t*>(ts.bs + t0));
         }
-        return m;
+        return t;
     };
     // how a tile lies in the buffer: bytes of the tile and of the piece of the outlier list that comes with it (from the
     // 16-byte boundary before its first entry; what lies behind its last one belongs to the read-ahead margin of the
@@ -533,7 +529,8 @@ __global__ void __launch_bounds__(Shape<NQ>::THREADS, Shape<NQ>::CTAS_PER_SM) de
     };
 
     int tile = tile_lo + warp;
-    Meta cur = fetch_meta(tile);
+    uint4 tk = fetch_tab(tabK, tile), tv = fetch_tab(tabV, tile);
+    Toks kt = fetch_toks(a.k, tile);
     if (lane == 0 && first_seg) { bar_init(bar); bar_init(bar + 8); asm volatile("fence.proxy.async.shared::cta;" ::: "memory"); }
 
     first_seg = false;
@@ -556,9 +553,9 @@ __global__ void __launch_bounds__(Shape<NQ>::THREADS, Shape<NQ>::CTAS_PER_SM) de
         qtop = fmaxf(qtop, qmax);
     }
     __syncwarp();
-    if (tile < tile_hi) stage(buf, layout(cur.tk), poolK, ogK, cur.tk, 0);
-    for (int i = lane; i < WS::VC * D; i += 32) (&ws.vcorr[0][0])[i] = 0;
-    for (int i = lane; i < NQ * D; i += 32) (&ws.macc[0][0])[i] = 0.f;
+    if (tile < tile_hi) stage(buf, layout(tk), poolK, ogK, tk, 0);
+    for (int i = 4 * lane; i < WS::VC * D; i += 128) *reinterpret_cast<uint4*>(&ws.vcorr[0][0] + i) = make_uint4(0u, 0u, 0u, 0u);
+    for (int i = 4 * lane; i < NQ * D; i += 128) *reinterpret_cast<float4*>(&ws.macc[0][0] + i) = make_float4(0.f, 0.f, 0.f, 0.f);
     // ---- operand words of q for all lanes, one or two per thread: nibble word u of lane ln, its low (even r) or high
     //      nibbles; column ln / 4: the high (even) or low (odd) digit of query ln / 8
     for (int idx = tid; idx < 32 * 2 * P; idx += S::THREADS) {
@@ -581,12 +578,9 @@ __global__ void __launch_bounds__(Shape<NQ>::THREADS, Shape<NQ>::CTAS_PER_SM) de
                 v |= (uint32_t)(dg & 0xFF) << (8 * i);
             }
         }
-        sm.qw[ln][r] = v;
+        sm.qw[r & 1][ln][r >> 1] = v;
     }
     __syncthreads();
-    uint32_t qa[P], qb[P];
-#pragma unroll
-    for (int u = 0; u < P; ++u) { qa[u] = sm.qw[lane][2 * u]; qb[u] = sm.qw[lane][2 * u + 1]; }
     // digit rows of the value weights this lane feeds: columns 0..3 of the first query of a pair, 4..7 of the second
     const bool wuse = NQ > 1 || fg < 4;
     const uint32_t wrow = smem_addr(&ws.wts[0][NQ > 1 ? fg >> 2 : 0][fg & 3][4 * ft]);
@@ -600,7 +594,7 @@ __global__ void __launch_bounds__(Shape<NQ>::THREADS, Shape<NQ>::CTAS_PER_SM) de
         for (int mb = 0; mb < MB; ++mb) { acc[pr][mb][0] = 0; acc[pr][mb][1] = 0; acc[pr][mb][2] = 0; acc[pr][mb][3] = 0; }
     int held = 0;                // tiles in the accumulators: a tile adds less than 2^22 (64 tokens, 255 * 255), 500 of them fit
     float m_ref[NQ], wunit[NQ];  // exponentials are taken relative to this logit; weight of one fixed-point unit, a power of two
-    float l_run[NQ], c_run[NQ], lx_run = 0.f;       // over this lane's tokens: sum of p, of p * (min + step/2) of the values, of the unperturbed p
+    float l_run[NQ], c_run[NQ];       // over this lane's tokens: sum of p, of p * (min + step/2) of the values
 #pragma unroll
     for (int j = 0; j < NQ; ++j) { m_ref[j] = NEG; wunit[j] = 0.f; l_run[j] = 0.f; c_run[j] = 0.f; }
     auto flush = [&]() {
@@ -628,83 +622,104 @@ __global__ void __launch_bounds__(Shape<NQ>::THREADS, Shape<NQ>::CTAS_PER_SM) de
 
 #pragma unroll 1
     for (; tile < tile_hi; tile += S::WARPS) {
-        const Lay lk = layout(cur.tk), lv = layout(cur.tv);
+        const Lay lk = layout(tk), lv = layout(tv);
         const uint32_t tV = buf + STAGE - lv.nb - lv.lb;
         // the tile before is done with: this tile's values come in behind its keys, if there is room
         const bool besideV = lk.nb + lk.lb + lv.nb + lv.lb <= STAGE;
-        if (besideV) stage(tV, lv, poolV, ogV, cur.tv, 1);
-        const Meta nxt = fetch_meta(tile + S::WARPS);
+        if (besideV) stage(tV, lv, poolV, ogV, tv, 1);
+        const uint4 tk_next = fetch_tab(tabK, tile + S::WARPS);
+        const Toks vt = fetch_toks(a.v, tile);
         const bool has_next = tile + S::WARPS < tile_hi;
         const int t0 = tile * QAQ_TILE + 2 * lane;              // this lane's tokens: t0 and t0 + 1
         const bool val[2] = {t0 < T, t0 + 1 < T};
-        int B[2];
-        float stepK[2], midK[2];
+        int B[2], sl[2];             // width; slot (tokens that are not there: a place nobody reads)
+        float step[2], mid[2];
+        auto scalars = [&](const Toks& tt) {
 #pragma unroll
-        for (int j = 0; j < 2; ++j) {
-            const uint32_t mm = j ? cur.mk.y : cur.mk.x;
-            B[j] = val[j] ? (int)((cur.bk >> (16 * j)) & 15u) : 0;
-            const float mn = __half2float(__ushort_as_half((unsigned short)(mm & 0xFFFF))), mx = __half2float(__ushort_as_half((unsigned short)(mm >> 16)));
-            stepK[j] = val[j] ? qaqc::step_of(mn, mx, B[j]) : 0.f;
-            midK[j] = val[j] ? fmaf(0.5f, stepK[j], mn) : 0.f;
-        }
-        *reinterpret_cast<float2*>(&ws.mid[2 * lane]) = make_float2(midK[0], midK[1]);
+            for (int i = 0; i < 2; ++i) {
+                const uint32_t mm = i ? tt.mm.y : tt.mm.x, bs = tt.b >> (16 * i);
+                B[i] = val[i] ? (int)(bs & 15u) : 0;
+                sl[i] = B[i] ? (int)((bs >> 8) & (QAQ_TILE - 1)) : QAQ_TILE;
+                const float mn = __half2float(__ushort_as_half((unsigned short)(mm & 0xFFFF))), mx = __half2float(__ushort_as_half((unsigned short)(mm >> 16)));
+                step[i] = val[i] ? qaqc::step_of(mn, mx, B[i]) : 0.f;
+                mid[i] = val[i] ? fmaf(0.5f, step[i], mn) : 0.f;
+            }
+        };
+        // the largest magnitude among this lane's ranges, as a binary16 pattern
+        auto top_range = [&](const Toks& tt) {
+            const uint32_t m = __vmaxu2(tt.mm.x & 0x7FFF7FFFu, tt.mm.y & 0x7FFF7FFFu);
+            return max(m & 0xFFFFu, m >> 16);
+        };
+        scalars(kt);
+        *reinterpret_cast<float2*>(&ws.mid[2 * lane]) = make_float2(mid[0], mid[1]);
+#pragma unroll
+        for (int i = 0; i < NQ; ++i) *reinterpret_cast<uint4*>(&ws.kcorr[i][0][4 * lane]) = make_uint4(0u, 0u, 0u, 0u);
         bool landed = bar_wait(bar, phase & 1u);
         __syncwarp();
 
         // ---- K: integer dot products, list by list
         {
+            uint32_t qa[P], qb[P];
+            lds_words<P>(smem_addr(sm.qw[0][lane]), qa);
+            lds_words<P>(smem_addr(sm.qw[1][lane]), qb);
             uint4 h = *reinterpret_cast<const uint4*>(ws.buf);
-            if (!cur.tk.y || !landed) h = make_uint4(0u, 0u, 0u, 0u);
+            if (!tk.y || !landed) h = make_uint4(0u, 0u, 0u, 0u);
+            uint32_t dots = smem_addr(&ws.dot[0][0][0]);
 #pragma unroll 1
-            for (int pass = 0; pass < (h.y ? 2 : 1); ++pass) {
+            for (int pass = 0;; ++pass) {
                 const Lists l = lists_of<P>(h, pass);
-                uint32_t dots = smem_addr(&ws.dot[pass][0][0]);
                 k_list<D, 4, NQ>(buf + l.o4, l.n4, dots, qa, qb, fg, ft);
-                dots += l.n4 * 4 * NQ;
-                k_list<D, 3, NQ>(buf + l.o3, l.n3, dots, qa, qb, fg, ft);
-                dots += l.n3 * 4 * NQ;
-                k_list<D, 2, NQ>(buf + l.o2, l.n2, dots, qa, qb, fg, ft);
-                dots += l.n2 * 4 * NQ;
-                k_list<D, 1, NQ>(buf + l.o1, l.n1, dots, qa, qb, fg, ft);
+                k_list<D, 3, NQ>(buf + l.o3, l.n3, dots + l.n4 * 4 * NQ, qa, qb, fg, ft);
+                k_list<D, 2, NQ>(buf + l.o2, l.n2, dots + (l.n4 + l.n3) * 4 * NQ, qa, qb, fg, ft);
+                k_list<D, 1, NQ>(buf + l.o1, l.n1, dots + (l.n4 + l.n3 + l.n2) * 4 * NQ, qa, qb, fg, ft);
+                if (pass || !h.y) break;
+                dots += WS::DOTS * 4 * NQ;
             }
         }
-        // ---- key outliers: q_ch * (x - mid) per token
-        float kunit = 0.f;          // > 0: the corrections are one word in this unit; 0: none; < 0: two words
-        if (cur.tk.w && landed) {
-            const uint32_t oc = cur.tk.w, sc = min(min(oc, LIST_STAGED), lk.lb / 4 - (cur.tk.z & 3u));       // entries, of which staged
-            const uint32_t* list = reinterpret_cast<const uint32_t*>(ws.buf + lk.nb) + (cur.tk.z & 3u);
-#pragma unroll
-            for (int i = 0; i < NQ; ++i) *reinterpret_cast<uint4*>(&ws.kcorr[i][0][4 * lane]) = make_uint4(0u, 0u, 0u, 0u);
-            // largest value of the tile: outliers and ranges
-            uint32_t top = max(max(cur.mk.x & 0x7FFFu, (cur.mk.x >> 16) & 0x7FFFu), max(cur.mk.y & 0x7FFFu, (cur.mk.y >> 16) & 0x7FFFu));
-#pragma unroll 4
-            for (uint32_t e = lane; e < sc; e += 32) top = max(top, list[e] & 0x7FFFu);
-            top = sc == oc ? __reduce_max_sync(0xFFFFFFFFu, top) : SMALL_MAX + 1;
-            auto entry = [&](uint32_t v, int& tok, float& dx) {
+        // ---- key outliers: q_ch * (x - mid) per token; up to 128 entries stay in registers between the two looks at them
+        float kunit = 0.f;          // > 0: the corrections are one word in this unit; < 0: two words
+        if (tk.w && landed) {
+            const uint32_t oc = tk.w, sc = min(min(oc, LIST_STAGED), lk.lb / 4 - (tk.z & 3u));       // entries, of which staged
+            const uint32_t* list = reinterpret_cast<const uint32_t*>(ws.buf + lk.nb) + (tk.z & 3u);
+            auto term = [&](uint32_t v, float inv, int& tok, float (&tm)[NQ]) {
                 tok = (v >> 24) & (QAQ_TILE - 1);
-                dx = __half2float(__ushort_as_half((unsigned short)(v & 0xFFFF))) - ws.mid[tok];
-                return &sm.qf[(v >> 16) & (D - 1)][0];
+                const float dx = (__half2float(__ushort_as_half((unsigned short)(v & 0xFFFF))) - ws.mid[tok]) * inv;
+                const float* qv = &sm.qf[(v >> 16) & (D - 1)][0];
+#pragma unroll
+                for (int j = 0; j < NQ; ++j) tm[j] = qv[j] * dx;
             };
-            __syncwarp();
+            uint32_t e[4], top = top_range(kt);
+#pragma unroll
+            for (int k = 0; k < 4; ++k) {
+                e[k] = 0;
+                if (lane + 32u * k < sc) e[k] = list[lane + 32 * k];
+                top = max(top, e[k] & 0x7FFFu);
+            }
+#pragma unroll 1
+            for (uint32_t i = lane + 128; i < sc; i += 32) top = max(top, list[i] & 0x7FFFu);
+            top = sc == oc ? __reduce_max_sync(0xFFFFFFFFu, top) : SMALL_MAX + 1;
             if (top <= SMALL_MAX) {
                 float inv;
                 fixed_unit(qtop * 2.0f * __half2float(__ushort_as_half((unsigned short)top)), inv, kunit);
-#pragma unroll 4
-                for (uint32_t e = lane; e < sc; e += 32) {
-                    int tok; float dx;
-                    const float* qv = entry(list[e], tok, dx);
-                    dx *= inv;
+                auto add = [&](uint32_t v, bool there) {
+                    int tok; float tm[NQ];
+                    term(v, inv, tok, tm);
 #pragma unroll
-                    for (int j = 0; j < NQ; ++j) atomicAdd(&ws.kcorr[j][0][tok], __float2int_rn(qv[j] * dx));
-                }
+                    for (int j = 0; j < NQ; ++j) if (there) atomicAdd(&ws.kcorr[j][0][tok], __float2int_rn(tm[j]));
+                };
+#pragma unroll
+                for (int k = 0; k < 4; ++k)
+                    if (32u * k < sc) add(e[k], lane + 32u * k < sc);
+#pragma unroll 1
+                for (uint32_t i = 128; i < sc; i += 32) add(list[min(i + lane, sc - 1)], i + lane < sc);
             } else {
                 kunit = -1.0f;
 #pragma unroll 1
-                for (uint32_t e = lane; e < oc; e += 32) {
-                    int tok; float dx;
-                    const float* qv = entry(e < sc ? list[e] : __ldg(ogK + cur.tk.z + e), tok, dx);
+                for (uint32_t i = lane; i < oc; i += 32) {
+                    int tok; float tm[NQ];
+                    term(i < sc ? list[i] : __ldg(ogK + tk.z + i), 1.0f, tok, tm);
 #pragma unroll
-                    for (int j = 0; j < NQ; ++j) wide_add(&ws.kcorr[j][0][tok], &ws.kcorr[j][1][tok], qv[j] * dx);
+                    for (int j = 0; j < NQ; ++j) wide_add(&ws.kcorr[j][0][tok], &ws.kcorr[j][1][tok], tm[j]);
                 }
             }
         }
@@ -712,43 +727,37 @@ __global__ void __launch_bounds__(Shape<NQ>::THREADS, Shape<NQ>::CTAS_PER_SM) de
         // ---- logits of this lane's tokens
         float lg[NQ][2];
 #pragma unroll
-        for (int i = 0; i < 2; ++i) {
-            const int sl = (cur.bk >> (16 * i + 8)) & (QAQ_TILE - 1);
-#pragma unroll
-            for (int j = 0; j < NQ; ++j) {
-                int dot = B[i] ? ws.dot[0][sl][j] : 0;
-                if (B[i] > 4) dot += ws.dot[1][sl][j] << 4;
-                float kc = 0.f;
-                if (kunit > 0.f) kc = (float)ws.kcorr[j][0][2 * lane + i] * kunit;
-                else if (kunit < 0.f) kc = wide_sum(ws.kcorr[j][0][2 * lane + i], ws.kcorr[j][1][2 * lane + i]);
-                const float qk = fmaf(qscale[j] * stepK[i], (float)dot, fmaf(midK[i], qsum[j], kc));
-                lg[j][i] = val[i] ? a.scale * qk : NEG;
+        for (int j = 0; j < NQ; ++j) {
+            const int2 k0 = *reinterpret_cast<const int2*>(&ws.kcorr[j][0][2 * lane]);
+            float kc[2] = {(float)k0.x * kunit, (float)k0.y * kunit};
+            if (kunit < 0.f) {
+                const int2 k1 = *reinterpret_cast<const int2*>(&ws.kcorr[j][1][2 * lane]);
+                kc[0] = wide_sum(k0.x, k1.x); kc[1] = wide_sum(k0.y, k1.y);
             }
-            if (NQ == 1 && a.scores && val[i]) a.scores[(size_t)bh * a.scores_stride + t0 + i] = lg[0][i];
+#pragma unroll
+            for (int i = 0; i < 2; ++i) {
+                const int lo = ws.dot[0][sl[i]][j], hi = ws.dot[1][sl[i]][j];
+                const int dot = lo + (B[i] > 4 ? hi << 4 : 0);       // a token that is not there has step 0
+                const float qk = fmaf(qscale[j] * step[i], (float)dot, fmaf(mid[i], qsum[j], kc[i]));
+                lg[j][i] = val[i] ? a.scale * qk : NEG;
+                if (NQ == 1 && a.scores && val[i]) a.scores[(size_t)bh * a.scores_stride + t0 + i] = lg[j][i];
+            }
         }
         __syncwarp();
         // ---- the front of the buffer is free: start the copy of the next tile's keys (beside this tile's values)
-        if (!besideV) stage(tV, lv, poolV, ogV, cur.tv, 1);
-        const Lay ln = layout(nxt.tk);
+        if (!besideV) stage(tV, lv, poolV, ogV, tv, 1);
+        const Lay ln = layout(tk_next);
         const bool besideK = ln.nb + ln.lb + lv.nb + lv.lb <= STAGE;
-        if (has_next && besideK) stage(buf, ln, poolK, ogK, nxt.tk, 0);
+        if (has_next && besideK) stage(buf, ln, poolK, ogK, tk_next, 0);
+        const uint4 tv_next = fetch_tab(tabV, tile + S::WARPS);
+        kt = fetch_toks(a.k, tile + S::WARPS);
 
         // ---- p relative to a reference somewhat above the largest logit, which is moved only when a logit exceeds it (so
         //      p never exceeds 1), and value weights p * step as fixed point of up to 28 bits.  (A token's step falls with
-        //      its width, so next to a 2-bit token an 8-bit token of the same p has a weight 64 times smaller.)  p is
-        //      replaced by what the rounded weight stands for, so that the codes, the constant part and the softmax
-        //      denominator all see the same (slightly perturbed) probability.  The largest weight of every tile takes 21
-        //      bits or more: the unit stays while it takes between 2^21 and 2^28 units, and is set so that it takes 2^24
-        //      to 2^25.
-        float stepV[2], midV[2];
-#pragma unroll
-        for (int i = 0; i < 2; ++i) {
-            const uint32_t mm = i ? cur.mv.y : cur.mv.x;
-            B[i] = val[i] ? (int)((cur.bv >> (16 * i)) & 15u) : 0;
-            const float mn = __half2float(__ushort_as_half((unsigned short)(mm & 0xFFFF))), mx = __half2float(__ushort_as_half((unsigned short)(mm >> 16)));
-            stepV[i] = val[i] ? qaqc::step_of(mn, mx, B[i]) : 0.f;
-            midV[i] = val[i] ? fmaf(0.5f, stepV[i], mn) : 0.f;
-        }
+        //      its width, so next to a 2-bit token an 8-bit token of the same p has a weight 64 times smaller.)  The largest
+        //      weight of every tile takes 21 bits or more: the unit stays while it takes between 2^21 and 2^28 units, and is
+        //      set so that it takes 2^24 to 2^25.
+        scalars(vt);
         float alpha[NQ], wnew[NQ];
         bool wok[NQ], any_w = false, change = held == 500;
 #pragma unroll
@@ -762,9 +771,9 @@ __global__ void __launch_bounds__(Shape<NQ>::THREADS, Shape<NQ>::CTAS_PER_SM) de
             }
             lg[j][0] = __expf(lg[j][0] - m_ref[j]);              // from here on: p (0 for slots beyond T)
             lg[j][1] = __expf(lg[j][1] - m_ref[j]);
-            const float wmax = warp_max(fmaxf(B[0] ? lg[j][0] * stepV[0] : 0.f, B[1] ? lg[j][1] * stepV[1] : 0.f));
+            const float wmax = warp_max(fmaxf(lg[j][0] * step[0], lg[j][1] * step[1]));
             const int wex = (__float_as_int(wmax) >> 23) & 0xFF;
-            wok[j] = wex > 28 && wex < 255 && cur.tv.y;             // zero, tiny or non-finite weights: the codes add nothing
+            wok[j] = wex > 28 && wex < 255 && tv.y;             // zero, tiny or non-finite weights: the codes add nothing
             any_w = any_w || wok[j];
             wnew[j] = wunit[j];
             if (wok[j] && !(wmax >= 2097152.0f * wunit[j] && wmax < 268435440.0f * wunit[j])) {
@@ -781,39 +790,33 @@ __global__ void __launch_bounds__(Shape<NQ>::THREADS, Shape<NQ>::CTAS_PER_SM) de
 #pragma unroll
                     for (int k = 0; k < CPL; ++k) ws.macc[j][lane + 32 * k] *= alpha[j];
                     c_run[j] *= alpha[j]; l_run[j] *= alpha[j];
-                    if (NQ == 1) lx_run *= alpha[j];
                 }
             }
         }
+        const bool wide = __any_sync(0xFFFFFFFFu, max(B[0], B[1]) > 4);
 #pragma unroll
         for (int j = 0; j < NQ; ++j) {
             const float winv = wok[j] ? __int_as_float((254 << 23) - __float_as_int(wunit[j])) : 0.f;       // 1 / wunit
-            float2 pm[2];
 #pragma unroll
             for (int i = 0; i < 2; ++i) {
-                const uint32_t iw = __float2uint_rn(lg[j][i] * stepV[i] * winv);
-                float p = lg[j][i];
-                if (stepV[i] > 0.f && wok[j] && B[i]) p = __fdividef((float)iw * wunit[j], stepV[i]);
-                uint8_t* gp = &ws.wts[0][j][0][(cur.bv >> (16 * i + 8)) & (QAQ_TILE - 1)];
-                if (B[i]) {
-                    gp[0] = (uint8_t)(iw >> 24);
-                    gp[WS::WROW] = (uint8_t)(iw >> 16);
-                    gp[2 * WS::WROW] = (uint8_t)(iw >> 8);
-                    gp[3 * WS::WROW] = (uint8_t)iw;
-                }
-                if (B[i] > 4) {                      // 16 times the weight, for the bits above the low four
+                const uint32_t iw = __float2uint_rn(lg[j][i] * step[i] * winv);
+                uint8_t* gp = &ws.wts[0][j][0][sl[i]];
+                gp[0] = (uint8_t)(iw >> 24);
+                gp[WS::WROW] = (uint8_t)(iw >> 16);
+                gp[2 * WS::WROW] = (uint8_t)(iw >> 8);
+                gp[3 * WS::WROW] = (uint8_t)iw;
+                if (wide) {                          // 16 times the weight, for the bits above the low four
                     gp += 4 * NQ * WS::WROW;
                     gp[0] = (uint8_t)(iw >> 20);
                     gp[WS::WROW] = (uint8_t)(iw >> 12);
                     gp[2 * WS::WROW] = (uint8_t)(iw >> 4);
                     gp[3 * WS::WROW] = (uint8_t)(iw << 4);
                 }
-                pm[i] = make_float2(p, p * midV[i]);
-                c_run[j] += pm[i].y;
-                l_run[j] += p;
-                if (NQ == 1) lx_run += lg[j][i];
             }
-            *reinterpret_cast<float4*>(&ws.tok[j][2 * lane]) = make_float4(pm[0].x, pm[0].y, pm[1].x, pm[1].y);
+            const float c0 = lg[j][0] * mid[0], c1 = lg[j][1] * mid[1];
+            c_run[j] += c0 + c1;
+            l_run[j] += lg[j][0] + lg[j][1];
+            *reinterpret_cast<float4*>(&ws.tok[j][2 * lane]) = make_float4(lg[j][0], c0, lg[j][1], c1);
         }
         landed = bar_wait(bar + 8, phase & 1u) && landed;     // this tile's values are there
         __syncwarp();
@@ -821,44 +824,54 @@ __global__ void __launch_bounds__(Shape<NQ>::THREADS, Shape<NQ>::CTAS_PER_SM) de
         // ---- V: integer weighted sums, list by list
         if (any_w && landed) {
             const uint4 h = *reinterpret_cast<const uint4*>(ws.buf + STAGE - lv.nb - lv.lb);
+            uint32_t wt = wrow;
 #pragma unroll 1
-            for (int pass = 0; pass < (h.y ? 2 : 1); ++pass) {
+            for (int pass = 0;; ++pass) {
                 const Lists l = lists_of<D / 8>(h, pass);
-                uint32_t wt = wrow + pass * 4 * NQ * WS::WROW;
                 v_list<D, 4, NQ>(tV + l.o4, l.n4, wt, wuse, acc, fg, ft);
-                wt += 4 * l.n4;
-                v_list<D, 3, NQ>(tV + l.o3, l.n3, wt, wuse, acc, fg, ft);
-                wt += 4 * l.n3;
-                v_list<D, 2, NQ>(tV + l.o2, l.n2, wt, wuse, acc, fg, ft);
-                wt += 4 * l.n2;
-                v_list<D, 1, NQ>(tV + l.o1, l.n1, wt, wuse, acc, fg, ft);
+                v_list<D, 3, NQ>(tV + l.o3, l.n3, wt + 4 * l.n4, wuse, acc, fg, ft);
+                v_list<D, 2, NQ>(tV + l.o2, l.n2, wt + 4 * (l.n4 + l.n3), wuse, acc, fg, ft);
+                v_list<D, 1, NQ>(tV + l.o1, l.n1, wt + 4 * (l.n4 + l.n3 + l.n2), wuse, acc, fg, ft);
+                if (pass || !h.y) break;
+                wt += 4 * NQ * WS::WROW;
             }
             ++held;
         }
         // ---- value outliers: p_t * (v - mid) per channel
-        if (cur.tv.w && landed) {
-            const uint32_t oc = cur.tv.w, sc = min(min(oc, LIST_STAGED), lv.lb / 4 - (cur.tv.z & 3u));
-            const uint32_t* list = reinterpret_cast<const uint32_t*>(ws.buf + STAGE - lv.lb) + (cur.tv.z & 3u);
-            uint32_t top = max(max(cur.mv.x & 0x7FFFu, (cur.mv.x >> 16) & 0x7FFFu), max(cur.mv.y & 0x7FFFu, (cur.mv.y >> 16) & 0x7FFFu));
-#pragma unroll 4
-            for (uint32_t e = lane; e < sc; e += 32) top = max(top, list[e] & 0x7FFFu);
+        if (tv.w && landed) {
+            const uint32_t oc = tv.w, sc = min(min(oc, LIST_STAGED), lv.lb / 4 - (tv.z & 3u));
+            const uint32_t* list = reinterpret_cast<const uint32_t*>(ws.buf + STAGE - lv.lb) + (tv.z & 3u);
+            auto term = [&](uint32_t v, int j) {
+                const float2 pm = ws.tok[j][(v >> 24) & (QAQ_TILE - 1)];
+                return fmaf(__half2float(__ushort_as_half((unsigned short)(v & 0xFFFF))), pm.x, -pm.y);
+            };
+            uint32_t e[4], top = top_range(vt);
+#pragma unroll
+            for (int k = 0; k < 4; ++k) {
+                e[k] = 0;
+                if (lane + 32u * k < sc) e[k] = list[lane + 32 * k];
+                top = max(top, e[k] & 0x7FFFu);
+            }
+#pragma unroll 1
+            for (uint32_t i = lane + 128; i < sc; i += 32) top = max(top, list[i] & 0x7FFFu);
             top = sc == oc ? __reduce_max_sync(0xFFFFFFFFu, top) : SMALL_MAX + 1;
             if (top <= SMALL_MAX) {
                 float inv[NQ], unit[NQ];
 #pragma unroll
                 for (int j = 0; j < NQ; ++j)
                     fixed_unit(warp_max(fmaxf(lg[j][0], lg[j][1])) * 2.5f * __half2float(__ushort_as_half((unsigned short)top)), inv[j], unit[j]);
-#pragma unroll 4
-                for (uint32_t e = lane; e < sc; e += 32) {
-                    const uint32_t v = list[e];
-                    const int tk = (v >> 24) & (QAQ_TILE - 1), ch = (v >> 16) & (D - 1);
-                    const float x = __half2float(__ushort_as_half((unsigned short)(v & 0xFFFF)));
+                auto add = [&](uint32_t v, bool there) {
 #pragma unroll
                     for (int j = 0; j < NQ; ++j) {
-                        const float2 pm = ws.tok[j][tk];
-                        atomicAdd(&ws.vcorr[j][ch], __float2int_rn(fmaf(x, pm.x, -pm.y) * inv[j]));
+                        const int x = __float2int_rn(term(v, j) * inv[j]);
+                        if (there) atomicAdd(&ws.vcorr[j][(v >> 16) & (D - 1)], x);
                     }
-                }
+                };
+#pragma unroll
+                for (int k = 0; k < 4; ++k)
+                    if (32u * k < sc) add(e[k], lane + 32u * k < sc);
+#pragma unroll 1
+                for (uint32_t i = 128; i < sc; i += 32) add(list[min(i + lane, sc - 1)], i + lane < sc);
                 __syncwarp();
 #pragma unroll
                 for (int j = 0; j < NQ; ++j)
@@ -872,11 +885,10 @@ __global__ void __launch_bounds__(Shape<NQ>::THREADS, Shape<NQ>::CTAS_PER_SM) de
 #pragma unroll 1
                 for (int j = 0; j < NQ; ++j) {
 #pragma unroll 1
-                    for (uint32_t e = lane; e < oc; e += 32) {
-                        const uint32_t v = e < sc ? list[e] : __ldg(ogV + cur.tv.z + e);
-                        const int tk = (v >> 24) & (QAQ_TILE - 1), ch = (v >> 16) & (D - 1);
-                        const float2 pm = ws.tok[j][tk];
-                        wide_add(&ws.vcorr[0][ch], &ws.vcorr[1][ch], fmaf(__half2float(__ushort_as_half((unsigned short)(v & 0xFFFF))), pm.x, -pm.y));
+                    for (uint32_t i = lane; i < oc; i += 32) {
+                        const uint32_t v = i < sc ? list[i] : __ldg(ogV + tv.z + i);
+                        const int ch = (v >> 16) & (D - 1);
+                        wide_add(&ws.vcorr[0][ch], &ws.vcorr[1][ch], term(v, j));
                     }
                     __syncwarp();
 #pragma unroll
@@ -890,10 +902,11 @@ __global__ void __launch_bounds__(Shape<NQ>::THREADS, Shape<NQ>::CTAS_PER_SM) de
             }
         }
         __syncwarp();
-        if (has_next && !besideK) stage(buf, ln, poolK, ogK, nxt.tk, 0);
+        if (has_next && !besideK) stage(buf, ln, poolK, ogK, tk_next, 0);
         if (!landed) atomicMax(a.status, (int)QAQ_ERR_CUDA);
         phase ^= 1u;
-        cur = nxt;
+        tk = tk_next;
+        tv = tv_next;
     }
     if (held) flush();
 
@@ -903,10 +916,6 @@ __global__ void __launch_bounds__(Shape<NQ>::THREADS, Shape<NQ>::CTAS_PER_SM) de
         const float l = warp_sum(l_run[j]), cs = warp_sum(c_run[j]);
         if (lane == 0) { sm.mm[warp][j] = m_ref[j]; sm.ml[warp][j] = l; sm.cs[warp][j] = cs; }
     }
-    if (NQ == 1) {
-        const float lx = warp_sum(lx_run);
-        if (lane == 0) sm.mlx[warp] = lx;
-    }
     __syncthreads();
     // ---- merge the warps (log-sum-exp) into this segment's partial
     const bool alone = tile_hi - tile_lo == ntiles;        // the whole (b,h) in this CTA: nothing to merge with
@@ -915,24 +924,23 @@ __global__ void __launch_bounds__(Shape<NQ>::THREADS, Shape<NQ>::CTAS_PER_SM) de
         float M = NEG;
 #pragma unroll
         for (int i = 0; i < S::WARPS; ++i) M = fmaxf(M, sm.mm[i][j]);
-        float L = 0.f, LX = 0.f, x = 0.f;
+        float L = 0.f, x = 0.f;
 #pragma unroll
         for (int i = 0; i < S::WARPS; ++i) {
             const float wgt = sm.mm[i][j] == NEG ? 0.f : __expf(sm.mm[i][j] - M);
             L = fmaf(wgt, sm.ml[i][j], L);
-            if (NQ == 1) LX = fmaf(wgt, sm.mlx[i], LX);
             if (tid < D) x = fmaf(wgt, sm.ws[i].macc[j][tid] + sm.cs[i][j], x);
         }
         float* dst = a.part + ((size_t)(2 * cta + seg) * NQ + j) * (D + 4);
         if (alone) {
             if (tid < D) a.out[(size_t)bh * a.out_stride + j * D + tid] = L > 0.f ? x / L : 0.f;
             if (NQ == 1) {
-                if (a.ml && tid == 0) { a.ml[2 * bh] = M; a.ml[2 * bh + 1] = LX; }
-                if (a.scores && !a.ml) normalise_scores<S::THREADS>(a.scores + (size_t)bh * a.scores_stride, T, M, LX);
+                if (a.ml && tid == 0) { a.ml[2 * bh] = M; a.ml[2 * bh + 1] = L; }
+                if (a.scores && !a.ml) normalise_scores<S::THREADS>(a.scores + (size_t)bh * a.scores_stride, T, M, L);
             }
         } else {
             if (tid < D) __stcg(dst + tid, x);
-            if (tid == 0) __stcg(reinterpret_cast<float4*>(dst + D), make_float4(M, L, LX, 0.f));
+            if (tid == 0) __stcg(reinterpret_cast<float2*>(dst + D), make_float2(M, L));
         }
     }
     if (!alone) finish_split<D, NQ>(a, sm, bh, ntiles, run, T);
