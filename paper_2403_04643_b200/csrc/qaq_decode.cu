@@ -22,8 +22,10 @@
 //         accumulators while they share the reference of the exponentials and the size of a unit.
 //
 // One CTA = one run of consecutive tiles of the flattened (b,h, tile) sequence (runs of equal length, so every SM
-// gets the same amount of work); each warp works through whole tiles (QAQ_TILE tokens) on its own, with its own
-// running sums and no CTA barrier in the tile loop; warps are merged once at the end.  Lane l looks after tokens 2l and
+// gets the same amount of work), cut once more into one piece per warp; each warp works through its tiles (QAQ_TILE
+// tokens) on its own, with its own running sums and no CTA barrier; warps are merged once at the end.  (With the tiles
+// of a (b,h) dealt out to the warps in turn, warps waited for each other at every (b,h) boundary: 11 % of a 7B layer at
+// batch 8.)  Lane l looks after tokens 2l and
 // 2l + 1 of the tile (logit, softmax weight, value weight); the tokens of a tile are stored sorted by width, so the
 // section loops run one extraction routine over full row blocks, write dot products and read weights by slot, and a
 // token finds its own through the slot in its metadata.
@@ -114,8 +116,17 @@ __device__ __forceinline__ float warp_sum(float x) {
 // ------------------------------------------------------------------------------------------ shapes
 // Warps per CTA and CTAs per SM by queries per pass: 16 warps per SM for one query (128 registers each), 12 for four
 // (168 registers: four times the accumulators on the value side).
+#ifndef DEC_W1
+#define DEC_W1 8
+#define DEC_C1 2
+#define DEC_ST1 84
+#endif
+#ifndef DEC_W4
+#define DEC_W4 4
+#define DEC_C4 3
+#endif
 template <int NQ> struct Shape {
-    static constexpr int WARPS = NQ == 4 ? 4 : 8, CTAS_PER_SM = NQ == 4 ? 3 : 2, THREADS = 32 * WARPS, SLOTS = 148 * CTAS_PER_SM;
+    static constexpr int WARPS = NQ == 4 ? DEC_W4 : (NQ == 2 ? 8 : DEC_W1), CTAS_PER_SM = NQ == 4 ? DEC_C4 : (NQ == 2 ? 2 : DEC_C1), THREADS = 32 * WARPS, SLOTS = 148 * CTAS_PER_SM;
 };
 constexpr int SCORES_FUSED_TOKENS = 8192;          // up to here the CTA that merges a (b,h) normalises its score row too
 constexpr uint32_t LIST_STAGED = 1024;             // outlier entries per tile and tensor that come through shared memory at most; more are read in place
@@ -143,15 +154,14 @@ struct DecArgs {
 };
 
 // The flattened sequence of BH * ntiles tiles is cut into runs of `run` consecutive tiles, one CTA
-// each: enough CTAs to fill every SM evenly, at least one tile per warp where there are that many, and never more than
-// one (b,h) boundary inside a run.
+// each, and a run into pieces of ceil(run / warps), one warp each: as few tiles per warp as fill every SM evenly, and
+// never more than one (b,h) boundary inside a run.
 struct DecPlan { int run, ncta; };
 template <int NQ>
 __host__ __device__ inline DecPlan plan_decode(int BH, int ntiles) {
-    const long long total = (long long)BH * ntiles;
-    long long run = (total + Shape<NQ>::SLOTS - 1) / Shape<NQ>::SLOTS;
-    const int floor_run = ntiles < Shape<NQ>::WARPS ? ntiles : Shape<NQ>::WARPS;
-    if (run < floor_run) run = floor_run;
+    using S = Shape<NQ>;
+    const long long total = (long long)BH * ntiles, warps = (long long)S::SLOTS * S::WARPS;
+    long long run = (total + warps - 1) / warps * S::WARPS;
     if (run > ntiles) run = ntiles;
     DecPlan p;
     p.run = (int)run;
@@ -163,34 +173,39 @@ __host__ __device__ inline DecPlan plan_decode(int BH, int ntiles) {
 // per-warp scratch for the tile a warp is working on
 template <int D, int NQ>
 struct WarpScratch {
-    static constexpr int STAGE = (NQ == 1 ? 86 : 72) * D;      // bytes of the staging buffer; any tile of one tensor fits alone
+    static constexpr int STAGE = (NQ == 1 ? DEC_ST1 : 72) * D;      // bytes of the staging buffer; any tile of one tensor fits alone
     static constexpr int DOTS = QAQ_TILE + 16;                 // the last row block of a list may store up to 15 rows too many
     static constexpr int WROW = QAQ_TILE + 4;                  // digit rows are spread over the banks
     static constexpr int VC = NQ < 2 ? 2 : NQ;
     static_assert(STAGE % 16 == 0 && STAGE >= qaqc::tile_bytes_max(D), "staging buffer");
     alignas(16) uint8_t buf[STAGE];           // keys (tile, outlier list) from the front, values to the back
-    union alignas(16) {                       // the key phase is over (logits taken) before the value weights are written
+    union alignas(16) {                       // used one after the other: key phase (until the logits are taken), value lists, value outliers
         int dot[2][DOTS][NQ];                 // integer q . (low 4 bits of the code), q . (the bits above) by slot
         uint8_t wts[2][NQ][4][WROW];          // the four byte digits (highest first) of the value weights, and of 16 times them, by slot
+        int vcorr[VC][D];                     // fixed-point sums of the value-outlier corrections per channel
     };
     union alignas(16) {                       // likewise
         int kcorr[NQ][2][QAQ_TILE];           // fixed-point sums of the key-outlier corrections per token (second word: the low part)
         float2 tok[NQ][QAQ_TILE];             // p, p * (min + step/2) of the values
     };
     alignas(8) float mid[QAQ_TILE];           // min + step/2 of the keys
-    alignas(16) int vcorr[VC][D];             // fixed-point sums of the value-outlier corrections per channel (zero between uses)
     alignas(16) float macc[NQ][D];            // weighted sums of the values, as far as they have left the integer accumulators
     alignas(8) unsigned long long bar[2];     // transaction barriers of the keys and of the values
 };
 
 template <int D, int NQ>
 struct DecSmem {
-    WarpScratch<D, NQ> ws[Shape<NQ>::WARPS];
-    alignas(16) float qf[D][NQ];
-    alignas(16) uint32_t qw[2][32][D / 32];   // operand words of q per lane: low nibbles of its words, high nibbles
-    float mm[Shape<NQ>::WARPS][NQ], ml[Shape<NQ>::WARPS][NQ], cs[Shape<NQ>::WARPS][NQ];
-    float red[2 * Shape<NQ>::WARPS];
-    int flag;
+    static constexpr int W = Shape<NQ>::WARPS;
+    WarpScratch<D, NQ> ws[W];
+    alignas(16) float qf[2][D][NQ];           // the queries of the run's two (b,h)
+    alignas(16) uint32_t qw[2][2][32][D / 32];// operand words of q per lane: low nibbles of its words, high nibbles
+    float qscale[2][NQ], qsum[2][NQ];
+    // results of the warps; the warp that meets the (b,h) boundary leaves what it has of the first one in entry W
+    float cross[NQ][D];
+    float mm[W + 1][NQ], ml[W + 1][NQ], cs[W + 1][NQ];
+    int seg[W + 1];                           // which of the two (b,h) an entry belongs to, -1: none
+    float red[2 * W];
+    int last[2];
 };
 
 // ------------------------------------------------------------------------------------------ lists of rows
@@ -360,41 +375,47 @@ __device__ __forceinline__ void normalise_scores(float* row, int T, float M, flo
     for (; t < T; t += THREADS) row[t] = __expf(__ldcg(row + t) - M) * inv;
 }
 
-// The partial of this CTA's segment is complete (written by all threads).  The CTA that finds all partials of the
-// (b,h) complete merges them (log-sum-exp), in CTA order, so the result does not depend on which one it is.
+// The CTA that finds all partials of a (b,h) complete merges them (log-sum-exp), in CTA order, so the result does not
+// depend on which one it is.
 //
 // The CTAs are counted in a word of the workspace, which comes uninitialised: the count carries the tag of the call, a
 // number no other call uses, and a word with another tag counts as zero.  The last CTA clears the word, so that a replay
 // of the same launch (a CUDA graph carries the same tag) starts from zero again.
+__device__ __forceinline__ bool count_partial(unsigned long long* word, unsigned long long tag, int n) {
+    asm volatile("fence.acq_rel.gpu;" ::: "memory");
+    unsigned long long cur = *(volatile unsigned long long*)word, next;
+    for (;;) {           // a failed exchange means that another CTA has been counted: at most n rounds
+        next = ((cur ^ tag) >> 12) == 0 ? cur + 1 : tag + 1;
+        const unsigned long long was = atomicCAS(word, cur, next);
+        if (was == cur) break;
+        cur = was;
+    }
+    const bool last = (int)(next & 0xFFF) == n;
+    if (last) *word = 0ull;
+    asm volatile("fence.acq_rel.gpu;" ::: "memory");
+    return last;
+}
+
+// The CTAs whose runs meet a (b,h): the first of them and how many; only the first can have begun in the (b,h) before
+// (then the partial is that of its second segment).
+__device__ __forceinline__ void split_of(int bh, int ntiles, int run, int& first, int& n) {
+    first = (bh * ntiles) / run;
+    n = ((bh + 1) * ntiles - 1) / run - first + 1;
+}
+
+// log-sum-exp merge of the partials of a (b,h), by the whole CTA
 template <int D, int NQ>
-__device__ void finish_split(const DecArgs& a, DecSmem<D, NQ>& sm, int bh, int ntiles, int run, int T) {
+__device__ void merge_split(const DecArgs& a, DecSmem<D, NQ>& sm, int bh, int ntiles, int run, int T) {
     using S = Shape<NQ>;
-    const int c_lo = (bh * ntiles) / run, n = ((bh + 1) * ntiles - 1) / run - c_lo + 1;
-    // the CTAs whose runs meet this (b,h); only the first of them can have begun in the (b,h) before (then its second segment)
+    int c_lo, n;
+    split_of(bh, ntiles, run, c_lo, n);
     const int first_slot = 2 * c_lo + (c_lo * run < bh * ntiles ? 1 : 0);
     constexpr int PS = D + 4;
     auto part = [&](int i, int j) { return a.part + ((size_t)(i == 0 ? first_slot : 2 * (c_lo + i)) * NQ + j) * PS; };
     const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
-    __syncthreads();
-    if (tid == 0) {
-        asm volatile("fence.acq_rel.gpu;" ::: "memory");
-        unsigned long long cur = *(volatile unsigned long long*)(a.done + bh), next;
-        for (;;) {           // a failed exchange means that another CTA has been counted: at most n rounds
-            next = ((cur ^ a.tag) >> 12) == 0 ? cur + 1 : a.tag + 1;
-            const unsigned long long was = atomicCAS(a.done + bh, cur, next);
-            if (was == cur) break;
-            cur = was;
-        }
-        const bool last = (int)(next & 0xFFF) == n;
-        if (last) a.done[bh] = 0ull;
-        asm volatile("fence.acq_rel.gpu;" ::: "memory");
-        sm.flag = last;
-    }
-    __syncthreads();
-    if (!sm.flag) return;
     float* s_w = reinterpret_cast<float*>(sm.ws[0].buf);            // [n] <= SLOTS
     float4* s_x = reinterpret_cast<float4*>(sm.ws[1].buf);          // [THREADS]
-    static_assert(S::SLOTS * sizeof(float) <= sizeof(sm.ws[0].buf) && S::THREADS * sizeof(float4) <= sizeof(sm.ws[1]), "scratch of the merge");
+    static_assert(S::SLOTS * sizeof(float) <= sizeof(sm.ws[0].buf) && S::THREADS * sizeof(float4) <= 2 * sizeof(sm.ws[0]), "scratch of the merge");
     for (int j = 0; j < NQ; ++j) {
         // ---- weights of the partials, sums of the softmax denominators
         float M = __int_as_float(0xff800000);
@@ -439,14 +460,13 @@ __device__ void finish_split(const DecArgs& a, DecSmem<D, NQ>& sm, int bh, int n
         if (NQ == 1) {
             if (a.ml && tid == 0) { a.ml[2 * bh] = M; a.ml[2 * bh + 1] = L; }
             if (a.scores && !a.ml) normalise_scores<S::THREADS>(a.scores + (size_t)bh * a.scores_stride, T, M, L);
-        } else {
-            __syncthreads();
         }
+        __syncthreads();
     }
 }
 
-// The body runs once per (b,h) segment of the CTA's run (one or two) and leaves one partial per segment, or the result
-// where a (b,h) is one CTA's alone.  In the section loops lane 4g+t is lane (g, t) of the tensor-core fragments.
+// A CTA's run meets one or two (b,h); it leaves one partial for each, or the result where a (b,h) is one CTA's alone.
+// In the loops over lists lane 4g+t is lane (g, t) of the tensor-core fragments.
 // COUNTED: the token count is read from device memory and the split derived from it here (the grid is then the
 // largest one any count needs; CTAs beyond the split find no tiles and leave).
 template <int D, int NQ, bool COUNTED>
@@ -470,40 +490,33 @@ __global__ void __launch_bounds__(Shape<NQ>::THREADS, Shape<NQ>::CTAS_PER_SM) de
             if (tid < D) a.out[(size_t)bh * a.out_stride + tid] = 0.f;
         return;
     }
-    const int run = COUNTED ? plan_decode<NQ>(a.BH, (T + QAQ_TILE - 1) / QAQ_TILE).run : a.run;
-
-    uint32_t phase = 0;          // of the warp's two transaction barriers
-    bool first_seg = true;
-#pragma unroll 1
-    for (int seg = 0; seg < 2; ++seg) {
-    // this CTA's run of the flattened (b,h, tile) sequence; it touches at most two (b,h).  The block
-    // index is read afresh for each segment so that none of this stays in registers over the tile loop.
-    int cta;
-    asm volatile("mov.u32 %0, %%ctaid.x;" : "=r"(cta));
+    // this CTA's run of the flattened (b,h, tile) sequence: it begins in bh0 and may reach into bh0 + 1, which begins at f_bound
     const int ntiles = (T + QAQ_TILE - 1) / QAQ_TILE;
-    const int flat_lo = cta * run, flat_hi = min(a.BH * ntiles, flat_lo + run);
-    const int bh = flat_lo / ntiles + seg;
-    const int tile_lo = max(flat_lo, bh * ntiles) - bh * ntiles, tile_hi = min(flat_hi, (bh + 1) * ntiles) - bh * ntiles;
-    if (tile_lo >= tile_hi) continue;   // the same for every thread of the CTA
-
-    const size_t mrow = (size_t)bh * a.tmax_pad + 2 * lane;
-    const uint4* tabK = a.k.tile + (size_t)bh * a.ntiles_max;
-    const uint4* tabV = a.v.tile + (size_t)bh * a.ntiles_max;
-    const uint8_t* poolK = a.k.codes + (size_t)bh * a.pool_bytes;
-    const uint8_t* poolV = a.v.codes + (size_t)bh * a.pool_bytes;
-    const uint32_t* ogK = a.k.outl + (size_t)bh * a.ocap;
-    const uint32_t* ogV = a.v.outl + (size_t)bh * a.ocap;
+    const int run = COUNTED ? plan_decode<NQ>(a.BH, ntiles).run : a.run;
+    const int flat_lo = blockIdx.x * run, flat_hi = min(a.BH * ntiles, flat_lo + run);
+    if (flat_lo >= flat_hi) return;
+    const int bh0 = flat_lo / ntiles, f_bound = (bh0 + 1) * ntiles;
+    const int nseg = flat_hi > f_bound ? 2 : 1;
+    // this warp's piece of it
+    const int piece = (run + S::WARPS - 1) / S::WARPS;
+    int f = flat_lo + warp * piece;
+    const int f_end = min(f + piece, flat_hi);
+    auto bh_of = [&](int i) { return bh0 + (i >= f_bound ? 1 : 0); };
     const uint32_t buf = smem_addr(ws.buf), bar = smem_addr(ws.bar);
 
     // ---- tile metadata: the table words (offset and length of the bytes, first entry and length of the outlier list),
     //      min/max, widths and slots of tokens 2*lane, 2*lane+1; fetched as late as their latency allows
-    auto fetch_tab = [&](const uint4* tab, int tile) { return tile < tile_hi ? __ldg(tab + tile) : make_uint4(0u, 0u, 0u, 0u); };
+    auto fetch_tab = [&](const uint4* tab, int i) {
+        const int b = bh_of(i);
+        return i < f_end ? __ldg(tab + ((size_t)b * a.ntiles_max + (i - b * ntiles))) : make_uint4(0u, 0u, 0u, 0u);
+    };
     struct Toks { uint2 mm; uint32_t b; };      // min | max << 16; width | slot << 8 of two tokens
-    auto fetch_toks = [&](const TensorStore& ts, int tile) {
+    auto fetch_toks = [&](const TensorStore& ts, int i) {
         Toks t;
         t.mm = make_uint2(0u, 0u); t.b = 0;
-        if (tile < tile_hi) {
-            const size_t t0 = mrow + (size_t)tile * QAQ_TILE;
+        if (i < f_end) {
+            const int b = bh_of(i);
+            const size_t t0 = (size_t)b * a.tmax_pad + (i - b * ntiles) * QAQ_TILE + 2 * lane;
             t.mm = __ldg(reinterpret_cast<const uint2*>(ts.mnmx + t0));
             t.b = __ldg(reinterpret_cast<const uint32_t*>(ts.bs + t0));
         }
@@ -520,70 +533,62 @@ __global__ void __launch_bounds__(Shape<NQ>::THREADS, Shape<NQ>::CTAS_PER_SM) de
         l.lb = min(l.lb, STAGE - l.nb);
         return l;
     };
-    auto stage = [&](uint32_t dst, const Lay& l, const uint8_t* pool, const uint32_t* og, const uint4& tb, int x) {
+    auto stage = [&](uint32_t dst, const Lay& l, const TensorStore& ts, int b, const uint4& tb, int x) {
         if (lane == 0) {
             bar_expect(bar + 8 * x, l.nb + l.lb);
-            if (l.nb) bulk_copy(dst, pool + tb.x, l.nb, bar + 8 * x);
-            if (l.lb) bulk_copy(dst + l.nb, og + (tb.z & ~3u), l.lb, bar + 8 * x);
+            if (l.nb) bulk_copy(dst, ts.codes + (size_t)b * a.pool_bytes + tb.x, l.nb, bar + 8 * x);
+            if (l.lb) bulk_copy(dst + l.nb, ts.outl + (size_t)b * a.ocap + (tb.z & ~3u), l.lb, bar + 8 * x);
         }
     };
 
-    int tile = tile_lo + warp;
-    uint4 tk = fetch_tab(tabK, tile), tv = fetch_tab(tabV, tile);
-    Toks kt = fetch_toks(a.k, tile);
-    if (lane == 0 && first_seg) { bar_init(bar); bar_init(bar + 8); asm volatile("fence.proxy.async.shared::cta;" ::: "memory"); }
-
-    first_seg = false;
-
-    // ---- q: float copies, scales and sums (every warp for itself)
-    float qscale[NQ], qsum[NQ], qtop = 0.f;
-#pragma unroll
-    for (int j = 0; j < NQ; ++j) {
+    uint4 tk = fetch_tab(a.k.tile, f), tv = fetch_tab(a.v.tile, f);
+    Toks kt = fetch_toks(a.k, f);
+    if (lane == 0) { bar_init(bar); bar_init(bar + 8); asm volatile("fence.proxy.async.shared::cta;" ::: "memory"); }
+    // ---- queries of the run's (b,h): float copies, scales and sums (one warp each)
+    for (int i = warp; i < nseg * NQ; i += S::WARPS) {
+        const int sg = i / NQ, j = i % NQ;
         float qmax = 0.f, qs = 0.f;
 #pragma unroll
-        for (int i = 0; i < D / 32; ++i) {
-            const float f = __half2float(a.q[(size_t)bh * a.q_stride + j * D + lane + 32 * i]);
-            if (warp == 0) sm.qf[lane + 32 * i][j] = f;
-            qmax = fmaxf(qmax, fabsf(f));
-            qs += f;
+        for (int k = 0; k < D / 32; ++k) {
+            const float x = __half2float(a.q[(size_t)(bh0 + sg) * a.q_stride + j * D + lane + 32 * k]);
+            sm.qf[sg][lane + 32 * k][j] = x;
+            qmax = fmaxf(qmax, fabsf(x));
+            qs += x;
         }
         qmax = warp_max(qmax);
-        qsum[j] = warp_sum(qs);
-        qscale[j] = qmax / 32639.0f;             // |q| <= 32639 units: both byte digits of 256 * hi + lo stay signed bytes
-        qtop = fmaxf(qtop, qmax);
+        qs = warp_sum(qs);
+        if (lane == 0) { sm.qscale[sg][j] = qmax / 32639.0f; sm.qsum[sg][j] = qs; }     // |q| <= 32639 units: both byte digits of 256 * hi + lo stay signed bytes
     }
     __syncwarp();
-    if (tile < tile_hi) stage(buf, layout(tk), poolK, ogK, tk, 0);
-    for (int i = 4 * lane; i < WS::VC * D; i += 128) *reinterpret_cast<uint4*>(&ws.vcorr[0][0] + i) = make_uint4(0u, 0u, 0u, 0u);
+    if (f < f_end) stage(buf, layout(tk), a.k, bh_of(f), tk, 0);
     for (int i = 4 * lane; i < NQ * D; i += 128) *reinterpret_cast<float4*>(&ws.macc[0][0] + i) = make_float4(0.f, 0.f, 0.f, 0.f);
-    // ---- operand words of q for all lanes, one or two per thread: nibble word u of lane ln, its low (even r) or high
-    //      nibbles; column ln / 4: the high (even) or low (odd) digit of query ln / 8
-    for (int idx = tid; idx < 32 * 2 * P; idx += S::THREADS) {
-        const int ln = idx / (2 * P), r = idx % (2 * P), lg = ln >> 2, lt = ln & 3, jq = lg >> 1;
+    if (tid == 0) sm.seg[S::WARPS] = -1;
+    __syncthreads();
+    // ---- operand words of q for all lanes: nibble word r / 2 of lane ln, its low (even r) or high nibbles; column ln / 4:
+    //      the high (even) or low (odd) digit of query ln / 8
+    for (int idx = tid; idx < nseg * 64 * P; idx += S::THREADS) {
+        const int sg = idx / (64 * P), ln = idx / (2 * P) % 32, r = idx % (2 * P), lg = ln >> 2, lt = ln & 3, jq = lg >> 1;
         uint32_t v = 0;
         if (jq < NQ) {
-            float qsc = qscale[0];
-#pragma unroll
-            for (int j = 1; j < NQ; ++j) if (jq == j) qsc = qscale[j];
-            const float qinv = qsc > 0.f ? 1.0f / qsc : 0.f;
-            // first channel: unit p = lt * P / 4, word (lt * P mod 4) + u of it
+            const float qsc = sm.qscale[sg][jq], qinv = qsc > 0.f ? 1.0f / qsc : 0.f;
+            // first channel: unit p = lt * P / 4, word (lt * P mod 4) + r / 2 of it
             const int ch = 32 * (lt * P >> 2) + 8 * ((lt * P & 3) + (r >> 1)) + 4 * (r & 1);
-            const uint2 raw = __ldg(reinterpret_cast<const uint2*>(a.q + (size_t)bh * a.q_stride + jq * D + ch));
 #pragma unroll
             for (int i = 0; i < 4; ++i) {
-                const uint32_t w = i < 2 ? raw.x : raw.y;
-                int qi = __float2int_rn(__half2float(__ushort_as_half((unsigned short)(w >> (16 * (i & 1))))) * qinv);
+                int qi = __float2int_rn(sm.qf[sg][ch + i][jq] * qinv);
                 qi = max(-32639, min(32639, qi));
                 const int dg = (lg & 1) == 0 ? ((qi + 128) >> 8) : qi;     // 256 * hi + lo with lo in [-128, 127]
                 v |= (uint32_t)(dg & 0xFF) << (8 * i);
             }
         }
-        sm.qw[r & 1][ln][r >> 1] = v;
+        sm.qw[sg][r & 1][ln][r >> 1] = v;
     }
     __syncthreads();
+
     // digit rows of the value weights this lane feeds: columns 0..3 of the first query of a pair, 4..7 of the second
     const bool wuse = NQ > 1 || fg < 4;
     const uint32_t wrow = smem_addr(&ws.wts[0][NQ > 1 ? fg >> 2 : 0][fg & 3][4 * ft]);
+    uint32_t phase = 0;          // of the warp's two transaction barriers
 
     // The value sums of several tiles stay in integer accumulators (exact) as long as the tiles agree on the reference
     // of the exponentials and on the size of one fixed-point unit; they are added to ws.macc when one of the two changes.
@@ -594,9 +599,7 @@ __global__ void __launch_bounds__(Shape<NQ>::THREADS, Shape<NQ>::CTAS_PER_SM) de
         for (int mb = 0; mb < MB; ++mb) { acc[pr][mb][0] = 0; acc[pr][mb][1] = 0; acc[pr][mb][2] = 0; acc[pr][mb][3] = 0; }
     int held = 0;                // tiles in the accumulators: a tile adds less than 2^22 (64 tokens, 255 * 255), 500 of them fit
     float m_ref[NQ], wunit[NQ];  // exponentials are taken relative to this logit; weight of one fixed-point unit, a power of two
-    float l_run[NQ], c_run[NQ];       // over this lane's tokens: sum of p, of p * (min + step/2) of the values
-#pragma unroll
-    for (int j = 0; j < NQ; ++j) { m_ref[j] = NEG; wunit[j] = 0.f; l_run[j] = 0.f; c_run[j] = 0.f; }
+    float l_run[NQ], c_run[NQ];  // over this lane's tokens: sum of p, of p * (min + step/2) of the values
     auto flush = [&]() {
         // digits 2^24, 2^16, 2^8, 1: columns 0..3 (lanes ft = 0, 1) are the first query of a pair, columns 4..7 the second
         const float d0 = (ft & 1) ? 256.0f : 16777216.0f, d1 = (ft & 1) ? 1.0f : 65536.0f;
@@ -620,17 +623,29 @@ __global__ void __launch_bounds__(Shape<NQ>::THREADS, Shape<NQ>::CTAS_PER_SM) de
         __syncwarp();
     };
 
+    if (f >= f_end && lane == 0) sm.seg[warp] = -1;
 #pragma unroll 1
-    for (; tile < tile_hi; tile += S::WARPS) {
+    while (f < f_end) {          // once per (b,h) of the warp's piece: one or two times
+    const int bh = bh_of(f), seg = bh - bh0, f_stop = seg ? f_end : min(f_end, f_bound);
+    float qscale[NQ], qsum[NQ], qtop = 0.f;
+#pragma unroll
+    for (int j = 0; j < NQ; ++j) {
+        qscale[j] = sm.qscale[seg][j];
+        qsum[j] = sm.qsum[seg][j];
+        qtop = fmaxf(qtop, qscale[j] * 32639.0f);
+        m_ref[j] = NEG; wunit[j] = 0.f; l_run[j] = 0.f; c_run[j] = 0.f;
+    }
+#pragma unroll 1
+    for (; f < f_stop; ++f) {
         const Lay lk = layout(tk), lv = layout(tv);
         const uint32_t tV = buf + STAGE - lv.nb - lv.lb;
         // the tile before is done with: this tile's values come in behind its keys, if there is room
         const bool besideV = lk.nb + lk.lb + lv.nb + lv.lb <= STAGE;
-        if (besideV) stage(tV, lv, poolV, ogV, tv, 1);
-        const uint4 tk_next = fetch_tab(tabK, tile + S::WARPS);
-        const Toks vt = fetch_toks(a.v, tile);
-        const bool has_next = tile + S::WARPS < tile_hi;
-        const int t0 = tile * QAQ_TILE + 2 * lane;              // this lane's tokens: t0 and t0 + 1
+        if (besideV) stage(tV, lv, a.v, bh, tv, 1);
+        const uint4 tk_next = fetch_tab(a.k.tile, f + 1);
+        const Toks vt = fetch_toks(a.v, f);
+        const bool has_next = f + 1 < f_end;
+        const int t0 = (f - bh * ntiles) * QAQ_TILE + 2 * lane;              // this lane's tokens: t0 and t0 + 1
         const bool val[2] = {t0 < T, t0 + 1 < T};
         int B[2], sl[2];             // width; slot (tokens that are not there: a place nobody reads)
         float step[2], mid[2];
@@ -660,8 +675,8 @@ __global__ void __launch_bounds__(Shape<NQ>::THREADS, Shape<NQ>::CTAS_PER_SM) de
         // ---- K: integer dot products, list by list
         {
             uint32_t qa[P], qb[P];
-            lds_words<P>(smem_addr(sm.qw[0][lane]), qa);
-            lds_words<P>(smem_addr(sm.qw[1][lane]), qb);
+            lds_words<P>(smem_addr(sm.qw[seg][0][lane]), qa);
+            lds_words<P>(smem_addr(sm.qw[seg][1][lane]), qb);
             uint4 h = *reinterpret_cast<const uint4*>(ws.buf);
             if (!tk.y || !landed) h = make_uint4(0u, 0u, 0u, 0u);
             uint32_t dots = smem_addr(&ws.dot[0][0][0]);
@@ -684,7 +699,7 @@ __global__ void __launch_bounds__(Shape<NQ>::THREADS, Shape<NQ>::CTAS_PER_SM) de
             auto term = [&](uint32_t v, float inv, int& tok, float (&tm)[NQ]) {
                 tok = (v >> 24) & (QAQ_TILE - 1);
                 const float dx = (__half2float(__ushort_as_half((unsigned short)(v & 0xFFFF))) - ws.mid[tok]) * inv;
-                const float* qv = &sm.qf[(v >> 16) & (D - 1)][0];
+                const float* qv = &sm.qf[seg][(v >> 16) & (D - 1)][0];
 #pragma unroll
                 for (int j = 0; j < NQ; ++j) tm[j] = qv[j] * dx;
             };
@@ -717,7 +732,7 @@ __global__ void __launch_bounds__(Shape<NQ>::THREADS, Shape<NQ>::CTAS_PER_SM) de
 #pragma unroll 1
                 for (uint32_t i = lane; i < oc; i += 32) {
                     int tok; float tm[NQ];
-                    term(i < sc ? list[i] : __ldg(ogK + tk.z + i), 1.0f, tok, tm);
+                    term(i < sc ? list[i] : __ldg(a.k.outl + (size_t)bh * a.ocap + tk.z + i), 1.0f, tok, tm);
 #pragma unroll
                     for (int j = 0; j < NQ; ++j) wide_add(&ws.kcorr[j][0][tok], &ws.kcorr[j][1][tok], tm[j]);
                 }
@@ -745,12 +760,12 @@ __global__ void __launch_bounds__(Shape<NQ>::THREADS, Shape<NQ>::CTAS_PER_SM) de
         }
         __syncwarp();
         // ---- the front of the buffer is free: start the copy of the next tile's keys (beside this tile's values)
-        if (!besideV) stage(tV, lv, poolV, ogV, tv, 1);
+        if (!besideV) stage(tV, lv, a.v, bh, tv, 1);
         const Lay ln = layout(tk_next);
         const bool besideK = ln.nb + ln.lb + lv.nb + lv.lb <= STAGE;
-        if (has_next && besideK) stage(buf, ln, poolK, ogK, tk_next, 0);
-        const uint4 tv_next = fetch_tab(tabV, tile + S::WARPS);
-        kt = fetch_toks(a.k, tile + S::WARPS);
+        if (has_next && besideK) stage(buf, ln, a.k, bh_of(f + 1), tk_next, 0);
+        const uint4 tv_next = fetch_tab(a.v.tile, f + 1);
+        kt = fetch_toks(a.k, f + 1);
 
         // ---- p relative to a reference somewhat above the largest logit, which is moved only when a logit exceeds it (so
         //      p never exceeds 1), and value weights p * step as fixed point of up to 28 bits.  (A token's step falls with
@@ -845,6 +860,9 @@ __global__ void __launch_bounds__(Shape<NQ>::THREADS, Shape<NQ>::CTAS_PER_SM) de
                 const float2 pm = ws.tok[j][(v >> 24) & (QAQ_TILE - 1)];
                 return fmaf(__half2float(__ushort_as_half((unsigned short)(v & 0xFFFF))), pm.x, -pm.y);
             };
+            auto clear_vcorr = [&](int rows) {
+                for (int i = 4 * lane; i < rows * D; i += 128) *reinterpret_cast<uint4*>(&ws.vcorr[0][0] + i) = make_uint4(0u, 0u, 0u, 0u);
+            };
             uint32_t e[4], top = top_range(vt);
 #pragma unroll
             for (int k = 0; k < 4; ++k) {
@@ -857,9 +875,12 @@ __global__ void __launch_bounds__(Shape<NQ>::THREADS, Shape<NQ>::CTAS_PER_SM) de
             top = sc == oc ? __reduce_max_sync(0xFFFFFFFFu, top) : SMALL_MAX + 1;
             if (top <= SMALL_MAX) {
                 float inv[NQ], unit[NQ];
+                __syncwarp();
+                clear_vcorr(NQ);
 #pragma unroll
                 for (int j = 0; j < NQ; ++j)
                     fixed_unit(warp_max(fmaxf(lg[j][0], lg[j][1])) * 2.5f * __half2float(__ushort_as_half((unsigned short)top)), inv[j], unit[j]);
+                __syncwarp();
                 auto add = [&](uint32_t v, bool there) {
 #pragma unroll
                     for (int j = 0; j < NQ; ++j) {
@@ -879,14 +900,16 @@ __global__ void __launch_bounds__(Shape<NQ>::THREADS, Shape<NQ>::CTAS_PER_SM) de
                     for (int k = 0; k < CPL; ++k) {
                         const int d = lane + 32 * k;
                         ws.macc[j][d] += (float)ws.vcorr[j][d] * unit[j];
-                        ws.vcorr[j][d] = 0;
                     }
             } else {
 #pragma unroll 1
                 for (int j = 0; j < NQ; ++j) {
+                    __syncwarp();
+                    clear_vcorr(2);
+                    __syncwarp();
 #pragma unroll 1
                     for (uint32_t i = lane; i < oc; i += 32) {
-                        const uint32_t v = i < sc ? list[i] : __ldg(ogV + tv.z + i);
+                        const uint32_t v = i < sc ? list[i] : __ldg(a.v.outl + (size_t)bh * a.ocap + tv.z + i);
                         const int ch = (v >> 16) & (D - 1);
                         wide_add(&ws.vcorr[0][ch], &ws.vcorr[1][ch], term(v, j));
                     }
@@ -895,57 +918,76 @@ __global__ void __launch_bounds__(Shape<NQ>::THREADS, Shape<NQ>::CTAS_PER_SM) de
                     for (int k = 0; k < CPL; ++k) {
                         const int d = lane + 32 * k;
                         ws.macc[j][d] += wide_sum(ws.vcorr[0][d], ws.vcorr[1][d]);
-                        ws.vcorr[0][d] = 0; ws.vcorr[1][d] = 0;
                     }
-                    __syncwarp();
                 }
             }
         }
         __syncwarp();
-        if (has_next && !besideK) stage(buf, ln, poolK, ogK, tk_next, 0);
+        if (has_next && !besideK) stage(buf, ln, a.k, bh_of(f + 1), tk_next, 0);
         if (!landed) atomicMax(a.status, (int)QAQ_ERR_CUDA);
         phase ^= 1u;
         tk = tk_next;
         tv = tv_next;
     }
     if (held) flush();
-
-    // ---- warp result
+    // ---- what the warp has of this (b,h)
+    const bool cross = f < f_end;                     // it goes on in the next one
+    const int entry = cross ? S::WARPS : warp;
 #pragma unroll
     for (int j = 0; j < NQ; ++j) {
         const float l = warp_sum(l_run[j]), cs = warp_sum(c_run[j]);
-        if (lane == 0) { sm.mm[warp][j] = m_ref[j]; sm.ml[warp][j] = l; sm.cs[warp][j] = cs; }
+        if (lane == 0) { sm.mm[entry][j] = m_ref[j]; sm.ml[entry][j] = l; sm.cs[entry][j] = cs; }
+        if (cross) {
+#pragma unroll
+            for (int k = 0; k < CPL; ++k) { sm.cross[j][lane + 32 * k] = ws.macc[j][lane + 32 * k]; ws.macc[j][lane + 32 * k] = 0.f; }
+        }
+    }
+    if (lane == 0) sm.seg[entry] = seg;
+    __syncwarp();
     }
     __syncthreads();
-    // ---- merge the warps (log-sum-exp) into this segment's partial
-    const bool alone = tile_hi - tile_lo == ntiles;        // the whole (b,h) in this CTA: nothing to merge with
+    // ---- merge the warps (log-sum-exp) into the partials of the (b,h)
 #pragma unroll 1
-    for (int j = 0; j < NQ; ++j) {
-        float M = NEG;
+    for (int seg = 0; seg < nseg; ++seg) {
+        const int bh = bh0 + seg;
+        const bool alone = min(flat_hi, (bh + 1) * ntiles) - max(flat_lo, bh * ntiles) == ntiles;        // nothing to merge with
+#pragma unroll 1
+        for (int j = 0; j < NQ; ++j) {
+            float M = NEG;
 #pragma unroll
-        for (int i = 0; i < S::WARPS; ++i) M = fmaxf(M, sm.mm[i][j]);
-        float L = 0.f, x = 0.f;
+            for (int i = 0; i <= S::WARPS; ++i) if (sm.seg[i] == seg) M = fmaxf(M, sm.mm[i][j]);
+            float L = 0.f, x = 0.f;
 #pragma unroll
-        for (int i = 0; i < S::WARPS; ++i) {
-            const float wgt = sm.mm[i][j] == NEG ? 0.f : __expf(sm.mm[i][j] - M);
-            L = fmaf(wgt, sm.ml[i][j], L);
-            if (tid < D) x = fmaf(wgt, sm.ws[i].macc[j][tid] + sm.cs[i][j], x);
-        }
-        float* dst = a.part + ((size_t)(2 * cta + seg) * NQ + j) * (D + 4);
-        if (alone) {
-            if (tid < D) a.out[(size_t)bh * a.out_stride + j * D + tid] = L > 0.f ? x / L : 0.f;
-            if (NQ == 1) {
-                if (a.ml && tid == 0) { a.ml[2 * bh] = M; a.ml[2 * bh + 1] = L; }
-                if (a.scores && !a.ml) normalise_scores<S::THREADS>(a.scores + (size_t)bh * a.scores_stride, T, M, L);
+            for (int i = 0; i <= S::WARPS; ++i) {
+                if (sm.seg[i] != seg || sm.mm[i][j] == NEG) continue;
+                const float wgt = __expf(sm.mm[i][j] - M);
+                L = fmaf(wgt, sm.ml[i][j], L);
+                if (tid < D) x = fmaf(wgt, (i == S::WARPS ? sm.cross[j][tid] : sm.ws[i < S::WARPS ? i : 0].macc[j][tid]) + sm.cs[i][j], x);
             }
-        } else {
-            if (tid < D) __stcg(dst + tid, x);
-            if (tid == 0) __stcg(reinterpret_cast<float2*>(dst + D), make_float2(M, L));
+            float* dst = a.part + ((size_t)(2 * blockIdx.x + seg) * NQ + j) * (D + 4);
+            if (alone) {
+                if (tid < D) a.out[(size_t)bh * a.out_stride + j * D + tid] = L > 0.f ? x / L : 0.f;
+                if (NQ == 1) {
+                    if (a.ml && tid == 0) { a.ml[2 * bh] = M; a.ml[2 * bh + 1] = L; }
+                    if (a.scores && !a.ml) normalise_scores<S::THREADS>(a.scores + (size_t)bh * a.scores_stride, T, M, L);
+                }
+            } else {
+                if (tid < D) __stcg(dst + tid, x);
+                if (tid == 0) __stcg(reinterpret_cast<float2*>(dst + D), make_float2(M, L));
+            }
         }
     }
-    if (!alone) finish_split<D, NQ>(a, sm, bh, ntiles, run, T);
-    __syncthreads();   // the shared arrays are reused by the second segment
+    __syncthreads();
+    if (lane == 0 && warp < nseg) {
+        const int bh = bh0 + warp;
+        int first, n;
+        split_of(bh, ntiles, run, first, n);
+        sm.last[warp] = n > 1 && count_partial(a.done + bh, a.tag, n);
     }
+    __syncthreads();
+#pragma unroll 1
+    for (int seg = 0; seg < nseg; ++seg)
+        if (sm.last[seg]) merge_split<D, NQ>(a, sm, bh0 + seg, ntiles, run, T);
 }
 
 // Score rows too long for one CTA to normalise on the side.
