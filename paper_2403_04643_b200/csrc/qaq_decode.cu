@@ -85,6 +85,23 @@ __device__ __forceinline__ void lds_words(uint32_t addr, uint32_t (&x)[W]) {
 }
 __device__ __forceinline__ void sts_word(uint32_t addr, int v) { asm volatile("st.shared.u32 [%0], %1;" ::"r"(addr), "r"(v) : "memory"); }
 
+// Loads that stay where they are written: the metadata of the next tile is fetched long before its use.
+__device__ __forceinline__ uint4 ldg_now4(const uint4* p) {
+    uint4 v;
+    asm volatile("ld.global.nc.v4.u32 {%0,%1,%2,%3}, [%4];" : "=r"(v.x), "=r"(v.y), "=r"(v.z), "=r"(v.w) : "l"(p));
+    return v;
+}
+__device__ __forceinline__ uint2 ldg_now2(const void* p) {
+    uint2 v;
+    asm volatile("ld.global.nc.v2.u32 {%0,%1}, [%2];" : "=r"(v.x), "=r"(v.y) : "l"(p));
+    return v;
+}
+__device__ __forceinline__ uint32_t ldg_now1(const void* p) {
+    uint32_t v;
+    asm volatile("ld.global.nc.u32 %0, [%1];" : "=r"(v) : "l"(p));
+    return v;
+}
+
 // bulk copies into shared memory, completion on a transaction barrier
 __device__ __forceinline__ void bar_init(uint32_t bar) { asm volatile("mbarrier.init.shared::cta.b64 [%0], 1;" ::"r"(bar) : "memory"); }
 __device__ __forceinline__ void bar_expect(uint32_t bar, uint32_t bytes) {
@@ -500,26 +517,26 @@ __global__ void __launch_bounds__(Shape<NQ>::THREADS, Shape<NQ>::CTAS_PER_SM) de
     // this warp's piece of it
     const int piece = (run + S::WARPS - 1) / S::WARPS;
     int f = flat_lo + warp * piece;
-    const int f_end = min(f + piece, flat_hi);
+    const int f_end = min(f + piece, flat_hi), f_last = min(f_end, flat_hi) - 1;
     auto bh_of = [&](int i) { return bh0 + (i >= f_bound ? 1 : 0); };
     const uint32_t buf = smem_addr(ws.buf), bar = smem_addr(ws.bar);
 
     // ---- tile metadata: the table words (offset and length of the bytes, first entry and length of the outlier list),
     //      min/max, widths and slots of tokens 2*lane, 2*lane+1; fetched as late as their latency allows
+    //      (a piece that has no tile i fetches its last one again: a load behind a condition would be waited for on the spot)
     auto fetch_tab = [&](const uint4* tab, int i) {
+        i = min(i, f_last);
         const int b = bh_of(i);
-        return i < f_end ? __ldg(tab + ((size_t)b * a.ntiles_max + (i - b * ntiles))) : make_uint4(0u, 0u, 0u, 0u);
+        return ldg_now4(tab + ((size_t)b * a.ntiles_max + (i - b * ntiles)));
     };
     struct Toks { uint2 mm; uint32_t b; };      // min | max << 16; width | slot << 8 of two tokens
     auto fetch_toks = [&](const TensorStore& ts, int i) {
+        i = min(i, f_last);
+        const int b = bh_of(i);
+        const size_t t0 = (size_t)b * a.tmax_pad + (i - b * ntiles) * QAQ_TILE + 2 * lane;
         Toks t;
-        t.mm = make_uint2(0u, 0u); t.b = 0;
-        if (i < f_end) {
-            const int b = bh_of(i);
-            const size_t t0 = (size_t)b * a.tmax_pad + (i - b * ntiles) * QAQ_TILE + 2 * lane;
-            t.mm = __ldg(reinterpret_cast<const uint2*>(ts.mnmx + t0));
-            t.b = __ldg(reinterpret_cast<const uint32_t*>(ts.bs + t0));
-        }
+        t.mm = ldg_now2(ts.mnmx + t0);
+        t.b = ldg_now1(ts.bs + t0);
         return t;
     };
     // how a tile lies in the buffer: bytes of the tile and of the piece of the outlier list that comes with it (from the
@@ -710,7 +727,7 @@ __global__ void __launch_bounds__(Shape<NQ>::THREADS, Shape<NQ>::CTAS_PER_SM) de
                 if (lane + 32u * k < sc) e[k] = list[lane + 32 * k];
                 top = max(top, e[k] & 0x7FFFu);
             }
-#pragma unroll 1
+#pragma unroll 4
             for (uint32_t i = lane + 128; i < sc; i += 32) top = max(top, list[i] & 0x7FFFu);
             top = sc == oc ? __reduce_max_sync(0xFFFFFFFFu, top) : SMALL_MAX + 1;
             if (top <= SMALL_MAX) {
@@ -722,11 +739,15 @@ __global__ void __launch_bounds__(Shape<NQ>::THREADS, Shape<NQ>::CTAS_PER_SM) de
 #pragma unroll
                     for (int j = 0; j < NQ; ++j) if (there) atomicAdd(&ws.kcorr[j][0][tok], __float2int_rn(tm[j]));
                 };
-#pragma unroll
-                for (int k = 0; k < 4; ++k)
-                    if (32u * k < sc) add(e[k], lane + 32u * k < sc);
 #pragma unroll 1
-                for (uint32_t i = 128; i < sc; i += 32) add(list[min(i + lane, sc - 1)], i + lane < sc);
+                for (uint32_t i = 0;;) {
+#pragma unroll
+                    for (int k = 0; k < 4; ++k)
+                        if (i + 32u * k < sc) add(e[k], i + lane + 32u * k < sc);
+                    if ((i += 128) >= sc) break;
+#pragma unroll
+                    for (int k = 0; k < 4; ++k) e[k] = list[min(i + lane + 32u * k, sc - 1)];
+                }
             } else {
                 kunit = -1.0f;
 #pragma unroll 1
@@ -870,7 +891,7 @@ __global__ void __launch_bounds__(Shape<NQ>::THREADS, Shape<NQ>::CTAS_PER_SM) de
                 if (lane + 32u * k < sc) e[k] = list[lane + 32 * k];
                 top = max(top, e[k] & 0x7FFFu);
             }
-#pragma unroll 1
+#pragma unroll 4
             for (uint32_t i = lane + 128; i < sc; i += 32) top = max(top, list[i] & 0x7FFFu);
             top = sc == oc ? __reduce_max_sync(0xFFFFFFFFu, top) : SMALL_MAX + 1;
             if (top <= SMALL_MAX) {
@@ -888,11 +909,15 @@ __global__ void __launch_bounds__(Shape<NQ>::THREADS, Shape<NQ>::CTAS_PER_SM) de
                         if (there) atomicAdd(&ws.vcorr[j][(v >> 16) & (D - 1)], x);
                     }
                 };
-#pragma unroll
-                for (int k = 0; k < 4; ++k)
-                    if (32u * k < sc) add(e[k], lane + 32u * k < sc);
 #pragma unroll 1
-                for (uint32_t i = 128; i < sc; i += 32) add(list[min(i + lane, sc - 1)], i + lane < sc);
+                for (uint32_t i = 0;;) {
+#pragma unroll
+                    for (int k = 0; k < 4; ++k)
+                        if (i + 32u * k < sc) add(e[k], i + lane + 32u * k < sc);
+                    if ((i += 128) >= sc) break;
+#pragma unroll
+                    for (int k = 0; k < 4; ++k) e[k] = list[min(i + lane + 32u * k, sc - 1)];
+                }
                 __syncwarp();
 #pragma unroll
                 for (int j = 0; j < NQ; ++j)
