@@ -111,11 +111,11 @@ __device__ __forceinline__ void bulk_copy(uint32_t dst, const void* src, uint32_
     asm volatile("cp.async.bulk.shared::cluster.global.mbarrier::complete_tx::bytes [%0], [%1], %2, [%3];" ::"r"(dst), "l"(src), "r"(bytes), "r"(bar)
                  : "memory");
 }
-// false if the phase did not complete within the limit (seconds; a copy takes microseconds)
+// false if the phase did not complete within the limit (a copy takes microseconds; every try waits for a while itself)
 __device__ __forceinline__ bool bar_wait(uint32_t bar, uint32_t parity) {
     uint32_t done = 0;
 #pragma unroll 1
-    for (int i = 0; i < (1 << 22) && !done; ++i)
+    for (int i = 0; i < (1 << 14) && !done; ++i)
         asm volatile("{\n.reg .pred p;\nmbarrier.try_wait.parity.shared::cta.b64 p, [%1], %2;\nselp.u32 %0, 1, 0, p;\n}" : "=r"(done) : "r"(bar), "r"(parity) : "memory");
     return done != 0;
 }
@@ -221,7 +221,6 @@ struct DecSmem {
     float cross[NQ][D];
     float mm[W + 1][NQ], ml[W + 1][NQ], cs[W + 1][NQ];
     int seg[W + 1];                           // which of the two (b,h) an entry belongs to, -1: none
-    float red[2 * W];
     int last[2];
 };
 
@@ -392,24 +391,27 @@ __device__ __forceinline__ void normalise_scores(float* row, int T, float M, flo
     for (; t < T; t += THREADS) row[t] = __expf(__ldcg(row + t) - M) * inv;
 }
 
-// The CTA that finds all partials of a (b,h) complete merges them (log-sum-exp), in CTA order, so the result does not
-// depend on which one it is.
+// The CTA that completes the partials of a (b,h) merges them (log-sum-exp), in CTA order, so the result does not depend
+// on which one it is.
 //
 // The CTAs are counted in a word of the workspace, which comes uninitialised: the count carries the tag of the call, a
-// number no other call uses, and a word with another tag counts as zero.  The last CTA clears the word, so that a replay
-// of the same launch (a CUDA graph carries the same tag) starts from zero again.
-__device__ __forceinline__ bool count_partial(unsigned long long* word, unsigned long long tag, int n) {
-    asm volatile("fence.acq_rel.gpu;" ::: "memory");
-    unsigned long long cur = *(volatile unsigned long long*)word, next;
-    for (;;) {           // a failed exchange means that another CTA has been counted: at most n rounds
-        next = ((cur ^ tag) >> 12) == 0 ? cur + 1 : tag + 1;
-        const unsigned long long was = atomicCAS(word, cur, next);
+// number no other call uses.  Every CTA sees to it when it begins that the word carries the tag (with a count of zero, if
+// nobody has put it there yet), so that being counted at the end is one atomic addition; with the tag checked there, in
+// a compare-and-swap loop, eight CTAs took up to 5 us to be counted.  The last CTA clears the word, so that a replay of
+// the same launch (a CUDA graph carries the same tag) starts anew.
+__device__ __forceinline__ void open_count(unsigned long long* word, unsigned long long tag) {
+    unsigned long long cur = *(volatile unsigned long long*)word;
+    while (((cur ^ tag) >> 12) != 0) {       // a failed exchange means that another CTA has put the tag there: two rounds at most
+        const unsigned long long was = atomicCAS(word, cur, tag);
         if (was == cur) break;
         cur = was;
     }
-    const bool last = (int)(next & 0xFFF) == n;
+}
+__device__ __forceinline__ bool count_partial(unsigned long long* word, int n) {
+    unsigned long long was;
+    asm volatile("fence.acq_rel.gpu;\natom.add.relaxed.gpu.global.u64 %0, [%1], 1;\nfence.acq_rel.gpu;" : "=l"(was) : "l"(word) : "memory");
+    const bool last = (int)(was & 0xFFF) + 1 == n;
     if (last) *word = 0ull;
-    asm volatile("fence.acq_rel.gpu;" ::: "memory");
     return last;
 }
 
@@ -420,63 +422,69 @@ __device__ __forceinline__ void split_of(int bh, int ntiles, int run, int& first
     n = ((bh + 1) * ntiles - 1) / run - first + 1;
 }
 
-// log-sum-exp merge of the partials of a (b,h), by the whole CTA
+// log-sum-exp merge of the partials of a (b,h), by the whole CTA: D/4 threads take a partial, four channels each, every
+// group of D/4 threads its share of the partials with the next four on their way; the groups meet in shared memory
 template <int D, int NQ>
 __device__ void merge_split(const DecArgs& a, DecSmem<D, NQ>& sm, int bh, int ntiles, int run, int T) {
     using S = Shape<NQ>;
     int c_lo, n;
     split_of(bh, ntiles, run, c_lo, n);
     const int first_slot = 2 * c_lo + (c_lo * run < bh * ntiles ? 1 : 0);
-    constexpr int PS = D + 4;
-    auto part = [&](int i, int j) { return a.part + ((size_t)(i == 0 ? first_slot : 2 * (c_lo + i)) * NQ + j) * PS; };
-    const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
-    float* s_w = reinterpret_cast<float*>(sm.ws[0].buf);            // [n] <= SLOTS
-    float4* s_x = reinterpret_cast<float4*>(sm.ws[1].buf);          // [THREADS]
-    static_assert(S::SLOTS * sizeof(float) <= sizeof(sm.ws[0].buf) && S::THREADS * sizeof(float4) <= 2 * sizeof(sm.ws[0]), "scratch of the merge");
+    constexpr int PS = D + 4, CT = D / 4, G = S::THREADS / CT, AHEAD = 4;
+    const float NEG = __int_as_float(0xff800000);
+    const int tid = threadIdx.x, d4 = tid % CT, grp = tid / CT;
+    struct Part { float4 x; float m, l; };
+    Part* s_part = reinterpret_cast<Part*>(sm.ws[0].buf);          // [G][CT], then the group's reference and sum beside each
+    static_assert(S::THREADS * sizeof(Part) <= sizeof(sm.ws), "scratch of the merge");
+    auto fold = [&](Part& to, const Part& p) {
+        const float m = fmaxf(to.m, p.m);
+        const float wa = to.m == NEG ? 0.f : __expf(to.m - m), wb = p.m == NEG ? 0.f : __expf(p.m - m);
+        to.x.x = fmaf(wb, p.x.x, wa * to.x.x); to.x.y = fmaf(wb, p.x.y, wa * to.x.y);
+        to.x.z = fmaf(wb, p.x.z, wa * to.x.z); to.x.w = fmaf(wb, p.x.w, wa * to.x.w);
+        to.l = fmaf(wb, p.l, wa * to.l);
+        to.m = m;
+    };
     for (int j = 0; j < NQ; ++j) {
-        // ---- weights of the partials, sums of the softmax denominators
-        float M = __int_as_float(0xff800000);
-        for (int i = tid; i < n; i += S::THREADS) M = fmaxf(M, __ldcg(part(i, j) + D));
-        M = warp_max(M);
-        if (lane == 0) sm.red[warp] = M;
-        __syncthreads();
-        M = sm.red[0];
+        Part mine;
+        mine.x = make_float4(0.f, 0.f, 0.f, 0.f); mine.m = NEG; mine.l = 0.f;
+        for (int i0 = grp; i0 < n; i0 += AHEAD * G) {
+            Part p[AHEAD];
 #pragma unroll
-        for (int w = 1; w < S::WARPS; ++w) M = fmaxf(M, sm.red[w]);
-        float L = 0.f;
-        for (int i = tid; i < n; i += S::THREADS) {
-            const float2 h = __ldcg(reinterpret_cast<const float2*>(part(i, j) + D));    // reference, sum
-            const float w = h.x == __int_as_float(0xff800000) ? 0.f : __expf(h.x - M);
-            s_w[i] = w;
-            L = fmaf(w, h.y, L);
-        }
-        L = warp_sum(L);
-        if (lane == 0) sm.red[S::WARPS + warp] = L;
-        __syncthreads();
-        L = 0.f;
+            for (int k = 0; k < AHEAD; ++k) {
+                const int i = min(i0 + k * G, n - 1);
+                const float* src = a.part + ((size_t)(i == 0 ? first_slot : 2 * (c_lo + i)) * NQ + j) * PS;
+                p[k].x = __ldcg(reinterpret_cast<const float4*>(src) + d4);
+                const float2 ml = __ldcg(reinterpret_cast<const float2*>(src + D));
+                p[k].m = ml.x; p[k].l = ml.y;
+            }
 #pragma unroll
-        for (int w = 0; w < S::WARPS; ++w) L += sm.red[S::WARPS + w];
-        // ---- the channels: D/4 threads per partial, four channels each
-        constexpr int CT = D / 4, SH = S::THREADS / CT;
-        const int d4 = tid % CT, sh = tid / CT;
-        float4 x = make_float4(0.f, 0.f, 0.f, 0.f);
-#pragma unroll 4
-        for (int i = sh; i < n; i += SH) {
-            const float w = s_w[i];
-            const float4 v = __ldcg(reinterpret_cast<const float4*>(part(i, j)) + d4);
-            if (w != 0.f) { x.x = fmaf(w, v.x, x.x); x.y = fmaf(w, v.y, x.y); x.z = fmaf(w, v.z, x.z); x.w = fmaf(w, v.w, x.w); }
+            for (int k = 0; k < AHEAD; ++k) if (i0 + k * G < n) fold(mine, p[k]);
         }
-        s_x[tid] = x;
+        s_part[tid] = mine;
         __syncthreads();
-        if (tid < D) {
-            float y = 0.f;
-#pragma unroll
-            for (int k = 0; k < SH; ++k) y += reinterpret_cast<const float*>(s_x + k * CT)[tid];
-            a.out[(size_t)bh * a.out_stride + j * D + tid] = L > 0.f ? y / L : 0.f;
-        }
-        if (NQ == 1) {
-            if (a.ml && tid == 0) { a.ml[2 * bh] = M; a.ml[2 * bh + 1] = L; }
-            if (a.scores && !a.ml) normalise_scores<S::THREADS>(a.scores + (size_t)bh * a.scores_stride, T, M, L);
+        // whole warps only from here to the barrier: those that hold channels, all of them where a score row is normalised
+        if (tid < (CT > 32 ? CT : 32) || (NQ == 1 && a.scores)) {
+            float M = NEG;
+#pragma unroll 8
+            for (int g = 0; g < G; ++g) M = fmaxf(M, s_part[g * CT + d4].m);
+            mine.x = make_float4(0.f, 0.f, 0.f, 0.f); mine.m = M; mine.l = 0.f;
+#pragma unroll 8
+            for (int g = 0; g < G; ++g) {
+                const Part p = s_part[g * CT + d4];
+                const float w = p.m == NEG ? 0.f : __expf(p.m - M);
+                mine.x.x = fmaf(w, p.x.x, mine.x.x); mine.x.y = fmaf(w, p.x.y, mine.x.y);
+                mine.x.z = fmaf(w, p.x.z, mine.x.z); mine.x.w = fmaf(w, p.x.w, mine.x.w);
+                mine.l = fmaf(w, p.l, mine.l);
+            }
+            if (tid < CT) {
+                const float inv = mine.l > 0.f ? 1.0f / mine.l : 0.f;
+                float* o = a.out + (size_t)bh * a.out_stride + j * D + 4 * d4;
+                o[0] = mine.x.x * inv; o[1] = mine.x.y * inv; o[2] = mine.x.z * inv; o[3] = mine.x.w * inv;
+            }
+            if (NQ == 1) {
+                if (a.ml && tid == 0) { a.ml[2 * bh] = mine.m; a.ml[2 * bh + 1] = mine.l; }
+                if (a.scores && !a.ml) normalise_scores<S::THREADS>(a.scores + (size_t)bh * a.scores_stride, T, mine.m, mine.l);
+            }
         }
         __syncthreads();
     }
@@ -560,46 +568,83 @@ __global__ void __launch_bounds__(Shape<NQ>::THREADS, Shape<NQ>::CTAS_PER_SM) de
 
     uint4 tk = fetch_tab(a.k.tile, f), tv = fetch_tab(a.v.tile, f);
     Toks kt = fetch_toks(a.k, f);
-    if (lane == 0) { bar_init(bar); bar_init(bar + 8); asm volatile("fence.proxy.async.shared::cta;" ::: "memory"); }
-    // ---- queries of the run's (b,h): float copies, scales and sums (one warp each)
-    for (int i = warp; i < nseg * NQ; i += S::WARPS) {
-        const int sg = i / NQ, j = i % NQ;
-        float qmax = 0.f, qs = 0.f;
+    // ---- queries of the run's (b,h), by all warps alike: four channels per lane of every query, and the four channels whose
+    //      operand word the thread makes; all loads first
+    constexpr int WORDS = 64 * P, PER = (2 * WORDS + S::THREADS - 1) / S::THREADS;      // operand words of a (b,h); words per thread
+    uint2 qrow[2][NQ], qword[PER];
+    const bool q_aligned = ((uintptr_t)a.q & 7) == 0 && (a.q_stride & 3) == 0;
+    auto load4 = [&](const __half* p) {
+        if (q_aligned) return __ldg(reinterpret_cast<const uint2*>(p));
+        const unsigned short* h = reinterpret_cast<const unsigned short*>(p);
+        return make_uint2((uint32_t)__ldg(h) | ((uint32_t)__ldg(h + 1) << 16), (uint32_t)__ldg(h + 2) | ((uint32_t)__ldg(h + 3) << 16));
+    };
 #pragma unroll
-        for (int k = 0; k < D / 32; ++k) {
-            const float x = __half2float(a.q[(size_t)(bh0 + sg) * a.q_stride + j * D + lane + 32 * k]);
-            sm.qf[sg][lane + 32 * k][j] = x;
-            qmax = fmaxf(qmax, fabsf(x));
-            qs += x;
+    for (int sg = 0; sg < 2; ++sg)
+#pragma unroll
+        for (int j = 0; j < NQ; ++j) {
+            qrow[sg][j] = make_uint2(0u, 0u);
+            if (sg < nseg && 4 * lane < D) qrow[sg][j] = load4(a.q + (size_t)(bh0 + sg) * a.q_stride + j * D + 4 * lane);
         }
-        qmax = warp_max(qmax);
-        qs = warp_sum(qs);
-        if (lane == 0) { sm.qscale[sg][j] = qmax / 32639.0f; sm.qsum[sg][j] = qs; }     // |q| <= 32639 units: both byte digits of 256 * hi + lo stay signed bytes
+    // word idx: nibble word r / 2 of lane ln of (b,h) sg, its low (even r) or high nibbles; column ln / 4: the high (even) or
+    // low (odd) digit of query ln / 8; first channel: unit p = lt * P / 4, word (lt * P mod 4) + r / 2 of it
+    auto word_of = [&](int idx, int& sg, int& ln, int& r, int& ch) {
+        sg = idx / WORDS; ln = idx / (2 * P) % 32; r = idx % (2 * P);
+        ch = 32 * ((ln & 3) * P >> 2) + 8 * (((ln & 3) * P & 3) + (r >> 1)) + 4 * (r & 1);
+    };
+#pragma unroll
+    for (int k = 0; k < PER; ++k) {
+        int sg, ln, r, ch;
+        word_of(tid + k * S::THREADS, sg, ln, r, ch);
+        qword[k] = make_uint2(0u, 0u);
+        if (sg < nseg && ln < 8 * NQ) qword[k] = load4(a.q + (size_t)(bh0 + sg) * a.q_stride + (ln >> 3) * D + ch);
     }
+    if (lane == 0) { bar_init(bar); bar_init(bar + 8); asm volatile("fence.proxy.async.shared::cta;" ::: "memory"); }
     __syncwarp();
     if (f < f_end) stage(buf, layout(tk), a.k, bh_of(f), tk, 0);
+    if (lane == 0 && warp < nseg) {
+        int first, n;
+        split_of(bh0 + warp, ntiles, run, first, n);
+        if (n > 1) open_count(a.done + bh0 + warp, a.tag);
+    }
     for (int i = 4 * lane; i < NQ * D; i += 128) *reinterpret_cast<float4*>(&ws.macc[0][0] + i) = make_float4(0.f, 0.f, 0.f, 0.f);
-    if (tid == 0) sm.seg[S::WARPS] = -1;
-    __syncthreads();
-    // ---- operand words of q for all lanes: nibble word r / 2 of lane ln, its low (even r) or high nibbles; column ln / 4:
-    //      the high (even) or low (odd) digit of query ln / 8
-    for (int idx = tid; idx < nseg * 64 * P; idx += S::THREADS) {
-        const int sg = idx / (64 * P), ln = idx / (2 * P) % 32, r = idx % (2 * P), lg = ln >> 2, lt = ln & 3, jq = lg >> 1;
-        uint32_t v = 0;
-        if (jq < NQ) {
-            const float qsc = sm.qscale[sg][jq], qinv = qsc > 0.f ? 1.0f / qsc : 0.f;
-            // first channel: unit p = lt * P / 4, word (lt * P mod 4) + r / 2 of it
-            const int ch = 32 * (lt * P >> 2) + 8 * ((lt * P & 3) + (r >> 1)) + 4 * (r & 1);
+    auto half_at = [](const uint2& v, int i) { return __half2float(__ushort_as_half((unsigned short)((i < 2 ? v.x : v.y) >> (16 * (i & 1))))); };
+    float qsc[2][NQ];
 #pragma unroll
-            for (int i = 0; i < 4; ++i) {
-                int qi = __float2int_rn(sm.qf[sg][ch + i][jq] * qinv);
-                qi = max(-32639, min(32639, qi));
-                const int dg = (lg & 1) == 0 ? ((qi + 128) >> 8) : qi;     // 256 * hi + lo with lo in [-128, 127]
-                v |= (uint32_t)(dg & 0xFF) << (8 * i);
+    for (int sg = 0; sg < 2; ++sg)
+#pragma unroll
+        for (int j = 0; j < NQ; ++j) {
+            float qmax = 0.f, qs = 0.f;
+#pragma unroll
+            for (int i = 0; i < 4; ++i) { const float x = half_at(qrow[sg][j], i); qmax = fmaxf(qmax, fabsf(x)); qs += x; }
+            qsc[sg][j] = warp_max(qmax) / 32639.0f;             // |q| <= 32639 units: both byte digits of 256 * hi + lo stay signed bytes
+            if (warp == (sg * NQ + j) % S::WARPS && sg < nseg) {
+                qs = warp_sum(qs);
+                if (lane == 0) { sm.qscale[sg][j] = qsc[sg][j]; sm.qsum[sg][j] = qs; }
+                if (4 * lane < D)
+#pragma unroll
+                    for (int i = 0; i < 4; ++i) sm.qf[sg][4 * lane + i][j] = half_at(qrow[sg][j], i);
             }
         }
-        sm.qw[sg][r & 1][ln][r >> 1] = v;
+#pragma unroll
+    for (int k = 0; k < PER; ++k) {
+        int sg, ln, r, ch;
+        word_of(tid + k * S::THREADS, sg, ln, r, ch);
+        float sc = 0.f;
+#pragma unroll
+        for (int j = 0; j < NQ; ++j) if ((ln >> 3) == j) sc = sg ? qsc[1][j] : qsc[0][j];
+        const float qinv = sc > 0.f ? 1.0f / sc : 0.f;
+        uint32_t v = 0;
+#pragma unroll
+        for (int i = 0; i < 4; ++i) {
+            int qi = __float2int_rn(half_at(qword[k], i) * qinv);
+            qi = max(-32639, min(32639, qi));
+            const int dg = ((ln >> 2) & 1) == 0 ? ((qi + 128) >> 8) : qi;     // 256 * hi + lo with lo in [-128, 127]
+            v |= (uint32_t)(dg & 0xFF) << (8 * i);
+        }
+        if (sg < nseg) sm.qw[sg][r & 1][ln][r >> 1] = v;
     }
+    if (tid == 0) sm.seg[S::WARPS] = -1;
+    for (int i = tid; i < NQ * D; i += S::THREADS) (&sm.cross[0][0])[i] = 0.f;
     __syncthreads();
 
     // digit rows of the value weights this lane feeds: columns 0..3 of the first query of a pair, 4..7 of the second
@@ -971,24 +1016,22 @@ __global__ void __launch_bounds__(Shape<NQ>::THREADS, Shape<NQ>::CTAS_PER_SM) de
     __syncwarp();
     }
     __syncthreads();
-    // ---- merge the warps (log-sum-exp) into the partials of the (b,h)
+    // ---- merge the warps (log-sum-exp) into the partials of the (b,h): lane i knows the weight of entry i
 #pragma unroll 1
     for (int seg = 0; seg < nseg; ++seg) {
         const int bh = bh0 + seg;
         const bool alone = min(flat_hi, (bh + 1) * ntiles) - max(flat_lo, bh * ntiles) == ntiles;        // nothing to merge with
+        const bool mine = lane <= S::WARPS && sm.seg[min(lane, S::WARPS)] == seg;
 #pragma unroll 1
         for (int j = 0; j < NQ; ++j) {
-            float M = NEG;
+            const float m = mine ? sm.mm[lane][j] : NEG, M = warp_max(m);
+            const float wgt = m == NEG ? 0.f : __expf(m - M);
+            const float L = warp_sum(mine ? wgt * sm.ml[lane][j] : 0.f);
+            float x = warp_sum(mine ? wgt * sm.cs[lane][j] : 0.f);
+            const int d = tid < D ? tid : 0;
 #pragma unroll
-            for (int i = 0; i <= S::WARPS; ++i) if (sm.seg[i] == seg) M = fmaxf(M, sm.mm[i][j]);
-            float L = 0.f, x = 0.f;
-#pragma unroll
-            for (int i = 0; i <= S::WARPS; ++i) {
-                if (sm.seg[i] != seg || sm.mm[i][j] == NEG) continue;
-                const float wgt = __expf(sm.mm[i][j] - M);
-                L = fmaf(wgt, sm.ml[i][j], L);
-                if (tid < D) x = fmaf(wgt, (i == S::WARPS ? sm.cross[j][tid] : sm.ws[i < S::WARPS ? i : 0].macc[j][tid]) + sm.cs[i][j], x);
-            }
+            for (int i = 0; i < S::WARPS; ++i) x = fmaf(__shfl_sync(0xFFFFFFFFu, wgt, i), sm.ws[i].macc[j][d], x);
+            x = fmaf(__shfl_sync(0xFFFFFFFFu, wgt, S::WARPS), sm.cross[j][d], x);
             float* dst = a.part + ((size_t)(2 * blockIdx.x + seg) * NQ + j) * (D + 4);
             if (alone) {
                 if (tid < D) a.out[(size_t)bh * a.out_stride + j * D + tid] = L > 0.f ? x / L : 0.f;
@@ -1004,10 +1047,9 @@ __global__ void __launch_bounds__(Shape<NQ>::THREADS, Shape<NQ>::CTAS_PER_SM) de
     }
     __syncthreads();
     if (lane == 0 && warp < nseg) {
-        const int bh = bh0 + warp;
         int first, n;
-        split_of(bh, ntiles, run, first, n);
-        sm.last[warp] = n > 1 && count_partial(a.done + bh, a.tag, n);
+        split_of(bh0 + warp, ntiles, run, first, n);
+        sm.last[warp] = n > 1 && count_partial(a.done + bh0 + warp, n);
     }
     __syncthreads();
 #pragma unroll 1
