@@ -120,15 +120,14 @@ extern "C" qaq_status qaq_cache_reset(qaq_cache* c, void* stream) {
 }
 
 namespace {
-__global__ void set_count_kernel(int* count, unsigned* ticket, int value) { *count = value; *ticket = 0u; }
+__global__ void set_count_kernel(int* count, unsigned* ticket, int value) { qaq_dependency(); *count = value; *ticket = 0u; }
 }  // namespace
 
 // The token count moves to device memory (qaq_stream_begin) and back (qaq_stream_end); between the two the
 // qaq_stream_* calls read and advance it there, and the host counter is stale.
 extern "C" qaq_status qaq_stream_begin(qaq_cache* c, void* stream) {
     if (!c) return QAQ_ERR_INVALID_ARG;
-    set_count_kernel<<<1, 1, 0, (cudaStream_t)stream>>>(qaq_d_count(c), qaq_d_ticket(c), (int)c->tokens);
-    QAQ_CUDA_TRY(cudaGetLastError());
+    QAQ_CUDA_TRY(qaq_launch(set_count_kernel, dim3(1), dim3(1), 0, (cudaStream_t)stream, qaq_d_count(c), qaq_d_ticket(c), (int)c->tokens));
     return QAQ_OK;
 }
 

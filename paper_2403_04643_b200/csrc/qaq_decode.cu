@@ -39,7 +39,6 @@
 //
 // The partials of a (b,h) that was split over several CTAs are merged by the last of these CTAs to finish, in the
 // same launch (see finish_split).
-#include <atomic>
 #include <chrono>
 #include <mutex>
 
@@ -88,17 +87,17 @@ __device__ __forceinline__ void sts_word(uint32_t addr, int v) { asm volatile("s
 // Loads that stay where they are written: the metadata of the next tile is fetched long before its use.
 __device__ __forceinline__ uint4 ldg_now4(const uint4* p) {
     uint4 v;
-    asm volatile("ld.global.nc.v4.u32 {%0,%1,%2,%3}, [%4];" : "=r"(v.x), "=r"(v.y), "=r"(v.z), "=r"(v.w) : "l"(p));
+    asm volatile("ld.global.v4.u32 {%0,%1,%2,%3}, [%4];" : "=r"(v.x), "=r"(v.y), "=r"(v.z), "=r"(v.w) : "l"(p));
     return v;
 }
 __device__ __forceinline__ uint2 ldg_now2(const void* p) {
     uint2 v;
-    asm volatile("ld.global.nc.v2.u32 {%0,%1}, [%2];" : "=r"(v.x), "=r"(v.y) : "l"(p));
+    asm volatile("ld.global.v2.u32 {%0,%1}, [%2];" : "=r"(v.x), "=r"(v.y) : "l"(p));
     return v;
 }
 __device__ __forceinline__ uint32_t ldg_now1(const void* p) {
     uint32_t v;
-    asm volatile("ld.global.nc.u32 %0, [%1];" : "=r"(v) : "l"(p));
+    asm volatile("ld.global.u32 %0, [%1];" : "=r"(v) : "l"(p));
     return v;
 }
 
@@ -509,6 +508,8 @@ __global__ void __launch_bounds__(Shape<NQ>::THREADS, Shape<NQ>::CTAS_PER_SM) de
     const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
     const int fg = lane >> 2, ft = lane & 3;
     WS& ws = sm.ws[warp];
+    if (lane == 0) { bar_init(smem_addr(ws.bar)); bar_init(smem_addr(ws.bar) + 8); asm volatile("fence.proxy.async.shared::cta;" ::: "memory"); }
+    qaq_dependency();
     const int T = COUNTED ? *a.d_count : a.T;
     if (COUNTED && T < 1) {          // nothing cached: zeros
         for (int bh = blockIdx.x; bh < a.BH; bh += gridDim.x)
@@ -574,9 +575,9 @@ __global__ void __launch_bounds__(Shape<NQ>::THREADS, Shape<NQ>::CTAS_PER_SM) de
     uint2 qrow[2][NQ], qword[PER];
     const bool q_aligned = ((uintptr_t)a.q & 7) == 0 && (a.q_stride & 3) == 0;
     auto load4 = [&](const __half* p) {
-        if (q_aligned) return __ldg(reinterpret_cast<const uint2*>(p));
+        if (q_aligned) return (*(reinterpret_cast<const uint2*>(p)));
         const unsigned short* h = reinterpret_cast<const unsigned short*>(p);
-        return make_uint2((uint32_t)__ldg(h) | ((uint32_t)__ldg(h + 1) << 16), (uint32_t)__ldg(h + 2) | ((uint32_t)__ldg(h + 3) << 16));
+        return make_uint2((uint32_t)(*(h)) | ((uint32_t)(*(h + 1)) << 16), (uint32_t)(*(h + 2)) | ((uint32_t)(*(h + 3)) << 16));
     };
 #pragma unroll
     for (int sg = 0; sg < 2; ++sg)
@@ -598,7 +599,6 @@ __global__ void __launch_bounds__(Shape<NQ>::THREADS, Shape<NQ>::CTAS_PER_SM) de
         qword[k] = make_uint2(0u, 0u);
         if (sg < nseg && ln < 8 * NQ) qword[k] = load4(a.q + (size_t)(bh0 + sg) * a.q_stride + (ln >> 3) * D + ch);
     }
-    if (lane == 0) { bar_init(bar); bar_init(bar + 8); asm volatile("fence.proxy.async.shared::cta;" ::: "memory"); }
     __syncwarp();
     if (f < f_end) stage(buf, layout(tk), a.k, bh_of(f), tk, 0);
     if (lane == 0 && warp < nseg) {
@@ -798,7 +798,7 @@ __global__ void __launch_bounds__(Shape<NQ>::THREADS, Shape<NQ>::CTAS_PER_SM) de
 #pragma unroll 1
                 for (uint32_t i = lane; i < oc; i += 32) {
                     int tok; float tm[NQ];
-                    term(i < sc ? list[i] : __ldg(a.k.outl + (size_t)bh * a.ocap + tk.z + i), 1.0f, tok, tm);
+                    term(i < sc ? list[i] : (*(a.k.outl + (size_t)bh * a.ocap + tk.z + i)), 1.0f, tok, tm);
 #pragma unroll
                     for (int j = 0; j < NQ; ++j) wide_add(&ws.kcorr[j][0][tok], &ws.kcorr[j][1][tok], tm[j]);
                 }
@@ -979,7 +979,7 @@ __global__ void __launch_bounds__(Shape<NQ>::THREADS, Shape<NQ>::CTAS_PER_SM) de
                     __syncwarp();
 #pragma unroll 1
                     for (uint32_t i = lane; i < oc; i += 32) {
-                        const uint32_t v = i < sc ? list[i] : __ldg(a.v.outl + (size_t)bh * a.ocap + tv.z + i);
+                        const uint32_t v = i < sc ? list[i] : (*(a.v.outl + (size_t)bh * a.ocap + tv.z + i));
                         const int ch = (v >> 16) & (D - 1);
                         wide_add(&ws.vcorr[0][ch], &ws.vcorr[1][ch], term(v, j));
                     }
@@ -1059,6 +1059,7 @@ __global__ void __launch_bounds__(Shape<NQ>::THREADS, Shape<NQ>::CTAS_PER_SM) de
 
 // Score rows too long for one CTA to normalise on the side.
 __global__ void scores_kernel(float* scores, long stride, const float* ml, int T, const int* d_count) {
+    qaq_dependency();
     const int bh = blockIdx.y;
     if (d_count) T = *d_count;
     const float M = ml[2 * bh], L = ml[2 * bh + 1];
@@ -1090,15 +1091,14 @@ template <int D, int NQ, bool COUNTED>
 qaq_status launch_decode(const DecArgs& a, cudaStream_t s) {
     const size_t smem = sizeof(DecSmem<D, NQ>);
     static_assert(sizeof(DecSmem<D, NQ>) + 1024 <= 227 * 1024 / Shape<NQ>::CTAS_PER_SM, "shared memory of the CTAs of an SM");
-    if (smem > 48 * 1024)
-        QAQ_CUDA_TRY(cudaFuncSetAttribute(decode_kernel<D, NQ, COUNTED>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem));
-    decode_kernel<D, NQ, COUNTED><<<a.ncta, Shape<NQ>::THREADS, smem, s>>>(a);
+    static std::atomic<unsigned long long> seen{0};
+    QAQ_CUDA_TRY(qaq_allow_smem((const void*)decode_kernel<D, NQ, COUNTED>, smem, seen));
+    QAQ_CUDA_TRY(qaq_launch(decode_kernel<D, NQ, COUNTED>, dim3(a.ncta), dim3(Shape<NQ>::THREADS), smem, s, a));
     if (NQ == 1 && a.ml) {
         int gx = (a.T + 1023) / 1024;     // counted: a.T holds the capacity
         if (gx > 64) gx = 64;
-        scores_kernel<<<dim3(gx, a.BH), 256, 0, s>>>(a.scores, a.scores_stride, a.ml, a.T, COUNTED ? a.d_count : nullptr);
+        QAQ_CUDA_TRY(qaq_launch(scores_kernel, dim3(gx, a.BH), dim3(256), 0, s, a.scores, a.scores_stride, a.ml, a.T, COUNTED ? a.d_count : nullptr));
     }
-    QAQ_CUDA_TRY(cudaGetLastError());
     return QAQ_OK;
 }
 

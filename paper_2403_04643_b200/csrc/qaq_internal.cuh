@@ -4,6 +4,8 @@
 #include <cuda_runtime.h>
 #include <stdint.h>
 
+#include <atomic>
+
 #include "qaq.h"
 
 #define QAQ_TILE QAQ_TILE_TOKENS
@@ -58,6 +60,38 @@ static inline int* qaq_d_count(const qaq_cache* c) { return c->d_status + 1; }
 static inline unsigned* qaq_d_ticket(const qaq_cache* c) { return (unsigned*)(c->d_status + 2); }
 
 #ifdef __CUDACC__
+// Kernels of this library are launched with programmatic dependent launch: the launch of a kernel is prepared while the
+// one before runs, its CTAs begin as the last ones of the one before leave, and wait there (qaq_dependency) until all
+// writes of the one before are visible.  Every kernel launched with qaq_launch calls qaq_dependency first thing in every
+// CTA; so a kernel that has got past it has everything before it in the stream behind it.  Such a kernel must not use
+// non-coherent loads (__ldg) for what its predecessor writes.  Letting the successor begin earlier
+// (griddepcontrol.launch_dependents) was slower: its waiting CTAs take room (a captured step of four layers: 24.1 us per
+// layer without, 26.7 with it at the start of the kernels, 24.4 without dependent launch; a 333-token prefill 58, 64, 75).
+__device__ __forceinline__ void qaq_dependency() {
+    asm volatile("griddepcontrol.wait;" ::: "memory");
+}
+template <typename... P, typename... A>
+static inline cudaError_t qaq_launch(void (*kernel)(P...), dim3 grid, dim3 block, size_t smem, cudaStream_t s, A... args) {
+    cudaLaunchAttribute at[1];
+    at[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
+    at[0].val.programmaticStreamSerializationAllowed = 1;
+    cudaLaunchConfig_t lc = {};
+    lc.gridDim = grid; lc.blockDim = block; lc.dynamicSmemBytes = smem; lc.stream = s; lc.attrs = at; lc.numAttrs = 1;
+    return cudaLaunchKernelEx(&lc, kernel, P(args)...);
+}
+// Shared memory beyond 48 KB has to be allowed once per kernel and device; `seen` (one per kernel) remembers where that
+// has been done (devices 0..63; others are asked every time).
+static inline cudaError_t qaq_allow_smem(const void* kernel, size_t smem, std::atomic<unsigned long long>& seen) {
+    int dev = 0;
+    cudaError_t e = cudaGetDevice(&dev);
+    if (e != cudaSuccess) return e;
+    const unsigned long long bit = dev < 64 ? 1ull << dev : 0ull;
+    if (seen.load(std::memory_order_acquire) & bit) return cudaSuccess;
+    e = cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+    if (e == cudaSuccess) seen.fetch_or(bit, std::memory_order_release);
+    return e;
+}
+
 // Space taken from a pool that turned out not to fit is given back only while nothing has been taken behind it: with a
 // plain subtraction a later taker could be handed space that somebody else holds.  Otherwise it stays taken until
 // qaq_cache_compact or qaq_cache_reset.

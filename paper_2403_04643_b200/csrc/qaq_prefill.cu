@@ -49,6 +49,7 @@ template <int D>
 __global__ void __launch_bounds__(PW_WARPS * 32) window_logits_kernel(const PrefillArgs a) {
     constexpr int WPL = D / 8;          // 32-bit words per lane and row
     constexpr int KS = D / 16;          // k-steps
+    qaq_dependency();
     const int bh = blockIdx.y, chunk = blockIdx.x;
     const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
     const int g = lane >> 2, c = lane & 3;
@@ -167,6 +168,7 @@ __global__ void __launch_bounds__(PW_WARPS * 32) window_logits_kernel(const Pref
 }
 
 __global__ void __launch_bounds__(256) window_normalize_kernel(const PrefillArgs a) {
+    qaq_dependency();
     const int bh = blockIdx.y, chunk = blockIdx.x;
     __shared__ float s_m[PW_MAXQ], s_inv[PW_MAXQ];
     const float NEG = __int_as_float(0xff800000);
@@ -221,6 +223,7 @@ __global__ void __launch_bounds__(PC_WARPS * 32, PC_MINCTA) window_cluster_kerne
     __shared__ float2 s_all[PC_MAXCTA][PW_MAXQ];             // (max, sum of exponentials) of every row over the tokens of every CTA
                                                              // of the cluster: each CTA writes its entries into all the copies
     __shared__ float s_inv[PW_MAXQ];
+    qaq_dependency();
     const int bh = blockIdx.y, chunk = blockIdx.x;
     const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
     const int g = lane >> 2, c = lane & 3;
@@ -493,10 +496,12 @@ extern "C" qaq_status qaq_prefill_window(const qaq_config* cfg, const void* Q, c
         lc.blockDim = dim3(PC_WARPS * 32);
         lc.dynamicSmemBytes = smem;
         lc.stream = s;
-        cudaLaunchAttribute at[1];
+        cudaLaunchAttribute at[2];
+        at[1].id = cudaLaunchAttributeProgrammaticStreamSerialization;
+        at[1].val.programmaticStreamSerializationAllowed = 1;
         at[0].id = cudaLaunchAttributeClusterDimension;
         at[0].val.clusterDim.x = (unsigned)ncl; at[0].val.clusterDim.y = 1; at[0].val.clusterDim.z = 1;
-        lc.attrs = at; lc.numAttrs = 1;
+        lc.attrs = at; lc.numAttrs = 2;
         switch (cfg->head_dim) {
             case 32:
                 QAQ_CUDA_TRY(cudaFuncSetAttribute(window_cluster_kernel<32>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem));
@@ -514,13 +519,12 @@ extern "C" qaq_status qaq_prefill_window(const qaq_config* cfg, const void* Q, c
     }
     const dim3 grid((unsigned)a.nchunk, (unsigned)(cfg->batch * cfg->heads));
     switch (cfg->head_dim) {
-        case 32: window_logits_kernel<32><<<grid, PW_WARPS * 32, 0, s>>>(a); break;
-        case 64: window_logits_kernel<64><<<grid, PW_WARPS * 32, 0, s>>>(a); break;
-        case 128: window_logits_kernel<128><<<grid, PW_WARPS * 32, 0, s>>>(a); break;
+        case 32: QAQ_CUDA_TRY(qaq_launch(window_logits_kernel<32>, grid, dim3(PW_WARPS * 32), 0, s, a)); break;
+        case 64: QAQ_CUDA_TRY(qaq_launch(window_logits_kernel<64>, grid, dim3(PW_WARPS * 32), 0, s, a)); break;
+        case 128: QAQ_CUDA_TRY(qaq_launch(window_logits_kernel<128>, grid, dim3(PW_WARPS * 32), 0, s, a)); break;
         default: return QAQ_ERR_UNSUPPORTED_SHAPE;
     }
-    window_normalize_kernel<<<grid, 256, 0, s>>>(a);
-    QAQ_CUDA_TRY(cudaGetLastError());
+    QAQ_CUDA_TRY(qaq_launch(window_normalize_kernel, grid, dim3(256), 0, s, a));
     return QAQ_OK;
 }
 

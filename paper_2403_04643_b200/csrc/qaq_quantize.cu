@@ -135,6 +135,7 @@ __global__ void __launch_bounds__(2 * D, XSEL < 0 ? (D == 128 ? 3 : 4) : (D == 1
     const int bh = blockIdx.y;
     const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
     const int slot = tid / P, p = tid % P;
+    qaq_dependency();
     int t_old = a.t_old, first_tile = a.first_tile;
     if (COUNTED && a.d_count) {
         t_old = *a.d_count;                // the same value in every thread of the launch: it is written only by tick()
@@ -246,12 +247,12 @@ __global__ void __launch_bounds__(2 * D, XSEL < 0 ? (D == 128 ? 3 : 4) : (D == 1
             for (; i + 7 * P < a.W; i += 8 * P) {
                 float v[8];
 #pragma unroll
-                for (int u = 0; u < 8; ++u) v[u] = __ldg(r + (size_t)(i + u * P) * a.n_new);
+                for (int u = 0; u < 8; ++u) v[u] = (*(r + (size_t)(i + u * P) * a.n_new));
 #pragma unroll
                 for (int u = 0; u < 8; ++u) if (i + u * P < nv_tok) shat = fmaxf(shat, v[u]);
             }
             for (; i < a.W; i += P) {
-                const float v = __ldg(r + (size_t)i * a.n_new);
+                const float v = (*(r + (size_t)i * a.n_new));
                 if (i < nv_tok) shat = fmaxf(shat, v);
             }
         }
@@ -561,9 +562,9 @@ __global__ void __launch_bounds__(2 * D, XSEL < 0 ? (D == 128 ? 3 : 4) : (D == 1
 template <bool SELECT_ONLY, int XSEL>
 qaq_status launch_x(int D, dim3 grid, const QuantArgs& a, cudaStream_t s) {
     switch (D) {
-        case 32: quant_kernel<32, SELECT_ONLY, XSEL><<<grid, 64, 0, s>>>(a); break;
-        case 64: quant_kernel<64, SELECT_ONLY, XSEL><<<grid, 128, 0, s>>>(a); break;
-        case 128: quant_kernel<128, SELECT_ONLY, XSEL><<<grid, 256, 0, s>>>(a); break;
+        case 32: QAQ_CUDA_TRY(qaq_launch(quant_kernel<32, SELECT_ONLY, XSEL>, grid, dim3(64), 0, s, a)); break;
+        case 64: QAQ_CUDA_TRY(qaq_launch(quant_kernel<64, SELECT_ONLY, XSEL>, grid, dim3(128), 0, s, a)); break;
+        case 128: QAQ_CUDA_TRY(qaq_launch(quant_kernel<128, SELECT_ONLY, XSEL>, grid, dim3(256), 0, s, a)); break;
         default: return QAQ_ERR_UNSUPPORTED_SHAPE;
     }
     return QAQ_OK;
@@ -578,9 +579,7 @@ qaq_status launch(int D, dim3 grid, const QuantArgs& a, cudaStream_t s) {
         st = launch_x<SELECT_ONLY, 0>(D, grid, a, s);
         if (st == QAQ_OK) st = launch_x<SELECT_ONLY, 1>(D, grid, a, s);
     }
-    if (st != QAQ_OK) return st;
-    QAQ_CUDA_TRY(cudaGetLastError());
-    return QAQ_OK;
+    return st;
 }
 
 qaq_status check_dense(const void* K, const void* V, long sb, long sh, long st, int D) {
@@ -692,7 +691,5 @@ extern "C" qaq_status qaq_stream_append(qaq_cache* c, const void* k_new, const v
     a.tmax_pad = c->tmax_pad; a.ntiles = c->ntiles; a.status = c->d_status;
     a.d_count = qaq_d_count(c); a.d_ticket = qaq_d_ticket(c); a.max_tokens = (int)c->cfg.max_tokens;
     st = launch_x<false, -1>(D, dim3(1, c->BH), a, (cudaStream_t)stream);
-    if (st != QAQ_OK) return st;
-    QAQ_CUDA_TRY(cudaGetLastError());
-    return QAQ_OK;
+    return st;
 }

@@ -68,6 +68,7 @@ __global__ void __launch_bounds__(2 * D) requant_kernel(const RequantArgs a) {
     constexpr int P = D / 32;
     constexpr int NT = 2 * D;
     constexpr int IMG = qaqc::tile_bytes_max(D);
+    qaq_dependency();
     const int tile = a.first_tile + blockIdx.x, bh = blockIdx.y;
     const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
     const int slot = tid / P, p = tid % P;
@@ -299,12 +300,11 @@ __global__ void __launch_bounds__(2 * D) requant_kernel(const RequantArgs a) {
 template <bool UP>
 qaq_status launch_requant(int D, dim3 grid, const RequantArgs& a, cudaStream_t s) {
     switch (D) {
-        case 32: requant_kernel<32, UP><<<grid, 64, 0, s>>>(a); break;
-        case 64: requant_kernel<64, UP><<<grid, 128, 0, s>>>(a); break;
-        case 128: requant_kernel<128, UP><<<grid, 256, 0, s>>>(a); break;
+        case 32: QAQ_CUDA_TRY(qaq_launch(requant_kernel<32, UP>, grid, dim3(64), 0, s, a)); break;
+        case 64: QAQ_CUDA_TRY(qaq_launch(requant_kernel<64, UP>, grid, dim3(128), 0, s, a)); break;
+        case 128: QAQ_CUDA_TRY(qaq_launch(requant_kernel<128, UP>, grid, dim3(256), 0, s, a)); break;
         default: return QAQ_ERR_UNSUPPORTED_SHAPE;
     }
-    QAQ_CUDA_TRY(cudaGetLastError());
     return QAQ_OK;
 }
 
@@ -387,6 +387,7 @@ struct CompactArgs {
 };
 
 __global__ void __launch_bounds__(256) compact_kernel(const CompactArgs a) {
+    qaq_dependency();
     const int bh = blockIdx.x;
     const TensorStore& ts = a.t[blockIdx.y];
     __shared__ unsigned long long s_key[COMPACT_MAX_TILES];   // current offset << 32 | tile index
@@ -452,8 +453,7 @@ extern "C" qaq_status qaq_cache_compact(qaq_cache* c, void* stream) {
     if (nt > COMPACT_MAX_TILES) return QAQ_ERR_UNSUPPORTED_SHAPE;
     CompactArgs a;
     a.t[0] = c->t[0]; a.t[1] = c->t[1]; a.pool_bytes = c->pool_bytes; a.ntiles = c->ntiles; a.T = (int)c->tokens;
-    compact_kernel<<<dim3((unsigned)c->BH, 2), 256, 0, (cudaStream_t)stream>>>(a);
-    QAQ_CUDA_TRY(cudaGetLastError());
+    QAQ_CUDA_TRY(qaq_launch(compact_kernel, dim3((unsigned)c->BH, 2), dim3(256), 0, (cudaStream_t)stream, a));
     return QAQ_OK;
 }
 

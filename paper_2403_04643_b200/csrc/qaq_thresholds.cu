@@ -238,6 +238,7 @@ __device__ __forceinline__ unsigned long long rank_k(double alpha, unsigned long
 
 // ---- 1. sample: brackets (or the exact answer when the sample is the whole problem)
 __global__ void __launch_bounds__(256) thr_sample_kernel(const ThrArgs a) {
+    qaq_dependency();
     const int bhx = blockIdx.x, bh = bhx >> 1, x = bhx & 1;
     __shared__ __align__(16) unsigned short s_keys[SAMPLE_TOKENS * 128];
     __shared__ uint32_t hist[2048], s_tmp[4], s_cnt[2];
@@ -309,6 +310,7 @@ __global__ void __launch_bounds__(256) thr_sample_kernel(const ThrArgs a) {
 // together the warp looks at them entry by entry with all lanes busy.  Nothing in the loop needs the other warps:
 // no CTA barrier, one shared-memory reservation per warp, tail and batch of set-aside pieces.
 __global__ void __launch_bounds__(256) thr_scan_kernel(const ThrArgs a) {
+    qaq_dependency();
     const int bhx = blockIdx.y, bh = bhx >> 1, x = bhx & 1;
     Problem* pr = a.prob + bhx;
     if (pr->done) return;
@@ -440,6 +442,7 @@ __global__ void __launch_bounds__(256) thr_scan_kernel(const ThrArgs a) {
 // ---- 3. exact select among the candidates, exact fallback over the data when that is not possible.
 // One CTA per (problem, tail): the two tails are independent order statistics.
 __global__ void __launch_bounds__(256) thr_select_kernel(const ThrArgs a) {
+    qaq_dependency();
     const int bhx = blockIdx.x >> 1, side = blockIdx.x & 1, bh = bhx >> 1, x = bhx & 1;
     Problem* pr = a.prob + bhx;
     if (pr->done) return;
@@ -537,13 +540,12 @@ extern "C" qaq_status qaq_outlier_thresholds(const qaq_config* cfg, const void* 
     a.list = (unsigned short*)((char*)ws + head);
     a.thr = thr;
     a.scan_tokens = SCAN_TOKENS_MAX;
-    thr_sample_kernel<<<BH * 2, 256, 0, s>>>(a);
+    QAQ_CUDA_TRY(qaq_launch(thr_sample_kernel, dim3(BH * 2), dim3(256), 0, s, a));
     if (n_tokens > SAMPLE_TOKENS) {
         a.scan_tokens = scan_tokens_for(cfg->outlier_frac, cfg->head_dim);
         dim3 grid((n_tokens + a.scan_tokens - 1) / a.scan_tokens, BH * 2);
-        thr_scan_kernel<<<grid, 256, 0, s>>>(a);
-        thr_select_kernel<<<BH * 4, 256, 0, s>>>(a);
+        QAQ_CUDA_TRY(qaq_launch(thr_scan_kernel, grid, dim3(256), 0, s, a));
+        QAQ_CUDA_TRY(qaq_launch(thr_select_kernel, dim3(BH * 4), dim3(256), 0, s, a));
     }
-    QAQ_CUDA_TRY(cudaGetLastError());
     return QAQ_OK;
 }
