@@ -10,17 +10,17 @@
 // on the tensor cores (mma.sync m16n8k16, binary16 in, binary32 accumulate); with n <= 64 rows it is
 // bound by reading K once.  Sequences of up to 4096 tokens take one kernel whose CTAs form a
 // thread-block cluster per (b,h) (logits stay in shared memory, row statistics travel through
-// distributed shared memory, the ring is written once); longer ones take two kernels: logits +
-// per-chunk (max, sum of exponentials) of every row, then the rows are normalised in place with
-// the merged (max, sum).
+// distributed shared memory, the ring is written once); longer ones take two passes of one kernel: the first
+// leaves (max, sum of exponentials) of every row per chunk of tokens, the second computes the logits again
+// and writes the rows normalised with the merged statistics.
 #include <cooperative_groups.h>
 
 #include "qaq_internal.cuh"
 
 namespace {
 
-constexpr int PW_WARPS = 4;
-constexpr int PW_CHUNK = 256;          // tokens per CTA: 64 per warp, 8 at a time
+constexpr int PW_WARPS = 16;           // two CTAs per SM (64 registers per thread)
+constexpr int PW_CHUNK = 512;          // tokens per CTA: 32 per warp, 16 at a time
 constexpr int PW_MAXQ = 64;            // rows (queries) at most
 
 struct PrefillArgs {
@@ -42,159 +42,173 @@ __device__ __forceinline__ void mma_16816(float (&c)[4], const uint32_t (&a)[4],
                  : "r"(a[0]), "r"(a[1]), "r"(a[2]), "r"(a[3]), "r"(b0), "r"(b1));
 }
 
-// The contraction index is permuted the same way in both operands: lane c (of the four lanes that
-// share a row / a token) owns channels [c*D/4, (c+1)*D/4), read with 16-byte loads; k-step ks takes
-// words 2ks and 2ks+1 of them.
+// The queries as A-operand fragments in shared memory, one uint4 per (16-row tile, k step, lane): every warp reads the
+// same ones.  The contraction index is permuted the same way in both operands: lane (., c) of k step ks takes words
+// 2 (ks mod 2), + 1 of the 16-byte piece 4 (ks / 2) + c of a row.
 template <int D>
-__global__ void __launch_bounds__(PW_WARPS * 32) window_logits_kernel(const PrefillArgs a) {
-    constexpr int WPL = D / 8;          // 32-bit words per lane and row
+__device__ __forceinline__ void lay_out_queries(uint4* s_q, const __half* Qb, int n) {
+    constexpr int KS = D / 16;
+    const int ntile = 2 * ((n + 31) / 32);
+    for (int idx = threadIdx.x; idx < ntile * KS * 32; idx += blockDim.x) {
+        const int ln = idx & 31, ks = (idx >> 5) % KS, tile = idx / (32 * KS);
+        const int r0 = tile * 16 + (ln >> 2), r1 = r0 + 8, cc = ln & 3;
+        const int w0 = 4 * (4 * (ks >> 1) + cc) + 2 * (ks & 1);
+        const uint32_t* q0 = reinterpret_cast<const uint32_t*>(Qb + (size_t)r0 * D) + w0;
+        const uint32_t* q1 = reinterpret_cast<const uint32_t*>(Qb + (size_t)r1 * D) + w0;
+        uint4 f;
+        f.x = r0 < n ? q0[0] : 0u;
+        f.y = r1 < n ? q1[0] : 0u;
+        f.z = r0 < n ? q0[1] : 0u;
+        f.w = r1 < n ? q1[1] : 0u;
+        s_q[idx] = f;
+    }
+}
+
+template <int D>
+__device__ __forceinline__ void query_norms(const PrefillArgs& a, int bh) {
+    const __half* Qb = a.Q + (size_t)bh * a.n * D;
+    for (int i = threadIdx.x; i < a.n; i += blockDim.x) {
+        float s = 0.f;
+        for (int d = 0; d < D; ++d) { const float f = a.scale * __half2float(Qb[(size_t)i * D + d]); s = fmaf(f, f, s); }
+        a.qnorm2[(size_t)bh * a.n + i] = s;
+    }
+}
+
+__device__ __forceinline__ void fold_stats(float2& to, const float2& p) {          // (max, sum of exponentials)
+    const float NEG = __int_as_float(0xff800000), m = fmaxf(to.x, p.x);
+    to.y = (to.x == NEG ? 0.f : to.y * __expf(to.x - m)) + (p.x == NEG ? 0.f : p.y * __expf(p.x - m));
+    to.x = m;
+}
+
+// Sequences of more than a cluster of CTAs.  What bounds it is memory: the keys are read twice and the rows written once.
+// (Logits written by the first pass and normalised in place by a second kernel - the keys read once, the rows written
+// twice and read once - took 374 + 217 us for 160 (b,h) x 8192 tokens and 64 rows.)  A warp takes 16 tokens per
+// step; column g of its two 8-token operands is token 4 (g / 2) + (g mod 2) resp. that + 2, so that a lane ends up with
+// four consecutive tokens of a row.  STATS: the first pass.
+template <int D, bool STATS>
+__global__ void __launch_bounds__(PW_WARPS * 32, 2) window_long_kernel(const PrefillArgs a) {
+    constexpr int WPL = D / 8;          // 32-bit words per lane and token
     constexpr int KS = D / 16;          // k-steps
+    extern __shared__ __align__(16) float s_dyn[];
+    uint4* s_q = reinterpret_cast<uint4*>(s_dyn);
+    __shared__ float2 s_part[PW_WARPS][PW_MAXQ];             // STATS: per warp; else entry 0: what the rows are normalised with
     qaq_dependency();
     const int bh = blockIdx.y, chunk = blockIdx.x;
     const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
     const int g = lane >> 2, c = lane & 3;
-    const int b_idx = bh / a.H, h_idx = bh % a.H;
-    const __half* Kb = a.K + (size_t)b_idx * a.sb + (size_t)h_idx * a.sh;
-    const __half* Qb = a.Q + (size_t)bh * a.n * D;
-    __shared__ float2 s_part[PW_WARPS][PW_MAXQ];
-
-    if (a.qnorm2 && chunk == 0) {
-        for (int i = threadIdx.x; i < a.n; i += blockDim.x) {
-            float s = 0.f;
-            for (int d = 0; d < D; ++d) { const float f = a.scale * __half2float(Qb[(size_t)i * D + d]); s = fmaf(f, f, s); }
-            a.qnorm2[(size_t)bh * a.n + i] = s;
+    const float NEG = __int_as_float(0xff800000);
+    const __half* Kb = a.K + (size_t)(bh / a.H) * a.sb + (size_t)(bh % a.H) * a.sh;
+    const int t_warp = chunk * PW_CHUNK + warp * (PW_CHUNK / PW_WARPS);
+    // this warp's keys are on their way to L2 while the queries are laid out
+    constexpr int LPT = D >= 64 ? D / 64 : 1;                                    // 128-byte lines per token
+    for (int ln = lane; ln < (PW_CHUNK / PW_WARPS) * LPT; ln += 32) {
+        const int t = t_warp + ln / LPT;
+        if (t < a.T) asm volatile("prefetch.global.L2 [%0];" ::"l"(Kb + (size_t)t * a.st + (ln % LPT) * 64));
+    }
+    if (STATS && a.qnorm2 && chunk == 0) query_norms<D>(a, bh);
+    lay_out_queries<D>(s_q, a.Q + (size_t)bh * a.n * D, a.n);
+    if (!STATS) {      // merged statistics of the rows: eight threads per row
+        const int i = threadIdx.x >> 3, part = threadIdx.x & 7;
+        float2 st = make_float2(NEG, 0.f);
+        if (i < a.n)
+            for (int ch = part; ch < a.nchunk; ch += 8) fold_stats(st, a.part[((size_t)bh * a.nchunk + ch) * a.n + i]);
+#pragma unroll
+        for (int o = 1; o < 8; o <<= 1) fold_stats(st, make_float2(__shfl_xor_sync(0xFFFFFFFFu, st.x, o), __shfl_xor_sync(0xFFFFFFFFu, st.y, o)));
+        if (i < a.n && part == 0) s_part[0][i] = make_float2(st.x, st.y > 0.f ? 1.0f / st.y : 0.f);
+        for (int k = threadIdx.x; k < PW_CHUNK; k += blockDim.x) {
+            const int t = chunk * PW_CHUNK + k;
+            if (t < a.T) a.nvalid[(size_t)bh * a.T + t] = (uint8_t)min(a.n, a.T - t);
         }
     }
-    const int t_warp = chunk * PW_CHUNK + warp * (PW_CHUNK / PW_WARPS);
-    const float NEG = __int_as_float(0xff800000);
+    __syncthreads();
+    const bool vec_ok = (a.T & 3) == 0 && ((uintptr_t)a.ring & 15) == 0;      // rows start 16-byte aligned, no ragged end
 
     for (int mp = 0; mp * 32 < a.n; ++mp) {            // two 16-row tiles of queries at a time
-        uint32_t afr[2][KS][4];
+        float2 st[2][2];                // rows g, g + 8 of the two tiles over the tokens this lane sees
 #pragma unroll
-        for (int mt = 0; mt < 2; ++mt) {
-            const int r0 = mp * 32 + mt * 16 + g, r1 = r0 + 8;
-#pragma unroll
-            for (int ks = 0; ks < KS; ++ks) {
-                const uint32_t* q0 = reinterpret_cast<const uint32_t*>(Qb + (size_t)r0 * D + c * (D / 4)) + 2 * ks;
-                const uint32_t* q1 = reinterpret_cast<const uint32_t*>(Qb + (size_t)r1 * D + c * (D / 4)) + 2 * ks;
-                afr[mt][ks][0] = r0 < a.n ? q0[0] : 0u;
-                afr[mt][ks][1] = r1 < a.n ? q1[0] : 0u;
-                afr[mt][ks][2] = r0 < a.n ? q0[1] : 0u;
-                afr[mt][ks][3] = r1 < a.n ? q1[1] : 0u;
-            }
-        }
-        // running (max, sum) of this lane's share of rows (mt, g) and (mt, g+8)
-        float rm[2][2], rs[2][2];
-#pragma unroll
-        for (int mt = 0; mt < 2; ++mt) { rm[mt][0] = rm[mt][1] = NEG; rs[mt][0] = rs[mt][1] = 0.f; }
-
-#pragma unroll 2
-        for (int step = 0; step < PW_CHUNK / PW_WARPS / 8; ++step) {
-            const int t0 = t_warp + 8 * step;
+        for (int mt = 0; mt < 2; ++mt) st[mt][0] = st[mt][1] = make_float2(NEG, 0.f);
+#pragma unroll 1
+        for (int step = 0; step < PW_CHUNK / PW_WARPS / 16; ++step) {
+            const int t0 = t_warp + 16 * step;
             if (t0 >= a.T) break;
-            uint32_t bw[WPL];
-            {
-                const int t = t0 + g;
-                const uint4* src = reinterpret_cast<const uint4*>(Kb + (size_t)(t < a.T ? t : 0) * a.st + c * (D / 4));
+            uint32_t bw[2][WPL];
+#pragma unroll
+            for (int h = 0; h < 2; ++h) {
+                const int t = t0 + 4 * (g >> 1) + (g & 1) + 2 * h;
+                const uint4* src = reinterpret_cast<const uint4*>(Kb + (size_t)(t < a.T ? t : 0) * a.st) + c;
 #pragma unroll
                 for (int i = 0; i < WPL / 4; ++i) {
                     uint4 v = make_uint4(0, 0, 0, 0);
-                    if (t < a.T) v = src[i];
-                    bw[4 * i] = v.x; bw[4 * i + 1] = v.y; bw[4 * i + 2] = v.z; bw[4 * i + 3] = v.w;
+                    if (t < a.T) v = src[4 * i];
+                    bw[h][4 * i] = v.x; bw[h][4 * i + 1] = v.y; bw[h][4 * i + 2] = v.z; bw[h][4 * i + 3] = v.w;
                 }
             }
-            float acc[2][4];
 #pragma unroll
             for (int mt = 0; mt < 2; ++mt) {
+                float acc[2][4];
 #pragma unroll
-                for (int i = 0; i < 4; ++i) acc[mt][i] = 0.f;
+                for (int i = 0; i < 4; ++i) { acc[0][i] = 0.f; acc[1][i] = 0.f; }
 #pragma unroll
-                for (int ks = 0; ks < KS; ++ks) mma_16816(acc[mt], afr[mt][ks], bw[2 * ks], bw[2 * ks + 1]);
-            }
-            // acc[mt][0..1]: row g, tokens t0+2c, t0+2c+1;  acc[mt][2..3]: row g+8
-#pragma unroll
-            for (int mt = 0; mt < 2; ++mt)
+                for (int ks = 0; ks < KS; ++ks) {
+                    const uint4 f = s_q[((2 * mp + mt) * KS + ks) * 32 + lane];
+                    const uint32_t fr[4] = {f.x, f.y, f.z, f.w};
+                    mma_16816(acc[0], fr, bw[0][2 * ks], bw[0][2 * ks + 1]);
+                    mma_16816(acc[1], fr, bw[1][2 * ks], bw[1][2 * ks + 1]);
+                }
+                // acc[h][2 hr], acc[h][2 hr + 1]: row g + 8 hr, tokens t0 + 4c + 2h, + 1
 #pragma unroll
                 for (int hr = 0; hr < 2; ++hr) {
                     const int i = mp * 32 + mt * 16 + g + 8 * hr;          // query
                     if (i >= a.n) continue;
-                    const int last = a.T - a.n + i;                         // last token the query sees
-                    float* row = a.ring + ((size_t)bh * a.n + (a.n - 1 - i)) * a.T;
+                    const int t = t0 + 4 * c, left = a.T - a.n + i - t + 1; // how many of the lane's tokens the query sees (or more)
+                    const float l[4] = {a.scale * acc[0][2 * hr], a.scale * acc[0][2 * hr + 1], a.scale * acc[1][2 * hr], a.scale * acc[1][2 * hr + 1]};
+                    if (STATS) {
+                        float m = NEG;
 #pragma unroll
-                    for (int e = 0; e < 2; ++e) {
-                        const int t = t0 + 2 * c + e;
-                        if (t >= a.T) continue;
-                        const float l = a.scale * acc[mt][2 * hr + e];
-                        row[t] = l;
-                        if (t <= last) {
-                            const float mnew = fmaxf(rm[mt][hr], l);
-                            rs[mt][hr] = rs[mt][hr] * __expf(rm[mt][hr] - mnew) + __expf(l - mnew);
-                            rm[mt][hr] = mnew;
+                        for (int e = 0; e < 4; ++e) if (e < left) m = fmaxf(m, l[e]);
+                        float sum = 0.f;
+#pragma unroll
+                        for (int e = 0; e < 4; ++e) if (e < left) sum += __expf(l[e] - m);
+                        fold_stats(st[mt][hr], make_float2(m, sum));
+                    } else {
+                        const float2 mi = s_part[0][i];
+                        float4 o;
+                        o.x = left > 0 ? __expf(l[0] - mi.x) * mi.y : 0.f;
+                        o.y = left > 1 ? __expf(l[1] - mi.x) * mi.y : 0.f;
+                        o.z = left > 2 ? __expf(l[2] - mi.x) * mi.y : 0.f;
+                        o.w = left > 3 ? __expf(l[3] - mi.x) * mi.y : 0.f;
+                        float* row = a.ring + ((size_t)bh * a.n + (a.n - 1 - i)) * a.T + t;
+                        if (vec_ok) { if (t < a.T) *reinterpret_cast<float4*>(row) = o; }
+                        else {
+                            if (t < a.T) row[0] = o.x;
+                            if (t + 1 < a.T) row[1] = o.y;
+                            if (t + 2 < a.T) row[2] = o.z;
+                            if (t + 3 < a.T) row[3] = o.w;
                         }
                     }
                 }
+            }
         }
-        // merge the four lanes of a row, then the warps, into the chunk's partial
+        if (STATS) {      // merge the four lanes of a row
 #pragma unroll
-        for (int mt = 0; mt < 2; ++mt)
+            for (int mt = 0; mt < 2; ++mt)
 #pragma unroll
-            for (int hr = 0; hr < 2; ++hr) {
-                float m = rm[mt][hr], s = rs[mt][hr];
-#pragma unroll
-                for (int o = 1; o < 4; o <<= 1) {
-                    const float m2 = __shfl_xor_sync(0xFFFFFFFFu, m, o), s2 = __shfl_xor_sync(0xFFFFFFFFu, s, o);
-                    const float mn = fmaxf(m, m2);
-                    s = (m == NEG ? 0.f : s * __expf(m - mn)) + (m2 == NEG ? 0.f : s2 * __expf(m2 - mn));
-                    m = mn;
+                for (int hr = 0; hr < 2; ++hr) {
+                    float2 v = st[mt][hr];
+                    fold_stats(v, make_float2(__shfl_xor_sync(0xFFFFFFFFu, v.x, 1), __shfl_xor_sync(0xFFFFFFFFu, v.y, 1)));
+                    fold_stats(v, make_float2(__shfl_xor_sync(0xFFFFFFFFu, v.x, 2), __shfl_xor_sync(0xFFFFFFFFu, v.y, 2)));
+                    if (c == 0) s_part[warp][mp * 32 + mt * 16 + g + 8 * hr] = v;
                 }
-                const int il = mt * 16 + g + 8 * hr;                        // row inside this pair of tiles
-                if (c == 0) s_part[warp][il] = make_float2(m, s);
-            }
-        __syncthreads();
-        for (int il = threadIdx.x; il < 32; il += blockDim.x) {
-            const int i = mp * 32 + il;
-            if (i >= a.n) continue;
-            float m = NEG, s = 0.f;
-            for (int w = 0; w < PW_WARPS; ++w) {
-                const float2 p = s_part[w][il];
-                const float mn = fmaxf(m, p.x);
-                s = (m == NEG ? 0.f : s * __expf(m - mn)) + (p.x == NEG ? 0.f : p.y * __expf(p.x - mn));
-                m = mn;
-            }
-            a.part[((size_t)bh * a.nchunk + chunk) * a.n + i] = make_float2(m, s);
         }
-        __syncthreads();
     }
-}
-
-__global__ void __launch_bounds__(256) window_normalize_kernel(const PrefillArgs a) {
-    qaq_dependency();
-    const int bh = blockIdx.y, chunk = blockIdx.x;
-    __shared__ float s_m[PW_MAXQ], s_inv[PW_MAXQ];
-    const float NEG = __int_as_float(0xff800000);
-    for (int i = threadIdx.x; i < a.n; i += blockDim.x) {
-        float m = NEG, s = 0.f;
-        for (int ch = 0; ch < a.nchunk; ++ch) {
-            const float2 p = a.part[((size_t)bh * a.nchunk + ch) * a.n + i];
-            const float mn = fmaxf(m, p.x);
-            s = (m == NEG ? 0.f : s * __expf(m - mn)) + (p.x == NEG ? 0.f : p.y * __expf(p.x - mn));
-            m = mn;
+    if (STATS) {          // then the warps
+        __syncthreads();
+        if ((int)threadIdx.x < a.n) {
+            float2 v = make_float2(NEG, 0.f);
+#pragma unroll
+            for (int w = 0; w < PW_WARPS; ++w) fold_stats(v, s_part[w][threadIdx.x]);
+            a.part[((size_t)bh * a.nchunk + chunk) * a.n + threadIdx.x] = v;
         }
-        s_m[i] = m;
-        s_inv[i] = s > 0.f ? 1.0f / s : 0.f;
-    }
-    __syncthreads();
-    const int t_lo = chunk * PW_CHUNK;
-    const int nt = min(PW_CHUNK, a.T - t_lo);
-    for (int k = threadIdx.x; k < nt; k += blockDim.x) {      // a thread takes a token through all rows
-        const int t = t_lo + k;
-        float* p = a.ring + (size_t)bh * a.n * a.T + t;
-#pragma unroll 4
-        for (int r = 0; r < a.n; ++r) {
-            const int i = a.n - 1 - r;
-            p[(size_t)r * a.T] = (t <= a.T - a.n + i) ? __expf(p[(size_t)r * a.T] - s_m[i]) * s_inv[i] : 0.f;
-        }
-        a.nvalid[(size_t)bh * a.T + t] = (uint8_t)min(a.n, a.T - t);
     }
 }
 
@@ -232,13 +246,7 @@ __global__ void __launch_bounds__(PC_WARPS * 32, PC_MINCTA) window_cluster_kerne
     const __half* Qb = a.Q + (size_t)bh * a.n * D;
     const float NEG = __int_as_float(0xff800000);
 
-    if (a.qnorm2 && chunk == 0) {
-        for (int i = threadIdx.x; i < a.n; i += blockDim.x) {
-            float s = 0.f;
-            for (int d = 0; d < D; ++d) { const float f = a.scale * __half2float(Qb[(size_t)i * D + d]); s = fmaf(f, f, s); }
-            a.qnorm2[(size_t)bh * a.n + i] = s;
-        }
-    }
+    if (a.qnorm2 && chunk == 0) query_norms<D>(a, bh);
     const int t_cta = chunk * PC_CHUNK;
     const int t_warp = t_cta + warp * (PC_CHUNK / PC_WARPS);
     // this warp's keys are on their way to L2 while the queries are laid out
@@ -251,21 +259,7 @@ __global__ void __launch_bounds__(PC_WARPS * 32, PC_MINCTA) window_cluster_kerne
     // to be running (its shared memory may be written)
     asm volatile("barrier.cluster.arrive.release.aligned;" ::: "memory");
 
-    const int ntile = 2 * ((a.n + 31) / 32);
-    for (int idx = threadIdx.x; idx < ntile * KS * 32; idx += blockDim.x) {
-        const int ln = idx & 31, ks = (idx >> 5) % KS, tile = idx / (32 * KS);
-        const int r0 = tile * 16 + (ln >> 2), r1 = r0 + 8, cc = ln & 3;
-        // k step ks of lane (., cc): words 2 (ks mod 2), + 1 of the 16-byte piece 4 (ks / 2) + cc of the row
-        const int w0 = 4 * (4 * (ks >> 1) + cc) + 2 * (ks & 1);
-        const uint32_t* q0 = reinterpret_cast<const uint32_t*>(Qb + (size_t)r0 * D) + w0;
-        const uint32_t* q1 = reinterpret_cast<const uint32_t*>(Qb + (size_t)r1 * D) + w0;
-        uint4 f;
-        f.x = r0 < a.n ? q0[0] : 0u;
-        f.y = r1 < a.n ? q1[0] : 0u;
-        f.z = r0 < a.n ? q0[1] : 0u;
-        f.w = r1 < a.n ? q1[1] : 0u;
-        s_q[idx] = f;
-    }
+    lay_out_queries<D>(s_q, Qb, a.n);
     __syncthreads();
 
     for (int mp = 0; mp * 32 < a.n; ++mp) {            // two 16-row tiles of queries at a time
@@ -400,6 +394,15 @@ __global__ void __launch_bounds__(PC_WARPS * 32, PC_MINCTA) window_cluster_kerne
     for (int k = threadIdx.x; k < nt; k += blockDim.x) a.nvalid[(size_t)bh * a.T + t_cta + k] = (uint8_t)min(a.n, a.T - (t_cta + k));
 }
 
+template <int D>
+qaq_status run_long(const PrefillArgs& a, int BH, cudaStream_t s) {
+    const dim3 grid((unsigned)a.nchunk, (unsigned)BH);
+    const size_t smem = (size_t)(2 * ((a.n + 31) / 32)) * (D / 16) * 32 * sizeof(uint4);       // at most 16 KB
+    QAQ_CUDA_TRY(qaq_launch(window_long_kernel<D, true>, grid, dim3(PW_WARPS * 32), smem, s, a));
+    QAQ_CUDA_TRY(qaq_launch(window_long_kernel<D, false>, grid, dim3(PW_WARPS * 32), smem, s, a));
+    return QAQ_OK;
+}
+
 // Upper quantile of a list of binary32 values (the squared query norms): exact 4 x 8-bit radix select on
 // order-preserving keys by one CTA.  NaNs are not counted.
 constexpr int QS_THREADS = 1024;
@@ -517,15 +520,12 @@ extern "C" qaq_status qaq_prefill_window(const qaq_config* cfg, const void* Q, c
         QAQ_CUDA_TRY(cudaGetLastError());
         return QAQ_OK;
     }
-    const dim3 grid((unsigned)a.nchunk, (unsigned)(cfg->batch * cfg->heads));
     switch (cfg->head_dim) {
-        case 32: QAQ_CUDA_TRY(qaq_launch(window_logits_kernel<32>, grid, dim3(PW_WARPS * 32), 0, s, a)); break;
-        case 64: QAQ_CUDA_TRY(qaq_launch(window_logits_kernel<64>, grid, dim3(PW_WARPS * 32), 0, s, a)); break;
-        case 128: QAQ_CUDA_TRY(qaq_launch(window_logits_kernel<128>, grid, dim3(PW_WARPS * 32), 0, s, a)); break;
-        default: return QAQ_ERR_UNSUPPORTED_SHAPE;
+        case 32: return run_long<32>(a, cfg->batch * cfg->heads, s);
+        case 64: return run_long<64>(a, cfg->batch * cfg->heads, s);
+        case 128: return run_long<128>(a, cfg->batch * cfg->heads, s);
     }
-    QAQ_CUDA_TRY(qaq_launch(window_normalize_kernel, grid, dim3(256), 0, s, a));
-    return QAQ_OK;
+    return QAQ_ERR_UNSUPPORTED_SHAPE;
 }
 
 extern "C" qaq_status qaq_qnorm2_quantile(const float* values, long n, double upper_frac, float* out, void* stream) {

@@ -11,14 +11,16 @@
 // The new widths come from the caller or from the rules of Section 4.1 applied to the stored
 // range (max - min of the token's metadata) with the current score window and policy scalars.
 //
-// One CTA = one tile (QAQ_TILE tokens) of one (b,h), both tensors; head_dim/32 lanes own a
+// One CTA = one tile (QAQ_TILE tokens) of one (b,h) and tensor; head_dim/32 lanes own a
 // token, each lane the codes of 32 consecutive channels, one byte per code in 8 registers.
-// All of a tile's old bytes are in registers before the first new byte is written (the new
-// words are built in a shared-memory image of the tile first), so a tile that does not grow is
-// rewritten in place.  A closed tile that grows takes a new place at the end of its pool (the
-// old bytes stay unused); the open (last, partly filled) tile is handled in a launch of its own
+// A CTA whose widths stay as they are leaves after reading them.  Otherwise the tile's bytes come to
+// shared memory with wide loads, the codes from there to registers, and the image of the new tile takes
+// the same place, so a tile that does not grow is rewritten in place.  (With both tensors in one CTA and
+// the codes read byte by byte from global memory, lowering a 4096-token layer at batch 4 took 135 us and raising it
+// 201; now see the launch below.)  A closed tile that grows takes a new place at the end of its pool (the
+// old bytes stay unused); the open (last, partly filled) tile is then handled in a launch of its own
 // after the closed ones and is kept - or made again - the last thing in its pool, so that later
-// appends continue right behind it.
+// appends continue right behind it.  Lowered widths never make a tile grow.
 #include "qaq_codec.cuh"
 #include "qaq_internal.cuh"
 
@@ -61,239 +63,212 @@ __device__ __forceinline__ void fresh_codes(const __half* row, float lo, float h
     qaqc::codes32(v, mn, mx, B, creg);
 }
 
-// UP: widths may be raised (the unquantized copy is there).  A tile whose bytes grow takes a new place at the end of
-// its pool; closed tiles are handled by one launch, the open tile by a launch of its own after it.
+// UP: widths may be raised (the unquantized copy is there); blockIdx.z: keys or values.
 template <int D, bool UP>
 __global__ void __launch_bounds__(2 * D) requant_kernel(const RequantArgs a) {
     constexpr int P = D / 32;
     constexpr int NT = 2 * D;
     constexpr int IMG = qaqc::tile_bytes_max(D);
     qaq_dependency();
-    const int tile = a.first_tile + blockIdx.x, bh = blockIdx.y;
+    const int tile = a.first_tile + blockIdx.x, bh = blockIdx.y, x = blockIdx.z;
     const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
     const int slot = tid / P, p = tid % P;
     const int tok = tile * QAQ_TILE + slot;
     const bool valid = tok < a.T;
     const bool given = a.bitsK != nullptr;
+    const TensorStore& ts = x ? a.v : a.k;
+    const size_t ti = (size_t)bh * a.ntiles + tile;
 
     __shared__ float s_part[P][QAQ_TILE];
-    __shared__ uint8_t s_nv[QAQ_TILE];
-    __shared__ uint8_t s_bo[2][QAQ_TILE], s_bn[2][QAQ_TILE];      // widths before and after
-    __shared__ qaqc::Section s_otab[2][9], s_tab[2][9];             // sections before and after
-    __shared__ unsigned short s_place[2][QAQ_TILE];                 // new slot | width of its row << 8
-    __shared__ uint8_t s_sorted[2][QAQ_TILE], s_orow[QAQ_TILE / 4]; // new width of every slot; stored width of the rows of values
-    __shared__ uint32_t s_tot[2], s_off[2];                        // new bytes of the tile, where they go in the pool
-    __shared__ int s_skip[2];
-    __shared__ __align__(16) uint8_t s_img[2][IMG];
+    __shared__ uint8_t s_bn[QAQ_TILE];                       // widths afterwards
+    __shared__ qaqc::Section s_otab[9], s_tab[9];            // sections before and after
+    __shared__ unsigned short s_place[QAQ_TILE];             // new slot | width of its row << 8
+    __shared__ uint8_t s_sorted[QAQ_TILE], s_orow[QAQ_TILE / 4];   // new width of every slot; stored width of the rows of values
+    __shared__ uint32_t s_head[4];
+    __shared__ uint32_t s_tot, s_off;                        // new bytes of the tile, where they go in the pool
+    __shared__ int s_skip, s_holes;                          // no room; some slots of the last group of values are empty
+    __shared__ __align__(16) uint8_t s_img[IMG];             // the tile as it was, then as it will be
 
-    // empty slots of the value groups have to read as zero
-    for (int o = tid; o < IMG / 16; o += NT) reinterpret_cast<uint4*>(s_img[1])[o] = make_uint4(0, 0, 0, 0);
-
-    // ---- attention window of the tile's tokens (value rule); P threads share a token's rows
-    {
-        const int g = tid / QAQ_TILE, tk = tid % QAQ_TILE;
-        const int t2 = tile * QAQ_TILE + tk;
-        float m = __int_as_float(0xff800000);
-        int nv = 0;
-        if (!given && t2 < a.T) {
-            nv = a.nvalid[(size_t)bh * a.ncols + t2];
-            nv = nv < a.W ? nv : a.W;
-            const float* r = a.ring + (size_t)bh * a.W * a.ncols + t2;
-            for (int i = g; i < nv; i += P) m = fmaxf(m, r[(size_t)i * a.ncols]);
-        }
-        s_part[g][tk] = m;
-        if (g == 0) s_nv[tk] = (uint8_t)nv;
-    }
-    // ---- current widths and ranges
+    // ---- current width and range of this thread's token
     const size_t mt = (size_t)bh * a.tmax_pad + tok;
-    int Bo[2] = {0, 0}, oslot[2] = {0, 0};
-    float rng[2] = {0.f, 0.f}, mnf[2] = {0.f, 0.f}, mxf[2] = {0.f, 0.f};
+    const uint4 tw = ts.tile[ti];
+    int Bo = 0, oslot = 0;
+    float rng = 0.f, mn = 0.f, mx = 0.f;
     if (valid) {
-#pragma unroll
-        for (int x = 0; x < 2; ++x) {
-            const TensorStore& ts = x ? a.v : a.k;
-            const uint32_t bs = ts.bs[mt];
-            Bo[x] = min((int)(bs & 0xFFu), 8);
-            oslot[x] = (int)((bs >> 8) & (QAQ_TILE - 1));
-            const uint32_t mm = ts.mnmx[mt];
-            mnf[x] = __half2float(__ushort_as_half((unsigned short)(mm & 0xFFFF)));
-            mxf[x] = __half2float(__ushort_as_half((unsigned short)(mm >> 16)));
-            rng[x] = __fsub_rn(mxf[x], mnf[x]);
-        }
+        const uint32_t bs = ts.bs[mt], mm = ts.mnmx[mt];
+        Bo = min((int)(bs & 0xFFu), 8);
+        oslot = (int)((bs >> 8) & (QAQ_TILE - 1));
+        mn = __half2float(__ushort_as_half((unsigned short)(mm & 0xFFFF)));
+        mx = __half2float(__ushort_as_half((unsigned short)(mm >> 16)));
+        rng = __fsub_rn(mx, mn);
     }
-    __syncthreads();   // window partials visible
-
-    // ---- new widths: the rule's (or the caller's) width; without the unquantized copy only where it is lower
-    int Bn[2];
-    bool changed[2];
+    // ---- attention window of the tile's tokens (value rule); P threads share a token's rows.  All rows are read (the
+    //      ring is allocated in full), rows a token has no score in are left out of the maximum: no load waits for another.
+    const bool window = x && !given;
+    int nv = 0;
+    if (window) {
+        const int g = tid / QAQ_TILE, tk = tid % QAQ_TILE, t2 = tile * QAQ_TILE + tk;
+        float m = __int_as_float(0xff800000);
+        if (t2 < a.T) {
+            const int nvt = a.nvalid[(size_t)bh * a.ncols + t2];
+            const float* r = a.ring + (size_t)bh * a.W * a.ncols + t2;
+            int i = g;
+            for (; i + 7 * P < a.W; i += 8 * P) {
+                float v[8];
 #pragma unroll
-    for (int x = 0; x < 2; ++x) {
-        int B = 8;
-        if (valid) {
-            if (given) {
-                B = (x ? a.bitsV : a.bitsK)[(size_t)bh * a.ncols + tok];
-                B = B < 1 ? 1 : (B > 8 ? 8 : B);
-            } else if (x == 0) {
-                B = ladder(rng[0], a.cK, a.bmin, a.bmax);
-            } else {
-                float sh = __int_as_float(0xff800000);
+                for (int u = 0; u < 8; ++u) v[u] = r[(size_t)(i + u * P) * a.ncols];
 #pragma unroll
-                for (int g = 0; g < P; ++g) sh = fmaxf(sh, s_part[g][slot]);
-                B = (s_nv[slot] == 0) ? a.bmax : ladder(__fmul_rn(rng[1], sh), a.cV, a.bmin, a.bmax);
+                for (int u = 0; u < 8; ++u) if (i + u * P < nvt) m = fmaxf(m, v[u]);
+            }
+            for (; i < a.W; i += P) {
+                const float v = r[(size_t)i * a.ncols];
+                if (i < nvt) m = fmaxf(m, v);
             }
         }
-        Bn[x] = !valid ? 0 : ((UP || B < Bo[x]) ? B : Bo[x]);
-        if (p == 0) {
-            s_bo[x][slot] = (uint8_t)Bo[x];
-            s_bn[x][slot] = (uint8_t)Bn[x];
-        }
-        changed[x] = __syncthreads_or(Bn[x] != Bo[x]) != 0;   // also makes the widths visible
+        if (valid) nv = a.nvalid[(size_t)bh * a.ncols + tok];
+        s_part[g][tk] = m;
+        __syncthreads();
     }
+    // ---- new width: the rule's (or the caller's) width; without the unquantized copy only where it is lower
+    int Bn = 0;
+    if (valid) {
+        int B;
+        if (given) {
+            B = (x ? a.bitsV : a.bitsK)[(size_t)bh * a.ncols + tok];
+            B = B < 1 ? 1 : (B > 8 ? 8 : B);
+        } else if (x == 0) {
+            B = ladder(rng, a.cK, a.bmin, a.bmax);
+        } else {
+            float sh = __int_as_float(0xff800000);
+#pragma unroll
+            for (int g = 0; g < P; ++g) sh = fmaxf(sh, s_part[g][slot]);
+            B = min(nv, a.W) == 0 ? a.bmax : ladder(__fmul_rn(rng, sh), a.cV, a.bmin, a.bmax);
+        }
+        Bn = (UP || B < Bo) ? B : Bo;
+    }
+    if (p == 0) s_bn[slot] = (uint8_t)Bn;
+    bool changed = __syncthreads_or(Bn != Bo) != 0;          // also makes the widths visible
     // An open tile has to be the last thing in its pool.  If closed tiles of this (b,h) have just been moved
     // behind it, it moves to the end as well, whether its own tokens change or not.
     const bool open = tile == a.T / QAQ_TILE && (a.T % QAQ_TILE) != 0;
-    bool relocate[2] = {false, false};
-    if (open) {
-        const size_t ti0 = (size_t)bh * a.ntiles + tile;
-#pragma unroll
-        for (int x = 0; x < 2; ++x) {
-            const TensorStore& ts = x ? a.v : a.k;
-            relocate[x] = ts.tile[ti0].x + ts.tile[ti0].y != ts.pool_end[bh];
-            changed[x] = changed[x] || relocate[x];
-        }
-    }
-    if (!changed[0] && !changed[1]) return;
+    const bool relocate = open && tw.x + tw.y != ts.pool_end[bh];
+    changed = changed || relocate;
+    if (!changed) return;
 
-    // ---- warp 0: which slots have a piece of each width, before and after; size and place of the new tile
+    // ---- the stored bytes come to shared memory; warp 0: tokens sorted by their new widths, size and place of the new tile
+    const uint8_t* src = ts.codes + (size_t)bh * a.pool_bytes + tw.x;
+    for (uint32_t o = tid * 16; o < ((tw.y + 15u) & ~15u); o += NT * 16)
+        *reinterpret_cast<uint4*>(s_img + o) = *reinterpret_cast<const uint4*>(src + o);
     if (warp == 0) {
-#pragma unroll
-        for (int x = 0; x < 2; ++x) {
-            {   // the sections as they are stored
-                const TensorStore& ts = x ? a.v : a.k;
-                const size_t ti0 = (size_t)bh * a.ntiles + tile;
-                uint2 h = make_uint2(0u, 0u);
-                if (ts.tile[ti0].y) h = *reinterpret_cast<const uint2*>(ts.codes + (size_t)bh * a.pool_bytes + ts.tile[ti0].x);
-                int n[9];
-                qaqc::counts_of(h.x, h.y, n);
-                if (lane == 0) {
-                    if (x) qaqc::make_sections<qaqc::UNITS<D, true>>(n, s_otab[x], nullptr);
-                    else qaqc::make_sections<qaqc::UNITS<D, false>>(n, s_otab[x], nullptr);
+        int n[9];
+        const int b0 = s_bn[lane], b1 = s_bn[lane + 32];
+        const qaqc::Sorted so = x ? qaqc::sort_tile<true>(lane, b0, b1, n, s_sorted) : qaqc::sort_tile<false>(lane, b0, b1, n, s_sorted);
+        s_place[lane] = (unsigned short)(so.slot[0] | (so.row_w[0] << 8));
+        s_place[lane + 32] = (unsigned short)(so.slot[1] | (so.row_w[1] << 8));
+        const int tokens = __popc(__ballot_sync(0xFFFFFFFFu, b0 != 0)) + __popc(__ballot_sync(0xFFFFFFFFu, b1 != 0));
+        if (lane == 0) {
+            const uint32_t nb = x ? qaqc::make_sections<qaqc::UNITS<D, true>>(n, s_tab, s_head) : qaqc::make_sections<qaqc::UNITS<D, false>>(n, s_tab, s_head);
+            // where the new tile goes: in place unless it grows
+            const uint32_t off = tw.x, old_nb = tw.y;
+            const uint32_t old_own = open ? old_nb : ((old_nb + 15u) & ~15u);   // closed tiles own a rounded amount
+            uint32_t noff = off;
+            int skip = 0;
+            if (nb > old_own || relocate) {
+                if (open && off + old_nb == ts.pool_end[bh]) {
+                    // still the last thing in its pool: it grows where it is
+                    if ((size_t)off + nb + 16 > a.pool_bytes) skip = 1;
+                    else ts.pool_end[bh] = off + nb;
+                } else if (open) {
+                    // behind everything else, 16-byte aligned, and exactly as long as its bytes: the last thing
+                    // in the pool again (one CTA per pool does this, and nobody else touches the pool in its launch)
+                    noff = (ts.pool_end[bh] + 15u) & ~15u;
+                    if ((size_t)noff + nb + 16 > a.pool_bytes) skip = 1;
+                    else ts.pool_end[bh] = noff + nb;
+                } else {
+                    // the end of the pool need not be aligned while a tile is open: take 16 bytes more and align;
+                    // space that does not fit is given back
+                    const uint32_t take = ((nb + 15u) & ~15u) + 16u;
+                    const bool full = *(volatile uint32_t*)&ts.pool_end[bh] > a.pool_bytes;      // takes nothing: the end must not run away
+                    const uint32_t at = full ? 0u : atomicAdd(&ts.pool_end[bh], take);
+                    noff = (at + 15u) & ~15u;
+                    if (full) skip = 1;
+                    else if ((size_t)at + take + 16 > a.pool_bytes) { skip = 1; pool_give_back(&ts.pool_end[bh], at, take); }
                 }
-                if (x && lane < QAQ_TILE / 4) {
-                    int w = 0, end = 0;
-#pragma unroll
-                    for (int k = 8; k >= 1; --k) {
-                        if (lane >= end && lane < end + n[k]) w = k;
-                        end += n[k];
-                    }
-                    s_orow[lane] = (uint8_t)w;
-                }
+                if (skip) atomicMax(a.status, (int)QAQ_ERR_CAPACITY);
             }
-            int n[9];
-            const int b0 = s_bn[x][lane], b1 = s_bn[x][lane + 32];
-            const qaqc::Sorted so = x ? qaqc::sort_tile<true>(lane, b0, b1, n, s_sorted[x]) : qaqc::sort_tile<false>(lane, b0, b1, n, s_sorted[x]);
-            s_place[x][lane] = (unsigned short)(so.slot[0] | (so.row_w[0] << 8));
-            s_place[x][lane + 32] = (unsigned short)(so.slot[1] | (so.row_w[1] << 8));
-            if (lane == 0) {
-                uint32_t* head = reinterpret_cast<uint32_t*>(s_img[x]);
-                const uint32_t nb = x ? qaqc::make_sections<qaqc::UNITS<D, true>>(n, s_tab[x], head)
-                                      : qaqc::make_sections<qaqc::UNITS<D, false>>(n, s_tab[x], head);
-                // where the new tile goes: in place unless it grows
-                const TensorStore& ts = x ? a.v : a.k;
-                const size_t ti0 = (size_t)bh * a.ntiles + tile;
-                const uint32_t off = ts.tile[ti0].x, old_nb = ts.tile[ti0].y;
-                const uint32_t old_own = open ? old_nb : ((old_nb + 15u) & ~15u);   // closed tiles own a rounded amount
-                uint32_t noff = off;
-                int skip = 0;
-                if (changed[x] && (nb > old_own || relocate[x])) {
-                    if (open && off + old_nb == ts.pool_end[bh]) {
-                        // still the last thing in its pool: it grows where it is
-                        if ((size_t)off + nb + 16 > a.pool_bytes) skip = 1;
-                        else ts.pool_end[bh] = off + nb;
-                    } else if (open) {
-                        // behind everything else, 16-byte aligned, and exactly as long as its bytes: the last thing
-                        // in the pool again (this launch has one CTA per (b,h), nobody else touches the pool)
-                        noff = (ts.pool_end[bh] + 15u) & ~15u;
-                        if ((size_t)noff + nb + 16 > a.pool_bytes) skip = 1;
-                        else ts.pool_end[bh] = noff + nb;
-                    } else {
-                        // the end of the pool need not be aligned while a tile is open: take 16 bytes more and align;
-                        // space that does not fit is given back
-                        const uint32_t take = ((nb + 15u) & ~15u) + 16u;
-                        const bool full = *(volatile uint32_t*)&ts.pool_end[bh] > a.pool_bytes;      // takes nothing: the end must not run away
-                        const uint32_t at = full ? 0u : atomicAdd(&ts.pool_end[bh], take);
-                        noff = (at + 15u) & ~15u;
-                        if (full) skip = 1;
-                        else if ((size_t)at + take + 16 > a.pool_bytes) { skip = 1; pool_give_back(&ts.pool_end[bh], at, take); }
-                    }
-                    if (skip) atomicMax(a.status, (int)QAQ_ERR_CAPACITY);
-                }
-                s_tot[x] = nb; s_off[x] = noff; s_skip[x] = skip;
-            }
+            s_tot = nb; s_off = noff; s_skip = skip; s_holes = x && (tokens & 3);
         }
     }
     __syncthreads();
-    // no room in the pool: that tensor's tile stays as it is
-    if (s_skip[0]) changed[0] = false;
-    if (s_skip[1]) changed[1] = false;
-
-    // ---- old pieces -> codes -> low bits dropped -> new pieces in the shared-memory image
-    const size_t ti = (size_t)bh * a.ntiles + tile;
+    if (s_skip) return;                  // no room in the pool: the tile stays as it is
+    // ---- the sections as they are stored
+    if (warp == NT / 32 - 1) {
+        int n[9];
+        const uint32_t* h = reinterpret_cast<const uint32_t*>(s_img);
+        qaqc::counts_of(tw.y ? h[0] : 0u, tw.y ? h[1] : 0u, n);
+        if (lane == 0) {
+            if (x) qaqc::make_sections<qaqc::UNITS<D, true>>(n, s_otab, nullptr);
+            else qaqc::make_sections<qaqc::UNITS<D, false>>(n, s_otab, nullptr);
+        }
+        if (x && lane < QAQ_TILE / 4) {
+            int w = 0, end = 0;
 #pragma unroll
-    for (int x = 0; x < 2; ++x) {
-        if (!changed[x]) continue;
-        const TensorStore& ts = x ? a.v : a.k;
-        uint32_t creg[8];
-        if (valid && Bn[x]) {
-            if (UP && Bn[x] > Bo[x]) {
-                // raised: codes from the unquantized row, with the token's stored min / max and the thresholds
-                const __half* row = (x ? a.Vs : a.Ks) + (size_t)(bh / a.H) * a.sb + (size_t)(bh % a.H) * a.sh +
-                                    (size_t)tok * a.st + 32 * p;
-                fresh_codes(row, a.thr[(size_t)bh * 4 + 2 * x], a.thr[(size_t)bh * 4 + 2 * x + 1], mnf[x], mxf[x], Bn[x], creg);
-            } else {
-                const uint8_t* src = ts.codes + (size_t)bh * a.pool_bytes + ts.tile[ti].x;
-                const int w = x ? (int)s_orow[oslot[x] >> 2] : Bo[x];
-                if (x == 0) qaqc::read_token<D, false>(src, s_otab[x][w], oslot[x], w, p, creg);
-                else        qaqc::read_token<D, true>(src, s_otab[x][w], oslot[x], w, p, creg);
-                const int drop = Bo[x] - Bn[x];
-                const uint32_t keep = 0x01010101u * (0xFFu >> drop);
-#pragma unroll
-                for (int j = 0; j < 8; ++j) creg[j] = (creg[j] >> drop) & keep;
+            for (int k = 8; k >= 1; --k) {
+                if (lane >= end && lane < end + n[k]) w = k;
+                end += n[k];
             }
-            const uint32_t pl = s_place[x][slot];
-            qaqc::write_token<D>(s_img[x], s_tab[x][pl >> 8], x == 1, (int)(pl & 0xFFu), (int)(pl >> 8), p, creg);
+            s_orow[lane] = (uint8_t)w;
         }
     }
-    __syncthreads();   // every old byte of the tile has been read, the image is complete
+    __syncthreads();
+
+    // ---- old words -> codes -> low bits dropped, or codes from the unquantized row
+    uint32_t creg[8];
+    if (Bn) {
+        if (UP && Bn > Bo) {
+            // raised: with the token's stored min / max and the thresholds
+            const __half* row = (x ? a.Vs : a.Ks) + (size_t)(bh / a.H) * a.sb + (size_t)(bh % a.H) * a.sh + (size_t)tok * a.st + 32 * p;
+            fresh_codes(row, a.thr[(size_t)bh * 4 + 2 * x], a.thr[(size_t)bh * 4 + 2 * x + 1], mn, mx, Bn, creg);
+        } else {
+            const int w = x ? (int)s_orow[oslot >> 2] : Bo;
+            if (x == 0) qaqc::read_token<D, false>(s_img, s_otab[w], oslot, w, p, creg);
+            else        qaqc::read_token<D, true>(s_img, s_otab[w], oslot, w, p, creg);
+            const int drop = Bo - Bn;
+            const uint32_t keep = 0x01010101u * (0xFFu >> drop);
+#pragma unroll
+            for (int j = 0; j < 8; ++j) creg[j] = (creg[j] >> drop) & keep;
+        }
+    }
+    __syncthreads();   // every old byte of the tile has been read
+    if (s_holes) {     // empty slots of the value groups have to read as zero
+        for (int o = tid; o < IMG / 16; o += NT) reinterpret_cast<uint4*>(s_img)[o] = make_uint4(0, 0, 0, 0);
+        __syncthreads();
+    }
+    if (tid < 4) reinterpret_cast<uint32_t*>(s_img)[tid] = s_head[tid];
+    const uint32_t pl = s_place[slot];
+    if (Bn) qaqc::write_token<D>(s_img, s_tab[pl >> 8], x == 1, (int)(pl & 0xFFu), (int)(pl >> 8), p, creg);
+    __syncthreads();   // the image is complete
 
     // ---- the image replaces the tile; widths and tile length follow
-#pragma unroll
-    for (int x = 0; x < 2; ++x) {
-        if (!changed[x]) continue;
-        const TensorStore& ts = x ? a.v : a.k;
-        const uint32_t off = s_off[x];
-        uint8_t* dst = ts.codes + (size_t)bh * a.pool_bytes + off;
-        const uint32_t nb = s_tot[x], nb16 = (nb + 15u) & ~15u;
-        if (x == 0) {
-            for (uint32_t o = tid * 16; o < nb16; o += NT * 16)
-                *reinterpret_cast<uint4*>(dst + o) = *reinterpret_cast<const uint4*>(s_img[x] + o);
-        } else {
-            const int row = (tid / (16 * P)) * 4 + (tid & 3), e = (tid >> 2) % (4 * P);
-            if (row < s_tab[x][1].start + s_tab[x][1].n) {
-                const int w = s_sorted[x][4 * row];
-                qaqc::group_out<D>(s_img[x], dst, s_tab[x][w], w, row, e);
-            }
-            if (tid == 0) *reinterpret_cast<uint4*>(dst) = *reinterpret_cast<const uint4*>(s_img[x]);
+    uint8_t* dst = ts.codes + (size_t)bh * a.pool_bytes + s_off;
+    if (x == 0) {
+        for (uint32_t o = tid * 16; o < ((s_tot + 15u) & ~15u); o += NT * 16)
+            *reinterpret_cast<uint4*>(dst + o) = *reinterpret_cast<const uint4*>(s_img + o);
+    } else {
+        const int row = (tid / (16 * P)) * 4 + (tid & 3), e = (tid >> 2) % (4 * P);
+        if (row < s_tab[1].start + s_tab[1].n) {
+            const int w = s_sorted[4 * row];
+            qaqc::group_out<D>(s_img, dst, s_tab[w], w, row, e);
         }
-        if (valid && p == 0) ts.bs[mt] = (unsigned short)(Bn[x] | ((s_place[x][slot] & 0xFFu) << 8));
-        if (tid == 0) {
-            // an open tile that is still the last thing in its pool gives back what it no longer needs:
-            // appends continue right behind its bytes
-            const uint32_t old_off = ts.tile[ti].x, old_nb = ts.tile[ti].y;
-            if (open && off == old_off && nb < old_nb && old_off + old_nb == ts.pool_end[bh]) ts.pool_end[bh] = off + nb;
-            ts.tile[ti].x = off;
-            ts.tile[ti].y = nb;
-        }
+        if (tid == 0) *reinterpret_cast<uint4*>(dst) = *reinterpret_cast<const uint4*>(s_img);
+    }
+    if (valid && p == 0) ts.bs[mt] = (unsigned short)(Bn | ((pl & 0xFFu) << 8));
+    if (tid == 0) {
+        // an open tile that is still the last thing in its pool gives back what it no longer needs:
+        // appends continue right behind its bytes
+        if (open && s_off == tw.x && s_tot < tw.y && tw.x + tw.y == ts.pool_end[bh]) ts.pool_end[bh] = s_off + s_tot;
+        ts.tile[ti].x = s_off;
+        ts.tile[ti].y = s_tot;
     }
 }
 
@@ -346,19 +321,21 @@ extern "C" qaq_status qaq_requantize(qaq_cache* c, const void* K_full, const voi
         if (!a.Ks || !a.Vs || ((uintptr_t)a.Ks & 15) || ((uintptr_t)a.Vs & 15)) return QAQ_ERR_INVALID_ARG;
         a.sb = stride_b; a.sh = stride_h; a.st = stride_t; a.thr = thr;
     }
-    // closed tiles first (a tile that grows moves to the end of its pool), then the open tile, which has to be
-    // the last thing in its pool when this call is over
+    // Where widths may be raised, closed tiles come first (a tile that grows moves to the end of its pool), then the open
+    // tile, which has to be the last thing in its pool when this call is over.  Lowered widths move nothing: one launch.
     const int closed = (int)(c->tokens / QAQ_TILE);
+    if (!up) {
+        a.first_tile = 0;
+        return launch_requant<false>(D, dim3((unsigned)ntile, (unsigned)c->BH, 2), a, s);
+    }
     qaq_status st = QAQ_OK;
     if (closed > 0) {
         a.first_tile = 0;
-        const dim3 grid((unsigned)closed, (unsigned)c->BH);
-        if ((st = up ? launch_requant<true>(D, grid, a, s) : launch_requant<false>(D, grid, a, s)) != QAQ_OK) return st;
+        if ((st = launch_requant<true>(D, dim3((unsigned)closed, (unsigned)c->BH, 2), a, s)) != QAQ_OK) return st;
     }
     if (closed < ntile) {
         a.first_tile = closed;
-        const dim3 grid(1, (unsigned)c->BH);
-        st = up ? launch_requant<true>(D, grid, a, s) : launch_requant<false>(D, grid, a, s);
+        st = launch_requant<true>(D, dim3(1, (unsigned)c->BH, 2), a, s);
     }
     return st;
 }
@@ -373,35 +350,40 @@ extern "C" qaq_status qaq_requantize_down(qaq_cache* c, const uint8_t* bitsK, co
 // Compaction of the code pools.  Tiles that grew in qaq_requantize were placed anew at the end
 // of their pool and left their old bytes behind; this closes the gaps again: the tiles of a
 // (b,h) pool are moved down, in the order in which they lie in memory, until they are
-// contiguous (16-byte aligned each), the open tile last.  One CTA per (b,h) and tensor works
-// through its tiles one after the other; a tile is copied forward in 4 KB pieces, every piece
-// read completely before it is written, so that overlapping source and destination are safe.
+// contiguous (16-byte aligned each), the open tile last.  One CTA per (b,h) and tensor: offsets sorted, new offsets
+// by a prefix sum, then the pool is written front to back in rounds of 32 KB, whatever tiles the bytes
+// belong to.  All loads of a round come before its first store; a byte moves to a lower address or
+// stays, so what a round overwrites no later round reads.  (Moved tile by tile in pieces of 4 KB, every piece a
+// round trip to memory, a pool of 64 tiles took 94 us.)
 namespace {
 
 constexpr int COMPACT_MAX_TILES = 4096;
+constexpr int COMPACT_THREADS = 256, COMPACT_REGS = 8;    // 16-byte pieces per thread and round
 
 struct CompactArgs {
     TensorStore t[2];
     size_t pool_bytes;
-    int ntiles, T;
+    int ntiles, T, n2;       // n2: tiles per (b,h), rounded up to a power of two
 };
 
-__global__ void __launch_bounds__(256) compact_kernel(const CompactArgs a) {
+// dynamic shared memory: n2 keys of 8 bytes, n2 + 1 new offsets, one partial sum per thread
+__global__ void __launch_bounds__(COMPACT_THREADS) compact_kernel(const CompactArgs a) {
     qaq_dependency();
-    const int bh = blockIdx.x;
+    const int bh = blockIdx.x, tid = threadIdx.x;
     const TensorStore& ts = a.t[blockIdx.y];
-    __shared__ unsigned long long s_key[COMPACT_MAX_TILES];   // current offset << 32 | tile index
+    extern __shared__ __align__(16) unsigned char smem_raw[];
+    unsigned long long* s_key = reinterpret_cast<unsigned long long*>(smem_raw);      // current offset << 32 | tile index
+    uint32_t* s_dst = reinterpret_cast<uint32_t*>(s_key + a.n2);                      // new offset of the tile of every rank, end
+    uint32_t* s_sum = s_dst + a.n2 + 1;
     const int nt = (a.T + QAQ_TILE - 1) / QAQ_TILE;
-    int n2 = 1;
-    while (n2 < nt) n2 <<= 1;
-    const size_t row = (size_t)bh * a.ntiles;
-    for (int i = threadIdx.x; i < n2; i += blockDim.x)
-        s_key[i] = i < nt ? ((unsigned long long)ts.tile[row + i].x << 32) | (unsigned)i : ~0ull;
+    uint4* tab = ts.tile + (size_t)bh * a.ntiles;
+    for (int i = tid; i < a.n2; i += COMPACT_THREADS)
+        s_key[i] = i < nt ? ((unsigned long long)tab[i].x << 32) | (unsigned)i : ~0ull;
     __syncthreads();
     // bitonic sort by current offset
-    for (int k = 2; k <= n2; k <<= 1)
+    for (int k = 2; k <= a.n2; k <<= 1)
         for (int j = k >> 1; j > 0; j >>= 1) {
-            for (int i = threadIdx.x; i < n2; i += blockDim.x) {
+            for (int i = tid; i < a.n2; i += COMPACT_THREADS) {
                 const int l = i ^ j;
                 if (l > i) {
                     const unsigned long long x = s_key[i], y = s_key[l];
@@ -411,29 +393,50 @@ __global__ void __launch_bounds__(256) compact_kernel(const CompactArgs a) {
             }
             __syncthreads();
         }
-    uint8_t* pool = ts.codes + (size_t)bh * a.pool_bytes;
-    uint32_t dst = 0;
-    for (int s = 0; s < nt; ++s) {
-        const uint32_t src = (uint32_t)(s_key[s] >> 32);
-        const int tile = (int)(s_key[s] & 0xFFFFFFFFu);
-        const uint32_t n = ts.tile[row + tile].y;
-        const uint32_t n16 = (n + 15u) & ~15u;
-        if (src != dst) {                                  // dst < src: tiles before this one only moved down
-            for (uint32_t o = 0; o < n16; o += 256 * 16) {
-                const uint32_t b = o + threadIdx.x * 16;
-                uint4 v = make_uint4(0, 0, 0, 0);
-                if (b < n16) v = *reinterpret_cast<const uint4*>(pool + src + b);
-                __syncthreads();
-                if (b < n16) *reinterpret_cast<uint4*>(pool + dst + b) = v;
-            }
-            if (threadIdx.x == 0) ts.tile[row + tile].x = dst;
-        }
-        // closed tiles own a 16-byte rounded amount; the open tile, which is the last one, its exact bytes
-        const bool open = tile == a.T / QAQ_TILE && (a.T % QAQ_TILE) != 0;
-        dst += open ? n : n16;
-        __syncthreads();                                   // the next tile's source may be this tile's old place
+    // new offsets: closed tiles own a 16-byte rounded amount; the open tile, if it is the last one, its exact bytes
+    const int per = (nt + COMPACT_THREADS - 1) / COMPACT_THREADS, lo = min(nt, tid * per), hi = min(nt, lo + per);
+    uint32_t sum = 0;
+    for (int i = lo; i < hi; ++i) {
+        const uint32_t n = tab[(uint32_t)s_key[i]].y;
+        s_dst[i] = sum;
+        sum += (i == nt - 1 && (a.T % QAQ_TILE) != 0 && (int)(uint32_t)s_key[i] == a.T / QAQ_TILE) ? n : (n + 15u) & ~15u;
     }
-    if (threadIdx.x == 0) ts.pool_end[bh] = dst;
+    s_sum[tid] = sum;
+    __syncthreads();
+    uint32_t before = 0;
+    for (int i = 0; i < tid; ++i) before += s_sum[i];
+    for (int i = lo; i < hi; ++i) s_dst[i] += before;
+    if (tid == COMPACT_THREADS - 1) s_dst[nt] = before + sum;
+    __syncthreads();
+    // the bytes
+    uint8_t* pool = ts.codes + (size_t)bh * a.pool_bytes;
+    const uint32_t end = s_dst[nt];
+    int first = 0;                                 // tiles before this one are where they belong
+    while (first < nt && (uint32_t)(s_key[first] >> 32) == s_dst[first]) ++first;
+    if (first < nt)
+        for (uint32_t base = s_dst[first]; base < end; base += COMPACT_THREADS * COMPACT_REGS * 16) {
+            uint4 v[COMPACT_REGS];
+#pragma unroll
+            for (int r = 0; r < COMPACT_REGS; ++r) {
+                const uint32_t o = base + (uint32_t)(r * COMPACT_THREADS + tid) * 16;
+                if (o >= end) continue;
+                int l = first, h = nt - 1;         // the last tile whose new offset is at most o
+                while (l < h) {
+                    const int m = (l + h + 1) >> 1;
+                    if (s_dst[m] <= o) l = m; else h = m - 1;
+                }
+                v[r] = *reinterpret_cast<const uint4*>(pool + (uint32_t)(s_key[l] >> 32) + (o - s_dst[l]));
+            }
+            __syncthreads();
+#pragma unroll
+            for (int r = 0; r < COMPACT_REGS; ++r) {
+                const uint32_t o = base + (uint32_t)(r * COMPACT_THREADS + tid) * 16;
+                if (o < end) *reinterpret_cast<uint4*>(pool + o) = v[r];
+            }
+            __syncthreads();
+        }
+    for (int i = tid; i < nt; i += COMPACT_THREADS) tab[(uint32_t)s_key[i]].x = s_dst[i];
+    if (tid == 0) ts.pool_end[bh] = end;
 }
 
 // (a pool end can stand beyond the pool's capacity when takers that found no room could not give their space back)
@@ -453,7 +456,12 @@ extern "C" qaq_status qaq_cache_compact(qaq_cache* c, void* stream) {
     if (nt > COMPACT_MAX_TILES) return QAQ_ERR_UNSUPPORTED_SHAPE;
     CompactArgs a;
     a.t[0] = c->t[0]; a.t[1] = c->t[1]; a.pool_bytes = c->pool_bytes; a.ntiles = c->ntiles; a.T = (int)c->tokens;
-    QAQ_CUDA_TRY(qaq_launch(compact_kernel, dim3((unsigned)c->BH, 2), dim3(256), 0, (cudaStream_t)stream, a));
+    a.n2 = 1;
+    while (a.n2 < nt) a.n2 <<= 1;
+    auto smem_for = [](int n2) { return (size_t)n2 * 8 + (size_t)(n2 + 1) * 4 + COMPACT_THREADS * 4; };
+    static std::atomic<unsigned long long> seen{0};
+    QAQ_CUDA_TRY(qaq_allow_smem((const void*)compact_kernel, smem_for(COMPACT_MAX_TILES), seen));
+    QAQ_CUDA_TRY(qaq_launch(compact_kernel, dim3((unsigned)c->BH, 2), dim3(COMPACT_THREADS), smem_for(a.n2), (cudaStream_t)stream, a));
     return QAQ_OK;
 }
 
