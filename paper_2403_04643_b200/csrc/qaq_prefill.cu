@@ -19,8 +19,8 @@
 
 namespace {
 
-constexpr int PW_WARPS = 16;           // two CTAs per SM (64 registers per thread)
-constexpr int PW_CHUNK = 512;          // tokens per CTA: 32 per warp, 16 at a time
+constexpr int PW_WARPS = 8;            // three CTAs per SM (80 registers per thread)
+constexpr int PW_CHUNK = 512;          // tokens per CTA: 64 per warp, 16 at a time
 constexpr int PW_MAXQ = 64;            // rows (queries) at most
 
 struct PrefillArgs {
@@ -86,7 +86,7 @@ __device__ __forceinline__ void fold_stats(float2& to, const float2& p) {       
 // step; column g of its two 8-token operands is token 4 (g / 2) + (g mod 2) resp. that + 2, so that a lane ends up with
 // four consecutive tokens of a row.  STATS: the first pass.
 template <int D, bool STATS>
-__global__ void __launch_bounds__(PW_WARPS * 32, 2) window_long_kernel(const PrefillArgs a) {
+__global__ void __launch_bounds__(PW_WARPS * 32, 3) window_long_kernel(const PrefillArgs a) {
     constexpr int WPL = D / 8;          // 32-bit words per lane and token
     constexpr int KS = D / 16;          // k-steps
     extern __shared__ __align__(16) float s_dyn[];
@@ -107,13 +107,13 @@ __global__ void __launch_bounds__(PW_WARPS * 32, 2) window_long_kernel(const Pre
     }
     if (STATS && a.qnorm2 && chunk == 0) query_norms<D>(a, bh);
     lay_out_queries<D>(s_q, a.Q + (size_t)bh * a.n * D, a.n);
-    if (!STATS) {      // merged statistics of the rows: eight threads per row
-        const int i = threadIdx.x >> 3, part = threadIdx.x & 7;
+    if (!STATS) {      // merged statistics of the rows: four threads per row
+        const int i = threadIdx.x >> 2, part = threadIdx.x & 3;
         float2 st = make_float2(NEG, 0.f);
         if (i < a.n)
-            for (int ch = part; ch < a.nchunk; ch += 8) fold_stats(st, a.part[((size_t)bh * a.nchunk + ch) * a.n + i]);
+            for (int ch = part; ch < a.nchunk; ch += 4) fold_stats(st, a.part[((size_t)bh * a.nchunk + ch) * a.n + i]);
 #pragma unroll
-        for (int o = 1; o < 8; o <<= 1) fold_stats(st, make_float2(__shfl_xor_sync(0xFFFFFFFFu, st.x, o), __shfl_xor_sync(0xFFFFFFFFu, st.y, o)));
+        for (int o = 1; o < 4; o <<= 1) fold_stats(st, make_float2(__shfl_xor_sync(0xFFFFFFFFu, st.x, o), __shfl_xor_sync(0xFFFFFFFFu, st.y, o)));
         if (i < a.n && part == 0) s_part[0][i] = make_float2(st.x, st.y > 0.f ? 1.0f / st.y : 0.f);
         for (int k = threadIdx.x; k < PW_CHUNK; k += blockDim.x) {
             const int t = chunk * PW_CHUNK + k;
@@ -123,10 +123,11 @@ __global__ void __launch_bounds__(PW_WARPS * 32, 2) window_long_kernel(const Pre
     __syncthreads();
     const bool vec_ok = (a.T & 3) == 0 && ((uintptr_t)a.ring & 15) == 0;      // rows start 16-byte aligned, no ragged end
 
-    for (int mp = 0; mp * 32 < a.n; ++mp) {            // two 16-row tiles of queries at a time
-        float2 st[2][2];                // rows g, g + 8 of the two tiles over the tokens this lane sees
+    {
+        constexpr int MT = PW_MAXQ / 16;                // 16-row tiles of queries: a warp's keys are read once for all of them
+        float2 st[MT][2];               // rows g, g + 8 of the tiles over the tokens this lane sees
 #pragma unroll
-        for (int mt = 0; mt < 2; ++mt) st[mt][0] = st[mt][1] = make_float2(NEG, 0.f);
+        for (int mt = 0; mt < MT; ++mt) st[mt][0] = st[mt][1] = make_float2(NEG, 0.f);
 #pragma unroll 1
         for (int step = 0; step < PW_CHUNK / PW_WARPS / 16; ++step) {
             const int t0 = t_warp + 16 * step;
@@ -144,13 +145,14 @@ __global__ void __launch_bounds__(PW_WARPS * 32, 2) window_long_kernel(const Pre
                 }
             }
 #pragma unroll
-            for (int mt = 0; mt < 2; ++mt) {
+            for (int mt = 0; mt < MT; ++mt) {
+                if (mt * 16 >= a.n) break;
                 float acc[2][4];
 #pragma unroll
                 for (int i = 0; i < 4; ++i) { acc[0][i] = 0.f; acc[1][i] = 0.f; }
 #pragma unroll
                 for (int ks = 0; ks < KS; ++ks) {
-                    const uint4 f = s_q[((2 * mp + mt) * KS + ks) * 32 + lane];
+                    const uint4 f = s_q[(mt * KS + ks) * 32 + lane];
                     const uint32_t fr[4] = {f.x, f.y, f.z, f.w};
                     mma_16816(acc[0], fr, bw[0][2 * ks], bw[0][2 * ks + 1]);
                     mma_16816(acc[1], fr, bw[1][2 * ks], bw[1][2 * ks + 1]);
@@ -158,7 +160,7 @@ __global__ void __launch_bounds__(PW_WARPS * 32, 2) window_long_kernel(const Pre
                 // acc[h][2 hr], acc[h][2 hr + 1]: row g + 8 hr, tokens t0 + 4c + 2h, + 1
 #pragma unroll
                 for (int hr = 0; hr < 2; ++hr) {
-                    const int i = mp * 32 + mt * 16 + g + 8 * hr;          // query
+                    const int i = mt * 16 + g + 8 * hr;          // query
                     if (i >= a.n) continue;
                     const int t = t0 + 4 * c, left = a.T - a.n + i - t + 1; // how many of the lane's tokens the query sees (or more)
                     const float l[4] = {a.scale * acc[0][2 * hr], a.scale * acc[0][2 * hr + 1], a.scale * acc[1][2 * hr], a.scale * acc[1][2 * hr + 1]};
@@ -191,13 +193,13 @@ __global__ void __launch_bounds__(PW_WARPS * 32, 2) window_long_kernel(const Pre
         }
         if (STATS) {      // merge the four lanes of a row
 #pragma unroll
-            for (int mt = 0; mt < 2; ++mt)
+            for (int mt = 0; mt < MT; ++mt)
 #pragma unroll
                 for (int hr = 0; hr < 2; ++hr) {
                     float2 v = st[mt][hr];
                     fold_stats(v, make_float2(__shfl_xor_sync(0xFFFFFFFFu, v.x, 1), __shfl_xor_sync(0xFFFFFFFFu, v.y, 1)));
                     fold_stats(v, make_float2(__shfl_xor_sync(0xFFFFFFFFu, v.x, 2), __shfl_xor_sync(0xFFFFFFFFu, v.y, 2)));
-                    if (c == 0) s_part[warp][mp * 32 + mt * 16 + g + 8 * hr] = v;
+                    if (c == 0) s_part[warp][mt * 16 + g + 8 * hr] = v;
                 }
         }
     }
