@@ -132,17 +132,8 @@ __device__ __forceinline__ float warp_sum(float x) {
 // ------------------------------------------------------------------------------------------ shapes
 // Warps per CTA and CTAs per SM by queries per pass: 16 warps per SM for one query (128 registers each), 12 for four
 // (168 registers: four times the accumulators on the value side).
-#ifndef DEC_W1
-#define DEC_W1 8
-#define DEC_C1 2
-#define DEC_ST1 84
-#endif
-#ifndef DEC_W4
-#define DEC_W4 4
-#define DEC_C4 3
-#endif
 template <int NQ> struct Shape {
-    static constexpr int WARPS = NQ == 4 ? DEC_W4 : (NQ == 2 ? 8 : DEC_W1), CTAS_PER_SM = NQ == 4 ? DEC_C4 : (NQ == 2 ? 2 : DEC_C1), THREADS = 32 * WARPS, SLOTS = 148 * CTAS_PER_SM;
+    static constexpr int WARPS = NQ == 4 ? 4 : 8, CTAS_PER_SM = NQ == 4 ? 3 : 2, THREADS = 32 * WARPS, SLOTS = 148 * CTAS_PER_SM;
 };
 constexpr int SCORES_FUSED_TOKENS = 8192;          // up to here the CTA that merges a (b,h) normalises its score row too
 constexpr uint32_t LIST_STAGED = 1024;             // outlier entries per tile and tensor that come through shared memory at most; more are read in place
@@ -163,6 +154,7 @@ struct DecArgs {
     unsigned long long tag;      // of this call; the low 12 bits are zero
     float* ml;         // [BH][2]   merged (max, sum) for the normalisation of long score rows, or null
     int BH, run, ncta; // (b,h) count; tiles per CTA of the flattened (b,h, tile) sequence; CTAs
+    int nq, groups;    // queries of the launch and groups of NQ of them; blockIdx.y is the group (the last one may be short of queries)
     float* out;
     float* scores;     // [BH][scores_stride] or null (one query only)
     long scores_stride;
@@ -173,10 +165,11 @@ struct DecArgs {
 // each, and a run into pieces of ceil(run / warps), one warp each: as few tiles per warp as fill every SM evenly, and
 // never more than one (b,h) boundary inside a run.
 struct DecPlan { int run, ncta; };
+// Groups of queries share the chip.
 template <int NQ>
-__host__ __device__ inline DecPlan plan_decode(int BH, int ntiles) {
+__host__ __device__ inline DecPlan plan_decode(int BH, int ntiles, int groups) {
     using S = Shape<NQ>;
-    const long long total = (long long)BH * ntiles, warps = (long long)S::SLOTS * S::WARPS;
+    const long long total = (long long)BH * ntiles, warps = (long long)(S::SLOTS / groups) * S::WARPS;
     long long run = (total + warps - 1) / warps * S::WARPS;
     if (run > ntiles) run = ntiles;
     DecPlan p;
@@ -185,11 +178,29 @@ __host__ __device__ inline DecPlan plan_decode(int BH, int ntiles) {
     return p;
 }
 
+// What the CTAs of a group of queries work on.
+template <int D, int NQ>
+struct Group {
+    const __half* q;
+    float *out, *part;
+    unsigned long long* done;
+    int nq;
+    __device__ __forceinline__ explicit Group(const DecArgs& a) : q(a.q), out(a.out), part(a.part), done(a.done), nq(NQ) {
+        if (NQ == 1) return;
+        const int g = blockIdx.y;
+        q += g * NQ * D;
+        out += g * NQ * D;
+        part += (size_t)g * 2 * (Shape<NQ>::SLOTS / a.groups) * NQ * (D + 4);
+        done += (size_t)g * a.BH;
+        nq = min(NQ, a.nq - g * NQ);
+    }
+};
+
 // ------------------------------------------------------------------------------------------ shared memory
 // per-warp scratch for the tile a warp is working on
 template <int D, int NQ>
 struct WarpScratch {
-    static constexpr int STAGE = (NQ == 1 ? DEC_ST1 : 72) * D;      // bytes of the staging buffer; any tile of one tensor fits alone
+    static constexpr int STAGE = (NQ == 1 ? 84 : 72) * D;      // bytes of the staging buffer; any tile of one tensor fits alone
     static constexpr int DOTS = QAQ_TILE + 16;                 // the last row block of a list may store up to 15 rows too many
     static constexpr int WROW = QAQ_TILE + 4;                  // digit rows are spread over the banks
     static constexpr int VC = NQ < 2 ? 2 : NQ;
@@ -432,6 +443,7 @@ __device__ void merge_split(const DecArgs& a, DecSmem<D, NQ>& sm, int bh, int nt
     constexpr int PS = D + 4, CT = D / 4, G = S::THREADS / CT, AHEAD = 4;
     const float NEG = __int_as_float(0xff800000);
     const int tid = threadIdx.x, d4 = tid % CT, grp = tid / CT;
+    const Group<D, NQ> gr(a);
     struct Part { float4 x; float m, l; };
     Part* s_part = reinterpret_cast<Part*>(sm.ws[0].buf);          // [G][CT], then the group's reference and sum beside each
     static_assert(S::THREADS * sizeof(Part) <= sizeof(sm.ws), "scratch of the merge");
@@ -443,7 +455,7 @@ __device__ void merge_split(const DecArgs& a, DecSmem<D, NQ>& sm, int bh, int nt
         to.l = fmaf(wb, p.l, wa * to.l);
         to.m = m;
     };
-    for (int j = 0; j < NQ; ++j) {
+    for (int j = 0; j < gr.nq; ++j) {
         Part mine;
         mine.x = make_float4(0.f, 0.f, 0.f, 0.f); mine.m = NEG; mine.l = 0.f;
         for (int i0 = grp; i0 < n; i0 += AHEAD * G) {
@@ -451,7 +463,7 @@ __device__ void merge_split(const DecArgs& a, DecSmem<D, NQ>& sm, int bh, int nt
 #pragma unroll
             for (int k = 0; k < AHEAD; ++k) {
                 const int i = min(i0 + k * G, n - 1);
-                const float* src = a.part + ((size_t)(i == 0 ? first_slot : 2 * (c_lo + i)) * NQ + j) * PS;
+                const float* src = gr.part + ((size_t)(i == 0 ? first_slot : 2 * (c_lo + i)) * NQ + j) * PS;
                 p[k].x = __ldcg(reinterpret_cast<const float4*>(src) + d4);
                 const float2 ml = __ldcg(reinterpret_cast<const float2*>(src + D));
                 p[k].m = ml.x; p[k].l = ml.y;
@@ -477,7 +489,7 @@ __device__ void merge_split(const DecArgs& a, DecSmem<D, NQ>& sm, int bh, int nt
             }
             if (tid < CT) {
                 const float inv = mine.l > 0.f ? 1.0f / mine.l : 0.f;
-                float* o = a.out + (size_t)bh * a.out_stride + j * D + 4 * d4;
+                float* o = gr.out + (size_t)bh * a.out_stride + j * D + 4 * d4;
                 o[0] = mine.x.x * inv; o[1] = mine.x.y * inv; o[2] = mine.x.z * inv; o[3] = mine.x.w * inv;
             }
             if (NQ == 1) {
@@ -509,6 +521,7 @@ __global__ void __launch_bounds__(Shape<NQ>::THREADS, Shape<NQ>::CTAS_PER_SM) de
     const int fg = lane >> 2, ft = lane & 3;
     WS& ws = sm.ws[warp];
     if (lane == 0) { bar_init(smem_addr(ws.bar)); bar_init(smem_addr(ws.bar) + 8); asm volatile("fence.proxy.async.shared::cta;" ::: "memory"); }
+    const Group<D, NQ> gr(a);
     qaq_dependency();
     const int T = COUNTED ? *a.d_count : a.T;
     if (COUNTED && T < 1) {          // nothing cached: zeros
@@ -518,7 +531,7 @@ __global__ void __launch_bounds__(Shape<NQ>::THREADS, Shape<NQ>::CTAS_PER_SM) de
     }
     // this CTA's run of the flattened (b,h, tile) sequence: it begins in bh0 and may reach into bh0 + 1, which begins at f_bound
     const int ntiles = (T + QAQ_TILE - 1) / QAQ_TILE;
-    const int run = COUNTED ? plan_decode<NQ>(a.BH, ntiles).run : a.run;
+    const int run = COUNTED ? plan_decode<NQ>(a.BH, ntiles, 1).run : a.run;
     const int flat_lo = blockIdx.x * run, flat_hi = min(a.BH * ntiles, flat_lo + run);
     if (flat_lo >= flat_hi) return;
     const int bh0 = flat_lo / ntiles, f_bound = (bh0 + 1) * ntiles;
@@ -575,16 +588,16 @@ __global__ void __launch_bounds__(Shape<NQ>::THREADS, Shape<NQ>::CTAS_PER_SM) de
     uint2 qrow[2][NQ], qword[PER];
     const bool q_aligned = ((uintptr_t)a.q & 7) == 0 && (a.q_stride & 3) == 0;
     auto load4 = [&](const __half* p) {
-        if (q_aligned) return (*(reinterpret_cast<const uint2*>(p)));
+        if (q_aligned) return *reinterpret_cast<const uint2*>(p);
         const unsigned short* h = reinterpret_cast<const unsigned short*>(p);
-        return make_uint2((uint32_t)(*(h)) | ((uint32_t)(*(h + 1)) << 16), (uint32_t)(*(h + 2)) | ((uint32_t)(*(h + 3)) << 16));
+        return make_uint2(h[0] | (uint32_t)h[1] << 16, h[2] | (uint32_t)h[3] << 16);
     };
 #pragma unroll
     for (int sg = 0; sg < 2; ++sg)
 #pragma unroll
         for (int j = 0; j < NQ; ++j) {
             qrow[sg][j] = make_uint2(0u, 0u);
-            if (sg < nseg && 4 * lane < D) qrow[sg][j] = load4(a.q + (size_t)(bh0 + sg) * a.q_stride + j * D + 4 * lane);
+            if (sg < nseg && 4 * lane < D && j < gr.nq) qrow[sg][j] = load4(gr.q + (size_t)(bh0 + sg) * a.q_stride + j * D + 4 * lane);
         }
     // word idx: nibble word r / 2 of lane ln of (b,h) sg, its low (even r) or high nibbles; column ln / 4: the high (even) or
     // low (odd) digit of query ln / 8; first channel: unit p = lt * P / 4, word (lt * P mod 4) + r / 2 of it
@@ -597,14 +610,14 @@ __global__ void __launch_bounds__(Shape<NQ>::THREADS, Shape<NQ>::CTAS_PER_SM) de
         int sg, ln, r, ch;
         word_of(tid + k * S::THREADS, sg, ln, r, ch);
         qword[k] = make_uint2(0u, 0u);
-        if (sg < nseg && ln < 8 * NQ) qword[k] = load4(a.q + (size_t)(bh0 + sg) * a.q_stride + (ln >> 3) * D + ch);
+        if (sg < nseg && ln < 8 * gr.nq) qword[k] = load4(gr.q + (size_t)(bh0 + sg) * a.q_stride + (ln >> 3) * D + ch);
     }
     __syncwarp();
     if (f < f_end) stage(buf, layout(tk), a.k, bh_of(f), tk, 0);
     if (lane == 0 && warp < nseg) {
         int first, n;
         split_of(bh0 + warp, ntiles, run, first, n);
-        if (n > 1) open_count(a.done + bh0 + warp, a.tag);
+        if (n > 1) open_count(gr.done + bh0 + warp, a.tag);
     }
     for (int i = 4 * lane; i < NQ * D; i += 128) *reinterpret_cast<float4*>(&ws.macc[0][0] + i) = make_float4(0.f, 0.f, 0.f, 0.f);
     auto half_at = [](const uint2& v, int i) { return __half2float(__ushort_as_half((unsigned short)((i < 2 ? v.x : v.y) >> (16 * (i & 1))))); };
@@ -798,7 +811,7 @@ __global__ void __launch_bounds__(Shape<NQ>::THREADS, Shape<NQ>::CTAS_PER_SM) de
 #pragma unroll 1
                 for (uint32_t i = lane; i < oc; i += 32) {
                     int tok; float tm[NQ];
-                    term(i < sc ? list[i] : (*(a.k.outl + (size_t)bh * a.ocap + tk.z + i)), 1.0f, tok, tm);
+                    term(i < sc ? list[i] : a.k.outl[(size_t)bh * a.ocap + tk.z + i], 1.0f, tok, tm);
 #pragma unroll
                     for (int j = 0; j < NQ; ++j) wide_add(&ws.kcorr[j][0][tok], &ws.kcorr[j][1][tok], tm[j]);
                 }
@@ -979,7 +992,7 @@ __global__ void __launch_bounds__(Shape<NQ>::THREADS, Shape<NQ>::CTAS_PER_SM) de
                     __syncwarp();
 #pragma unroll 1
                     for (uint32_t i = lane; i < oc; i += 32) {
-                        const uint32_t v = i < sc ? list[i] : (*(a.v.outl + (size_t)bh * a.ocap + tv.z + i));
+                        const uint32_t v = i < sc ? list[i] : a.v.outl[(size_t)bh * a.ocap + tv.z + i];
                         const int ch = (v >> 16) & (D - 1);
                         wide_add(&ws.vcorr[0][ch], &ws.vcorr[1][ch], term(v, j));
                     }
@@ -1023,7 +1036,7 @@ __global__ void __launch_bounds__(Shape<NQ>::THREADS, Shape<NQ>::CTAS_PER_SM) de
         const bool alone = min(flat_hi, (bh + 1) * ntiles) - max(flat_lo, bh * ntiles) == ntiles;        // nothing to merge with
         const bool mine = lane <= S::WARPS && sm.seg[min(lane, S::WARPS)] == seg;
 #pragma unroll 1
-        for (int j = 0; j < NQ; ++j) {
+        for (int j = 0; j < gr.nq; ++j) {
             const float m = mine ? sm.mm[lane][j] : NEG, M = warp_max(m);
             const float wgt = m == NEG ? 0.f : __expf(m - M);
             const float L = warp_sum(mine ? wgt * sm.ml[lane][j] : 0.f);
@@ -1032,9 +1045,9 @@ __global__ void __launch_bounds__(Shape<NQ>::THREADS, Shape<NQ>::CTAS_PER_SM) de
 #pragma unroll
             for (int i = 0; i < S::WARPS; ++i) x = fmaf(__shfl_sync(0xFFFFFFFFu, wgt, i), sm.ws[i].macc[j][d], x);
             x = fmaf(__shfl_sync(0xFFFFFFFFu, wgt, S::WARPS), sm.cross[j][d], x);
-            float* dst = a.part + ((size_t)(2 * blockIdx.x + seg) * NQ + j) * (D + 4);
+            float* dst = gr.part + ((size_t)(2 * blockIdx.x + seg) * NQ + j) * (D + 4);
             if (alone) {
-                if (tid < D) a.out[(size_t)bh * a.out_stride + j * D + tid] = L > 0.f ? x / L : 0.f;
+                if (tid < D) gr.out[(size_t)bh * a.out_stride + j * D + tid] = L > 0.f ? x / L : 0.f;
                 if (NQ == 1) {
                     if (a.ml && tid == 0) { a.ml[2 * bh] = M; a.ml[2 * bh + 1] = L; }
                     if (a.scores && !a.ml) normalise_scores<S::THREADS>(a.scores + (size_t)bh * a.scores_stride, T, M, L);
@@ -1049,7 +1062,7 @@ __global__ void __launch_bounds__(Shape<NQ>::THREADS, Shape<NQ>::CTAS_PER_SM) de
     if (lane == 0 && warp < nseg) {
         int first, n;
         split_of(bh0 + warp, ntiles, run, first, n);
-        sm.last[warp] = n > 1 && count_partial(a.done + bh0 + warp, n);
+        sm.last[warp] = n > 1 && count_partial(gr.done + bh0 + warp, n);
     }
     __syncthreads();
 #pragma unroll 1
@@ -1073,8 +1086,8 @@ __global__ void scores_kernel(float* scores, long stride, const float* ml, int T
 // bytes of workspace: the partials of split (b,h) (two slots per CTA; a grid of more than SLOTS CTAs splits none), the
 // counting words, the merged (max, sum) pairs
 template <int NQ>
-size_t decode_ws_bytes(int BH, int D) {
-    return (size_t)2 * Shape<NQ>::SLOTS * NQ * (D + 4) * sizeof(float) + (size_t)BH * (sizeof(unsigned long long) + 2 * sizeof(float));
+size_t decode_ws_bytes(int BH, int D, int groups) {
+    return (size_t)2 * Shape<NQ>::SLOTS * NQ * (D + 4) * sizeof(float) + (size_t)BH * (groups * sizeof(unsigned long long) + 2 * sizeof(float));
 }
 
 // a number no other call of this process uses (splitmix64 of a counter that starts at the clock), the low 12 bits zero
@@ -1093,7 +1106,7 @@ qaq_status launch_decode(const DecArgs& a, cudaStream_t s) {
     static_assert(sizeof(DecSmem<D, NQ>) + 1024 <= 227 * 1024 / Shape<NQ>::CTAS_PER_SM, "shared memory of the CTAs of an SM");
     static std::atomic<unsigned long long> seen{0};
     QAQ_CUDA_TRY(qaq_allow_smem((const void*)decode_kernel<D, NQ, COUNTED>, smem, seen));
-    QAQ_CUDA_TRY(qaq_launch(decode_kernel<D, NQ, COUNTED>, dim3(a.ncta), dim3(Shape<NQ>::THREADS), smem, s, a));
+    QAQ_CUDA_TRY(qaq_launch(decode_kernel<D, NQ, COUNTED>, dim3(a.ncta, a.groups), dim3(Shape<NQ>::THREADS), smem, s, a));
     if (NQ == 1 && a.ml) {
         int gx = (a.T + 1023) / 1024;     // counted: a.T holds the capacity
         if (gx > 64) gx = 64;
@@ -1102,11 +1115,11 @@ qaq_status launch_decode(const DecArgs& a, cudaStream_t s) {
     return QAQ_OK;
 }
 
-// NQ queries per (b,h) (D elements apart inside a row of q and of out; rows of consecutive (b,h) lie q_stride /
+// nq queries per (b,h), NQ to a CTA (D elements apart inside a row of q and of out; rows of consecutive (b,h) lie q_stride /
 // out_stride elements apart); counted: the token count is taken from device memory
 template <int NQ, bool COUNTED>
 qaq_status decode(const qaq_cache* c, const void* q, long q_stride, float softmax_scale, float* out, long out_stride, float* scores,
-                  long scores_stride, void* ws, cudaStream_t s) {
+                  long scores_stride, void* ws, cudaStream_t s, int nq = NQ) {
     const int D = c->cfg.head_dim, BH = c->BH;
     DecArgs a;
     a.k = c->t[0]; a.v = c->t[1]; a.pool_bytes = c->pool_bytes; a.ocap = c->ocap;
@@ -1115,7 +1128,9 @@ qaq_status decode(const qaq_cache* c, const void* q, long q_stride, float softma
     a.d_count = COUNTED ? qaq_d_count(c) : nullptr;
     a.q = (const __half*)q; a.q_stride = q_stride; a.scale = softmax_scale;
     a.out = out; a.out_stride = out_stride; a.scores = scores; a.scores_stride = scores_stride; a.status = c->d_status;
-    const DecPlan plan = plan_decode<NQ>(BH, (a.T + QAQ_TILE - 1) / QAQ_TILE);
+    a.nq = nq;
+    a.groups = (nq + NQ - 1) / NQ;
+    const DecPlan plan = plan_decode<NQ>(BH, (a.T + QAQ_TILE - 1) / QAQ_TILE, a.groups);
     a.BH = BH;
     a.run = COUNTED ? 0 : plan.run;
     a.ncta = COUNTED ? (BH > Shape<NQ>::SLOTS ? BH : Shape<NQ>::SLOTS) : plan.ncta;   // counted: the largest grid any count needs
@@ -1136,7 +1151,7 @@ qaq_status decode(const qaq_cache* c, const void* q, long q_stride, float softma
 
 extern "C" qaq_status qaq_decode_workspace_bytes(const qaq_cache* c, size_t* host_out) {
     if (!c || !host_out) return QAQ_ERR_INVALID_ARG;
-    *host_out = decode_ws_bytes<1>(c->BH, c->cfg.head_dim);
+    *host_out = decode_ws_bytes<1>(c->BH, c->cfg.head_dim, 1);
     return QAQ_OK;
 }
 
@@ -1151,11 +1166,25 @@ extern "C" qaq_status qaq_decode_attention(const qaq_cache* c, const void* q, fl
 }
 
 // ---------------------------------------------------------------------------------------
-// Several queries per (b,h): passes of four, two or one query.
+// Several queries per (b,h): one, two, or three and four (one launch: at 256 (b,h) of 4096 tokens 110 us against 114 us for
+// three queries as two and one, at 40 of 380 tokens 20 against 23 us).  Five to eight are two groups of up to four, either side
+// by side in one launch or one after the other (a second group of one or two queries as what it is): the first has one
+// start and one end and cuts finer (16 (b,h) of 10175 tokens, five queries: 41 against 59 us; 24 of 2000 tokens: 21 against
+// 30 us), the other does not read every code with four queries' instructions for the sake of one or two (256 (b,h) of 4096
+// tokens: 161 against 262 us) and is needed where half of the chip has fewer places than there are (b,h).
+static bool side_by_side(int BH, int ntiles, int n) {
+    const DecPlan both = plan_decode<4>(BH, ntiles, 2), four = plan_decode<4>(BH, ntiles, 1), few = plan_decode<1>(BH, ntiles, 1);
+    if (both.ncta > Shape<4>::SLOTS / 2) return false;
+    // tiles per warp; a tile takes a warp about 11 us with four queries, half of that with one or two; a launch costs as much again
+    auto tiles = [](int run, int warps) { return (run + warps - 1) / warps; };
+    const int w4 = tiles(four.run, Shape<4>::WARPS);
+    return 2 * tiles(both.run, Shape<4>::WARPS) <= 2 * w4 + (n > 6 ? 2 * w4 : tiles(few.run, Shape<1>::WARPS)) + 2;
+}
+
 extern "C" qaq_status qaq_decode_multi_workspace_bytes(const qaq_cache* c, size_t* host_out) {
     if (!c || !host_out) return QAQ_ERR_INVALID_ARG;
     const int D = c->cfg.head_dim, BH = c->BH;       // the passes of a call reuse the space
-    const size_t b1 = decode_ws_bytes<1>(BH, D), b2 = decode_ws_bytes<2>(BH, D), b4 = decode_ws_bytes<4>(BH, D);
+    const size_t b1 = decode_ws_bytes<1>(BH, D, 1), b2 = decode_ws_bytes<2>(BH, D, 1), b4 = decode_ws_bytes<4>(BH, D, 2);
     *host_out = b1 > b2 ? (b1 > b4 ? b1 : b4) : (b2 > b4 ? b2 : b4);
     return QAQ_OK;
 }
@@ -1170,15 +1199,17 @@ extern "C" qaq_status qaq_decode_attention_multi(const qaq_cache* c, const void*
     const int D = c->cfg.head_dim;
     const long row = (long)n_q * D;
     cudaStream_t s = (cudaStream_t)stream;
+    const int ntiles = (int)((c->tokens + QAQ_TILE - 1) / QAQ_TILE);
     for (int q0 = 0; q0 < n_q;) {
         const int left = n_q - q0;
         const __half* qp = (const __half*)q + (size_t)q0 * D;
         float* op = out + (size_t)q0 * D;
-        qaq_status st;
-        if (left >= 4) { st = decode<4, false>(c, qp, row, softmax_scale, op, row, nullptr, 0, ws, s); q0 += 4; }
-        else if (left >= 2) { st = decode<2, false>(c, qp, row, softmax_scale, op, row, nullptr, 0, ws, s); q0 += 2; }
-        else { st = decode<1, false>(c, qp, row, softmax_scale, op, row, nullptr, 0, ws, s); q0 += 1; }
+        const int n = left > 4 && !side_by_side(c->BH, ntiles, left) ? 4 : left;
+        const qaq_status st = n >= 3 ? decode<4, false>(c, qp, row, softmax_scale, op, row, nullptr, 0, ws, s, n)
+                              : n == 2 ? decode<2, false>(c, qp, row, softmax_scale, op, row, nullptr, 0, ws, s)
+                                       : decode<1, false>(c, qp, row, softmax_scale, op, row, nullptr, 0, ws, s);
         if (st != QAQ_OK) return st;
+        q0 += n;
     }
     return QAQ_OK;
 }
@@ -1213,7 +1244,7 @@ extern "C" qaq_status qaq_decode_attention_static(const qaq_cache* c, const void
     if (c->tokens < 1) return QAQ_ERR_INVALID_ARG;
     const int D = c->cfg.head_dim;
     if (!static_scratch_fits(c->BH, c->tokens, D)) return QAQ_ERR_WORKSPACE;  // shape too large for the built-in scratch
-    if (decode_ws_bytes<1>(c->BH, D) > QAQ_STATIC_SCRATCH_BYTES) return QAQ_ERR_WORKSPACE;   // never: the limit above is the tighter one
+    if (decode_ws_bytes<1>(c->BH, D, 1) > QAQ_STATIC_SCRATCH_BYTES) return QAQ_ERR_WORKSPACE;   // never: the limit above is the tighter one
 
     int dev = -1;
     QAQ_CUDA_TRY(cudaGetDevice(&dev));
