@@ -386,6 +386,20 @@ __device__ __forceinline__ void fixed_unit(float x, float& inv, float& unit) {
     unit = __int_as_float((ex + 1 - 22) << 23);
 }
 
+// What of a tile's outlier list did not fit into the staging buffer (entries from..to, dense wide tiles only), read in
+// place with four loads in flight.
+template <class F>
+__device__ __forceinline__ void unstaged(const uint32_t* list, uint32_t from, uint32_t to, F&& each) {
+#pragma unroll 1
+    for (uint32_t i = from + (threadIdx.x & 31); i < to; i += 128) {
+        uint32_t e[4];
+#pragma unroll
+        for (int k = 0; k < 4; ++k) e[k] = ldg_now1(list + min(i + 32u * k, to - 1));
+#pragma unroll
+        for (int k = 0; k < 4; ++k) if (i + 32u * k < to) each(e[k]);
+    }
+}
+
 // The score row of one (b,h), normalised in place by the whole CTA.
 template <int THREADS>
 __device__ __forceinline__ void normalise_scores(float* row, int T, float M, float L) {
@@ -787,7 +801,9 @@ __global__ void __launch_bounds__(Shape<NQ>::THREADS, Shape<NQ>::CTAS_PER_SM) de
             }
 #pragma unroll 4
             for (uint32_t i = lane + 128; i < sc; i += 32) top = max(top, list[i] & 0x7FFFu);
-            top = sc == oc ? __reduce_max_sync(0xFFFFFFFFu, top) : SMALL_MAX + 1;
+            const uint32_t* all = a.k.outl + (size_t)bh * a.ocap + tk.z;
+            if (sc < oc) unstaged(all, sc, oc, [&](uint32_t v) { top = max(top, v & 0x7FFFu); });
+            top = __reduce_max_sync(0xFFFFFFFFu, top);
             if (top <= SMALL_MAX) {
                 float inv;
                 fixed_unit(qtop * 2.0f * __half2float(__ushort_as_half((unsigned short)top)), inv, kunit);
@@ -806,15 +822,18 @@ __global__ void __launch_bounds__(Shape<NQ>::THREADS, Shape<NQ>::CTAS_PER_SM) de
 #pragma unroll
                     for (int k = 0; k < 4; ++k) e[k] = list[min(i + lane + 32u * k, sc - 1)];
                 }
+                if (sc < oc) unstaged(all, sc, oc, [&](uint32_t v) { add(v, true); });
             } else {
                 kunit = -1.0f;
-#pragma unroll 1
-                for (uint32_t i = lane; i < oc; i += 32) {
+                auto add = [&](uint32_t v) {
                     int tok; float tm[NQ];
-                    term(i < sc ? list[i] : a.k.outl[(size_t)bh * a.ocap + tk.z + i], 1.0f, tok, tm);
+                    term(v, 1.0f, tok, tm);
 #pragma unroll
                     for (int j = 0; j < NQ; ++j) wide_add(&ws.kcorr[j][0][tok], &ws.kcorr[j][1][tok], tm[j]);
-                }
+                };
+#pragma unroll 1
+                for (uint32_t i = lane; i < sc; i += 32) add(list[i]);
+                if (sc < oc) unstaged(all, sc, oc, add);
             }
         }
         __syncwarp();
@@ -951,7 +970,9 @@ __global__ void __launch_bounds__(Shape<NQ>::THREADS, Shape<NQ>::CTAS_PER_SM) de
             }
 #pragma unroll 4
             for (uint32_t i = lane + 128; i < sc; i += 32) top = max(top, list[i] & 0x7FFFu);
-            top = sc == oc ? __reduce_max_sync(0xFFFFFFFFu, top) : SMALL_MAX + 1;
+            const uint32_t* all = a.v.outl + (size_t)bh * a.ocap + tv.z;
+            if (sc < oc) unstaged(all, sc, oc, [&](uint32_t v) { top = max(top, v & 0x7FFFu); });
+            top = __reduce_max_sync(0xFFFFFFFFu, top);
             if (top <= SMALL_MAX) {
                 float inv[NQ], unit[NQ];
                 __syncwarp();
@@ -976,6 +997,7 @@ __global__ void __launch_bounds__(Shape<NQ>::THREADS, Shape<NQ>::CTAS_PER_SM) de
 #pragma unroll
                     for (int k = 0; k < 4; ++k) e[k] = list[min(i + lane + 32u * k, sc - 1)];
                 }
+                if (sc < oc) unstaged(all, sc, oc, [&](uint32_t v) { add(v, true); });
                 __syncwarp();
 #pragma unroll
                 for (int j = 0; j < NQ; ++j)
@@ -990,12 +1012,13 @@ __global__ void __launch_bounds__(Shape<NQ>::THREADS, Shape<NQ>::CTAS_PER_SM) de
                     __syncwarp();
                     clear_vcorr(2);
                     __syncwarp();
-#pragma unroll 1
-                    for (uint32_t i = lane; i < oc; i += 32) {
-                        const uint32_t v = i < sc ? list[i] : a.v.outl[(size_t)bh * a.ocap + tv.z + i];
+                    auto add = [&](uint32_t v) {
                         const int ch = (v >> 16) & (D - 1);
                         wide_add(&ws.vcorr[0][ch], &ws.vcorr[1][ch], term(v, j));
-                    }
+                    };
+#pragma unroll 1
+                    for (uint32_t i = lane; i < sc; i += 32) add(list[i]);
+                    if (sc < oc) unstaged(all, sc, oc, add);
                     __syncwarp();
 #pragma unroll
                     for (int k = 0; k < CPL; ++k) {
