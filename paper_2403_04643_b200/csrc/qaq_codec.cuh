@@ -219,14 +219,8 @@ constexpr uint32_t NIB = 0x0F0F0F0Fu;
 // (a & m) | (b & ~m)
 __device__ __forceinline__ uint32_t bitsel(uint32_t a, uint32_t b, uint32_t m) { return (a & m) | (b & ~m); }
 
-// The w-bit words of a unit (codes one per byte in creg; bits shift .. shift+3 of them, of which w are in use).
-__device__ __forceinline__ void store_part(uint8_t* dst, int w, int shift, const uint32_t (&creg)[8]) {
-    uint32_t v[4];
-#pragma unroll
-    for (int u = 0; u < 4; ++u) {
-        const uint32_t a = shift ? creg[2 * u] >> 4 : creg[2 * u], b = shift ? creg[2 * u + 1] : creg[2 * u + 1] << 4;
-        v[u] = bitsel(a, b, NIB);
-    }
+// The w-bit words of a unit, from its nibble words (bits beyond the w lowest of a nibble are zero).
+__device__ __forceinline__ void store_nibbles(uint8_t* dst, int w, const uint32_t (&v)[4]) {
     if (w == 4) {
         *reinterpret_cast<uint4*>(dst) = make_uint4(v[0], v[1], v[2], v[3]);
     } else if (w == 3) {
@@ -239,6 +233,19 @@ __device__ __forceinline__ void store_part(uint8_t* dst, int w, int shift, const
     } else {
         *reinterpret_cast<uint32_t*>(dst) = v[0] | (v[1] << 1) | (v[2] << 2) | (v[3] << 3);
     }
+}
+// The nibble words of codes one per byte: bits shift .. shift+3 of them.
+__device__ __forceinline__ void nibbles_of(const uint32_t (&creg)[8], int shift, uint32_t (&v)[4]) {
+#pragma unroll
+    for (int u = 0; u < 4; ++u) {
+        const uint32_t a = shift ? creg[2 * u] >> 4 : creg[2 * u], b = shift ? creg[2 * u + 1] : creg[2 * u + 1] << 4;
+        v[u] = bitsel(a, b, NIB);
+    }
+}
+__device__ __forceinline__ void store_part(uint8_t* dst, int w, int shift, const uint32_t (&creg)[8]) {
+    uint32_t v[4];
+    nibbles_of(creg, shift, v);
+    store_nibbles(dst, w, v);
 }
 // The nibble words of a unit of w-bit words.  Bits of a nibble beyond the w lowest are undefined.
 template <int W>
