@@ -351,4 +351,128 @@ __device__ __forceinline__ void read_token(const uint8_t* tile, const Section& s
     }
 }
 
+// ------------------------------------------------------------------------------------------ a tile by two warps
+// What the kernels that give a tile 64 threads, one per token, find out about it.  Counts by width are kept a byte each, widths
+// 1..4 in one word and 5..8 in the other, and sums over widths are taken in the bytes (they stay below 256).
+constexpr uint32_t ONES = 0x01010101u;
+__device__ __forceinline__ uint32_t byte_of(uint32_t lo, uint32_t hi, int w) { return prmt(lo, hi, (uint32_t)(w - 1)) & 0xFFu; }
+
+// The lanes of this warp whose token has the same width (0: no token), and for the other warp how many have which.
+__device__ __forceinline__ uint32_t count_half(int b, int lane, uint32_t (&count)[2]) {
+    const uint32_t b0 = __ballot_sync(0xFFFFFFFFu, (b - 1) & 1), b1 = __ballot_sync(0xFFFFFFFFu, (b - 1) & 2), b2 = __ballot_sync(0xFFFFFFFFu, (b - 1) & 4);
+    const uint32_t there = __ballot_sync(0xFFFFFFFFu, b != 0);
+    auto tokens_of = [&](int k) { return (k & 1 ? b0 : ~b0) & (k & 2 ? b1 : ~b1) & (k & 4 ? b2 : ~b2) & there; };
+    if (lane < 8) reinterpret_cast<uint8_t*>(count)[lane] = (uint8_t)__popc(tokens_of(lane));
+    return tokens_of(b - 1);
+}
+
+// Rows of a tile by width: how many, and the first one.
+struct TileRows { uint32_t nlo, nhi, slo, shi; };
+// from the stored counts of rows
+__device__ __forceinline__ TileRows rows_of_header(uint32_t nlo, uint32_t nhi) {
+    const uint32_t ulo = nlo * ONES, uhi = nhi * ONES + (ulo >> 24) * ONES, all = (uhi >> 24) * ONES;      // rows of a width or less
+    return {nlo, nhi, all - ulo, all - uhi};
+}
+// from the tokens of the halves of the tile; slot: this thread's token's place in the order
+template <bool IS_V>
+__device__ __forceinline__ TileRows rows_of_counts(const uint32_t (&count)[2][2], int b, uint32_t alike, int warp, int lane, int& slot) {
+    const uint32_t clo = count[0][0] + count[1][0], chi = count[0][1] + count[1][1];
+    const uint32_t ulo = clo * ONES, uhi = chi * ONES + (ulo >> 24) * ONES, n = uhi >> 24;
+    slot = (int)(n - byte_of(ulo, uhi, b) + (warp ? byte_of(count[0][0], count[0][1], b) : 0u)) + __popc(alike & ((1u << lane) - 1u));
+    if (!IS_V) return {clo, chi, n * ONES - ulo, n * ONES - uhi};
+    // groups of four slots; a section has those whose first slot is in it
+    TileRows r;
+    r.slo = (((n + 3) * ONES - ulo) >> 2) & 0x3F3F3F3Fu;
+    r.shi = (((n + 3) * ONES - uhi) >> 2) & 0x3F3F3F3Fu;
+    r.nlo = ((r.slo << 8) | ((n + 3) >> 2)) - r.slo;
+    r.nhi = __funnelshift_l(r.slo, r.shi, 8) - r.shi;
+    return r;
+}
+// width of a row: one more than the widths that begin behind it
+__device__ __forceinline__ int width_of_row(const TileRows& r, int row) {
+    const uint32_t y = (uint32_t)row * ONES | 0x80808080u;
+    return 9 - __popc((y - r.slo) & 0x80808080u) - __popc((y - r.shi) & 0x80808080u);
+}
+// Offsets of the parts as in make_sections, in words per unit: dot products of the rows of every width.
+template <int D, bool IS_V>
+__device__ __forceinline__ uint32_t at_words(const TileRows& r, uint32_t wlo, uint32_t whi) {
+    return (uint32_t)QAQ_TILE_HDR + (uint32_t)(4 * UNITS<D, IS_V>) * __dp4a(r.nlo, wlo, __dp4a(r.nhi, whi, 0u));
+}
+template <int D, bool IS_V> __device__ __forceinline__ uint32_t at_h8(const TileRows& r) { return at_words<D, IS_V>(r, 0x04000000u, 0x04040404u); }
+template <int D, bool IS_V> __device__ __forceinline__ uint32_t at_z2(const TileRows& r) { return at_words<D, IS_V>(r, 0x04000000u, 0x08040404u); }
+template <int D, bool IS_V> __device__ __forceinline__ uint32_t at_z13(const TileRows& r) { return at_words<D, IS_V>(r, 0x04000200u, 0x08040604u); }
+template <int D, bool IS_V> __device__ __forceinline__ uint32_t tile_total(const TileRows& r) { return at_words<D, IS_V>(r, 0x04030201u, 0x08070605u); }
+template <int D, bool IS_V>
+__device__ __forceinline__ uint4 header_of(const TileRows& r) {
+    return make_uint4(r.nlo, r.nhi, at_h8<D, IS_V>(r) | (at_z2<D, IS_V>(r) << 16), at_z13<D, IS_V>(r) | (tile_total<D, IS_V>(r) << 16));
+}
+// Where a row of width w lies: byte offsets of its main and high part, and for values how far apart its units are (in units).
+struct RowPlace { uint32_t main, high, mm, mh; };
+template <int D, bool IS_V>
+__device__ __forceinline__ RowPlace place_row(const TileRows& r, int row, int w) {
+    constexpr int P = D / 32;
+    const uint32_t m3 = at_words<D, IS_V>(r, 0x04000200u, 0x08070604u), m2 = at_words<D, IS_V>(r, 0x04000000u, 0x08040604u);
+    const uint32_t m1 = at_words<D, IS_V>(r, 0x04030200u, 0x08070605u), h5 = at_words<D, IS_V>(r, 0x04030200u, 0x08070604u);
+    const int wm = min(w, 4), wh = max(w - 4, 0), start = (int)byte_of(r.slo, r.shi, w), n = (int)byte_of(r.nlo, r.nhi, w);
+    const int rm = w >= 4 ? row : row - start, rh = row - start;
+    RowPlace o;
+    o.main = w >= 4 ? (uint32_t)QAQ_TILE_HDR : w == 3 ? m3 : w == 2 ? m2 : m1;
+    o.high = w == 8 ? at_h8<D, IS_V>(r) : w == 7 ? at_z13<D, IS_V>(r) : w == 6 ? at_z2<D, IS_V>(r) : h5;
+    o.mm = o.mh = 0;
+    if (!IS_V) {
+        o.main += rm * P * 4 * wm;
+        o.high += rh * P * 4 * wh;
+    } else {                           // unit e of the row lies at e * m units from here; main parts of 4 bits and more are one list
+        const int rows = w >= 4 ? (int)((r.slo >> 16) & 0xFFu) : n;
+        o.mm = min(4, rows - (rm & ~3)); o.mh = min(4, n - (rh & ~3));
+        o.main += ((rm & ~3) * (D / 8) + (rm & 3)) * 4 * wm;
+        o.high += ((rh & ~3) * (D / 8) + (rh & 3)) * 4 * wh;
+    }
+    return o;
+}
+// The largest of the first nv of W scores, `stride` apart.  Every row of the window is read (the ring is allocated in full),
+// rows the token has no score in are left out of the maximum: the loads then depend on nothing and go out together.
+// By whole warps.
+__device__ __forceinline__ float window_max(const float* r, int W, long stride, int nv) {
+    float m = __int_as_float(0xff800000);
+    int i = 0;
+#pragma unroll 1
+    for (; i + 16 <= W; i += 16, r += 16 * stride) {
+        float v[16];
+#pragma unroll
+        for (int u = 0; u < 16; ++u) v[u] = r[u * stride];
+        if (__all_sync(0xFFFFFFFFu, i + 16 <= nv)) {
+#pragma unroll
+            for (int u = 0; u < 16; ++u) m = fmaxf(m, v[u]);
+        } else {
+#pragma unroll
+            for (int u = 0; u < 16; ++u) if (i + u < nv) m = fmaxf(m, v[u]);
+        }
+    }
+#pragma unroll 1
+    for (; i < W; ++i, r += stride) {
+        const float v = *r;
+        if (i < nv) m = fmaxf(m, v);
+    }
+    return m;
+}
+// 4 x 4 bytes of every word, transposed over the four lanes that are S and 2S apart: lane i of them gets byte i of all four
+template <int S>
+__device__ __forceinline__ void transpose4(uint32_t (&v)[4], int i) {
+#pragma unroll
+    for (int step = 0; step < 2; ++step) {
+        const bool up = step ? (i & 1) : (i >> 1);
+        // the halves of a word (step 0) or its odd and even bytes (step 1): one stays, the other goes
+        const uint32_t away = step ? (up ? 0x6420u : 0x7531u) : (up ? 0x5410u : 0x7632u);
+        const uint32_t join0 = step ? (up ? 0x3514u : 0x5240u) : (up ? 0x3254u : 0x5410u);
+        const uint32_t join1 = step ? (up ? 0x3716u : 0x7260u) : (up ? 0x3276u : 0x7610u);
+#pragma unroll
+        for (int k = 0; k < 4; k += 2) {
+            const uint32_t o = __shfl_xor_sync(0xFFFFFFFFu, prmt(v[k], v[k + 1], away), step ? S : 2 * S);
+            v[k] = prmt(v[k], o, join0);
+            v[k + 1] = prmt(v[k + 1], o, join1);
+        }
+    }
+}
+
 }  // namespace qaqc

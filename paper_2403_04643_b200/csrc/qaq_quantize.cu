@@ -651,25 +651,6 @@ __device__ __forceinline__ uint32_t prefix(uint32_t x, int lane, uint32_t& sum) 
     sum = __shfl_sync(0xFFFFFFFFu, inc, 31);
     return inc - x;
 }
-// 4 x 4 bytes of every word, transposed over the four lanes that are S and 2S apart: lane i of them gets byte i of all four
-template <int S>
-__device__ __forceinline__ void transpose4(uint32_t (&v)[4], int i) {
-#pragma unroll
-    for (int step = 0; step < 2; ++step) {
-        const bool up = step ? (i & 1) : (i >> 1);
-        // the halves of a word (step 0) or its odd and even bytes (step 1): one stays, the other goes
-        const uint32_t away = step ? (up ? 0x6420u : 0x7531u) : (up ? 0x5410u : 0x7632u);
-        const uint32_t join0 = step ? (up ? 0x3514u : 0x5240u) : (up ? 0x3254u : 0x5410u);
-        const uint32_t join1 = step ? (up ? 0x3716u : 0x7260u) : (up ? 0x3276u : 0x7610u);
-#pragma unroll
-        for (int k = 0; k < 4; k += 2) {
-            const uint32_t o = __shfl_xor_sync(0xFFFFFFFFu, qaqc::prmt(v[k], v[k + 1], away), step ? S : 2 * S);
-            v[k] = qaqc::prmt(v[k], o, join0);
-            v[k + 1] = qaqc::prmt(v[k + 1], o, join1);
-        }
-    }
-}
-
 // One tile of one tensor, by two warps: half of its tokens each until the widths are known, half of the slots each from there.
 template <int D, bool IS_V>
 __device__ __forceinline__ void quantize_tile(const QuantArgs& a, TileScratch<D>& sm, uint32_t* list, const uint32_t cap) {
@@ -701,28 +682,7 @@ __device__ __forceinline__ void quantize_tile(const QuantArgs& a, TileScratch<D>
         b = (IS_V ? a.bitsV : a.bitsK)[(size_t)bh * a.n_new + tn0 + tid];
     } else if (IS_V) {
         nv = min((int)a.nvalid[(size_t)bh * a.n_new + tn0 + tid], a.W);
-        // every row of the window is read (the ring is allocated in full), rows the token has no score in are
-        // left out of the maximum: the loads then depend on nothing and go out together
-        const float* r = a.ring + (size_t)bh * a.W * a.n_new + tn0 + tid;
-        int i = 0;
-#pragma unroll 1
-        for (; i + 16 <= a.W; i += 16, r += (size_t)16 * a.n_new) {
-            float v[16];
-#pragma unroll
-            for (int u = 0; u < 16; ++u) v[u] = r[(size_t)u * a.n_new];
-            if (__all_sync(0xFFFFFFFFu, i + 16 <= nv)) {
-#pragma unroll
-                for (int u = 0; u < 16; ++u) shat = fmaxf(shat, v[u]);
-            } else {
-#pragma unroll
-                for (int u = 0; u < 16; ++u) if (i + u < nv) shat = fmaxf(shat, v[u]);
-            }
-        }
-#pragma unroll 1
-        for (; i < a.W; ++i, r += a.n_new) {
-            const float v = *r;
-            if (i < nv) shat = fmaxf(shat, v);
-        }
+        shat = qaqc::window_max(a.ring + (size_t)bh * a.W * a.n_new + tn0 + tid, a.W, a.n_new, nv);
     }
     asm volatile("cp.async.wait_all;" ::: "memory");
     __syncwarp();
@@ -779,64 +739,25 @@ __device__ __forceinline__ void quantize_tile(const QuantArgs& a, TileScratch<D>
         else if (!IS_V) b = ladder(r, a.cK, a.bmin, a.bmax);
         else b = nv == 0 ? a.bmax : ladder(__fmul_rn(r, shat), a.cV, a.bmin, a.bmax);
     }
-    // The tokens of a width by the three bits of width - 1; how many there are, a byte per width, for the other warp.
-    const uint32_t b0 = __ballot_sync(0xFFFFFFFFu, (b - 1) & 1), b1 = __ballot_sync(0xFFFFFFFFu, (b - 1) & 2), b2 = __ballot_sync(0xFFFFFFFFu, (b - 1) & 4);
-    auto tokens_of = [&](int k) { return (k & 1 ? b0 : ~b0) & (k & 2 ? b1 : ~b1) & (k & 4 ? b2 : ~b2); };
-    const uint32_t alike = tokens_of(b - 1);
-    if (lane < 8) reinterpret_cast<uint8_t*>(sm.count[warp])[lane] = (uint8_t)__popc(tokens_of(lane));
+    const uint32_t alike = qaqc::count_half(b, lane, sm.count[warp]);
     if (lane == 0) sm.nout[warp] = nout;
     __syncthreads();
-    // ---- order and sections, by both warps alike: the sums over the widths are taken in the bytes of a pair of words
-    //      (upto: tokens of a width or less, which is 64 minus the width's first slot)
-    const uint32_t ones = 0x01010101u;
-    const uint32_t h0lo = sm.count[0][0], h0hi = sm.count[0][1], clo = h0lo + sm.count[1][0], chi = h0hi + sm.count[1][1];
-    const uint32_t upto_lo = clo * ones, upto_hi = chi * ones + (upto_lo >> 24) * ones;
-    const int slot = QAQ_TILE - (int)(qaqc::prmt(upto_lo, upto_hi, (uint32_t)(b - 1)) & 0xFFu) +
-                     (warp ? (int)(qaqc::prmt(h0lo, h0hi, (uint32_t)(b - 1)) & 0xFFu) : 0) + __popc(alike & ((1u << lane) - 1u));
-    // rows of every width, the rows of a width or less, and this token's row: its slot, or the group of four slots that it
-    // is in, which has the width of its first (the only one with upto[w - 1] < 64 - first slot <= upto[w])
-    uint32_t nlo = clo, nhi = chi, rlo = upto_lo, rhi = upto_hi;
-    int row = slot, row_w = b;
-    constexpr int ROWS = IS_V ? QAQ_TILE / 4 : QAQ_TILE;
-    if (IS_V) {
-        rlo = (upto_lo >> 2) & 0x3F3F3F3Fu; rhi = (upto_hi >> 2) & 0x3F3F3F3Fu;
-        nlo = rlo - (rlo << 8); nhi = rhi - __funnelshift_l(rlo, rhi, 8);
-        row = slot >> 2;
-        const uint32_t y = (uint32_t)(QAQ_TILE - 4 * row) * ones;
-        row_w = 9 - __popc(((upto_lo | 0x80808080u) - y) & 0x80808080u) - __popc(((upto_hi | 0x80808080u) - y) & 0x80808080u);
-    }
-    // offsets of the parts as in make_sections, in words per unit: a dot product with the rows of every width
-    constexpr uint32_t WORD = 4 * qaqc::UNITS<D, IS_V>;
-    auto at_words = [&](uint32_t wlo, uint32_t whi) { return (uint32_t)qaqc::QAQ_TILE_HDR + WORD * __dp4a(nlo, wlo, __dp4a(nhi, whi, 0u)); };
-    const uint32_t h8 = at_words(0x04000000u, 0x04040404u), z2 = at_words(0x04000000u, 0x08040404u), z13 = at_words(0x04000200u, 0x08040604u);
-    const uint32_t total = at_words(0x04030201u, 0x08070605u);
+    // ---- order and sections, by both warps alike; space from the pools
+    int slot;
+    const qaqc::TileRows rows = qaqc::rows_of_counts<IS_V>(sm.count, b, alike, warp, lane, slot);
+    const uint32_t total = qaqc::tile_total<D, IS_V>(rows);
     const uint32_t nout0 = sm.nout[0], nall = nout0 + sm.nout[1];
     uint32_t base = 0, taken = 0;
     if (tid < 2) base = pool_take(pool, lane ? nall : total, lane ? 3u : 15u, true, true, pool_now > (lane ? a.ocap : a.pool_bytes), taken);
     {
-        const uint32_t m3 = at_words(0x04000200u, 0x08070604u), m2 = at_words(0x04000000u, 0x08040604u), m1 = at_words(0x04030200u, 0x08070605u);
-        const uint32_t h5 = at_words(0x04030200u, 0x08070604u);
-        const int wm = min(row_w, 4), wh = max(row_w - 4, 0);
-        const int start = ROWS - (int)(qaqc::prmt(rlo, rhi, (uint32_t)(row_w - 1)) & 0xFFu), n = (int)(qaqc::prmt(nlo, nhi, (uint32_t)(row_w - 1)) & 0xFFu);
-        uint32_t main = row_w >= 4 ? (uint32_t)qaqc::QAQ_TILE_HDR : row_w == 3 ? m3 : row_w == 2 ? m2 : m1;
-        uint32_t high = row_w == 8 ? h8 : row_w == 7 ? z13 : row_w == 6 ? z2 : h5;
-        const int rm = row_w >= 4 ? row : row - start, rh = row - start;
-        uint32_t mm = 0, mh = 0;
-        if (!IS_V) {
-            main += rm * P * 4 * wm;
-            high += rh * P * 4 * wh;
-        } else {                       // unit e of the row lies at e * m units from here
-            const int mn_rows = row_w >= 4 ? ROWS - (int)((rlo >> 16) & 0xFFu) : n;          // main parts of 4 bits and more are one list
-            mm = min(4, mn_rows - (rm & ~3)); mh = min(4, n - (rh & ~3));
-            main += ((rm & ~3) * (D / 8) + (rm & 3)) * 4 * wm;
-            high += ((rh & ~3) * (D / 8) + (rh & 3)) * 4 * wh;
-        }
+        const int row = IS_V ? slot >> 2 : slot, row_w = IS_V ? qaqc::width_of_row(rows, row) : b;
+        const qaqc::RowPlace pl = qaqc::place_row<D, IS_V>(rows, row, row_w);
         // the reciprocal of the step without its power of two (the range of binary16 numbers is nowhere near the ends of
         // binary32: both are the same number but for the exponent)
         const float len = __fsub_rn(mx, mn), inv = len > 0.f ? __fdiv_rn(1.0f, len) : 0.f;
         const bool endless = len > 0.f && inv == 0.f;         // a range that is not finite
-        sm.slot[slot] = make_uint4(__float_as_uint(mn), __float_as_uint(inv), main | (high << 16),
-                                   (uint32_t)tid | ((uint32_t)b << 8) | ((uint32_t)row_w << 16) | (mm << 20) | (mh << 24) | (endless ? 0x80000000u : 0u));
+        sm.slot[slot] = make_uint4(__float_as_uint(mn), __float_as_uint(inv), pl.main | (pl.high << 16),
+                                   (uint32_t)tid | ((uint32_t)b << 8) | ((uint32_t)row_w << 16) | (pl.mm << 20) | (pl.mh << 24) | (endless ? 0x80000000u : 0u));
     }
     // ---- a pool without room: the space is given back, nothing about the tile is published; the device status reports
     //      the lost tokens
@@ -860,7 +781,7 @@ __device__ __forceinline__ void quantize_tile(const QuantArgs& a, TileScratch<D>
     if (tid == 0) {
         if (stored < nall) atomicMax(a.status, (int)QAQ_ERR_CAPACITY);
         ts.tile[(size_t)bh * a.ntiles + tile] = make_uint4(off, total, obase, stored);
-        *reinterpret_cast<uint4*>(dst) = make_uint4(nlo, nhi, h8 | (z2 << 16), z13 | (total << 16));
+        *reinterpret_cast<uint4*>(dst) = qaqc::header_of<D, IS_V>(rows);
     }
     {
         const size_t mt = (size_t)bh * a.tmax_pad + (size_t)tile * QAQ_TILE + tid;
@@ -936,12 +857,12 @@ __device__ __forceinline__ void quantize_tile(const QuantArgs& a, TileScratch<D>
 #pragma unroll
             for (int u = 0; u < 4; ++u) lo[u] = qaqc::prmt(mad(c[4 * u + 2], a.k16, c[4 * u]), mad(c[4 * u + 3], a.k16, c[4 * u + 1]), 0x6420u);
         }
-        if (IS_V) transpose4<P>(lo, g & 3);
+        if (IS_V) qaqc::transpose4<P>(lo, g & 3);
         const int e = IS_V ? 4 * p + (g & 3) : p;
         const int wm = min(w, 4);
         qaqc::store_nibbles(dst + (q.z & 0xFFFFu) + (IS_V ? e * (int)((q.w >> 20) & 7u) : e) * 4 * wm, wm, lo);
         if (wide) {
-            if (IS_V) transpose4<P>(hi, g & 3);
+            if (IS_V) qaqc::transpose4<P>(hi, g & 3);
             if (w > 4) qaqc::store_nibbles(dst + (q.z >> 16) + (IS_V ? e * (int)((q.w >> 24) & 7u) : e) * 4 * (w - 4), w - 4, hi);
         }
     }

@@ -11,16 +11,19 @@
 // The new widths come from the caller or from the rules of Section 4.1 applied to the stored
 // range (max - min of the token's metadata) with the current score window and policy scalars.
 //
-// One CTA = one tile (QAQ_TILE tokens) of one (b,h) and tensor; head_dim/32 lanes own a
-// token, each lane the codes of 32 consecutive channels, one byte per code in 8 registers.
-// A CTA whose widths stay as they are leaves after reading them.  Otherwise the tile's bytes come to
-// shared memory with wide loads, the codes from there to registers, and the image of the new tile takes
-// the same place, so a tile that does not grow is rewritten in place.  (With both tensors in one CTA and
-// the codes read byte by byte from global memory, lowering a 4096-token layer at batch 4 took 135 us and raising it
-// 201; now see the launch below.)  A closed tile that grows takes a new place at the end of its pool (the
+// Two warps = one tile (QAQ_TILE tokens) of one (b,h) and tensor.  A thread finds the new width of one token; a CTA whose
+// widths stay as they are leaves.  Otherwise the tile's bytes come to shared memory, and the tokens are gone through in
+// their new order, head_dim/32 lanes to a token: words of the old tile, low bits dropped in the nibbles (or codes from
+// the unquantized row), words of the new tile straight to where they belong, which is where the tile was, unless it grows.
+// A closed tile that grows takes a new place at the end of its pool (the
 // old bytes stay unused); the open (last, partly filled) tile is then handled in a launch of its own
 // after the closed ones and is kept - or made again - the last thing in its pool, so that later
 // appends continue right behind it.  Lowered widths never make a tile grow.
+//
+// What bounds it: instructions, and where few tiles change the latency of the metadata and of the window.  With a thread per
+// 32 channels from the start, every tile of changed widths decoded to codes, encoded to an image and copied out, lowering
+// a 4096-token layer at batch 4 took 120 us and raising it again 170; as it is now 61 and 116.  With a step's few changes
+// (2048 tokens, batch 4) 29.6 us became 16.8.
 #include "qaq_codec.cuh"
 #include "qaq_internal.cuh"
 
@@ -63,221 +66,243 @@ __device__ __forceinline__ void fresh_codes(const __half* row, float lo, float h
     qaqc::codes32(v, mn, mx, B, creg);
 }
 
-// UP: widths may be raised (the unquantized copy is there); blockIdx.z: keys or values.
-template <int D, bool UP>
-__global__ void __launch_bounds__(2 * D) requant_kernel(const RequantArgs a) {
-    constexpr int P = D / 32;
-    constexpr int NT = 2 * D;
-    constexpr int IMG = qaqc::tile_bytes_max(D);
-    qaq_dependency();
-    const int tile = a.first_tile + blockIdx.x, bh = blockIdx.y, x = blockIdx.z;
-    const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
-    const int slot = tid / P, p = tid % P;
-    const int tok = tile * QAQ_TILE + slot;
+// 32 codes, one per nibble pair of lo and hi (bits 0..3 and 4..7 of the codes, in nibble words), without their low d bits
+__device__ __forceinline__ void drop_bits(uint32_t (&lo)[4], uint32_t (&hi)[4], int d) {
+    if (d >= 4) {
+#pragma unroll
+        for (int u = 0; u < 4; ++u) { lo[u] = hi[u]; hi[u] = 0; }
+        d -= 4;
+    }
+    const uint32_t keep = 0x11111111u * (0xFu >> d);
+#pragma unroll
+    for (int u = 0; u < 4; ++u) {
+        lo[u] = ((lo[u] >> d) & keep) | ((hi[u] << (4 - d)) & ~keep);
+        hi[u] = (hi[u] >> d) & keep;
+    }
+}
+// The nibble words of one part (w bits, 1..4) of a lane's 32 channels of one token.  Keys: the unit at `at`; values: byte i of
+// units 4p .. 4p+3, which lie m units apart from `at` on.
+template <int W, bool IS_V>
+__device__ __forceinline__ void take_words(const uint8_t* at, uint32_t m, int i, uint32_t (&v)[4]) {
+    uint32_t x[W];
+    if (!IS_V) {
+        qaqc::load_words<W>(at, x);
+    } else {
+        uint32_t u[4][W];
+#pragma unroll
+        for (int b = 0; b < 4; ++b) qaqc::load_words<W>(at + b * m * 4 * W, u[b]);
+        const uint32_t sel = 0x0040u + 0x0011u * (uint32_t)i;          // byte i of both operands
+#pragma unroll
+        for (int c = 0; c < W; ++c) x[c] = qaqc::prmt(qaqc::prmt(u[0][c], u[1][c], sel), qaqc::prmt(u[2][c], u[3][c], sel), 0x5410u);
+    }
+    qaqc::nibble_words<W>(x, v);
+    constexpr uint32_t mask = 0x11111111u * ((1u << W) - 1u);
+#pragma unroll
+    for (int k = 0; k < 4; ++k) v[k] &= mask;
+}
+template <bool IS_V>
+__device__ __forceinline__ void take_part(const uint8_t* at, int w, uint32_t m, int i, uint32_t (&v)[4]) {
+    if (w == 4) take_words<4, IS_V>(at, m, i, v);
+    else if (w == 3) take_words<3, IS_V>(at, m, i, v);
+    else if (w == 2) take_words<2, IS_V>(at, m, i, v);
+    else take_words<1, IS_V>(at, m, i, v);
+}
+
+// What the CTA keeps of its tile.
+template <int D>
+struct RequantScratch {
+    alignas(16) uint8_t old[qaqc::tile_bytes_max(D)];
+    // by new slot: byte offsets of the row's parts before | and after << 16 (main, high); token, widths before and after, row
+    // widths before and after; for values the distances of the units and the old slot's place in its group
+    alignas(16) uint4 slot[QAQ_TILE];
+    uint32_t range[QAQ_TILE];
+    alignas(8) uint32_t count[2][2];
+    uint32_t off;
+    int skip;
+};
+
+// One tile of one tensor.  UP: widths may be raised (the unquantized copy is there).
+template <int D, bool UP, bool IS_V>
+__device__ __forceinline__ void requantize_tile(const RequantArgs& a, RequantScratch<D>& sm) {
+    constexpr int P = D / 32, TPI = 32 / P, IT = QAQ_TILE / 2 / TPI;      // lanes per token, tokens of a warp at a time, rounds
+    const int tile = a.first_tile + blockIdx.x, bh = blockIdx.y;
+    const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31, g = lane / P, p = lane % P;
+    const int tok = tile * QAQ_TILE + tid;
     const bool valid = tok < a.T;
-    const bool given = a.bitsK != nullptr;
-    const TensorStore& ts = x ? a.v : a.k;
+    const TensorStore& ts = IS_V ? a.v : a.k;
     const size_t ti = (size_t)bh * a.ntiles + tile;
 
-    __shared__ float s_part[P][QAQ_TILE];
-    __shared__ uint8_t s_bn[QAQ_TILE];                       // widths afterwards
-    __shared__ qaqc::Section s_otab[9], s_tab[9];            // sections before and after
-    __shared__ unsigned short s_place[QAQ_TILE];             // new slot | width of its row << 8
-    __shared__ uint8_t s_sorted[QAQ_TILE], s_orow[QAQ_TILE / 4];   // new width of every slot; stored width of the rows of values
-    __shared__ uint32_t s_head[4];
-    __shared__ uint32_t s_tot, s_off;                        // new bytes of the tile, where they go in the pool
-    __shared__ int s_skip, s_holes;                          // no room; some slots of the last group of values are empty
-    __shared__ __align__(16) uint8_t s_img[IMG];             // the tile as it was, then as it will be
-
-    // ---- current width and range of this thread's token
+    // ---- current width and range of this thread's token, its new width: the rule's (or the caller's) width; without the
+    //      unquantized copy only where it is lower
     const size_t mt = (size_t)bh * a.tmax_pad + tok;
     const uint4 tw = ts.tile[ti];
-    int Bo = 0, oslot = 0;
-    float rng = 0.f, mn = 0.f, mx = 0.f;
+    const uint32_t pool_end = ts.pool_end[bh];
+    int Bo = 0, oslot = 0, Bn = 0;
+    uint32_t range = 0;
     if (valid) {
-        const uint32_t bs = ts.bs[mt], mm = ts.mnmx[mt];
+        const uint32_t bs = ts.bs[mt];
+        range = ts.mnmx[mt];
         Bo = min((int)(bs & 0xFFu), 8);
         oslot = (int)((bs >> 8) & (QAQ_TILE - 1));
-        mn = __half2float(__ushort_as_half((unsigned short)(mm & 0xFFFF)));
-        mx = __half2float(__ushort_as_half((unsigned short)(mm >> 16)));
-        rng = __fsub_rn(mx, mn);
     }
-    // ---- attention window of the tile's tokens (value rule); P threads share a token's rows.  All rows are read (the
-    //      ring is allocated in full), rows a token has no score in are left out of the maximum: no load waits for another.
-    const bool window = x && !given;
-    int nv = 0;
-    if (window) {
-        const int g = tid / QAQ_TILE, tk = tid % QAQ_TILE, t2 = tile * QAQ_TILE + tk;
-        float m = __int_as_float(0xff800000);
-        if (t2 < a.T) {
-            const int nvt = a.nvalid[(size_t)bh * a.ncols + t2];
-            const float* r = a.ring + (size_t)bh * a.W * a.ncols + t2;
-            int i = g;
-            for (; i + 7 * P < a.W; i += 8 * P) {
-                float v[8];
-#pragma unroll
-                for (int u = 0; u < 8; ++u) v[u] = r[(size_t)(i + u * P) * a.ncols];
-#pragma unroll
-                for (int u = 0; u < 8; ++u) if (i + u * P < nvt) m = fmaxf(m, v[u]);
-            }
-            for (; i < a.W; i += P) {
-                const float v = r[(size_t)i * a.ncols];
-                if (i < nvt) m = fmaxf(m, v);
-            }
-        }
-        if (valid) nv = a.nvalid[(size_t)bh * a.ncols + tok];
-        s_part[g][tk] = m;
-        __syncthreads();
-    }
-    // ---- new width: the rule's (or the caller's) width; without the unquantized copy only where it is lower
-    int Bn = 0;
-    if (valid) {
-        int B;
-        if (given) {
-            B = (x ? a.bitsV : a.bitsK)[(size_t)bh * a.ncols + tok];
+    const float rng = __fsub_rn(__half2float(__ushort_as_half((unsigned short)(range >> 16))), __half2float(__ushort_as_half((unsigned short)(range & 0xFFFF))));
+    {
+        int B = 0;
+        if (a.bitsK) {
+            if (valid) B = (IS_V ? a.bitsV : a.bitsK)[(size_t)bh * a.ncols + tok];
             B = B < 1 ? 1 : (B > 8 ? 8 : B);
-        } else if (x == 0) {
+        } else if (!IS_V) {
             B = ladder(rng, a.cK, a.bmin, a.bmax);
         } else {
-            float sh = __int_as_float(0xff800000);
-#pragma unroll
-            for (int g = 0; g < P; ++g) sh = fmaxf(sh, s_part[g][slot]);
-            B = min(nv, a.W) == 0 ? a.bmax : ladder(__fmul_rn(rng, sh), a.cV, a.bmin, a.bmax);
+            const long col = (long)min(tok, a.T - 1);           // whole warps read the window; columns beyond the last are not used
+            const int nv = min((int)a.nvalid[(size_t)bh * a.ncols + col], a.W);
+            const float sh = qaqc::window_max(a.ring + (size_t)bh * a.W * a.ncols + col, a.W, a.ncols, nv);
+            B = nv == 0 ? a.bmax : ladder(__fmul_rn(rng, sh), a.cV, a.bmin, a.bmax);
         }
-        Bn = (UP || B < Bo) ? B : Bo;
+        if (valid) Bn = (UP || B < Bo) ? B : Bo;
     }
-    if (p == 0) s_bn[slot] = (uint8_t)Bn;
-    bool changed = __syncthreads_or(Bn != Bo) != 0;          // also makes the widths visible
+    const uint32_t alike = qaqc::count_half(Bn, lane, sm.count[warp]);
+    bool changed = __syncthreads_or(Bn != Bo) != 0;          // also makes the counts visible
     // An open tile has to be the last thing in its pool.  If closed tiles of this (b,h) have just been moved
     // behind it, it moves to the end as well, whether its own tokens change or not.
     const bool open = tile == a.T / QAQ_TILE && (a.T % QAQ_TILE) != 0;
-    const bool relocate = open && tw.x + tw.y != ts.pool_end[bh];
+    const bool relocate = open && tw.x + tw.y != pool_end;
     changed = changed || relocate;
     if (!changed) return;
 
-    // ---- the stored bytes come to shared memory; warp 0: tokens sorted by their new widths, size and place of the new tile
+    // ---- the stored bytes come to shared memory; order, size and place of the new tile
     const uint8_t* src = ts.codes + (size_t)bh * a.pool_bytes + tw.x;
-    for (uint32_t o = tid * 16; o < ((tw.y + 15u) & ~15u); o += NT * 16)
-        *reinterpret_cast<uint4*>(s_img + o) = *reinterpret_cast<const uint4*>(src + o);
-    if (warp == 0) {
-        int n[9];
-        const int b0 = s_bn[lane], b1 = s_bn[lane + 32];
-        const qaqc::Sorted so = x ? qaqc::sort_tile<true>(lane, b0, b1, n, s_sorted) : qaqc::sort_tile<false>(lane, b0, b1, n, s_sorted);
-        s_place[lane] = (unsigned short)(so.slot[0] | (so.row_w[0] << 8));
-        s_place[lane + 32] = (unsigned short)(so.slot[1] | (so.row_w[1] << 8));
-        const int tokens = __popc(__ballot_sync(0xFFFFFFFFu, b0 != 0)) + __popc(__ballot_sync(0xFFFFFFFFu, b1 != 0));
-        if (lane == 0) {
-            const uint32_t nb = x ? qaqc::make_sections<qaqc::UNITS<D, true>>(n, s_tab, s_head) : qaqc::make_sections<qaqc::UNITS<D, false>>(n, s_tab, s_head);
-            // where the new tile goes: in place unless it grows
-            const uint32_t off = tw.x, old_nb = tw.y;
-            const uint32_t old_own = open ? old_nb : ((old_nb + 15u) & ~15u);   // closed tiles own a rounded amount
-            uint32_t noff = off;
-            int skip = 0;
-            if (nb > old_own || relocate) {
-                if (open && off + old_nb == ts.pool_end[bh]) {
-                    // still the last thing in its pool: it grows where it is
-                    if ((size_t)off + nb + 16 > a.pool_bytes) skip = 1;
-                    else ts.pool_end[bh] = off + nb;
-                } else if (open) {
-                    // behind everything else, 16-byte aligned, and exactly as long as its bytes: the last thing
-                    // in the pool again (one CTA per pool does this, and nobody else touches the pool in its launch)
-                    noff = (ts.pool_end[bh] + 15u) & ~15u;
-                    if ((size_t)noff + nb + 16 > a.pool_bytes) skip = 1;
-                    else ts.pool_end[bh] = noff + nb;
-                } else {
-                    // the end of the pool need not be aligned while a tile is open: take 16 bytes more and align;
-                    // space that does not fit is given back
-                    const uint32_t take = ((nb + 15u) & ~15u) + 16u;
-                    const bool full = *(volatile uint32_t*)&ts.pool_end[bh] > a.pool_bytes;      // takes nothing: the end must not run away
-                    const uint32_t at = full ? 0u : atomicAdd(&ts.pool_end[bh], take);
-                    noff = (at + 15u) & ~15u;
-                    if (full) skip = 1;
-                    else if ((size_t)at + take + 16 > a.pool_bytes) { skip = 1; pool_give_back(&ts.pool_end[bh], at, take); }
-                }
-                if (skip) atomicMax(a.status, (int)QAQ_ERR_CAPACITY);
-            }
-            s_tot = nb; s_off = noff; s_skip = skip; s_holes = x && (tokens & 3);
-        }
-    }
-    __syncthreads();
-    if (s_skip) return;                  // no room in the pool: the tile stays as it is
-    // ---- the sections as they are stored
-    if (warp == NT / 32 - 1) {
-        int n[9];
-        const uint32_t* h = reinterpret_cast<const uint32_t*>(s_img);
-        qaqc::counts_of(tw.y ? h[0] : 0u, tw.y ? h[1] : 0u, n);
-        if (lane == 0) {
-            if (x) qaqc::make_sections<qaqc::UNITS<D, true>>(n, s_otab, nullptr);
-            else qaqc::make_sections<qaqc::UNITS<D, false>>(n, s_otab, nullptr);
-        }
-        if (x && lane < QAQ_TILE / 4) {
-            int w = 0, end = 0;
-#pragma unroll
-            for (int k = 8; k >= 1; --k) {
-                if (lane >= end && lane < end + n[k]) w = k;
-                end += n[k];
-            }
-            s_orow[lane] = (uint8_t)w;
-        }
-    }
-    __syncthreads();
-
-    // ---- old words -> codes -> low bits dropped, or codes from the unquantized row
-    uint32_t creg[8];
-    if (Bn) {
-        if (UP && Bn > Bo) {
-            // raised: with the token's stored min / max and the thresholds
-            const __half* row = (x ? a.Vs : a.Ks) + (size_t)(bh / a.H) * a.sb + (size_t)(bh % a.H) * a.sh + (size_t)tok * a.st + 32 * p;
-            fresh_codes(row, a.thr[(size_t)bh * 4 + 2 * x], a.thr[(size_t)bh * 4 + 2 * x + 1], mn, mx, Bn, creg);
-        } else {
-            const int w = x ? (int)s_orow[oslot >> 2] : Bo;
-            if (x == 0) qaqc::read_token<D, false>(s_img, s_otab[w], oslot, w, p, creg);
-            else        qaqc::read_token<D, true>(s_img, s_otab[w], oslot, w, p, creg);
-            const int drop = Bo - Bn;
-            const uint32_t keep = 0x01010101u * (0xFFu >> drop);
-#pragma unroll
-            for (int j = 0; j < 8; ++j) creg[j] = (creg[j] >> drop) & keep;
-        }
-    }
-    __syncthreads();   // every old byte of the tile has been read
-    if (s_holes) {     // empty slots of the value groups have to read as zero
-        for (int o = tid; o < IMG / 16; o += NT) reinterpret_cast<uint4*>(s_img)[o] = make_uint4(0, 0, 0, 0);
-        __syncthreads();
-    }
-    if (tid < 4) reinterpret_cast<uint32_t*>(s_img)[tid] = s_head[tid];
-    const uint32_t pl = s_place[slot];
-    if (Bn) qaqc::write_token<D>(s_img, s_tab[pl >> 8], x == 1, (int)(pl & 0xFFu), (int)(pl >> 8), p, creg);
-    __syncthreads();   // the image is complete
-
-    // ---- the image replaces the tile; widths and tile length follow
-    uint8_t* dst = ts.codes + (size_t)bh * a.pool_bytes + s_off;
-    if (x == 0) {
-        for (uint32_t o = tid * 16; o < ((s_tot + 15u) & ~15u); o += NT * 16)
-            *reinterpret_cast<uint4*>(dst + o) = *reinterpret_cast<const uint4*>(s_img + o);
-    } else {
-        const int row = (tid / (16 * P)) * 4 + (tid & 3), e = (tid >> 2) % (4 * P);
-        if (row < s_tab[1].start + s_tab[1].n) {
-            const int w = s_sorted[4 * row];
-            qaqc::group_out<D>(s_img, dst, s_tab[w], w, row, e);
-        }
-        if (tid == 0) *reinterpret_cast<uint4*>(dst) = *reinterpret_cast<const uint4*>(s_img);
-    }
-    if (valid && p == 0) ts.bs[mt] = (unsigned short)(Bn | ((pl & 0xFFu) << 8));
+    const uint32_t old_nb = min(tw.y, (uint32_t)qaqc::tile_bytes_max(D));
+    for (uint32_t o = tid * 16; o < old_nb; o += 64 * 16)
+        asm volatile("cp.async.cg.shared.global [%0], [%1], 16;" ::"r"((uint32_t)__cvta_generic_to_shared(sm.old + o)), "l"(src + o) : "memory");
+    int slot;
+    const qaqc::TileRows rows = qaqc::rows_of_counts<IS_V>(sm.count, Bn, alike, warp, lane, slot);
+    const uint32_t nb = qaqc::tile_total<D, IS_V>(rows);
+    sm.range[tid] = range;
     if (tid == 0) {
+        // where the new tile goes: in place unless it grows
+        const uint32_t off = tw.x;
+        const uint32_t old_own = open ? old_nb : ((old_nb + 15u) & ~15u);   // closed tiles own a rounded amount
+        uint32_t noff = off;
+        int skip = 0;
+        if (nb > old_own || relocate) {
+            if (open && off + old_nb == pool_end) {
+                // still the last thing in its pool: it grows where it is
+                if ((size_t)off + nb + 16 > a.pool_bytes) skip = 1;
+                else ts.pool_end[bh] = off + nb;
+            } else if (open) {
+                // behind everything else, 16-byte aligned, and exactly as long as its bytes: the last thing
+                // in the pool again (one CTA per pool does this, and nobody else touches the pool in its launch)
+                noff = (pool_end + 15u) & ~15u;
+                if ((size_t)noff + nb + 16 > a.pool_bytes) skip = 1;
+                else ts.pool_end[bh] = noff + nb;
+            } else {
+                // the end of the pool need not be aligned while a tile is open: take 16 bytes more and align;
+                // space that does not fit is given back
+                const uint32_t take = ((nb + 15u) & ~15u) + 16u;
+                const bool full = *(volatile uint32_t*)&ts.pool_end[bh] > a.pool_bytes;      // takes nothing: the end must not run away
+                const uint32_t at = full ? 0u : atomicAdd(&ts.pool_end[bh], take);
+                noff = (at + 15u) & ~15u;
+                if (full) skip = 1;
+                else if ((size_t)at + take + 16 > a.pool_bytes) { skip = 1; pool_give_back(&ts.pool_end[bh], at, take); }
+            }
+            if (skip) atomicMax(a.status, (int)QAQ_ERR_CAPACITY);
+        }
+        sm.off = noff; sm.skip = skip;
+    }
+    asm volatile("cp.async.wait_all;" ::: "memory");
+    __syncthreads();
+    if (sm.skip) return;                 // no room in the pool: the tile stays as it is
+    const uint32_t noff = sm.off;
+    if (valid && Bn) {
+        uint4 h = *reinterpret_cast<const uint4*>(sm.old);
+        if (!tw.y) h = make_uint4(0u, 0u, 0u, 0u);
+        const qaqc::TileRows orows = qaqc::rows_of_header(h.x, h.y);
+        const int orow = IS_V ? oslot >> 2 : oslot, ow = IS_V ? max(1, min(8, qaqc::width_of_row(orows, orow))) : max(Bo, 1);
+        const qaqc::RowPlace o = qaqc::place_row<D, IS_V>(orows, orow, ow);
+        const int row = IS_V ? slot >> 2 : slot, w = IS_V ? qaqc::width_of_row(rows, row) : Bn;
+        const qaqc::RowPlace n = qaqc::place_row<D, IS_V>(rows, row, w);
+        sm.slot[slot] = make_uint4(o.main | (n.main << 16), o.high | (n.high << 16),
+                                   (uint32_t)tid | ((uint32_t)Bo << 8) | ((uint32_t)Bn << 12) | ((uint32_t)ow << 16) | ((uint32_t)w << 20),
+                                   o.mm | (o.mh << 4) | (n.mm << 8) | (n.mh << 12) | ((uint32_t)(oslot & 3) << 16));
+    }
+    __syncthreads();
+
+    uint8_t* dst = ts.codes + (size_t)bh * a.pool_bytes + noff;
+    const int nt = (int)(((sm.count[0][0] + sm.count[1][0]) * qaqc::ONES >> 24) + ((sm.count[0][1] + sm.count[1][1]) * qaqc::ONES >> 24));     // slots in use
+#pragma unroll 1
+    for (int it = 0; it < IT; ++it) {
+        const int sl = 32 * warp + it * TPI + g;
+        uint32_t lo[4] = {0, 0, 0, 0}, hi[4] = {0, 0, 0, 0};
+        uint4 q = make_uint4(0u, 0u, 0u, 0u);
+        if (sl < nt) {
+            q = sm.slot[sl];
+            const int t = (int)(q.z & 63u), bo = (int)((q.z >> 8) & 15u), bn = (int)((q.z >> 12) & 15u), ow = (int)((q.z >> 16) & 15u);
+            if (UP && bn > bo) {
+                // raised: with the token's stored min / max and the thresholds
+                const uint32_t mm = sm.range[t];
+                const float mn = __half2float(__ushort_as_half((unsigned short)(mm & 0xFFFF))), mx = __half2float(__ushort_as_half((unsigned short)(mm >> 16)));
+                const __half* row = (IS_V ? a.Vs : a.Ks) + (size_t)(bh / a.H) * a.sb + (size_t)(bh % a.H) * a.sh + (size_t)(tile * QAQ_TILE + t) * a.st + 32 * p;
+                uint32_t creg[8];
+                fresh_codes(row, a.thr[(size_t)bh * 4 + 2 * IS_V], a.thr[(size_t)bh * 4 + 2 * IS_V + 1], mn, mx, bn, creg);
+                qaqc::nibbles_of(creg, 0, lo);
+                qaqc::nibbles_of(creg, 4, hi);
+            } else {
+                const int wm = min(ow, 4);
+                constexpr uint32_t LAST = sizeof(sm.old) - 16;      // whatever the metadata say, nothing beyond the buffer is read
+                const uint32_t mm = q.w & 15u, mh = (q.w >> 4) & 15u;
+                const int i = (int)((q.w >> 16) & 3u);
+                const uint32_t m_at = (q.x & 0xFFFFu) + (IS_V ? 4 * p * mm : (uint32_t)p) * 4 * wm, m_end = m_at + (IS_V ? 3 * mm * 4 * wm : 0u);
+                if (m_end <= LAST) take_part<IS_V>(sm.old + m_at, wm, mm, i, lo);
+                if (ow > 4) {
+                    const uint32_t h_at = (q.y & 0xFFFFu) + (IS_V ? 4 * p * mh : (uint32_t)p) * 4 * (ow - 4), h_end = h_at + (IS_V ? 3 * mh * 4 * (ow - 4) : 0u);
+                    if (h_end <= LAST) take_part<IS_V>(sm.old + h_at, ow - 4, mh, i, hi);
+                }
+                drop_bits(lo, hi, bo - bn);
+            }
+        }
+        __syncwarp();
+        if (IS_V) {                    // the group's row: that of its first slot
+            const int first = sl & ~3;
+            if (first < nt) q = sm.slot[first];
+        }
+        const int w = (int)((q.z >> 20) & 15u);
+        const bool wide = __any_sync(0xFFFFFFFFu, w > 4);
+        if (IS_V) qaqc::transpose4<P>(lo, g & 3);
+        if (IS_V && wide) qaqc::transpose4<P>(hi, g & 3);
+        const int e = IS_V ? 4 * p + (g & 3) : p;
+        if (w) {
+            const int wm = min(w, 4);
+            qaqc::store_nibbles(dst + (q.x >> 16) + (IS_V ? e * (int)((q.w >> 8) & 15u) : e) * 4 * wm, wm, lo);
+            if (w > 4) qaqc::store_nibbles(dst + (q.y >> 16) + (IS_V ? e * (int)((q.w >> 12) & 15u) : e) * 4 * (w - 4), w - 4, hi);
+        }
+    }
+    if (valid && Bn) ts.bs[mt] = (unsigned short)(Bn | (slot << 8));
+    if (tid == 0) {
+        *reinterpret_cast<uint4*>(dst) = qaqc::header_of<D, IS_V>(rows);
         // an open tile that is still the last thing in its pool gives back what it no longer needs:
         // appends continue right behind its bytes
-        if (open && s_off == tw.x && s_tot < tw.y && tw.x + tw.y == ts.pool_end[bh]) ts.pool_end[bh] = s_off + s_tot;
-        ts.tile[ti].x = s_off;
-        ts.tile[ti].y = s_tot;
+        if (open && noff == tw.x && nb < tw.y && tw.x + tw.y == pool_end) ts.pool_end[bh] = noff + nb;
+        ts.tile[ti].x = noff;
+        ts.tile[ti].y = nb;
     }
+}
+
+// blockIdx.z: keys or values
+template <int D, bool UP>
+__global__ void __launch_bounds__(64, 12) requant_kernel(const RequantArgs a) {
+    __shared__ RequantScratch<D> sm;
+    qaq_dependency();
+    if (blockIdx.z == 0) requantize_tile<D, UP, false>(a, sm);
+    else requantize_tile<D, UP, true>(a, sm);
 }
 
 template <bool UP>
 qaq_status launch_requant(int D, dim3 grid, const RequantArgs& a, cudaStream_t s) {
     switch (D) {
         case 32: QAQ_CUDA_TRY(qaq_launch(requant_kernel<32, UP>, grid, dim3(64), 0, s, a)); break;
-        case 64: QAQ_CUDA_TRY(qaq_launch(requant_kernel<64, UP>, grid, dim3(128), 0, s, a)); break;
-        case 128: QAQ_CUDA_TRY(qaq_launch(requant_kernel<128, UP>, grid, dim3(256), 0, s, a)); break;
+        case 64: QAQ_CUDA_TRY(qaq_launch(requant_kernel<64, UP>, grid, dim3(64), 0, s, a)); break;
+        case 128: QAQ_CUDA_TRY(qaq_launch(requant_kernel<128, UP>, grid, dim3(64), 0, s, a)); break;
         default: return QAQ_ERR_UNSUPPORTED_SHAPE;
     }
     return QAQ_OK;
