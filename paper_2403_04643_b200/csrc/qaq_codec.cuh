@@ -104,19 +104,7 @@ __device__ __forceinline__ void mask_outliers32(uint32_t (&v)[16], __half2 lo2, 
     }
 }
 
-template <int NW>
-__device__ __forceinline__ void store_words(uint8_t* p, const uint32_t* w) {   // aligned to the widest access it takes: 16 bytes for multiples of four words, 8 for two, else 4
-    if (NW % 4 == 0) {
-#pragma unroll
-        for (int i = 0; i < NW; i += 4) *reinterpret_cast<uint4*>(p + 4 * i) = make_uint4(w[i], w[i + 1], w[i + 2], w[i + 3]);
-    } else if (NW == 2) {
-        *reinterpret_cast<uint2*>(p) = make_uint2(w[0], w[1]);
-    } else {
-#pragma unroll
-        for (int i = 0; i < NW; ++i) reinterpret_cast<uint32_t*>(p)[i] = w[i];
-    }
-}
-template <int NW>
+template <int NW>          // aligned to the widest access taken: 16 bytes for multiples of four words, 8 for two, else 4
 __device__ __forceinline__ void load_words(const uint8_t* p, uint32_t* w) {
     if (NW % 4 == 0) {
 #pragma unroll
@@ -184,37 +172,6 @@ __device__ __forceinline__ void counts_of(uint32_t lo, uint32_t hi, int (&n)[9])
     for (int w = 1; w <= 4; ++w) { n[w] = (lo >> (8 * w - 8)) & 0xFF; n[w + 4] = (hi >> (8 * w - 8)) & 0xFF; }
 }
 
-// What one warp finds out about a tile from the widths of its 64 slots (lane: slots lane and lane + 32; 0 = empty):
-// the slots' places in the sorted order, the width of the row each one belongs to (values: of its group), the number of
-// rows of every width.  sorted: 64 bytes of shared memory.
-struct Sorted { int slot[2], row_w[2]; };
-template <bool IS_V>
-__device__ __forceinline__ Sorted sort_tile(int lane, int b0, int b1, int (&n)[9], uint8_t* sorted) {
-    const unsigned lt = (1u << lane) - 1u;
-    Sorted r;
-    r.slot[0] = r.slot[1] = 0;
-    int start = 0;
-    n[0] = 0;
-#pragma unroll
-    for (int w = 8; w >= 1; --w) {
-        const unsigned m0 = __ballot_sync(0xFFFFFFFFu, b0 == w), m1 = __ballot_sync(0xFFFFFFFFu, b1 == w);
-        const int c0 = __popc(m0), c = c0 + __popc(m1);
-        if (b0 == w) r.slot[0] = start + __popc(m0 & lt);
-        if (b1 == w) r.slot[1] = start + c0 + __popc(m1 & lt);
-        n[w] = IS_V ? ((start + c + 3) >> 2) - ((start + 3) >> 2) : c;   // groups whose first slot is in the section
-        start += c;
-    }
-    r.row_w[0] = b0; r.row_w[1] = b1;
-    if (IS_V) {
-        if (b0) sorted[r.slot[0]] = (uint8_t)b0;
-        if (b1) sorted[r.slot[1]] = (uint8_t)b1;
-        __syncwarp();
-        if (b0) r.row_w[0] = sorted[r.slot[0] & ~3];
-        if (b1) r.row_w[1] = sorted[r.slot[1] & ~3];
-    }
-    return r;
-}
-
 constexpr uint32_t NIB = 0x0F0F0F0Fu;
 // (a & m) | (b & ~m)
 __device__ __forceinline__ uint32_t bitsel(uint32_t a, uint32_t b, uint32_t m) { return (a & m) | (b & ~m); }
@@ -242,11 +199,6 @@ __device__ __forceinline__ void nibbles_of(const uint32_t (&creg)[8], int shift,
         v[u] = bitsel(a, b, NIB);
     }
 }
-__device__ __forceinline__ void store_part(uint8_t* dst, int w, int shift, const uint32_t (&creg)[8]) {
-    uint32_t v[4];
-    nibbles_of(creg, shift, v);
-    store_nibbles(dst, w, v);
-}
 // The nibble words of a unit of w-bit words.  Bits of a nibble beyond the w lowest are undefined.
 template <int W>
 __device__ __forceinline__ void nibble_words(const uint32_t* x, uint32_t (&v)[4]) {
@@ -262,93 +214,10 @@ __device__ __forceinline__ void nibble_words(const uint32_t* x, uint32_t (&v)[4]
         v[0] = x[0]; v[1] = x[0] >> 1; v[2] = x[0] >> 2; v[3] = x[0] >> 3;
     }
 }
-// the codes (one per byte) of a unit's words, or'd into creg at bit `shift` (0 or 4)
-__device__ __forceinline__ void take_part(const uint32_t (&x)[4], int w, int shift, uint32_t (&creg)[8]) {
-    uint32_t v[4];
-    if (w == 4) nibble_words<4>(x, v);
-    else if (w == 3) nibble_words<3>(x, v);
-    else if (w == 2) nibble_words<2>(x, v);
-    else nibble_words<1>(x, v);
-    const uint32_t m = 0x01010101u * ((1u << w) - 1u);
-#pragma unroll
-    for (int u = 0; u < 4; ++u) {
-        creg[2 * u] |= (v[u] & m) << shift;
-        creg[2 * u + 1] |= ((v[u] >> 4) & m) << shift;
-    }
-}
-
 // index of unit e of row r (counted from the section's first row) of a section of n rows of values
 __device__ __forceinline__ uint32_t v_unit(int D, int n, int r, int e) {
     const int k4 = r & ~3, m = n - k4 < 4 ? n - k4 : 4;
     return (uint32_t)(k4 * (D / 8) + e * m + (r & 3));
-}
-
-// One thread's 32 channels (block p) of a token, codes one per byte, written at its slot into a tile image:
-// keys as they are stored, values token by token (the token's words of a row take the quarter slot & 3 of the row's
-// bytes; group_out turns rows into the stored form).  B: width of the row.
-template <int D>
-__device__ __forceinline__ void write_token(uint8_t* img, const Section& s, bool is_v, int slot, int B, int p, const uint32_t (&creg)[8]) {
-    const int w = B < 4 ? B : 4;
-    store_part(img + s.main + ((slot - (is_v ? 4 * s.mstart : s.mstart)) * (D / 32) + p) * 4 * w, w, 0, creg);
-    if (B > 4) store_part(img + s.high + ((slot - (is_v ? 4 * s.start : s.start)) * (D / 32) + p) * 4 * (B - 4), B - 4, 4, creg);
-}
-
-// Values: one part of unit 4p + b of row r of a section as it is stored, from the words of its four tokens in the image.
-template <int D, int W>
-__device__ __forceinline__ void group_part(const uint8_t* img, uint8_t* dst, uint32_t base, int n, int r, int e) {
-    const uint32_t* src = reinterpret_cast<const uint32_t*>(img + base) + (uint32_t)(4 * r * (D / 32) + (e >> 2)) * W;
-    const uint32_t s01 = 0x0040u + 0x0011u * (uint32_t)(e & 3);     // byte e & 3 of both operands
-    uint32_t y[W];
-    uint32_t x[4][W];
-#pragma unroll
-    for (int i = 0; i < 4; ++i) load_words<W>(reinterpret_cast<const uint8_t*>(src + i * (D / 32) * W), x[i]);
-#pragma unroll
-    for (int c = 0; c < W; ++c) y[c] = prmt(prmt(x[0][c], x[1][c], s01), prmt(x[2][c], x[3][c], s01), 0x5410u);
-    store_words<W>(dst + base + v_unit(D, n, r, e) * 4 * W, y);
-}
-template <int D>
-__device__ __forceinline__ void group_out(const uint8_t* img, uint8_t* dst, const Section& s, int W, int row, int e) {
-    const int r = row - s.start, n = s.n, rm = row - s.mstart;
-    switch (W) {
-        case 1: group_part<D, 1>(img, dst, s.main, s.mn, rm, e); break;
-        case 2: group_part<D, 2>(img, dst, s.main, s.mn, rm, e); break;
-        case 3: group_part<D, 3>(img, dst, s.main, s.mn, rm, e); break;
-        default:
-            group_part<D, 4>(img, dst, s.main, s.mn, rm, e);
-            if (W == 5) group_part<D, 1>(img, dst, s.high, n, r, e);
-            else if (W == 6) group_part<D, 2>(img, dst, s.high, n, r, e);
-            else if (W == 7) group_part<D, 3>(img, dst, s.high, n, r, e);
-            else if (W == 8) group_part<D, 4>(img, dst, s.high, n, r, e);
-    }
-}
-
-// The inverse of write_token (and of group_out) on a stored tile: codes of one thread's 32 channels, one per byte.
-// B: width of the token's row.
-template <int D, bool IS_V>
-__device__ __forceinline__ void read_token(const uint8_t* tile, const Section& s, int slot, int B, int p, uint32_t (&creg)[8]) {
-#pragma unroll
-    for (int j = 0; j < 8; ++j) creg[j] = 0;
-#pragma unroll
-    for (int part = 0; part < 2; ++part) {
-        const int w = part ? B - 4 : (B < 4 ? B : 4);
-        if (w < 1) continue;
-        const uint8_t* src = tile + (part ? s.high : s.main);
-        const int first = part ? s.start : s.mstart, n = part ? s.n : s.mn;
-        uint32_t x[4] = {0, 0, 0, 0};
-        if (!IS_V) {
-            const uint32_t* u = reinterpret_cast<const uint32_t*>(src + (uint32_t)((slot - first) * (D / 32) + p) * 4 * w);
-#pragma unroll
-            for (int c = 0; c < 4; ++c) if (c < w) x[c] = u[c];
-        } else {
-#pragma unroll
-            for (int b = 0; b < 4; ++b) {
-                const uint8_t* u = src + v_unit(D, n, (slot >> 2) - first, 4 * p + b) * 4 * w + (slot & 3);
-#pragma unroll
-                for (int c = 0; c < 4; ++c) if (c < w) x[c] |= (uint32_t)u[4 * c] << (8 * b);
-            }
-        }
-        take_part(x, w, 4 * part, creg);
-    }
 }
 
 // ------------------------------------------------------------------------------------------ a tile by two warps
@@ -433,20 +302,21 @@ __device__ __forceinline__ RowPlace place_row(const TileRows& r, int row, int w)
 // The largest of the first nv of W scores, `stride` apart.  Every row of the window is read (the ring is allocated in full),
 // rows the token has no score in are left out of the maximum: the loads then depend on nothing and go out together.
 // By whole warps.
+template <int BATCH = 16>
 __device__ __forceinline__ float window_max(const float* r, int W, long stride, int nv) {
     float m = __int_as_float(0xff800000);
     int i = 0;
 #pragma unroll 1
-    for (; i + 16 <= W; i += 16, r += 16 * stride) {
-        float v[16];
+    for (; i + BATCH <= W; i += BATCH, r += BATCH * stride) {
+        float v[BATCH];
 #pragma unroll
-        for (int u = 0; u < 16; ++u) v[u] = r[u * stride];
-        if (__all_sync(0xFFFFFFFFu, i + 16 <= nv)) {
+        for (int u = 0; u < BATCH; ++u) v[u] = r[u * stride];
+        if (__all_sync(0xFFFFFFFFu, i + BATCH <= nv)) {
 #pragma unroll
-            for (int u = 0; u < 16; ++u) m = fmaxf(m, v[u]);
+            for (int u = 0; u < BATCH; ++u) m = fmaxf(m, v[u]);
         } else {
 #pragma unroll
-            for (int u = 0; u < 16; ++u) if (i + u < nv) m = fmaxf(m, v[u]);
+            for (int u = 0; u < BATCH; ++u) if (i + u < nv) m = fmaxf(m, v[u]);
         }
     }
 #pragma unroll 1
@@ -455,6 +325,47 @@ __device__ __forceinline__ float window_max(const float* r, int W, long stride, 
         if (i < nv) m = fmaxf(m, v);
     }
     return m;
+}
+// The nibble words of one part (w bits, 1..4) of a lane's 32 channels of one token.  Keys: the unit at `at`; values: byte i of
+// units 4p .. 4p+3, which lie m units apart from `at` on.
+template <int W, bool IS_V>
+__device__ __forceinline__ void take_words(const uint8_t* at, uint32_t m, int i, uint32_t (&v)[4]) {
+    uint32_t x[W];
+    if (!IS_V) {
+        load_words<W>(at, x);
+    } else {
+        uint32_t u[4][W];
+#pragma unroll
+        for (int b = 0; b < 4; ++b) load_words<W>(at + b * m * 4 * W, u[b]);
+        const uint32_t sel = 0x0040u + 0x0011u * (uint32_t)i;          // byte i of both operands
+#pragma unroll
+        for (int c = 0; c < W; ++c) x[c] = prmt(prmt(u[0][c], u[1][c], sel), prmt(u[2][c], u[3][c], sel), 0x5410u);
+    }
+    nibble_words<W>(x, v);
+    constexpr uint32_t mask = 0x11111111u * ((1u << W) - 1u);
+#pragma unroll
+    for (int k = 0; k < 4; ++k) v[k] &= mask;
+}
+template <bool IS_V>
+__device__ __forceinline__ void take_nibbles(const uint8_t* at, int w, uint32_t m, int i, uint32_t (&v)[4]) {
+    if (w == 4) take_words<4, IS_V>(at, m, i, v);
+    else if (w == 3) take_words<3, IS_V>(at, m, i, v);
+    else if (w == 2) take_words<2, IS_V>(at, m, i, v);
+    else take_words<1, IS_V>(at, m, i, v);
+}
+// Both parts of a stored token out of a tile in shared memory (`bytes` long): lo, hi are the nibble words of bits 0..3 and
+// 4..7 of its codes.  main, high: byte offsets of its row, ow: the row's width, mm, mh: distances of the units of values,
+// i: the slot's place in its group.  Whatever the metadata say, nothing beyond the buffer is read.
+template <int D, bool IS_V>
+__device__ __forceinline__ void take_token(const uint8_t* tile, uint32_t bytes, uint32_t main, uint32_t high, int ow, uint32_t mm, uint32_t mh, int i, int p,
+                                           uint32_t (&lo)[4], uint32_t (&hi)[4]) {
+    const int wm = min(ow, 4), wh = ow - 4;
+    const uint32_t m_at = main + (IS_V ? 4 * p * mm : (uint32_t)p) * 4 * wm;
+    if (m_at + (IS_V ? 3 * mm * 4 * wm : 0u) + 16 <= bytes) take_nibbles<IS_V>(tile + m_at, wm, mm, i, lo);
+    if (wh > 0) {
+        const uint32_t h_at = high + (IS_V ? 4 * p * mh : (uint32_t)p) * 4 * wh;
+        if (h_at + (IS_V ? 3 * mh * 4 * wh : 0u) + 16 <= bytes) take_nibbles<IS_V>(tile + h_at, wh, mh, i, hi);
+    }
 }
 // 4 x 4 bytes of every word, transposed over the four lanes that are S and 2S apart: lane i of them gets byte i of all four
 template <int S>

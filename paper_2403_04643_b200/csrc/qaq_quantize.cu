@@ -1,23 +1,14 @@
 // S1-S3: bit-width selection, outlier split, uniform quantization and bit-packing.
 //
-// Two kernels: whole tiles, which is all of a prompt but its last tokens, by two warps per tile and tensor
-// (quant_tiles_kernel, further down); partly filled tiles, tiles that are continued, the launches that take the token count
-// from device memory, and the selection of widths alone by a CTA per tile (quant_kernel):
-//
-// One CTA handles one tile (QAQ_TILE consecutive tokens) of one (b,h); head_dim/32 lanes
-// own one token, each lane 32 consecutive channels of K and of V (64 bytes each), held in
-// registers from the min/max pass to the packing pass, so K and V are read from HBM once.
-//   phase 0  attention-window maximum of the score rows (Section 4.2)
-//   phase 1  outlier masks and min/max of the non-outliers in binary16 pair arithmetic
-//            (exact: the inputs are binary16), width from the exponents (Section 4.1)
-//   phase 2  warp 0: the tokens sorted by width (ballots), sections and size of the tile,
-//            exclusive scan of the outlier counts, space taken from the (b,h) pools by atomicAdd
-//   phase 3  codes (binary32: one sub, one mul, round down), packed words written into a shared-memory
-//            image of the tile in the section layout of qaq_codec.cuh (values token by token, which
-//            the copy-out transposes into rows of four tokens), vector stores; outlier
-//            entries placed by popc ranks
-// A tile that is continued (an append behind a partly filled tile) is built anew: the codes of
-// its old tokens are read back from the pool, the image of old and new tokens replaces it.
+// One CTA handles one tile (QAQ_TILE consecutive tokens) of one (b,h) and tensor; K and V are read from HBM once.
+//   loads    the tokens' rows to shared memory; the attention-window maximum of a token by its thread (Section 4.2)
+//   pass 1   outlier masks and min/max of the non-outliers in binary16 pair arithmetic (exact: the inputs are
+//            binary16); the outliers listed; width from the exponents (Section 4.1)
+//   order    the tokens sorted by width, sections and size of the tile, space taken from the (b,h) pools
+//   pass 2   codes (binary32: one sub, one mul, round down), packed words to the section layout of qaq_codec.cuh;
+//            outlier entries, per-token metadata, the tile's table entry
+// A tile that is continued (an append behind a partly filled tile) is built anew: the words of its old tokens come
+// from the tile as it is stored and go to their new places without becoming codes.
 #include "qaq_codec.cuh"
 #include "qaq_internal.cuh"
 
@@ -46,7 +37,7 @@ struct QuantArgs {
     int tmax_pad, ntiles;
     int* status;
     int* d_count;          // null, or the token count kept in device memory: read instead of t_old / first_tile and
-    unsigned* d_ticket;    //   advanced by the last CTA of the launch to finish (small appends only)
+    unsigned* d_ticket;    //   advanced by the last CTA of the launch to have read it (one-token appends)
     int max_tokens;
     uint8_t* out_bitsK;    // selection only
     uint8_t* out_bitsV;
@@ -55,505 +46,15 @@ struct QuantArgs {
 
 using qaqc::ladder;
 
-__device__ __forceinline__ uint32_t lop3_sel(uint32_t a, uint32_t m, uint32_t c) {  // (a & m) | (c & ~m)
-    uint32_t d;
-    asm("lop3.b32 %0, %1, %2, %3, 0xE2;" : "=r"(d) : "r"(a), "r"(m), "r"(c));
-    return d;
-}
-__device__ __forceinline__ uint32_t lop3_and_or(uint32_t a, uint32_t b, uint32_t c) {  // (a & b) | c
-    uint32_t d;
-    asm("lop3.b32 %0, %1, %2, %3, 0xEA;" : "=r"(d) : "r"(a), "r"(b), "r"(c));
-    return d;
-}
 __device__ __forceinline__ __half2 as_h2(uint32_t x) { return *reinterpret_cast<__half2*>(&x); }
 __device__ __forceinline__ uint32_t as_u32(__half2 x) { return *reinterpret_cast<uint32_t*>(&x); }
-// One lane's 32 channels of one token and tensor: outlier masks, masked min / max.
-//   v[k] holds channels 2k, 2k+1 (binary16 pairs).  On return every outlier entry of v has
-//   been replaced by -inf: in the code computation that yields code byte 0 without a mask
-//   (the outlier's own value is re-read from memory when its list entry is written).
-//   inl : bit k = channel 2k is an inlier, bit 16+k = channel 2k+1 is an inlier
-__device__ __forceinline__ void analyze32(uint32_t (&v)[16], __half2 lo2, __half2 hi2, uint32_t& inl, __half2& mn2,
-                                          __half2& mx2) {
-    uint32_t mnacc = 0x7C007C00u, mxacc = 0xFC00FC00u, bits = 0;
-#pragma unroll
-    for (int k = 0; k < 16; ++k) {
-        const __half2 x = as_h2(v[k]);
-        const uint32_t m = __hge2_mask(x, lo2) & __hle2_mask(x, hi2);
-        mnacc = as_u32(__hmin2(as_h2(mnacc), as_h2(lop3_sel(v[k], m, 0x7C007C00u))));
-        v[k] = lop3_sel(v[k], m, 0xFC00FC00u);
-        mxacc = as_u32(__hmax2(as_h2(mxacc), as_h2(v[k])));
-        bits = lop3_and_or(m, 0x00010001u << k, bits);
-    }
-    inl = bits;
-    mn2 = as_h2(mnacc);
-    mx2 = as_h2(mxacc);
+// Space for a whole tile from a (b,h) pool: a rounded-up amount in one atomic.  `taken` is what the pool end moved by (to be
+// given back if the space turns out not to fit: pool_give_back).  full: the pool end already lay beyond the pool when the
+// CTA began; nothing is taken, so that the end cannot run away.
+__device__ __forceinline__ uint32_t pool_take(uint32_t* pool, uint32_t amount, uint32_t unit_mask, bool full, uint32_t& taken) {
+    taken = full ? 0u : (amount + unit_mask) & ~unit_mask;
+    return full ? 0xFFFF0000u : atomicAdd(pool, taken);
 }
-
-// space from a (b,h) pool: `whole` tiles take a rounded-up amount in one atomic; a tile that is
-// being continued takes the exact amount and is padded to the unit when it closes.  `taken` is
-// what the pool end moved by (to be given back if the space turns out not to fit: pool_give_back).
-// full: the pool end already lay beyond the pool when the CTA began; nothing is taken, so that the end cannot run away.
-__device__ __forceinline__ uint32_t pool_take(uint32_t* pool, uint32_t amount, uint32_t unit_mask, bool whole, bool closes, bool full,
-                                              uint32_t& taken) {
-    uint32_t base;
-    if (full) {
-        taken = 0;
-        base = 0xFFFF0000u;
-    } else if (whole) {
-        taken = (amount + unit_mask) & ~unit_mask;
-        base = atomicAdd(pool, taken);
-    } else {
-        base = atomicAdd(pool, amount);
-        taken = amount;
-        if (closes) {
-            const uint32_t pad = (0u - (base + amount)) & unit_mask;
-            if (pad) atomicAdd(pool, pad);
-            taken += pad;
-        }
-    }
-    return base;
-}
-
-// One CTA = one tile of 64 tokens of one (b,h); P = D/32 lanes own a token, each lane 32
-// consecutive channels (64 bytes) of K and of V, kept in registers across all phases.
-// Order of work (barriers in brackets): loads, attention window, outlier masks and ranges,
-// widths [A] warp 0 sorts the tile's tokens by width and sizes its sections, warp 1 scans the outlier counts and takes pool
-// space with four atomics in flight at once while every warp computes its codes [B] words into a
-// shared-memory image of the tile [C] the image goes out with 16-byte stores; outlier entries and
-// per-token metadata follow.  Slots below the first new token of a continued tile hold the tile's
-// old tokens: their widths come from the metadata, their codes from the tile as it is stored.
-template <int D, bool SELECT_ONLY>
-__global__ void __launch_bounds__(2 * D, D == 128 ? 3 : 4) quant_kernel(const QuantArgs a) {
-    constexpr int P = D / 32;            // lanes per token
-    constexpr int NT = 2 * D;            // threads
-    constexpr int IMG = qaqc::tile_bytes_max(D);
-    constexpr bool COUNTED = !SELECT_ONLY;   // the launches that may take the token count from device memory
-    const int bh = blockIdx.y;
-    const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
-    const int slot = tid / P, p = tid % P;
-    qaq_dependency();
-    int t_old = a.t_old, first_tile = a.first_tile;
-    if (COUNTED && a.d_count) {
-        t_old = *a.d_count;                // the same value in every thread of the launch: it is written only by tick()
-        first_tile = t_old / QAQ_TILE;
-        if (t_old + a.tok_hi > a.max_tokens) {             // no room: nothing is stored, the count stays
-            if (tid == 0) atomicMax(a.status, (int)QAQ_ERR_CAPACITY);
-            return;
-        }
-    }
-    const int tile = first_tile + blockIdx.x;
-    // counted launches: the last CTA to get here moves the count on.  Every thread of every CTA has used the count it
-    // read by then (the barrier), and nothing else of the launch reads it afterwards.
-    auto tick = [&]() {
-        if (COUNTED && a.d_count) {
-            __syncthreads();
-            if (tid == 0) {
-                __threadfence();
-                const unsigned n = gridDim.x * gridDim.y;
-                if (atomicInc(a.d_ticket, n - 1) == n - 1) *a.d_count = t_old + a.tok_hi;
-            }
-        }
-    };
-
-    const int abs_lo = max(tile * QAQ_TILE, t_old + a.tok_lo);
-    const int abs_hi = min((tile + 1) * QAQ_TILE, t_old + a.tok_hi);
-    const int s_lo = abs_lo - tile * QAQ_TILE, s_hi = abs_hi - tile * QAQ_TILE;
-    const bool valid = slot >= s_lo && slot < s_hi;       // a new token
-    const bool old = !SELECT_ONLY && slot < s_lo;         // a token the tile already holds
-    const int tn = tile * QAQ_TILE + slot - t_old;        // index among the new tokens
-
-    __shared__ uint8_t s_bits[2][QAQ_TILE];   // widths of the tile's slots (0: empty)
-    __shared__ uint32_t s_cnt[2][QAQ_TILE];   // outlier counts of the new tokens, then exclusive offsets
-    __shared__ qaqc::Section s_tab[2][9], s_otab[2][9];   // sections of the tile by width, and of the tile as it was (continued tiles)
-    __shared__ unsigned short s_place[2][QAQ_TILE];       // slot of every token in the sorted order | width of its row << 8
-    __shared__ uint8_t s_sorted[2][QAQ_TILE], s_orow[2][QAQ_TILE / 4];   // width of every slot; width of the stored rows of values
-    __shared__ uint32_t s_tot[2], s_base[2], s_obase[2], s_olimit[2], s_otot[2];
-    constexpr uint32_t OUT_STAGE = 4 * D;      // outliers of a tile whose (slot, channel) are listed on chip in entry order; more go out one by one
-    __shared__ unsigned short s_work[SELECT_ONLY ? 1 : 2][SELECT_ONLY ? 1 : OUT_STAGE];
-    __shared__ int s_skip;
-    __shared__ __align__(16) uint8_t s_img[SELECT_ONLY ? 1 : 2][SELECT_ONLY ? 16 : IMG];  // the tile as it will be stored
-
-    const float* thr = a.thr + (size_t)bh * 4;
-    const bool given = a.bitsK != nullptr;
-    const size_t ti = (size_t)bh * a.ntiles + tile;
-    const size_t mt = (size_t)bh * a.tmax_pad + (size_t)tile * QAQ_TILE + slot;
-
-    // ---- loads first (independent of everything else)
-    const int b_idx = bh / a.H, h_idx = bh % a.H;
-    uint32_t vk[16], vv[16];
-    {
-        const __half* Kr = a.K + (size_t)b_idx * a.sb + (size_t)h_idx * a.sh + (size_t)(valid ? tn : 0) * a.st + 32 * p;
-        const __half* Vr = a.V + (size_t)b_idx * a.sb + (size_t)h_idx * a.sh + (size_t)(valid ? tn : 0) * a.st + 32 * p;
-#pragma unroll
-        for (int i = 0; i < 4; ++i) {
-            uint4 x = make_uint4(0, 0, 0, 0), y = make_uint4(0, 0, 0, 0);
-            if (valid) {
-                x = *reinterpret_cast<const uint4*>(Kr + 8 * i);
-                y = *reinterpret_cast<const uint4*>(Vr + 8 * i);
-            }
-            vk[4 * i] = x.x; vk[4 * i + 1] = x.y; vk[4 * i + 2] = x.z; vk[4 * i + 3] = x.w;
-            vv[4 * i] = y.x; vv[4 * i + 1] = y.y; vv[4 * i + 2] = y.z; vv[4 * i + 3] = y.w;
-        }
-    }
-    uint32_t pool_now = 0;          // in the lanes that take space further down
-    if (!SELECT_ONLY && warp < 2 && lane < 4 && (lane & 1) == warp)
-        pool_now = (warp ? ((lane >> 1) ? a.v : a.k).opool_end : ((lane >> 1) ? a.v : a.k).pool_end)[bh];
-    // a continued tile: its sections as they are stored (warp x for tensor x; used behind the first barrier)
-    if (!SELECT_ONLY && s_lo > 0) {
-#pragma unroll
-        for (int x = 0; x < 2; ++x) {
-            if (warp != x) continue;
-            const TensorStore& ts = x ? a.v : a.k;
-            uint2 h = make_uint2(0u, 0u);
-            if (ts.tile[ti].y) h = *reinterpret_cast<const uint2*>(ts.codes + (size_t)bh * a.pool_bytes + ts.tile[ti].x);
-            int n[9];
-            qaqc::counts_of(h.x, h.y, n);
-            if (lane == 0) {
-                if (x) qaqc::make_sections<qaqc::UNITS<D, true>>(n, s_otab[x], nullptr);
-                else qaqc::make_sections<qaqc::UNITS<D, false>>(n, s_otab[x], nullptr);
-            }
-            if (x && lane < QAQ_TILE / 4) {
-                int w = 0, end = 0;
-#pragma unroll
-                for (int k = 8; k >= 1; --k) {
-                    if (lane >= end && lane < end + n[k]) w = k;
-                    end += n[k];
-                }
-                s_orow[x][lane] = (uint8_t)w;
-            }
-        }
-    }
-    // empty slots of the value groups have to read as zero
-    if (!SELECT_ONLY) {
-        uint4* z = reinterpret_cast<uint4*>(s_img[1]);
-        for (int o = tid; o < IMG / 16; o += NT) z[o] = make_uint4(0, 0, 0, 0);
-    }
-
-    // ---- attention window: the P lanes of a token take its rows p, p+P, ... and combine by shuffles
-    float shat = __int_as_float(0xff800000);
-    int nv_tok = 0;
-    {
-        if (!given && valid) {
-            nv_tok = a.nvalid[(size_t)bh * a.n_new + tn];
-            nv_tok = nv_tok < a.W ? nv_tok : a.W;
-            // every row of the window is read (the ring is allocated in full), rows the token has no score in are
-            // left out of the maximum: the loads then depend on nothing and go out together
-            const float* r = a.ring + (size_t)bh * a.W * a.n_new + tn;
-            int i = p;
-            for (; i + 7 * P < a.W; i += 8 * P) {
-                float v[8];
-#pragma unroll
-                for (int u = 0; u < 8; ++u) v[u] = r[(size_t)(i + u * P) * a.n_new];
-#pragma unroll
-                for (int u = 0; u < 8; ++u) if (i + u * P < nv_tok) shat = fmaxf(shat, v[u]);
-            }
-            for (; i < a.W; i += P) {
-                const float v = r[(size_t)i * a.n_new];
-                if (i < nv_tok) shat = fmaxf(shat, v);
-            }
-        }
-#pragma unroll
-        for (int o = 1; o < P; o <<= 1) shat = fmaxf(shat, __shfl_xor_sync(0xFFFFFFFFu, shat, o));
-    }
-
-    // ---- outlier masks and range of the rest (register work, needs nothing from shared memory)
-    uint32_t inl[2], cntx[2];
-    float mnf[2], mxf[2];
-#pragma unroll
-    for (int x = 0; x < 2; ++x) {
-        // thresholds as binary16 bounds that decide exactly like the binary32 ones on binary16 data
-        const __half lo = __float2half_ru(thr[2 * x]), hi = __float2half_rd(thr[2 * x + 1]);
-        __half2 mn2, mx2;
-        analyze32(x ? vv : vk, __half2half2(lo), __half2half2(hi), inl[x], mn2, mx2);
-        const __half lmin = __hmin(__low2half(mn2), __high2half(mn2));
-        const __half lmax = __hmax(__low2half(mx2), __high2half(mx2));
-        __half2 pk = __halves2half2(lmin, __hneg(lmax));
-#pragma unroll
-        for (int o = 1; o < P; o <<= 1) pk = __hmin2(pk, as_h2(__shfl_xor_sync(0xFFFFFFFFu, as_u32(pk), o)));
-        float mn = __low2float(pk), mx = -__high2float(pk);
-        if (mn > mx) { mn = 0.f; mx = 0.f; }   // no entry inside [lo, hi]
-        uint32_t cnt = 32u - (uint32_t)__popc(inl[x]);
-#pragma unroll
-        for (int o = 1; o < P; o <<= 1) cnt += __shfl_xor_sync(0xFFFFFFFFu, cnt, o);
-        mnf[x] = mn; mxf[x] = mx; cntx[x] = cnt;
-    }
-
-    // ---- widths
-    int Bx[2], oslot[2] = {0, 0};      // oslot: where an old token lies in the tile as it is stored
-#pragma unroll
-    for (int x = 0; x < 2; ++x) {
-        int B;
-        if (given) {
-            B = valid ? (x ? a.bitsV : a.bitsK)[(size_t)bh * a.n_new + tn] : 0;
-            B = B < 1 ? 1 : (B > 8 ? 8 : B);
-        } else {
-            const float r = __fsub_rn(mxf[x], mnf[x]);
-            if (x == 0) {
-                B = ladder(r, a.cK, a.bmin, a.bmax);
-            } else {
-                B = (nv_tok == 0) ? a.bmax : ladder(__fmul_rn(r, shat), a.cV, a.bmin, a.bmax);
-            }
-        }
-        Bx[x] = valid ? B : 0;
-        if (old) {
-            const uint32_t bs = (x ? a.v : a.k).bs[mt];
-            Bx[x] = min((int)(bs & 0xFFu), 8);
-            oslot[x] = (int)(bs >> 8);
-        }
-        if (p == 0) {                                   // every slot of the tile is written: empty ones count nothing
-            s_bits[x][slot] = (uint8_t)Bx[x];
-            s_cnt[x][slot] = valid ? cntx[x] : 0u;
-            if (SELECT_ONLY && valid) (x ? a.out_bitsV : a.out_bitsK)[(size_t)bh * a.n_new + tn] = (uint8_t)B;
-        }
-    }
-    if (SELECT_ONLY) return;
-    __syncthreads();   // [A] widths and outlier counts visible
-
-    // ---- warp 0: tokens sorted by width, sections and header of the tile, space for the bytes; warp 1: scan of the
-    //      outlier counts, space for the entries (the two halves do not depend on each other; the atomics - lane 2x of
-    //      warp 0 and lane 2x + 1 of warp 1 for tensor x - stay in flight while every warp computes its codes)
-    const bool starts = (s_lo == 0), closes = (s_hi == QAQ_TILE), whole = starts && closes;
-    uint32_t my_base = 0, my_amount = 0, my_taken = 0;
-    if (warp == 0) {
-        uint32_t amount[2];
-#pragma unroll
-        for (int x = 0; x < 2; ++x) {
-            const int b0 = s_bits[x][lane], b1 = s_bits[x][lane + 32];
-            int n[9];
-            const qaqc::Sorted so = x ? qaqc::sort_tile<true>(lane, b0, b1, n, s_sorted[x]) : qaqc::sort_tile<false>(lane, b0, b1, n, s_sorted[x]);
-            s_place[x][lane] = (unsigned short)(so.slot[0] | (so.row_w[0] << 8));
-            s_place[x][lane + 32] = (unsigned short)(so.slot[1] | (so.row_w[1] << 8));
-            uint32_t total = 0;
-            if (lane == 0) {
-                uint32_t* head = reinterpret_cast<uint32_t*>(s_img[x]);
-                total = x ? qaqc::make_sections<qaqc::UNITS<D, true>>(n, s_tab[x], head) : qaqc::make_sections<qaqc::UNITS<D, false>>(n, s_tab[x], head);
-                s_tot[x] = total;
-            }
-            total = __shfl_sync(0xFFFFFFFFu, total, 0);
-            // a continued tile stays where it is and takes only what it grows by behind its end
-            const uint32_t old_nb = starts ? 0u : (x ? a.v : a.k).tile[ti].y;
-            amount[x] = total - old_nb;
-        }
-        if (!(lane & 1) && lane < 4) {
-            const int x = lane >> 1;
-            my_amount = x ? amount[1] : amount[0];
-            my_base = pool_take(&(x ? a.v : a.k).pool_end[bh], my_amount, 15u, whole, closes, pool_now > a.pool_bytes, my_taken);
-        }
-    } else if (warp == 1) {
-        uint32_t amount[2];
-#pragma unroll
-        for (int x = 0; x < 2; ++x) {
-            const uint32_t c0 = s_cnt[x][lane], c1 = s_cnt[x][lane + 32];
-            uint32_t ic0 = c0, ic1 = c1;
-#pragma unroll
-            for (int d = 1; d < 32; d <<= 1) {
-                const uint32_t u0 = __shfl_up_sync(0xFFFFFFFFu, ic0, d), u1 = __shfl_up_sync(0xFFFFFFFFu, ic1, d);
-                if (lane >= d) { ic0 += u0; ic1 += u1; }
-            }
-            const uint32_t ctot0 = __shfl_sync(0xFFFFFFFFu, ic0, 31), ctot1 = __shfl_sync(0xFFFFFFFFu, ic1, 31);
-            s_cnt[x][lane] = ic0 - c0; s_cnt[x][lane + 32] = ctot0 + ic1 - c1;
-            amount[x] = ctot0 + ctot1;
-            if (lane == 0) s_otot[x] = ctot0 + ctot1;
-        }
-        if ((lane & 1) && lane < 4) {
-            const int x = lane >> 1;
-            my_amount = x ? amount[1] : amount[0];
-            my_base = pool_take(&(x ? a.v : a.k).opool_end[bh], my_amount, 3u, whole, closes, pool_now > a.ocap, my_taken);
-        }
-    }
-
-    // ---- codes of the new tokens (every warp; needs only registers): channels 4j..4j+3 in the byte lanes of creg[j]
-    uint32_t cregs[2][8];
-#pragma unroll
-    for (int x = 0; x < 2; ++x) qaqc::codes32(x ? vv : vk, mnf[x], mxf[x], Bx[x], cregs[x]);
-    // old tokens of a continued tile: their codes from the tile as it is stored (read before anything is written)
-    if (!starts) {
-#pragma unroll
-        for (int x = 0; x < 2; ++x) {
-            if (!old) continue;
-            const TensorStore& ts = x ? a.v : a.k;
-            const uint8_t* src = ts.codes + (size_t)bh * a.pool_bytes + ts.tile[ti].x;
-            const int w = x ? (int)s_orow[x][(oslot[x] >> 2) & (QAQ_TILE / 4 - 1)] : Bx[x];
-            if (!Bx[x]) continue;                       // never stored (the pool was full)
-            if (x == 0) qaqc::read_token<D, false>(src, s_otab[x][w], oslot[x], w, p, cregs[x]);
-            else        qaqc::read_token<D, true>(src, s_otab[x][w], oslot[x], w, p, cregs[x]);
-        }
-    }
-    __syncthreads();   // [B] sections visible
-
-    // ---- packed words into the shared-memory image of the tile (the values token by token: the copy to global memory
-    //      turns them into rows of four tokens)
-#pragma unroll
-    for (int x = 0; x < 2; ++x) {
-        const uint32_t pl = s_place[x][slot & (QAQ_TILE - 1)];
-        const int w = (int)(pl >> 8);
-        if ((valid || old) && w) qaqc::write_token<D>(s_img[x], s_tab[x][w], x == 1, (int)(pl & 0xFFu), w, p, cregs[x]);
-    }
-    // ---- where the outliers of the new tokens are: (slot, channel) in (token, channel) order - entries of lanes
-    //      p' < p of a token come first - listed in shared memory; their place needs only the scan of the counts.
-    //      The values are fetched and the entries written afterwards by all threads, one entry each.
-#pragma unroll
-    for (int x = 0; x < 2; ++x) {
-        uint32_t ob = valid ? ~inl[x] : 0u;
-        const uint32_t mine = (uint32_t)__popc(ob);
-        uint32_t before = 0;
-#pragma unroll
-        for (int d = 1; d < P; ++d) {
-            const uint32_t o = __shfl_up_sync(0xFFFFFFFFu, mine, d);
-            if (p >= d) before += o;
-        }
-        if (ob) {
-            const uint32_t all = ob;
-            const uint32_t lp0 = s_cnt[x][slot & (QAQ_TILE - 1)] + before;
-            while (ob) {
-                const int bit = __ffs(ob) - 1;
-                ob &= ob - 1;
-                const int k = bit & 15, hi = bit >> 4;
-                const int c = 2 * k + hi;                                   // channel inside the lane's 32
-                // entries of lower channels: pairs k' < k, plus channel 2k when this is 2k+1
-                const uint32_t lower = (((1u << k) - 1u) * 0x00010001u) | (hi ? (1u << k) : 0u);
-                const uint32_t lp = lp0 + (uint32_t)__popc(all & lower);
-                if (lp < OUT_STAGE) s_work[x][lp] = (unsigned short)(((slot & (QAQ_TILE - 1)) << 8) | (32 * p + c));
-            }
-        }
-    }
-    // ---- allocation results (the atomics were issued before the codes were computed).  A pool without room:
-    //      the space is given back, nothing about the tile is published and the CTA stops; the device status
-    //      reports the lost tokens.
-    if (warp == 0) {          // the byte pools
-        bool fail = false;
-        const bool mine = !(lane & 1) && lane < 4;
-        const int x = lane >> 1;
-        const TensorStore& ts = x ? a.v : a.k;
-        if (mine) {
-            const uint32_t off = starts ? my_base : ts.tile[ti].x;
-            fail = (size_t)my_base + my_taken + 16 > a.pool_bytes || (size_t)off + s_tot[x] + 16 > a.pool_bytes;
-            // a continued tile grows into what lies behind it: that has to be the space just taken (an open tile that
-            // re-quantization could not keep the last thing in a full pool cannot grow)
-            if (!starts && my_base != off + ts.tile[ti].y) fail = true;
-            s_base[x] = off;
-        }
-        const bool any_fail = __any_sync(0xFFFFFFFFu, fail);
-        if (mine) {
-            if (any_fail) {
-                pool_give_back(&ts.pool_end[bh], my_base, my_taken);
-            } else {
-                if (starts) ts.tile[ti].x = my_base;
-                ts.tile[ti].y = s_tot[x];
-            }
-        }
-        if (lane == 0) {
-            s_skip = any_fail ? 1 : 0;
-            if (any_fail) atomicMax(a.status, (int)QAQ_ERR_CAPACITY);
-        }
-    } else if (warp == 1) {   // the outlier lists: what fits is known now, the table is written once the byte pools have answered
-        if ((lane & 1) && lane < 4) {
-            const int x = lane >> 1;
-            const uint32_t room = (size_t)my_base + 8 < a.ocap ? a.ocap - 8 - my_base : 0;  // 8 entries of read-ahead margin
-            const uint32_t stored = my_amount < room ? my_amount : room;
-            if (stored < my_amount) atomicMax(a.status, (int)QAQ_ERR_CAPACITY);
-            s_obase[x] = my_base;
-            s_olimit[x] = my_base + stored;
-        }
-    }
-    __syncthreads();   // [C] image complete, pool positions known, every old byte of the tile has been read
-    if (warp == 1 && (lane & 1) && lane < 4) {
-        const int x = lane >> 1;
-        const TensorStore& ts = x ? a.v : a.k;
-        if (s_skip) {
-            pool_give_back(&ts.opool_end[bh], my_base, my_taken);
-        } else {
-            const uint32_t stored = s_olimit[x] - s_obase[x];
-            if (starts) { ts.tile[ti].z = my_base; ts.tile[ti].w = stored; }
-            else ts.tile[ti].w += stored;
-        }
-    }
-    if (s_skip) { tick(); return; }
-
-    // ---- the image goes out with vector stores; outlier list; per-token metadata
-#pragma unroll
-    for (int x = 0; x < 2; ++x) {
-        const TensorStore& ts = x ? a.v : a.k;
-        uint8_t* dst = ts.codes + (size_t)bh * a.pool_bytes + s_base[x];
-        const uint32_t nb = (s_tot[x] + 15u) & ~15u;     // tiles start 16-byte aligned and own a rounded amount
-        // the value of the first listed outlier of this thread is on its way (read again from the input: the
-        // registers hold -inf in its place) while the image goes out
-        const uint32_t ntot = s_otot[x], nst = ntot < OUT_STAGE ? ntot : OUT_STAGE;
-        const __half* X = (x ? a.V : a.K) + (size_t)b_idx * a.sb + (size_t)h_idx * a.sh;
-        uint32_t w_first = 0;
-        unsigned short v_first = 0;
-        if ((uint32_t)tid < nst) {
-            w_first = s_work[x][tid];
-            v_first = __half_as_ushort(X[(size_t)(tile * QAQ_TILE + (int)(w_first >> 8) - t_old) * a.st + (w_first & 0xFFu)]);
-        }
-        if (x == 0) {
-            for (uint32_t o = tid * 16; o < nb; o += NT * 16)
-                *reinterpret_cast<uint4*>(dst + o) = *reinterpret_cast<const uint4*>(s_img[x] + o);
-        } else {
-            // one unit per thread, the four rows that are interleaved side by side
-            const int row = (tid / (16 * P)) * 4 + (tid & 3), e = (tid >> 2) % (4 * P);
-            if (row < s_tab[x][1].start + s_tab[x][1].n) {
-                const int w = s_sorted[x][4 * row];
-                qaqc::group_out<D>(s_img[x], dst, s_tab[x][w], w, row, e);
-            }
-            if (tid == 0) *reinterpret_cast<uint4*>(dst) = *reinterpret_cast<const uint4*>(s_img[x]);
-        }
-        // outlier entries: one listed outlier per thread (value read again from the input: the registers hold -inf in
-        // its place), stores next to each other; a tile with more outliers than are listed writes the rest one by one
-        {
-            if ((uint32_t)tid < nst) {
-                const uint32_t pos = s_obase[x] + tid;
-                if (pos < s_olimit[x]) ts.outl[(size_t)bh * a.ocap + pos] = (uint32_t)v_first | ((w_first & 0xFFu) << 16) | ((w_first >> 8) << 24);
-            }
-            for (uint32_t i = tid + NT; i < nst; i += NT) {
-                const uint32_t w = s_work[x][i], sl = w >> 8, ch = w & 0xFFu;
-                const uint32_t pos = s_obase[x] + i;
-                if (pos < s_olimit[x])
-                    ts.outl[(size_t)bh * a.ocap + pos] = (uint32_t)__half_as_ushort(X[(size_t)(tile * QAQ_TILE + (int)sl - t_old) * a.st + ch]) |
-                                                          (ch << 16) | (sl << 24);
-            }
-            if (ntot > OUT_STAGE) {
-                // rare.  Nothing of the listing pass is kept in registers for this: the lane reads its 32 channels
-                // again and repeats the outlier test (same bounds, same bit order as analyze32)
-                const __half2 lo2 = __half2half2(__float2half_ru(thr[2 * x])), hi2 = __half2half2(__float2half_rd(thr[2 * x + 1]));
-                const __half* row = X + (size_t)(valid ? tn : 0) * a.st + 32 * p;
-                uint32_t ob = 0;
-                if (valid) {
-#pragma unroll
-                    for (int k = 0; k < 16; ++k) {
-                        const __half2 v = as_h2(reinterpret_cast<const uint32_t*>(row)[k]);
-                        ob |= (~(__hge2_mask(v, lo2) & __hle2_mask(v, hi2)) & 0x00010001u) << k;
-                    }
-                }
-                const uint32_t mine = (uint32_t)__popc(ob);
-                uint32_t lp0 = s_cnt[x][slot & (QAQ_TILE - 1)];
-#pragma unroll
-                for (int d = 1; d < P; ++d) {
-                    const uint32_t o = __shfl_up_sync(0xFFFFFFFFu, mine, d);
-                    if (p >= d) lp0 += o;
-                }
-                const uint32_t all = ob;
-                while (ob) {
-                    const int bit = __ffs(ob) - 1;
-                    ob &= ob - 1;
-                    const int k = bit & 15, hi = bit >> 4;
-                    const int c = 2 * k + hi;
-                    const uint32_t lower = (((1u << k) - 1u) * 0x00010001u) | (hi ? (1u << k) : 0u);
-                    const uint32_t lp = lp0 + (uint32_t)__popc(all & lower);
-                    if (lp >= OUT_STAGE && s_obase[x] + lp < s_olimit[x])
-                        ts.outl[(size_t)bh * a.ocap + s_obase[x] + lp] = (uint32_t)__half_as_ushort(row[c]) | ((uint32_t)(32 * p + c) << 16) |
-                                                                           ((uint32_t)(slot & (QAQ_TILE - 1)) << 24);
-                }
-            }
-        }
-        if ((valid || old) && p == 0) ts.bs[mt] = (unsigned short)(Bx[x] | ((s_place[x][slot & (QAQ_TILE - 1)] & 0xFFu) << 8));
-        if (valid && p == 0) {
-            ts.mnmx[mt] = (uint32_t)__half_as_ushort(__float2half_rn(mnf[x])) | ((uint32_t)__half_as_ushort(__float2half_rn(mxf[x])) << 16);
-        }
-    }
-    tick();
-}
-
 
 // ------------------------------------------------------------------------------------------ whole tiles, two warps each
 // A tile of one tensor comes to shared memory by asynchronous copies and is gone through twice: tokens in order for the
@@ -562,12 +63,15 @@ __global__ void __launch_bounds__(2 * D, D == 128 ? 3 : 4) quant_kernel(const Qu
 // a group of values swap bytes by shuffles).  What is done once per tile - the order, the sections, the space from the
 // pools - is done for 64 tokens by 64 threads.
 //
-// What bounds it: instructions (70 % of the issue slots, 60 % of the integer unit's cycles at 7B, batch 8).  The kernel for
-// any tile takes 7300 (keys) and 9100 (values) warp instructions per tile, this one 4200 on average.  4096 tokens, 256
-// (b,h), head_dim 128: 188 us for keys and values, against 323 us for the other kernel in a launch for each; one warp per
-// tile 231 us (11 tiles in flight per SM either way, for their shared memory); rounds unrolled by two 200 us, by four
-// 226 us (the code of one round is what the instruction cache holds).  It is the faster one down to the smallest launch:
-// 32 (b,h) of one tile 7.0 against 7.7 us, of 16 tiles 10.5 against 17.2 us.
+// What bounds it: instructions (70 % of the issue slots, 60 % of the integer unit's cycles at 7B, batch 8).  A kernel with
+// 256 threads per tile, a lane per 32 channels of a token throughout and an image of the tile in shared memory took
+// 7300 (keys) and 9100 (values) warp instructions per tile, this one 4200 on average.  4096 tokens, 256 (b,h), head_dim
+// 128: 188 us for keys and values, against 323 us; one warp per tile 231 us (11 tiles in flight per SM either way, for
+// their shared memory); rounds unrolled by two 200 us, by four 226 us (the code of one round is what the instruction
+// cache holds).  32 (b,h) of one tile 7.0 against 7.7 us, of 16 tiles 10.5 against 17.2 us.
+// A one-token append is a chain of memory latencies (token count; table and metadata; the tile) and of instructions: four
+// warps share the rounds of pass 2, and nothing but the tile itself waits for the table.  32 (b,h), a tile of 1 to 64
+// tokens: 6.3 us, against 8.4 us with two warps and the window read in two parts, as much as the kernel of 256 threads.
 // The integer unit limits this kernel (compares, minima, byte shuffles and selects all run there, at half rate), so sums,
 // shifts and packing are put where the multipliers are.
 __device__ __forceinline__ uint64_t pair_of(float a, float b) {
@@ -640,6 +144,14 @@ __device__ __forceinline__ uint32_t outliers_and_range(const uint32_t (&v)[16], 
     mn2 = mn; mx2 = mx;
     return qaqc::prmt(qaqc::prmt((uint32_t)out[0], (uint32_t)out[1], 0x0040u), qaqc::prmt((uint32_t)out[2], (uint32_t)out[3], 0x0040u), 0x5410u);
 }
+// of a token, from those of its P lanes: min | max << 16; 0, 0 where there is no inlier
+template <int P>
+__device__ __forceinline__ uint32_t range_of_token(__half2 mn2, __half2 mx2) {
+    __half2 pk = __halves2half2(__hmin(__low2half(mn2), __high2half(mn2)), __hneg(__hmax(__low2half(mx2), __high2half(mx2))));
+#pragma unroll
+    for (int o = 1; o < P; o <<= 1) pk = __hmin2(pk, as_h2(__shfl_xor_sync(0xFFFFFFFFu, as_u32(pk), o)));
+    return __hgt(__low2half(pk), __hneg(__high2half(pk))) ? 0u : as_u32(pk) ^ 0x80000000u;
+}
 // exclusive prefix over the lanes, and the sum
 __device__ __forceinline__ uint32_t prefix(uint32_t x, int lane, uint32_t& sum) {
     uint32_t inc = x;
@@ -651,62 +163,95 @@ __device__ __forceinline__ uint32_t prefix(uint32_t x, int lane, uint32_t& sum) 
     sum = __shfl_sync(0xFFFFFFFFu, inc, 31);
     return inc - x;
 }
+constexpr int OPEN_WARPS = 4;           // warps of a CTA with an open tile
+constexpr uint32_t STORED = 1u << 30;   // of a slot's last word: the token is taken from the stored tile
+
 // One tile of one tensor, by two warps: half of its tokens each until the widths are known, half of the slots each from there.
-template <int D, bool IS_V>
-__device__ __forceinline__ void quantize_tile(const QuantArgs& a, TileScratch<D>& sm, uint32_t* list, const uint32_t cap) {
+// OPEN: a tile that is begun, continued or closed, the only one of its (b,h) in the launch: its tokens up to s_lo are cached
+// already (and come from the tile as it is stored), those from s_lo to s_hi are new.
+template <int D, bool IS_V, bool OPEN>
+__device__ __forceinline__ void quantize_tile(const QuantArgs& a, TileScratch<D>& sm, uint8_t* stored_tile, uint32_t* list, const uint32_t cap) {
     constexpr int P = D / 32, TPI = 32 / P, IT = QAQ_TILE / 2 / TPI;  // lanes per token, tokens of a warp at a time, rounds
-    constexpr int PR = D / 8;                                         // 16-byte pieces of a row
+    constexpr int PR = D / 8, NW = OPEN ? OPEN_WARPS : 2;             // 16-byte pieces of a row; warps
     const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31, g = lane / P, p = lane % P;
-    const int tile = a.first_tile + blockIdx.x, bh = blockIdx.y, tn0 = tile * QAQ_TILE - a.t_old;
-    const TensorStore& ts = IS_V ? a.v : a.k;
-    const __half* X = (IS_V ? a.V : a.K) + (size_t)(bh / a.H) * a.sb + (size_t)(bh % a.H) * a.sh + (size_t)tn0 * a.st;
-    const uint32_t data = (uint32_t)__cvta_generic_to_shared(sm.data);
-    {
-        const __half* src = X + (size_t)(32 * warp + lane / PR) * a.st + 8 * (lane % PR);
-        const uint32_t dst = data + warp * (QAQ_TILE * D) + 16 * (lane ^ ((lane >> 3) & 3));
-#pragma unroll
-        for (int i = 0; i < PR; ++i, src += (32 / PR) * a.st)
-            asm volatile("cp.async.cg.shared.global [%0], [%1], 16;" ::"r"(dst + 512 * i), "l"(src) : "memory");
+    const bool counted = OPEN && a.d_count;
+    const int t_old = counted ? *a.d_count : a.t_old;
+    if (counted && t_old + a.tok_hi > a.max_tokens) {       // no room: nothing is stored, the count stays
+        if (tid == 0) atomicMax(a.status, (int)QAQ_ERR_CAPACITY);
+        return;
     }
+    const int tile = (counted ? t_old / QAQ_TILE : a.first_tile) + blockIdx.x, bh = blockIdx.y, tn0 = tile * QAQ_TILE - t_old;
+    const int s_lo = OPEN ? max(0, a.tok_lo - tn0) : 0, s_hi = OPEN ? min(QAQ_TILE, a.tok_hi - tn0) : QAQ_TILE;
+    const bool old = OPEN && tid < s_lo, fresh = !OPEN || (tid >= s_lo && tid < s_hi);      // this thread's token
+    const TensorStore& ts = IS_V ? a.v : a.k;
+    const bool main = !OPEN || warp < 2;                   // the threads of the 64 tokens; the others of an open tile help with the codes
+    const size_t mt = (size_t)bh * a.tmax_pad + (size_t)tile * QAQ_TILE + tid;
+    uint4* const tab = ts.tile + (size_t)bh * a.ntiles + tile;
+    const __half* X = (IS_V ? a.V : a.K) + (size_t)(bh / a.H) * a.sb + (size_t)(bh % a.H) * a.sh + (ptrdiff_t)tn0 * a.st;
+    const uint32_t data = (uint32_t)__cvta_generic_to_shared(sm.data);
+    // ---- all loads that wait for nothing else
+    uint4 tw = make_uint4(0u, 0u, 0u, 0u);
+    uint32_t bs_old = 0;
+    if (OPEN && s_lo > 0) tw = *tab;
+    if (OPEN && old) bs_old = ts.bs[mt];
     const float* thr = a.thr + (size_t)bh * 4 + (IS_V ? 2 : 0);
-    // thresholds as binary16 bounds that decide exactly like the binary32 ones on binary16 data
-    const __half2 lo2 = __half2half2(__float2half_ru(thr[0])), hi2 = __half2half2(__float2half_rd(thr[1]));
+    const float thr_lo = thr[0], thr_hi = thr[1];
     uint32_t* const pool = (lane ? ts.opool_end : ts.pool_end) + bh;
     uint32_t pool_now = 0;
     if (tid < 2) pool_now = *pool;
-    // ---- attention window of this thread's token
     const bool given = a.bitsK != nullptr;
+    const int col = OPEN ? min(max(tn0 + tid, 0), a.n_new - 1) : tn0 + tid;       // whole warps read; not every thread has a new token
     int b = 0, nv = 0;
-    float shat = __int_as_float(0xff800000);
-    if (given) {
-        b = (IS_V ? a.bitsV : a.bitsK)[(size_t)bh * a.n_new + tn0 + tid];
-    } else if (IS_V) {
-        nv = min((int)a.nvalid[(size_t)bh * a.n_new + tn0 + tid], a.W);
-        shat = qaqc::window_max(a.ring + (size_t)bh * a.W * a.n_new + tn0 + tid, a.W, a.n_new, nv);
+    if (main) {
+        if (given) b = (IS_V ? a.bitsV : a.bitsK)[(size_t)bh * a.n_new + col];
+        else if (IS_V) nv = a.nvalid[(size_t)bh * a.n_new + col];
+        const int row = 32 * warp + lane / PR;
+        const __half* src = X + (ptrdiff_t)row * a.st + 8 * (lane % PR);
+        const uint32_t dst = data + warp * (QAQ_TILE * D) + 16 * (lane ^ ((lane >> 3) & 3));
+#pragma unroll
+        for (int i = 0; i < PR; ++i, src += (32 / PR) * a.st)
+            if (!OPEN || (row + i * (32 / PR) >= s_lo && row + i * (32 / PR) < s_hi))
+                asm volatile("cp.async.cg.shared.global [%0], [%1], 16;" ::"r"(dst + 512 * i), "l"(src) : "memory");
     }
-    asm volatile("cp.async.wait_all;" ::: "memory");
+    // ---- attention window of this thread's token
+    float shat = __int_as_float(0xff800000);
+    if (IS_V && !given && main) {
+        nv = min(nv, a.W);
+        shat = qaqc::window_max<OPEN ? 32 : 16>(a.ring + (size_t)bh * a.W * a.n_new + col, a.W, a.n_new, nv);
+    }
+    if (OPEN) {                        // the tile as it is stored follows on its own: it is needed later
+        asm volatile("cp.async.commit_group;" ::: "memory");
+        const uint8_t* src = ts.codes + (size_t)bh * a.pool_bytes + tw.x;
+        for (uint32_t o = tid * 16; o < min(tw.y, (uint32_t)qaqc::tile_bytes_max(D)); o += 64 * NW / 2 * 16)
+            asm volatile("cp.async.cg.shared.global [%0], [%1], 16;" ::"r"((uint32_t)__cvta_generic_to_shared(stored_tile + o)), "l"(src + o) : "memory");
+        asm volatile("cp.async.commit_group;" ::: "memory");
+    }
+    // thresholds as binary16 bounds that decide exactly like the binary32 ones on binary16 data
+    const __half2 lo2 = __half2half2(__float2half_ru(thr_lo)), hi2 = __half2half2(__float2half_rd(thr_hi));
+    if (OPEN) asm volatile("cp.async.wait_group 1;" ::: "memory");
+    else asm volatile("cp.async.wait_all;" ::: "memory");
     __syncwarp();
 
     // ---- ranges and outliers, tokens in order: an outlier goes to the warp's list, its place is marked
     list += warp * cap;
 #pragma unroll 1
     for (int it = 0; it < IT; ++it) {
+        if (OPEN && !main) break;
+        if (OPEN && (32 * warp + it * TPI >= s_hi || 32 * warp + (it + 1) * TPI <= s_lo)) continue;        // no new token among them
         const int tok = 32 * warp + it * TPI + g, U = tok * PR + 4 * p;
         const uint32_t at = data + 16 * (U ^ ((U >> 3) & 3));
         uint32_t v[16];
         load_row(at, v);
         __half2 mn2, mx2;
         uint32_t ob = outliers_and_range(v, lo2, hi2, mn2, mx2);
-        __half2 pk = __halves2half2(__hmin(__low2half(mn2), __high2half(mn2)), __hneg(__hmax(__low2half(mx2), __high2half(mx2))));
-#pragma unroll
-        for (int o = 1; o < P; o <<= 1) pk = __hmin2(pk, as_h2(__shfl_xor_sync(0xFFFFFFFFu, as_u32(pk), o)));
-        if (p == 0) sm.range[tok] = __hgt(__low2half(pk), __hneg(__high2half(pk))) ? 0u : as_u32(pk) ^ 0x80000000u;    // 0, 0: no inlier
+        const uint32_t range = range_of_token<P>(mn2, mx2);
+        if (p == 0) sm.range[tok] = range;
         sm.out[tok * P + p] = ob;
     }
     __syncwarp();
     // ---- the outliers go to the warp's list, a token per lane, their places are marked
-    uint32_t nout;
-    {
+    uint32_t nout = 0;
+    if (main) {
         uint32_t ob[P], cnt = 0;
         if constexpr (P == 4) {
             const uint4 x = *reinterpret_cast<const uint4*>(&sm.out[tid * P]);
@@ -716,7 +261,10 @@ __device__ __forceinline__ void quantize_tile(const QuantArgs& a, TileScratch<D>
             for (int k = 0; k < P; ++k) ob[k] = sm.out[tid * P + k];
         }
 #pragma unroll
-        for (int k = 0; k < P; ++k) cnt += (uint32_t)__popc(ob[k]);
+        for (int k = 0; k < P; ++k) {
+            if (!fresh) ob[k] = 0;
+            cnt += (uint32_t)__popc(ob[k]);
+        }
         uint32_t pos = prefix(cnt, lane, nout);
 #pragma unroll
         for (int k = 0; k < P; ++k)
@@ -731,40 +279,76 @@ __device__ __forceinline__ void quantize_tile(const QuantArgs& a, TileScratch<D>
     }
 
     // ---- widths; which tokens have which
-    const uint32_t range = sm.range[tid];
+    const uint32_t range = sm.range[tid & (QAQ_TILE - 1)];
     const float mn = __low2float(as_h2(range)), mx = __high2float(as_h2(range));
     {
         const float r = __fsub_rn(mx, mn);
         if (given) b = b < 1 ? 1 : (b > 8 ? 8 : b);
         else if (!IS_V) b = ladder(r, a.cK, a.bmin, a.bmax);
         else b = nv == 0 ? a.bmax : ladder(__fmul_rn(r, shat), a.cV, a.bmin, a.bmax);
+        if (OPEN && !fresh) b = old ? min((int)(bs_old & 0xFFu), 8) : 0;
     }
-    const uint32_t alike = qaqc::count_half(b, lane, sm.count[warp]);
-    if (lane == 0) sm.nout[warp] = nout;
+    uint32_t alike = 0;
+    if (main) {
+        alike = qaqc::count_half(b, lane, sm.count[warp]);
+        if (lane == 0) sm.nout[warp] = nout;
+    }
+    if (OPEN) asm volatile("cp.async.wait_all;" ::: "memory");
     __syncthreads();
+    // the CTA that is the last to have read the token count moves it on
+    if (counted && tid == 0) {
+        const unsigned n = gridDim.x * gridDim.y * gridDim.z;
+        if (atomicInc(a.d_ticket, n - 1) == n - 1) *a.d_count = t_old + a.tok_hi;
+    }
     // ---- order and sections, by both warps alike; space from the pools
     int slot;
     const qaqc::TileRows rows = qaqc::rows_of_counts<IS_V>(sm.count, b, alike, warp, lane, slot);
     const uint32_t total = qaqc::tile_total<D, IS_V>(rows);
     const uint32_t nout0 = sm.nout[0], nall = nout0 + sm.nout[1];
     uint32_t base = 0, taken = 0;
-    if (tid < 2) base = pool_take(pool, lane ? nall : total, lane ? 3u : 15u, true, true, pool_now > (lane ? a.ocap : a.pool_bytes), taken);
-    {
+    if (!OPEN && tid < 2) base = pool_take(pool, lane ? nall : total, lane ? 3u : 15u, pool_now > (lane ? a.ocap : a.pool_bytes), taken);
+    if (!OPEN || b) {
         const int row = IS_V ? slot >> 2 : slot, row_w = IS_V ? qaqc::width_of_row(rows, row) : b;
         const qaqc::RowPlace pl = qaqc::place_row<D, IS_V>(rows, row, row_w);
         // the reciprocal of the step without its power of two (the range of binary16 numbers is nowhere near the ends of
         // binary32: both are the same number but for the exponent)
         const float len = __fsub_rn(mx, mn), inv = len > 0.f ? __fdiv_rn(1.0f, len) : 0.f;
         const bool endless = len > 0.f && inv == 0.f;         // a range that is not finite
-        sm.slot[slot] = make_uint4(__float_as_uint(mn), __float_as_uint(inv), pl.main | (pl.high << 16),
-                                   (uint32_t)tid | ((uint32_t)b << 8) | ((uint32_t)row_w << 16) | (pl.mm << 20) | (pl.mh << 24) | (endless ? 0x80000000u : 0u));
+        uint4 q = make_uint4(__float_as_uint(mn), __float_as_uint(inv), pl.main | (pl.high << 16),
+                             (uint32_t)tid | ((uint32_t)b << 8) | ((uint32_t)row_w << 16) | (pl.mm << 20) | (pl.mh << 24) | (endless ? 0x80000000u : 0u));
+        if (OPEN && old) {             // where it is in the tile as it is stored, instead of the range
+            const int oslot = (int)((bs_old >> 8) & (QAQ_TILE - 1));
+            uint4 h = *reinterpret_cast<const uint4*>(stored_tile);
+            if (!tw.y) h = make_uint4(0u, 0u, 0u, 0u);
+            const qaqc::TileRows orows = qaqc::rows_of_header(h.x, h.y);
+            const int orow = IS_V ? oslot >> 2 : oslot, ow = IS_V ? max(1, min(8, qaqc::width_of_row(orows, orow))) : b;
+            const qaqc::RowPlace o = qaqc::place_row<D, IS_V>(orows, orow, ow);
+            q.x = o.main | (o.high << 16);
+            q.y = (uint32_t)ow | (o.mm << 4) | (o.mh << 8) | ((uint32_t)(oslot & 3) << 12);
+            q.w = (q.w & 0x7FFFFFFFu) | STORED;
+        }
+        sm.slot[slot] = q;
     }
-    // ---- a pool without room: the space is given back, nothing about the tile is published; the device status reports
-    //      the lost tokens
+    // ---- a pool without room: the space is given back (or not taken), nothing about the tile is published; the device
+    //      status reports the lost tokens
     if (warp == 0) {
-        const uint32_t off = __shfl_sync(0xFFFFFFFFu, base, 0);
-        const bool fail = (size_t)off + __shfl_sync(0xFFFFFFFFu, taken, 0) + 16 > a.pool_bytes || (size_t)off + total + 16 > a.pool_bytes;
-        if (fail && lane < 2) pool_give_back(pool, base, taken);
+        bool fail;
+        if (OPEN) {
+            // nobody else is at these pools: a tile that is begun goes to the end, one that is continued has to be the last
+            // thing before it (an open tile that re-quantization could not keep there, in a full pool, cannot grow); what is
+            // closed takes a rounded amount
+            const uint32_t pool_end = __shfl_sync(0xFFFFFFFFu, pool_now, 0), opool_end = __shfl_sync(0xFFFFFFFFu, pool_now, 1);
+            const uint32_t off = s_lo ? tw.x : pool_end, end = s_hi == QAQ_TILE ? (off + total + 15u) & ~15u : off + total;
+            fail = pool_end > a.pool_bytes || (size_t)end + 16 > a.pool_bytes || (s_lo && pool_end != tw.x + tw.y);
+            const bool full = opool_end > a.ocap;
+            base = lane == 0 ? off : (full ? 0xFFFF0000u : opool_end);
+            if (lane == 0 && !fail) *pool = end;
+            if (lane == 1 && !fail && !full) *pool = s_hi == QAQ_TILE ? (opool_end + nall + 3u) & ~3u : opool_end + nall;
+        } else {
+            const uint32_t off = __shfl_sync(0xFFFFFFFFu, base, 0);
+            fail = (size_t)off + __shfl_sync(0xFFFFFFFFu, taken, 0) + 16 > a.pool_bytes || (size_t)off + total + 16 > a.pool_bytes;
+            if (fail && lane < 2) pool_give_back(pool, base, taken);
+        }
         if (lane < 2) sm.base[lane] = base;
         if (lane == 0) {
             sm.skip = fail;
@@ -780,23 +364,21 @@ __device__ __forceinline__ void quantize_tile(const QuantArgs& a, TileScratch<D>
     uint32_t* const outl = ts.outl + (size_t)bh * a.ocap + obase;
     if (tid == 0) {
         if (stored < nall) atomicMax(a.status, (int)QAQ_ERR_CAPACITY);
-        ts.tile[(size_t)bh * a.ntiles + tile] = make_uint4(off, total, obase, stored);
+        *tab = s_lo ? make_uint4(off, total, tw.z, tw.w + stored) : make_uint4(off, total, obase, stored);
         *reinterpret_cast<uint4*>(dst) = qaqc::header_of<D, IS_V>(rows);
     }
-    {
-        const size_t mt = (size_t)bh * a.tmax_pad + (size_t)tile * QAQ_TILE + tid;
-        ts.bs[mt] = (unsigned short)(b | (slot << 8));
-        ts.mnmx[mt] = range;
-    }
+    if (!OPEN || b) ts.bs[mt] = (unsigned short)(b | (slot << 8));
+    if (fresh) ts.mnmx[mt] = range;
     const uint32_t first = warp ? nout0 : 0u;
-    for (uint32_t i = lane; i < min(nout, cap); i += 32)
+    for (uint32_t i = lane; i < min(nout, cap); i += 32)          // (none beyond the first two warps)
         if (first + i < stored) outl[first + i] = list[i];
     if (nout > cap) {                  // more outliers than were listed: the rest is found once more in the input
         uint32_t seen = 0;
 #pragma unroll 1
         for (int it = 0; it < IT; ++it) {
             const int tok = 32 * warp + it * TPI + g;
-            const __half* row = X + (size_t)tok * a.st + 32 * p;
+            const bool there = !OPEN || (tok >= s_lo && tok < s_hi);
+            const __half* row = X + (ptrdiff_t)(there ? tok : s_lo) * a.st + 32 * p;
             uint32_t v[16];
 #pragma unroll
             for (int i = 0; i < 4; ++i) {
@@ -805,6 +387,7 @@ __device__ __forceinline__ void quantize_tile(const QuantArgs& a, TileScratch<D>
             }
             __half2 mn2, mx2;
             uint32_t ob = outliers_and_range(v, lo2, hi2, mn2, mx2);
+            if (!there) ob = 0;
             uint32_t sum, pos = seen + prefix((uint32_t)__popc(ob), lane, sum);
             seen += sum;
             for (; ob; ob &= ob - 1, ++pos) {
@@ -818,11 +401,18 @@ __device__ __forceinline__ void quantize_tile(const QuantArgs& a, TileScratch<D>
     // ---- codes, tokens by slot
     Scale sc;
     sc.k64 = a.k64;
+    const int nt = OPEN ? (int)(((sm.count[0][0] + sm.count[1][0]) * qaqc::ONES >> 24) + ((sm.count[0][1] + sm.count[1][1]) * qaqc::ONES >> 24)) : QAQ_TILE;
 #pragma unroll 1
-    for (int it = 0; it < IT; ++it) {
-        const uint4 q = sm.slot[32 * warp + it * TPI + g];
-        const int U = (int)(q.w & 63u) * PR + 4 * p, B = (int)((q.w >> 8) & 15u), w = (int)((q.w >> 16) & 15u);
-        uint32_t v[16], c[16], lo[4], hi[4];
+    for (int s0 = warp * TPI; s0 < nt; s0 += NW * TPI) {
+        const int sl = s0 + g;
+        uint4 q = make_uint4(0u, 0u, 0u, 0u);
+        if (!OPEN || sl < nt) q = sm.slot[sl];
+        const int U = (int)(q.w & 63u) * PR + 4 * p, B = (int)((q.w >> 8) & 15u);
+        const int w = OPEN && IS_V ? ((sl & ~3) < nt ? (int)((sm.slot[sl & ~3].w >> 16) & 15u) : 0) : (int)((q.w >> 16) & 15u);
+        uint32_t lo[4], hi[4];
+        const bool wide = __any_sync(0xFFFFFFFFu, w > 4);
+        if (!OPEN || __any_sync(0xFFFFFFFFu, sl < nt && !(q.w & STORED))) {
+        uint32_t v[16], c[16];
         load_row(data + 16 * (U ^ ((U >> 3) & 3)), v);
         sc.mn = __uint_as_float(q.x);
         sc.inv = __uint_as_float(q.y);
@@ -846,7 +436,6 @@ __device__ __forceinline__ void quantize_tile(const QuantArgs& a, TileScratch<D>
             }
             __syncwarp();
         }
-        const bool wide = __any_sync(0xFFFFFFFFu, w > 4);
         if (wide) {
             uint32_t creg[8];
 #pragma unroll
@@ -857,10 +446,21 @@ __device__ __forceinline__ void quantize_tile(const QuantArgs& a, TileScratch<D>
 #pragma unroll
             for (int u = 0; u < 4; ++u) lo[u] = qaqc::prmt(mad(c[4 * u + 2], a.k16, c[4 * u]), mad(c[4 * u + 3], a.k16, c[4 * u + 1]), 0x6420u);
         }
+        }
+        if (OPEN) {
+            if ((q.w & STORED) || sl >= nt) {
+#pragma unroll
+                for (int u = 0; u < 4; ++u) lo[u] = hi[u] = 0;
+                if (sl < nt) qaqc::take_token<D, IS_V>(stored_tile, qaqc::tile_bytes_max(D) + 16, q.x & 0xFFFFu, q.x >> 16, (int)(q.y & 15u), (q.y >> 4) & 15u,
+                                                       (q.y >> 8) & 15u, (int)((q.y >> 12) & 3u), p, lo, hi);
+            }
+            __syncwarp();
+            if (IS_V && (sl & ~3) < nt) q = sm.slot[sl & ~3];       // empty slots of the last group have its row
+        }
         if (IS_V) qaqc::transpose4<P>(lo, g & 3);
         const int e = IS_V ? 4 * p + (g & 3) : p;
         const int wm = min(w, 4);
-        qaqc::store_nibbles(dst + (q.z & 0xFFFFu) + (IS_V ? e * (int)((q.w >> 20) & 7u) : e) * 4 * wm, wm, lo);
+        if (!OPEN || w) qaqc::store_nibbles(dst + (q.z & 0xFFFFu) + (IS_V ? e * (int)((q.w >> 20) & 7u) : e) * 4 * wm, wm, lo);
         if (wide) {
             if (IS_V) qaqc::transpose4<P>(hi, g & 3);
             if (w > 4) qaqc::store_nibbles(dst + (q.z >> 16) + (IS_V ? e * (int)((q.w >> 24) & 7u) : e) * 4 * (w - 4), w - 4, hi);
@@ -868,44 +468,79 @@ __device__ __forceinline__ void quantize_tile(const QuantArgs& a, TileScratch<D>
     }
 }
 
-template <int D>
-__global__ void __launch_bounds__(64, D == 128 ? 11 : 12) quant_tiles_kernel(const QuantArgs a, uint32_t cap) {
+// dynamic shared memory: the scratch, the tile as it is stored (OPEN), the warps' lists of outliers
+template <int D, bool OPEN>
+__global__ void __launch_bounds__(OPEN ? 32 * OPEN_WARPS : 64, OPEN ? 4 : (D == 128 ? 11 : 12)) quant_tiles_kernel(const QuantArgs a, uint32_t cap) {
     extern __shared__ __align__(64) unsigned char tiles_smem[];
     TileScratch<D>& sm = *reinterpret_cast<TileScratch<D>*>(tiles_smem);
-    uint32_t* list = reinterpret_cast<uint32_t*>(tiles_smem + sizeof(TileScratch<D>));
+    uint8_t* stored_tile = tiles_smem + sizeof(TileScratch<D>);
+    uint32_t* list = reinterpret_cast<uint32_t*>(stored_tile + (OPEN ? qaqc::tile_bytes_max(D) + 16 : 0));
     qaq_dependency();
-    if (blockIdx.z == 0) quantize_tile<D, false>(a, sm, list, cap);
-    else quantize_tile<D, true>(a, sm, list, cap);
+    if (blockIdx.z == 0) quantize_tile<D, false, OPEN>(a, sm, stored_tile, list, cap);
+    else quantize_tile<D, true, OPEN>(a, sm, stored_tile, list, cap);
 }
 
-template <int D>
-qaq_status launch_tiles(dim3 grid, const QuantArgs& a, double alpha, cudaStream_t s) {
+// tiles.x tiles of every (b,h), all whole, or one that is not (or may not be)
+template <int D, bool OPEN>
+qaq_status launch_tiles(int tiles, int BH, const QuantArgs& a, double alpha, cudaStream_t s) {
     // the list holds a third more than the share of outliers asked for gives a tile, and some
     const uint32_t want = (uint32_t)(alpha * (QAQ_TILE * D) * 1.34) + 96, cap = (want < 2048 ? want : 2048) / 2;
-    QAQ_CUDA_TRY(qaq_launch(quant_tiles_kernel<D>, grid, dim3(64), sizeof(TileScratch<D>) + 2 * cap * sizeof(uint32_t), s, a, cap));
+    const size_t smem = sizeof(TileScratch<D>) + (OPEN ? qaqc::tile_bytes_max(D) + 16 : 0) + 2 * cap * sizeof(uint32_t);
+    static_assert(sizeof(TileScratch<D>) + qaqc::tile_bytes_max(D) + 16 + 2048 * sizeof(uint32_t) <= 48 * 1024, "shared memory that needs no attribute");
+    QAQ_CUDA_TRY(qaq_launch(quant_tiles_kernel<D, OPEN>, dim3((unsigned)tiles, (unsigned)BH, 2), dim3(OPEN ? 32 * OPEN_WARPS : 64), smem, s, a, cap));
     return QAQ_OK;
 }
-
-template <bool SELECT_ONLY>
-qaq_status launch(int D, dim3 grid, const QuantArgs& a, cudaStream_t s) {
+template <bool OPEN>
+qaq_status launch(int D, int tiles, int BH, const QuantArgs& a, double alpha, cudaStream_t s) {
     switch (D) {
-        case 32: QAQ_CUDA_TRY(qaq_launch(quant_kernel<32, SELECT_ONLY>, grid, dim3(64), 0, s, a)); break;
-        case 64: QAQ_CUDA_TRY(qaq_launch(quant_kernel<64, SELECT_ONLY>, grid, dim3(128), 0, s, a)); break;
-        case 128: QAQ_CUDA_TRY(qaq_launch(quant_kernel<128, SELECT_ONLY>, grid, dim3(256), 0, s, a)); break;
-        default: return QAQ_ERR_UNSUPPORTED_SHAPE;
-    }
-    return QAQ_OK;
-}
-
-// whole tiles
-qaq_status launch_whole(int D, dim3 grid, const QuantArgs& a, double alpha, cudaStream_t s) {
-    grid.z = 2;
-    switch (D) {
-        case 32: return launch_tiles<32>(grid, a, alpha, s);
-        case 64: return launch_tiles<64>(grid, a, alpha, s);
-        case 128: return launch_tiles<128>(grid, a, alpha, s);
+        case 32: return launch_tiles<32, OPEN>(tiles, BH, a, alpha, s);
+        case 64: return launch_tiles<64, OPEN>(tiles, BH, a, alpha, s);
+        case 128: return launch_tiles<128, OPEN>(tiles, BH, a, alpha, s);
     }
     return QAQ_ERR_UNSUPPORTED_SHAPE;
+}
+
+// Widths alone: one CTA = 64 tokens of one (b,h); P = D/32 lanes own a token, each lane 32 consecutive channels (64 bytes) of
+// K and of V.
+template <int D>
+__global__ void __launch_bounds__(2 * D) select_kernel(const QuantArgs a) {
+    constexpr int P = D / 32;
+    qaq_dependency();
+    const int bh = blockIdx.y, tn = blockIdx.x * QAQ_TILE + threadIdx.x / P, p = threadIdx.x % P;
+    const bool valid = tn < a.n_new;
+    const float* thr = a.thr + (size_t)bh * 4;
+    uint32_t v[2][16];
+#pragma unroll
+    for (int x = 0; x < 2; ++x) {
+        const __half* row = (x ? a.V : a.K) + (size_t)(bh / a.H) * a.sb + (size_t)(bh % a.H) * a.sh + (size_t)(valid ? tn : 0) * a.st + 32 * p;
+#pragma unroll
+        for (int i = 0; i < 4; ++i) {
+            const uint4 y = *reinterpret_cast<const uint4*>(row + 8 * i);
+            v[x][4 * i] = y.x; v[x][4 * i + 1] = y.y; v[x][4 * i + 2] = y.z; v[x][4 * i + 3] = y.w;
+        }
+    }
+    // the P lanes of a token take rows p, p+P, ... of its window
+    float shat = __int_as_float(0xff800000);
+    int nv = 0;
+    if (valid) {
+        nv = min((int)a.nvalid[(size_t)bh * a.n_new + tn], a.W);
+        const float* r = a.ring + (size_t)bh * a.W * a.n_new + tn;
+        for (int i = p; i < nv; i += P) shat = fmaxf(shat, r[(size_t)i * a.n_new]);
+    }
+#pragma unroll
+    for (int o = 1; o < P; o <<= 1) shat = fmaxf(shat, __shfl_xor_sync(0xFFFFFFFFu, shat, o));
+#pragma unroll
+    for (int x = 0; x < 2; ++x) {
+        const __half2 lo2 = __half2half2(__float2half_ru(thr[2 * x])), hi2 = __half2half2(__float2half_rd(thr[2 * x + 1]));
+        __half2 mn2, mx2;
+        outliers_and_range(v[x], lo2, hi2, mn2, mx2);
+        const uint32_t range = range_of_token<P>(mn2, mx2);
+        const float r = __fsub_rn(__high2float(as_h2(range)), __low2float(as_h2(range)));
+        if (valid && p == 0) {
+            const int b = x == 0 ? ladder(r, a.cK, a.bmin, a.bmax) : (nv == 0 ? a.bmax : ladder(__fmul_rn(r, shat), a.cV, a.bmin, a.bmax));
+            (x ? a.out_bitsV : a.out_bitsK)[(size_t)bh * a.n_new + tn] = (uint8_t)b;
+        }
+    }
 }
 
 qaq_status check_dense(const void* K, const void* V, long sb, long sh, long st, int D) {
@@ -926,8 +561,14 @@ qaq_status qaq_launch_select(const qaq_config* cfg, const qaq_policy* pol, const
     a.ring = ring; a.nvalid = nvalid; a.W = cfg->window; a.thr = thr;
     a.cK = pol->cK; a.cV = pol->cV; a.bmin = cfg->bits_min; a.bmax = cfg->bits_max;
     a.out_bitsK = bitsK; a.out_bitsV = bitsV;
-    dim3 grid((n + QAQ_TILE - 1) / QAQ_TILE, cfg->batch * cfg->heads);
-    return launch<true>(cfg->head_dim, grid, a, s);
+    const dim3 grid((n + QAQ_TILE - 1) / QAQ_TILE, cfg->batch * cfg->heads);
+    switch (cfg->head_dim) {
+        case 32: QAQ_CUDA_TRY(qaq_launch(select_kernel<32>, grid, dim3(64), 0, s, a)); break;
+        case 64: QAQ_CUDA_TRY(qaq_launch(select_kernel<64>, grid, dim3(128), 0, s, a)); break;
+        case 128: QAQ_CUDA_TRY(qaq_launch(select_kernel<128>, grid, dim3(256), 0, s, a)); break;
+        default: return QAQ_ERR_UNSUPPORTED_SHAPE;
+    }
+    return QAQ_OK;
 }
 
 qaq_status qaq_launch_append(qaq_cache* c, const void* K, const void* V, long sb, long sh, long st, int n_new,
@@ -950,18 +591,18 @@ qaq_status qaq_launch_append(qaq_cache* c, const void* K, const void* V, long sb
     if (cur % QAQ_TILE != 0) {  // head: finish (or extend) the open tile
         const int end = min(t1, (cur / QAQ_TILE + 1) * QAQ_TILE);
         a.tok_lo = cur - t0; a.tok_hi = end - t0; a.first_tile = cur / QAQ_TILE;
-        if ((stt = launch<false>(D, dim3(1, BH), a, s)) != QAQ_OK) return stt;
+        if ((stt = launch<true>(D, 1, BH, a, c->cfg.outlier_frac, s)) != QAQ_OK) return stt;
         cur = end;
     }
     const int full_end = t1 / QAQ_TILE * QAQ_TILE;
     if (cur < full_end) {       // body: whole tiles
         a.tok_lo = cur - t0; a.tok_hi = full_end - t0; a.first_tile = cur / QAQ_TILE;
-        if ((stt = launch_whole(D, dim3((full_end - cur) / QAQ_TILE, BH), a, c->cfg.outlier_frac, s)) != QAQ_OK) return stt;
+        if ((stt = launch<false>(D, (full_end - cur) / QAQ_TILE, BH, a, c->cfg.outlier_frac, s)) != QAQ_OK) return stt;
         cur = full_end;
     }
     if (cur < t1) {             // tail: a new, partly filled tile
         a.tok_lo = cur - t0; a.tok_hi = t1 - t0; a.first_tile = cur / QAQ_TILE;
-        if ((stt = launch<false>(D, dim3(1, BH), a, s)) != QAQ_OK) return stt;
+        if ((stt = launch<true>(D, 1, BH, a, c->cfg.outlier_frac, s)) != QAQ_OK) return stt;
     }
     c->tokens = t1;
     return QAQ_OK;
@@ -1016,6 +657,5 @@ extern "C" qaq_status qaq_stream_append(qaq_cache* c, const void* k_new, const v
     a.k = c->t[0]; a.v = c->t[1]; a.pool_bytes = c->pool_bytes; a.ocap = c->ocap;
     a.tmax_pad = c->tmax_pad; a.ntiles = c->ntiles; a.status = c->d_status;
     a.d_count = qaq_d_count(c); a.d_ticket = qaq_d_ticket(c); a.max_tokens = (int)c->cfg.max_tokens;
-    st = launch<false>(D, dim3(1, c->BH), a, (cudaStream_t)stream);
-    return st;
+    return launch<true>(D, 1, c->BH, a, c->cfg.outlier_frac, (cudaStream_t)stream);
 }

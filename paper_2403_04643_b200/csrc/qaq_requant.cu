@@ -80,38 +80,10 @@ __device__ __forceinline__ void drop_bits(uint32_t (&lo)[4], uint32_t (&hi)[4], 
         hi[u] = (hi[u] >> d) & keep;
     }
 }
-// The nibble words of one part (w bits, 1..4) of a lane's 32 channels of one token.  Keys: the unit at `at`; values: byte i of
-// units 4p .. 4p+3, which lie m units apart from `at` on.
-template <int W, bool IS_V>
-__device__ __forceinline__ void take_words(const uint8_t* at, uint32_t m, int i, uint32_t (&v)[4]) {
-    uint32_t x[W];
-    if (!IS_V) {
-        qaqc::load_words<W>(at, x);
-    } else {
-        uint32_t u[4][W];
-#pragma unroll
-        for (int b = 0; b < 4; ++b) qaqc::load_words<W>(at + b * m * 4 * W, u[b]);
-        const uint32_t sel = 0x0040u + 0x0011u * (uint32_t)i;          // byte i of both operands
-#pragma unroll
-        for (int c = 0; c < W; ++c) x[c] = qaqc::prmt(qaqc::prmt(u[0][c], u[1][c], sel), qaqc::prmt(u[2][c], u[3][c], sel), 0x5410u);
-    }
-    qaqc::nibble_words<W>(x, v);
-    constexpr uint32_t mask = 0x11111111u * ((1u << W) - 1u);
-#pragma unroll
-    for (int k = 0; k < 4; ++k) v[k] &= mask;
-}
-template <bool IS_V>
-__device__ __forceinline__ void take_part(const uint8_t* at, int w, uint32_t m, int i, uint32_t (&v)[4]) {
-    if (w == 4) take_words<4, IS_V>(at, m, i, v);
-    else if (w == 3) take_words<3, IS_V>(at, m, i, v);
-    else if (w == 2) take_words<2, IS_V>(at, m, i, v);
-    else take_words<1, IS_V>(at, m, i, v);
-}
-
 // What the CTA keeps of its tile.
 template <int D>
 struct RequantScratch {
-    alignas(16) uint8_t old[qaqc::tile_bytes_max(D)];
+    alignas(16) uint8_t old[qaqc::tile_bytes_max(D) + 16];
     // by new slot: byte offsets of the row's parts before | and after << 16 (main, high); token, widths before and after, row
     // widths before and after; for values the distances of the units and the old slot's place in its group
     alignas(16) uint4 slot[QAQ_TILE];
@@ -248,16 +220,7 @@ __device__ __forceinline__ void requantize_tile(const RequantArgs& a, RequantScr
                 qaqc::nibbles_of(creg, 0, lo);
                 qaqc::nibbles_of(creg, 4, hi);
             } else {
-                const int wm = min(ow, 4);
-                constexpr uint32_t LAST = sizeof(sm.old) - 16;      // whatever the metadata say, nothing beyond the buffer is read
-                const uint32_t mm = q.w & 15u, mh = (q.w >> 4) & 15u;
-                const int i = (int)((q.w >> 16) & 3u);
-                const uint32_t m_at = (q.x & 0xFFFFu) + (IS_V ? 4 * p * mm : (uint32_t)p) * 4 * wm, m_end = m_at + (IS_V ? 3 * mm * 4 * wm : 0u);
-                if (m_end <= LAST) take_part<IS_V>(sm.old + m_at, wm, mm, i, lo);
-                if (ow > 4) {
-                    const uint32_t h_at = (q.y & 0xFFFFu) + (IS_V ? 4 * p * mh : (uint32_t)p) * 4 * (ow - 4), h_end = h_at + (IS_V ? 3 * mh * 4 * (ow - 4) : 0u);
-                    if (h_end <= LAST) take_part<IS_V>(sm.old + h_at, ow - 4, mh, i, hi);
-                }
+                qaqc::take_token<D, IS_V>(sm.old, sizeof(sm.old), q.x & 0xFFFFu, q.y & 0xFFFFu, ow, q.w & 15u, (q.w >> 4) & 15u, (int)((q.w >> 16) & 3u), p, lo, hi);
                 drop_bits(lo, hi, bo - bn);
             }
         }
