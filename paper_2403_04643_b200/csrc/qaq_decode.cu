@@ -154,6 +154,7 @@ struct DecArgs {
     unsigned long long tag;      // of this call; the low 12 bits are zero
     float* ml;         // [BH][2]   merged (max, sum) for the normalisation of long score rows, or null
     int BH, run, ncta; // (b,h) count; tiles per CTA of the flattened (b,h, tile) sequence; CTAs
+    int cluster;       // CTAs per (b,h), a thread-block cluster, or 0: runs of the flattened sequence
     int nq, groups;    // queries of the launch and groups of NQ of them; blockIdx.y is the group (the last one may be short of queries)
     float* out;
     float* scores;     // [BH][scores_stride] or null (one query only)
@@ -195,6 +196,20 @@ struct Group {
         nq = min(NQ, a.nq - g * NQ);
     }
 };
+
+// Short sequences: the CTAs of a (b,h) are a thread-block cluster, with as many tiles each, and their results meet in shared
+// memory.  (Through memory - partials stored, CTAs counted by an atomic, partials loaded by the last one - a split costs 3 to
+// 4 us: 32 (b,h) of 8 tiles, one CTA each, 8.3 us, of 9 tiles 12.4.)  Taken where a portable cluster makes no warp do
+// more tiles than the flattened sequence would.  Returns the size of the cluster, 0: the flattened sequence.
+template <int NQ>
+inline int plan_cluster(int BH, int ntiles, int groups) {
+    using S = Shape<NQ>;
+    const int places = S::SLOTS / groups / BH;               // CTAs a (b,h) can have at once
+    const int k = min(min(8, places), (ntiles + S::WARPS - 1) / S::WARPS);
+    if (k < 2) return 0;
+    const int run = plan_decode<NQ>(BH, ntiles, groups).run, crun = (ntiles + k - 1) / k;
+    return (crun + S::WARPS - 1) / S::WARPS <= (run + S::WARPS - 1) / S::WARPS ? k : 0;
+}
 
 // ------------------------------------------------------------------------------------------ shared memory
 // per-warp scratch for the tile a warp is working on
@@ -515,11 +530,51 @@ __device__ void merge_split(const DecArgs& a, DecSmem<D, NQ>& sm, int bh, int nt
     }
 }
 
+// The same for the CTAs of a cluster, which find each other's results in shared memory: query j is put together by CTA
+// j mod cluster; every CTA normalises the scores of its own tiles (from tile_lo to tile_hi).
+__device__ __forceinline__ void cluster_barrier() {
+    asm volatile("barrier.cluster.arrive.release.aligned;\nbarrier.cluster.wait.acquire.aligned;" ::: "memory");
+}
+__device__ __forceinline__ float peer_load(const float* p, int rank) {
+    float x;
+    asm volatile("{\n.reg .u32 a;\nmapa.shared::cluster.u32 a, %1, %2;\nld.shared::cluster.f32 %0, [a];\n}" : "=f"(x) : "r"(smem_addr(p)), "r"(rank) : "memory");
+    return x;
+}
+template <int D, int NQ>
+__device__ __forceinline__ void merge_cluster(const DecArgs& a, DecSmem<D, NQ>& sm, const Group<D, NQ>& gr, int bh, int rank, int tile_lo, int tile_hi, int T) {
+    using S = Shape<NQ>;
+    const float NEG = __int_as_float(0xff800000);
+    const int tid = threadIdx.x, lane = tid & 31, ncl = a.cluster;
+    cluster_barrier();
+#pragma unroll 1
+    for (int j = 0; j < gr.nq; ++j) {
+        if (j % ncl != rank && !(NQ == 1 && (a.scores || a.ml))) continue;
+        float m = NEG, l = 0.f;
+        if (lane < ncl) { m = peer_load(&sm.mm[S::WARPS][j], lane); l = peer_load(&sm.ml[S::WARPS][j], lane); }
+        const float M = warp_max(m), w = m == NEG ? 0.f : __expf(m - M), L = warp_sum(w * l);
+        if (j % ncl == rank) {
+            float x[8], sum = 0.f;
+            const int d = tid < D ? tid : 0;
+#pragma unroll
+            for (int i = 0; i < 8; ++i) x[i] = i < ncl ? peer_load(&sm.cross[j][d], i) : 0.f;
+#pragma unroll
+            for (int i = 0; i < 8; ++i) sum = fmaf(__shfl_sync(0xFFFFFFFFu, w, i), x[i], sum);
+            if (tid < D) gr.out[(size_t)bh * a.out_stride + j * D + tid] = L > 0.f ? sum / L : 0.f;
+            if (NQ == 1 && a.ml && tid == 0) { a.ml[2 * bh] = M; a.ml[2 * bh + 1] = L; }
+        }
+        if (NQ == 1 && a.scores && !a.ml)
+            normalise_scores<S::THREADS>(a.scores + (size_t)bh * a.scores_stride + tile_lo * QAQ_TILE, min(tile_hi * QAQ_TILE, T) - tile_lo * QAQ_TILE, M, L);
+    }
+    cluster_barrier();                  // nobody leaves while its results are being read
+}
+
 // A CTA's run meets one or two (b,h); it leaves one partial for each, or the result where a (b,h) is one CTA's alone.
 // In the loops over lists lane 4g+t is lane (g, t) of the tensor-core fragments.
 // COUNTED: the token count is read from device memory and the split derived from it here (the grid is then the
 // largest one any count needs; CTAs beyond the split find no tiles and leave).
-template <int D, int NQ, bool COUNTED>
+// CLUSTER: the CTAs of a (b,h) are a cluster (a kernel of its own: decided at run time, 256 (b,h) of 4096 tokens took
+// 52.7 us instead of 50.4).
+template <int D, int NQ, bool COUNTED, bool CLUSTER>
 __global__ void __launch_bounds__(Shape<NQ>::THREADS, Shape<NQ>::CTAS_PER_SM) decode_kernel(const DecArgs a) {
     using S = Shape<NQ>;
     using WS = WarpScratch<D, NQ>;
@@ -545,11 +600,18 @@ __global__ void __launch_bounds__(Shape<NQ>::THREADS, Shape<NQ>::CTAS_PER_SM) de
     }
     // this CTA's run of the flattened (b,h, tile) sequence: it begins in bh0 and may reach into bh0 + 1, which begins at f_bound
     const int ntiles = (T + QAQ_TILE - 1) / QAQ_TILE;
-    const int run = COUNTED ? plan_decode<NQ>(a.BH, ntiles, 1).run : a.run;
-    const int flat_lo = blockIdx.x * run, flat_hi = min(a.BH * ntiles, flat_lo + run);
-    if (flat_lo >= flat_hi) return;
-    const int bh0 = flat_lo / ntiles, f_bound = (bh0 + 1) * ntiles;
-    const int nseg = flat_hi > f_bound ? 2 : 1;
+    const int ncl = CLUSTER ? a.cluster : 0, rank = CLUSTER ? blockIdx.x % ncl : 0;
+    const int run = CLUSTER ? (ntiles + ncl - 1) / ncl : COUNTED ? plan_decode<NQ>(a.BH, ntiles, 1).run : a.run;
+    int flat_lo = blockIdx.x * run, bh0;
+    if (CLUSTER) {
+        bh0 = blockIdx.x / ncl;
+        flat_lo = bh0 * ntiles + min(rank * run, ntiles);    // the last CTAs of a cluster may find no tiles
+    } else {
+        if (flat_lo >= a.BH * ntiles) return;
+        bh0 = flat_lo / ntiles;
+    }
+    const int f_bound = (bh0 + 1) * ntiles, flat_hi = min(CLUSTER ? f_bound : a.BH * ntiles, flat_lo + run);
+    const int nseg = !CLUSTER && flat_hi > f_bound ? 2 : 1;
     // this warp's piece of it
     const int piece = (run + S::WARPS - 1) / S::WARPS;
     int f = flat_lo + warp * piece;
@@ -628,7 +690,7 @@ __global__ void __launch_bounds__(Shape<NQ>::THREADS, Shape<NQ>::CTAS_PER_SM) de
     }
     __syncwarp();
     if (f < f_end) stage(buf, layout(tk), a.k, bh_of(f), tk, 0);
-    if (lane == 0 && warp < nseg) {
+    if (lane == 0 && warp < nseg && !CLUSTER) {
         int first, n;
         split_of(bh0 + warp, ntiles, run, first, n);
         if (n > 1) open_count(gr.done + bh0 + warp, a.tag);
@@ -1056,7 +1118,7 @@ __global__ void __launch_bounds__(Shape<NQ>::THREADS, Shape<NQ>::CTAS_PER_SM) de
 #pragma unroll 1
     for (int seg = 0; seg < nseg; ++seg) {
         const int bh = bh0 + seg;
-        const bool alone = min(flat_hi, (bh + 1) * ntiles) - max(flat_lo, bh * ntiles) == ntiles;        // nothing to merge with
+        const bool alone = !CLUSTER && min(flat_hi, (bh + 1) * ntiles) - max(flat_lo, bh * ntiles) == ntiles;        // nothing to merge with
         const bool mine = lane <= S::WARPS && sm.seg[min(lane, S::WARPS)] == seg;
 #pragma unroll 1
         for (int j = 0; j < gr.nq; ++j) {
@@ -1075,11 +1137,18 @@ __global__ void __launch_bounds__(Shape<NQ>::THREADS, Shape<NQ>::CTAS_PER_SM) de
                     if (a.ml && tid == 0) { a.ml[2 * bh] = M; a.ml[2 * bh + 1] = L; }
                     if (a.scores && !a.ml) normalise_scores<S::THREADS>(a.scores + (size_t)bh * a.scores_stride, T, M, L);
                 }
+            } else if (CLUSTER) {          // (entry W is free: no warp crosses into another (b,h))
+                if (tid < D) sm.cross[j][tid] = x;
+                if (tid == 0) { sm.mm[S::WARPS][j] = M; sm.ml[S::WARPS][j] = L; }
             } else {
                 if (tid < D) __stcg(dst + tid, x);
                 if (tid == 0) __stcg(reinterpret_cast<float2*>(dst + D), make_float2(M, L));
             }
         }
+    }
+    if (CLUSTER) {
+        merge_cluster<D, NQ>(a, sm, gr, bh0, rank, flat_lo - bh0 * ntiles, flat_hi - bh0 * ntiles, T);
+        return;
     }
     __syncthreads();
     if (lane == 0 && warp < nseg) {
@@ -1127,9 +1196,15 @@ template <int D, int NQ, bool COUNTED>
 qaq_status launch_decode(const DecArgs& a, cudaStream_t s) {
     const size_t smem = sizeof(DecSmem<D, NQ>);
     static_assert(sizeof(DecSmem<D, NQ>) + 1024 <= 227 * 1024 / Shape<NQ>::CTAS_PER_SM, "shared memory of the CTAs of an SM");
-    static std::atomic<unsigned long long> seen{0};
-    QAQ_CUDA_TRY(qaq_allow_smem((const void*)decode_kernel<D, NQ, COUNTED>, smem, seen));
-    QAQ_CUDA_TRY(qaq_launch(decode_kernel<D, NQ, COUNTED>, dim3(a.ncta, a.groups), dim3(Shape<NQ>::THREADS), smem, s, a));
+    static std::atomic<unsigned long long> seen[2];
+    const dim3 grid(a.ncta, a.groups), block(Shape<NQ>::THREADS);
+    if (a.cluster) {
+        QAQ_CUDA_TRY(qaq_allow_smem((const void*)decode_kernel<D, NQ, COUNTED, true>, smem, seen[1]));
+        QAQ_CUDA_TRY(qaq_launch_cluster(decode_kernel<D, NQ, COUNTED, true>, grid, block, a.cluster, smem, s, a));
+    } else {
+        QAQ_CUDA_TRY(qaq_allow_smem((const void*)decode_kernel<D, NQ, COUNTED, false>, smem, seen[0]));
+        QAQ_CUDA_TRY(qaq_launch(decode_kernel<D, NQ, COUNTED, false>, grid, block, smem, s, a));
+    }
     if (NQ == 1 && a.ml) {
         int gx = (a.T + 1023) / 1024;     // counted: a.T holds the capacity
         if (gx > 64) gx = 64;
@@ -1157,6 +1232,8 @@ qaq_status decode(const qaq_cache* c, const void* q, long q_stride, float softma
     a.BH = BH;
     a.run = COUNTED ? 0 : plan.run;
     a.ncta = COUNTED ? (BH > Shape<NQ>::SLOTS ? BH : Shape<NQ>::SLOTS) : plan.ncta;   // counted: the largest grid any count needs
+    a.cluster = plan_cluster<NQ>(BH, (a.T + QAQ_TILE - 1) / QAQ_TILE, a.groups);
+    if (a.cluster) a.ncta = BH * a.cluster;
     // nothing in the workspace is read before it is written (the counting words: see finish_split)
     a.part = (float*)ws;
     a.done = (unsigned long long*)(a.part + (size_t)(BH > Shape<NQ>::SLOTS ? 0 : 2 * Shape<NQ>::SLOTS) * NQ * (D + 4));

@@ -70,14 +70,21 @@ static inline unsigned* qaq_d_ticket(const qaq_cache* c) { return (unsigned*)(c-
 __device__ __forceinline__ void qaq_dependency() {
     asm volatile("griddepcontrol.wait;" ::: "memory");
 }
+// cluster: CTAs (consecutive in x) that form a thread-block cluster
 template <typename... P, typename... A>
-static inline cudaError_t qaq_launch(void (*kernel)(P...), dim3 grid, dim3 block, size_t smem, cudaStream_t s, A... args) {
-    cudaLaunchAttribute at[1];
+static inline cudaError_t qaq_launch_cluster(void (*kernel)(P...), dim3 grid, dim3 block, int cluster, size_t smem, cudaStream_t s, A... args) {
+    cudaLaunchAttribute at[2];
     at[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
     at[0].val.programmaticStreamSerializationAllowed = 1;
+    at[1].id = cudaLaunchAttributeClusterDimension;
+    at[1].val.clusterDim.x = (unsigned)cluster; at[1].val.clusterDim.y = 1; at[1].val.clusterDim.z = 1;
     cudaLaunchConfig_t lc = {};
-    lc.gridDim = grid; lc.blockDim = block; lc.dynamicSmemBytes = smem; lc.stream = s; lc.attrs = at; lc.numAttrs = 1;
+    lc.gridDim = grid; lc.blockDim = block; lc.dynamicSmemBytes = smem; lc.stream = s; lc.attrs = at; lc.numAttrs = cluster > 1 ? 2 : 1;
     return cudaLaunchKernelEx(&lc, kernel, P(args)...);
+}
+template <typename... P, typename... A>
+static inline cudaError_t qaq_launch(void (*kernel)(P...), dim3 grid, dim3 block, size_t smem, cudaStream_t s, A... args) {
+    return qaq_launch_cluster(kernel, grid, block, 1, smem, s, args...);
 }
 // Shared memory beyond 48 KB has to be allowed once per kernel and device; `seen` (one per kernel) remembers where that
 // has been done (devices 0..63; others are asked every time).
