@@ -600,10 +600,10 @@ __global__ void __launch_bounds__(Shape<NQ>::THREADS, Shape<NQ>::CTAS_PER_SM) de
     }
     // this CTA's run of the flattened (b,h, tile) sequence: it begins in bh0 and may reach into bh0 + 1, which begins at f_bound
     const int ntiles = (T + QAQ_TILE - 1) / QAQ_TILE;
-    const int ncl = CLUSTER ? a.cluster : 0, rank = CLUSTER ? blockIdx.x % ncl : 0;
+    const int ncl = CLUSTER ? a.cluster : 1, rank = CLUSTER ? blockIdx.x % ncl : 0;
     const int run = CLUSTER ? (ntiles + ncl - 1) / ncl : COUNTED ? plan_decode<NQ>(a.BH, ntiles, 1).run : a.run;
     int flat_lo = blockIdx.x * run, bh0;
-    if (CLUSTER) {
+    if constexpr (CLUSTER) {
         bh0 = blockIdx.x / ncl;
         flat_lo = bh0 * ntiles + min(rank * run, ntiles);    // the last CTAs of a cluster may find no tiles
     } else {

@@ -397,6 +397,15 @@ __global__ void __launch_bounds__(PC_WARPS * 32, PC_MINCTA) window_cluster_kerne
 }
 
 template <int D>
+qaq_status run_cluster(const PrefillArgs& a, int BH, int ncl, size_t smem, cudaStream_t s) {
+    static std::atomic<unsigned long long> seen{0};
+    const size_t most = (size_t)PW_MAXQ * PC_PITCH * sizeof(float) + 4 * (D / 16) * 32 * sizeof(uint4);
+    QAQ_CUDA_TRY(qaq_allow_smem((const void*)window_cluster_kernel<D>, most, seen));
+    QAQ_CUDA_TRY(qaq_launch_cluster(window_cluster_kernel<D>, dim3((unsigned)ncl, (unsigned)BH), dim3(PC_WARPS * 32), ncl, smem, s, a));
+    return QAQ_OK;
+}
+
+template <int D>
 qaq_status run_long(const PrefillArgs& a, int BH, cudaStream_t s) {
     const dim3 grid((unsigned)a.nchunk, (unsigned)BH);
     const size_t smem = (size_t)(2 * ((a.n + 31) / 32)) * (D / 16) * 32 * sizeof(uint4);       // at most 16 KB
@@ -496,31 +505,13 @@ extern "C" qaq_status qaq_prefill_window(const qaq_config* cfg, const void* Q, c
         // one pass: the CTAs of a (b,h) are one cluster
         const size_t smem = (size_t)cfg->window * PC_PITCH * sizeof(float) +
                             (size_t)(2 * ((cfg->window + 31) / 32)) * (cfg->head_dim / 16) * 32 * sizeof(uint4);   // logits, query fragments
-        cudaLaunchConfig_t lc = {};
-        lc.gridDim = dim3((unsigned)ncl, (unsigned)(cfg->batch * cfg->heads));
-        lc.blockDim = dim3(PC_WARPS * 32);
-        lc.dynamicSmemBytes = smem;
-        lc.stream = s;
-        cudaLaunchAttribute at[2];
-        at[1].id = cudaLaunchAttributeProgrammaticStreamSerialization;
-        at[1].val.programmaticStreamSerializationAllowed = 1;
-        at[0].id = cudaLaunchAttributeClusterDimension;
-        at[0].val.clusterDim.x = (unsigned)ncl; at[0].val.clusterDim.y = 1; at[0].val.clusterDim.z = 1;
-        lc.attrs = at; lc.numAttrs = 2;
+        const int BH = cfg->batch * cfg->heads;
         switch (cfg->head_dim) {
-            case 32:
-                QAQ_CUDA_TRY(cudaFuncSetAttribute(window_cluster_kernel<32>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem));
-                QAQ_CUDA_TRY(cudaLaunchKernelEx(&lc, window_cluster_kernel<32>, a)); break;
-            case 64:
-                QAQ_CUDA_TRY(cudaFuncSetAttribute(window_cluster_kernel<64>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem));
-                QAQ_CUDA_TRY(cudaLaunchKernelEx(&lc, window_cluster_kernel<64>, a)); break;
-            case 128:
-                QAQ_CUDA_TRY(cudaFuncSetAttribute(window_cluster_kernel<128>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem));
-                QAQ_CUDA_TRY(cudaLaunchKernelEx(&lc, window_cluster_kernel<128>, a)); break;
-            default: return QAQ_ERR_UNSUPPORTED_SHAPE;
+            case 32: return run_cluster<32>(a, BH, ncl, smem, s);
+            case 64: return run_cluster<64>(a, BH, ncl, smem, s);
+            case 128: return run_cluster<128>(a, BH, ncl, smem, s);
         }
-        QAQ_CUDA_TRY(cudaGetLastError());
-        return QAQ_OK;
+        return QAQ_ERR_UNSUPPORTED_SHAPE;
     }
     switch (cfg->head_dim) {
         case 32: return run_long<32>(a, cfg->batch * cfg->heads, s);

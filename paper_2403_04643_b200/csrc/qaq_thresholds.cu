@@ -18,11 +18,8 @@
 namespace {
 
 constexpr int SAMPLE_TOKENS = 64;
-#ifndef QWARP_FLAGS
-#define QWARP_FLAGS 192
-#endif
 constexpr int SCAN_TOKENS_MAX = 512; // tokens per CTA of the scan (fewer where alpha is large: see scan_tokens_for)
-constexpr int WARP_FLAGS = QWARP_FLAGS;      // 16-byte pieces a warp of the scan can set aside before it has to look at them
+constexpr int WARP_FLAGS = 192;      // 16-byte pieces a warp of the scan can set aside before it has to look at them
 constexpr int CTA_LIST = 4096;       // candidates per tail a scan CTA can hold
 constexpr int SELECT_KEYS = 16384;   // candidates of one tail the select kernel keeps in shared memory
 
@@ -139,8 +136,10 @@ __device__ uint32_t cta_select(Get get, uint32_t n, uint32_t want, uint32_t* his
 // counts here, NaN patterns too: as keys they sort below -inf (sign set) or above +inf, so a caller
 // whose ranks are meant among the non-NaN values adds the number of negative NaNs to them.
 // s_tmp: 4 words.
+template <int THREADS = 256>
 __device__ void cta_select_keys(const unsigned short* keys, uint32_t n, uint32_t wantA, uint32_t wantB, uint32_t* hist,
                                 uint32_t* s_tmp, uint32_t& outA, uint32_t& outB) {
+    constexpr int BINS = 2048 / THREADS;                     // of a thread
     const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
     const uint4* k8 = reinterpret_cast<const uint4*>(keys);
     const uint32_t n8 = (n + 7) / 8;
@@ -157,9 +156,9 @@ __device__ void cta_select_keys(const unsigned short* keys, uint32_t n, uint32_t
         }
     }
     __syncthreads();
-    uint32_t c[8], tot = 0;
+    uint32_t c[BINS], tot = 0;
 #pragma unroll
-    for (int j = 0; j < 8; ++j) { c[j] = hist[8 * threadIdx.x + j]; tot += c[j]; }
+    for (int j = 0; j < BINS; ++j) { c[j] = hist[BINS * threadIdx.x + j]; tot += c[j]; }
     uint32_t inc = tot;
 #pragma unroll
     for (int d = 1; d < 32; d <<= 1) {
@@ -171,12 +170,12 @@ __device__ void cta_select_keys(const unsigned short* keys, uint32_t n, uint32_t
     __syncthreads();
     uint32_t before = 0, all = 0;
 #pragma unroll
-    for (int w = 0; w < 8; ++w) {
+    for (int w = 0; w < THREADS / 32; ++w) {
         const uint32_t v = hist[w];
         if (w < warp) before += v;
         all += v;
     }
-    const uint32_t first = before + inc - tot;               // keys in the bins before this thread's eight
+    const uint32_t first = before + inc - tot;               // keys in the bins before this thread's
 #pragma unroll
     for (int r = 0; r < 2; ++r) {
         const uint32_t want = r ? wantB : wantA;
@@ -185,11 +184,11 @@ __device__ void cta_select_keys(const unsigned short* keys, uint32_t n, uint32_t
             uint32_t acc = first;
             int bsel = 0;
 #pragma unroll
-            for (int j = 0; j < 8; ++j) {
-                if (w2 >= acc + c[j] && j < 7) { acc += c[j]; bsel = j + 1; }
+            for (int j = 0; j < BINS; ++j) {
+                if (w2 >= acc + c[j] && j < BINS - 1) { acc += c[j]; bsel = j + 1; }
                 else break;
             }
-            s_tmp[2 * r] = (uint32_t)(8 * threadIdx.x + bsel);
+            s_tmp[2 * r] = (uint32_t)(BINS * threadIdx.x + bsel);
             s_tmp[2 * r + 1] = w2 - acc;
         }
     }
@@ -236,6 +235,23 @@ __device__ __forceinline__ unsigned long long rank_k(double alpha, unsigned long
     return k;
 }
 
+// binary16 pair -> pair of keys (a set sign flips all 16 bits, a clear one only the sign bit); NaNs are counted
+__device__ __forceinline__ uint32_t keys_of(uint32_t w, uint32_t& nn, uint32_t& nneg) {
+    const uint32_t mag = w & 0x7FFF7FFFu;
+    const uint32_t nan_lo = (mag & 0xFFFFu) > 0x7C00u, nan_hi = (mag >> 16) > 0x7C00u;
+    nn += nan_lo + nan_hi;
+    nneg += (nan_lo & (w >> 15)) + (nan_hi & (w >> 31));
+    return w ^ (((w >> 15) & 0x00010001u) * 0xFFFFu | 0x80008000u);
+}
+// Rank of 1.25 times the wanted tail mass plus four standard deviations of the count in a sample of M (a wider bracket
+// makes the scan set aside more pieces: 2.0 times costs 7 % more time on stationary data; a bracket that
+// turns out too tight only sends that problem to the exact two-pass select).
+__device__ __forceinline__ uint32_t bracket_rank(double alpha, uint32_t M) {
+    const double f2 = 1.25 * 0.5 * alpha * (double)M;
+    const uint32_t r = (uint32_t)ceil(f2 + 4.0 * sqrt(f2 + 1.0) + 2.0);
+    return r > (M - 1) / 2 ? (M - 1) / 2 : r;
+}
+
 // ---- 1. sample: brackets (or the exact answer when the sample is the whole problem)
 __global__ void __launch_bounds__(256) thr_sample_kernel(const ThrArgs a) {
     qaq_dependency();
@@ -249,21 +265,22 @@ __global__ void __launch_bounds__(256) thr_sample_kernel(const ThrArgs a) {
     if (threadIdx.x < 2) s_cnt[threadIdx.x] = 0;
     __syncthreads();
     uint32_t nn = 0, nneg = 0;                                  // NaNs, NaNs with the sign set
-    for (int i = threadIdx.x; i < M / 8; i += blockDim.x) {    // 16-byte pieces
-        const int s = (i * 8) / a.D, c = (i * 8) % a.D;
-        const long t = (long)s * a.T / ns;                        // tokens spread over the sequence
-        const uint4 r = *reinterpret_cast<const uint4*>(X + (size_t)t * a.st + c);
-        uint32_t w[4] = {r.x, r.y, r.z, r.w};
+    // all 16-byte pieces of a thread (four at most) are on their way before the first is looked at
+    uint4 raw[4];
 #pragma unroll
-        for (int j = 0; j < 4; ++j) {
-            const uint32_t mag = w[j] & 0x7FFF7FFFu;
-            const uint32_t nan_lo = (mag & 0xFFFFu) > 0x7C00u, nan_hi = (mag >> 16) > 0x7C00u;
-            nn += nan_lo + nan_hi;
-            nneg += (nan_lo & (w[j] >> 15)) + (nan_hi & (w[j] >> 31));
-            // keys of both halves: a set sign flips all 16 bits, a clear one only the sign bit
-            const uint32_t neg = ((w[j] >> 15) & 0x00010001u) * 0xFFFFu;
-            w[j] ^= neg | 0x80008000u;
-        }
+    for (int k = 0; k < 4; ++k) {
+        const int i = min((int)threadIdx.x + 256 * k, M / 8 - 1);
+        const int sp = (i * 8) / a.D, c = (i * 8) % a.D;
+        const long t = (long)sp * a.T / ns;                       // tokens spread over the sequence
+        raw[k] = *reinterpret_cast<const uint4*>(X + (size_t)t * a.st + c);
+    }
+#pragma unroll
+    for (int k = 0; k < 4; ++k) {
+        const int i = threadIdx.x + 256 * k;
+        if (i >= M / 8) break;
+        uint32_t w[4] = {raw[k].x, raw[k].y, raw[k].z, raw[k].w};
+#pragma unroll
+        for (int j = 0; j < 4; ++j) w[j] = keys_of(w[j], nn, nneg);
         *reinterpret_cast<uint4*>(&s_keys[8 * i]) = make_uint4(w[0], w[1], w[2], w[3]);
     }
     if (nn) { atomicAdd(&s_cnt[0], nn); atomicAdd(&s_cnt[1], nneg); }
@@ -284,12 +301,7 @@ __global__ void __launch_bounds__(256) thr_sample_kernel(const ThrArgs a) {
         const unsigned long long k = rank_k(a.alpha, Mv);
         r_lo = (uint32_t)k; r_hi = (uint32_t)(Mv - 1 - k);
     } else {
-        // rank of 1.25 times the wanted tail mass plus four standard deviations of the sample count (a wider bracket
-        // makes the scan set aside more pieces: 2.0 times costs 7 % more time on stationary data; a bracket that
-        // turns out too tight only sends that problem to the exact two-pass select)
-        const double f2 = 1.25 * 0.5 * a.alpha * (double)Mv;
-        uint32_t r = (uint32_t)ceil(f2 + 4.0 * sqrt(f2 + 1.0) + 2.0);
-        if (r > (Mv - 1) / 2) r = (Mv - 1) / 2;
+        const uint32_t r = bracket_rank(a.alpha, Mv);
         r_lo = r; r_hi = Mv - 1 - r;
     }
     uint32_t klo, khi;
@@ -468,7 +480,7 @@ __global__ void __launch_bounds__(256) thr_select_kernel(const ThrArgs a) {
                 res = float_of_key(key);
             } else {
                 // a longer list is read twice where it lies, eight keys at a time (one at a time: 124 us for 640 lists of
-                // 52000 keys, eight: see the launch)
+                // 52000 keys, eight: 43 us)
                 uint32_t key, same;
                 cta_select_keys(l, c, want, want, hist, s_tmp, key, same);
                 res = float_of_key(key);
@@ -488,12 +500,113 @@ __global__ void __launch_bounds__(256) thr_select_kernel(const ThrArgs a) {
     if (threadIdx.x == 0) a.thr[(size_t)bh * 4 + 2 * x + side] = res;
 }
 
+// ---- short sequences: the three steps by one CTA per problem, on keys that stay in shared memory.
+// The chain of three launches is latency: 32 (b,h) of 100 tokens 16.8 us, this kernel 13.8; 256 (b,h) 33.8 against 23.4 us;
+// but 32 of 333 tokens 17.5 against 25.4 us (19 with 1024 threads, which are slower at 100 tokens of many (b,h)).
+constexpr uint32_t SMALL_KEYS = 16384;     // keys of a problem at most
+constexpr uint32_t SMALL_LIST = 4096;      // candidates of a tail at most
+constexpr int SMALL_THREADS = 256;
+struct SmallScratch {
+    uint32_t hist[2048], tmp[4], n[2], cnt[4];
+    alignas(16) unsigned short list[2 * SMALL_LIST];       // the sample, then the candidates
+    alignas(16) unsigned short keys[8];                    // T * D of them
+};
+__global__ void __launch_bounds__(SMALL_THREADS) thr_small_kernel(const ThrArgs a) {
+    extern __shared__ __align__(16) unsigned char small_smem[];
+    SmallScratch& sm = *reinterpret_cast<SmallScratch*>(small_smem);
+    static_assert(2 * SMALL_LIST >= SAMPLE_TOKENS * 128, "the sample fits the list");
+    const int bhx = blockIdx.x, bh = bhx >> 1, x = bhx & 1, tid = threadIdx.x;
+    if (tid < 4) sm.cnt[tid] = 0;
+    if (tid < 2) sm.n[tid] = 0;
+    __syncthreads();
+    qaq_dependency();
+    const int shift = 31 - __clz(a.D / 8);                 // 16-byte pieces per token
+    const uint32_t total = (uint32_t)a.T * (uint32_t)a.D, n8 = total / 8;
+    const __half* X = a.X[x] + (size_t)(bh / a.H) * a.sb + (size_t)(bh % a.H) * a.sh;
+    uint4* keys = reinterpret_cast<uint4*>(sm.keys);
+    uint32_t nn = 0, nneg = 0;                             // NaNs, NaNs with the sign set
+    for (uint32_t i0 = tid; i0 < n8; i0 += 8 * SMALL_THREADS) {
+        uint4 raw[8];
+#pragma unroll
+        for (int u = 0; u < 8; ++u) {
+            const uint32_t i = min(i0 + SMALL_THREADS * u, n8 - 1);
+            raw[u] = *reinterpret_cast<const uint4*>(X + (size_t)(i >> shift) * a.st + ((i & ((1u << shift) - 1)) << 3));
+        }
+#pragma unroll
+        for (int u = 0; u < 8; ++u) {
+            if (i0 + SMALL_THREADS * u >= n8) break;
+            uint32_t w[4] = {raw[u].x, raw[u].y, raw[u].z, raw[u].w};
+#pragma unroll
+            for (int j = 0; j < 4; ++j) w[j] = keys_of(w[j], nn, nneg);
+            keys[i0 + SMALL_THREADS * u] = make_uint4(w[0], w[1], w[2], w[3]);
+        }
+    }
+    if (nn) { atomicAdd(&sm.cnt[0], nn); atomicAdd(&sm.cnt[1], nneg); }
+    __syncthreads();
+    const uint32_t N = total - sm.cnt[0], neg_nan = sm.cnt[1];
+    float* thr = a.thr + (size_t)bh * 4 + 2 * x;
+    if (N == 0) {
+        if (tid < 2) thr[tid] = 0.f;
+        return;
+    }
+    const uint32_t k = (uint32_t)rank_k(a.alpha, N);
+    // the sample, brackets from it; its NaNs only make a bracket wider or tighter than meant
+    constexpr uint32_t NS = SAMPLE_TOKENS;
+    const uint32_t M = NS * (uint32_t)a.D;
+    for (uint32_t i = tid; i < M / 8; i += SMALL_THREADS) {
+        const uint32_t t = (uint32_t)((unsigned long long)(i >> shift) * a.T / NS);
+        reinterpret_cast<uint4*>(sm.list)[i] = keys[(t << shift) + (i & ((1u << shift) - 1))];
+    }
+    __syncthreads();
+    const uint32_t r = bracket_rank(a.alpha, M);
+    uint32_t klo, khi;
+    cta_select_keys<SMALL_THREADS>(sm.list, M, r, M - 1 - r, sm.hist, sm.tmp, klo, khi);
+    // candidates (no NaNs: their keys lie below that of -inf and above that of +inf)
+    const uint32_t first = key_of(0xFC00u), last = key_of(0x7C00u);
+    for (uint32_t i = tid; i < n8; i += SMALL_THREADS) {
+        const uint4 q = keys[i];
+        const uint32_t w[4] = {q.x, q.y, q.z, q.w};
+#pragma unroll
+        for (int j = 0; j < 8; ++j) {
+            const uint32_t key = (w[j >> 1] >> (16 * (j & 1))) & 0xFFFFu;
+            if (key < klo && key >= first) {
+                const uint32_t at = atomicAdd(&sm.n[0], 1u);
+                if (at < SMALL_LIST) sm.list[at] = (unsigned short)key;
+            }
+            if (key > khi && key <= last) {
+                const uint32_t at = atomicAdd(&sm.n[1], 1u);
+                if (at < SMALL_LIST) sm.list[SMALL_LIST + at] = (unsigned short)key;
+            }
+        }
+    }
+    __syncthreads();
+    const uint32_t c0 = sm.n[0], c1 = sm.n[1];
+    uint32_t kA, kB;
+    if (c0 > k && c1 > k && c0 <= SMALL_LIST && c1 <= SMALL_LIST) {
+        // the upper candidates move up behind the lower ones
+        unsigned short v[SMALL_LIST / SMALL_THREADS];
+#pragma unroll
+        for (uint32_t u = 0; u < SMALL_LIST / SMALL_THREADS; ++u) v[u] = tid + SMALL_THREADS * u < c1 ? sm.list[SMALL_LIST + tid + SMALL_THREADS * u] : (unsigned short)0;
+        __syncthreads();
+#pragma unroll
+        for (uint32_t u = 0; u < SMALL_LIST / SMALL_THREADS; ++u) if (tid + SMALL_THREADS * u < c1) sm.list[c0 + tid + SMALL_THREADS * u] = v[u];
+        __syncthreads();
+        cta_select_keys<SMALL_THREADS>(sm.list, c0 + c1, k, c0 + c1 - 1 - k, sm.hist, sm.tmp, kA, kB);
+    } else {
+        cta_select_keys<SMALL_THREADS>(sm.keys, total, k + neg_nan, N - 1 - k + neg_nan, sm.hist, sm.tmp, kA, kB);
+    }
+    if (tid < 2) thr[tid] = float_of_key(tid ? kB : kA);
+}
+
 // Tokens per CTA of the scan: as many as keep the expected number of candidates per tail (1.25 times the tail mass
 // plus the bracket's slack) well inside the CTA's list; a CTA that overflows sends its problem to the exact fallback.
-int scan_tokens_for(double alpha, int D) {
+// Fewer too while the launch does not fill the chip: a thread's loads then come one round after the other for nothing
+// (32 (b,h) of 333 tokens: one CTA for each and tensor 8.5 us, six 4.9).
+int scan_tokens_for(double alpha, int D, int BH, int T) {
     const double per_token = (0.625 * alpha + 0.004) * D;
     int tokens = SCAN_TOKENS_MAX;
     while (tokens > 64 && per_token * tokens > 0.6 * CTA_LIST) tokens /= 2;
+    while (tokens > 64 && (long long)BH * 2 * ((T + tokens - 1) / tokens) < 4 * 148) tokens /= 2;
     return tokens;
 }
 
@@ -543,9 +656,16 @@ extern "C" qaq_status qaq_outlier_thresholds(const qaq_config* cfg, const void* 
     a.list = (unsigned short*)((char*)ws + head);
     a.thr = thr;
     a.scan_tokens = SCAN_TOKENS_MAX;
+    const size_t keys = (size_t)n_tokens * cfg->head_dim, small = sizeof(SmallScratch) + keys * sizeof(unsigned short);
+    if (n_tokens > SAMPLE_TOKENS && keys <= SMALL_KEYS) {
+        static std::atomic<unsigned long long> seen{0};
+        QAQ_CUDA_TRY(qaq_allow_smem((const void*)thr_small_kernel, sizeof(SmallScratch) + SMALL_KEYS * sizeof(unsigned short), seen));
+        QAQ_CUDA_TRY(qaq_launch(thr_small_kernel, dim3(BH * 2), dim3(SMALL_THREADS), small, s, a));
+        return QAQ_OK;
+    }
     QAQ_CUDA_TRY(qaq_launch(thr_sample_kernel, dim3(BH * 2), dim3(256), 0, s, a));
     if (n_tokens > SAMPLE_TOKENS) {
-        a.scan_tokens = scan_tokens_for(cfg->outlier_frac, cfg->head_dim);
+        a.scan_tokens = scan_tokens_for(cfg->outlier_frac, cfg->head_dim, BH, n_tokens);
         dim3 grid((n_tokens + a.scan_tokens - 1) / a.scan_tokens, BH * 2);
         QAQ_CUDA_TRY(qaq_launch(thr_scan_kernel, grid, dim3(256), 0, s, a));
         QAQ_CUDA_TRY(qaq_launch(thr_select_kernel, dim3(BH * 4), dim3(256), 0, s, a));

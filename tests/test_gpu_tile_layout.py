@@ -177,3 +177,20 @@ def test_long_windows_of_any_length_and_number_of_rows(D, window, tokens):
         assert np.array_equal(nvalid.cpu().numpy().reshape(wl.bh, tokens)[bh], nv)
         assert np.all(ring[bh][want == 0] == 0)
         assert np.all(np.abs(ring[bh] - want) <= 1e-6 + 1e-2 * want)
+
+
+@pytest.mark.parametrize("D,tokens", [(128, 65), (128, 128), (128, 129), (32, 512), (32, 513), (64, 255)])
+@pytest.mark.parametrize("alpha,kind", [(0.01, "normal"), (1.0, "normal"), (0.0, "normal"), (0.3, "sorted"), (0.02, "nan"), (0.5, "few values")])
+def test_thresholds_of_short_sequences(D, tokens, alpha, kind):
+    # up to 16384 entries one kernel, beyond three; a bracket that misses, lists that overflow, NaNs of both signs
+    g = torch.Generator().manual_seed(tokens)
+    K, V = (torch.randn((1, 3, tokens, D), generator=g).half() for _ in range(2))
+    if kind == "sorted": K = K.reshape(3, -1).sort(dim=1).values.reshape(1, 3, tokens, D).contiguous()      # the sample is off
+    if kind == "nan":
+        K[0, 0, 1::3] = math.nan; K[0, 1, 5] = -math.nan; V[:] = math.nan; V[0, 2, 0, 0] = 1.0
+    if kind == "few values": K = (K * 2).round().half(); V[:] = 0.0
+    cfg = qaq.make_config(1, 3, D, tokens, 2, 8, 4, alpha)
+    thr = qaq.qaq_outlier_thresholds(cfg, K.cuda(), V.cuda()).cpu().numpy()
+    ku, vu = u16(K).reshape(3, tokens, D), u16(V).reshape(3, tokens, D)
+    want = np.array([[*oracle.thresholds(ku[b], alpha), *oracle.thresholds(vu[b], alpha)] for b in range(3)], dtype=np.float32)
+    assert np.array_equal(thr, want)
