@@ -18,10 +18,10 @@
 namespace {
 
 constexpr int SAMPLE_TOKENS = 64;
-constexpr int SCAN_TOKENS_MAX = 512; // tokens per CTA of the scan (fewer where alpha is large: see scan_tokens_for)
+constexpr int SCAN_TOKENS_MAX = 1024; // tokens per CTA of the scan (fewer where alpha is large: see scan_tokens_for)
 constexpr int WARP_FLAGS = 192;      // 16-byte pieces a warp of the scan can set aside before it has to look at them
-constexpr int CTA_LIST = 4096;       // candidates per tail a scan CTA can hold
-constexpr int SELECT_KEYS = 16384;   // candidates of one tail the select kernel keeps in shared memory
+constexpr int CTA_LIST = 8192;       // candidates a scan CTA can hold
+constexpr int SELECT_KEYS = 16384;   // candidates the select kernel keeps in shared memory
 
 __device__ __forceinline__ uint32_t key_of(unsigned short h) { return (h & 0x8000u) ? (uint32_t)(~h & 0xFFFFu) : (uint32_t)(h | 0x8000u); }
 __device__ __forceinline__ unsigned short half_of_key(uint32_t k) { return (k & 0x8000u) ? (unsigned short)(k & 0x7FFFu) : (unsigned short)(~k & 0xFFFFu); }
@@ -31,11 +31,11 @@ __device__ __forceinline__ float float_of_key(uint32_t k) { return __half2float(
 
 struct Problem {          // per (b,h,tensor), in the workspace
     uint32_t klo, khi;    // bracket keys: candidates are keys < klo and keys > khi
-    uint32_t cnt[2];      // candidates found (may exceed the capacity: then the list is incomplete)
+    uint32_t cnt[2];      // candidates found below and above (their sum may exceed the capacity: then the list is incomplete)
     uint32_t nan;         // NaN entries seen by the scan
     uint32_t done;        // solved by the sample kernel
-    uint32_t overflow;    // bit `tail`: a scan CTA found more candidates than it can hold, the list has holes
-    uint32_t pad;
+    uint32_t overflow;    // a scan CTA found more candidates than it can hold, the list has holes
+    uint32_t n;           // places taken in the list
 };
 
 struct ThrArgs {
@@ -44,7 +44,7 @@ struct ThrArgs {
     int H, T, D;
     double alpha;
     Problem* prob;        // [BH*2]
-    unsigned short* list; // [BH*2][2][cap]
+    unsigned short* list; // [BH*2][cap]: candidates of both tails in any order (every lower one is below every upper one)
     uint32_t cap;
     int scan_tokens;      // tokens per CTA of the scan
     float* thr;           // [BH][4]
@@ -57,8 +57,9 @@ struct ThrArgs {
 // counters; 11 bits spread them over 32 bins per octave.  In the first pass every thread sums 8 bins and a
 // CTA-wide prefix sum finds the bin holding the wanted rank; the second pass has 32 bins, one per lane of
 // warp 0.
-template <typename Get>
+template <int THREADS, typename Get>
 __device__ uint32_t cta_select(Get get, uint32_t n, uint32_t want, uint32_t* hist, uint32_t* s_tmp) {
+    constexpr int BINS = 2048 / THREADS;                     // of a thread
     const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
     // ---- first pass: upper 11 bits
     for (int i = threadIdx.x; i < 2048; i += blockDim.x) hist[i] = 0;
@@ -68,9 +69,9 @@ __device__ uint32_t cta_select(Get get, uint32_t n, uint32_t want, uint32_t* his
         if (k <= 0xFFFFu) atomicAdd(&hist[k >> 5], 1u);     // larger: NaN marker
     }
     __syncthreads();
-    uint32_t c[8], tot = 0;
+    uint32_t c[BINS], tot = 0;
 #pragma unroll
-    for (int j = 0; j < 8; ++j) { c[j] = hist[8 * threadIdx.x + j]; tot += c[j]; }
+    for (int j = 0; j < BINS; ++j) { c[j] = hist[BINS * threadIdx.x + j]; tot += c[j]; }
     uint32_t inc = tot;
 #pragma unroll
     for (int d = 1; d < 32; d <<= 1) {
@@ -82,23 +83,23 @@ __device__ uint32_t cta_select(Get get, uint32_t n, uint32_t want, uint32_t* his
     __syncthreads();
     uint32_t before = 0, all = 0;
 #pragma unroll
-    for (int w = 0; w < 8; ++w) {
+    for (int w = 0; w < THREADS / 32; ++w) {
         const uint32_t v = hist[w];
         if (w < warp) before += v;
         all += v;
     }
-    uint32_t acc = before + inc - tot;                       // keys in the bins before this thread's eight
+    uint32_t acc = before + inc - tot;                       // keys in the bins before this thread's
     const uint32_t w2 = want < all ? want : (all ? all - 1 : 0);   // defensive clamp
     if (threadIdx.x == 0) { s_tmp[0] = 0; s_tmp[1] = 0; }    // all == 0: no key at all
     __syncthreads();
     if (tot > 0 && w2 >= acc && w2 < acc + tot) {            // exactly one thread
         int bsel = 0;
 #pragma unroll
-        for (int j = 0; j < 8; ++j) {
-            if (w2 >= acc + c[j] && j < 7) { acc += c[j]; bsel = j + 1; }
+        for (int j = 0; j < BINS; ++j) {
+            if (w2 >= acc + c[j] && j < BINS - 1) { acc += c[j]; bsel = j + 1; }
             else break;
         }
-        s_tmp[0] = (uint32_t)(8 * threadIdx.x + bsel);
+        s_tmp[0] = (uint32_t)(BINS * threadIdx.x + bsel);
         s_tmp[1] = w2 - acc;
     }
     __syncthreads();
@@ -291,7 +292,7 @@ __global__ void __launch_bounds__(256) thr_sample_kernel(const ThrArgs a) {
     const bool whole = (ns == a.T);
     if (Mv == 0) {
         if (threadIdx.x == 0) {
-            pr->klo = 0; pr->khi = 0xFFFF; pr->cnt[0] = pr->cnt[1] = 0; pr->nan = 0; pr->overflow = 0; pr->done = whole ? 1u : 0u;
+            pr->klo = 0; pr->khi = 0xFFFF; pr->cnt[0] = pr->cnt[1] = 0; pr->nan = 0; pr->overflow = 0; pr->n = 0; pr->done = whole ? 1u : 0u;
             if (whole) { a.thr[(size_t)bh * 4 + 2 * x] = 0.f; a.thr[(size_t)bh * 4 + 2 * x + 1] = 0.f; }
         }
         return;
@@ -307,7 +308,7 @@ __global__ void __launch_bounds__(256) thr_sample_kernel(const ThrArgs a) {
     uint32_t klo, khi;
     cta_select_keys(s_keys, (uint32_t)M, r_lo + n_neg_nan, r_hi + n_neg_nan, hist, s_tmp, klo, khi);
     if (threadIdx.x == 0) {
-        pr->klo = klo; pr->khi = khi; pr->cnt[0] = pr->cnt[1] = 0; pr->nan = 0; pr->overflow = 0; pr->done = whole ? 1u : 0u;
+        pr->klo = klo; pr->khi = khi; pr->cnt[0] = pr->cnt[1] = 0; pr->nan = 0; pr->overflow = 0; pr->n = 0; pr->done = whole ? 1u : 0u;
         if (whole) {
             a.thr[(size_t)bh * 4 + 2 * x] = float_of_key(klo);
             a.thr[(size_t)bh * 4 + 2 * x + 1] = float_of_key(khi);
@@ -320,19 +321,23 @@ __global__ void __launch_bounds__(256) thr_sample_kernel(const ThrArgs a) {
 // at least lo and whose largest is at most hi (NaN-propagating min / max, so a NaN fails both) is dropped; the others
 // (about one in ten at alpha = 1 %) are set aside in a buffer of the warp's own, and when enough of them have come
 // together the warp looks at them entry by entry with all lanes busy.  Nothing in the loop needs the other warps:
-// no CTA barrier, one shared-memory reservation per warp, tail and batch of set-aside pieces.
+// no CTA barrier, one shared-memory reservation per warp and batch of set-aside pieces; the candidates of both tails share a
+// list, which the select takes apart by rank.
+// What bounds it: memory where outliers are few (256 (b,h) of 4096 tokens, alpha = 1 %: 105 us, 5.1 TB/s; 124 us without
+// the next pieces on their way while four are looked at, and with 512 tokens per CTA), the extraction where they are many
+// (160 (b,h) of 8192 tokens, 5 %: 215 us; 269 with a list, a prefix sum and a loop for each tail).  60 registers, four
+// CTAs per SM: held to five it takes 114 us, to six 169.
 __global__ void __launch_bounds__(256) thr_scan_kernel(const ThrArgs a) {
     qaq_dependency();
     const int bhx = blockIdx.y, bh = bhx >> 1, x = bhx & 1;
     Problem* pr = a.prob + bhx;
     if (pr->done) return;
-    __shared__ unsigned short s_list[2][CTA_LIST];
+    __shared__ unsigned short s_list[CTA_LIST];
     __shared__ uint4 s_flag[8][WARP_FLAGS];                   // per warp: pieces with something outside [lo, hi]
-    __shared__ uint32_t s_n[2], s_base[2], s_nan;
+    __shared__ uint32_t s_n, s_low, s_base, s_nan;
     const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
     const unsigned lt = (1u << lane) - 1u;
-    if (threadIdx.x < 2) s_n[threadIdx.x] = 0;
-    if (threadIdx.x == 2) s_nan = 0;
+    if (threadIdx.x == 0) { s_n = 0; s_low = 0; s_nan = 0; }
     __syncthreads();
     const float flo = float_of_key(pr->klo), fhi = float_of_key(pr->khi);
     const __half2 lo2 = __float2half2_rn(flo), hi2 = __float2half2_rn(fhi);   // exact: both are binary16 values
@@ -347,20 +352,25 @@ __global__ void __launch_bounds__(256) thr_scan_kernel(const ThrArgs a) {
     const size_t ptr_step = (size_t)tok_step * a.st;
     uint4* wflag = s_flag[warp];
     uint32_t nflag = 0;      // pieces set aside by this warp (the same in all its lanes)
-    uint32_t nnan = 0;
+    uint32_t nnan = 0, nlow = 0;
 
+    // four independent 16-byte loads per thread, the next four on their way while these are looked at
+    uint4 next[4];
+#pragma unroll
+    for (int u = 0; u < 4; ++u) {
+        next[u] = make_uint4(0, 0, 0, 0);
+        if (tok + u * tok_step < ntok) next[u] = *reinterpret_cast<const uint4*>(ptr + u * ptr_step);
+    }
     for (int c0 = 0; c0 < ntok; c0 += 4 * tok_step) {
-        // four independent 16-byte loads per thread before any of them is looked at
         uint4 raw[4];
         bool in_range[4];
 #pragma unroll
-        for (int u = 0; u < 4; ++u) {
-            in_range[u] = tok + u * tok_step < ntok;
-            raw[u] = make_uint4(0, 0, 0, 0);
-            if (in_range[u]) raw[u] = *reinterpret_cast<const uint4*>(ptr + u * ptr_step);
-        }
+        for (int u = 0; u < 4; ++u) { in_range[u] = tok + u * tok_step < ntok; raw[u] = next[u]; }
         tok += 4 * tok_step;
         ptr += 4 * ptr_step;
+#pragma unroll
+        for (int u = 0; u < 4; ++u)
+            if (tok + u * tok_step < ntok) next[u] = *reinterpret_cast<const uint4*>(ptr + u * ptr_step);
 #pragma unroll
         for (int u = 0; u < 4; ++u) {
             const __half2 v0 = h2_of(raw[u].x), v1 = h2_of(raw[u].y), v2 = h2_of(raw[u].z), v3 = h2_of(raw[u].w);
@@ -395,32 +405,26 @@ __global__ void __launch_bounds__(256) thr_scan_kernel(const ThrArgs a) {
             }
             if (!have) { below = 0; above = 0; nans = 0; }
             nnan += (uint32_t)__popc(nans);
-            const uint32_t pk = (uint32_t)__popc(below) | ((uint32_t)__popc(above) << 16);   // at most 8 each
-            uint32_t inc = pk;
+            nlow += (uint32_t)__popc(below);
+            uint32_t m = below | above;
+            const uint32_t mine = (uint32_t)__popc(m);            // at most 8
+            uint32_t inc = mine;
 #pragma unroll
             for (int d = 1; d < 32; d <<= 1) {
                 const uint32_t t = __shfl_up_sync(0xFFFFFFFFu, inc, d);
                 if (lane >= d) inc += t;
             }
-            const uint32_t tot = __shfl_sync(0xFFFFFFFFu, inc, 31);
-            uint32_t b0 = 0, b1 = 0;
-            if (lane == 0) {
-                if (tot & 0xFFFFu) b0 = atomicAdd(&s_n[0], tot & 0xFFFFu);
-                if (tot >> 16) b1 = atomicAdd(&s_n[1], tot >> 16);
-            }
-            uint32_t pos[2] = {__shfl_sync(0xFFFFFFFFu, b0, 0) + ((inc - pk) & 0xFFFFu), __shfl_sync(0xFFFFFFFFu, b1, 0) + ((inc - pk) >> 16)};
-#pragma unroll
-            for (int side = 0; side < 2; ++side) {
-                uint32_t m = side ? above : below;
-                while (m) {
-                    const int bit = __ffs(m) - 1;
-                    m &= m - 1;
-                    const int j = bit & 3;
-                    const uint32_t wj = (j & 2) ? ((j & 1) ? w[3] : w[2]) : ((j & 1) ? w[1] : w[0]);
-                    const unsigned short h = (unsigned short)((bit >> 4) ? (wj >> 16) : (wj & 0xFFFFu));
-                    if (pos[side] < (uint32_t)CTA_LIST) s_list[side][pos[side]] = (unsigned short)key_of(h);
-                    ++pos[side];
-                }
+            uint32_t b0 = 0;
+            if (lane == 31 && inc) b0 = atomicAdd(&s_n, inc);
+            uint32_t pos = __shfl_sync(0xFFFFFFFFu, b0, 31) + inc - mine;
+            while (m) {
+                const int bit = __ffs(m) - 1;
+                m &= m - 1;
+                const int j = bit & 3;
+                const uint32_t wj = (j & 2) ? ((j & 1) ? w[3] : w[2]) : ((j & 1) ? w[1] : w[0]);
+                const unsigned short h = (unsigned short)((bit >> 4) ? (wj >> 16) : (wj & 0xFFFFu));
+                if (pos < (uint32_t)CTA_LIST) s_list[pos] = (unsigned short)key_of(h);
+                ++pos;
             }
         }
         const uint32_t left = nflag - ntake;           // fewer than 32
@@ -432,59 +436,58 @@ __global__ void __launch_bounds__(256) thr_scan_kernel(const ThrArgs a) {
         __syncwarp();     // the rest of the buffer is free again
     }
 #pragma unroll
-    for (int o = 16; o > 0; o >>= 1) nnan += __shfl_xor_sync(0xFFFFFFFFu, nnan, o);
+    for (int o = 16; o > 0; o >>= 1) { nnan += __shfl_xor_sync(0xFFFFFFFFu, nnan, o); nlow += __shfl_xor_sync(0xFFFFFFFFu, nlow, o); }
     if (lane == 0 && nnan) atomicAdd(&s_nan, nnan);
+    if (lane == 0 && nlow) atomicAdd(&s_low, nlow);
     __syncthreads();
-    if (threadIdx.x < 2) s_base[threadIdx.x] = s_n[threadIdx.x] ? atomicAdd(&pr->cnt[threadIdx.x], s_n[threadIdx.x]) : 0u;
-    if (threadIdx.x == 2 && s_nan) atomicAdd(&pr->nan, s_nan);
+    const uint32_t cnt = s_n, low = s_low;
+    if (threadIdx.x == 0) {
+        s_base = cnt ? atomicAdd(&pr->n, cnt) : 0u;
+        if (low) atomicAdd(&pr->cnt[0], low);
+        if (cnt > low) atomicAdd(&pr->cnt[1], cnt - low);
+        if (s_nan) atomicAdd(&pr->nan, s_nan);
+        if (cnt > CTA_LIST) atomicOr(&pr->overflow, 1u);       // leaves a hole in the list: the select kernel falls back
+    }
     __syncthreads();
-#pragma unroll
-    for (int side = 0; side < 2; ++side) {
-        const uint32_t cnt = s_n[side];
-        // a CTA list that overflowed leaves a hole in the global list: the select kernel falls back for that tail
-        if (cnt > CTA_LIST) { if (threadIdx.x == 0) atomicOr(&pr->overflow, 1u << side); continue; }
-        unsigned short* dst = a.list + ((size_t)bhx * 2 + side) * a.cap;
-        for (uint32_t i = threadIdx.x; i < cnt; i += blockDim.x) {
-            const uint32_t pos = s_base[side] + i;
-            if (pos < a.cap) dst[pos] = s_list[side][i];
-        }
+    if (cnt > CTA_LIST) return;
+    unsigned short* dst = a.list + (size_t)bhx * a.cap;
+    for (uint32_t i = threadIdx.x; i < cnt; i += blockDim.x) {
+        const uint32_t pos = s_base + i;
+        if (pos < a.cap) dst[pos] = s_list[i];
     }
 }
 
 // ---- 3. exact select among the candidates, exact fallback over the data when that is not possible.
-// One CTA per (problem, tail): the two tails are independent order statistics.
-__global__ void __launch_bounds__(256) thr_select_kernel(const ThrArgs a) {
+template <int THREADS>
+__global__ void __launch_bounds__(THREADS) thr_select_kernel(const ThrArgs a) {
     qaq_dependency();
-    const int bhx = blockIdx.x >> 1, side = blockIdx.x & 1, bh = bhx >> 1, x = bhx & 1;
+    const int bhx = blockIdx.x, bh = bhx >> 1, x = bhx & 1;
     Problem* pr = a.prob + bhx;
     if (pr->done) return;
     __shared__ uint32_t hist[2048], s_tmp[4];
     __shared__ __align__(16) unsigned short s_keys[SELECT_KEYS];
     const unsigned long long total = (unsigned long long)a.T * a.D;
     const unsigned long long N = total - pr->nan;
-    float res = 0.f;
+    float res[2] = {0.f, 0.f};
     if (N > 0) {
         const unsigned long long k = rank_k(a.alpha, N);
-        const uint32_t c = pr->cnt[side];
-        if (c > k && c <= a.cap && !((pr->overflow >> side) & 1u)) {
-            // rank k from below in the low list, rank k from above in the high list
-            const uint32_t want = side == 0 ? (uint32_t)k : (uint32_t)(c - 1 - k);
-            const unsigned short* l = a.list + ((size_t)bhx * 2 + side) * a.cap;   // 16-byte aligned
+        const uint32_t c0 = pr->cnt[0], c1 = pr->cnt[1], c = c0 + c1;
+        if (c0 > k && c1 > k && c <= a.cap && !pr->overflow) {
+            // rank k from below and rank k from above
+            const unsigned short* l = a.list + (size_t)bhx * a.cap;                // 16-byte aligned
+            const unsigned short* keys = l;
             if (c <= (uint32_t)SELECT_KEYS) {
-                // the usual case: the list fits in shared memory; bring it in with independent wide loads
-                for (uint32_t i = threadIdx.x; i < (c + 7) / 8; i += blockDim.x)
+                // the usual case: the list fits in shared memory; bring it in with independent wide loads.  (A longer
+                // list is read twice where it lies, eight keys at a time; one at a time: 124 us for 640 lists of 52000
+                // keys, eight: 43 us)
+                for (uint32_t i = threadIdx.x; i < (c + 7) / 8; i += THREADS)
                     reinterpret_cast<uint4*>(s_keys)[i] = reinterpret_cast<const uint4*>(l)[i];
                 __syncthreads();
-                uint32_t key, same;
-                cta_select_keys(s_keys, c, want, want, hist, s_tmp, key, same);
-                res = float_of_key(key);
-            } else {
-                // a longer list is read twice where it lies, eight keys at a time (one at a time: 124 us for 640 lists of
-                // 52000 keys, eight: 43 us)
-                uint32_t key, same;
-                cta_select_keys(l, c, want, want, hist, s_tmp, key, same);
-                res = float_of_key(key);
+                keys = s_keys;
             }
+            uint32_t lo, hi;
+            cta_select_keys<THREADS>(keys, c, (uint32_t)k, (uint32_t)(c - 1 - k), hist, s_tmp, lo, hi);
+            res[0] = float_of_key(lo); res[1] = float_of_key(hi);
         } else {
             // bracket too tight or list overflow: two-pass radix select over this problem's data
             const int b_idx = bh / a.H, h_idx = bh % a.H;
@@ -494,10 +497,12 @@ __global__ void __launch_bounds__(256) thr_select_kernel(const ThrArgs a) {
                 const unsigned short h = __half_as_ushort(X[(size_t)(i / D) * a.st + (i % D)]);
                 return is_nan_bits(h) ? 0x10000u : key_of(h);
             };
-            res = float_of_key(cta_select(getx, (uint32_t)total, side == 0 ? (uint32_t)k : (uint32_t)(N - 1 - k), hist, s_tmp));
+#pragma unroll 1
+            for (int side = 0; side < 2; ++side)
+                res[side] = float_of_key(cta_select<THREADS>(getx, (uint32_t)total, side == 0 ? (uint32_t)k : (uint32_t)(N - 1 - k), hist, s_tmp));
         }
     }
-    if (threadIdx.x == 0) a.thr[(size_t)bh * 4 + 2 * x + side] = res;
+    if (threadIdx.x < 2) a.thr[(size_t)bh * 4 + 2 * x + threadIdx.x] = threadIdx.x ? res[1] : res[0];
 }
 
 // ---- short sequences: the three steps by one CTA per problem, on keys that stay in shared memory.
@@ -598,12 +603,12 @@ __global__ void __launch_bounds__(SMALL_THREADS) thr_small_kernel(const ThrArgs 
     if (tid < 2) thr[tid] = float_of_key(tid ? kB : kA);
 }
 
-// Tokens per CTA of the scan: as many as keep the expected number of candidates per tail (1.25 times the tail mass
-// plus the bracket's slack) well inside the CTA's list; a CTA that overflows sends its problem to the exact fallback.
+// Tokens per CTA of the scan: as many as keep the expected number of candidates (1.25 times the tail mass
+// plus the bracket's slack, of both tails) well inside the CTA's list; a CTA that overflows sends its problem to the exact fallback.
 // Fewer too while the launch does not fill the chip: a thread's loads then come one round after the other for nothing
 // (32 (b,h) of 333 tokens: one CTA for each and tensor 8.5 us, six 4.9).
 int scan_tokens_for(double alpha, int D, int BH, int T) {
-    const double per_token = (0.625 * alpha + 0.004) * D;
+    const double per_token = 2.0 * (0.625 * alpha + 0.004) * D;
     int tokens = SCAN_TOKENS_MAX;
     while (tokens > 64 && per_token * tokens > 0.6 * CTA_LIST) tokens /= 2;
     while (tokens > 64 && (long long)BH * 2 * ((T + tokens - 1) / tokens) < 4 * 148) tokens /= 2;
@@ -650,7 +655,7 @@ extern "C" qaq_status qaq_outlier_thresholds(const qaq_config* cfg, const void* 
     a.prob = (Problem*)ws;
     // the candidate lists take whatever the workspace offers beyond the problem records
     const size_t head = ((size_t)BH * 2 * sizeof(Problem) + 255) / 256 * 256;
-    const size_t per_list = (ws_bytes - head) / ((size_t)BH * 4 * sizeof(unsigned short));
+    const size_t per_list = (ws_bytes - head) / ((size_t)BH * 2 * sizeof(unsigned short));
     a.cap = (uint32_t)(per_list > 0x3FFFFFC0u ? 0x3FFFFFC0u : per_list) & ~63u;
     if (a.cap < 64) return QAQ_ERR_WORKSPACE;
     a.list = (unsigned short*)((char*)ws + head);
@@ -668,7 +673,10 @@ extern "C" qaq_status qaq_outlier_thresholds(const qaq_config* cfg, const void* 
         a.scan_tokens = scan_tokens_for(cfg->outlier_frac, cfg->head_dim, BH, n_tokens);
         dim3 grid((n_tokens + a.scan_tokens - 1) / a.scan_tokens, BH * 2);
         QAQ_CUDA_TRY(qaq_launch(thr_scan_kernel, grid, dim3(256), 0, s, a));
-        QAQ_CUDA_TRY(qaq_launch(thr_select_kernel, dim3(BH * 4), dim3(256), 0, s, a));
+        // lists that stay in shared memory are a matter of latency (256 (b,h) of 4096 tokens, alpha = 1 %: 14.6 us with 256
+        // threads, 19.1 with 512), longer ones of throughput (160 of 8192 tokens, 5 %: 68.3 and 48.7 us)
+        if (1.25 * cfg->outlier_frac * (double)keys <= SELECT_KEYS) QAQ_CUDA_TRY(qaq_launch(thr_select_kernel<256>, dim3(BH * 2), dim3(256), 0, s, a));
+        else QAQ_CUDA_TRY(qaq_launch(thr_select_kernel<512>, dim3(BH * 2), dim3(512), 0, s, a));
     }
     return QAQ_OK;
 }
