@@ -84,26 +84,25 @@ __device__ __forceinline__ uint32_t mad(uint32_t a, uint32_t b, uint32_t c) {
     asm("mad.lo.u32 %0, %1, %2, %3;" : "=r"(d) : "r"(a), "r"(b), "r"(c));
     return d;
 }
-struct Scale {                 // of a token: code = min(floor(sat((x - mn) * inv) * 2^B), 2^B - 1)
-    float mn, inv;             // 1 / (max - min), which is 2^-B times the reciprocal of the step; 0 for a constant token
-    uint64_t levels;           // 2^B, twice
+struct Scale {                 // of a token: code = min(floor((x - mn) * inv), 2^B - 1)
+    float mn;
+    uint64_t inv;              // the reciprocal of the step, twice; 0 for a constant token
     uint32_t top;              // 2^B - 1 in the low half, that and the bits of 2^23 in the high half
     uint32_t k64;              // 65536, kept from the compiler, which would take a byte shuffle
 };
 // Codes of a binary16 pair: the first in the low byte, the second in byte 2 (byte 3 is not clean).  2^23 + floor(t) has
-// the code in its low bits; an outlier's place holds a number that is none, which saturates to 0.
+// the code in its low bits; an outlier's place holds the minimum, which has code 0.
 __device__ __forceinline__ uint32_t code_pair(uint32_t v, const Scale& s) {
-    float x0, x1, u0, u1;
+    float x0, x1;
     asm("{\n.reg .b16 h0, h1;\nmov.b32 {h0, h1}, %2;\nsub.rn.f32.f16 %0, h0, %3;\nsub.rn.f32.f16 %1, h1, %3;\n}" : "=f"(x0), "=f"(x1) : "r"(v), "f"(s.mn));
-    asm("mul.rn.sat.f32 %0, %1, %2;" : "=f"(u0) : "f"(x0), "f"(s.inv));
-    asm("mul.rn.sat.f32 %0, %1, %2;" : "=f"(u1) : "f"(x1), "f"(s.inv));
     uint64_t t;
-    asm("fma.rm.f32x2 %0, %1, %2, %3;" : "=l"(t) : "l"(pair_of(u0, u1)), "l"(s.levels), "l"(pair_of(8388608.0f, 8388608.0f)));
+    asm("mul.rn.f32x2 %0, %1, %2;" : "=l"(t) : "l"(pair_of(x0, x1)), "l"(s.inv));
+    asm("add.rm.f32x2 %0, %1, %2;" : "=l"(t) : "l"(t), "l"(pair_of(8388608.0f, 8388608.0f)));
     uint32_t d;
     asm("min.u16x2 %0, %1, %2;" : "=r"(d) : "r"(mad((uint32_t)(t >> 32), s.k64, (uint32_t)t)), "r"(s.top));
     return d;
 }
-constexpr uint32_t GONE = 0xFFFFu;      // in the place of an outlier: not a number
+constexpr uint32_t GONE = 0xFFFFu;      // in the place of an outlier of a token whose range is not finite: not a number
 
 // What a warp keeps of its tile in shared memory.  The 16-byte pieces of the rows are stored swizzled (piece U at U ^ (U/8
 // mod 4)), so that lanes that read 64 bytes each do not meet in the banks.
@@ -266,6 +265,7 @@ __device__ __forceinline__ void quantize_tile(const QuantArgs& a, TileScratch<D>
             cnt += (uint32_t)__popc(ob[k]);
         }
         uint32_t pos = prefix(cnt, lane, nout);
+        const uint32_t r = sm.range[tid], fill = ((r & 0x7C00u) == 0x7C00u || (r >> 16 & 0x7C00u) == 0x7C00u) ? GONE : r & 0xFFFFu;
 #pragma unroll
         for (int k = 0; k < P; ++k)
             while (ob[k]) {
@@ -273,7 +273,7 @@ __device__ __forceinline__ void quantize_tile(const QuantArgs& a, TileScratch<D>
                 ob[k] &= ob[k] - 1;
                 unsigned short* where = reinterpret_cast<unsigned short*>(sm.data + 16 * (U ^ ((U >> 3) & 3))) + (c & 7);
                 if (pos < cap) list[pos] = ((uint32_t)tid << 24) | (c << 16) | *where;
-                *where = GONE;
+                *where = (unsigned short)fill;
                 ++pos;
             }
     }
@@ -310,10 +310,8 @@ __device__ __forceinline__ void quantize_tile(const QuantArgs& a, TileScratch<D>
     if (!OPEN || b) {
         const int row = IS_V ? slot >> 2 : slot, row_w = IS_V ? qaqc::width_of_row(rows, row) : b;
         const qaqc::RowPlace pl = qaqc::place_row<D, IS_V>(rows, row, row_w);
-        // the reciprocal of the step without its power of two (the range of binary16 numbers is nowhere near the ends of
-        // binary32: both are the same number but for the exponent)
-        const float len = __fsub_rn(mx, mn), inv = len > 0.f ? __fdiv_rn(1.0f, len) : 0.f;
-        const bool endless = len > 0.f && inv == 0.f;         // a range that is not finite
+        const float step = qaqc::step_of(mn, mx, b), inv = step > 0.f ? __fdiv_rn(1.0f, step) : 0.f;
+        const bool endless = ((range & 0x7C00u) == 0x7C00u || (range >> 16 & 0x7C00u) == 0x7C00u);
         uint4 q = make_uint4(__float_as_uint(mn), __float_as_uint(inv), pl.main | (pl.high << 16),
                              (uint32_t)tid | ((uint32_t)b << 8) | ((uint32_t)row_w << 16) | (pl.mm << 20) | (pl.mh << 24) | (endless ? 0x80000000u : 0u));
         if (OPEN && old) {             // where it is in the tile as it is stored, instead of the range
@@ -415,14 +413,12 @@ __device__ __forceinline__ void quantize_tile(const QuantArgs& a, TileScratch<D>
         uint32_t v[16], c[16];
         load_row(data + 16 * (U ^ ((U >> 3) & 3)), v);
         sc.mn = __uint_as_float(q.x);
-        sc.inv = __uint_as_float(q.y);
-        const float levels = __int_as_float((127 + B) << 23);
-        sc.levels = pair_of(levels, levels);
+        sc.inv = pair_of(__uint_as_float(q.y), __uint_as_float(q.y));
         sc.top = ((1u << B) - 1u) * 0x00010001u + 0x4B000000u;
 #pragma unroll
         for (int k = 0; k < 16; ++k) c[k] = code_pair(v[k], sc);
         if (__any_sync(0xFFFFFFFFu, q.w >> 31)) {
-            if (q.w >> 31) {           // marks become -inf, which the plain arithmetic takes to code 0
+            if (q.w >> 31) {           // a range that is not finite: marks become -inf, which the plain arithmetic takes to code 0
                 uint32_t creg[8];
 #pragma unroll
                 for (int k = 0; k < 16; ++k) {

@@ -133,6 +133,12 @@ __device__ __forceinline__ void requantize_tile(const RequantArgs& a, RequantScr
         }
         if (valid) Bn = (UP || B < Bo) ? B : Bo;
     }
+    // a raised token's row is on its way to L2 while the tile's order is found
+    if (UP && Bn > Bo) {
+        const __half* row = (IS_V ? a.Vs : a.Ks) + (size_t)(bh / a.H) * a.sb + (size_t)(bh % a.H) * a.sh + (size_t)tok * a.st;
+#pragma unroll
+        for (int i = 0; i < D; i += 64) asm volatile("prefetch.global.L2 [%0];" ::"l"(row + i));
+    }
     const uint32_t alike = qaqc::count_half(Bn, lane, sm.count[warp]);
     bool changed = __syncthreads_or(Bn != Bo) != 0;          // also makes the counts visible
     // An open tile has to be the last thing in its pool.  If closed tiles of this (b,h) have just been moved
