@@ -39,8 +39,7 @@ import hashlib
 COUNTERS_JSON = os.path.join(ROOT, "profiles", "counters_C3.json")
 CSRC = os.path.join(ROOT, "paper_2403_04643_b200", "csrc")
 ISSUE_SLOTS_PER_CLOCK = 148 * 4
-KERNEL_KEYS = {"quant_keys": "quant_kernel<128, 0, 0>", "quant_values": "quant_kernel<128, 0, 1>", "decode": "decode_kernel<128, 1, 0>",
-               "thr_scan": "thr_scan_kernel"}
+KERNEL_KEYS = {"quant": "quant_tiles_kernel<128, 0>", "decode": "decode_kernel<128, 1, 0, 0>", "thr_scan": "thr_scan_kernel"}
 
 
 def csrc_hash():
@@ -292,7 +291,7 @@ def main():
         hyper_source = "calibrated in this run"
 
     # layers are independent problems: outside the per-stage timing pass they are spread over a few streams, so that
-    # the short, latency-bound kernels of one layer (threshold sample / select, merge) overlap another layer's long ones
+    # the short, latency-bound kernels of one layer (threshold sample / select) overlap another layer's long ones
     side = [torch.cuda.Stream(device=dev) for _ in range(max(0, args.streams - 1))]
 
     def step(timers=None):
@@ -403,15 +402,15 @@ def main():
                        "cached_tokens_per_s": round(wl.batch * T / (stage_ms["dec"] * 1e-3), 1),
                        "generated_tokens_per_s": round(wl.batch / (L * stage_ms["dec"] * 1e-3), 2)},
         },
-        "roofline": {"kernel": "quant_kernel, keys launch + values launch (fused select + outlier split + quantize + pack)", "bound": "hbm",
+        "roofline": {"kernel": "quant_tiles_kernel, keys and values (fused select + outlier split + quantize + pack)", "bound": "hbm",
                      "achieved": round(quant_gbs, 1), "peak": peak, "unit": "GB/s", "frac": round(quant_gbs / peak, 3),
-                     "traffic": traffic("quant_keys", "quant_values"), "traffic_note": cnote, "peak_kind": peak_kind, "bytes_per_launch": ab["quantize"]},
-        "roofline_decode": {"kernel": "decode_kernel (+ merge)", "bound": "hbm", "achieved": round(dec_gbs, 1), "peak": peak,
+                     "traffic": traffic("quant"), "traffic_note": cnote, "peak_kind": peak_kind, "bytes_per_launch": ab["quantize"]},
+        "roofline_decode": {"kernel": "decode_kernel", "bound": "hbm", "achieved": round(dec_gbs, 1), "peak": peak,
                             "unit": "GB/s", "frac": round(dec_gbs / peak, 3), "traffic": traffic("decode"), "traffic_note": cnote, "peak_kind": peak_kind,
                             "bytes_per_launch": ab["decode"]},
-        "roofline_issue": {"quant_kernel": issue_roofline(instr("quant_keys", "quant_values"), stage_ms["quant"] * 1e-3, clocks.get("sm_mhz")),
+        "roofline_issue": {"quant_tiles_kernel": issue_roofline(instr("quant"), stage_ms["quant"] * 1e-3, clocks.get("sm_mhz")),
                            "decode_kernel": issue_roofline(instr("decode"), stage_ms["dec"] * 1e-3, clocks.get("sm_mhz"))},
-        "gpu_launches": args.steps * L * 7,   # thresholds 3 (sample, scan, select), quantize 2 (keys, values), decode 2 (+ merge)
+        "gpu_launches": args.steps * L * 5,   # thresholds 3 (sample, scan, select), quantize 1, decode 1
         "clocks": clocks,
     }
 
@@ -736,7 +735,7 @@ def stream_c5(qaq, dev):
     res = {"steps": T1 - T0, "seconds": round(sec, 2), "us_per_step": round(sec / (T1 - T0) * 1e6, 1),
            "generated_tokens_per_s": round(wl.batch * (T1 - T0) / sec, 1), "final_tokens": int(st.tokens),
            "device_status": int(st.device_status),
-           "note": "host-launched steps (one append launch, decode + merge per step); values of appended tokens stay at 8 bits"}
+           "note": "host-launched steps (one append launch and one decode launch per step); values of appended tokens stay at 8 bits"}
     # the same run with the token count in device memory: one captured append + decode pair replayed 98304 times, the
     # new token's rows copied into the captured buffers before every replay
     cache.reset()

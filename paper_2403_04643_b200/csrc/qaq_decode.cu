@@ -38,7 +38,7 @@
 // depend on the order in which lanes arrive.
 //
 // The partials of a (b,h) that was split over several CTAs are merged by the last of these CTAs to finish, in the
-// same launch (see finish_split).
+// same launch (see merge_split).
 #include <chrono>
 #include <mutex>
 
@@ -47,7 +47,6 @@
 
 namespace {
 
-using qaqc::Section;
 
 // ------------------------------------------------------------------------------------------ instructions
 // D(16x8, s32) += A(16x32, u8, row) * B(32x8, s8, col).  Lane = 4*g + t holds
@@ -150,7 +149,7 @@ struct DecArgs {
     long q_stride, out_stride;   // elements between the rows of consecutive (b,h) in q and in out (queries of a (b,h) are D apart)
     float scale;
     float* part;       // [ncta][2][NQ][D+4]: accumulators, reference of the exponentials, sum of p
-    unsigned long long* done;    // [BH]: tag of the call | partials that are complete (see finish_split)
+    unsigned long long* done;    // [BH]: tag of the call | partials that are complete (see merge_split)
     unsigned long long tag;      // of this call; the low 12 bits are zero
     float* ml;         // [BH][2]   merged (max, sum) for the normalisation of long score rows, or null
     int BH, run, ncta; // (b,h) count; tiles per CTA of the flattened (b,h, tile) sequence; CTAs
@@ -1234,7 +1233,7 @@ qaq_status decode(const qaq_cache* c, const void* q, long q_stride, float softma
     a.ncta = COUNTED ? (BH > Shape<NQ>::SLOTS ? BH : Shape<NQ>::SLOTS) : plan.ncta;   // counted: the largest grid any count needs
     a.cluster = plan_cluster<NQ>(BH, (a.T + QAQ_TILE - 1) / QAQ_TILE, a.groups);
     if (a.cluster) a.ncta = BH * a.cluster;
-    // nothing in the workspace is read before it is written (the counting words: see finish_split)
+    // nothing in the workspace is read before it is written (the counting words: see merge_split)
     a.part = (float*)ws;
     a.done = (unsigned long long*)(a.part + (size_t)(BH > Shape<NQ>::SLOTS ? 0 : 2 * Shape<NQ>::SLOTS) * NQ * (D + 4));
     a.tag = call_tag();

@@ -194,3 +194,29 @@ def test_thresholds_of_short_sequences(D, tokens, alpha, kind):
     ku, vu = u16(K).reshape(3, tokens, D), u16(V).reshape(3, tokens, D)
     want = np.array([[*oracle.thresholds(ku[b], alpha), *oracle.thresholds(vu[b], alpha)] for b in range(3)], dtype=np.float32)
     assert np.array_equal(thr, want)
+
+
+@pytest.mark.parametrize("D,tokens", [(128, 513), (64, 576), (128, 1025), (32, 3650), (128, 4096)])
+def test_sequences_split_over_a_cluster(D, tokens):
+    # 9, 9, 17, 58 and 64 tiles: clusters of 2, 2, 3, 8 and 8 CTAs; then the same query with the token count in device memory, in
+    # clusters of the size that the capacity of 4160 tokens asks for, most of whose CTAs find nothing at 70 tokens
+    wl = synth.scaled(synth.CONFIGS["C2"], heads=2, head_dim=D, tokens=tokens)
+    K, V, q, ring, nv = make_inputs(wl, ragged=True)
+    pol = qaq.qaq_policy_from_hyper(*HYPER, tokens)
+    cfg, cache, thr, out, scores, dev = gpu_pipeline(wl, K, V, q, ring, nv, pol, max_tokens=4160)
+    ref = oracle_batch(wl, K, V, q, ring, nv, pol.cK, pol.cV)
+    assert_attention_close(out.cpu().numpy(), ref.X)
+    S = scores.cpu().numpy().astype(np.float64)
+    assert np.all(np.abs(S - ref.S) <= 1e-6 + 1e-2 * ref.S) and np.allclose(S.sum(1), 1.0, atol=1e-3)
+    for n in (tokens, 70):
+        if n != tokens:
+            cache.reset()
+            qaq.qaq_quantize_append(cache, dev[0][:, :, :n], dev[1][:, :, :n], thr, policy=pol, ring=dev[3][..., :n].contiguous(), nvalid=dev[4][..., :n].contiguous())
+        want = qaq.qaq_decode_attention(cache, dev[2], 1 / math.sqrt(D))
+        got, row = torch.empty_like(want), torch.empty((wl.bh, 4160), dtype=torch.float32, device="cuda")
+        qaq.qaq_stream_begin(cache)
+        qaq.qaq_stream_decode(cache, dev[2], 1 / math.sqrt(D), got, row)
+        qaq.qaq_stream_end(cache)
+        # the same tiles, summed in another order: binary32 rounding of at most 65 partial sums and weights
+        assert (got - want).abs().max().item() <= 65 * 2.0 ** -23 * 4 * V.abs().max().item()
+        assert torch.allclose(row[:, :n].sum(1), torch.ones(wl.bh, device="cuda"), atol=1e-3)
