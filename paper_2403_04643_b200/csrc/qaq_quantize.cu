@@ -66,9 +66,9 @@ __device__ __forceinline__ uint32_t pool_take(uint32_t* pool, uint32_t amount, u
 // What bounds it: instructions (70 % of the issue slots, 60 % of the integer unit's cycles at 7B, batch 8).  A kernel with
 // 256 threads per tile, a lane per 32 channels of a token throughout and an image of the tile in shared memory took
 // 7300 (keys) and 9100 (values) warp instructions per tile, this one 4200 on average.  4096 tokens, 256 (b,h), head_dim
-// 128: 188 us for keys and values, against 323 us; one warp per tile 231 us (11 tiles in flight per SM either way, for
-// their shared memory); rounds unrolled by two 200 us, by four 226 us (the code of one round is what the instruction
-// cache holds).  32 (b,h) of one tile 7.0 against 7.7 us, of 16 tiles 10.5 against 17.2 us.
+// 128: 173 us for keys and values, against 323 us; one warp per tile 231 us (as many tiles in flight per SM, for their
+// shared memory); rounds unrolled by two 7 % slower, by four 20 % (the code of one round is what the instruction cache
+// holds); the window in batches of 16 loads 3 % slower, eleven CTAs per SM 3 %.  32 (b,h) of one tile 7.0 against 7.7 us, of 16 tiles 10.5 against 17.2 us.
 // A one-token append is a chain of memory latencies (token count; table and metadata; the tile) and of instructions: four
 // warps share the rounds of pass 2, and nothing but the tile itself waits for the table.  32 (b,h), a tile of 1 to 64
 // tokens: 6.3 us, against 8.4 us with two warps and the window read in two parts, as much as the kernel of 256 threads.
@@ -109,9 +109,11 @@ constexpr uint32_t GONE = 0xFFFFu;      // in the place of an outlier of a token
 template <int D>
 struct TileScratch {
     alignas(64) uint8_t data[QAQ_TILE * D * 2];
-    uint4 slot[QAQ_TILE];              // by slot: minimum, 1 / step, byte offsets of the parts, what else a lane has to know
+    union {                            // one after the other
+        alignas(16) uint32_t out[QAQ_TILE * D / 32];   // by token and 32 channels: which are outliers
+        uint4 slot[QAQ_TILE];          // by slot: minimum, 1 / step, byte offsets of the parts, what else a lane has to know
+    };
     uint32_t range[QAQ_TILE];          // by token: min | max << 16
-    alignas(16) uint32_t out[QAQ_TILE * D / 32];  // by token and 32 channels: which are outliers
     alignas(8) uint32_t count[2][2];   // by half of the tile: tokens of every width, a byte each
     uint32_t nout[2], base[2];         // outliers of the halves; space taken for the tile and for its outlier list
     int skip;
@@ -216,7 +218,7 @@ __device__ __forceinline__ void quantize_tile(const QuantArgs& a, TileScratch<D>
     float shat = __int_as_float(0xff800000);
     if (IS_V && !given && main) {
         nv = min(nv, a.W);
-        shat = qaqc::window_max<OPEN ? 32 : 16>(a.ring + (size_t)bh * a.W * a.n_new + col, a.W, a.n_new, nv);
+        shat = qaqc::window_max<32>(a.ring + (size_t)bh * a.W * a.n_new + col, a.W, a.n_new, nv);
     }
     if (OPEN) {                        // the tile as it is stored follows on its own: it is needed later
         asm volatile("cp.async.commit_group;" ::: "memory");
@@ -466,7 +468,7 @@ __device__ __forceinline__ void quantize_tile(const QuantArgs& a, TileScratch<D>
 
 // dynamic shared memory: the scratch, the tile as it is stored (OPEN), the warps' lists of outliers
 template <int D, bool OPEN>
-__global__ void __launch_bounds__(OPEN ? 32 * OPEN_WARPS : 64, OPEN ? 4 : (D == 128 ? 11 : 12)) quant_tiles_kernel(const QuantArgs a, uint32_t cap) {
+__global__ void __launch_bounds__(OPEN ? 32 * OPEN_WARPS : 64, OPEN ? 4 : (12)) quant_tiles_kernel(const QuantArgs a, uint32_t cap) {
     extern __shared__ __align__(64) unsigned char tiles_smem[];
     TileScratch<D>& sm = *reinterpret_cast<TileScratch<D>*>(tiles_smem);
     uint8_t* stored_tile = tiles_smem + sizeof(TileScratch<D>);
@@ -479,8 +481,8 @@ __global__ void __launch_bounds__(OPEN ? 32 * OPEN_WARPS : 64, OPEN ? 4 : (D == 
 // tiles.x tiles of every (b,h), all whole, or one that is not (or may not be)
 template <int D, bool OPEN>
 qaq_status launch_tiles(int tiles, int BH, const QuantArgs& a, double alpha, cudaStream_t s) {
-    // the list holds a third more than the share of outliers asked for gives a tile, and some
-    const uint32_t want = (uint32_t)(alpha * (QAQ_TILE * D) * 1.34) + 96, cap = (want < 2048 ? want : 2048) / 2;
+    // the lists hold a tenth more than the share of outliers asked for gives a tile, and some (twelve CTAs per SM at 1 %)
+    const uint32_t want = (uint32_t)(alpha * (QAQ_TILE * D) * 1.1) + 60, cap = (want < 2048 ? want : 2048) / 2;
     const size_t smem = sizeof(TileScratch<D>) + (OPEN ? qaqc::tile_bytes_max(D) + 16 : 0) + 2 * cap * sizeof(uint32_t);
     static_assert(sizeof(TileScratch<D>) + qaqc::tile_bytes_max(D) + 16 + 2048 * sizeof(uint32_t) <= 48 * 1024, "shared memory that needs no attribute");
     QAQ_CUDA_TRY(qaq_launch(quant_tiles_kernel<D, OPEN>, dim3((unsigned)tiles, (unsigned)BH, 2), dim3(OPEN ? 32 * OPEN_WARPS : 64), smem, s, a, cap));

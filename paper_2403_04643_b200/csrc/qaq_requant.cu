@@ -22,8 +22,8 @@
 //
 // What bounds it: instructions, and where few tiles change the latency of the metadata and of the window.  With a thread per
 // 32 channels from the start, every tile of changed widths decoded to codes, encoded to an image and copied out, lowering
-// a 4096-token layer at batch 4 took 120 us and raising it again 170; as it is now 61 and 116.  With a step's few changes
-// (2048 tokens, batch 4) 29.6 us became 16.8.
+// a 4096-token layer at batch 4 took 120 us and raising it again 170; as it is now 55 and 103.  With a step's few changes
+// (2048 tokens, batch 4) 29.6 us became 15.9.
 #include "qaq_codec.cuh"
 #include "qaq_internal.cuh"
 
@@ -257,9 +257,10 @@ __device__ __forceinline__ void requantize_tile(const RequantArgs& a, RequantScr
     }
 }
 
-// blockIdx.z: keys or values
+// blockIdx.z: keys or values.  64 registers, 16 CTAs per SM: with 80 and 12 lowering a 4096-token layer at batch 4 takes 61
+// instead of 55 us, raising it 111 instead of 103; 51 and 20 are no better.
 template <int D, bool UP>
-__global__ void __launch_bounds__(64, 12) requant_kernel(const RequantArgs a) {
+__global__ void __launch_bounds__(64, 16) requant_kernel(const RequantArgs a) {
     __shared__ RequantScratch<D> sm;
     qaq_dependency();
     if (blockIdx.z == 0) requantize_tile<D, UP, false>(a, sm);
