@@ -254,7 +254,9 @@ __device__ __forceinline__ uint32_t bracket_rank(double alpha, uint32_t M) {
 }
 
 // ---- 1. sample: brackets (or the exact answer when the sample is the whole problem)
-__global__ void __launch_bounds__(256) thr_sample_kernel(const ThrArgs a) {
+template <int THREADS>
+__global__ void __launch_bounds__(THREADS) thr_sample_kernel(const ThrArgs a) {
+    constexpr int PIECES = SAMPLE_TOKENS * 128 / 8 / THREADS;            // 16-byte pieces of a thread at most
     qaq_dependency();
     const int bhx = blockIdx.x, bh = bhx >> 1, x = bhx & 1;
     __shared__ __align__(16) unsigned short s_keys[SAMPLE_TOKENS * 128];
@@ -266,18 +268,18 @@ __global__ void __launch_bounds__(256) thr_sample_kernel(const ThrArgs a) {
     if (threadIdx.x < 2) s_cnt[threadIdx.x] = 0;
     __syncthreads();
     uint32_t nn = 0, nneg = 0;                                  // NaNs, NaNs with the sign set
-    // all 16-byte pieces of a thread (four at most) are on their way before the first is looked at
-    uint4 raw[4];
+    // all 16-byte pieces of a thread are on their way before the first is looked at
+    uint4 raw[PIECES];
 #pragma unroll
-    for (int k = 0; k < 4; ++k) {
-        const int i = min((int)threadIdx.x + 256 * k, M / 8 - 1);
+    for (int k = 0; k < PIECES; ++k) {
+        const int i = min((int)threadIdx.x + THREADS * k, M / 8 - 1);
         const int sp = (i * 8) / a.D, c = (i * 8) % a.D;
         const long t = (long)sp * a.T / ns;                       // tokens spread over the sequence
         raw[k] = *reinterpret_cast<const uint4*>(X + (size_t)t * a.st + c);
     }
 #pragma unroll
-    for (int k = 0; k < 4; ++k) {
-        const int i = threadIdx.x + 256 * k;
+    for (int k = 0; k < PIECES; ++k) {
+        const int i = threadIdx.x + THREADS * k;
         if (i >= M / 8) break;
         uint32_t w[4] = {raw[k].x, raw[k].y, raw[k].z, raw[k].w};
 #pragma unroll
@@ -306,7 +308,7 @@ __global__ void __launch_bounds__(256) thr_sample_kernel(const ThrArgs a) {
         r_lo = r; r_hi = Mv - 1 - r;
     }
     uint32_t klo, khi;
-    cta_select_keys(s_keys, (uint32_t)M, r_lo + n_neg_nan, r_hi + n_neg_nan, hist, s_tmp, klo, khi);
+    cta_select_keys<THREADS>(s_keys, (uint32_t)M, r_lo + n_neg_nan, r_hi + n_neg_nan, hist, s_tmp, klo, khi);
     if (threadIdx.x == 0) {
         pr->klo = klo; pr->khi = khi; pr->cnt[0] = pr->cnt[1] = 0; pr->nan = 0; pr->overflow = 0; pr->n = 0; pr->done = whole ? 1u : 0u;
         if (whole) {
@@ -668,7 +670,10 @@ extern "C" qaq_status qaq_outlier_thresholds(const qaq_config* cfg, const void* 
         QAQ_CUDA_TRY(qaq_launch(thr_small_kernel, dim3(BH * 2), dim3(SMALL_THREADS), small, s, a));
         return QAQ_OK;
     }
-    QAQ_CUDA_TRY(qaq_launch(thr_sample_kernel, dim3(BH * 2), dim3(256), 0, s, a));
+    // 512 threads while a problem has an SM to itself or shares it with one (32 (b,h): 6.4 against 7.9 us), else 256 (256
+    // (b,h): 14.4 against 15.6)
+    if (BH * 2 <= 2 * 148) QAQ_CUDA_TRY(qaq_launch(thr_sample_kernel<512>, dim3(BH * 2), dim3(512), 0, s, a));
+    else QAQ_CUDA_TRY(qaq_launch(thr_sample_kernel<256>, dim3(BH * 2), dim3(256), 0, s, a));
     if (n_tokens > SAMPLE_TOKENS) {
         a.scan_tokens = scan_tokens_for(cfg->outlier_frac, cfg->head_dim, BH, n_tokens);
         dim3 grid((n_tokens + a.scan_tokens - 1) / a.scan_tokens, BH * 2);
