@@ -202,7 +202,8 @@ def _prepare_generate(c, seed):
         new.append(torch.stack([k1.permute(2, 0, 1, 3), v1.permute(2, 0, 1, 3), q1], dim=1))
         layers.append({"cache": qaq.Cache(cfg), "K": K, "V": V, "ring": ring, "nvalid": nvalid,
                        "thr": torch.empty((B * H, 4), dtype=torch.float32, device="cuda")})
-    s = {"case": c, "cfg": cfg, "layers": layers, "policy": policy, "step_in": step_in, "step_out": step_out,
+    # (the captured step reads no_score and no_rows at every replay: the program keeps them as long as the graph)
+    s = {"case": c, "cfg": cfg, "layers": layers, "policy": policy, "step_in": step_in, "step_out": step_out, "no_score": no_score, "no_rows": no_rows,
          "new": torch.stack(new, dim=1).contiguous(), "outs": torch.zeros((n, c["layers"], B * H, D), dtype=torch.float32, device="cuda")}
 
     def step():
