@@ -136,6 +136,11 @@ template <int NQ> struct Shape {
 };
 constexpr int SCORES_FUSED_TOKENS = 8192;          // up to here the CTA that merges a (b,h) normalises its score row too
 constexpr uint32_t LIST_STAGED = 1024;             // outlier entries per tile and tensor that come through shared memory at most; more are read in place
+// Tiles whose value sums may stay in the 32-bit accumulators.  The row blocks of high nibbles add most: bytes up to 240 times
+// digits up to 255, 64 tokens, once for the low four bits of a code (digits of the weight) and once for those above (digits of
+// 16 times the weight).  (Up to 500 tiles, the bound of one of the two, sums of 6- to 8-bit codes wrapped where weights were equal.)
+constexpr int HELD_TILES = 256;
+static_assert(2LL * QAQ_TILE * 255 * 240 * HELD_TILES < (1LL << 31), "sums of the held tiles");
 constexpr uint32_t SMALL_MAX = 0x5800u;            // 128 as binary16: up to here outlier terms are summed in one 32-bit word
 
 struct DecArgs {
@@ -749,7 +754,7 @@ __global__ void __launch_bounds__(Shape<NQ>::THREADS, Shape<NQ>::CTAS_PER_SM) de
     for (int pr = 0; pr < NP; ++pr)
 #pragma unroll
         for (int mb = 0; mb < MB; ++mb) { acc[pr][mb][0] = 0; acc[pr][mb][1] = 0; acc[pr][mb][2] = 0; acc[pr][mb][3] = 0; }
-    int held = 0;                // tiles in the accumulators: a tile adds less than 2^22 (64 tokens, 255 * 255), 500 of them fit
+    int held = 0;                // tiles in the accumulators, at most HELD_TILES
     float m_ref[NQ], wunit[NQ];  // exponentials are taken relative to this logit; weight of one fixed-point unit, a power of two
     float l_run[NQ], c_run[NQ];  // over this lane's tokens: sum of p, of p * (min + step/2) of the values
     auto flush = [&]() {
@@ -933,7 +938,7 @@ __global__ void __launch_bounds__(Shape<NQ>::THREADS, Shape<NQ>::CTAS_PER_SM) de
         //      set so that it takes 2^24 to 2^25.
         scalars(vt);
         float alpha[NQ], wnew[NQ];
-        bool wok[NQ], any_w = false, change = held == 500;
+        bool wok[NQ], any_w = false, change = held == HELD_TILES;
 #pragma unroll
         for (int j = 0; j < NQ; ++j) {
             const float m = warp_max(fmaxf(lg[j][0], lg[j][1]));
