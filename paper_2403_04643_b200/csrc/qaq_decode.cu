@@ -817,9 +817,10 @@ __global__ void __launch_bounds__(Shape<NQ>::THREADS, Shape<NQ>::CTAS_PER_SM) de
                 mid[i] = val[i] ? fmaf(0.5f, step[i], mn) : 0.f;
             }
         };
-        // the largest magnitude among this lane's ranges, as a binary16 pattern
+        // the largest magnitude among this lane's ranges, as a binary16 pattern (the places of tokens that are not there hold
+        // whatever the cache held before)
         auto top_range = [&](const Toks& tt) {
-            const uint32_t m = __vmaxu2(tt.mm.x & 0x7FFF7FFFu, tt.mm.y & 0x7FFF7FFFu);
+            const uint32_t m = __vmaxu2(val[0] ? tt.mm.x & 0x7FFF7FFFu : 0u, val[1] ? tt.mm.y & 0x7FFF7FFFu : 0u);
             return max(m & 0xFFFFu, m >> 16);
         };
         scalars(kt);

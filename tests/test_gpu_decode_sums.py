@@ -1,12 +1,17 @@
-"""GPU checks of what the decode kernels sum in integers."""
+"""GPU checks of what the decode kernels sum in integers: that long pieces of equal weights stay inside the 32-bit
+accumulators, and that the unit of the outlier sums follows from what is cached, not from what a cache held before."""
 import math
 
 import pytest
 import torch
 
-from paper_2403_04643_b200 import qaq
+from paper_2403_04643_b200 import qaq, synth
+
+from gpu_helpers import gpu_pipeline, make_inputs
 
 pytestmark = pytest.mark.gpu
+
+HYPER = (0.002, 0.01, 128.0)
 
 
 def test_value_sums_of_long_pieces_of_equal_weights():
@@ -38,3 +43,24 @@ def test_value_sums_of_long_pieces_of_equal_weights():
         for j in range(n_q):
             off = ((out[:, j] - rows.float()).abs() / step).max().item()
             assert off <= 0.51, (n_q, j, off)
+
+
+@pytest.mark.parametrize("tokens", [1, 100, 300])
+def test_a_reset_cache_gives_the_bits_of_a_fresh_one(tokens):
+    # the open tile of the second filling has places for tokens that the first one filled with values a thousand times larger
+    wl = synth.scaled(synth.CONFIGS["C2"], heads=3, tokens=tokens, alpha=0.05)
+    K, V, q, ring, nv = make_inputs(wl)
+    pol = qaq.qaq_policy_from_hyper(*HYPER, 320)
+    cfg, fresh, thr, out, scores, dev = gpu_pipeline(wl, K, V, q, ring, nv, pol, max_tokens=320)
+    used = qaq.Cache(cfg)
+    big = [torch.cat([x] * (320 // tokens + 1), dim=2)[:, :, :320].mul(1000).clamp(-60000, 60000).contiguous() for x in dev[:2]]
+    wide = torch.full((wl.bh, 320), 8, dtype=torch.uint8, device="cuda")
+    qaq.qaq_quantize_append(used, *big, qaq.qaq_outlier_thresholds(cfg, *big), bitsK=wide, bitsV=wide)
+    used.reset()
+    qaq.qaq_quantize_append(used, dev[0], dev[1], thr, policy=pol, ring=dev[3], nvalid=dev[4])
+    row = torch.empty_like(scores)
+    assert torch.equal(qaq.qaq_decode_attention(used, dev[2], 1 / math.sqrt(wl.head_dim), scores_out=row), out)
+    assert torch.equal(row, scores)
+    q4 = torch.stack([synth.make_query(wl, step=i).view(wl.bh, -1) for i in range(4)], dim=1).cuda().contiguous()
+    a, b = (qaq.qaq_decode_attention_multi(c, q4, 1 / math.sqrt(wl.head_dim)) for c in (fresh, used))
+    assert torch.equal(a, b)
