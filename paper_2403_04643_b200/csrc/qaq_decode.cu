@@ -243,9 +243,9 @@ template <int D, int NQ>
 struct DecSmem {
     static constexpr int W = Shape<NQ>::WARPS;
     WarpScratch<D, NQ> ws[W];
-    alignas(16) float qf[2][D][NQ];           // the queries of the run's two (b,h)
+    alignas(16) float qf[2][D][NQ];           // the queries of the run's two (b,h), each over its power of two (largest entry in [1, 2))
     alignas(16) uint32_t qw[2][2][32][D / 32];// operand words of q per lane: low nibbles of its words, high nibbles
-    float qscale[2][NQ], qsum[2][NQ];
+    float qscale[2][NQ], qsum[2][NQ], qpow[2][NQ];
     // results of the warps; the warp that meets the (b,h) boundary leaves what it has of the first one in entry W
     float cross[NQ][D];
     float mm[W + 1][NQ], ml[W + 1][NQ], cs[W + 1][NQ];
@@ -385,7 +385,8 @@ __device__ __forceinline__ int v_channel(int mb, int g, int s) {
 
 // ------------------------------------------------------------------------------------------ outlier sums
 // Outlier terms are summed in fixed point.  Where all values of a tile are small (up to 128) one word is enough: a unit
-// is 2^-22 of a bound on the largest term, so that the 128 terms a token can have (64 per channel) stay inside 32 bits.
+// is 2^-24 of a bound on the largest term, so that a channel's 64 terms stay inside 32 bits, and a token's 127 (128 have half
+// of the bound: without an inlier the minimum is 0).  The bound of a query's terms is its own, whatever queries share the pass.
 // Otherwise a term is a high part in units of 2^-4 and the exact remainder in units of 2^-28; terms of 2^18 or more (and
 // non-finite ones) are left out.
 constexpr float OC_LIMIT = 262144.0f;
@@ -398,11 +399,11 @@ __device__ __forceinline__ void wide_add(int* hi_cell, int* lo_cell, float tm) {
     }
 }
 __device__ __forceinline__ float wide_sum(int hi, int lo) { return fmaf((float)lo, 1.0f / 268435456.0f, (float)hi * 0.0625f); }
-// 2^22 over a power of two above x (x > 0, normal), and its inverse
+// 2^24 over a power of two above x (x > 0, normal), and its inverse
 __device__ __forceinline__ void fixed_unit(float x, float& inv, float& unit) {
     const int ex = min(max((__float_as_int(x) >> 23) & 0xFF, 40), 240);
-    inv = __int_as_float((254 - ex - 1 + 22) << 23);
-    unit = __int_as_float((ex + 1 - 22) << 23);
+    inv = __int_as_float((254 - ex - 1 + 24) << 23);
+    unit = __int_as_float((ex + 1 - 24) << 23);
 }
 
 // What of a tile's outlier list did not fit into the staging buffer (entries from..to, dense wide tiles only), read in
@@ -711,13 +712,15 @@ __global__ void __launch_bounds__(Shape<NQ>::THREADS, Shape<NQ>::CTAS_PER_SM) de
             float qmax = 0.f, qs = 0.f;
 #pragma unroll
             for (int i = 0; i < 4; ++i) { const float x = half_at(qrow[sg][j], i); qmax = fmaxf(qmax, fabsf(x)); qs += x; }
-            qsc[sg][j] = warp_max(qmax) / 32639.0f;             // |q| <= 32639 units: both byte digits of 256 * hi + lo stay signed bytes
+            qmax = warp_max(qmax);
+            qsc[sg][j] = qmax / 32639.0f;                       // |q| <= 32639 units: both byte digits of 256 * hi + lo stay signed bytes
             if (warp == (sg * NQ + j) % S::WARPS && sg < nseg) {
                 qs = warp_sum(qs);
-                if (lane == 0) { sm.qscale[sg][j] = qsc[sg][j]; sm.qsum[sg][j] = qs; }
+                const int qex = __float_as_int(qmax) >> 23, ex = qex == 0 || qex == 255 ? 127 : qex;       // (no power of two for zero and infinity)
+                if (lane == 0) { sm.qscale[sg][j] = qsc[sg][j]; sm.qsum[sg][j] = qs; sm.qpow[sg][j] = __int_as_float(ex << 23); }
                 if (4 * lane < D)
 #pragma unroll
-                    for (int i = 0; i < 4; ++i) sm.qf[sg][4 * lane + i][j] = half_at(qrow[sg][j], i);
+                    for (int i = 0; i < 4; ++i) sm.qf[sg][4 * lane + i][j] = half_at(qrow[sg][j], i) * __int_as_float((254 - ex) << 23);
             }
         }
 #pragma unroll
@@ -784,12 +787,11 @@ __global__ void __launch_bounds__(Shape<NQ>::THREADS, Shape<NQ>::CTAS_PER_SM) de
 #pragma unroll 1
     while (f < f_end) {          // once per (b,h) of the warp's piece: one or two times
     const int bh = bh_of(f), seg = bh - bh0, f_stop = seg ? f_end : min(f_end, f_bound);
-    float qscale[NQ], qsum[NQ], qtop = 0.f;
+    float qscale[NQ], qsum[NQ];
 #pragma unroll
     for (int j = 0; j < NQ; ++j) {
         qscale[j] = sm.qscale[seg][j];
         qsum[j] = sm.qsum[seg][j];
-        qtop = fmaxf(qtop, qscale[j] * 32639.0f);
         m_ref[j] = NEG; wunit[j] = 0.f; l_run[j] = 0.f; c_run[j] = 0.f;
     }
 #pragma unroll 1
@@ -850,7 +852,7 @@ __global__ void __launch_bounds__(Shape<NQ>::THREADS, Shape<NQ>::CTAS_PER_SM) de
             }
         }
         // ---- key outliers: q_ch * (x - mid) per token; up to 128 entries stay in registers between the two looks at them
-        float kunit = 0.f;          // > 0: the corrections are one word in this unit; < 0: two words
+        float kunit = 0.f;          // > 0: the corrections are one word in this unit (of a query over its power of two); < 0: two words
         if (tk.w && landed) {
             const uint32_t oc = tk.w, sc = min(min(oc, LIST_STAGED), lk.lb / 4 - (tk.z & 3u));       // entries, of which staged
             const uint32_t* list = reinterpret_cast<const uint32_t*>(ws.buf + lk.nb) + (tk.z & 3u);
@@ -874,7 +876,7 @@ __global__ void __launch_bounds__(Shape<NQ>::THREADS, Shape<NQ>::CTAS_PER_SM) de
             top = sc == oc ? __reduce_max_sync(0xFFFFFFFFu, top) : SMALL_MAX + 1;
             if (top <= SMALL_MAX) {
                 float inv;
-                fixed_unit(qtop * 2.0f * __half2float(__ushort_as_half((unsigned short)top)), inv, kunit);
+                fixed_unit(4.0f * __half2float(__ushort_as_half((unsigned short)top)), inv, kunit);       // |q| < 2, |x - mid| <= 2 top
                 auto add = [&](uint32_t v, bool there) {
                     int tok; float tm[NQ];
                     term(v, inv, tok, tm);
@@ -896,7 +898,7 @@ __global__ void __launch_bounds__(Shape<NQ>::THREADS, Shape<NQ>::CTAS_PER_SM) de
                     int tok; float tm[NQ];
                     term(v, 1.0f, tok, tm);
 #pragma unroll
-                    for (int j = 0; j < NQ; ++j) wide_add(&ws.kcorr[j][0][tok], &ws.kcorr[j][1][tok], tm[j]);
+                    for (int j = 0; j < NQ; ++j) wide_add(&ws.kcorr[j][0][tok], &ws.kcorr[j][1][tok], tm[j] * sm.qpow[seg][j]);
                 };
 #pragma unroll 1
                 for (uint32_t i = lane; i < sc; i += 32) add(list[i]);
@@ -909,7 +911,8 @@ __global__ void __launch_bounds__(Shape<NQ>::THREADS, Shape<NQ>::CTAS_PER_SM) de
 #pragma unroll
         for (int j = 0; j < NQ; ++j) {
             const int2 k0 = *reinterpret_cast<const int2*>(&ws.kcorr[j][0][2 * lane]);
-            float kc[2] = {(float)k0.x * kunit, (float)k0.y * kunit};
+            const float ku = kunit * sm.qpow[seg][j];
+            float kc[2] = {(float)k0.x * ku, (float)k0.y * ku};
             if (kunit < 0.f) {
                 const int2 k1 = *reinterpret_cast<const int2*>(&ws.kcorr[j][1][2 * lane]);
                 kc[0] = wide_sum(k0.x, k1.x); kc[1] = wide_sum(k0.y, k1.y);

@@ -1,5 +1,6 @@
 """GPU checks of what the decode kernels sum in integers: that long pieces of equal weights stay inside the 32-bit
-accumulators, and that the unit of the outlier sums follows from what is cached, not from what a cache held before."""
+accumulators, and that the unit of the outlier sums follows from what is cached and from the query itself, not from what a
+cache held before or from the queries beside it."""
 import math
 
 import pytest
@@ -64,3 +65,21 @@ def test_a_reset_cache_gives_the_bits_of_a_fresh_one(tokens):
     q4 = torch.stack([synth.make_query(wl, step=i).view(wl.bh, -1) for i in range(4)], dim=1).cuda().contiguous()
     a, b = (qaq.qaq_decode_attention_multi(c, q4, 1 / math.sqrt(wl.head_dim)) for c in (fresh, used))
     assert torch.equal(a, b)
+
+
+@pytest.mark.parametrize("D", [32, 64, 128])
+@pytest.mark.parametrize("beside", [2000.0, math.inf, math.nan])
+def test_a_query_gives_what_it_gives_alone_whatever_is_beside_it(D, beside):
+    wl = synth.scaled(synth.CONFIGS["C2"], heads=3, head_dim=D, tokens=700, alpha=0.05)
+    K, V, q, ring, nv = make_inputs(wl)
+    pol = qaq.qaq_policy_from_hyper(*HYPER, 700)
+    cfg, cache, thr, out, scores, dev = gpu_pipeline(wl, K, V, q, ring, nv, pol)
+    one = dev[2].view(wl.bh, D)
+    for n_q in (2, 4, 8):
+        qs = torch.stack([synth.make_query(wl, step=i).view(wl.bh, D) for i in range(n_q)], dim=1).cuda()
+        qs[:, 1] = (qs[:, 1] * beside).half()
+        qs[:, 0] = one
+        got = qaq.qaq_decode_attention_multi(cache, qs.contiguous(), 1 / math.sqrt(D))[:, 0]
+        # the same integer products, key corrections and weights; the accumulators are emptied at other tiles (11 of them), so
+        # binary32 sums differ in their order
+        assert (got - out).abs().max().item() <= 11 * 2.0 ** -22 * V.abs().max().item()
