@@ -952,8 +952,9 @@ __global__ void __launch_bounds__(Shape<NQ>::THREADS, Shape<NQ>::CTAS_PER_SM) de
                 m_ref[j] = m + 3.0f;
                 change = true;
             }
-            lg[j][0] = __expf(lg[j][0] - m_ref[j]);              // from here on: p (0 for slots beyond T)
-            lg[j][1] = __expf(lg[j][1] - m_ref[j]);
+            // from here on: p (0 for slots beyond T, and for a token whose logit is not a number: one with an infinite range)
+            lg[j][0] = fmaxf(__expf(lg[j][0] - m_ref[j]), 0.f);
+            lg[j][1] = fmaxf(__expf(lg[j][1] - m_ref[j]), 0.f);
             const float wmax = warp_max(fmaxf(lg[j][0] * step[0], lg[j][1] * step[1]));
             const int wex = (__float_as_int(wmax) >> 23) & 0xFF;
             wok[j] = wex > 28 && wex < 255 && tv.y;             // zero, tiny or non-finite weights: the codes add nothing

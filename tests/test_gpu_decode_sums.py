@@ -83,3 +83,26 @@ def test_a_query_gives_what_it_gives_alone_whatever_is_beside_it(D, beside):
         # the same integer products, key corrections and weights; the accumulators are emptied at other tiles (11 of them), so
         # binary32 sums differ in their order
         assert (got - out).abs().max().item() <= 11 * 2.0 ** -22 * V.abs().max().item()
+
+
+@pytest.mark.parametrize("n_q", [1, 2, 4])
+def test_a_token_whose_logit_is_not_a_number_takes_no_part(n_q):
+    # keys with infinities of both signs that are no outliers have no midpoint; the result is that of the other tokens
+    D, BH, T = 64, 3, 210
+    g = torch.Generator().manual_seed(1)
+    K, V = (torch.randn((1, BH, T, D), generator=g).half() for _ in range(2))
+    lost = torch.zeros(T, dtype=torch.bool)
+    lost[[0, 7, 63, 64, 140, 141, 209]] = True
+    K[:, :, lost, 5] = math.inf
+    K[:, :, lost, 9] = -math.inf
+    cfg = qaq.make_config(1, BH, D, T, 1, 8, 1, 0.0)
+    thr = torch.tensor([-math.inf, math.inf] * 2).repeat(BH, 1).cuda().contiguous()
+    q = torch.randn((BH, n_q, D), generator=g).half().cuda()
+    outs = []
+    for keep in (torch.ones(T, dtype=torch.bool), ~lost):
+        cache, n = qaq.Cache(cfg), int(keep.sum())
+        bits = torch.full((BH, n), 5, dtype=torch.uint8, device="cuda")
+        qaq.qaq_quantize_append(cache, K[:, :, keep].cuda().contiguous(), V[:, :, keep].cuda().contiguous(), thr, bitsK=bits, bitsV=bits)
+        outs.append(qaq.qaq_decode_attention_multi(cache, q, 1 / math.sqrt(D)))
+    # the same tokens in other tiles: binary32 sums of 210 weights in another order, weights of 21 bits or more
+    assert (outs[0] - outs[1]).abs().max().item() <= 210 * 2.0 ** -22 * V.abs().max().item()
