@@ -243,9 +243,10 @@ template <int D, int NQ>
 struct DecSmem {
     static constexpr int W = Shape<NQ>::WARPS;
     WarpScratch<D, NQ> ws[W];
-    alignas(16) float qf[2][D][NQ];           // the queries of the run's two (b,h), each over its power of two (largest entry in [1, 2))
+    // the queries of the run's two (b,h); several: each over a power of two (its largest entry below 2), which is behind them
+    alignas(16) float qf[2][D + (NQ > 1)][NQ];
     alignas(16) uint32_t qw[2][2][32][D / 32];// operand words of q per lane: low nibbles of its words, high nibbles
-    float qscale[2][NQ], qsum[2][NQ], qpow[2][NQ];
+    float qscale[2][NQ], qsum[2][NQ];
     // results of the warps; the warp that meets the (b,h) boundary leaves what it has of the first one in entry W
     float cross[NQ][D];
     float mm[W + 1][NQ], ml[W + 1][NQ], cs[W + 1][NQ];
@@ -712,15 +713,19 @@ __global__ void __launch_bounds__(Shape<NQ>::THREADS, Shape<NQ>::CTAS_PER_SM) de
             float qmax = 0.f, qs = 0.f;
 #pragma unroll
             for (int i = 0; i < 4; ++i) { const float x = half_at(qrow[sg][j], i); qmax = fmaxf(qmax, fabsf(x)); qs += x; }
-            qmax = warp_max(qmax);
-            qsc[sg][j] = qmax / 32639.0f;                       // |q| <= 32639 units: both byte digits of 256 * hi + lo stay signed bytes
+            qsc[sg][j] = warp_max(qmax) / 32639.0f;             // |q| <= 32639 units: both byte digits of 256 * hi + lo stay signed bytes
             if (warp == (sg * NQ + j) % S::WARPS && sg < nseg) {
                 qs = warp_sum(qs);
-                const int qex = __float_as_int(qmax) >> 23, ex = qex == 0 || qex == 255 ? 127 : qex;       // (no power of two for zero and infinity)
-                if (lane == 0) { sm.qscale[sg][j] = qsc[sg][j]; sm.qsum[sg][j] = qs; sm.qpow[sg][j] = __int_as_float(ex << 23); }
+                if (lane == 0) { sm.qscale[sg][j] = qsc[sg][j]; sm.qsum[sg][j] = qs; }
+                float over = 1.0f;
+                if constexpr (NQ > 1) {
+                    const int e = __float_as_int(qsc[sg][j]) >> 23, ex = e == 0 || e == 255 ? 127 : e + 15;       // 32639 < 2^15; zero and infinity have no power of two
+                    over = __int_as_float((254 - ex) << 23);
+                    if (lane == 0) sm.qf[sg][D][j] = __int_as_float(ex << 23);
+                }
                 if (4 * lane < D)
 #pragma unroll
-                    for (int i = 0; i < 4; ++i) sm.qf[sg][4 * lane + i][j] = half_at(qrow[sg][j], i) * __int_as_float((254 - ex) << 23);
+                    for (int i = 0; i < 4; ++i) sm.qf[sg][4 * lane + i][j] = half_at(qrow[sg][j], i) * over;
             }
         }
 #pragma unroll
@@ -787,11 +792,12 @@ __global__ void __launch_bounds__(Shape<NQ>::THREADS, Shape<NQ>::CTAS_PER_SM) de
 #pragma unroll 1
     while (f < f_end) {          // once per (b,h) of the warp's piece: one or two times
     const int bh = bh_of(f), seg = bh - bh0, f_stop = seg ? f_end : min(f_end, f_bound);
-    float qscale[NQ], qsum[NQ];
+    float qscale[NQ], qsum[NQ], qtop = NQ == 1 ? 0.f : 2.0f;       // qtop: a bound on the entries of the queries as they are kept
 #pragma unroll
     for (int j = 0; j < NQ; ++j) {
         qscale[j] = sm.qscale[seg][j];
         qsum[j] = sm.qsum[seg][j];
+        if (NQ == 1) qtop = fmaxf(qtop, qscale[j] * 32639.0f);
         m_ref[j] = NEG; wunit[j] = 0.f; l_run[j] = 0.f; c_run[j] = 0.f;
     }
 #pragma unroll 1
@@ -876,7 +882,7 @@ __global__ void __launch_bounds__(Shape<NQ>::THREADS, Shape<NQ>::CTAS_PER_SM) de
             top = sc == oc ? __reduce_max_sync(0xFFFFFFFFu, top) : SMALL_MAX + 1;
             if (top <= SMALL_MAX) {
                 float inv;
-                fixed_unit(4.0f * __half2float(__ushort_as_half((unsigned short)top)), inv, kunit);       // |q| < 2, |x - mid| <= 2 top
+                fixed_unit(qtop * 2.0f * __half2float(__ushort_as_half((unsigned short)top)), inv, kunit);        // |x - mid| <= 2 top
                 auto add = [&](uint32_t v, bool there) {
                     int tok; float tm[NQ];
                     term(v, inv, tok, tm);
@@ -898,7 +904,7 @@ __global__ void __launch_bounds__(Shape<NQ>::THREADS, Shape<NQ>::CTAS_PER_SM) de
                     int tok; float tm[NQ];
                     term(v, 1.0f, tok, tm);
 #pragma unroll
-                    for (int j = 0; j < NQ; ++j) wide_add(&ws.kcorr[j][0][tok], &ws.kcorr[j][1][tok], tm[j] * sm.qpow[seg][j]);
+                    for (int j = 0; j < NQ; ++j) wide_add(&ws.kcorr[j][0][tok], &ws.kcorr[j][1][tok], tm[j] * (NQ == 1 ? 1.0f : sm.qf[seg][D][j]));
                 };
 #pragma unroll 1
                 for (uint32_t i = lane; i < sc; i += 32) add(list[i]);
@@ -911,7 +917,7 @@ __global__ void __launch_bounds__(Shape<NQ>::THREADS, Shape<NQ>::CTAS_PER_SM) de
 #pragma unroll
         for (int j = 0; j < NQ; ++j) {
             const int2 k0 = *reinterpret_cast<const int2*>(&ws.kcorr[j][0][2 * lane]);
-            const float ku = kunit * sm.qpow[seg][j];
+            const float ku = NQ == 1 ? kunit : kunit * sm.qf[seg][D][j];
             float kc[2] = {(float)k0.x * ku, (float)k0.y * ku};
             if (kunit < 0.f) {
                 const int2 k1 = *reinterpret_cast<const int2*>(&ws.kcorr[j][1][2 * lane]);
