@@ -23,7 +23,7 @@ struct TensorStore {
     uint32_t* mnmx;         // [BH][tmax_pad]  half(min) | half(max) << 16
     uint4* tile;            // [BH][ntiles]    byte offset of the tile in its pool, bytes, first outlier entry, outlier entries
     uint32_t* outl;         // [BH][ocap]
-    uint32_t* pool_end;     // [BH] bump pointer, bytes
+    uint32_t* pool_end;     // [BH] bump pointer, bytes; a multiple of 16 unless the last thing before it is the open tile
     uint32_t* opool_end;    // [BH] bump pointer, entries
 };
 

@@ -336,13 +336,14 @@ __device__ __forceinline__ void quantize_tile(const QuantArgs& a, TileScratch<D>
         if (OPEN) {
             // nobody else is at these pools: a tile that is begun goes to the end, one that is continued has to be the last
             // thing before it (an open tile that re-quantization could not keep there, in a full pool, cannot grow); what is
-            // closed takes a rounded amount
+            // closed takes a rounded amount, and one that would have been closed leaves the end where the next tile can begin
             const uint32_t pool_end = __shfl_sync(0xFFFFFFFFu, pool_now, 0), opool_end = __shfl_sync(0xFFFFFFFFu, pool_now, 1);
-            const uint32_t off = s_lo ? tw.x : pool_end, end = s_hi == QAQ_TILE ? (off + total + 15u) & ~15u : off + total;
+            const uint32_t next = (pool_end + 15u) & ~15u;
+            const uint32_t off = s_lo ? tw.x : next, end = s_hi == QAQ_TILE ? (off + total + 15u) & ~15u : off + total;
             fail = pool_end > a.pool_bytes || (size_t)end + 16 > a.pool_bytes || (s_lo && pool_end != tw.x + tw.y);
             const bool full = opool_end > a.ocap;
             base = lane == 0 ? off : (full ? 0xFFFF0000u : opool_end);
-            if (lane == 0 && !fail) *pool = end;
+            if (lane == 0 && (!fail || s_hi == QAQ_TILE)) *pool = fail ? next : end;
             if (lane == 1 && !fail && !full) *pool = s_hi == QAQ_TILE ? (opool_end + nall + 3u) & ~3u : opool_end + nall;
         } else {
             const uint32_t off = __shfl_sync(0xFFFFFFFFu, base, 0);

@@ -173,7 +173,7 @@ __device__ __forceinline__ void requantize_tile(const RequantArgs& a, RequantScr
                 // in the pool again (one CTA per pool does this, and nobody else touches the pool in its launch)
                 noff = (pool_end + 15u) & ~15u;
                 if ((size_t)noff + nb + 16 > a.pool_bytes) skip = 1;
-                else ts.pool_end[bh] = noff + nb;
+                ts.pool_end[bh] = skip ? noff : noff + nb;         // (without room: where whole tiles can begin)
             } else {
                 // the end of the pool need not be aligned while a tile is open: take 16 bytes more and align;
                 // space that does not fit is given back
