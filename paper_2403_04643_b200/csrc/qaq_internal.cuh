@@ -35,7 +35,7 @@ struct qaq_cache {
     size_t pool_bytes;  // per (b,h)
     uint32_t ocap;      // outlier entries per (b,h)
     TensorStore t[2];
-    int* d_status;      // sticky device-side status; the two words behind it: see qaq_d_count / qaq_d_ticket
+    int* d_status;      // sticky device-side status; the words behind it: qaq_d_count, qaq_d_ticket, qaq_d_pool_use
     void* slab;         // the one allocation everything above lives in
     size_t slab_bytes;
     size_t reset_off, reset_bytes;   // the range of the slab that qaq_cache_reset clears
@@ -58,6 +58,8 @@ extern int g_qaq_last_cuda_error;
 // qaq_stream_end), and the arrival counter of the kernel that advances it (zero between launches)
 static inline int* qaq_d_count(const qaq_cache* c) { return c->d_status + 1; }
 static inline unsigned* qaq_d_ticket(const qaq_cache* c) { return (unsigned*)(c->d_status + 2); }
+// two words for what qaq_cache_pool_use finds
+static inline unsigned* qaq_d_pool_use(const qaq_cache* c) { return (unsigned*)(c->d_status + 4); }
 
 #ifdef __CUDACC__
 // Kernels of this library are launched with programmatic dependent launch: the launch of a kernel is prepared while the

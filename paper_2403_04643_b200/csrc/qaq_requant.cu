@@ -467,7 +467,7 @@ extern "C" qaq_status qaq_cache_compact(qaq_cache* c, void* stream) {
 extern "C" qaq_status qaq_cache_pool_use(const qaq_cache* c, long* host_used, long* host_capacity, void* stream) {
     if (!c || !host_used) return QAQ_ERR_INVALID_ARG;
     cudaStream_t s = (cudaStream_t)stream;
-    unsigned int* d = (unsigned int*)c->d_status + 2;      // two spare words behind the status word
+    unsigned int* d = qaq_d_pool_use(c);
     QAQ_CUDA_TRY(cudaMemsetAsync(d, 0, 8, s));
     pool_use_kernel<<<32, 256, 0, s>>>(c->t[0], c->t[1], c->BH, (unsigned)c->pool_bytes, d);
     QAQ_CUDA_TRY(cudaGetLastError());

@@ -57,3 +57,27 @@ def test_tiles_behind_an_open_tile_that_found_no_room(first, open_bits, moves, h
                 if want[t]:
                     i, j, n = int(got["off"][bh, t]), int(ref["off"][bh, t]), D * want[t] // 8
                     assert torch.equal(got["codes"][bh, i:i + n], ref["codes"][bh, j:j + n]), (x, bh, t)
+
+
+def test_pool_use_between_the_steps_of_a_stream():
+    # asked for between two one-token appends it leaves the count and its arrival counter alone: every token is where it belongs
+    D, BH, T0, n = 64, 5, 60, 9
+    g = torch.Generator().manual_seed(4)
+    K, V = (torch.randn((1, BH, T0 + n, D), generator=g).half().cuda() for _ in range(2))
+    thr = torch.tensor([-2.5, 2.5] * 2).repeat(BH, 1).cuda().contiguous()
+    cfg = qaq.make_config(1, BH, D, T0 + n, 1, 8, 1, 0.05)
+    bits = torch.randint(1, 9, (BH, T0 + n), generator=g, dtype=torch.uint8).cuda()
+    one, whole = qaq.Cache(cfg), qaq.Cache(cfg)
+    qaq.qaq_quantize_append(whole, K, V, thr, bitsK=bits, bitsV=bits)
+    first = bits[:, :T0].contiguous()
+    qaq.qaq_quantize_append(one, K[:, :, :T0], V[:, :, :T0], thr, bitsK=first, bitsV=first)
+    qaq.qaq_stream_begin(one)
+    for t in range(T0, T0 + n):
+        b = bits[:, t:t + 1].contiguous()
+        qaq.qaq_stream_append(one, K[:, :, t:t + 1], V[:, :, t:t + 1], thr, bitK=b, bitV=b)
+        use = qaq.qaq_cache_pool_use(one)
+        assert 0 < use[0] <= use[2] and 0 < use[1] <= use[2]
+    assert qaq.qaq_stream_end(one) == T0 + n
+    for x in range(2):
+        a, b = qaq.qaq_cache_export(one, x), qaq.qaq_cache_export(whole, x)
+        assert all(torch.equal(a[k], b[k]) for k in ("bits", "off", "codes", "rowptr", "ch"))
