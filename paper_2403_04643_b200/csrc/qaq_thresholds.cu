@@ -7,9 +7,10 @@
 //                          small enough to be sampled completely are solved right here.
 //   2. thr_scan_kernel     the one pass over all values: entries beyond the brackets ("candidates",
 //                          a few per cent) are compacted into per-problem lists (shared-memory lists
-//                          per CTA, one global reservation per CTA and tail), NaNs are counted.
+//                          per CTA, one global reservation per CTA; what a CTA's list does not hold goes to
+//                          the problem's directly), NaNs are counted.
 //   3. thr_select_kernel   exact radix select of rank k inside the candidate lists.  If a bracket
-//                          turned out too tight (fewer than k+1 candidates) or a list overflowed, the
+//                          turned out too tight (fewer than k+1 candidates) or a problem's list overflowed, the
 //                          problem is redone exactly by a two-pass radix select over its data, so the
 //                          result is always the exact order statistic.
 // binary16 patterns are mapped to 16-bit keys that sort like the values.
@@ -20,7 +21,7 @@ namespace {
 constexpr int SAMPLE_TOKENS = 64;
 constexpr int SCAN_TOKENS_MAX = 1024; // tokens per CTA of the scan (fewer where alpha is large: see scan_tokens_for)
 constexpr int WARP_FLAGS = 192;      // 16-byte pieces a warp of the scan can set aside before it has to look at them
-constexpr int CTA_LIST = 8192;       // candidates a scan CTA can hold
+constexpr int CTA_LIST = 8192;       // candidates a scan CTA can hold (see scan_tokens_for)
 constexpr int SELECT_KEYS = 16384;   // candidates the select kernel keeps in shared memory
 
 __device__ __forceinline__ uint32_t key_of(unsigned short h) { return (h & 0x8000u) ? (uint32_t)(~h & 0xFFFFu) : (uint32_t)(h | 0x8000u); }
@@ -34,8 +35,8 @@ struct Problem {          // per (b,h,tensor), in the workspace
     uint32_t cnt[2];      // candidates found below and above (their sum may exceed the capacity: then the list is incomplete)
     uint32_t nan;         // NaN entries seen by the scan
     uint32_t done;        // solved by the sample kernel
-    uint32_t overflow;    // a scan CTA found more candidates than it can hold, the list has holes
     uint32_t n;           // places taken in the list
+    uint32_t pad;
 };
 
 struct ThrArgs {
@@ -294,7 +295,7 @@ __global__ void __launch_bounds__(THREADS) thr_sample_kernel(const ThrArgs a) {
     const bool whole = (ns == a.T);
     if (Mv == 0) {
         if (threadIdx.x == 0) {
-            pr->klo = 0; pr->khi = 0xFFFF; pr->cnt[0] = pr->cnt[1] = 0; pr->nan = 0; pr->overflow = 0; pr->n = 0; pr->done = whole ? 1u : 0u;
+            pr->klo = 0; pr->khi = 0xFFFF; pr->cnt[0] = pr->cnt[1] = 0; pr->nan = 0; pr->n = 0; pr->done = whole ? 1u : 0u;
             if (whole) { a.thr[(size_t)bh * 4 + 2 * x] = 0.f; a.thr[(size_t)bh * 4 + 2 * x + 1] = 0.f; }
         }
         return;
@@ -310,7 +311,7 @@ __global__ void __launch_bounds__(THREADS) thr_sample_kernel(const ThrArgs a) {
     uint32_t klo, khi;
     cta_select_keys<THREADS>(s_keys, (uint32_t)M, r_lo + n_neg_nan, r_hi + n_neg_nan, hist, s_tmp, klo, khi);
     if (threadIdx.x == 0) {
-        pr->klo = klo; pr->khi = khi; pr->cnt[0] = pr->cnt[1] = 0; pr->nan = 0; pr->overflow = 0; pr->n = 0; pr->done = whole ? 1u : 0u;
+        pr->klo = klo; pr->khi = khi; pr->cnt[0] = pr->cnt[1] = 0; pr->nan = 0; pr->n = 0; pr->done = whole ? 1u : 0u;
         if (whole) {
             a.thr[(size_t)bh * 4 + 2 * x] = float_of_key(klo);
             a.thr[(size_t)bh * 4 + 2 * x + 1] = float_of_key(khi);
@@ -352,6 +353,7 @@ __global__ void __launch_bounds__(256) thr_scan_kernel(const ThrArgs a) {
     const __half* ptr = (x ? a.X[1] : a.X[0]) + (size_t)b_idx * a.sb + (size_t)h_idx * a.sh + (size_t)(t0 + tok) * a.st +
                         (((int)threadIdx.x & ((1 << tok_shift) - 1)) << 3);
     const size_t ptr_step = (size_t)tok_step * a.st;
+    unsigned short* const dst = a.list + (size_t)bhx * a.cap;
     uint4* wflag = s_flag[warp];
     uint32_t nflag = 0;      // pieces set aside by this warp (the same in all its lanes)
     uint32_t nnan = 0, nlow = 0;
@@ -416,9 +418,15 @@ __global__ void __launch_bounds__(256) thr_scan_kernel(const ThrArgs a) {
                 const uint32_t t = __shfl_up_sync(0xFFFFFFFFu, inc, d);
                 if (lane >= d) inc += t;
             }
-            uint32_t b0 = 0;
-            if (lane == 31 && inc) b0 = atomicAdd(&s_n, inc);
+            uint32_t b0 = 0, g0 = 0;
+            if (lane == 31 && inc) {
+                b0 = atomicAdd(&s_n, inc);
+                // beyond the CTA's list: entry `pos` goes to place g0 + pos of the problem's
+                const uint32_t from = max(b0, (uint32_t)CTA_LIST);
+                if (b0 + inc > from) g0 = atomicAdd(&pr->n, b0 + inc - from) - from;
+            }
             uint32_t pos = __shfl_sync(0xFFFFFFFFu, b0, 31) + inc - mine;
+            g0 = __shfl_sync(0xFFFFFFFFu, g0, 31);
             while (m) {
                 const int bit = __ffs(m) - 1;
                 m &= m - 1;
@@ -426,6 +434,7 @@ __global__ void __launch_bounds__(256) thr_scan_kernel(const ThrArgs a) {
                 const uint32_t wj = (j & 2) ? ((j & 1) ? w[3] : w[2]) : ((j & 1) ? w[1] : w[0]);
                 const unsigned short h = (unsigned short)((bit >> 4) ? (wj >> 16) : (wj & 0xFFFFu));
                 if (pos < (uint32_t)CTA_LIST) s_list[pos] = (unsigned short)key_of(h);
+                else if (g0 + pos < a.cap) dst[g0 + pos] = (unsigned short)key_of(h);
                 ++pos;
             }
         }
@@ -442,17 +451,14 @@ __global__ void __launch_bounds__(256) thr_scan_kernel(const ThrArgs a) {
     if (lane == 0 && nnan) atomicAdd(&s_nan, nnan);
     if (lane == 0 && nlow) atomicAdd(&s_low, nlow);
     __syncthreads();
-    const uint32_t cnt = s_n, low = s_low;
+    const uint32_t cnt = min(s_n, (uint32_t)CTA_LIST), low = s_low;
     if (threadIdx.x == 0) {
         s_base = cnt ? atomicAdd(&pr->n, cnt) : 0u;
         if (low) atomicAdd(&pr->cnt[0], low);
-        if (cnt > low) atomicAdd(&pr->cnt[1], cnt - low);
+        if (s_n > low) atomicAdd(&pr->cnt[1], s_n - low);
         if (s_nan) atomicAdd(&pr->nan, s_nan);
-        if (cnt > CTA_LIST) atomicOr(&pr->overflow, 1u);       // leaves a hole in the list: the select kernel falls back
     }
     __syncthreads();
-    if (cnt > CTA_LIST) return;
-    unsigned short* dst = a.list + (size_t)bhx * a.cap;
     for (uint32_t i = threadIdx.x; i < cnt; i += blockDim.x) {
         const uint32_t pos = s_base + i;
         if (pos < a.cap) dst[pos] = s_list[i];
@@ -474,7 +480,7 @@ __global__ void __launch_bounds__(THREADS) thr_select_kernel(const ThrArgs a) {
     if (N > 0) {
         const unsigned long long k = rank_k(a.alpha, N);
         const uint32_t c0 = pr->cnt[0], c1 = pr->cnt[1], c = c0 + c1;
-        if (c0 > k && c1 > k && c <= a.cap && !pr->overflow) {
+        if (c0 > k && c1 > k && c <= a.cap) {
             // rank k from below and rank k from above
             const unsigned short* l = a.list + (size_t)bhx * a.cap;                // 16-byte aligned
             const unsigned short* keys = l;
@@ -606,7 +612,9 @@ __global__ void __launch_bounds__(SMALL_THREADS) thr_small_kernel(const ThrArgs 
 }
 
 // Tokens per CTA of the scan: as many as keep the expected number of candidates (1.25 times the tail mass
-// plus the bracket's slack, of both tails) well inside the CTA's list; a CTA that overflows sends its problem to the exact fallback.
+// plus the bracket's slack, of both tails) inside the CTA's list.  Where tails are not spread evenly over the sequence a CTA
+// finds more; those go to the problem's list batch by batch (a tail in the first quarter of 256 (b,h) x 4096 tokens: 151 us,
+// 132 where it is spread evenly; as an overflow that sends the problem to the exact select over its data it took 4390).
 // Fewer too while the launch does not fill the chip: a thread's loads then come one round after the other for nothing
 // (32 (b,h) of 333 tokens: one CTA for each and tensor 8.5 us, six 4.9).
 int scan_tokens_for(double alpha, int D, int BH, int T) {

@@ -69,3 +69,15 @@ def test_tails_so_heavy_that_every_scan_block_overflows(alpha):
     wl = synth.scaled(synth.CONFIGS["C2"], heads=2, tokens=2048)
     K, V = synth.make_kv(wl, 0)
     check(K, V, wl, alpha)
+
+
+@pytest.mark.parametrize("alpha", [0.01, 0.05])
+@pytest.mark.parametrize("part,factor", [(4, 2.0), (4, 40.0), (16, 4.0), (64, 4.0)])
+def test_tails_that_lie_in_one_part_of_the_sequence(alpha, part, factor):
+    # the scan blocks of the first 1/part of the tokens find several times the candidates that their lists are laid out for:
+    # what these do not hold goes to the problem's list
+    wl = synth.scaled(synth.CONFIGS["C2"], heads=3, tokens=4096)
+    K, V = synth.make_kv(wl, 0)
+    K[:, :, :4096 // part] *= factor
+    V[:, 1:, -4096 // part:] *= factor
+    check(K, V, wl, alpha)
