@@ -81,3 +81,19 @@ def test_tails_that_lie_in_one_part_of_the_sequence(alpha, part, factor):
     K[:, :, :4096 // part] *= factor
     V[:, 1:, -4096 // part:] *= factor
     check(K, V, wl, alpha)
+
+
+@pytest.mark.parametrize("D,T,alpha", [(128, 4096, 0.01), (64, 2049, 0.3), (32, 700, 1.0), (128, 4097, 0.2)])
+def test_the_exact_select_over_the_data_passes_over_nans(D, T, alpha):
+    # sampled tokens all zero: lists overflow; NaNs of both signs, infinities, a problem of NaNs alone in its unsampled tokens
+    wl = synth.scaled(synth.CONFIGS["C2"], heads=3, head_dim=D, tokens=T)
+    K, V = synth.make_kv(wl, 0)
+    g = torch.Generator().manual_seed(D)
+    for X in (K, V):
+        m = torch.rand(X.shape, generator=g)
+        X[m < 0.02] = float("nan"); X[(m > 0.02) & (m < 0.04)] = -float("nan")
+        X[(m > 0.04) & (m < 0.041)] = float("inf"); X[(m > 0.041) & (m < 0.042)] = -float("inf")
+    K[:, 2] = float("nan")
+    K[:, :, sampled_tokens(T)] = 0
+    V[:, :, sampled_tokens(T)] = 0
+    check(K, V, wl, alpha)
