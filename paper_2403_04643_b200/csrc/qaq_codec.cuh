@@ -299,15 +299,17 @@ __device__ __forceinline__ RowPlace place_row(const TileRows& r, int row, int w)
     }
     return o;
 }
-// The largest of the first nv of W scores, `stride` apart.  Every row of the window is read (the ring is allocated in full),
-// rows the token has no score in are left out of the maximum: the loads then depend on nothing and go out together.
-// By whole warps.
-template <int BATCH = 16>
+// The largest of the first nv (at most W) of W scores, `stride` apart.  Rows a token has no score in are left out of the maximum,
+// not of the loads (the ring is allocated in full): those of a batch depend on nothing and go out together.  What is left after
+// whole batches is read eight at a time, the last row again where there are fewer.  (One at a time, 128 tokens with 255 rows
+// behind 32 (b,h) x 4096 took 29.2 us, so 17.4; 4096 tokens of 256 (b,h) with 16 rows 244 and 189.)  SEEN: rows from the 33rd on are read only as far as some token of the warp has a
+// score in them (re-selection of 32 (b,h) x 4096 with one score each in 255 rows: every row read 24.6 us, so 4.5; a vote in front
+// of every batch, 128 x 2048 with 32 rows take 7.4 instead of 6.6 us).  By whole warps.
+template <int BATCH, bool SEEN = false>
 __device__ __forceinline__ float window_max(const float* r, int W, long stride, int nv) {
     float m = __int_as_float(0xff800000);
     int i = 0;
-#pragma unroll 1
-    for (; i + BATCH <= W; i += BATCH, r += BATCH * stride) {
+    auto batch = [&]() {
         float v[BATCH];
 #pragma unroll
         for (int u = 0; u < BATCH; ++u) v[u] = r[u * stride];
@@ -318,11 +320,43 @@ __device__ __forceinline__ float window_max(const float* r, int W, long stride, 
 #pragma unroll
             for (int u = 0; u < BATCH; ++u) if (i + u < nv) m = fmaxf(m, v[u]);
         }
+        i += BATCH;
+        r += BATCH * stride;
+    };
+    const int first = SEEN ? min(W, 32) : W;
+#pragma unroll 1
+    while (i + BATCH <= first) batch();
+    if (SEEN && W > 32) {
+        W = max(32, __reduce_max_sync(0xFFFFFFFFu, nv));
+#pragma unroll 1
+        while (i + BATCH <= W) batch();
     }
 #pragma unroll 1
-    for (; i < W; ++i, r += stride) {
-        const float v = *r;
-        if (i < nv) m = fmaxf(m, v);
+    for (; i < W; i += 8, r += 8 * stride) {
+        float v[8];
+#pragma unroll
+        for (int u = 0; u < 8; ++u) v[u] = r[min(u, W - 1 - i) * stride];
+#pragma unroll
+        for (int u = 0; u < 8; ++u) if (i + u < nv) m = fmaxf(m, v[u]);
+    }
+    return m;
+}
+// The same by one loop, whose last batch reads the last row again where it is short of rows: less code to fetch, which a one-token
+// append waits for (with the loops above it takes 1 us more); whole tiles have the address arithmetic to pay (256 (b,h) x 4096: 3 us).
+template <int BATCH>
+__device__ __forceinline__ float window_max_one_loop(const float* r, int W, long stride, int nv) {
+    float m = __int_as_float(0xff800000);
+#pragma unroll 1
+    for (int i = 0; i < W; i += BATCH) {
+        const int rows = W - i;
+        float v[BATCH];
+#pragma unroll
+        for (int u = 0; u < BATCH; ++u) {
+            v[u] = *r;
+            if (u + 1 < rows) r += stride;
+        }
+#pragma unroll
+        for (int u = 0; u < BATCH; ++u) if (i + u < nv) m = fmaxf(m, v[u]);
     }
     return m;
 }

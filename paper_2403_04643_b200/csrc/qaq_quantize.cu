@@ -218,7 +218,8 @@ __device__ __forceinline__ void quantize_tile(const QuantArgs& a, TileScratch<D>
     float shat = __int_as_float(0xff800000);
     if (IS_V && !given && main) {
         nv = min(nv, a.W);
-        shat = qaqc::window_max<32>(a.ring + (size_t)bh * a.W * a.n_new + col, a.W, a.n_new, nv);
+        const float* scores = a.ring + (size_t)bh * a.W * a.n_new + col;
+        shat = OPEN ? qaqc::window_max_one_loop<32>(scores, a.W, a.n_new, nv) : qaqc::window_max<32>(scores, a.W, a.n_new, nv);
     }
     if (OPEN) {                        // the tile as it is stored follows on its own: it is needed later
         asm volatile("cp.async.commit_group;" ::: "memory");

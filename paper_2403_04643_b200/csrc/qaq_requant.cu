@@ -128,7 +128,7 @@ __device__ __forceinline__ void requantize_tile(const RequantArgs& a, RequantScr
         } else {
             const long col = (long)min(tok, a.T - 1);           // whole warps read the window; columns beyond the last are not used
             const int nv = min((int)a.nvalid[(size_t)bh * a.ncols + col], a.W);
-            const float sh = qaqc::window_max(a.ring + (size_t)bh * a.W * a.ncols + col, a.W, a.ncols, nv);
+            const float sh = qaqc::window_max<16, true>(a.ring + (size_t)bh * a.W * a.ncols + col, a.W, a.ncols, nv);
             B = nv == 0 ? a.bmax : ladder(__fmul_rn(rng, sh), a.cV, a.bmin, a.bmax);
         }
         if (valid) Bn = (UP || B < Bo) ? B : Bo;

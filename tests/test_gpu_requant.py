@@ -288,3 +288,24 @@ def test_appends_and_decode_after_a_pool_ran_full():
     qaq.qaq_cache_compact(cache)
     out2 = qaq.qaq_decode_attention(cache, qd, 1.0 / math.sqrt(wl.head_dim))
     assert np.array_equal(out2.cpu().numpy().view(np.uint32), out.cpu().numpy().view(np.uint32))
+
+
+@pytest.mark.parametrize("window", [1, 15, 16, 17, 32, 33, 48, 71, 255])
+def test_windows_of_any_number_of_rows_partly_seen(window):
+    # re-selection reads whole batches of rows, and beyond the 32nd only as many as some token has scores in: none, one, some, all
+    wl = synth.scaled(synth.CONFIGS["C2"], heads=4, tokens=200, window=window)
+    K, V, q, ring, nv = make_inputs(wl)
+    T = 200
+    top = torch.tensor([0, 1, (window + 1) // 2, window]).view(1, 4, 1)
+    nv = torch.minimum(torch.randint(0, window + 1, nv.shape, generator=torch.Generator().manual_seed(window)), top).to(torch.uint8)
+    nv[:, 2, 0], nv[:, 3, 130] = (window + 1) // 2, window
+    ring[:, :, -1, ::3] = 0.5                             # the last row holds the largest score of many tokens
+    wide = torch.full((wl.bh, T), 8, dtype=torch.uint8)
+    pol = qaq.qaq_policy_from_hyper(*LOOSER, T)
+    cfg, cache, thr, out, scores, dev = gpu_pipeline(wl, K, V, q, ring, nv, pol, bits=(wide, wide))
+    ref = oracle_batch(wl, K, V, q, ring, nv, pol.cK, pol.cV, bitsK=wide.numpy(), bitsV=wide.numpy())
+    qaq.qaq_requantize_down(cache, policy=pol, ring=dev[3], nvalid=dev[4])
+    r, n = ring.numpy().reshape(wl.bh, window, T), nv.numpy().reshape(wl.bh, T)
+    qk = [oracle.requantize_down(ref.K[bh], oracle.reselect_bits(ref.K[bh], False, None, None, pol.cK, wl.bits_min, wl.bits_max)) for bh in range(wl.bh)]
+    qv = [oracle.requantize_down(ref.V[bh], oracle.reselect_bits(ref.V[bh], True, r[bh], n[bh], pol.cV, wl.bits_min, wl.bits_max)) for bh in range(wl.bh)]
+    compare_export(cache, SimpleNamespace(K=qk, V=qv))

@@ -88,7 +88,7 @@ def test_whole_tiles_equal_tiles_filled_in_pieces(D, bounds):
     _same_cache(whole, pieces)
 
 
-@pytest.mark.parametrize("window", [1, 15, 16, 33])
+@pytest.mark.parametrize("window", [1, 15, 16, 33, 64, 71, 255])
 def test_windows_of_any_number_of_rows_choose_the_oracles_widths(window):
     wl = synth.scaled(synth.CONFIGS["C2"], heads=2, tokens=192, window=window)
     K, V, q, ring, nv = make_inputs(wl, ragged=True)
