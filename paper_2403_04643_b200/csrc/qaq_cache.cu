@@ -294,32 +294,9 @@ __global__ void export_scan_kernel(uint32_t* a, int T) {
     }
 }
 
-// the code of channel d of the token in `slot`, from the tile as it is stored (w: width of the token's row)
-__device__ uint32_t code_at(const uint8_t* tile, const qaqc::Section& s, int is_v, int D, int slot, int w, int d) {
-    const int p = d >> 5, u = (d >> 3) & 3, cls = (d >> 2) & 1, b = d & 3;
-    uint32_t code = 0;
-    for (int part = 0; part < 2; ++part) {
-        const int pw = part ? w - 4 : (w < 4 ? w : 4);
-        if (pw < 1) continue;
-        const uint8_t* src = tile + (part ? s.high : s.main);
-        const int first = part ? s.start : s.mstart, n = part ? s.n : s.mn;
-        // byte c of the words the channel is in
-        const uint8_t* x = is_v ? src + qaqc::v_unit(D, n, (slot >> 2) - first, 4 * p + b) * 4 * pw + (slot & 3)
-                                : src + (uint32_t)((slot - first) * (D / 32) + p) * 4 * pw + b;
-        uint32_t v = 0;
-        if (pw == 4) v = (x[4 * u] >> (4 * cls)) & 15u;
-        else if (pw == 3) {
-            if (u < 3) v = (x[4 * u] >> (4 * cls)) & 7u;
-            else for (int i = 0; i < 3; ++i) v |= (((uint32_t)x[4 * i] >> (4 * cls + 3)) & 1u) << i;
-        } else if (pw == 2) v = (x[4 * (u >> 1)] >> (4 * cls + 2 * (u & 1))) & 3u;
-        else v = (x[0] >> (4 * cls + u)) & 1u;
-        code |= v << (4 * part);
-    }
-    return code;
-}
 // one canonical byte of a token: byte y of its string (the planes of its pieces, widest first; inside the plane of
-// a piece of `w` bits channel d = 32p + 4j + i sits in word p*w + j*w/8 at bit 8i + w*(j mod 8/w))
-__device__ uint32_t canonical_byte(const uint8_t* tile, const qaqc::Section& s, int is_v, int D, int slot, int row_w, int B, uint32_t y) {
+// a piece of `w` bits channel d = 32p + 4j + i sits in word p*w + j*w/8 at bit 8i + w*(j mod 8/w)); code: by channel
+__device__ __forceinline__ uint32_t canonical_byte(const uint8_t* code, int D, int B, uint32_t y) {
     for (int c = 0; c < 4; ++c) {
         const int w = 8 >> c;
         if (!(B & w)) continue;
@@ -327,42 +304,38 @@ __device__ uint32_t canonical_byte(const uint8_t* tile, const qaqc::Section& s, 
         if (y >= plen) { y -= plen; continue; }
         const int per = 8 / w, cw = y >> 2, i = y & 3, p = cw / w, rr = cw % w;
         uint32_t v = 0;
-        for (int mm = 0; mm < per; ++mm)
-            v |= ((code_at(tile, s, is_v, D, slot, row_w, 32 * p + 4 * (rr * per + mm) + i) >> (B & (w - 1))) & ((1u << w) - 1u)) << (w * mm);
+        for (int mm = 0; mm < per; ++mm) v |= ((code[32 * p + 4 * (rr * per + mm) + i] >> (B & (w - 1))) & ((1u << w) - 1u)) << (w * mm);
         return v;
     }
     return 0;
 }
 
-__global__ void export_gather_kernel(TensorStore ts, int is_v, int T, int tmax_pad, int ntiles, int D, size_t pool_bytes, uint32_t ocap,
-                                     uint8_t* bits, float* mn, float* step, const uint32_t* off, uint8_t* codes,
-                                     long codes_stride, const uint32_t* rowptr, uint8_t* ch, __half* val, long outl_stride) {
-    const int bh = blockIdx.y, tile = blockIdx.x;
+// One CTA = one tile: its bytes come to shared memory, its codes by token and channel, the canonical bytes from these.  (Bit by
+// bit from the tile as it lies in the pool 128 (b,h) x 2048 tokens took 650 us, this way 407.)
+template <int D, bool IS_V>
+__global__ void __launch_bounds__(256) export_gather_kernel(TensorStore ts, int T, int tmax_pad, int ntiles, size_t pool_bytes, uint32_t ocap,
+                                                            uint8_t* bits, float* mn, float* step, const uint32_t* off, uint8_t* codes,
+                                                            long codes_stride, const uint32_t* rowptr, uint8_t* ch, __half* val, long outl_stride) {
+    constexpr int P = D / 32;
+    constexpr uint32_t BYTES = qaqc::tile_bytes_max(D) + 16;
+    const int bh = blockIdx.y, tile = blockIdx.x, tid = threadIdx.x;
+    __shared__ alignas(16) uint8_t s_tile[BYTES];
+    __shared__ alignas(16) uint32_t s_code[QAQ_TILE][D / 4];
     __shared__ uint32_t s_in[QAQ_TILE + 1];
-    __shared__ uint8_t s_b[QAQ_TILE], s_slot[QAQ_TILE], s_row[QAQ_TILE];
-    __shared__ qaqc::Section s_tab[9];
+    __shared__ uint8_t s_b[QAQ_TILE], s_slot[QAQ_TILE];
     const int t0 = tile * QAQ_TILE;
-    if (threadIdx.x < QAQ_TILE) {
-        const int t = t0 + threadIdx.x;
+    const uint4 tw = ts.tile[(size_t)bh * ntiles + tile];
+    if (tid < QAQ_TILE) {
+        const int t = t0 + tid;
         const unsigned bs = t < T ? ts.bs[(size_t)bh * tmax_pad + t] : 0u;
-        s_b[threadIdx.x] = (uint8_t)min(bs & 0xFFu, 8u);
-        s_slot[threadIdx.x] = (uint8_t)((bs >> 8) & (QAQ_TILE - 1));
+        s_b[tid] = (uint8_t)min(bs & 0xFFu, 8u);
+        s_slot[tid] = (uint8_t)((bs >> 8) & (QAQ_TILE - 1));
     }
-    const uint8_t* src = ts.codes + (size_t)bh * pool_bytes + ts.tile[(size_t)bh * ntiles + tile].x;
-    if (threadIdx.x == 0) {
-        int n[9];
-        const uint32_t* h = reinterpret_cast<const uint32_t*>(src);
-        const bool there = ts.tile[(size_t)bh * ntiles + tile].y != 0;
-        qaqc::counts_of(there ? h[0] : 0u, there ? h[1] : 0u, n);
-        const int units = is_v ? D / 8 : D / 32;
-        if (units == 1) qaqc::make_sections<1>(n, s_tab, nullptr);
-        else if (units == 2) qaqc::make_sections<2>(n, s_tab, nullptr);
-        else if (units == 4) qaqc::make_sections<4>(n, s_tab, nullptr);
-        else if (units == 8) qaqc::make_sections<8>(n, s_tab, nullptr);
-        else qaqc::make_sections<16>(n, s_tab, nullptr);
-    }
+    const uint8_t* src = ts.codes + (size_t)bh * pool_bytes + tw.x;
+    for (uint32_t o = tid * 16; o < min(tw.y, (uint32_t)qaqc::tile_bytes_max(D)); o += 256 * 16)
+        *reinterpret_cast<uint4*>(s_tile + o) = *reinterpret_cast<const uint4*>(src + o);
     __syncthreads();
-    if (threadIdx.x == 0) {
+    if (tid == 0) {
         uint32_t acc = 0;
         for (int k = 0; k < QAQ_TILE; ++k) {
             s_in[k] = acc;
@@ -370,18 +343,27 @@ __global__ void export_gather_kernel(TensorStore ts, int is_v, int T, int tmax_p
         }
         s_in[QAQ_TILE] = acc;
     }
-    if (threadIdx.x < QAQ_TILE) {      // width of the row a token is in
-        int w = s_b[threadIdx.x];
-        if (is_v && w) {
-            const int row = s_slot[threadIdx.x] >> 2;
-            for (int k = 8; k >= 1; --k) if (row >= s_tab[k].start && row < s_tab[k].start + s_tab[k].n) w = k;
+    uint4 h = *reinterpret_cast<const uint4*>(s_tile);
+    if (!tw.y) h = make_uint4(0u, 0u, 0u, 0u);
+    const qaqc::TileRows rows = qaqc::rows_of_header(h.x, h.y);
+    for (int i = tid; i < QAQ_TILE * P; i += 256) {
+        const int k = i / P, p = i % P, b = s_b[k], slot = s_slot[k];
+        uint32_t lo[4] = {0, 0, 0, 0}, hi[4] = {0, 0, 0, 0};
+        if (b) {
+            const int row = IS_V ? slot >> 2 : slot, w = IS_V ? max(1, min(8, qaqc::width_of_row(rows, row))) : b;
+            const qaqc::RowPlace at = qaqc::place_row<D, IS_V>(rows, row, w);
+            qaqc::take_token<D, IS_V>(s_tile, BYTES, at.main, at.high, w, at.mm, at.mh, slot & 3, p, lo, hi);
         }
-        s_row[threadIdx.x] = (uint8_t)w;
+#pragma unroll
+        for (int u = 0; u < 4; ++u) {                // channels 32p + 8u .. + 3, then the next four
+            s_code[k][8 * p + 2 * u] = qaqc::bitsel(lo[u], hi[u] << 4, qaqc::NIB);
+            s_code[k][8 * p + 2 * u + 1] = qaqc::bitsel(lo[u] >> 4, hi[u], qaqc::NIB);
+        }
     }
     __syncthreads();
-    if (threadIdx.x < QAQ_TILE && t0 + (int)threadIdx.x < T) {
-        const int t = t0 + threadIdx.x;
-        const int B = s_b[threadIdx.x];
+    if (tid < QAQ_TILE && t0 + tid < T) {
+        const int t = t0 + tid;
+        const int B = s_b[tid];
         const uint32_t mm = ts.mnmx[(size_t)bh * tmax_pad + t];
         const float fmn = __half2float(__ushort_as_half((unsigned short)(mm & 0xFFFF)));
         const float fmx = __half2float(__ushort_as_half((unsigned short)(mm >> 16)));
@@ -392,17 +374,16 @@ __global__ void export_gather_kernel(TensorStore ts, int is_v, int T, int tmax_p
     if (codes && off) {
         uint8_t* dst = codes + (size_t)bh * codes_stride + off[(size_t)bh * (T + 1) + t0];
         for (int k0 = 0; k0 < QAQ_TILE; k0 += 4) {
-            const int k = k0 + (threadIdx.x >> 6);
+            const int k = k0 + (tid >> 6);
             const uint32_t len = s_in[k + 1] - s_in[k];
-            for (uint32_t y = threadIdx.x & 63; y < len; y += 64)
-                dst[s_in[k] + y] = (uint8_t)canonical_byte(src, s_tab[s_row[k]], is_v, D, s_slot[k], s_row[k], s_b[k], y);
+            for (uint32_t y = tid & 63; y < len; y += 64)
+                dst[s_in[k] + y] = (uint8_t)canonical_byte(reinterpret_cast<const uint8_t*>(s_code[k]), D, s_b[k], y);
         }
     }
     if (rowptr && (ch || val)) {
-        const uint32_t n = ts.tile[(size_t)bh * ntiles + tile].w;
-        const uint32_t* e = ts.outl + (size_t)bh * ocap + ts.tile[(size_t)bh * ntiles + tile].z;
+        const uint32_t* e = ts.outl + (size_t)bh * ocap + tw.z;
         const uint32_t dst0 = rowptr[(size_t)bh * (T + 1) + t0];
-        for (uint32_t i = threadIdx.x; i < n; i += blockDim.x) {
+        for (uint32_t i = tid; i < tw.w; i += blockDim.x) {
             uint32_t v = e[i];
             if ((long)(dst0 + i) < outl_stride) {
                 if (ch) ch[(size_t)bh * outl_stride + dst0 + i] = (uint8_t)((v >> 16) & 0xFF);
@@ -434,8 +415,16 @@ extern "C" qaq_status qaq_cache_export(const qaq_cache* c, int tensor, uint8_t* 
         export_ocount_kernel<<<grid, 128, 0, s>>>(ts, T, c->ntiles, c->ocap, rowptr);
         export_scan_kernel<<<c->BH, 256, 0, s>>>(rowptr, T);
     }
-    export_gather_kernel<<<grid, 256, 0, s>>>(ts, tensor, T, c->tmax_pad, c->ntiles, c->cfg.head_dim, c->pool_bytes, c->ocap, bits, mn,
-                                              step, off, codes, codes_stride, rowptr, ch, (__half*)val, outl_stride);
+    auto gather = [&](auto kernel) {
+        kernel<<<grid, 256, 0, s>>>(ts, T, c->tmax_pad, c->ntiles, c->pool_bytes, c->ocap, bits, mn, step, off, codes, codes_stride, rowptr, ch, (__half*)val,
+                                    outl_stride);
+    };
+    switch (c->cfg.head_dim) {
+        case 32: tensor ? gather(export_gather_kernel<32, true>) : gather(export_gather_kernel<32, false>); break;
+        case 64: tensor ? gather(export_gather_kernel<64, true>) : gather(export_gather_kernel<64, false>); break;
+        case 128: tensor ? gather(export_gather_kernel<128, true>) : gather(export_gather_kernel<128, false>); break;
+        default: return QAQ_ERR_UNSUPPORTED_SHAPE;
+    }
     QAQ_CUDA_TRY(cudaGetLastError());
     return QAQ_OK;
 }

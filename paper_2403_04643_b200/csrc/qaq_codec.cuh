@@ -129,49 +129,6 @@ __host__ __device__ constexpr int tile_bytes_max(int D) { return QAQ_TILE_HDR + 
 // units per row: keys head_dim/32, values four times that
 template <int D, bool IS_V> constexpr int UNITS = IS_V ? D / 8 : D / 32;
 
-// Where the section of one width lies (byte offsets inside the tile) and which rows of the tile it holds.
-struct alignas(8) Section {
-    uint16_t main, high;     // first byte of the main and of the high part
-    uint8_t start, n;        // first row (in sorted order) and number of rows
-    uint8_t mstart, mn;      // the same for the list of rows the main part is in: all rows of 4 bits and more share one
-};
-
-// Sections of a tile with n[w] rows of width w (U units each): tab[1..8] and, if head is given, the header's four words.
-// Returns the bytes of the tile.
-template <int U>
-__device__ __forceinline__ uint32_t make_sections(const int (&n)[9], Section* tab, uint32_t* head) {
-    const int s7 = n[8], s6 = s7 + n[7], s5 = s6 + n[6], s4 = s5 + n[5], s3 = s4 + n[4], s2 = s3 + n[3], s1 = s2 + n[2];
-    const int h8 = QAQ_TILE_HDR + s3 * U * 16, z2 = h8 + n[8] * U * 16, m2 = z2 + n[6] * U * 8, z13 = m2 + n[2] * U * 8;
-    const int m3 = z13 + n[7] * U * 12, h5 = m3 + n[3] * U * 12, m1 = h5 + n[5] * U * 4, total = m1 + n[1] * U * 4;
-    auto put = [&](int w, int main, int high, int start) {
-        Section s;
-        s.main = (uint16_t)main; s.high = (uint16_t)high; s.start = (uint8_t)start; s.n = (uint8_t)n[w];
-        s.mstart = (uint8_t)(w >= 4 ? 0 : start); s.mn = (uint8_t)(w >= 4 ? s3 : n[w]);
-        tab[w] = s;
-    };
-    put(8, QAQ_TILE_HDR, h8, 0);
-    put(7, QAQ_TILE_HDR, z13, s7);
-    put(6, QAQ_TILE_HDR, z2, s6);
-    put(5, QAQ_TILE_HDR, h5, s5);
-    put(4, QAQ_TILE_HDR, 0, s4);
-    put(3, m3, 0, s3);
-    put(2, m2, 0, s2);
-    put(1, m1, 0, s1);
-    if (head) {
-        head[0] = (uint32_t)(n[1] | (n[2] << 8) | (n[3] << 16) | (n[4] << 24));
-        head[1] = (uint32_t)(n[5] | (n[6] << 8) | (n[7] << 16) | (n[8] << 24));
-        head[2] = (uint32_t)(h8 | (z2 << 16));
-        head[3] = (uint32_t)(z13 | (total << 16));
-    }
-    return (uint32_t)total;
-}
-// the counts of a stored header
-__device__ __forceinline__ void counts_of(uint32_t lo, uint32_t hi, int (&n)[9]) {
-    n[0] = 0;
-#pragma unroll
-    for (int w = 1; w <= 4; ++w) { n[w] = (lo >> (8 * w - 8)) & 0xFF; n[w + 4] = (hi >> (8 * w - 8)) & 0xFF; }
-}
-
 constexpr uint32_t NIB = 0x0F0F0F0Fu;
 // (a & m) | (b & ~m)
 __device__ __forceinline__ uint32_t bitsel(uint32_t a, uint32_t b, uint32_t m) { return (a & m) | (b & ~m); }
@@ -214,12 +171,6 @@ __device__ __forceinline__ void nibble_words(const uint32_t* x, uint32_t (&v)[4]
         v[0] = x[0]; v[1] = x[0] >> 1; v[2] = x[0] >> 2; v[3] = x[0] >> 3;
     }
 }
-// index of unit e of row r (counted from the section's first row) of a section of n rows of values
-__device__ __forceinline__ uint32_t v_unit(int D, int n, int r, int e) {
-    const int k4 = r & ~3, m = n - k4 < 4 ? n - k4 : 4;
-    return (uint32_t)(k4 * (D / 8) + e * m + (r & 3));
-}
-
 // ------------------------------------------------------------------------------------------ a tile by two warps
 // What the kernels that give a tile 64 threads, one per token, find out about it.  Counts by width are kept a byte each, widths
 // 1..4 in one word and 5..8 in the other, and sums over widths are taken in the bytes (they stay below 256).
@@ -262,7 +213,7 @@ __device__ __forceinline__ int width_of_row(const TileRows& r, int row) {
     const uint32_t y = (uint32_t)row * ONES | 0x80808080u;
     return 9 - __popc((y - r.slo) & 0x80808080u) - __popc((y - r.shi) & 0x80808080u);
 }
-// Offsets of the parts as in make_sections, in words per unit: dot products of the rows of every width.
+// Offsets of the parts (in the order of the storage, above), in words per unit: dot products of the rows of every width.
 template <int D, bool IS_V>
 __device__ __forceinline__ uint32_t at_words(const TileRows& r, uint32_t wlo, uint32_t whi) {
     return (uint32_t)QAQ_TILE_HDR + (uint32_t)(4 * UNITS<D, IS_V>) * __dp4a(r.nlo, wlo, __dp4a(r.nhi, whi, 0u));
