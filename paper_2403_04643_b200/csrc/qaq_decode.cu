@@ -1082,24 +1082,28 @@ __global__ void __launch_bounds__(Shape<NQ>::THREADS, Shape<NQ>::CTAS_PER_SM) de
                         ws.macc[j][d] += (float)ws.vcorr[j][d] * unit[j];
                     }
             } else {
+                constexpr int TOGETHER = NQ == 4 ? 2 : 1;             // queries whose two words have room
 #pragma unroll 1
-                for (int j = 0; j < NQ; ++j) {
+                for (int j = 0; j < NQ; j += TOGETHER) {
                     __syncwarp();
-                    clear_vcorr(2);
+                    clear_vcorr(2 * TOGETHER);
                     __syncwarp();
                     auto add = [&](uint32_t v) {
                         const int ch = (v >> 16) & (D - 1);
-                        wide_add(&ws.vcorr[0][ch], &ws.vcorr[1][ch], term(v, j));
+#pragma unroll
+                        for (int i = 0; i < TOGETHER; ++i) wide_add(&ws.vcorr[2 * i][ch], &ws.vcorr[2 * i + 1][ch], term(v, j + i));
                     };
 #pragma unroll 1
                     for (uint32_t i = lane; i < sc; i += 32) add(list[i]);
                     if (sc < oc) unstaged(all, sc, oc, add);
                     __syncwarp();
 #pragma unroll
-                    for (int k = 0; k < CPL; ++k) {
-                        const int d = lane + 32 * k;
-                        ws.macc[j][d] += wide_sum(ws.vcorr[0][d], ws.vcorr[1][d]);
-                    }
+                    for (int i = 0; i < TOGETHER; ++i)
+#pragma unroll
+                        for (int k = 0; k < CPL; ++k) {
+                            const int d = lane + 32 * k;
+                            ws.macc[j + i][d] += wide_sum(ws.vcorr[2 * i][d], ws.vcorr[2 * i + 1][d]);
+                        }
                 }
             }
         }
@@ -1294,6 +1298,14 @@ static bool side_by_side(int BH, int ntiles, int n) {
     return 2 * tiles(both.run, Shape<4>::WARPS) <= 2 * w4 + (n > 6 ? 2 * w4 : tiles(few.run, Shape<1>::WARPS)) + 2;
 }
 
+// Where many entries are outliers, their sums are most of the time, and four queries take longer for them than twice two: three,
+// five and six queries are taken two at a time from 10 % on, four from 20 % (32 (b,h) of 4096 tokens, 8 bits, 10 %: three 70 us
+// at once and 59 as two and one, five 118 and 94, four 70 and 71, eight 120 and 142; 4 bits, 50 %: three 381 and 279, four 381
+// and 361).
+static bool in_twos(double outlier_frac, int left) {
+    return left <= 6 && outlier_frac >= (left == 4 ? 0.2 : 0.1);
+}
+
 extern "C" qaq_status qaq_decode_multi_workspace_bytes(const qaq_cache* c, size_t* host_out) {
     if (!c || !host_out) return QAQ_ERR_INVALID_ARG;
     const int D = c->cfg.head_dim, BH = c->BH;       // the passes of a call reuse the space
@@ -1317,7 +1329,7 @@ extern "C" qaq_status qaq_decode_attention_multi(const qaq_cache* c, const void*
         const int left = n_q - q0;
         const __half* qp = (const __half*)q + (size_t)q0 * D;
         float* op = out + (size_t)q0 * D;
-        const int n = left > 4 && !side_by_side(c->BH, ntiles, left) ? 4 : left;
+        const int n = in_twos(c->cfg.outlier_frac, left) ? (left < 2 ? left : 2) : left > 4 && !side_by_side(c->BH, ntiles, left) ? 4 : left;
         const qaq_status st = n >= 3 ? decode<4, false>(c, qp, row, softmax_scale, op, row, nullptr, 0, ws, s, n)
                               : n == 2 ? decode<2, false>(c, qp, row, softmax_scale, op, row, nullptr, 0, ws, s)
                                        : decode<1, false>(c, qp, row, softmax_scale, op, row, nullptr, 0, ws, s);

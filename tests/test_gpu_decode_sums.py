@@ -106,3 +106,23 @@ def test_a_token_whose_logit_is_not_a_number_takes_no_part(n_q):
         outs.append(qaq.qaq_decode_attention_multi(cache, q, 1 / math.sqrt(D)))
     # the same tokens in other tiles: binary32 sums of 210 weights in another order, weights of 21 bits or more
     assert (outs[0] - outs[1]).abs().max().item() <= 210 * 2.0 ** -22 * V.abs().max().item()
+
+
+@pytest.mark.parametrize("n_q", [3, 4, 5, 6, 7])
+@pytest.mark.parametrize("D,alpha,scale", [(128, 0.1, 1.0), (128, 0.3, 1.0), (64, 0.5, 300.0)])
+def test_several_queries_where_many_entries_are_outliers(n_q, D, alpha, scale):
+    # two at a time or four, value outliers that are not staged (or too large for one word) in two words for two queries at once
+    wl = synth.scaled(synth.CONFIGS["C2"], heads=3, head_dim=D, tokens=300, alpha=alpha)
+    K, V, q, ring, nv = make_inputs(wl)
+    K, V = (K * scale).half(), (V * scale).half()
+    pol = qaq.qaq_policy_from_hyper(*HYPER, 300)
+    bits = torch.full((wl.bh, 300), 8, dtype=torch.uint8)
+    cfg, cache, thr, out, scores, dev = gpu_pipeline(wl, K, V, q, ring, nv, pol, bits=(bits, bits), max_outliers=300 * D)
+    qs = torch.stack([synth.make_query(wl, step=i).view(wl.bh, D) for i in range(n_q)], dim=1).cuda() / scale
+    got = qaq.qaq_decode_attention_multi(cache, qs.half().contiguous(), 1 / math.sqrt(D))
+    for j in range(n_q):
+        one = qaq.qaq_decode_attention(cache, qs[:, j].half().contiguous(), 1 / math.sqrt(D))
+        # One word: units of 2^-24 of at most four times the largest term, D terms to a logit.  Two words: the same words for all
+        # queries.  Beyond that binary32 sums of up to 128 terms in another order.
+        terms = D * 2.0 ** -22 * (qs.abs().max() * K.abs().max()).item() / math.sqrt(D)
+        assert (got[:, j] - one).abs().max().item() <= (2 * terms + 128 * 2.0 ** -23) * V.abs().max().item()
