@@ -244,9 +244,10 @@ qaq_status qaq_decode_attention_host(qaq_cache* c, const void* q, float softmax_
 /*
  * Decode attention for several queries per (b,h) in one call (Section 4.2, "Integration in text generation
  * process"; the packed cache is what every query reads).  Per query the result is what qaq_decode_attention
- * returns for it, within the same tolerance.  Up to four queries share what is taken apart of a tile (the queries are
- * columns of the tensor-core operand); five to eight are two groups, beside each other in one launch while that fills
- * the chip no worse, else one after the other.
+ * returns for it, within the same tolerance, whatever the other queries are.  Up to four queries share what is taken apart of
+ * a tile (the queries are columns of the tensor-core operand); five to eight are two groups, beside each other in one launch
+ * while that fills the chip no worse, else one after the other; where outlier_frac is 10 % or more, up to six are taken two at
+ * a time.
  * q: binary16 [batch*heads][n_q][head_dim]; out: binary32 [batch*heads][n_q][head_dim]; 1 <= n_q <= 8;
  * ws: qaq_decode_multi_workspace_bytes bytes, 16-byte aligned.  Device pointers, asynchronous on stream.
  * Errors: QAQ_ERR_INVALID_ARG (null pointer, empty cache, n_q outside 1..8), QAQ_ERR_WORKSPACE.
@@ -309,7 +310,8 @@ qaq_status qaq_stream_end(qaq_cache* c, void* stream);
  *   - All calls on a device share the one array.  Calls that may overlap on the GPU
  *     (different streams, no ordering between them) race on it and give wrong results;
  *     keep them on one stream or order them yourself.  The array keeps the previous
- *     call's contents; nothing in it needs clearing, every value is written before use.
+ *     call's contents; nothing in it needs clearing: partials are written before they are
+ *     read, and the words that count them carry the number of the call they belong to.
  *   - No scores_out here; results equal qaq_decode_attention's.
  */
 qaq_status qaq_decode_attention_static(const qaq_cache* c, const void* q, float softmax_scale, float* out,
@@ -339,7 +341,9 @@ qaq_status qaq_cache_export(const qaq_cache* c, int tensor, uint8_t* bits, float
  * Housekeeping for caches whose widths are raised (no counterpart in the paper, which keeps its
  * cache in framework tensors).  qaq_requantize places a tile that grows at the end of its (b,h)
  * pool and leaves the old bytes unused; qaq_cache_compact moves the tiles of every pool down
- * until they are contiguous again (order in memory kept, open tile last), so that the space can
+ * until they are contiguous again (order in memory kept: the open tile is the last one, unless it
+ * found no room in a full pool behind tiles that had grown; the next call of qaq_requantize_down or
+ * qaq_requantize moves it there, and until then it cannot be appended to), so that the space can
  * be appended to.  Contents, widths and outlier lists are unchanged; only tile offsets move.
  * At most 4096 tiles (262144 tokens) per (b,h), else QAQ_ERR_UNSUPPORTED_SHAPE.  Asynchronous
  * on stream.  qaq_cache_pool_use reports the largest pool fill over all (b,h), in bytes, for

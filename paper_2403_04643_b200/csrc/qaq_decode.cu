@@ -1353,7 +1353,7 @@ static std::mutex g_scratch_mutex;
 static void* g_scratch_addr[64];  // device address of g_decode_scratch, per device ordinal
 
 // the documented limit: what two partials per CTA of a split into at most 592 (or one per (b,h)) and a pair of words
-// per (b,h) would take
+// per (b,h) would take; decode_ws_bytes<1> never needs more than 4 MiB within it
 static bool static_scratch_fits(int BH, long tokens, int D) {
     const long ntiles = (tokens + QAQ_TILE - 1) / QAQ_TILE;
     const long long total = (long long)BH * ntiles, floor_run = ntiles < 4 ? ntiles : 4;
@@ -1369,7 +1369,6 @@ extern "C" qaq_status qaq_decode_attention_static(const qaq_cache* c, const void
     if (c->tokens < 1) return QAQ_ERR_INVALID_ARG;
     const int D = c->cfg.head_dim;
     if (!static_scratch_fits(c->BH, c->tokens, D)) return QAQ_ERR_WORKSPACE;  // shape too large for the built-in scratch
-    if (decode_ws_bytes<1>(c->BH, D, 1) > QAQ_STATIC_SCRATCH_BYTES) return QAQ_ERR_WORKSPACE;   // never: the limit above is the tighter one
 
     int dev = -1;
     QAQ_CUDA_TRY(cudaGetDevice(&dev));

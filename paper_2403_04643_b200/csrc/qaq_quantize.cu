@@ -65,7 +65,7 @@ __device__ __forceinline__ uint32_t pool_take(uint32_t* pool, uint32_t amount, u
 //
 // What bounds it: instructions (70 % of the issue slots, 60 % of the integer unit's cycles at 7B, batch 8).  A kernel with
 // 256 threads per tile, a lane per 32 channels of a token throughout and an image of the tile in shared memory took
-// 7300 (keys) and 9100 (values) warp instructions per tile, this one 4200 on average.  4096 tokens, 256 (b,h), head_dim
+// 7300 (keys) and 9100 (values) warp instructions per tile, this one 4400 on average.  4096 tokens, 256 (b,h), head_dim
 // 128: 173 us for keys and values, against 323 us; one warp per tile 231 us (as many tiles in flight per SM, for their
 // shared memory); rounds unrolled by two 7 % slower, by four 20 % (the code of one round is what the instruction cache
 // holds); the window in batches of 16 loads 3 % slower, eleven CTAs per SM 3 %.  32 (b,h) of one tile 7.0 against 7.7 us, of 16 tiles 10.5 against 17.2 us.
