@@ -527,7 +527,8 @@ __device__ void merge_split(const DecArgs& a, DecSmem<D, NQ>& sm, int bh, int nt
             if (tid < CT) {
                 const float inv = mine.l > 0.f ? 1.0f / mine.l : 0.f;
                 float* o = gr.out + (size_t)bh * a.out_stride + j * D + 4 * d4;
-                o[0] = mine.x.x * inv; o[1] = mine.x.y * inv; o[2] = mine.x.z * inv; o[3] = mine.x.w * inv;
+                const bool any = inv > 0.f;           // (a sum that is zero or not a number: zeros, as where nothing is merged)
+                o[0] = any ? mine.x.x * inv : 0.f; o[1] = any ? mine.x.y * inv : 0.f; o[2] = any ? mine.x.z * inv : 0.f; o[3] = any ? mine.x.w * inv : 0.f;
             }
             if (NQ == 1) {
                 if (a.ml && tid == 0) { a.ml[2 * bh] = mine.m; a.ml[2 * bh + 1] = mine.l; }

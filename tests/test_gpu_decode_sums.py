@@ -126,3 +126,19 @@ def test_several_queries_where_many_entries_are_outliers(n_q, D, alpha, scale):
         # queries.  Beyond that binary32 sums of up to 128 terms in another order.
         terms = D * 2.0 ** -22 * (qs.abs().max() * K.abs().max()).item() / math.sqrt(D)
         assert (got[:, j] - one).abs().max().item() <= (2 * terms + 128 * 2.0 ** -23) * V.abs().max().item()
+
+
+@pytest.mark.parametrize("heads,tokens,n_q", [(2, 100, 1), (3, 2100, 4), (14, 2100, 1), (14, 2100, 7), (200, 1000, 2)])
+def test_an_infinite_logit_gives_zeros_however_the_sequence_is_split(heads, tokens, n_q):
+    # one CTA, clusters, partials merged through memory: a key with an infinity that is no outlier has an infinite logit here
+    D = 128
+    g = torch.Generator().manual_seed(heads)
+    K, V = (torch.randn((1, heads, tokens, D), generator=g).half() for _ in range(2))
+    K[:, 0, tokens // 3, 5] = math.inf
+    cfg = qaq.make_config(1, heads, D, tokens, 1, 8, 1, 0.0)
+    thr = torch.tensor([-math.inf, math.inf] * 2).repeat(heads, 1).cuda().contiguous()
+    cache = qaq.Cache(cfg)
+    bits = torch.full((heads, tokens), 4, dtype=torch.uint8, device="cuda")
+    qaq.qaq_quantize_append(cache, K.cuda(), V.cuda(), thr, bitsK=bits, bitsV=bits)
+    out = qaq.qaq_decode_attention_multi(cache, torch.rand((heads, n_q, D), generator=g).half().cuda(), 1 / math.sqrt(D))
+    assert (out[0] == 0).all() and torch.isfinite(out).all() and (out[1:] != 0).any(dim=2).all()
