@@ -1214,7 +1214,7 @@ template <int D, int NQ, bool COUNTED>
 qaq_status launch_decode(const DecArgs& a, cudaStream_t s) {
     const size_t smem = sizeof(DecSmem<D, NQ>);
     static_assert(sizeof(DecSmem<D, NQ>) + 1024 <= 227 * 1024 / Shape<NQ>::CTAS_PER_SM, "shared memory of the CTAs of an SM");
-    static std::atomic<unsigned long long> seen[2];
+    static SmemSeen seen[2];
     const dim3 grid(a.ncta, a.groups), block(Shape<NQ>::THREADS);
     if (a.cluster) {
         QAQ_CUDA_TRY(qaq_allow_smem((const void*)decode_kernel<D, NQ, COUNTED, true>, smem, seen[1]));

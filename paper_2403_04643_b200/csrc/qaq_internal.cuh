@@ -88,16 +88,24 @@ template <typename... P, typename... A>
 static inline cudaError_t qaq_launch(void (*kernel)(P...), dim3 grid, dim3 block, size_t smem, cudaStream_t s, A... args) {
     return qaq_launch_cluster(kernel, grid, block, 1, smem, s, args...);
 }
-// Shared memory beyond 48 KB has to be allowed once per kernel and device; `seen` (one per kernel) remembers where that
-// has been done (devices 0..63; others are asked every time).
-static inline cudaError_t qaq_allow_smem(const void* kernel, size_t smem, std::atomic<unsigned long long>& seen) {
-    int dev = 0;
-    cudaError_t e = cudaGetDevice(&dev);
-    if (e != cudaSuccess) return e;
-    const unsigned long long bit = dev < 64 ? 1ull << dev : 0ull;
-    if (seen.load(std::memory_order_acquire) & bit) return cudaSuccess;
-    e = cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
-    if (e == cudaSuccess) seen.fetch_or(bit, std::memory_order_release);
+// Shared memory beyond 48 KB has to be allowed once per kernel and context.  `seen` (one per kernel) remembers contexts by their
+// ids, which are not used again; where a context has no id yet, or another one has taken its place, the kernel is allowed once more.
+struct SmemSeen { std::atomic<unsigned long long> id[8]; };
+static inline cudaError_t qaq_allow_smem(const void* kernel, size_t smem, SmemSeen& seen) {
+    typedef int (*GetId)(void* context, unsigned long long* id);          // cuCtxGetId; null: the current context
+    static const GetId get_id = [] {
+        void* f = nullptr;
+        cudaDriverEntryPointQueryResult found;
+        const cudaError_t e = cudaGetDriverEntryPointByVersion("cuCtxGetId", &f, 12000, cudaEnableDefault, &found);
+        if (e != cudaSuccess) (void)cudaGetLastError();
+        return e == cudaSuccess && found == cudaDriverEntryPointSuccess ? (GetId)f : (GetId) nullptr;
+    }();
+    unsigned long long id = 0;
+    const bool known = get_id && get_id(nullptr, &id) == 0;
+    // (an entry holds the id plus one: zero is an empty one)
+    if (known && seen.id[id % 8].load(std::memory_order_acquire) == id + 1) return cudaSuccess;
+    const cudaError_t e = cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+    if (e == cudaSuccess && known) seen.id[id % 8].store(id + 1, std::memory_order_release);
     return e;
 }
 

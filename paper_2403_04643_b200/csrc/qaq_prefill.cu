@@ -398,7 +398,7 @@ __global__ void __launch_bounds__(PC_WARPS * 32, PC_MINCTA) window_cluster_kerne
 
 template <int D>
 qaq_status run_cluster(const PrefillArgs& a, int BH, int ncl, size_t smem, cudaStream_t s) {
-    static std::atomic<unsigned long long> seen{0};
+    static SmemSeen seen;
     const size_t most = (size_t)PW_MAXQ * PC_PITCH * sizeof(float) + 4 * (D / 16) * 32 * sizeof(uint4);
     QAQ_CUDA_TRY(qaq_allow_smem((const void*)window_cluster_kernel<D>, most, seen));
     QAQ_CUDA_TRY(qaq_launch_cluster(window_cluster_kernel<D>, dim3((unsigned)ncl, (unsigned)BH), dim3(PC_WARPS * 32), ncl, smem, s, a));

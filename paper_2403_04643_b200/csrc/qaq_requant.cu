@@ -460,13 +460,13 @@ extern "C" qaq_status qaq_cache_compact(qaq_cache* c, void* stream) {
     while (a.n2 < nt) a.n2 <<= 1;
     // 512 threads while all pools are worked on at once (two to an SM), else 256 (256 (b,h) of 4096 tokens, one tile moved: 21.5
     // us with 512, 14.3 with 256, all tiles moved 50 and 44)
-    auto launch = [&](auto kernel, int threads, std::atomic<unsigned long long>& seen) {
+    auto launch = [&](auto kernel, int threads, SmemSeen& seen) {
         auto smem_for = [](int n2) { return (size_t)n2 * 8 + (size_t)(n2 + 1) * 4 + 16 * 4; };
         QAQ_CUDA_TRY(qaq_allow_smem((const void*)kernel, smem_for(COMPACT_MAX_TILES), seen));
         QAQ_CUDA_TRY(qaq_launch(kernel, dim3((unsigned)c->BH, 2), dim3((unsigned)threads), smem_for(a.n2), (cudaStream_t)stream, a));
         return QAQ_OK;
     };
-    static std::atomic<unsigned long long> seen[2];
+    static SmemSeen seen[2];
     return 2 * c->BH <= 2 * 148 ? launch(compact_kernel<512>, 512, seen[0]) : launch(compact_kernel<256>, 256, seen[1]);
 }
 

@@ -600,7 +600,7 @@ extern "C" qaq_status qaq_outlier_thresholds(const qaq_config* cfg, const void* 
     a.scan_tokens = SCAN_TOKENS_MAX;
     const size_t keys = (size_t)n_tokens * cfg->head_dim, small = sizeof(SmallScratch) + keys * sizeof(unsigned short);
     if (n_tokens > SAMPLE_TOKENS && keys <= SMALL_KEYS) {
-        static std::atomic<unsigned long long> seen{0};
+        static SmemSeen seen;
         QAQ_CUDA_TRY(qaq_allow_smem((const void*)thr_small_kernel, sizeof(SmallScratch) + SMALL_KEYS * sizeof(unsigned short), seen));
         QAQ_CUDA_TRY(qaq_launch(thr_small_kernel, dim3(BH * 2), dim3(SMALL_THREADS), small, s, a));
         return QAQ_OK;
