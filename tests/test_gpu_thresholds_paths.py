@@ -62,10 +62,10 @@ def test_constant_tensor_and_single_distinct_tail_value():
 
 
 @pytest.mark.parametrize("alpha", [0.3, 0.5, 1.0])
-def test_tails_so_heavy_that_every_scan_block_overflows(alpha):
-    # a third of the entries (or more) beyond the bracket per tail: every block of the scan finds more candidates
-    # than it can hold, while the global list would have room for the count - the holes must send the problem to the
-    # exact select over its data
+def test_tails_so_heavy_that_most_entries_are_candidates(alpha):
+    # a third of the entries (or more) beyond the bracket per tail: scan blocks of 64 tokens, whose lists hold them, and lists of
+    # a problem that are longer than what the select keeps on chip (blocks that find more than they hold: the tests of tails
+    # in one part of the sequence, and the collapsed bracket)
     wl = synth.scaled(synth.CONFIGS["C2"], heads=2, tokens=2048)
     K, V = synth.make_kv(wl, 0)
     check(K, V, wl, alpha)

@@ -131,9 +131,10 @@ def test_several_queries_in_one_launch_or_in_turn(n_q, heads, tokens):
     got = qaq.qaq_decode_attention_multi(cache, qs, 1 / math.sqrt(D))
     for j in range(n_q):
         one = qaq.qaq_decode_attention(cache, qs[:, j].contiguous(), 1 / math.sqrt(D))
-        # Both take the same integer products, but key corrections are summed in a unit that depends on the largest of the
-        # queries of a pass: 2^-22 of at most twice the bound 2 max|q| max|x|, so a token's few terms (at most 4 here) move a
-        # logit by at most 4 * 2^-22 * 2 max|q| max|x| / sqrt(D), and its weight relatively by as much.
+        # Both take the same integer products; key corrections are summed in units of 2^-24 of at most twice the query's own bound
+        # 2 max|q| max|x| (of the power of two above max|q| where several share a pass), so a token's few terms (at most 4
+        # here) move a logit by at most 4 * 2^-24 * 4 max|q| max|x| / sqrt(D), and its weight relatively by as much.  (The same
+        # bound pays for binary32 sums in another order.)
         bound = 4 * 2.0 ** -22 * 2 * qs.abs().max().item() * K.abs().max().item() / math.sqrt(D)
         assert (got[:, j] - one).abs().max().item() <= 2 * bound * V.abs().max().item()
 
