@@ -204,15 +204,20 @@ struct Group {
 // Short sequences: the CTAs of a (b,h) are a thread-block cluster, with as many tiles each, and their results meet in shared
 // memory.  (Through memory - partials stored, CTAs counted by an atomic, partials loaded by the last one - a split costs 3 to
 // 4 us: 32 (b,h) of 8 tiles, one CTA each, 8.3 us, of 9 tiles 12.4.)  Taken where a portable cluster makes no warp do
-// more tiles than the flattened sequence would.  Returns the size of the cluster, 0: the flattened sequence.
-template <int NQ>
-inline int plan_cluster(int BH, int ntiles, int groups) {
+// more tiles than the flattened sequence would and the clusters all run at once: fits(k) says how many of k CTAs can (a cluster
+// stays inside a part of the chip, so that 96 of three are fewer than 296 places promise: 96 (b,h) of 20975 tokens took 113 us in
+// clusters of three, 74 as a flattened sequence).  Returns the size of the cluster, 0: the flattened sequence.
+template <int NQ, class F>
+inline int plan_cluster(int BH, int ntiles, int groups, F&& fits) {
     using S = Shape<NQ>;
     const int places = S::SLOTS / groups / BH;               // CTAs a (b,h) can have at once
-    const int k = min(min(8, places), (ntiles + S::WARPS - 1) / S::WARPS);
-    if (k < 2) return 0;
-    const int run = plan_decode<NQ>(BH, ntiles, groups).run, crun = (ntiles + k - 1) / k;
-    return (crun + S::WARPS - 1) / S::WARPS <= (run + S::WARPS - 1) / S::WARPS ? k : 0;
+    const int run = plan_decode<NQ>(BH, ntiles, groups).run;
+    for (int k = min(min(8, places), (ntiles + S::WARPS - 1) / S::WARPS); k >= 2; --k) {
+        const int crun = (ntiles + k - 1) / k;
+        if ((crun + S::WARPS - 1) / S::WARPS > (run + S::WARPS - 1) / S::WARPS) return 0;
+        if (BH * groups <= fits(k)) return k;
+    }
+    return 0;
 }
 
 // ------------------------------------------------------------------------------------------ shared memory
@@ -1210,14 +1215,39 @@ unsigned long long call_tag() {
     return z ? z : 0x1000ull;
 }
 
+// How many clusters of k CTAs of a kernel run at once: asked once per kernel, k and context (whose id goes with the answer).
+struct ClusterRoom { std::atomic<unsigned long long> known[9]; };
+template <class K>
+int clusters_at_once(K kernel, int threads, size_t smem, int k, ClusterRoom& room) {
+    unsigned long long id = 0;
+    const bool named = qaq_context_id(id);
+    const unsigned long long was = room.known[k].load(std::memory_order_acquire);
+    if (named && (was >> 16) == id + 1) return (int)(was & 0xFFFFu);
+    cudaLaunchAttribute at;
+    at.id = cudaLaunchAttributeClusterDimension;
+    at.val.clusterDim.x = (unsigned)k; at.val.clusterDim.y = 1; at.val.clusterDim.z = 1;
+    cudaLaunchConfig_t lc = {};
+    lc.gridDim = dim3((unsigned)k); lc.blockDim = dim3((unsigned)threads); lc.dynamicSmemBytes = smem; lc.attrs = &at; lc.numAttrs = 1;
+    int n = 0;
+    if (cudaOccupancyMaxActiveClusters(&n, kernel, &lc) != cudaSuccess) { (void)cudaGetLastError(); return 0; }
+    n = n < 0 ? 0 : n > 0xFFFF ? 0xFFFF : n;
+    if (named) room.known[k].store((id + 1) << 16 | (unsigned)n, std::memory_order_release);
+    return n;
+}
+
 template <int D, int NQ, bool COUNTED>
-qaq_status launch_decode(const DecArgs& a, cudaStream_t s) {
+qaq_status launch_decode(DecArgs a, cudaStream_t s) {
     const size_t smem = sizeof(DecSmem<D, NQ>);
     static_assert(sizeof(DecSmem<D, NQ>) + 1024 <= 227 * 1024 / Shape<NQ>::CTAS_PER_SM, "shared memory of the CTAs of an SM");
     static SmemSeen seen[2];
+    static ClusterRoom room;
+    QAQ_CUDA_TRY(qaq_allow_smem((const void*)decode_kernel<D, NQ, COUNTED, true>, smem, seen[1]));
+    a.cluster = plan_cluster<NQ>(a.BH, (a.T + QAQ_TILE - 1) / QAQ_TILE, a.groups, [&](int k) {
+        return clusters_at_once(decode_kernel<D, NQ, COUNTED, true>, Shape<NQ>::THREADS, smem, k, room);
+    });
+    if (a.cluster) a.ncta = a.BH * a.cluster;
     const dim3 grid(a.ncta, a.groups), block(Shape<NQ>::THREADS);
     if (a.cluster) {
-        QAQ_CUDA_TRY(qaq_allow_smem((const void*)decode_kernel<D, NQ, COUNTED, true>, smem, seen[1]));
         QAQ_CUDA_TRY(qaq_launch_cluster(decode_kernel<D, NQ, COUNTED, true>, grid, block, a.cluster, smem, s, a));
     } else {
         QAQ_CUDA_TRY(qaq_allow_smem((const void*)decode_kernel<D, NQ, COUNTED, false>, smem, seen[0]));
@@ -1250,8 +1280,7 @@ qaq_status decode(const qaq_cache* c, const void* q, long q_stride, float softma
     a.BH = BH;
     a.run = COUNTED ? 0 : plan.run;
     a.ncta = COUNTED ? (BH > Shape<NQ>::SLOTS ? BH : Shape<NQ>::SLOTS) : plan.ncta;   // counted: the largest grid any count needs
-    a.cluster = plan_cluster<NQ>(BH, (a.T + QAQ_TILE - 1) / QAQ_TILE, a.groups);
-    if (a.cluster) a.ncta = BH * a.cluster;
+    a.cluster = 0;               // (launch_decode)
     // nothing in the workspace is read before it is written (the counting words: see merge_split)
     a.part = (float*)ws;
     a.done = (unsigned long long*)(a.part + (size_t)(BH > Shape<NQ>::SLOTS ? 0 : 2 * Shape<NQ>::SLOTS) * NQ * (D + 4));

@@ -91,7 +91,8 @@ static inline cudaError_t qaq_launch(void (*kernel)(P...), dim3 grid, dim3 block
 // Shared memory beyond 48 KB has to be allowed once per kernel and context.  `seen` (one per kernel) remembers contexts by their
 // ids, which are not used again; where a context has no id yet, or another one has taken its place, the kernel is allowed once more.
 struct SmemSeen { std::atomic<unsigned long long> id[8]; };
-static inline cudaError_t qaq_allow_smem(const void* kernel, size_t smem, SmemSeen& seen) {
+// the id of the current context; false where there is none
+static inline bool qaq_context_id(unsigned long long& id) {
     typedef int (*GetId)(void* context, unsigned long long* id);          // cuCtxGetId; null: the current context
     static const GetId get_id = [] {
         void* f = nullptr;
@@ -100,8 +101,11 @@ static inline cudaError_t qaq_allow_smem(const void* kernel, size_t smem, SmemSe
         if (e != cudaSuccess) (void)cudaGetLastError();
         return e == cudaSuccess && found == cudaDriverEntryPointSuccess ? (GetId)f : (GetId) nullptr;
     }();
+    return get_id && get_id(nullptr, &id) == 0;
+}
+static inline cudaError_t qaq_allow_smem(const void* kernel, size_t smem, SmemSeen& seen) {
     unsigned long long id = 0;
-    const bool known = get_id && get_id(nullptr, &id) == 0;
+    const bool known = qaq_context_id(id);
     // (an entry holds the id plus one: zero is an empty one)
     if (known && seen.id[id % 8].load(std::memory_order_acquire) == id + 1) return cudaSuccess;
     const cudaError_t e = cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);

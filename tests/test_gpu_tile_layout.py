@@ -221,3 +221,17 @@ def test_sequences_split_over_a_cluster(D, tokens):
         # the same tiles, summed in another order: binary32 rounding of at most 65 partial sums and weights
         assert (got - want).abs().max().item() <= 65 * 2.0 ** -23 * 4 * V.abs().max().item()
         assert torch.allclose(row[:, :n].sum(1), torch.ones(wl.bh, device="cuda"), atol=1e-3)
+
+
+@pytest.mark.parametrize("heads,tokens", [(37, 1100), (49, 1600), (73, 1025), (74, 1025), (96, 2000), (98, 2000), (148, 1100)])
+def test_sequences_of_many_heads_whose_clusters_may_not_all_run_at_once(heads, tokens):
+    # near the largest number of (b,h) for clusters of 8, 6, 4, 3 and 2 CTAs: smaller clusters or the flattened sequence, same result
+    D = 32
+    wl = synth.scaled(synth.CONFIGS["C2"], heads=heads, head_dim=D, tokens=tokens)
+    K, V, q, ring, nv = make_inputs(wl)
+    pol = qaq.qaq_policy_from_hyper(*HYPER, tokens)
+    cfg, cache, thr, out, scores, dev = gpu_pipeline(wl, K, V, q, ring, nv, pol)
+    ref = oracle_batch(wl, K, V, q, ring, nv, pol.cK, pol.cV)
+    assert_attention_close(out.cpu().numpy(), ref.X)
+    S = scores.cpu().numpy().astype(np.float64)
+    assert np.all(np.abs(S - ref.S) <= 1e-6 + 1e-2 * ref.S) and np.allclose(S.sum(1), 1.0, atol=1e-3)
