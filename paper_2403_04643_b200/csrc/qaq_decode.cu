@@ -70,7 +70,6 @@ __device__ __forceinline__ void mma_k32_first(int (&d)[4], uint32_t a0, uint32_t
                  : "=r"(d[0]), "=r"(d[1]), "=r"(d[2]), "=r"(d[3])
                  : "r"(a0), "r"(a1), "r"(a2), "r"(a3), "r"(b0), "r"(b1), "r"(0));
 }
-__device__ __forceinline__ uint32_t smem_addr(const void* p) { return (uint32_t)__cvta_generic_to_shared(p); }
 // W words from shared memory (aligned to the widest access taken: 16 bytes for four words, 8 for two, else 4)
 template <int W>
 __device__ __forceinline__ void lds_words(uint32_t addr, uint32_t (&x)[W]) {
@@ -101,26 +100,9 @@ __device__ __forceinline__ uint32_t ldg_now1(const void* p) {
 }
 
 // bulk copies into shared memory, completion on a transaction barrier
-__device__ __forceinline__ void bar_init(uint32_t bar) { asm volatile("mbarrier.init.shared::cta.b64 [%0], 1;" ::"r"(bar) : "memory"); }
-__device__ __forceinline__ void bar_expect(uint32_t bar, uint32_t bytes) {
-    asm volatile("mbarrier.arrive.expect_tx.shared::cta.b64 _, [%0], %1;" ::"r"(bar), "r"(bytes) : "memory");
-}
 __device__ __forceinline__ void bulk_copy(uint32_t dst, const void* src, uint32_t bytes, uint32_t bar) {
     asm volatile("cp.async.bulk.shared::cluster.global.mbarrier::complete_tx::bytes [%0], [%1], %2, [%3];" ::"r"(dst), "l"(src), "r"(bytes), "r"(bar)
                  : "memory");
-}
-// false if the phase did not complete within the limit (a copy takes microseconds; every try waits for a while itself)
-__device__ __forceinline__ bool bar_wait(uint32_t bar, uint32_t parity) {
-    uint32_t done = 0;
-#pragma unroll 1
-    for (int i = 0; i < (1 << 14) && !done; ++i)
-        asm volatile("{\n.reg .pred p;\nmbarrier.try_wait.parity.shared::cta.b64 p, [%1], %2;\nselp.u32 %0, 1, 0, p;\n}" : "=r"(done) : "r"(bar), "r"(parity) : "memory");
-    return done != 0;
-}
-__device__ __forceinline__ float warp_max(float x) {
-    float r;
-    asm("redux.sync.max.f32 %0, %1, 0xffffffff;" : "=f"(r) : "f"(x));
-    return r;
 }
 __device__ __forceinline__ float warp_sum(float x) {
 #pragma unroll
@@ -1213,26 +1195,6 @@ unsigned long long call_tag() {
     z = (z ^ (z >> 27)) * 0x94D049BB133111EBull;
     z = (z ^ (z >> 31)) & ~0xFFFull;
     return z ? z : 0x1000ull;
-}
-
-// How many clusters of k CTAs of a kernel run at once: asked once per kernel, k and context (whose id goes with the answer).
-struct ClusterRoom { std::atomic<unsigned long long> known[9]; };
-template <class K>
-int clusters_at_once(K kernel, int threads, size_t smem, int k, ClusterRoom& room) {
-    unsigned long long id = 0;
-    const bool named = qaq_context_id(id);
-    const unsigned long long was = room.known[k].load(std::memory_order_acquire);
-    if (named && (was >> 16) == id + 1) return (int)(was & 0xFFFFu);
-    cudaLaunchAttribute at;
-    at.id = cudaLaunchAttributeClusterDimension;
-    at.val.clusterDim.x = (unsigned)k; at.val.clusterDim.y = 1; at.val.clusterDim.z = 1;
-    cudaLaunchConfig_t lc = {};
-    lc.gridDim = dim3((unsigned)k); lc.blockDim = dim3((unsigned)threads); lc.dynamicSmemBytes = smem; lc.attrs = &at; lc.numAttrs = 1;
-    int n = 0;
-    if (cudaOccupancyMaxActiveClusters(&n, kernel, &lc) != cudaSuccess) { (void)cudaGetLastError(); return 0; }
-    n = n < 0 ? 0 : n > 0xFFFF ? 0xFFFF : n;
-    if (named) room.known[k].store((id + 1) << 16 | (unsigned)n, std::memory_order_release);
-    return n;
 }
 
 template <int D, int NQ, bool COUNTED>

@@ -72,6 +72,25 @@ static inline unsigned* qaq_d_pool_use(const qaq_cache* c) { return (unsigned*)(
 __device__ __forceinline__ void qaq_dependency() {
     asm volatile("griddepcontrol.wait;" ::: "memory");
 }
+__device__ __forceinline__ uint32_t smem_addr(const void* p) { return (uint32_t)__cvta_generic_to_shared(p); }
+// transaction barriers in shared memory, for one arrival
+__device__ __forceinline__ void bar_init(uint32_t bar) { asm volatile("mbarrier.init.shared::cta.b64 [%0], 1;" ::"r"(bar) : "memory"); }
+__device__ __forceinline__ void bar_expect(uint32_t bar, uint32_t bytes) {
+    asm volatile("mbarrier.arrive.expect_tx.shared::cta.b64 _, [%0], %1;" ::"r"(bar), "r"(bytes) : "memory");
+}
+// false if the phase did not complete within the limit (a copy takes microseconds; every try waits for a while itself)
+__device__ __forceinline__ bool bar_wait(uint32_t bar, uint32_t parity) {
+    uint32_t done = 0;
+#pragma unroll 1
+    for (int i = 0; i < (1 << 14) && !done; ++i)
+        asm volatile("{\n.reg .pred p;\nmbarrier.try_wait.parity.shared::cta.b64 p, [%1], %2;\nselp.u32 %0, 1, 0, p;\n}" : "=r"(done) : "r"(bar), "r"(parity) : "memory");
+    return done != 0;
+}
+__device__ __forceinline__ float warp_max(float x) {
+    float r;
+    asm("redux.sync.max.f32 %0, %1, 0xffffffff;" : "=f"(r) : "f"(x));
+    return r;
+}
 // cluster: CTAs (consecutive in x) that form a thread-block cluster
 template <typename... P, typename... A>
 static inline cudaError_t qaq_launch_cluster(void (*kernel)(P...), dim3 grid, dim3 block, int cluster, size_t smem, cudaStream_t s, A... args) {
@@ -111,6 +130,25 @@ static inline cudaError_t qaq_allow_smem(const void* kernel, size_t smem, SmemSe
     const cudaError_t e = cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
     if (e == cudaSuccess && known) seen.id[id % 8].store(id + 1, std::memory_order_release);
     return e;
+}
+// How many clusters of k CTAs of a kernel run at once: asked once per kernel, k and context (whose id goes with the answer).
+struct ClusterRoom { std::atomic<unsigned long long> known[9]; };
+template <class K>
+int clusters_at_once(K kernel, int threads, size_t smem, int k, ClusterRoom& room) {
+    unsigned long long id = 0;
+    const bool named = qaq_context_id(id);
+    const unsigned long long was = room.known[k].load(std::memory_order_acquire);
+    if (named && (was >> 16) == id + 1) return (int)(was & 0xFFFFu);
+    cudaLaunchAttribute at;
+    at.id = cudaLaunchAttributeClusterDimension;
+    at.val.clusterDim.x = (unsigned)k; at.val.clusterDim.y = 1; at.val.clusterDim.z = 1;
+    cudaLaunchConfig_t lc = {};
+    lc.gridDim = dim3((unsigned)k); lc.blockDim = dim3((unsigned)threads); lc.dynamicSmemBytes = smem; lc.attrs = &at; lc.numAttrs = 1;
+    int n = 0;
+    if (cudaOccupancyMaxActiveClusters(&n, kernel, &lc) != cudaSuccess) { (void)cudaGetLastError(); return 0; }
+    n = n < 0 ? 0 : n > 0xFFFF ? 0xFFFF : n;
+    if (named) room.known[k].store((id + 1) << 16 | (unsigned)n, std::memory_order_release);
+    return n;
 }
 
 // Space taken from a pool that turned out not to fit is given back only while nothing has been taken behind it: with a

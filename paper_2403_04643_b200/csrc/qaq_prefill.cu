@@ -6,412 +6,642 @@
 // Rows are written newest first (row r = query n-1-r), so that the rows in which token t exists
 // are 0..nvalid[t]-1 with nvalid[t] = min(n, T-t); entries of tokens a query cannot see are 0.
 //
-// This is the one dense contraction on the path ([n x D] x [D x T] per (b,h)), so the logits run
-// on the tensor cores (mma.sync m16n8k16, binary16 in, binary32 accumulate); with n <= 64 rows it is
-// bound by reading K once.  Sequences of up to 4096 tokens take one kernel whose CTAs form a
-// thread-block cluster per (b,h) (logits stay in shared memory, row statistics travel through
-// distributed shared memory, the ring is written once); longer ones take two passes of one kernel: the first
-// leaves (max, sum of exponentials) of every row per chunk of tokens, the second computes the logits again
-// and writes the rows normalised with the merged statistics.
-#include <cooperative_groups.h>
+// This is the one dense contraction on the path ([n x D] x [D x T] per (b,h)); with n <= 64 rows it is bound by reading K once, and by
+// the exponentials and stores of the rows.  The logits of 128 tokens are one accumulator of the fifth-generation tensor cores
+// (tcgen05.mma, binary16 in, binary32 sums in tensor memory: a token a lane, a query a column), so neither the keys nor the
+// logits pass through registers on their way there, and a row's 32 consecutive tokens are one store of a warp.  What the keys
+// wait for in the meantime decides between three ways:
+//   window_short_kernel   few tiles in all: the logits in registers, many CTAs per SM.
+//   window_kernel         one pass: resident CTAs, the logits of a (b,h) in the tensor memory of a cluster until the statistics of its
+//                         rows are known; K is read once and the rows written once.
+//                         Two passes, (b,h) longer than that (8192 tokens with 64 rows, 16384 with 32, 32768 with 16): statistics per
+//                         chunk of tokens, then the logits again and the rows.
+// Before (mma.sync fragments from global memory, logits in shared memory; beyond 4096 tokens two passes), now: 256 (b,h) of 4096
+// tokens, 32 rows 129 and 70 us, with 64 rows 345 and 115; 160 of 8192, 64 rows 321 and 152; 32 of 32768, 32 rows 187 and 118; 32 of 333
+// 8.3 and 5.5; 256 of 300 11.9 and 9.2.
+#include <cuda.h>
 
 #include "qaq_internal.cuh"
 
 namespace {
 
-constexpr int PW_WARPS = 8;            // three CTAs per SM (80 registers per thread)
-constexpr int PW_CHUNK = 512;          // tokens per CTA: 64 per warp, 16 at a time
+constexpr int PW_CHUNK = 512;          // tokens per entry of the workspace's statistics at least
 constexpr int PW_MAXQ = 64;            // rows (queries) at most
+constexpr int PW_TILE = 128;           // tokens per accumulator: rows of the tensor-core instruction
+constexpr int PW_CLUSTER = 8;          // CTAs of a cluster at most
+constexpr int PW_SMEM = 227 * 1024;    // all of it: a CTA has its SM, and the SM's tensor memory, to itself
+constexpr int PW_WORKERS = 16;         // warps that look at the logits: groups of four, up to 32 columns of a tile each
+constexpr int PW_THREADS = 32 * (2 + PW_WORKERS);
 
 struct PrefillArgs {
     const __half* Q;     // [BH][n][D]
-    const __half* K;
-    long sb, sh, st;
-    int H, T, n;
+    int H, BH, T, n;
     float scale;
     float* ring;         // [BH][n][T]
     uint8_t* nvalid;     // [BH][T]
     float* qnorm2;       // [BH][n] or null
-    float2* part;        // [BH][nchunk][n] (max, sum of exp) of the visible logits of a chunk
-    int nchunk;
+    float2* part;        // [BH][nchunk][n] (reference, sum of powers of two relative to it) of the visible logits of a chunk
+    int nchunk, tiles;   // chunks of a (b,h); tiles of a chunk, or of a CTA of a cluster
 };
 
-__device__ __forceinline__ void mma_16816(float (&c)[4], const uint32_t (&a)[4], uint32_t b0, uint32_t b1) {
-    asm volatile("mma.sync.aligned.m16n8k16.row.col.f32.f16.f16.f32 {%0,%1,%2,%3}, {%4,%5,%6,%7}, {%8,%9}, {%0,%1,%2,%3};\n"
-                 : "+f"(c[0]), "+f"(c[1]), "+f"(c[2]), "+f"(c[3])
-                 : "r"(a[0]), "r"(a[1]), "r"(a[2]), "r"(a[3]), "r"(b0), "r"(b1));
-}
+// ONE_PASS: the CTAs of a cluster share a (b,h) and keep its logits in tensor memory until they have the statistics of its rows.
+// STATS, ROWS: two passes over chunks of any length.
+enum { ONE_PASS, STATS, ROWS };
 
-// The queries as A-operand fragments in shared memory, one uint4 per (16-row tile, k step, lane): every warp reads the
-// same ones.  The contraction index is permuted the same way in both operands: lane (., c) of k step ks takes words
-// 2 (ks mod 2), + 1 of the 16-byte piece 4 (ks / 2) + c of a row.
-template <int D>
-__device__ __forceinline__ void lay_out_queries(uint4* s_q, const __half* Qb, int n) {
-    constexpr int KS = D / 16;
-    const int ntile = 2 * ((n + 31) / 32);
-    for (int idx = threadIdx.x; idx < ntile * KS * 32; idx += blockDim.x) {
-        const int ln = idx & 31, ks = (idx >> 5) % KS, tile = idx / (32 * KS);
-        const int r0 = tile * 16 + (ln >> 2), r1 = r0 + 8, cc = ln & 3;
-        const int w0 = 4 * (4 * (ks >> 1) + cc) + 2 * (ks & 1);
-        const uint32_t* q0 = reinterpret_cast<const uint32_t*>(Qb + (size_t)r0 * D) + w0;
-        const uint32_t* q1 = reinterpret_cast<const uint32_t*>(Qb + (size_t)r1 * D) + w0;
-        uint4 f;
-        f.x = r0 < n ? q0[0] : 0u;
-        f.y = r1 < n ? q1[0] : 0u;
-        f.z = r0 < n ? q0[1] : 0u;
-        f.w = r1 < n ? q1[1] : 0u;
-        s_q[idx] = f;
+// Operands in shared memory: rows of 64 channels (head_dim 128: two such regions) or 32, their 16-byte pieces swizzled.
+template <int D, int NC, int MODE>
+struct Window {
+    static constexpr int ROW_BYTES = D >= 64 ? 128 : 64, REGIONS = (D + 63) / 64;
+    static constexpr uint32_t TILE_BYTES = PW_TILE * D * 2, QUERY_BYTES = NC * D * 2;
+    static constexpr int SLOTS = 512 / NC;                   // accumulators in tensor memory
+    static constexpr bool SPLIT = MODE == ONE_PASS && NC <= 32;                                         // statistics and rows by warps of their own
+    static constexpr int TEAM = SPLIT ? PW_WORKERS / 2 : PW_WORKERS;                                    // warps with the same job
+    static constexpr int CW = NC < 32 ? NC : 32, PARTS = NC / CW, GROUPS = TEAM / 4 / PARTS;            // columns of a warp; groups that share a tile; tiles at a time
+    struct Shared {
+        unsigned long long full[8], empty[8];                // stages of the keys
+        unsigned long long there[SLOTS], taken[SLOTS];       // accumulators
+        unsigned long long q_free[2], stats[2], used[2];     // queries; statistics of the cluster's CTAs: there, no longer needed by any
+        alignas(16) float ref[2][TEAM][CW], sum[2][TEAM][CW];      // of a warp: reference and sum of every row over its tokens
+        alignas(16) float2 all[2][PW_CLUSTER][NC];           // the same of every CTA of the cluster, which all write here
+        alignas(16) float2 row[2][NC];                        // what the rows are normalised with: reference, 1 / sum
+        uint32_t tmem;
+    };
+    static constexpr int FIT = (PW_SMEM - 1024 - 2 * (int)QUERY_BYTES - (int)sizeof(Shared)) / (int)TILE_BYTES, STAGES = FIT < 8 ? FIT : 8;
+    static_assert(STAGES >= 4, "stages");
+};
+
+__device__ __forceinline__ void bulk_tile(uint32_t dst, const CUtensorMap* map, int x, int t, int h, int b, uint32_t bar) {
+    asm volatile("cp.async.bulk.tensor.4d.shared::cluster.global.mbarrier::complete_tx::bytes [%0], [%1, {%3, %4, %5, %6}], [%2];"
+                 ::"r"(dst), "l"(map), "r"(bar), "r"(x), "r"(t), "r"(h), "r"(b) : "memory");
+}
+__device__ __forceinline__ void bulk_rows(uint32_t dst, const CUtensorMap* map, int x, int row, uint32_t bar) {
+    asm volatile("cp.async.bulk.tensor.2d.shared::cluster.global.mbarrier::complete_tx::bytes [%0], [%1, {%3, %4}], [%2];"
+                 ::"r"(dst), "l"(map), "r"(bar), "r"(x), "r"(row) : "memory");
+}
+__device__ __forceinline__ void bar_init(uint32_t bar, uint32_t arrivals) { asm volatile("mbarrier.init.shared::cta.b64 [%0], %1;" ::"r"(bar), "r"(arrivals) : "memory"); }
+__device__ __forceinline__ void bar_arrive(uint32_t bar) { asm volatile("mbarrier.arrive.shared::cta.b64 _, [%0];" ::"r"(bar) : "memory"); }
+// for what other CTAs of the cluster have done
+__device__ __forceinline__ bool bar_wait_cluster(uint32_t bar, uint32_t parity) {
+    uint32_t done = 0;
+#pragma unroll 1
+    for (int i = 0; i < (1 << 14) && !done; ++i)
+        asm volatile("{\n.reg .pred p;\nmbarrier.try_wait.parity.acquire.cluster.shared::cta.b64 p, [%1], %2;\nselp.u32 %0, 1, 0, p;\n}" : "=r"(done) : "r"(bar), "r"(parity) : "memory");
+    return done != 0;
+}
+__device__ __forceinline__ void tensor_done(uint32_t bar) {           // arrives when what this thread has asked of the tensor cores is done
+    asm volatile("tcgen05.commit.cta_group::1.mbarrier::arrive::one.shared::cluster.b64 [%0];" ::"r"(bar) : "memory");
+}
+template <int ROW_BYTES>
+__device__ __forceinline__ uint64_t operand(uint32_t addr) {          // K-major, swizzled over its row length, eight rows and then the next eight
+    return (uint64_t)((addr & 0x3FFFFu) >> 4) | (1ull << 16) | ((uint64_t)(8 * ROW_BYTES / 16) << 32) | (1ull << 46) | ((uint64_t)(ROW_BYTES == 128 ? 2 : 4) << 61);
+}
+// accumulator (128 lanes x NC columns of tensor memory) = tile . queries; by one thread
+template <int D, int NC>
+__device__ __forceinline__ void multiply(uint32_t acc, uint32_t tile, uint32_t queries) {
+    constexpr uint32_t kind = (1u << 4) | (NC / 8) << 17 | (PW_TILE / 16) << 24;           // binary32 sums of binary16 products
+    constexpr int RB = Window<D, NC, STATS>::ROW_BYTES, PER = RB / 32;                            // steps of 16 channels per region
+#pragma unroll
+    for (int ks = 0; ks < D / 16; ++ks) {
+        const uint64_t x = operand<RB>(tile + (ks / PER) * (PW_TILE * RB) + (ks % PER) * 32), y = operand<RB>(queries + (ks / PER) * (NC * RB) + (ks % PER) * 32);
+        asm volatile("{\n.reg .pred p;\nsetp.ne.u32 p, %4, 0;\ntcgen05.mma.cta_group::1.kind::f16 [%0], %1, %2, %3, p;\n}"
+                     ::"r"(acc), "l"(x), "l"(y), "r"(kind), "r"(ks) : "memory");
     }
 }
-
-template <int D>
-__device__ __forceinline__ void query_norms(const PrefillArgs& a, int bh) {
-    const __half* Qb = a.Q + (size_t)bh * a.n * D;
-    for (int i = threadIdx.x; i < a.n; i += blockDim.x) {
-        float s = 0.f;
-        for (int d = 0; d < D; ++d) { const float f = a.scale * __half2float(Qb[(size_t)i * D + d]); s = fmaf(f, f, s); }
-        a.qnorm2[(size_t)bh * a.n + i] = s;
-    }
+// the columns of an accumulator from `at` on, for the thread's token
+__device__ __forceinline__ void load_acc(uint32_t at, float (&x)[32]) {
+    asm volatile(
+        "tcgen05.ld.sync.aligned.32x32b.x32.b32 {%0,%1,%2,%3,%4,%5,%6,%7,%8,%9,%10,%11,%12,%13,%14,%15,"
+        "%16,%17,%18,%19,%20,%21,%22,%23,%24,%25,%26,%27,%28,%29,%30,%31}, [%32];\n"
+        "tcgen05.wait::ld.sync.aligned;"
+        : "=f"(x[0]), "=f"(x[1]), "=f"(x[2]), "=f"(x[3]), "=f"(x[4]), "=f"(x[5]), "=f"(x[6]), "=f"(x[7]), "=f"(x[8]), "=f"(x[9]), "=f"(x[10]),
+          "=f"(x[11]), "=f"(x[12]), "=f"(x[13]), "=f"(x[14]), "=f"(x[15]), "=f"(x[16]), "=f"(x[17]), "=f"(x[18]), "=f"(x[19]), "=f"(x[20]),
+          "=f"(x[21]), "=f"(x[22]), "=f"(x[23]), "=f"(x[24]), "=f"(x[25]), "=f"(x[26]), "=f"(x[27]), "=f"(x[28]), "=f"(x[29]), "=f"(x[30]), "=f"(x[31])
+        : "r"(at)
+        : "memory");
 }
+__device__ __forceinline__ void load_acc(uint32_t at, float (&x)[16]) {
+    asm volatile(
+        "tcgen05.ld.sync.aligned.32x32b.x16.b32 {%0,%1,%2,%3,%4,%5,%6,%7,%8,%9,%10,%11,%12,%13,%14,%15}, [%16];\n"
+        "tcgen05.wait::ld.sync.aligned;"
+        : "=f"(x[0]), "=f"(x[1]), "=f"(x[2]), "=f"(x[3]), "=f"(x[4]), "=f"(x[5]), "=f"(x[6]), "=f"(x[7]), "=f"(x[8]), "=f"(x[9]), "=f"(x[10]),
+          "=f"(x[11]), "=f"(x[12]), "=f"(x[13]), "=f"(x[14]), "=f"(x[15])
+        : "r"(at)
+        : "memory");
+}
+__device__ __forceinline__ void tmem_before_sync() { asm volatile("tcgen05.fence::before_thread_sync;" ::: "memory"); }
+__device__ __forceinline__ void tmem_after_sync() { asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory"); }
+__device__ __forceinline__ void cluster_barrier() {
+    asm volatile("barrier.cluster.arrive.release.aligned;\nbarrier.cluster.wait.acquire.aligned;" ::: "memory");
+}
+template <int THREADS>
+__device__ __forceinline__ void team_sync(int team) { asm volatile("bar.sync %0, %1;" ::"r"(1 + team), "n"(THREADS) : "memory"); }
 
-__device__ __forceinline__ void fold_stats(float2& to, const float2& p) {          // (max, sum of exponentials)
+__device__ __forceinline__ float pow2(float x) {
+    float r;
+    asm("ex2.approx.ftz.f32 %0, %1;" : "=f"(r) : "f"(x));
+    return r;
+}
+// (reference, sum of 2^(logit - reference))
+__device__ __forceinline__ void fold_stats(float2& to, const float2& p) {
     const float NEG = __int_as_float(0xff800000), m = fmaxf(to.x, p.x);
-    to.y = (to.x == NEG ? 0.f : to.y * __expf(to.x - m)) + (p.x == NEG ? 0.f : p.y * __expf(p.x - m));
+    to.y = (to.x == NEG ? 0.f : to.y * pow2(to.x - m)) + (p.x == NEG ? 0.f : p.y * pow2(p.x - m));
     to.x = m;
 }
+// Sums of eight columns over the lanes of the warp: lane 4k (and the three behind it) gets that of column k.
+__device__ __forceinline__ float sum8(const float (&v)[8], int lane) {
+    float a[4];
+#pragma unroll
+    for (int k = 0; k < 4; ++k) a[k] = ((lane & 16) ? v[k + 4] : v[k]) + __shfl_xor_sync(0xFFFFFFFFu, (lane & 16) ? v[k] : v[k + 4], 16);
+    float b[2];
+#pragma unroll
+    for (int k = 0; k < 2; ++k) b[k] = ((lane & 8) ? a[k + 2] : a[k]) + __shfl_xor_sync(0xFFFFFFFFu, (lane & 8) ? a[k] : a[k + 2], 8);
+    float c = ((lane & 4) ? b[1] : b[0]) + __shfl_xor_sync(0xFFFFFFFFu, (lane & 4) ? b[0] : b[1], 4);
+    c += __shfl_xor_sync(0xFFFFFFFFu, c, 2);
+    return c + __shfl_xor_sync(0xFFFFFFFFu, c, 1);
+}
 
-// Sequences of more than a cluster of CTAs.  What bounds it is memory: the keys are read twice and the rows written once.
-// (Logits written by the first pass and normalised in place by a second kernel - the keys read once, the rows written
-// twice and read once - took 374 + 217 us for 160 (b,h) x 8192 tokens and 64 rows.)  A warp takes 16 tokens per
-// step; column g of its two 8-token operands is token 4 (g / 2) + (g mod 2) resp. that + 2, so that a lane ends up with
-// four consecutive tokens of a row.  STATS: the first pass.
-template <int D, bool STATS>
-__global__ void __launch_bounds__(PW_WARPS * 32, 3) window_long_kernel(const PrefillArgs a) {
-    constexpr int WPL = D / 8;          // 32-bit words per lane and token
-    constexpr int KS = D / 16;          // k-steps
-    extern __shared__ __align__(16) float s_dyn[];
-    uint4* s_q = reinterpret_cast<uint4*>(s_dyn);
-    __shared__ float2 s_part[PW_WARPS][PW_MAXQ];             // STATS: per warp; else entry 0: what the rows are normalised with
-    qaq_dependency();
-    const int bh = blockIdx.y, chunk = blockIdx.x;
-    const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
-    const int g = lane >> 2, c = lane & 3;
+template <int D>
+__device__ __forceinline__ void query_norm(const PrefillArgs& a, int bh, int i) {
+    const __half* q = a.Q + ((size_t)bh * a.n + i) * D;
+    float s = 0.f;
+    for (int d = 0; d < D; ++d) { const float f = a.scale * __half2float(q[d]); s = fmaf(f, f, s); }
+    a.qnorm2[(size_t)bh * a.n + i] = s;
+}
+
+// One CTA per SM, which goes through its share of the work: a warp asks for the keys (tiles of 128 tokens, a ring of stages), a
+// warp multiplies them, sixteen look at the accumulators.  Row t of an accumulator is a token, a thread's; column i a query.
+// The reference of a row is a warp's largest logit of its first tile; it is raised where a later logit exceeds it by 2^64.
+// A wait that runs out of tries (a copy or a peer that never came) ends the waiting: the rows are then not numbers.
+// Where the accumulators of two (b,h) have room (up to 32 rows) half of the sixteen warps take the statistics of the next one while
+// the others write the rows of the last (256 (b,h) of 4096 tokens, 32 rows: 70 us, 82 with all of them at one job after the other, 78
+// with eight warps); with 64 rows the tensor memory is full and the halves wait for each other (160 of 8192: 222 us, 152 together).
+template <int D, int NC, int MODE>
+__global__ void __launch_bounds__(PW_THREADS, 1) window_kernel(const __grid_constant__ CUtensorMap keys, const __grid_constant__ CUtensorMap queries, const PrefillArgs a) {
+    using W = Window<D, NC, MODE>;
+    constexpr int STAGES = W::STAGES, SLOTS = W::SLOTS;
     const float NEG = __int_as_float(0xff800000);
-    const __half* Kb = a.K + (size_t)(bh / a.H) * a.sb + (size_t)(bh % a.H) * a.sh;
-    const int t_warp = chunk * PW_CHUNK + warp * (PW_CHUNK / PW_WARPS);
-    // this warp's keys are on their way to L2 while the queries are laid out
-    constexpr int LPT = D >= 64 ? D / 64 : 1;                                    // 128-byte lines per token
-    for (int ln = lane; ln < (PW_CHUNK / PW_WARPS) * LPT; ln += 32) {
-        const int t = t_warp + ln / LPT;
-        if (t < a.T) asm volatile("prefetch.global.L2 [%0];" ::"l"(Kb + (size_t)t * a.st + (ln % LPT) * 64));
+    extern __shared__ unsigned char s_dyn[];
+    const uint32_t base = (smem_addr(s_dyn) + 1023u) & ~1023u, s_q = base + STAGES * W::TILE_BYTES;
+    typename W::Shared& sm = *reinterpret_cast<typename W::Shared*>(s_dyn + (s_q + 2 * W::QUERY_BYTES - smem_addr(s_dyn)));
+    const uint32_t full = smem_addr(sm.full), empty = smem_addr(sm.empty), there = smem_addr(sm.there), taken = smem_addr(sm.taken), q_free = smem_addr(sm.q_free), stats = smem_addr(sm.stats), used = smem_addr(sm.used);
+    const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
+    // items: (b,h), or chunks of them; of an item the CTA has the tiles from tile0(item) on
+    const int ncta = MODE == ONE_PASS ? (a.tiles ? ((a.T + PW_TILE - 1) / PW_TILE + a.tiles - 1) / a.tiles : 1) : 1;
+    const int rank = MODE == ONE_PASS ? blockIdx.x % ncta : 0, step = gridDim.x / ncta, items = MODE == ONE_PASS ? a.BH : a.BH * a.nchunk;
+    const int all_tiles = (a.T + PW_TILE - 1) / PW_TILE;
+    struct Item { int bh, chunk, tile, n; };
+    auto item_of = [&](int i) {
+        Item o;
+        if (MODE == ROWS) i = items - 1 - i;                 // backwards: the keys the first pass has read last are still in L2
+        o.bh = MODE == ONE_PASS ? i : i / a.nchunk;
+        o.chunk = MODE == ONE_PASS ? rank : i - o.bh * a.nchunk;
+        o.tile = o.chunk * a.tiles;
+        o.n = min(a.tiles, all_tiles - o.tile);
+        return o;
+    };
+    if (tid == 0) {
+        for (int i = 0; i < STAGES; ++i) { bar_init(full + 8 * i, 1); bar_init(empty + 8 * i, 1); }
+        for (int i = 0; i < SLOTS; ++i) { bar_init(there + 8 * i, 1); bar_init(taken + 8 * i, 4 * W::PARTS); }
+        for (int i = 0; i < 2; ++i) { bar_init(q_free + 8 * i, 1); bar_init(stats + 8 * i, 1); bar_init(used + 8 * i, ncta); }
+        asm volatile("fence.mbarrier_init.release.cluster;\nfence.proxy.async.shared::cta;" ::: "memory");
     }
-    if (STATS && a.qnorm2 && chunk == 0) query_norms<D>(a, bh);
-    lay_out_queries<D>(s_q, a.Q + (size_t)bh * a.n * D, a.n);
-    if (!STATS) {      // merged statistics of the rows: four threads per row
-        const int i = threadIdx.x >> 2, part = threadIdx.x & 3;
-        float2 st = make_float2(NEG, 0.f);
-        if (i < a.n)
-            for (int ch = part; ch < a.nchunk; ch += 4) fold_stats(st, a.part[((size_t)bh * a.nchunk + ch) * a.n + i]);
+    qaq_dependency();
+    if (warp == 1)
+        asm volatile("tcgen05.alloc.cta_group::1.sync.aligned.shared::cta.b32 [%0], 512;\ntcgen05.relinquish_alloc_permit.cta_group::1.sync.aligned;" ::"r"(smem_addr(&sm.tmem)) : "memory");
+    tmem_before_sync();
+    if (MODE == ONE_PASS) cluster_barrier(); else __syncthreads();
+    tmem_after_sync();
+    const uint32_t acc = *(volatile uint32_t*)&sm.tmem;
+    bool ok = true;
+    if (warp == 0) {
+        if (lane == 0) {
+            uint32_t g = 0;
+            int it = 0;
+            for (int i = blockIdx.x / ncta; i < items && ok; i += step, ++it) {
+                const Item o = item_of(i);
+                ok = bar_wait(q_free + 8 * (it & 1), ((uint32_t)(it >> 1) & 1u) ^ 1u);
+                for (int k = 0; k < o.n && ok; ++k, ++g) {
+                    const uint32_t st = g % STAGES, bar = full + 8 * st;
+                    ok = bar_wait(empty + 8 * st, ((g / STAGES) & 1u) ^ 1u);
+                    if (!ok) break;
+                    bar_expect(bar, W::TILE_BYTES + (k == 0 ? W::QUERY_BYTES : 0u));
 #pragma unroll
-        for (int o = 1; o < 4; o <<= 1) fold_stats(st, make_float2(__shfl_xor_sync(0xFFFFFFFFu, st.x, o), __shfl_xor_sync(0xFFFFFFFFu, st.y, o)));
-        if (i < a.n && part == 0) s_part[0][i] = make_float2(st.x, st.y > 0.f ? 1.0f / st.y : 0.f);
-        for (int k = threadIdx.x; k < PW_CHUNK; k += blockDim.x) {
-            const int t = chunk * PW_CHUNK + k;
-            if (t < a.T) a.nvalid[(size_t)bh * a.T + t] = (uint8_t)min(a.n, a.T - t);
-        }
-    }
-    __syncthreads();
-    const bool vec_ok = (a.T & 3) == 0 && ((uintptr_t)a.ring & 15) == 0;      // rows start 16-byte aligned, no ragged end
-
-    {
-        constexpr int MT = PW_MAXQ / 16;                // 16-row tiles of queries: a warp's keys are read once for all of them
-        float2 st[MT][2];               // rows g, g + 8 of the tiles over the tokens this lane sees
-#pragma unroll
-        for (int mt = 0; mt < MT; ++mt) st[mt][0] = st[mt][1] = make_float2(NEG, 0.f);
-#pragma unroll 1
-        for (int step = 0; step < PW_CHUNK / PW_WARPS / 16; ++step) {
-            const int t0 = t_warp + 16 * step;
-            if (t0 >= a.T) break;
-            uint32_t bw[2][WPL];
-#pragma unroll
-            for (int h = 0; h < 2; ++h) {
-                const int t = t0 + 4 * (g >> 1) + (g & 1) + 2 * h;
-                const uint4* src = reinterpret_cast<const uint4*>(Kb + (size_t)(t < a.T ? t : 0) * a.st) + c;
-#pragma unroll
-                for (int i = 0; i < WPL / 4; ++i) {
-                    uint4 v = make_uint4(0, 0, 0, 0);
-                    if (t < a.T) v = src[4 * i];
-                    bw[h][4 * i] = v.x; bw[h][4 * i + 1] = v.y; bw[h][4 * i + 2] = v.z; bw[h][4 * i + 3] = v.w;
-                }
-            }
-#pragma unroll
-            for (int mt = 0; mt < MT; ++mt) {
-                if (mt * 16 >= a.n) break;
-                float acc[2][4];
-#pragma unroll
-                for (int i = 0; i < 4; ++i) { acc[0][i] = 0.f; acc[1][i] = 0.f; }
-#pragma unroll
-                for (int ks = 0; ks < KS; ++ks) {
-                    const uint4 f = s_q[(mt * KS + ks) * 32 + lane];
-                    const uint32_t fr[4] = {f.x, f.y, f.z, f.w};
-                    mma_16816(acc[0], fr, bw[0][2 * ks], bw[0][2 * ks + 1]);
-                    mma_16816(acc[1], fr, bw[1][2 * ks], bw[1][2 * ks + 1]);
-                }
-                // acc[h][2 hr], acc[h][2 hr + 1]: row g + 8 hr, tokens t0 + 4c + 2h, + 1
-#pragma unroll
-                for (int hr = 0; hr < 2; ++hr) {
-                    const int i = mt * 16 + g + 8 * hr;          // query
-                    if (i >= a.n) continue;
-                    const int t = t0 + 4 * c, left = a.T - a.n + i - t + 1; // how many of the lane's tokens the query sees (or more)
-                    const float l[4] = {a.scale * acc[0][2 * hr], a.scale * acc[0][2 * hr + 1], a.scale * acc[1][2 * hr], a.scale * acc[1][2 * hr + 1]};
-                    if (STATS) {
-                        float m = NEG;
-#pragma unroll
-                        for (int e = 0; e < 4; ++e) if (e < left) m = fmaxf(m, l[e]);
-                        float sum = 0.f;
-#pragma unroll
-                        for (int e = 0; e < 4; ++e) if (e < left) sum += __expf(l[e] - m);
-                        fold_stats(st[mt][hr], make_float2(m, sum));
-                    } else {
-                        const float2 mi = s_part[0][i];
-                        float4 o;
-                        o.x = left > 0 ? __expf(l[0] - mi.x) * mi.y : 0.f;
-                        o.y = left > 1 ? __expf(l[1] - mi.x) * mi.y : 0.f;
-                        o.z = left > 2 ? __expf(l[2] - mi.x) * mi.y : 0.f;
-                        o.w = left > 3 ? __expf(l[3] - mi.x) * mi.y : 0.f;
-                        float* row = a.ring + ((size_t)bh * a.n + (a.n - 1 - i)) * a.T + t;
-                        if (vec_ok) { if (t < a.T) *reinterpret_cast<float4*>(row) = o; }
-                        else {
-                            if (t < a.T) row[0] = o.x;
-                            if (t + 1 < a.T) row[1] = o.y;
-                            if (t + 2 < a.T) row[2] = o.z;
-                            if (t + 3 < a.T) row[3] = o.w;
-                        }
+                    for (int r = 0; r < W::REGIONS; ++r) {
+                        if (k == 0) bulk_rows(s_q + (it & 1) * W::QUERY_BYTES + r * (NC * W::ROW_BYTES), &queries, 64 * r, o.bh * a.n, bar);
+                        bulk_tile(base + st * W::TILE_BYTES + r * (PW_TILE * W::ROW_BYTES), &keys, 64 * r, (o.tile + k) * PW_TILE, o.bh % a.H, o.bh / a.H, bar);
                     }
                 }
             }
+            if (!ok)                   // what is on its way arrives before the CTA leaves
+                for (uint32_t j = g > STAGES ? g - STAGES : 0; j < g; ++j) bar_wait(full + 8 * (j % STAGES), (j / STAGES) & 1u);
         }
-        if (STATS) {      // merge the four lanes of a row
-#pragma unroll
-            for (int mt = 0; mt < MT; ++mt)
-#pragma unroll
-                for (int hr = 0; hr < 2; ++hr) {
-                    float2 v = st[mt][hr];
-                    fold_stats(v, make_float2(__shfl_xor_sync(0xFFFFFFFFu, v.x, 1), __shfl_xor_sync(0xFFFFFFFFu, v.y, 1)));
-                    fold_stats(v, make_float2(__shfl_xor_sync(0xFFFFFFFFu, v.x, 2), __shfl_xor_sync(0xFFFFFFFFu, v.y, 2)));
-                    if (c == 0) s_part[warp][mt * 16 + g + 8 * hr] = v;
+    } else if (warp == 1) {
+        if (lane == 0) {
+            uint32_t g = 0;
+            int it = 0;
+            for (int i = blockIdx.x / ncta; i < items && ok; i += step, ++it) {
+                const Item o = item_of(i);
+                for (int k = 0; k < o.n && ok; ++k, ++g) {
+                    const uint32_t st = g % STAGES, slot = g % SLOTS;
+                    ok = bar_wait(full + 8 * st, (g / STAGES) & 1u) && bar_wait(taken + 8 * slot, ((g / SLOTS) & 1u) ^ 1u);
+                    if (!ok) break;
+                    tmem_after_sync();
+                    multiply<D, NC>(acc + slot * NC, base + st * W::TILE_BYTES, s_q + (it & 1) * W::QUERY_BYTES);
+                    tensor_done(empty + 8 * st);
+                    tensor_done(there + 8 * slot);
                 }
+                tensor_done(q_free + 8 * (it & 1));
+            }
         }
-    }
-    if (STATS) {          // then the warps
-        __syncthreads();
-        if ((int)threadIdx.x < a.n) {
-            float2 v = make_float2(NEG, 0.f);
+    } else {
+        constexpr int CW = W::CW, GROUPS = W::GROUPS, TEAM = W::TEAM;
+        // a warp reads the lanes of its quarter of a tile, columns h to h + CW - 1
+        const int team = (warp - 2) / TEAM, w = (warp - 2) % TEAM, e = 32 * w + lane, quarter = warp & 3, group = (w >> 2) / W::PARTS, h = (w >> 2) % W::PARTS * CW;
+        const float sc = a.scale * 1.4426950408889634f;
+        const uint32_t lanes = acc + ((uint32_t)(32 * quarter) << 16) + h;
+        auto logits = [&](uint32_t slot, float (&x)[CW]) {
+            load_acc(lanes + slot * NC, x);
+            if (!ok)
 #pragma unroll
-            for (int w = 0; w < PW_WARPS; ++w) fold_stats(v, s_part[w][threadIdx.x]);
-            a.part[((size_t)bh * a.nchunk + chunk) * a.n + threadIdx.x] = v;
+                for (int c = 0; c < CW; ++c) x[c] = __int_as_float(0x7fffffff);
+        };
+        auto wait_for = [&](uint32_t g) {
+            ok = __all_sync(0xFFFFFFFFu, ok && bar_wait(there + 8 * (g % SLOTS), (g / SLOTS) & 1u));
+            tmem_after_sync();
+        };
+        auto release = [&](uint32_t g) {
+            tmem_before_sync();
+            __syncwarp();
+            if (lane == 0) bar_arrive(taken + 8 * (g % SLOTS));
+        };
+        uint32_t g0 = 0;
+        int it = 0, bh_was = -1, buf = 0;
+        for (int i = blockIdx.x / ncta; i < items; i += step, ++it) {
+            const Item o = item_of(i);
+            const int t0 = o.tile * PW_TILE + 32 * quarter + lane;          // the thread's token of the first tile
+            // ---- statistics of the rows.  Query i sees token t if t <= T - n + i, that is from column t - (T - n) on.
+            if (MODE != ROWS && (!W::SPLIT || team == 0)) {
+                float sum[CW];
+#pragma unroll
+                for (int c = 0; c < CW; ++c) sum[c] = 0.f;
+                float* const ref = sm.ref[it & 1][w];
+#pragma unroll 1
+                for (int k = group; k < o.n; k += GROUPS) {
+                    const uint32_t g = g0 + k;
+                    wait_for(g);
+                    const int hidden = t0 + k * PW_TILE - (a.T - a.n) - h;
+                    const bool part_hidden = hidden - lane + 31 > 0;
+                    float x[CW];
+                    logits(g % SLOTS, x);
+                    if (MODE == STATS) release(g);
+                    if (k == group) {
+#pragma unroll
+                        for (int c = 0; c < CW; c += 4) {
+                            float m[4];
+#pragma unroll
+                            for (int j = 0; j < 4; ++j) { m[j] = warp_max(c + j < hidden ? NEG : x[c + j] * sc); m[j] = m[j] == NEG ? 0.f : m[j]; }
+                            if (lane == 0) *reinterpret_cast<float4*>(ref + c) = make_float4(m[0], m[1], m[2], m[3]);
+                        }
+                        __syncwarp();
+                    }
+#pragma unroll
+                    for (int c = 0; c < CW; c += 4) {
+                        const float4 r = *reinterpret_cast<const float4*>(ref + c);
+                        x[c] = fmaf(x[c], sc, -r.x); x[c + 1] = fmaf(x[c + 1], sc, -r.y); x[c + 2] = fmaf(x[c + 2], sc, -r.z); x[c + 3] = fmaf(x[c + 3], sc, -r.w);
+                    }
+                    if (part_hidden)
+#pragma unroll
+                        for (int c = 0; c < CW; ++c) if (c < hidden) x[c] = NEG;
+                    float top = NEG;
+#pragma unroll
+                    for (int c = 0; c < CW; c += 2) top = fmaxf(top, fmaxf(x[c], x[c + 1]));
+                    if (__any_sync(0xFFFFFFFFu, top > 64.0f)) {
+                        __syncwarp();
+#pragma unroll
+                        for (int c = 0; c < CW; ++c) {
+                            const float up = fmaxf(warp_max(x[c]), 0.f);
+                            if (up > 0.f) { x[c] -= up; sum[c] *= pow2(-up); }
+                            if (lane == 0) ref[c] += up;
+                        }
+                        __syncwarp();
+                    }
+#pragma unroll
+                    for (int c = 0; c < CW; ++c) sum[c] += pow2(x[c]);
+                }
+                __syncwarp();
+#pragma unroll
+                for (int c0 = 0; c0 < CW; c0 += 8) {
+                    float v[8];
+#pragma unroll
+                    for (int c = 0; c < 8; ++c) v[c] = sum[c0 + c];
+                    const float s = sum8(v, lane);
+                    if ((lane & 3) == 0) sm.sum[it & 1][w][c0 + (lane >> 2)] = s;
+                }
+                if (group >= o.n && lane < CW) { ref[lane] = NEG; sm.sum[it & 1][w][lane] = 0.f; }      // no tile for the group
+                team_sync<32 * TEAM>(0);
+                const int c = e % NC;
+                float2 st = make_float2(NEG, 0.f);
+                if (c < a.n)
+#pragma unroll
+                    for (int j = 0; j < 4 * GROUPS; ++j) {
+                        const int from = ((j >> 2) * W::PARTS + c / CW) * 4 + (j & 3);
+                        if (!(sm.sum[it & 1][from][c % CW] == 0.f)) fold_stats(st, make_float2(sm.ref[it & 1][from][c % CW], sm.sum[it & 1][from][c % CW]));
+                    }
+                if (MODE == STATS) {
+                    if (e < a.n) a.part[((size_t)o.bh * a.nchunk + o.chunk) * a.n + e] = st;
+                } else {
+                    // every CTA of the (b,h) gets the statistics of all of them, as soon as all have used those of two items before.
+                    // (A launch without clusters knows no asynchronous stores to a CTA of the cluster, its own included.)
+                    const uint32_t bar = stats + 8 * (it & 1);
+                    // Only warps that send wait: one that does not could come so late that the phase is over, and the one after.
+                    if ((e & ~31) < ncta * NC) ok = __all_sync(0xFFFFFFFFu, ok && bar_wait_cluster(used + 8 * (it & 1), ((uint32_t)(it >> 1) & 1u) ^ 1u));
+                    if (ncta == 1) {
+                        if (e < a.n) sm.all[it & 1][0][e] = st;
+                        team_sync<32 * TEAM>(0);
+                        if (e == 0) bar_arrive(bar);
+                    } else {
+                    if (e == 0) bar_expect(bar, (uint32_t)(ncta * a.n) * 8u);
+                    if (c < a.n)
+                        for (int r = e / NC; r < ncta; r += 32 * TEAM / NC)
+                            asm volatile("{\n.reg .u32 p, m;\nmapa.shared::cluster.u32 p, %0, %2;\nmapa.shared::cluster.u32 m, %1, %2;\n"
+                                         "st.async.shared::cluster.mbarrier::complete_tx::bytes.v2.f32 [p], {%3, %4}, [m];\n}"
+                                         ::"r"(smem_addr(&sm.all[it & 1][rank][c])), "r"(bar), "r"(r), "f"(st.x), "f"(st.y) : "memory");
+                    }
+                }
+                if (a.qnorm2 && o.chunk == 0 && e < a.n) query_norm<D>(a, o.bh, e);
+            }
+            // ---- normalised rows, newest first, written once; rows-per-token counts
+            if (MODE != STATS && (!W::SPLIT || team == 1)) {
+                if constexpr (MODE == ONE_PASS) {
+                    buf = it & 1;
+                    ok = __all_sync(0xFFFFFFFFu, ok && bar_wait_cluster(stats + 8 * buf, (uint32_t)(it >> 1) & 1u));
+                    if (e < a.n) {
+                        float2 st = make_float2(NEG, 0.f);
+                        for (int r = 0; r < ncta; ++r) fold_stats(st, sm.all[buf][r][e]);
+                        sm.row[buf][e] = make_float2(st.x, st.y > 0.f ? 1.0f / st.y : 0.f);
+                    }
+                    team_sync<32 * TEAM>(1);
+                    if (ncta == 1) {
+                        if (e == 0) bar_arrive(used + 8 * buf);
+                    } else if (e < ncta)
+                        asm volatile("{\n.reg .u32 m;\nmapa.shared::cluster.u32 m, %0, %1;\nmbarrier.arrive.release.cluster.shared::cluster.b64 _, [m];\n}" ::"r"(used + 8 * buf), "r"(e) : "memory");
+                } else if (o.bh != bh_was) {           // merged statistics of the chunks
+                    bh_was = o.bh;
+                    buf ^= 1;
+                    constexpr int EACH = 8;
+                    float2 st = make_float2(NEG, 0.f);
+                    static_assert(EACH <= PW_CLUSTER && EACH * NC <= 32 * TEAM, "parts");
+                    if (e < EACH * NC) {
+                        if (e % NC < a.n)
+                            for (int ch = e / NC; ch < a.nchunk; ch += EACH) fold_stats(st, a.part[((size_t)o.bh * a.nchunk + ch) * a.n + e % NC]);
+                        sm.all[buf][e / NC][e % NC] = st;
+                    }
+                    team_sync<32 * TEAM>(1);
+                    if (e < a.n) {
+                        for (int j = 1; j < EACH; ++j) fold_stats(st, sm.all[buf][j][e]);
+                        sm.row[buf][e] = make_float2(st.x, st.y > 0.f ? 1.0f / st.y : 0.f);
+                    }
+                    team_sync<32 * TEAM>(1);
+                }
+                float* row0 = a.ring + ((size_t)o.bh * a.n + (a.n - 1 - h)) * a.T + t0;
+#pragma unroll 1
+                for (int k = group; k < o.n; k += GROUPS) {
+                    const uint32_t g = g0 + k;
+                    wait_for(g);
+                    const int t = t0 + k * PW_TILE, hidden = t - (a.T - a.n) - h;
+                    const bool part_hidden = hidden - lane + 31 > 0;
+                    float* row = row0 + k * PW_TILE;
+                    float x[CW];
+                    logits(g % SLOTS, x);
+                    release(g);
+#pragma unroll
+                    for (int c = 0; c < CW; c += 2) {
+                        const float4 r = *reinterpret_cast<const float4*>(&sm.row[buf][h + c]);
+                        x[c] = pow2(fmaf(x[c], sc, -r.x)) * r.y;
+                        x[c + 1] = pow2(fmaf(x[c + 1], sc, -r.z)) * r.w;
+                    }
+                    if (part_hidden)
+#pragma unroll
+                        for (int c = 0; c < CW; ++c) x[c] = c < hidden ? 0.f : x[c];
+                    if (t < a.T) {
+                        if (a.n - h >= CW) {
+#pragma unroll
+                            for (int c = 0; c < CW; ++c) { *row = x[c]; row -= a.T; }
+                        } else {
+#pragma unroll
+                            for (int c = 0; c < CW; ++c) { if (h + c < a.n) *row = x[c]; row -= a.T; }
+                        }
+                        if (h == 0) a.nvalid[(size_t)o.bh * a.T + t] = (uint8_t)min(a.n, a.T - t);
+                    }
+                }
+            }
+            g0 += o.n;
         }
     }
+    __syncwarp();
+    tmem_before_sync();
+    if (MODE == ONE_PASS) cluster_barrier(); else __syncthreads();       // nobody leaves while somebody may write to its shared memory
+    if (warp == 1) { tmem_after_sync(); asm volatile("tcgen05.dealloc.cta_group::1.sync.aligned.b32 %0, 512;" ::"r"(acc) : "memory"); }
 }
 
-// ---- one pass: the CTAs of one (b,h) form a thread-block cluster.  Each keeps the logits of its 512 tokens in
-// shared memory, the per-row (max, sum) of the CTAs are exchanged through distributed shared memory, and the
-// normalised rows are written once: K is read once and the ring written once (no logits in global memory, no
-// workspace).  Used while a (b,h) fits a portable cluster (up to 8 x 512 tokens); longer sequences take the two
-// kernels above.
-constexpr int PC_WARPS = 16;            // 32 tokens per warp
-constexpr int PC_MINCTA = 2;            // two CTAs per SM (64 registers per thread)
-constexpr int PC_CHUNK = 512;           // tokens per CTA
-constexpr int PC_MAXCTA = 8;            // portable cluster size
-constexpr int PC_PITCH = PC_CHUNK + 8;  // row pitch of the logits tile in floats (spreads the rows of a fragment over the banks)
-
-template <int D>
-__global__ void __launch_bounds__(PC_WARPS * 32, PC_MINCTA) window_cluster_kernel(const PrefillArgs a) {
-    namespace cg = cooperative_groups;
-    cg::cluster_group cluster = cg::this_cluster();
-    constexpr int WPL = D / 8;
-    constexpr int KS = D / 16;
-    extern __shared__ __align__(16) float s_l[];            // [n][PC_PITCH] logits of this CTA's tokens, then the queries
-    // the queries as A-operand fragments, one uint4 per (16-row tile, k step, lane): every warp reads the same ones
-    uint4* s_q = reinterpret_cast<uint4*>(s_l + (size_t)a.n * PC_PITCH);
-    __shared__ float s_part[PC_WARPS][32];                   // per warp: maximum of every row of the current 32 over its tokens
-    __shared__ float s_mcta[PW_MAXQ];                        // maximum of every row over this CTA's tokens
-    __shared__ float2 s_all[PC_MAXCTA][PW_MAXQ];             // (max, sum of exponentials) of every row over the tokens of every CTA
-                                                             // of the cluster: each CTA writes its entries into all the copies
-    __shared__ float s_inv[PW_MAXQ];
-    qaq_dependency();
-    const int bh = blockIdx.y, chunk = blockIdx.x;
-    const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
-    const int g = lane >> 2, c = lane & 3;
-    const int b_idx = bh / a.H, h_idx = bh % a.H;
-    const __half* Kb = a.K + (size_t)b_idx * a.sb + (size_t)h_idx * a.sh;
-    const __half* Qb = a.Q + (size_t)bh * a.n * D;
-    const float NEG = __int_as_float(0xff800000);
-
-    if (a.qnorm2 && chunk == 0) query_norms<D>(a, bh);
-    const int t_cta = chunk * PC_CHUNK;
-    const int t_warp = t_cta + warp * (PC_CHUNK / PC_WARPS);
-    // this warp's keys are on their way to L2 while the queries are laid out
-    constexpr int LPT = D >= 64 ? D / 64 : 1;                                    // 128-byte lines per token
-    for (int ln = lane; ln < (PC_CHUNK / PC_WARPS) * LPT; ln += 32) {
-        const int t = t_warp + ln / LPT;
-        if (t < a.T) asm volatile("prefetch.global.L2 [%0];" ::"l"(Kb + (size_t)t * a.st + (ln % LPT) * 64));
+// ---- few tiles in all: a thread keeps the logits of its token in registers, a CTA is one tile to four (four warps each), and the CTAs
+// of a (b,h) form a cluster where it has more than one.  No warp waits for another's work but at barriers, several CTAs share an
+// SM, keys come by plain asynchronous copies.  Tensor memory is given back before the CTAs of a cluster wait for each other, so that
+// nobody waits for it who is waited for.  32 (b,h) of 333 tokens, 32 rows: 5.4 us, the kernel above 7.8 us.
+constexpr int PS_TILES = 4;            // tiles of a CTA at most
+template <int ROW_BYTES, int ROWS>     // rows of a [.][D] operand on their way to shared memory, by four warps; what lies beyond `rows` is not touched
+__device__ __forceinline__ void fetch_rows(uint32_t dst, const __half* src, long stride, int rows, int D, int thread) {
+    const int PR = D / 8, row = thread / PR, c = thread % PR, step = 128 / PR;           // 16-byte pieces of a row; rows at a time, a multiple of 8
+    constexpr int IN = ROW_BYTES / 16;
+    dst += (c / IN) * (ROWS * ROW_BYTES) + row * ROW_BYTES + (((c % IN) ^ (ROW_BYTES == 128 ? row & 7 : (row >> 1) & 3)) << 4);
+    src += (ptrdiff_t)row * stride + 8 * c;
+#pragma unroll 16
+    for (int r = row; r < ROWS; r += step, src += step * stride, dst += step * ROW_BYTES)
+        if (r < rows) asm volatile("cp.async.cg.shared.global [%0], [%1], 16;" ::"r"(dst), "l"(src) : "memory");
+}
+template <int D, int NC>
+__global__ void __launch_bounds__(128 * PS_TILES, 1) window_short_kernel(const PrefillArgs a, const __half* K, long sb, long sh, long st) {
+    using W = Window<D, NC, STATS>;
+    constexpr int RB = W::ROW_BYTES, CW = NC < 32 ? NC : 32;
+    const float NEG = __int_as_float(0xff800000), sc = a.scale * 1.4426950408889634f;
+    extern __shared__ unsigned char s_dyn[];
+    __shared__ alignas(8) unsigned long long s_bar[PS_TILES];
+    __shared__ uint32_t s_tmem;
+    __shared__ alignas(16) float s_max[4 * PS_TILES][NC], s_sum[4 * PS_TILES][NC];       // of a warp: reference and sum of every row over its tokens
+    __shared__ float2 s_all[PW_CLUSTER][NC];                 // the same of every CTA of the cluster, which all write here
+    const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31, group = warp >> 2, groups = blockDim.x >> 7, warps = 4 * groups;
+    const int bh = blockIdx.y, rank = blockIdx.x, ncta = gridDim.x;
+    const uint32_t base = (smem_addr(s_dyn) + 1023u) & ~1023u, queries = base + groups * W::TILE_BYTES, bar = smem_addr(s_bar) + 8 * group;
+    const uint32_t columns = max(32, 1 << (32 - __clz(groups * NC - 1)));                // (a power of two)
+    if (tid == 0) {
+        for (int i = 0; i < PS_TILES; ++i) bar_init(smem_addr(s_bar) + 8 * i, 1);
+        asm volatile("fence.proxy.async.shared::cta;" ::: "memory");
     }
+    qaq_dependency();
     // first half of a cluster barrier: by the time the row statistics are exchanged every CTA of the cluster is known
     // to be running (its shared memory may be written)
-    asm volatile("barrier.cluster.arrive.release.aligned;" ::: "memory");
-
-    lay_out_queries<D>(s_q, Qb, a.n);
+    if (ncta > 1) asm volatile("barrier.cluster.arrive.release.aligned;" ::: "memory");
+    const int t_group = (rank * groups + group) * PW_TILE;
+    fetch_rows<RB, PW_TILE>(base + group * W::TILE_BYTES, K + (size_t)(bh / a.H) * sb + (size_t)(bh % a.H) * sh + (ptrdiff_t)t_group * st, st, a.T - t_group, D, tid & 127);
+    if (group == 0) fetch_rows<RB, NC>(queries, a.Q + (size_t)bh * a.n * D, D, a.n, D, tid);      // (columns of rows that are not there are not looked at)
+    asm volatile("cp.async.commit_group;" ::: "memory");
+    if (warp == 0)
+        asm volatile("tcgen05.alloc.cta_group::1.sync.aligned.shared::cta.b32 [%0], %1;\ntcgen05.relinquish_alloc_permit.cta_group::1.sync.aligned;" ::"r"(smem_addr(&s_tmem)), "r"(columns) : "memory");
+    if (a.qnorm2 && rank == 0 && tid < a.n) query_norm<D>(a, bh, tid);
+    asm volatile("cp.async.wait_all;\nfence.proxy.async.shared::cta;" ::: "memory");
+    tmem_before_sync();
     __syncthreads();
-
-    for (int mp = 0; mp * 32 < a.n; ++mp) {            // two 16-row tiles of queries at a time
-        float rm[2][2];                 // running maximum of rows g, g + 8 of the two tiles over the tokens this lane sees
-#pragma unroll
-        for (int mt = 0; mt < 2; ++mt) rm[mt][0] = rm[mt][1] = NEG;
-
-#pragma unroll 1
-        for (int step = 0; step < PC_CHUNK / PC_WARPS / 8; step += 2) {    // two groups of 8 tokens per set of query fragments
-            const int t0 = t_warp + 8 * step;
-            if (t0 >= a.T) break;
-            // lane (g, c) holds, of token t0 + g (and t0 + 8 + g), the 16-byte pieces c, c + 4, ...: the four lanes of a
-            // token read 64 consecutive bytes at a time, and the words of piece 4i + c are the B operands of k steps
-            // 2i and 2i + 1 (the queries are laid out to match)
-            uint32_t bw[2][WPL];
-#pragma unroll
-            for (int h = 0; h < 2; ++h) {
-                const int t = t0 + 8 * h + g;
-                const uint4* src = reinterpret_cast<const uint4*>(Kb + (size_t)(t < a.T ? t : 0) * a.st) + c;
-#pragma unroll
-                for (int i = 0; i < WPL / 4; ++i) {
-                    uint4 v = make_uint4(0, 0, 0, 0);
-                    if (t < a.T) v = src[4 * i];
-                    bw[h][4 * i] = v.x; bw[h][4 * i + 1] = v.y; bw[h][4 * i + 2] = v.z; bw[h][4 * i + 3] = v.w;
-                }
-            }
-#pragma unroll
-            for (int mt = 0; mt < 2; ++mt) {
-                float acc[2][4];
-#pragma unroll
-                for (int i = 0; i < 4; ++i) { acc[0][i] = 0.f; acc[1][i] = 0.f; }
-#pragma unroll
-                for (int ks = 0; ks < KS; ++ks) {
-                    const uint4 f = s_q[((2 * mp + mt) * KS + ks) * 32 + lane];
-                    const uint32_t fr[4] = {f.x, f.y, f.z, f.w};
-                    mma_16816(acc[0], fr, bw[0][2 * ks], bw[0][2 * ks + 1]);
-                    mma_16816(acc[1], fr, bw[1][2 * ks], bw[1][2 * ks + 1]);
-                }
-                // acc[h][0..1]: row g, tokens t0+8h+2c, +1;  acc[h][2..3]: row g+8
-#pragma unroll
-                for (int hr = 0; hr < 2; ++hr) {
-                    const int i = mp * 32 + mt * 16 + g + 8 * hr;          // query
-                    if (i >= a.n) continue;
-                    const int last = a.T - a.n + i;                         // last token the query sees
-#pragma unroll
-                    for (int h = 0; h < 2; ++h) {
-                        const int t = t0 + 8 * h + 2 * c;
-                        const float l0 = a.scale * acc[h][2 * hr], l1 = a.scale * acc[h][2 * hr + 1];
-                        *reinterpret_cast<float2*>(&s_l[(size_t)i * PC_PITCH + (t - t_cta)]) = make_float2(l0, l1);
-                        if (t <= last) rm[mt][hr] = fmaxf(rm[mt][hr], l0);       // last < T: one bound does for both
-                        if (t + 1 <= last) rm[mt][hr] = fmaxf(rm[mt][hr], l1);
-                    }
-                }
-            }
-        }
-        // merge the four lanes of a row, then the warps, into this CTA's maximum of the row
-#pragma unroll
-        for (int mt = 0; mt < 2; ++mt)
-#pragma unroll
-            for (int hr = 0; hr < 2; ++hr) {
-                float m = rm[mt][hr];
-                m = fmaxf(m, __shfl_xor_sync(0xFFFFFFFFu, m, 1));
-                m = fmaxf(m, __shfl_xor_sync(0xFFFFFFFFu, m, 2));
-                if (c == 0) s_part[warp][mt * 16 + g + 8 * hr] = m;
-            }
-        __syncthreads();
-        if (threadIdx.x < 32 && mp * 32 + (int)threadIdx.x < a.n) {
-            float m = NEG;
-#pragma unroll
-            for (int w = 0; w < PC_WARPS; ++w) m = fmaxf(m, s_part[w][threadIdx.x]);
-            s_mcta[mp * 32 + threadIdx.x] = m;
-        }
-        __syncthreads();
+    tmem_after_sync();
+    const uint32_t acc = *(volatile uint32_t*)&s_tmem;
+    if ((tid & 127) == 0) {
+        multiply<D, NC>(acc + group * NC, base + group * W::TILE_BYTES, queries);
+        tensor_done(bar);
     }
-    // ---- the logits become exponentials relative to the CTA's row maximum, in place (one exponential per entry in
-    //      all; entries a query cannot see become 0), and every row gets its sum over this CTA's tokens
-    const int nt = min(PC_CHUNK, a.T - t_cta);
-    const unsigned ncta = cluster.num_blocks(), rank = cluster.block_rank();
-    asm volatile("barrier.cluster.wait.acquire.aligned;" ::: "memory");       // second half of the barrier begun at the start
-    for (int i = warp; i < a.n; i += PC_WARPS) {
-        const int last = a.T - a.n + i;
-        const float m = s_mcta[i];
-        float* rowl = s_l + (size_t)i * PC_PITCH;
-        float sum = 0.f;
-        for (int k = 4 * lane; k < nt; k += 128) {       // the pitch covers the four of a ragged end; what is there is not used
-            const float4 l = *reinterpret_cast<const float4*>(rowl + k);
-            float4 e;
-            e.x = (t_cta + k <= last) ? __expf(l.x - m) : 0.f;
-            e.y = (t_cta + k + 1 <= last) ? __expf(l.y - m) : 0.f;
-            e.z = (t_cta + k + 2 <= last) ? __expf(l.z - m) : 0.f;
-            e.w = (t_cta + k + 3 <= last) ? __expf(l.w - m) : 0.f;
-            *reinterpret_cast<float4*>(rowl + k) = e;
-            sum += (e.x + e.y) + (e.z + e.w);
-        }
+    __syncwarp();
+    const bool ok = __all_sync(0xFFFFFFFFu, bar_wait(bar, 0u));
+    tmem_after_sync();
+    float x[NC];
 #pragma unroll
-        for (int o = 16; o > 0; o >>= 1) sum += __shfl_xor_sync(0xFFFFFFFFu, sum, o);
-        if (lane < (int)ncta) *cluster.map_shared_rank(&s_all[rank][i], lane) = make_float2(m, sum);
+    for (int h = 0; h < NC; h += CW) {
+        float v[CW];
+        load_acc(acc + ((uint32_t)(32 * (warp & 3)) << 16) + group * NC + h, v);
+#pragma unroll
+        for (int c = 0; c < CW; ++c) x[h + c] = v[c] * sc;
     }
-    // ---- every CTA of the (b,h) has the row statistics of all of them (the remote stores are complete at the cluster
-    //      barrier, and nothing is read from or written to another CTA afterwards): merge them
-    cluster.sync();
-    for (int i = threadIdx.x; i < a.n; i += blockDim.x) {
-        float m = NEG, s = 0.f;
-        for (unsigned r = 0; r < ncta; ++r) {
-            const float2 p = s_all[r][i];
-            const float mn = fmaxf(m, p.x);
-            s = (m == NEG ? 0.f : s * __expf(m - mn)) + (p.x == NEG ? 0.f : p.y * __expf(p.x - mn));
-            m = mn;
+    if (!ok)
+#pragma unroll
+        for (int c = 0; c < NC; ++c) x[c] = __int_as_float(0x7fffffff);
+    // ---- per warp: maximum of every row over its tokens, the logits become powers of two relative to it (0 where the query cannot
+    //      see the token), and their sum
+    const int t = t_group + 32 * (warp & 3) + lane, hidden = t - (a.T - a.n);
+#pragma unroll
+    for (int c0 = 0; c0 < NC; c0 += 8) {
+        if (c0 >= a.n) break;
+        float m[8], sum[8];
+#pragma unroll
+        for (int c = 0; c < 8; ++c) {
+            const bool seen = c0 + c >= hidden;
+            m[c] = warp_max(seen ? x[c0 + c] : NEG);
+            sum[c] = x[c0 + c] = seen ? pow2(x[c0 + c] - m[c]) : 0.f;
         }
-        // what this CTA's exponentials are multiplied by: exp(own maximum - maximum of the row) / sum of the row
-        const float own = s_mcta[i];
-        s_inv[i] = (s > 0.f && own != NEG) ? __expf(own - m) / s : 0.f;
+        if (lane == 0) {
+            *reinterpret_cast<float4*>(&s_max[warp][c0]) = make_float4(m[0], m[1], m[2], m[3]);
+            *reinterpret_cast<float4*>(&s_max[warp][c0 + 4]) = make_float4(m[4], m[5], m[6], m[7]);
+        }
+        const float s = sum8(sum, lane);
+        if ((lane & 3) == 0) s_sum[warp][c0 + (lane >> 2)] = s;
     }
+    tmem_before_sync();
     __syncthreads();
-    // ---- normalised rows, newest first, written once; rows-per-token counts
-    const bool vec_ok = (a.T & 3) == 0 && ((uintptr_t)a.ring & 15) == 0;      // rows start 16-byte aligned, no ragged end
-    for (int r = warp; r < a.n; r += PC_WARPS) {
-        const int i = a.n - 1 - r;
-        const float f = s_inv[i];
-        float* row = a.ring + ((size_t)bh * a.n + r) * a.T + t_cta;
-        const float* src = s_l + (size_t)i * PC_PITCH;
-        if (vec_ok) {     // four tokens per lane and store
-            for (int k = 4 * lane; k < nt; k += 128) {
-                float4 o = *reinterpret_cast<const float4*>(src + k);
-                o.x *= f; o.y *= f; o.z *= f; o.w *= f;
-                *reinterpret_cast<float4*>(row + k) = o;
-            }
-        } else {
-            for (int k = lane; k < nt; k += 32) row[k] = src[k] * f;
+    if (warp == 0) { tmem_after_sync(); asm volatile("tcgen05.dealloc.cta_group::1.sync.aligned.b32 %0, %1;" ::"r"(acc), "r"(columns) : "memory"); }
+    if (ncta > 1) {
+        asm volatile("barrier.cluster.wait.acquire.aligned;" ::: "memory");              // second half of the barrier begun at the start
+        if (const int c = tid % NC; c < a.n) {
+            float2 own = make_float2(NEG, 0.f);
+            for (int w = 0; w < warps; ++w) fold_stats(own, make_float2(s_max[w][c], s_sum[w][c]));
+            for (int r = tid / NC; r < ncta; r += blockDim.x / NC)
+                asm volatile("{\n.reg .u32 p;\nmapa.shared::cluster.u32 p, %0, %1;\nst.shared::cluster.v2.f32 [p], {%2, %3};\n}"
+                             ::"r"(smem_addr(&s_all[rank][c])), "r"(r), "f"(own.x), "f"(own.y) : "memory");
         }
+        // every CTA has the statistics of all of them (the stores are complete at the barrier, and nothing is written to or read
+        // from another CTA afterwards)
+        cluster_barrier();
     }
-    for (int k = threadIdx.x; k < nt; k += blockDim.x) a.nvalid[(size_t)bh * a.T + t_cta + k] = (uint8_t)min(a.n, a.T - (t_cta + k));
+    // ---- what the warp's powers are multiplied by, a row per lane; normalised rows, newest first, written once; rows-per-token counts
+    float f[NC / CW];
+#pragma unroll
+    for (int h = 0; h < NC / CW; ++h) {
+        const int c = CW * h + lane % CW;
+        float2 all = make_float2(NEG, 0.f);
+        if (c < a.n) {
+            if (ncta > 1) for (int r = 0; r < ncta; ++r) fold_stats(all, s_all[r][c]);
+            else for (int w = 0; w < warps; ++w) fold_stats(all, make_float2(s_max[w][c], s_sum[w][c]));
+        }
+        const float own = c < a.n ? s_max[warp][c] : NEG;
+        f[h] = all.y > 0.f && own != NEG ? pow2(own - all.x) / all.y : 0.f;
+    }
+    float* row = a.ring + ((size_t)bh * a.n + (a.n - 1)) * a.T + t;
+#pragma unroll
+    for (int c = 0; c < NC; ++c) {
+        if (c >= a.n) break;
+        const float y = x[c] * __shfl_sync(0xFFFFFFFFu, f[c / CW], c % CW);
+        if (t < a.T) *row = y;
+        row -= a.T;
+    }
+    if (t < a.T) a.nvalid[(size_t)bh * a.T + t] = (uint8_t)min(a.n, a.T - t);
 }
-
-template <int D>
-qaq_status run_cluster(const PrefillArgs& a, int BH, int ncl, size_t smem, cudaStream_t s) {
+template <int D, int NC>
+qaq_status run_short(const PrefillArgs& a, const void* K, long sb, long sh, long st, int groups, int ncta, cudaStream_t s) {
+    using W = Window<D, NC, STATS>;
     static SmemSeen seen;
-    const size_t most = (size_t)PW_MAXQ * PC_PITCH * sizeof(float) + 4 * (D / 16) * 32 * sizeof(uint4);
-    QAQ_CUDA_TRY(qaq_allow_smem((const void*)window_cluster_kernel<D>, most, seen));
-    QAQ_CUDA_TRY(qaq_launch_cluster(window_cluster_kernel<D>, dim3((unsigned)ncl, (unsigned)BH), dim3(PC_WARPS * 32), ncl, smem, s, a));
+    QAQ_CUDA_TRY(qaq_allow_smem((const void*)window_short_kernel<D, NC>, 1024 + PS_TILES * W::TILE_BYTES + W::QUERY_BYTES, seen));
+    QAQ_CUDA_TRY(qaq_launch_cluster(window_short_kernel<D, NC>, dim3((unsigned)ncta, (unsigned)a.BH), dim3(128u * groups), ncta, 1024 + groups * W::TILE_BYTES + W::QUERY_BYTES, s,
+                                    a, (const __half*)K, sb, sh, st));
+    return QAQ_OK;
+}
+
+// Descriptions of K ([batch][head][token][channel] with the caller's strides) and of the queries for the copies of tiles.
+typedef CUresult (*EncodeTiled)(CUtensorMap*, CUtensorMapDataType, cuuint32_t, void*, const cuuint64_t*, const cuuint64_t*, const cuuint32_t*, const cuuint32_t*,
+                                CUtensorMapInterleave, CUtensorMapSwizzle, CUtensorMapL2promotion, CUtensorMapFloatOOBfill);
+bool describe(CUtensorMap* map, const void* at, int rank, const cuuint64_t* size, const cuuint64_t* stride, const cuuint32_t* box, int D) {
+    static const EncodeTiled encode = [] {
+        void* f = nullptr;
+        cudaDriverEntryPointQueryResult found;
+        const cudaError_t e = cudaGetDriverEntryPointByVersion("cuTensorMapEncodeTiled", &f, 12000, cudaEnableDefault, &found);
+        if (e != cudaSuccess) (void)cudaGetLastError();
+        return e == cudaSuccess && found == cudaDriverEntryPointSuccess ? (EncodeTiled)f : (EncodeTiled) nullptr;
+    }();
+    const cuuint32_t each[4] = {1, 1, 1, 1};
+    return encode && encode(map, CU_TENSOR_MAP_DATA_TYPE_FLOAT16, rank, const_cast<void*>(at), size, stride, box, each, CU_TENSOR_MAP_INTERLEAVE_NONE,
+                            D >= 64 ? CU_TENSOR_MAP_SWIZZLE_128B : CU_TENSOR_MAP_SWIZZLE_64B, CU_TENSOR_MAP_L2_PROMOTION_L2_256B, CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE) == CUDA_SUCCESS;
+}
+
+template <int D, int NC>
+qaq_status run_window(PrefillArgs a, const void* K, long sb, long sh, long st, int batch, cudaStream_t s) {
+    using W = Window<D, NC, ONE_PASS>;
+    const int tiles = (a.T + PW_TILE - 1) / PW_TILE;
+    // few tiles: one-tile CTAs while all of them run at once (two to an SM: 32 (b,h) of 1000 tokens 9.2 us, 9.0 by the kernel below, of 333
+    // 6.0 and 7.8), else a (b,h) to a CTA (256 of 300 tokens 9.2 and 12.8)
+    if (tiles <= PW_CLUSTER && (long long)a.BH * tiles <= 2 * 148) return run_short<D, NC>(a, K, sb, sh, st, 1, tiles, s);
+    if (tiles <= PS_TILES) return run_short<D, NC>(a, K, sb, sh, st, tiles, 1, s);
+    CUtensorMap keys, queries;
+    const cuuint32_t inner = D >= 64 ? 64 : 32;
+    const cuuint64_t ksize[4] = {(cuuint64_t)D, (cuuint64_t)a.T, (cuuint64_t)a.H, (cuuint64_t)batch}, kstride[3] = {2ull * st, 2ull * sh, 2ull * sb};
+    const cuuint64_t qsize[2] = {(cuuint64_t)D, (cuuint64_t)a.BH * a.n}, qstride[1] = {2ull * D};
+    const cuuint32_t kbox[4] = {inner, PW_TILE, 1, 1}, qbox[2] = {inner, NC};
+    if (!describe(&keys, K, 4, ksize, kstride, kbox, D) || !describe(&queries, a.Q, 2, qsize, qstride, qbox, D)) return QAQ_ERR_CUDA;
+    static SmemSeen seen[3];
+    static ClusterRoom room;
+    QAQ_CUDA_TRY(qaq_allow_smem((const void*)window_kernel<D, NC, ONE_PASS>, PW_SMEM, seen[0]));
+    // the size of the cluster: the fewest tiles one after the other, and where that is the same, accumulators of two (b,h) at a time
+    int best = 0, most = 0;
+    long long least = 0;
+    for (int k = 1; k <= PW_CLUSTER && k <= tiles; ++k) {
+        const int each = (tiles + k - 1) / k;
+        if (each > W::SLOTS || (tiles + each - 1) / each != k) continue;
+        const int n = clusters_at_once(window_kernel<D, NC, ONE_PASS>, PW_THREADS, PW_SMEM, k, room);
+        if (n < 1) continue;
+        const long long time = (long long)((a.BH + n - 1) / n) * each;
+        if (!best || time < least || (time == least && 2 * a.tiles > W::SLOTS)) { best = k; least = time; a.tiles = each; most = min(a.BH, n); }
+    }
+    if (best) {
+        QAQ_CUDA_TRY(qaq_launch_cluster(window_kernel<D, NC, ONE_PASS>, dim3((unsigned)(most * best)), dim3(PW_THREADS), best, PW_SMEM, s, keys, queries, a));
+        return QAQ_OK;
+    }
+    // chunks of at least PW_CHUNK tokens (the workspace's), as long as every SM gets eight
+    QAQ_CUDA_TRY(qaq_allow_smem((const void*)window_kernel<D, NC, STATS>, PW_SMEM, seen[1]));
+    QAQ_CUDA_TRY(qaq_allow_smem((const void*)window_kernel<D, NC, ROWS>, PW_SMEM, seen[2]));
+    a.tiles = max(PW_CHUNK / PW_TILE, (int)((long long)tiles * a.BH / (8 * 148)));
+    a.nchunk = (tiles + a.tiles - 1) / a.tiles;
+    const dim3 grid((unsigned)min(148, a.BH * a.nchunk));
+    QAQ_CUDA_TRY(qaq_launch(window_kernel<D, NC, STATS>, grid, dim3(PW_THREADS), PW_SMEM, s, keys, queries, a));
+    QAQ_CUDA_TRY(qaq_launch(window_kernel<D, NC, ROWS>, grid, dim3(PW_THREADS), PW_SMEM, s, keys, queries, a));
     return QAQ_OK;
 }
 
 template <int D>
-qaq_status run_long(const PrefillArgs& a, int BH, cudaStream_t s) {
-    const dim3 grid((unsigned)a.nchunk, (unsigned)BH);
-    const size_t smem = (size_t)(2 * ((a.n + 31) / 32)) * (D / 16) * 32 * sizeof(uint4);       // at most 16 KB
-    QAQ_CUDA_TRY(qaq_launch(window_long_kernel<D, true>, grid, dim3(PW_WARPS * 32), smem, s, a));
-    QAQ_CUDA_TRY(qaq_launch(window_long_kernel<D, false>, grid, dim3(PW_WARPS * 32), smem, s, a));
-    return QAQ_OK;
+qaq_status pick_window(const PrefillArgs& a, const void* K, long sb, long sh, long st, int batch, cudaStream_t s) {
+    return a.n <= 16 ? run_window<D, 16>(a, K, sb, sh, st, batch, s) : a.n <= 32 ? run_window<D, 32>(a, K, sb, sh, st, batch, s) : run_window<D, 64>(a, K, sb, sh, st, batch, s);
 }
 
 // Upper quantile of a list of binary32 values (the squared query norms): exact 4 x 8-bit radix select on
@@ -495,28 +725,14 @@ extern "C" qaq_status qaq_prefill_window(const qaq_config* cfg, const void* Q, c
     qaq_prefill_window_workspace_bytes(cfg, n_tokens, &need);
     if (ws_bytes < need || ((uintptr_t)ws & 7)) return QAQ_ERR_WORKSPACE;
     PrefillArgs a;
-    a.Q = (const __half*)Q; a.K = (const __half*)K; a.sb = stride_b; a.sh = stride_h; a.st = stride_t;
-    a.H = cfg->heads; a.T = n_tokens; a.n = cfg->window; a.scale = softmax_scale;
+    a.Q = (const __half*)Q; a.H = cfg->heads; a.BH = cfg->batch * cfg->heads; a.T = n_tokens; a.n = cfg->window; a.scale = softmax_scale;
     a.ring = score_ring; a.nvalid = nvalid; a.qnorm2 = qnorm2; a.part = (float2*)ws;
-    a.nchunk = (n_tokens + PW_CHUNK - 1) / PW_CHUNK;
+    a.nchunk = a.tiles = 0;
     cudaStream_t s = (cudaStream_t)stream;
-    const int ncl = (n_tokens + PC_CHUNK - 1) / PC_CHUNK;
-    if (ncl <= PC_MAXCTA) {
-        // one pass: the CTAs of a (b,h) are one cluster
-        const size_t smem = (size_t)cfg->window * PC_PITCH * sizeof(float) +
-                            (size_t)(2 * ((cfg->window + 31) / 32)) * (cfg->head_dim / 16) * 32 * sizeof(uint4);   // logits, query fragments
-        const int BH = cfg->batch * cfg->heads;
-        switch (cfg->head_dim) {
-            case 32: return run_cluster<32>(a, BH, ncl, smem, s);
-            case 64: return run_cluster<64>(a, BH, ncl, smem, s);
-            case 128: return run_cluster<128>(a, BH, ncl, smem, s);
-        }
-        return QAQ_ERR_UNSUPPORTED_SHAPE;
-    }
     switch (cfg->head_dim) {
-        case 32: return run_long<32>(a, cfg->batch * cfg->heads, s);
-        case 64: return run_long<64>(a, cfg->batch * cfg->heads, s);
-        case 128: return run_long<128>(a, cfg->batch * cfg->heads, s);
+        case 32: return pick_window<32>(a, K, stride_b, stride_h, stride_t, cfg->batch, s);
+        case 64: return pick_window<64>(a, K, stride_b, stride_h, stride_t, cfg->batch, s);
+        case 128: return pick_window<128>(a, K, stride_b, stride_h, stride_t, cfg->batch, s);
     }
     return QAQ_ERR_UNSUPPORTED_SHAPE;
 }

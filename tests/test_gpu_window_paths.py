@@ -1,0 +1,76 @@
+"""Score window after a prefill (Section 4.2): each way it is computed - few tiles (one CTA or a cluster per (b,h)), one pass of
+resident CTAs, two passes over chunks - at the edges of tiles and of the sizes the ways divide at, against the oracle's causal
+softmax rows.  Bound of a row: 1e-6 + 1e-2 of the entry, as everywhere for scores (the logits differ by binary32 sums of 128 products)."""
+import math
+
+import numpy as np
+import pytest
+import torch
+
+import oracle
+from paper_2403_04643_b200 import qaq
+
+from gpu_helpers import u16
+
+pytestmark = pytest.mark.gpu
+
+
+def rows_match(K, Q, heads, which):
+    B, H, T, D = K.shape
+    n, scale = Q.shape[1], 1.0 / math.sqrt(D)
+    cfg = qaq.make_config(B, heads, D, T, 2, 8, n, 0.01)
+    ring, nvalid = qaq.qaq_prefill_window(cfg, Q.cuda(), K, scale)
+    ring, nvalid = ring.view(B * H, n, T), nvalid.view(B * H, T)
+    for bh in which:
+        want, nv, _ = oracle.prefill_window(u16(Q[bh]), u16(K[bh // H, bh % H]), scale)
+        got = ring[bh].cpu().numpy().astype(np.float64)
+        assert np.array_equal(nvalid[bh].cpu().numpy(), nv)
+        assert np.all(got[want == 0] == 0)
+        assert np.all(np.abs(got - want) <= 1e-6 + 1e-2 * want), (bh, np.abs(got - want).max())
+    return ring
+
+
+def keys(B, H, T, D, token_major, seed):
+    g = torch.Generator(device="cuda").manual_seed(seed)
+    K = torch.randn((B, T, H, D) if token_major else (B, H, T, D), generator=g, device="cuda").half()
+    return K.transpose(1, 2) if token_major else K
+
+
+@pytest.mark.parametrize("D", [32, 64, 128])
+@pytest.mark.parametrize("heads,T,n", [
+    (2, 1, 1), (2, 127, 16), (2, 129, 17), (3, 1024, 33),           # a cluster of one-tile CTAs
+    (320, 128, 32), (110, 300, 5), (80, 512, 64),                   # up to four tiles in a CTA
+    (40, 1025, 64), (75, 513, 32), (9, 2048, 16), (5, 4097, 32), (3, 8191, 64),      # one pass, clusters of several sizes
+    (160, 640, 1),                                                  # more (b,h) than CTAs
+    (2, 8193, 64), (2, 16385, 32),                                  # two passes
+])
+def test_window_rows_of_every_way(D, heads, T, n):
+    K = keys(1, heads, T, D, token_major=heads % 2 == 1, seed=D + T)
+    Q = torch.randn((heads, n, D), generator=torch.Generator().manual_seed(n)).half()
+    rows_match(K, Q, heads, {0, heads // 2, heads - 1})
+
+
+@pytest.mark.parametrize("T,n", [(700, 40), (4100, 32), (8200, 64)])
+def test_a_reference_far_below_a_later_logit(T, n):
+    # the logits of the first tiles are near zero, those of later tokens beyond 2^64 times their exponentials
+    K = keys(2, 2, T, 64, token_major=False, seed=T) * 0.01
+    K[:, :, T - T // 3:] *= 3000.0
+    Q = torch.randn((4, n, 64), generator=torch.Generator().manual_seed(n)).half() * 4
+    ring = rows_match(K, Q, 2, range(4))
+    assert torch.allclose(ring.sum(2), torch.ones(4, n, device="cuda"), atol=1e-4)
+
+
+@pytest.mark.parametrize("T", [100, 1500, 9000])
+def test_heads_that_share_keys_and_keys_that_are_not_numbers(T):
+    # one set of keys under several heads by a stride of zero; a NaN stays in its token and row, the other tokens of the row become 0
+    K = keys(1, 1, T, 128, token_major=False, seed=T)
+    Q = torch.randn((3, 8, 128), generator=torch.Generator().manual_seed(1)).half()
+    shared = rows_match(K.expand(1, 3, T, 128), Q, 3, range(3))
+    bad = K.clone()
+    bad[0, 0, T // 2, 5] = math.nan
+    cfg = qaq.make_config(1, 3, 128, T, 2, 8, 8, 0.01)
+    ring, _ = qaq.qaq_prefill_window(cfg, Q.cuda(), bad.expand(1, 3, T, 128), 1 / math.sqrt(128))
+    ring = ring.view(3, 8, T)
+    assert torch.isnan(ring[:, :, T // 2]).all()
+    ring[:, :, T // 2] = 0
+    assert (ring == 0).all() and (shared.sum() > 0)
