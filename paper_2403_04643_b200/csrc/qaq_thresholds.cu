@@ -3,8 +3,7 @@
 // Wanted: lo = k-th smallest and hi = k-th largest of the N non-NaN values, k = floor(alpha*N/2).
 // Only the two tails matter, so the bulk of the data is never histogrammed:
 //   1. thr_sample_kernel   a few tokens spread over the sequence give a bracket per tail: a value
-//                          below (above) which somewhat more than the wanted tail mass lies.  Problems
-//                          small enough to be sampled completely are solved right here.
+//                          below (above) which somewhat more than the wanted tail mass lies.
 //   2. thr_scan_kernel     the one pass over all values: entries beyond the brackets ("candidates",
 //                          a few per cent) are compacted into per-problem lists (shared-memory lists
 //                          per CTA, one global reservation per CTA; what a CTA's list does not hold goes to
@@ -13,6 +12,7 @@
 //                          turned out too tight (fewer than k+1 candidates) or a problem's list overflowed, the
 //                          problem is redone exactly by a two-pass radix select over its data, so the
 //                          result is always the exact order statistic.
+// Short sequences take one kernel (thr_short_kernel).
 // binary16 patterns are mapped to 16-bit keys that sort like the values.
 #include "qaq_internal.cuh"
 
@@ -33,9 +33,8 @@ struct Problem {          // per (b,h,tensor), in the workspace
     uint32_t klo, khi;    // bracket keys: candidates are keys < klo and keys > khi
     uint32_t cnt[2];      // candidates found below and above (their sum may exceed the capacity: then the list is incomplete)
     uint32_t nan;         // NaN entries seen by the scan
-    uint32_t done;        // solved by the sample kernel
     uint32_t n;           // places taken in the list
-    uint32_t pad;
+    uint32_t pad[2];
 };
 
 struct ThrArgs {
@@ -182,7 +181,7 @@ __device__ __forceinline__ uint32_t bracket_rank(double alpha, uint32_t M) {
     return r > (M - 1) / 2 ? (M - 1) / 2 : r;
 }
 
-// ---- 1. sample: brackets (or the exact answer when the sample is the whole problem)
+// ---- 1. sample: brackets
 template <int THREADS>
 __global__ void __launch_bounds__(THREADS) thr_sample_kernel(const ThrArgs a) {
     constexpr int PIECES = SAMPLE_TOKENS * 128 / 8 / THREADS;            // 16-byte pieces of a thread at most
@@ -192,7 +191,7 @@ __global__ void __launch_bounds__(THREADS) thr_sample_kernel(const ThrArgs a) {
     __shared__ uint32_t hist[2048], s_tmp[4], s_cnt[2];
     const int b_idx = bh / a.H, h_idx = bh % a.H;
     const __half* X = a.X[x] + (size_t)b_idx * a.sb + (size_t)h_idx * a.sh;
-    const int ns = a.T < SAMPLE_TOKENS ? a.T : SAMPLE_TOKENS;
+    constexpr int ns = SAMPLE_TOKENS;                            // (shorter sequences: thr_short_kernel)
     const int M = ns * a.D;
     if (threadIdx.x < 2) s_cnt[threadIdx.x] = 0;
     __syncthreads();
@@ -220,31 +219,14 @@ __global__ void __launch_bounds__(THREADS) thr_sample_kernel(const ThrArgs a) {
     const uint32_t Mv = (uint32_t)M - s_cnt[0];                    // non-NaN sample values
     const uint32_t n_neg_nan = s_cnt[1];
     Problem* pr = a.prob + bhx;
-    const bool whole = (ns == a.T);
     if (Mv == 0) {
-        if (threadIdx.x == 0) {
-            pr->klo = 0; pr->khi = 0xFFFF; pr->cnt[0] = pr->cnt[1] = 0; pr->nan = 0; pr->n = 0; pr->done = whole ? 1u : 0u;
-            if (whole) { a.thr[(size_t)bh * 4 + 2 * x] = 0.f; a.thr[(size_t)bh * 4 + 2 * x + 1] = 0.f; }
-        }
+        if (threadIdx.x == 0) { pr->klo = 0; pr->khi = 0xFFFF; pr->cnt[0] = pr->cnt[1] = 0; pr->nan = 0; pr->n = 0; }
         return;
     }
-    uint32_t r_lo, r_hi;
-    if (whole) {
-        const unsigned long long k = rank_k(a.alpha, Mv);
-        r_lo = (uint32_t)k; r_hi = (uint32_t)(Mv - 1 - k);
-    } else {
-        const uint32_t r = bracket_rank(a.alpha, Mv);
-        r_lo = r; r_hi = Mv - 1 - r;
-    }
+    const uint32_t r = bracket_rank(a.alpha, Mv);
     uint32_t klo, khi;
-    cta_select_keys<THREADS>(s_keys, (uint32_t)M, r_lo + n_neg_nan, r_hi + n_neg_nan, hist, s_tmp, klo, khi);
-    if (threadIdx.x == 0) {
-        pr->klo = klo; pr->khi = khi; pr->cnt[0] = pr->cnt[1] = 0; pr->nan = 0; pr->n = 0; pr->done = whole ? 1u : 0u;
-        if (whole) {
-            a.thr[(size_t)bh * 4 + 2 * x] = float_of_key(klo);
-            a.thr[(size_t)bh * 4 + 2 * x + 1] = float_of_key(khi);
-        }
-    }
+    cta_select_keys<THREADS>(s_keys, (uint32_t)M, r + n_neg_nan, Mv - 1 - r + n_neg_nan, hist, s_tmp, klo, khi);
+    if (threadIdx.x == 0) { pr->klo = klo; pr->khi = khi; pr->cnt[0] = pr->cnt[1] = 0; pr->nan = 0; pr->n = 0; }
 }
 
 // ---- 2. the one pass over the data: compaction of the tail candidates.
@@ -256,13 +238,12 @@ __global__ void __launch_bounds__(THREADS) thr_sample_kernel(const ThrArgs a) {
 // list, which the select takes apart by rank.
 // What bounds it: memory where outliers are few (256 (b,h) of 4096 tokens, alpha = 1 %: 105 us, 5.1 TB/s; 124 us without
 // the next pieces on their way while four are looked at, and with 512 tokens per CTA), the extraction where they are many
-// (160 (b,h) of 8192 tokens, 5 %: 215 us; 269 with a list, a prefix sum and a loop for each tail).  60 registers, four
+// (160 (b,h) of 8192 tokens, 5 %: 204 us; 215 with a loop over the candidates of a piece).  60 registers, four
 // CTAs per SM: held to five it takes 114 us, to six 169.
 __global__ void __launch_bounds__(256) thr_scan_kernel(const ThrArgs a) {
     qaq_dependency();
     const int bhx = blockIdx.y, bh = bhx >> 1, x = bhx & 1;
     Problem* pr = a.prob + bhx;
-    if (pr->done) return;
     __shared__ unsigned short s_list[CTA_LIST];
     __shared__ uint4 s_flag[8][WARP_FLAGS];                   // per warp: pieces with something outside [lo, hi]
     __shared__ uint32_t s_n, s_low, s_base, s_nan;
@@ -270,7 +251,8 @@ __global__ void __launch_bounds__(256) thr_scan_kernel(const ThrArgs a) {
     const unsigned lt = (1u << lane) - 1u;
     if (threadIdx.x == 0) { s_n = 0; s_low = 0; s_nan = 0; }
     __syncthreads();
-    const float flo = float_of_key(pr->klo), fhi = float_of_key(pr->khi);
+    const uint32_t klo = pr->klo;
+    const float flo = float_of_key(klo), fhi = float_of_key(pr->khi);
     const __half2 lo2 = __float2half2_rn(flo), hi2 = __float2half2_rn(fhi);   // exact: both are binary16 values
     const int b_idx = bh / a.H, h_idx = bh % a.H;
     const int t0 = blockIdx.x * a.scan_tokens, ntok = min(a.T, t0 + a.scan_tokens) - t0;
@@ -326,19 +308,15 @@ __global__ void __launch_bounds__(256) thr_scan_kernel(const ThrArgs a) {
             const bool have = i0 + lane < ntake;
             const uint4 r = have ? wflag[i0 + lane] : make_uint4(0, 0, 0, 0);
             const uint32_t w[4] = {r.x, r.y, r.z, r.w};
-            uint32_t below = 0, above = 0, nans = 0;              // bit j / 16 + j: low / high half of word j
+            uint32_t m = 0, numbers = 0;                          // bit j / 16 + j: low / high half of word j
 #pragma unroll
             for (int j = 0; j < 4; ++j) {
                 const __half2 v = h2_of(w[j]);
-                const uint32_t ge = __hge2_mask(v, lo2), le = __hle2_mask(v, hi2);   // a NaN compares false twice
-                below |= (~ge & le & 0x00010001u) << j;
-                above |= (ge & ~le & 0x00010001u) << j;
-                nans |= (~(ge | le) & 0x00010001u) << j;
+                m |= (__hlt2_mask(v, lo2) | __hgt2_mask(v, hi2)) & (0x00010001u << j);       // a NaN is neither
+                numbers |= __heq2_mask(v, v) & (0x00010001u << j);
             }
-            if (!have) { below = 0; above = 0; nans = 0; }
-            nnan += (uint32_t)__popc(nans);
-            nlow += (uint32_t)__popc(below);
-            uint32_t m = below | above;
+            if (!have) m = 0;
+            else nnan += 8u - (uint32_t)__popc(numbers);
             const uint32_t mine = (uint32_t)__popc(m);            // at most 8
             uint32_t inc = mine;
 #pragma unroll
@@ -354,16 +332,28 @@ __global__ void __launch_bounds__(256) thr_scan_kernel(const ThrArgs a) {
                 if (b0 + inc > from) g0 = atomicAdd(&pr->n, b0 + inc - from) - from;
             }
             uint32_t pos = __shfl_sync(0xFFFFFFFFu, b0, 31) + inc - mine;
-            g0 = __shfl_sync(0xFFFFFFFFu, g0, 31);
-            while (m) {
-                const int bit = __ffs(m) - 1;
-                m &= m - 1;
-                const int j = bit & 3;
-                const uint32_t wj = (j & 2) ? ((j & 1) ? w[3] : w[2]) : ((j & 1) ? w[1] : w[0]);
-                const unsigned short h = (unsigned short)((bit >> 4) ? (wj >> 16) : (wj & 0xFFFFu));
-                if (pos < (uint32_t)CTA_LIST) s_list[pos] = (unsigned short)key_of(h);
-                else if (g0 + pos < a.cap) dst[g0 + pos] = (unsigned short)key_of(h);
-                ++pos;
+            if (__all_sync(0xFFFFFFFFu, pos + mine <= (uint32_t)CTA_LIST)) {
+                // entry by entry without a loop over the set bits (whose address and selection took more than half of the batch)
+#pragma unroll
+                for (int j = 0; j < 8; ++j)
+                    if (m & (1u << ((j >> 1) + 16 * (j & 1)))) s_list[pos++] = (unsigned short)(w[j >> 1] >> (16 * (j & 1)));
+            } else {
+                g0 = __shfl_sync(0xFFFFFFFFu, g0, 31);
+                while (m) {
+                    const int bit = __ffs(m) - 1;
+                    m &= m - 1;
+                    const int j = bit & 3;
+                    const uint32_t wj = (j & 2) ? ((j & 1) ? w[3] : w[2]) : ((j & 1) ? w[1] : w[0]);
+                    const unsigned short h = (unsigned short)((bit >> 4) ? (wj >> 16) : (wj & 0xFFFFu));
+                    if (pos < (uint32_t)CTA_LIST) s_list[pos] = h;
+                    else {
+                        const uint32_t key = key_of(h);
+                        if (key < klo) ++nlow;
+                        if (g0 + pos < a.cap) dst[g0 + pos] = (unsigned short)key;
+                    }
+                    ++pos;
+                }
+                __syncwarp();
             }
         }
         const uint32_t left = nflag - ntake;           // fewer than 32
@@ -374,22 +364,25 @@ __global__ void __launch_bounds__(256) thr_scan_kernel(const ThrArgs a) {
         nflag = left;
         __syncwarp();     // the rest of the buffer is free again
     }
-#pragma unroll
-    for (int o = 16; o > 0; o >>= 1) { nnan += __shfl_xor_sync(0xFFFFFFFFu, nnan, o); nlow += __shfl_xor_sync(0xFFFFFFFFu, nlow, o); }
+    nnan = __reduce_add_sync(0xFFFFFFFFu, nnan);
     if (lane == 0 && nnan) atomicAdd(&s_nan, nnan);
+    __syncthreads();
+    const uint32_t cnt = min(s_n, (uint32_t)CTA_LIST);
+    if (threadIdx.x == 0) s_base = cnt ? atomicAdd(&pr->n, cnt) : 0u;
+    __syncthreads();
+    for (uint32_t i = threadIdx.x; i < cnt; i += blockDim.x) {
+        const uint32_t pos = s_base + i, key = key_of(s_list[i]);
+        if (key < klo) ++nlow;
+        if (pos < a.cap) dst[pos] = (unsigned short)key;
+    }
+    nlow = __reduce_add_sync(0xFFFFFFFFu, nlow);
     if (lane == 0 && nlow) atomicAdd(&s_low, nlow);
     __syncthreads();
-    const uint32_t cnt = min(s_n, (uint32_t)CTA_LIST), low = s_low;
     if (threadIdx.x == 0) {
-        s_base = cnt ? atomicAdd(&pr->n, cnt) : 0u;
+        const uint32_t low = s_low;
         if (low) atomicAdd(&pr->cnt[0], low);
         if (s_n > low) atomicAdd(&pr->cnt[1], s_n - low);
         if (s_nan) atomicAdd(&pr->nan, s_nan);
-    }
-    __syncthreads();
-    for (uint32_t i = threadIdx.x; i < cnt; i += blockDim.x) {
-        const uint32_t pos = s_base + i;
-        if (pos < a.cap) dst[pos] = s_list[i];
     }
 }
 
@@ -399,7 +392,6 @@ __global__ void __launch_bounds__(THREADS) thr_select_kernel(const ThrArgs a) {
     qaq_dependency();
     const int bhx = blockIdx.x, bh = bhx >> 1, x = bhx & 1;
     Problem* pr = a.prob + bhx;
-    if (pr->done) return;
     __shared__ uint32_t hist[2048], s_tmp[4];
     __shared__ __align__(16) unsigned short s_keys[SELECT_KEYS];
     const unsigned long long total = (unsigned long long)a.T * a.D;
@@ -441,101 +433,126 @@ __global__ void __launch_bounds__(THREADS) thr_select_kernel(const ThrArgs a) {
     if (threadIdx.x < 2) a.thr[(size_t)bh * 4 + 2 * x + threadIdx.x] = threadIdx.x ? res[1] : res[0];
 }
 
-// ---- short sequences: the three steps by one CTA per problem, on keys that stay in shared memory.
-// The chain of three launches is latency: 32 (b,h) of 100 tokens 16.8 us, this kernel 13.8; 256 (b,h) 33.8 against 23.4 us;
-// but 32 of 333 tokens 17.5 against 25.4 us (19 with 1024 threads, which are slower at 100 tokens of many (b,h)).
-constexpr uint32_t SMALL_KEYS = 16384;     // keys of a problem at most
-constexpr uint32_t SMALL_LIST = 4096;      // candidates of a tail at most
-constexpr int SMALL_THREADS = 256;
-struct SmallScratch {
-    uint32_t hist[2048], tmp[4], n[2], cnt[4];
-    alignas(16) unsigned short list[2 * SMALL_LIST];       // the sample, then the candidates
-    alignas(16) unsigned short keys[8];                    // T * D of them
-};
-__global__ void __launch_bounds__(SMALL_THREADS) thr_small_kernel(const ThrArgs a) {
-    extern __shared__ __align__(16) unsigned char small_smem[];
-    SmallScratch& sm = *reinterpret_cast<SmallScratch*>(small_smem);
-    static_assert(2 * SMALL_LIST >= SAMPLE_TOKENS * 128, "the sample fits the list");
-    const int bhx = blockIdx.x, bh = bhx >> 1, x = bhx & 1, tid = threadIdx.x;
-    if (tid < 4) sm.cnt[tid] = 0;
-    if (tid < 2) sm.n[tid] = 0;
+// ---- short sequences: one launch, a CTA per problem, its keys in registers.
+// A key among the k + 1 smallest is not above the (k + 1)-th smallest of the pieces' minima (a piece: eight keys), so the minima
+// and the maxima give a bin of 32 keys for either tail; the keys up to the one and from the other on are counted by bins, which
+// gives the bin of each rank, and a second count, of the keys inside these two bins, the keys themselves.  Nothing is guessed, there
+// is no other path to fall back to.  What bounds it: the latency of one load after the other step.  32 (b,h) of 100 tokens 13.2 us
+// with a sample, brackets from it and lists of candidates, 7.8 this way; 256 of 100 22.5 and 21.4; 64 of 400, head_dim 64, 15.5 and 10.9.  (The keys of a problem spread over a thread-block cluster, whose
+// counts meet in distributed shared memory: 32 (b,h) of 1000 tokens 25 to 36 us, the three kernels above 19.)
+constexpr int SHORT_THREADS = 512, SHORT_PIECES = 8;                             // pieces of a thread
+__global__ void __launch_bounds__(SHORT_THREADS, 2) thr_short_kernel(const ThrArgs a) {
+    constexpr int THREADS = SHORT_THREADS;
+    constexpr int PER = 2048 / THREADS;                                          // bins of a thread
+    __shared__ uint32_t s_lo[2048], s_hi[2048];                                  // counts by the upper 11 bits of the key: minima, maxima; then s_lo: keys
+    __shared__ uint32_t s_fine[64], s_nan, s_part[2][32], s_found[4];            // counts by the lower 5 bits; NaNs
+    const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31, bhx = blockIdx.x, bh = bhx >> 1, x = bhx & 1;
+    for (int i = tid; i < 2048; i += THREADS) { s_lo[i] = 0; s_hi[i] = 0; }
+    if (tid < 64) s_fine[tid] = 0;
+    if (tid == 0) { s_nan = 0; s_found[0] = 2047; s_found[2] = 0; }              // (fewer pieces than the rank: all keys are counted)
     __syncthreads();
     qaq_dependency();
-    const int shift = 31 - __clz(a.D / 8);                 // 16-byte pieces per token
+    const int shift = 31 - __clz(a.D / 8);                                       // pieces of a token
     const uint32_t total = (uint32_t)a.T * (uint32_t)a.D, n8 = total / 8;
-    const __half* X = a.X[x] + (size_t)(bh / a.H) * a.sb + (size_t)(bh % a.H) * a.sh;
-    uint4* keys = reinterpret_cast<uint4*>(sm.keys);
-    uint32_t nn = 0, nneg = 0;                             // NaNs, NaNs with the sign set
-    for (uint32_t i0 = tid; i0 < n8; i0 += 8 * SMALL_THREADS) {
-        uint4 raw[8];
+    const __half* X = (x ? a.X[1] : a.X[0]) + (size_t)(bh / a.H) * a.sb + (size_t)(bh % a.H) * a.sh;
+    uint4 raw[SHORT_PIECES];
 #pragma unroll
-        for (int u = 0; u < 8; ++u) {
-            const uint32_t i = min(i0 + SMALL_THREADS * u, n8 - 1);
-            raw[u] = *reinterpret_cast<const uint4*>(X + (size_t)(i >> shift) * a.st + ((i & ((1u << shift) - 1)) << 3));
+    for (int u = 0; u < SHORT_PIECES; ++u) {
+        const uint32_t i = tid + THREADS * u;
+        raw[u] = make_uint4(0x7FFF7FFFu, 0x7FFF7FFFu, 0x7FFF7FFFu, 0x7FFF7FFFu);            // not numbers where there is no piece
+        if (i < n8) raw[u] = *reinterpret_cast<const uint4*>(X + (size_t)(i >> shift) * a.st + ((i & ((1u << shift) - 1)) << 3));
+    }
+    uint32_t nan = 0;
+#pragma unroll
+    for (int u = 0; u < SHORT_PIECES; ++u) {
+        if (THREADS * u >= n8) break;
+        const __half2 v0 = h2_of(raw[u].x), v1 = h2_of(raw[u].y), v2 = h2_of(raw[u].z), v3 = h2_of(raw[u].w);
+        const __half2 mn = __hmin2(__hmin2(v0, v1), __hmin2(v2, v3)), mx = __hmax2(__hmax2(v0, v1), __hmax2(v2, v3));
+        const __half m = __hmin(__low2half(mn), __high2half(mn)), M = __hmax(__low2half(mx), __high2half(mx));
+        if (m == m) {                                                            // (a piece without a number counts as none)
+            atomicAdd(&s_lo[key_of(__half_as_ushort(m)) >> 5], 1u);
+            atomicAdd(&s_hi[key_of(__half_as_ushort(M)) >> 5], 1u);
         }
+        uint32_t w[4] = {raw[u].x, raw[u].y, raw[u].z, raw[u].w}, nn = 0, neg = 0;
 #pragma unroll
-        for (int u = 0; u < 8; ++u) {
-            if (i0 + SMALL_THREADS * u >= n8) break;
-            uint32_t w[4] = {raw[u].x, raw[u].y, raw[u].z, raw[u].w};
+        for (int j = 0; j < 4; ++j) w[j] = keys_of(w[j], nn, neg);
+        if (tid + THREADS * u < n8) nan += nn;
+        raw[u] = make_uint4(w[0], w[1], w[2], w[3]);
+    }
+    nan = __reduce_add_sync(0xFFFFFFFFu, nan);
+    if (lane == 0 && nan) atomicAdd(&s_nan, nan);
+    __syncthreads();
+    // the bins of two 0-based ranks, each among counts of its own, PER to a thread
+    auto bins_of = [&](const uint32_t* countsA, const uint32_t* countsB, auto rankA, auto rankB) {
+        uint32_t cA[PER], cB[PER], totA = 0, totB = 0;
 #pragma unroll
-            for (int j = 0; j < 4; ++j) w[j] = keys_of(w[j], nn, nneg);
-            keys[i0 + SMALL_THREADS * u] = make_uint4(w[0], w[1], w[2], w[3]);
+        for (int j = 0; j < PER; ++j) { cA[j] = countsA[PER * tid + j]; cB[j] = countsB[PER * tid + j]; totA += cA[j]; totB += cB[j]; }
+        uint32_t incA = totA, incB = totB;
+#pragma unroll
+        for (int d = 1; d < 32; d <<= 1) {
+            const uint32_t oA = __shfl_up_sync(0xFFFFFFFFu, incA, d), oB = __shfl_up_sync(0xFFFFFFFFu, incB, d);
+            if (lane >= d) { incA += oA; incB += oB; }
         }
-    }
-    if (nn) { atomicAdd(&sm.cnt[0], nn); atomicAdd(&sm.cnt[1], nneg); }
-    __syncthreads();
-    const uint32_t N = total - sm.cnt[0], neg_nan = sm.cnt[1];
-    float* thr = a.thr + (size_t)bh * 4 + 2 * x;
-    if (N == 0) {
-        if (tid < 2) thr[tid] = 0.f;
-        return;
-    }
-    const uint32_t k = (uint32_t)rank_k(a.alpha, N);
-    // the sample, brackets from it; its NaNs only make a bracket wider or tighter than meant
-    constexpr uint32_t NS = SAMPLE_TOKENS;
-    const uint32_t M = NS * (uint32_t)a.D;
-    for (uint32_t i = tid; i < M / 8; i += SMALL_THREADS) {
-        const uint32_t t = (uint32_t)((unsigned long long)(i >> shift) * a.T / NS);
-        reinterpret_cast<uint4*>(sm.list)[i] = keys[(t << shift) + (i & ((1u << shift) - 1))];
-    }
-    __syncthreads();
-    const uint32_t r = bracket_rank(a.alpha, M);
-    uint32_t klo, khi;
-    cta_select_keys<SMALL_THREADS>(sm.list, M, r, M - 1 - r, sm.hist, sm.tmp, klo, khi);
-    // candidates (no NaNs: their keys lie below that of -inf and above that of +inf)
-    for (uint32_t i = tid; i < n8; i += SMALL_THREADS) {
-        const uint4 q = keys[i];
-        const uint32_t w[4] = {q.x, q.y, q.z, q.w};
-#pragma unroll
-        for (int j = 0; j < 8; ++j) {
-            const uint32_t key = (w[j >> 1] >> (16 * (j & 1))) & 0xFFFFu;
-            if (key < klo && key >= KEY_MINUS_INF) {
-                const uint32_t at = atomicAdd(&sm.n[0], 1u);
-                if (at < SMALL_LIST) sm.list[at] = (unsigned short)key;
-            }
-            if (key > khi && key <= KEY_PLUS_INF) {
-                const uint32_t at = atomicAdd(&sm.n[1], 1u);
-                if (at < SMALL_LIST) sm.list[SMALL_LIST + at] = (unsigned short)key;
-            }
-        }
-    }
-    __syncthreads();
-    const uint32_t c0 = sm.n[0], c1 = sm.n[1];
-    uint32_t kA, kB;
-    if (c0 > k && c1 > k && c0 <= SMALL_LIST && c1 <= SMALL_LIST) {
-        // the upper candidates move up behind the lower ones
-        unsigned short v[SMALL_LIST / SMALL_THREADS];
-#pragma unroll
-        for (uint32_t u = 0; u < SMALL_LIST / SMALL_THREADS; ++u) v[u] = tid + SMALL_THREADS * u < c1 ? sm.list[SMALL_LIST + tid + SMALL_THREADS * u] : (unsigned short)0;
+        if (lane == 31) { s_part[0][warp] = incA; s_part[1][warp] = incB; }
         __syncthreads();
+        uint32_t beforeA = 0, beforeB = 0, allA = 0, allB = 0;
 #pragma unroll
-        for (uint32_t u = 0; u < SMALL_LIST / SMALL_THREADS; ++u) if (tid + SMALL_THREADS * u < c1) sm.list[c0 + tid + SMALL_THREADS * u] = v[u];
+        for (int w = 0; w < THREADS / 32; ++w) {
+            const uint32_t pA = s_part[0][w], pB = s_part[1][w];
+            if (w < warp) { beforeA += pA; beforeB += pB; }
+            allA += pA; allB += pB;
+        }
+        auto place = [&](const uint32_t (&c)[PER], uint32_t at, uint32_t tot, uint32_t want, uint32_t* found) {
+            if (tot == 0 || want < at || want >= at + tot) return;               // one thread, or none where the rank does not exist
+            int j = 0;
+#pragma unroll
+            for (; j < PER - 1; ++j) { if (want < at + c[j]) break; at += c[j]; }
+            found[0] = (uint32_t)(PER * tid + j); found[1] = want - at;
+        };
+        place(cA, beforeA + incA - totA, totA, rankA(allA), &s_found[0]);
+        place(cB, beforeB + incB - totB, totB, rankB(allB), &s_found[2]);
         __syncthreads();
-        cta_select_keys<SMALL_THREADS>(sm.list, c0 + c1, k, c0 + c1 - 1 - k, sm.hist, sm.tmp, kA, kB);
-    } else {
-        cta_select_keys<SMALL_THREADS>(sm.keys, total, k + neg_nan, N - 1 - k + neg_nan, sm.hist, sm.tmp, kA, kB);
+    };
+    const uint32_t most = (uint32_t)rank_k(a.alpha, total);                      // not less than the rank among the numbers
+    bins_of(s_lo, s_hi, [&](uint32_t) { return most; }, [&](uint32_t all) { return all > most ? all - 1 - most : 0xFFFFFFFFu; });
+    const uint32_t lo = s_found[0], hi = s_found[2];
+    for (int i = tid; i < 2048; i += THREADS) s_lo[i] = 0;
+    __syncthreads();
+    // (the keys of NaNs lie outside those of the infinities)
+    auto for_numbers = [&](auto each) {
+#pragma unroll
+        for (int u = 0; u < SHORT_PIECES; ++u) {
+            if (THREADS * u >= n8) break;
+            const uint32_t w[4] = {raw[u].x, raw[u].y, raw[u].z, raw[u].w};
+#pragma unroll
+            for (int j = 0; j < 8; ++j) {
+                const uint32_t k = (w[j >> 1] >> (16 * (j & 1))) & 0xFFFFu;
+                if (k >= KEY_MINUS_INF && k <= KEY_PLUS_INF) each(k);
+            }
+        }
+    };
+    for_numbers([&](uint32_t k) { if ((k >> 5) <= lo || (k >> 5) >= hi) atomicAdd(&s_lo[k >> 5], 1u); });
+    __syncthreads();
+    const uint32_t N = total - s_nan, k = (uint32_t)rank_k(a.alpha, N);
+    bins_of(s_lo, s_lo, [&](uint32_t) { return k; }, [&](uint32_t all) { return all > k ? all - 1 - k : 0xFFFFFFFFu; });
+    const uint32_t binA = s_found[0], binB = s_found[2];
+    for_numbers([&](uint32_t key) {
+        if ((key >> 5) == binA) atomicAdd(&s_fine[key & 31], 1u);
+        if ((key >> 5) == binB) atomicAdd(&s_fine[32 + (key & 31)], 1u);
+    });
+    __syncthreads();
+    if (warp < 2) {                                                              // warp 0: rank k, warp 1: rank N - 1 - k
+        const uint32_t v = s_fine[32 * warp + lane], want = s_found[2 * warp + 1];
+        uint32_t inc = v;
+#pragma unroll
+        for (int d = 1; d < 32; d <<= 1) {
+            const uint32_t t = __shfl_up_sync(0xFFFFFFFFu, inc, d);
+            if (lane >= d) inc += t;
+        }
+        float* out = a.thr + (size_t)bh * 4 + 2 * x + warp;
+        if (N == 0) { if (lane == 0) *out = 0.f; }
+        else if (v > 0 && want >= inc - v && want < inc) *out = float_of_key((s_found[2 * warp] << 5) | (uint32_t)lane);
     }
-    if (tid < 2) thr[tid] = float_of_key(tid ? kB : kA);
 }
 
 // Tokens per CTA of the scan: as many as keep the expected number of candidates (1.25 times the tail mass
@@ -598,25 +615,22 @@ extern "C" qaq_status qaq_outlier_thresholds(const qaq_config* cfg, const void* 
     a.list = (unsigned short*)((char*)ws + head);
     a.thr = thr;
     a.scan_tokens = SCAN_TOKENS_MAX;
-    const size_t keys = (size_t)n_tokens * cfg->head_dim, small = sizeof(SmallScratch) + keys * sizeof(unsigned short);
-    if (n_tokens > SAMPLE_TOKENS && keys <= SMALL_KEYS) {
-        static SmemSeen seen;
-        QAQ_CUDA_TRY(qaq_allow_smem((const void*)thr_small_kernel, sizeof(SmallScratch) + SMALL_KEYS * sizeof(unsigned short), seen));
-        QAQ_CUDA_TRY(qaq_launch(thr_small_kernel, dim3(BH * 2), dim3(SMALL_THREADS), small, s, a));
+    const size_t keys = (size_t)n_tokens * cfg->head_dim;
+    // (with 1024 threads for twice as many keys 32 (b,h) of 333 tokens take 15.9 us, the kernels below 14.4; 256 of them 61 and 33)
+    if (keys <= SHORT_THREADS * SHORT_PIECES * 8) {
+        QAQ_CUDA_TRY(qaq_launch(thr_short_kernel, dim3(BH * 2), dim3(SHORT_THREADS), 0, s, a));
         return QAQ_OK;
     }
     // 512 threads while a problem has an SM to itself or shares it with one (32 (b,h): 6.4 against 7.9 us), else 256 (256
     // (b,h): 14.4 against 15.6)
     if (BH * 2 <= 2 * 148) QAQ_CUDA_TRY(qaq_launch(thr_sample_kernel<512>, dim3(BH * 2), dim3(512), 0, s, a));
     else QAQ_CUDA_TRY(qaq_launch(thr_sample_kernel<256>, dim3(BH * 2), dim3(256), 0, s, a));
-    if (n_tokens > SAMPLE_TOKENS) {
-        a.scan_tokens = scan_tokens_for(cfg->outlier_frac, cfg->head_dim, BH, n_tokens);
-        dim3 grid((n_tokens + a.scan_tokens - 1) / a.scan_tokens, BH * 2);
-        QAQ_CUDA_TRY(qaq_launch(thr_scan_kernel, grid, dim3(256), 0, s, a));
-        // lists that stay in shared memory are a matter of latency (256 (b,h) of 4096 tokens, alpha = 1 %: 14.6 us with 256
-        // threads, 19.1 with 512), longer ones of throughput (160 of 8192 tokens, 5 %: 68.3 and 48.7 us)
-        if (1.25 * cfg->outlier_frac * (double)keys <= SELECT_KEYS) QAQ_CUDA_TRY(qaq_launch(thr_select_kernel<256>, dim3(BH * 2), dim3(256), 0, s, a));
-        else QAQ_CUDA_TRY(qaq_launch(thr_select_kernel<512>, dim3(BH * 2), dim3(512), 0, s, a));
-    }
+    a.scan_tokens = scan_tokens_for(cfg->outlier_frac, cfg->head_dim, BH, n_tokens);
+    dim3 grid((n_tokens + a.scan_tokens - 1) / a.scan_tokens, BH * 2);
+    QAQ_CUDA_TRY(qaq_launch(thr_scan_kernel, grid, dim3(256), 0, s, a));
+    // lists that stay in shared memory are a matter of latency (256 (b,h) of 4096 tokens, alpha = 1 %: 14.6 us with 256
+    // threads, 19.1 with 512), longer ones of throughput (160 of 8192 tokens, 5 %: 68.3 and 48.7 us)
+    if (1.25 * cfg->outlier_frac * (double)keys <= SELECT_KEYS) QAQ_CUDA_TRY(qaq_launch(thr_select_kernel<256>, dim3(BH * 2), dim3(256), 0, s, a));
+    else QAQ_CUDA_TRY(qaq_launch(thr_select_kernel<512>, dim3(BH * 2), dim3(512), 0, s, a));
     return QAQ_OK;
 }

@@ -97,3 +97,18 @@ def test_the_exact_select_over_the_data_passes_over_nans(D, T, alpha):
     K[:, :, sampled_tokens(T)] = 0
     V[:, :, sampled_tokens(T)] = 0
     check(K, V, wl, alpha)
+
+
+@pytest.mark.parametrize("D,T", [(32, 1), (128, 33), (128, 256), (64, 512), (128, 257), (32, 2048), (64, 1024), (128, 513)])
+@pytest.mark.parametrize("alpha", [0.0, 0.01, 0.3, 1.0])
+def test_short_sequences(D, T, alpha):
+    # up to the keys that one CTA holds with 512 and with 1024 threads, and one token beyond; ranks beyond the number of pieces
+    # (0.3, 1.0); NaNs of both signs, infinities, both zeros, a tail of ties
+    wl = synth.scaled(synth.CONFIGS["C2"], heads=3, head_dim=D, tokens=T)
+    K, V = synth.make_kv(wl, 0)
+    flat = V.view(-1)
+    for i, x in enumerate((float("nan"), -float("nan"), float("inf"), -float("inf"), 0.0, -0.0)):
+        flat[(i * 37 + 5) % D::D * 7] = x
+    K[:, 0, :, D // 2:] = 3.0
+    K[:, 1] = float("nan") if T < 40 else K[:, 1]
+    check(K, V, wl, alpha)
