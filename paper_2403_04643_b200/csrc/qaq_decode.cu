@@ -527,27 +527,30 @@ __device__ void merge_split(const DecArgs& a, DecSmem<D, NQ>& sm, int bh, int nt
 }
 
 // The same for the CTAs of a cluster, which find each other's results in shared memory: query j is put together by CTA
-// j mod cluster; every CTA normalises the scores of its own tiles (from tile_lo to tile_hi).
-__device__ __forceinline__ void cluster_barrier() {
-    asm volatile("barrier.cluster.arrive.release.aligned;\nbarrier.cluster.wait.acquire.aligned;" ::: "memory");
-}
+// j mod cluster; every CTA normalises its share of the scores.
+__device__ __forceinline__ void cluster_arrive() { asm volatile("barrier.cluster.arrive.release.aligned;" ::: "memory"); }
+__device__ __forceinline__ void cluster_wait() { asm volatile("barrier.cluster.wait.acquire.aligned;" ::: "memory"); }
 __device__ __forceinline__ float peer_load(const float* p, int rank) {
     float x;
     asm volatile("{\n.reg .u32 a;\nmapa.shared::cluster.u32 a, %1, %2;\nld.shared::cluster.f32 %0, [a];\n}" : "=f"(x) : "r"(smem_addr(p)), "r"(rank) : "memory");
     return x;
 }
 template <int D, int NQ>
-__device__ __forceinline__ void merge_cluster(const DecArgs& a, DecSmem<D, NQ>& sm, const Group<D, NQ>& gr, int bh, int rank, int tile_lo, int tile_hi, int T) {
+__device__ __forceinline__ void merge_cluster(const DecArgs& a, DecSmem<D, NQ>& sm, const Group<D, NQ>& gr, int bh, int rank, int T, bool kept) {
     using S = Shape<NQ>;
     const float NEG = __int_as_float(0xff800000);
     const int tid = threadIdx.x, lane = tid & 31, ncl = a.cluster;
-    cluster_barrier();
+    float M = NEG, L = 0.f;
+    cluster_arrive();
+    cluster_wait();
 #pragma unroll 1
     for (int j = 0; j < gr.nq; ++j) {
         if (j % ncl != rank && !(NQ == 1 && (a.scores || a.ml))) continue;
         float m = NEG, l = 0.f;
         if (lane < ncl) { m = peer_load(&sm.mm[S::WARPS][j], lane); l = peer_load(&sm.ml[S::WARPS][j], lane); }
-        const float M = warp_max(m), w = m == NEG ? 0.f : __expf(m - M), L = warp_sum(w * l);
+        M = warp_max(m);
+        const float w = m == NEG ? 0.f : __expf(m - M);
+        L = warp_sum(w * l);
         if (j % ncl == rank) {
             float x[8], sum = 0.f;
             const int d = tid < D ? tid : 0;
@@ -558,10 +561,22 @@ __device__ __forceinline__ void merge_cluster(const DecArgs& a, DecSmem<D, NQ>& 
             if (tid < D) gr.out[(size_t)bh * a.out_stride + j * D + tid] = L > 0.f ? sum / L : 0.f;
             if (NQ == 1 && a.ml && tid == 0) { a.ml[2 * bh] = M; a.ml[2 * bh + 1] = L; }
         }
-        if (NQ == 1 && a.scores && !a.ml)
-            normalise_scores<S::THREADS>(a.scores + (size_t)bh * a.scores_stride + tile_lo * QAQ_TILE, min(tile_hi * QAQ_TILE, T) - tile_lo * QAQ_TILE, M, L);
     }
-    cluster_barrier();                  // nobody leaves while its results are being read
+    cluster_arrive();                   // (its second half: nobody leaves while its results are being read)
+    if (NQ == 1 && a.scores && !a.ml) {
+        float* row = a.scores + (size_t)bh * a.scores_stride;
+        const int t = (rank + ncl * (tid >> 5)) * QAQ_TILE + 2 * lane;
+        if (!kept) {                    // a piece of the row, whoever wrote it
+            const int each = (T + ncl - 1) / ncl, lo = min(rank * each, T);
+            normalise_scores<S::THREADS>(row + lo, min(each, T - lo), M, L);
+        } else {
+            const float2 lg = *reinterpret_cast<const float2*>(&sm.ws[tid >> 5].mid[2 * lane]);
+            const float inv = L > 0.f ? 1.0f / L : 0.f;
+            if (t < T) row[t] = __expf(lg.x - M) * inv;
+            if (t + 1 < T) row[t + 1] = __expf(lg.y - M) * inv;
+        }
+    }
+    cluster_wait();
 }
 
 // A CTA's run meets one or two (b,h); it leaves one partial for each, or the result where a (b,h) is one CTA's alone.
@@ -578,6 +593,7 @@ __global__ void __launch_bounds__(Shape<NQ>::THREADS, Shape<NQ>::CTAS_PER_SM) de
     constexpr int MB = D / 16;       // 16-channel row blocks of the value side
     constexpr int NP = (NQ + 1) / 2; // pairs of queries that share an instruction on the value side
     constexpr int CPL = D / 32;      // channels per lane in the outlier sums of the values
+    constexpr int TWO = NQ < 4 ? 2 : 1;      // outlier entries of a lane at a time: their chains of dependent loads run beside each other
     constexpr uint32_t STAGE = WS::STAGE;
     const float NEG = __int_as_float(0xff800000);
     extern __shared__ __align__(16) unsigned char smem_raw[];
@@ -588,51 +604,59 @@ __global__ void __launch_bounds__(Shape<NQ>::THREADS, Shape<NQ>::CTAS_PER_SM) de
     if (lane == 0) { bar_init(smem_addr(ws.bar)); bar_init(smem_addr(ws.bar) + 8); asm volatile("fence.proxy.async.shared::cta;" ::: "memory"); }
     const Group<D, NQ> gr(a);
     qaq_dependency();
-    const int T = COUNTED ? *a.d_count : a.T;
-    if (COUNTED && T < 1) {          // nothing cached: zeros
-        for (int bh = blockIdx.x; bh < a.BH; bh += gridDim.x)
-            if (tid < D) a.out[(size_t)bh * a.out_stride + tid] = 0.f;
-        return;
-    }
-    // this CTA's run of the flattened (b,h, tile) sequence: it begins in bh0 and may reach into bh0 + 1, which begins at f_bound
-    const int ntiles = (T + QAQ_TILE - 1) / QAQ_TILE;
-    const int ncl = CLUSTER ? a.cluster : 1, rank = CLUSTER ? blockIdx.x % ncl : 0;
-    const int run = CLUSTER ? (ntiles + ncl - 1) / ncl : COUNTED ? plan_decode<NQ>(a.BH, ntiles, 1).run : a.run;
-    int flat_lo = blockIdx.x * run, bh0;
-    if constexpr (CLUSTER) {
-        bh0 = blockIdx.x / ncl;
-        flat_lo = bh0 * ntiles + min(rank * run, ntiles);    // the last CTAs of a cluster may find no tiles
-    } else {
-        if (flat_lo >= a.BH * ntiles) return;
-        bh0 = flat_lo / ntiles;
-    }
-    const int f_bound = (bh0 + 1) * ntiles, flat_hi = min(CLUSTER ? f_bound : a.BH * ntiles, flat_lo + run);
-    const int nseg = !CLUSTER && flat_hi > f_bound ? 2 : 1;
-    // this warp's piece of it
-    const int piece = (run + S::WARPS - 1) / S::WARPS;
-    int f = flat_lo + warp * piece;
-    const int f_end = min(f + piece, flat_hi), f_last = min(f_end, flat_hi) - 1;
-    auto bh_of = [&](int i) { return bh0 + (i >= f_bound ? 1 : 0); };
-    const uint32_t buf = smem_addr(ws.buf), bar = smem_addr(ws.bar);
-
-    // ---- tile metadata: the table words (offset and length of the bytes, first entry and length of the outlier list),
-    //      min/max, widths and slots of tokens 2*lane, 2*lane+1; fetched as late as their latency allows
-    //      (a piece that has no tile i fetches its last one again: a load behind a condition would be waited for on the spot)
-    auto fetch_tab = [&](const uint4* tab, int i) {
-        i = min(i, f_last);
-        const int b = bh_of(i);
-        return ldg_now4(tab + ((size_t)b * a.ntiles_max + (i - b * ntiles)));
-    };
+    // Clusters: the warps of a (b,h) take its tiles in turn, so that a warp knows its first tile before it knows how many there are
+    // (counted: their table entries and the count are one wait, not two).
+    const int ncl = CLUSTER ? a.cluster : 1, rank = CLUSTER ? blockIdx.x % ncl : 0, stride = CLUSTER ? ncl * S::WARPS : 1;
+    int T = a.T;
+    if (COUNTED) T = (int)ldg_now1(a.d_count);
+    uint4 tk, tv;
     struct Toks { uint2 mm; uint32_t b; };      // min | max << 16; width | slot << 8 of two tokens
-    auto fetch_toks = [&](const TensorStore& ts, int i) {
-        i = min(i, f_last);
-        const int b = bh_of(i);
-        const size_t t0 = (size_t)b * a.tmax_pad + (i - b * ntiles) * QAQ_TILE + 2 * lane;
+    Toks kt;
+    auto tab_at = [&](const uint4* tab, uint32_t place) { return ldg_now4(tab + place); };
+    auto toks_at = [&](const TensorStore& ts, uint32_t place) {
+        const size_t t0 = (size_t)place * QAQ_TILE + 2 * lane;
         Toks t;
         t.mm = ldg_now2(ts.mnmx + t0);
         t.b = ldg_now1(ts.bs + t0);
         return t;
     };
+    if (CLUSTER) {
+        const uint32_t place = (uint32_t)(blockIdx.x / ncl) * (uint32_t)a.ntiles_max + (uint32_t)min(rank + ncl * warp, a.ntiles_max - 1);
+        tk = tab_at(a.k.tile, place); tv = tab_at(a.v.tile, place); kt = toks_at(a.k, place);
+    }
+    if (COUNTED && T < 1) {          // nothing cached: zeros
+        for (int bh = blockIdx.x; bh < a.BH; bh += gridDim.x)
+            if (tid < D) a.out[(size_t)bh * a.out_stride + tid] = 0.f;
+        return;
+    }
+    // this CTA's run of the flattened (b,h, tile) sequence: it begins in bh0 and may reach into bh0 + 1, which begins at f_bound;
+    // in a cluster the CTA has one (b,h)
+    const int ntiles = (T + QAQ_TILE - 1) / QAQ_TILE;
+    const int run = CLUSTER ? (ntiles + ncl - 1) / ncl : COUNTED ? plan_decode<NQ>(a.BH, ntiles, 1).run : a.run;
+    const int flat_lo = CLUSTER ? 0 : blockIdx.x * run;
+    if (!CLUSTER && flat_lo >= a.BH * ntiles) return;
+    const int bh0 = CLUSTER ? blockIdx.x / ncl : flat_lo / ntiles;
+    const int f_bound = CLUSTER ? ntiles : (bh0 + 1) * ntiles, flat_hi = CLUSTER ? ntiles : min(a.BH * ntiles, flat_lo + run);
+    const int nseg = !CLUSTER && flat_hi > f_bound ? 2 : 1;
+    // a warp that has one tile at most keeps its logits until they can be normalised (through memory: 0.4 us more of a call)
+    const bool kept = CLUSTER && NQ == 1 && a.scores && !a.ml && run <= S::WARPS;
+    // this warp's piece of it
+    const int piece = (run + S::WARPS - 1) / S::WARPS;
+    int f = CLUSTER ? rank + ncl * warp : flat_lo + warp * piece;
+    const int f_end = CLUSTER ? ntiles : min(f + piece, flat_hi), f_last = min(f_end, flat_hi) - 1;
+    auto bh_of = [&](int i) { return bh0 + (!CLUSTER && i >= f_bound ? 1 : 0); };
+    const uint32_t buf = smem_addr(ws.buf), bar = smem_addr(ws.bar);
+
+    // ---- tile metadata: the table words (offset and length of the bytes, first entry and length of the outlier list),
+    //      min/max, widths and slots of tokens 2*lane, 2*lane+1; fetched as late as their latency allows
+    //      (a piece that has no tile i fetches its last one again: a load behind a condition would be waited for on the spot)
+    auto place_of = [&](int i) {
+        i = min(i, f_last);
+        const int b = bh_of(i);
+        return (uint32_t)(CLUSTER ? b * a.ntiles_max + i : b * a.ntiles_max + (i - b * ntiles));
+    };
+    auto fetch_tab = [&](const uint4* tab, int i) { return tab_at(tab, place_of(i)); };
+    auto fetch_toks = [&](const TensorStore& ts, int i) { return toks_at(ts, place_of(i)); };
     // how a tile lies in the buffer: bytes of the tile and of the piece of the outlier list that comes with it (from the
     // 16-byte boundary before its first entry; what lies behind its last one belongs to the read-ahead margin of the
     // list's capacity), both multiples of 16
@@ -652,8 +676,7 @@ __global__ void __launch_bounds__(Shape<NQ>::THREADS, Shape<NQ>::CTAS_PER_SM) de
         }
     };
 
-    uint4 tk = fetch_tab(a.k.tile, f), tv = fetch_tab(a.v.tile, f);
-    Toks kt = fetch_toks(a.k, f);
+    if (!CLUSTER) { tk = fetch_tab(a.k.tile, f); tv = fetch_tab(a.v.tile, f); kt = fetch_toks(a.k, f); }
     // ---- queries of the run's (b,h), by all warps alike: four channels per lane of every query, and the four channels whose
     //      operand word the thread makes; all loads first
     constexpr int WORDS = 64 * P, PER = (2 * WORDS + S::THREADS - 1) / S::THREADS;      // operand words of a (b,h); words per thread
@@ -779,7 +802,7 @@ __global__ void __launch_bounds__(Shape<NQ>::THREADS, Shape<NQ>::CTAS_PER_SM) de
     if (f >= f_end && lane == 0) sm.seg[warp] = -1;
 #pragma unroll 1
     while (f < f_end) {          // once per (b,h) of the warp's piece: one or two times
-    const int bh = bh_of(f), seg = bh - bh0, f_stop = seg ? f_end : min(f_end, f_bound);
+    const int bh = bh_of(f), seg = bh - bh0, f_stop = CLUSTER || seg ? f_end : min(f_end, f_bound);
     float qscale[NQ], qsum[NQ], qtop = NQ == 1 ? 0.f : 2.0f;       // qtop: a bound on the entries of the queries as they are kept
 #pragma unroll
     for (int j = 0; j < NQ; ++j) {
@@ -789,16 +812,16 @@ __global__ void __launch_bounds__(Shape<NQ>::THREADS, Shape<NQ>::CTAS_PER_SM) de
         m_ref[j] = NEG; wunit[j] = 0.f; l_run[j] = 0.f; c_run[j] = 0.f;
     }
 #pragma unroll 1
-    for (; f < f_stop; ++f) {
+    for (; f < f_stop; f += stride) {
         const Lay lk = layout(tk), lv = layout(tv);
         const uint32_t tV = buf + STAGE - lv.nb - lv.lb;
         // the tile before is done with: this tile's values come in behind its keys, if there is room
         const bool besideV = lk.nb + lk.lb + lv.nb + lv.lb <= STAGE;
         if (besideV) stage(tV, lv, a.v, bh, tv, 1);
-        const uint4 tk_next = fetch_tab(a.k.tile, f + 1);
+        const uint4 tk_next = fetch_tab(a.k.tile, f + stride);
         const Toks vt = fetch_toks(a.v, f);
-        const bool has_next = f + 1 < f_end;
-        const int t0 = (f - bh * ntiles) * QAQ_TILE + 2 * lane;              // this lane's tokens: t0 and t0 + 1
+        const bool has_next = f + stride < f_end;
+        const int t0 = (CLUSTER ? f : f - bh * ntiles) * QAQ_TILE + 2 * lane;              // this lane's tokens: t0 and t0 + 1
         const bool val[2] = {t0 < T, t0 + 1 < T};
         int B[2], sl[2];             // width; slot (tokens that are not there: a place nobody reads)
         float step[2], mid[2];
@@ -871,17 +894,20 @@ __global__ void __launch_bounds__(Shape<NQ>::THREADS, Shape<NQ>::CTAS_PER_SM) de
             if (top <= SMALL_MAX) {
                 float inv;
                 fixed_unit(qtop * 2.0f * __half2float(__ushort_as_half((unsigned short)top)), inv, kunit);        // |x - mid| <= 2 top
-                auto add = [&](uint32_t v, bool there) {
-                    int tok; float tm[NQ];
-                    term(v, inv, tok, tm);
+                auto add = [&](const uint32_t* v, uint32_t i) {
+                    int tok[TWO]; float tm[TWO][NQ];
 #pragma unroll
-                    for (int j = 0; j < NQ; ++j) if (there) atomicAdd(&ws.kcorr[j][0][tok], __float2int_rn(tm[j]));
+                    for (int k = 0; k < TWO; ++k) term(v[k], inv, tok[k], tm[k]);
+#pragma unroll
+                    for (int k = 0; k < TWO; ++k)
+#pragma unroll
+                        for (int j = 0; j < NQ; ++j) if (i + 32u * k < sc) atomicAdd(&ws.kcorr[j][0][tok[k]], __float2int_rn(tm[k][j]));
                 };
 #pragma unroll 1
                 for (uint32_t i = 0;;) {
 #pragma unroll
-                    for (int k = 0; k < 4; ++k)
-                        if (i + 32u * k < sc) add(e[k], i + lane + 32u * k < sc);
+                    for (int k = 0; k < 4; k += TWO)
+                        if (i + 32u * k < sc) add(e + k, i + lane + 32u * k);
                     if ((i += 128) >= sc) break;
 #pragma unroll
                     for (int k = 0; k < 4; ++k) e[k] = list[min(i + lane + 32u * k, sc - 1)];
@@ -917,17 +943,18 @@ __global__ void __launch_bounds__(Shape<NQ>::THREADS, Shape<NQ>::CTAS_PER_SM) de
                 const int dot = lo + (B[i] > 4 ? hi << 4 : 0);       // a token that is not there has step 0
                 const float qk = fmaf(qscale[j] * step[i], (float)dot, fmaf(mid[i], qsum[j], kc[i]));
                 lg[j][i] = val[i] ? a.scale * qk : NEG;
-                if (NQ == 1 && a.scores && val[i]) a.scores[(size_t)bh * a.scores_stride + t0 + i] = lg[j][i];
+                if (NQ == 1 && a.scores && !kept && val[i]) a.scores[(size_t)bh * a.scores_stride + t0 + i] = lg[j][i];
             }
+            if (NQ == 1 && kept) *reinterpret_cast<float2*>(&ws.mid[2 * lane]) = make_float2(lg[j][0], lg[j][1]);
         }
         __syncwarp();
         // ---- the front of the buffer is free: start the copy of the next tile's keys (beside this tile's values)
         if (!besideV) stage(tV, lv, a.v, bh, tv, 1);
         const Lay ln = layout(tk_next);
         const bool besideK = ln.nb + ln.lb + lv.nb + lv.lb <= STAGE;
-        if (has_next && besideK) stage(buf, ln, a.k, bh_of(f + 1), tk_next, 0);
-        const uint4 tv_next = fetch_tab(a.v.tile, f + 1);
-        kt = fetch_toks(a.k, f + 1);
+        if (has_next && besideK) stage(buf, ln, a.k, bh_of(f + stride), tk_next, 0);
+        const uint4 tv_next = fetch_tab(a.v.tile, f + stride);
+        kt = fetch_toks(a.k, f + stride);
 
         // ---- p relative to a reference somewhat above the largest logit, which is moved only when a logit exceeds it (so
         //      p never exceeds 1), and value weights p * step as fixed point of up to 28 bits.  (A token's step falls with
@@ -1045,18 +1072,22 @@ __global__ void __launch_bounds__(Shape<NQ>::THREADS, Shape<NQ>::CTAS_PER_SM) de
                 for (int j = 0; j < NQ; ++j)
                     fixed_unit(warp_max(fmaxf(lg[j][0], lg[j][1])) * 2.5f * __half2float(__ushort_as_half((unsigned short)top)), inv[j], unit[j]);
                 __syncwarp();
-                auto add = [&](uint32_t v, bool there) {
+                auto add = [&](const uint32_t* v, uint32_t i) {
+                    int x[TWO][NQ];
 #pragma unroll
-                    for (int j = 0; j < NQ; ++j) {
-                        const int x = __float2int_rn(term(v, j) * inv[j]);
-                        if (there) atomicAdd(&ws.vcorr[j][(v >> 16) & (D - 1)], x);
-                    }
+                    for (int k = 0; k < TWO; ++k)
+#pragma unroll
+                        for (int j = 0; j < NQ; ++j) x[k][j] = __float2int_rn(term(v[k], j) * inv[j]);
+#pragma unroll
+                    for (int k = 0; k < TWO; ++k)
+#pragma unroll
+                        for (int j = 0; j < NQ; ++j) if (i + 32u * k < sc) atomicAdd(&ws.vcorr[j][(v[k] >> 16) & (D - 1)], x[k][j]);
                 };
 #pragma unroll 1
                 for (uint32_t i = 0;;) {
 #pragma unroll
-                    for (int k = 0; k < 4; ++k)
-                        if (i + 32u * k < sc) add(e[k], i + lane + 32u * k < sc);
+                    for (int k = 0; k < 4; k += TWO)
+                        if (i + 32u * k < sc) add(e + k, i + lane + 32u * k);
                     if ((i += 128) >= sc) break;
 #pragma unroll
                     for (int k = 0; k < 4; ++k) e[k] = list[min(i + lane + 32u * k, sc - 1)];
@@ -1096,7 +1127,7 @@ __global__ void __launch_bounds__(Shape<NQ>::THREADS, Shape<NQ>::CTAS_PER_SM) de
             }
         }
         __syncwarp();
-        if (has_next && !besideK) stage(buf, ln, a.k, bh_of(f + 1), tk_next, 0);
+        if (has_next && !besideK) stage(buf, ln, a.k, bh_of(f + stride), tk_next, 0);
         if (!landed) atomicMax(a.status, (int)QAQ_ERR_CUDA);
         phase ^= 1u;
         tk = tk_next;
@@ -1104,7 +1135,7 @@ __global__ void __launch_bounds__(Shape<NQ>::THREADS, Shape<NQ>::CTAS_PER_SM) de
     }
     if (held) flush();
     // ---- what the warp has of this (b,h)
-    const bool cross = f < f_end;                     // it goes on in the next one
+    const bool cross = !CLUSTER && f < f_end;                     // it goes on in the next one
     const int entry = cross ? S::WARPS : warp;
 #pragma unroll
     for (int j = 0; j < NQ; ++j) {
@@ -1152,7 +1183,7 @@ __global__ void __launch_bounds__(Shape<NQ>::THREADS, Shape<NQ>::CTAS_PER_SM) de
         }
     }
     if (CLUSTER) {
-        merge_cluster<D, NQ>(a, sm, gr, bh0, rank, flat_lo - bh0 * ntiles, flat_hi - bh0 * ntiles, T);
+        merge_cluster<D, NQ>(a, sm, gr, bh0, rank, T, kept);
         return;
     }
     __syncthreads();
