@@ -25,7 +25,8 @@
 //   values:  unit 4p + b of a row = byte b of those words for its four tokens: byte i of v_u belongs to slot 4G + i, A and
 //            B as above.  Rows of a list are interleaved by fours (the last m rows of a list by m): unit e of row
 //            4k + t lies at index 16k * head_dim/32 + e * m + t, which makes the loads of a warp contiguous.
-// Storage: a header of QAQ_TILE_HDR bytes (number of rows of every width, byte offsets of the zones below, total), then
+// Storage: a header of QAQ_TILE_HDR bytes (number of rows of every width, byte offsets of the zones below, the largest magnitude
+// among the ranges and the outliers of the tile as a binary16 pattern), then
 // the parts of the sections ordered by unit size so that every load is aligned: zone 4 (main parts of widths 8 .. 4,
 // 16-byte units; then the high part of width 8), zone 2 (high part of width 6, then width 2; 8-byte units), zone 13 (high
 // part of width 7, width 3, high part of width 5, width 1; 12- and 4-byte units).  A tile of keys takes the header plus
@@ -223,9 +224,11 @@ template <int D, bool IS_V> __device__ __forceinline__ uint32_t at_z2(const Tile
 template <int D, bool IS_V> __device__ __forceinline__ uint32_t at_z13(const TileRows& r) { return at_words<D, IS_V>(r, 0x04000200u, 0x08040604u); }
 template <int D, bool IS_V> __device__ __forceinline__ uint32_t tile_total(const TileRows& r) { return at_words<D, IS_V>(r, 0x04030201u, 0x08070605u); }
 template <int D, bool IS_V>
-__device__ __forceinline__ uint4 header_of(const TileRows& r) {
-    return make_uint4(r.nlo, r.nhi, at_h8<D, IS_V>(r) | (at_z2<D, IS_V>(r) << 16), at_z13<D, IS_V>(r) | (tile_total<D, IS_V>(r) << 16));
+__device__ __forceinline__ uint4 header_of(const TileRows& r, uint32_t top) {
+    return make_uint4(r.nlo, r.nhi, at_h8<D, IS_V>(r) | (at_z2<D, IS_V>(r) << 16), at_z13<D, IS_V>(r) | (top << 16));
 }
+// the largest magnitude a range (min | max << 16, binary16) has
+__device__ __forceinline__ uint32_t top_of(uint32_t range) { return max(range & 0x7FFFu, (range >> 16) & 0x7FFFu); }
 // Where a row of width w lies: byte offsets of its main and high part, and for values how far apart its units are (in units).
 struct RowPlace { uint32_t main, high, mm, mh; };
 template <int D, bool IS_V>

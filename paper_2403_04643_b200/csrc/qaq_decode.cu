@@ -375,7 +375,7 @@ __device__ __forceinline__ int v_channel(int mb, int g, int s) {
 // Outlier terms are summed in fixed point.  Where all values of a tile are small (up to 128) one word is enough: a unit
 // is 2^-24 of a bound on the largest term, so that a channel's 64 terms stay inside 32 bits, and a token's 127 (128 have half
 // of the bound: without an inlier the minimum is 0).  The bound of a query's terms is its own, whatever queries share the pass.
-// Otherwise a term is a high part in units of 2^-4 and the exact remainder in units of 2^-28; terms of 2^18 or more (and
+// (The largest value of a tile is in its header.)  Otherwise a term is a high part in units of 2^-4 and the exact remainder in units of 2^-28; terms of 2^18 or more (and
 // non-finite ones) are left out.
 constexpr float OC_LIMIT = 262144.0f;
 __device__ __forceinline__ void wide_add(int* hi_cell, int* lo_cell, float tm) {
@@ -836,12 +836,6 @@ __global__ void __launch_bounds__(Shape<NQ>::THREADS, Shape<NQ>::CTAS_PER_SM) de
                 mid[i] = val[i] ? fmaf(0.5f, step[i], mn) : 0.f;
             }
         };
-        // the largest magnitude among this lane's ranges, as a binary16 pattern (the places of tokens that are not there hold
-        // whatever the cache held before)
-        auto top_range = [&](const Toks& tt) {
-            const uint32_t m = __vmaxu2(val[0] ? tt.mm.x & 0x7FFF7FFFu : 0u, val[1] ? tt.mm.y & 0x7FFF7FFFu : 0u);
-            return max(m & 0xFFFFu, m >> 16);
-        };
         scalars(kt);
         *reinterpret_cast<float2*>(&ws.mid[2 * lane]) = make_float2(mid[0], mid[1]);
 #pragma unroll
@@ -880,17 +874,8 @@ __global__ void __launch_bounds__(Shape<NQ>::THREADS, Shape<NQ>::CTAS_PER_SM) de
 #pragma unroll
                 for (int j = 0; j < NQ; ++j) tm[j] = qv[j] * dx;
             };
-            uint32_t e[4], top = top_range(kt);
-#pragma unroll
-            for (int k = 0; k < 4; ++k) {
-                e[k] = 0;
-                if (lane + 32u * k < sc) e[k] = list[lane + 32 * k];
-                top = max(top, e[k] & 0x7FFFu);
-            }
-#pragma unroll 4
-            for (uint32_t i = lane + 128; i < sc; i += 32) top = max(top, list[i] & 0x7FFFu);
             const uint32_t* all = a.k.outl + (size_t)bh * a.ocap + tk.z;
-            top = sc == oc ? __reduce_max_sync(0xFFFFFFFFu, top) : SMALL_MAX + 1;
+            const uint32_t top = sc == oc ? reinterpret_cast<const uint4*>(ws.buf)->w >> 16 : SMALL_MAX + 1;
             if (top <= SMALL_MAX) {
                 float inv;
                 fixed_unit(qtop * 2.0f * __half2float(__ushort_as_half((unsigned short)top)), inv, kunit);        // |x - mid| <= 2 top
@@ -904,13 +889,11 @@ __global__ void __launch_bounds__(Shape<NQ>::THREADS, Shape<NQ>::CTAS_PER_SM) de
                         for (int j = 0; j < NQ; ++j) if (i + 32u * k < sc) atomicAdd(&ws.kcorr[j][0][tok[k]], __float2int_rn(tm[k][j]));
                 };
 #pragma unroll 1
-                for (uint32_t i = 0;;) {
+                for (uint32_t i = lane; i - lane < sc; i += 32 * TWO) {
+                    uint32_t e[TWO];
 #pragma unroll
-                    for (int k = 0; k < 4; k += TWO)
-                        if (i + 32u * k < sc) add(e + k, i + lane + 32u * k);
-                    if ((i += 128) >= sc) break;
-#pragma unroll
-                    for (int k = 0; k < 4; ++k) e[k] = list[min(i + lane + 32u * k, sc - 1)];
+                    for (int k = 0; k < TWO; ++k) e[k] = list[min(i + 32u * k, sc - 1)];
+                    add(e, i);
                 }
             } else {
                 kunit = -1.0f;
@@ -1053,17 +1036,8 @@ __global__ void __launch_bounds__(Shape<NQ>::THREADS, Shape<NQ>::CTAS_PER_SM) de
             auto clear_vcorr = [&](int rows) {
                 for (int i = 4 * lane; i < rows * D; i += 128) *reinterpret_cast<uint4*>(&ws.vcorr[0][0] + i) = make_uint4(0u, 0u, 0u, 0u);
             };
-            uint32_t e[4], top = top_range(vt);
-#pragma unroll
-            for (int k = 0; k < 4; ++k) {
-                e[k] = 0;
-                if (lane + 32u * k < sc) e[k] = list[lane + 32 * k];
-                top = max(top, e[k] & 0x7FFFu);
-            }
-#pragma unroll 4
-            for (uint32_t i = lane + 128; i < sc; i += 32) top = max(top, list[i] & 0x7FFFu);
             const uint32_t* all = a.v.outl + (size_t)bh * a.ocap + tv.z;
-            top = sc == oc ? __reduce_max_sync(0xFFFFFFFFu, top) : SMALL_MAX + 1;
+            const uint32_t top = sc == oc ? reinterpret_cast<const uint4*>(ws.buf + STAGE - lv.nb - lv.lb)->w >> 16 : SMALL_MAX + 1;
             if (top <= SMALL_MAX) {
                 float inv[NQ], unit[NQ];
                 __syncwarp();
@@ -1084,13 +1058,11 @@ __global__ void __launch_bounds__(Shape<NQ>::THREADS, Shape<NQ>::CTAS_PER_SM) de
                         for (int j = 0; j < NQ; ++j) if (i + 32u * k < sc) atomicAdd(&ws.vcorr[j][(v[k] >> 16) & (D - 1)], x[k][j]);
                 };
 #pragma unroll 1
-                for (uint32_t i = 0;;) {
+                for (uint32_t i = lane; i - lane < sc; i += 32 * TWO) {
+                    uint32_t e[TWO];
 #pragma unroll
-                    for (int k = 0; k < 4; k += TWO)
-                        if (i + 32u * k < sc) add(e + k, i + lane + 32u * k);
-                    if ((i += 128) >= sc) break;
-#pragma unroll
-                    for (int k = 0; k < 4; ++k) e[k] = list[min(i + lane + 32u * k, sc - 1)];
+                    for (int k = 0; k < TWO; ++k) e[k] = list[min(i + 32u * k, sc - 1)];
+                    add(e, i);
                 }
                 __syncwarp();
 #pragma unroll

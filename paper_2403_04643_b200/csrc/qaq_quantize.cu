@@ -115,7 +115,7 @@ struct TileScratch {
     };
     uint32_t range[QAQ_TILE];          // by token: min | max << 16
     alignas(8) uint32_t count[2][2];   // by half of the tile: tokens of every width, a byte each
-    uint32_t nout[2], base[2];         // outliers of the halves; space taken for the tile and for its outlier list
+    uint32_t nout[2], top[2], base[2]; // outliers of the halves, largest magnitudes of their new tokens; space taken for the tile and for its outlier list
     int skip;
 };
 __device__ __forceinline__ uint4 lds4(uint32_t addr) {
@@ -252,7 +252,7 @@ __device__ __forceinline__ void quantize_tile(const QuantArgs& a, TileScratch<D>
     }
     __syncwarp();
     // ---- the outliers go to the warp's list, a token per lane, their places are marked
-    uint32_t nout = 0;
+    uint32_t nout = 0, top = 0;
     if (main) {
         uint32_t ob[P], cnt = 0;
         if constexpr (P == 4) {
@@ -275,7 +275,9 @@ __device__ __forceinline__ void quantize_tile(const QuantArgs& a, TileScratch<D>
                 const uint32_t c = 32 * k + (uint32_t)__ffs(ob[k]) - 1u, U = tid * PR + (c >> 3);
                 ob[k] &= ob[k] - 1;
                 unsigned short* where = reinterpret_cast<unsigned short*>(sm.data + 16 * (U ^ ((U >> 3) & 3))) + (c & 7);
-                if (pos < cap) list[pos] = ((uint32_t)tid << 24) | (c << 16) | *where;
+                const uint32_t x = *where;
+                if (pos < cap) list[pos] = ((uint32_t)tid << 24) | (c << 16) | x;
+                top = max(top, x & 0x7FFFu);
                 *where = (unsigned short)fill;
                 ++pos;
             }
@@ -294,7 +296,8 @@ __device__ __forceinline__ void quantize_tile(const QuantArgs& a, TileScratch<D>
     uint32_t alike = 0;
     if (main) {
         alike = qaqc::count_half(b, lane, sm.count[warp]);
-        if (lane == 0) sm.nout[warp] = nout;
+        top = __reduce_max_sync(0xFFFFFFFFu, fresh ? max(top, qaqc::top_of(range)) : 0u);
+        if (lane == 0) { sm.nout[warp] = nout; sm.top[warp] = top; }
     }
     if (OPEN) asm volatile("cp.async.wait_all;" ::: "memory");
     __syncthreads();
@@ -367,7 +370,9 @@ __device__ __forceinline__ void quantize_tile(const QuantArgs& a, TileScratch<D>
     if (tid == 0) {
         if (stored < nall) atomicMax(a.status, (int)QAQ_ERR_CAPACITY);
         *tab = s_lo ? make_uint4(off, total, tw.z, tw.w + stored) : make_uint4(off, total, obase, stored);
-        *reinterpret_cast<uint4*>(dst) = qaqc::header_of<D, IS_V>(rows);
+        top = max(sm.top[0], sm.top[1]);
+        if (OPEN && s_lo && tw.y) top = max(top, reinterpret_cast<const uint4*>(stored_tile)->w >> 16);
+        *reinterpret_cast<uint4*>(dst) = qaqc::header_of<D, IS_V>(rows, top);
     }
     if (!OPEN || b) ts.bs[mt] = (unsigned short)(b | (slot << 8));
     if (fresh) ts.mnmx[mt] = range;

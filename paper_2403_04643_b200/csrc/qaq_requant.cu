@@ -248,7 +248,7 @@ __device__ __forceinline__ void requantize_tile(const RequantArgs& a, RequantScr
     }
     if (valid && Bn) ts.bs[mt] = (unsigned short)(Bn | (slot << 8));
     if (tid == 0) {
-        *reinterpret_cast<uint4*>(dst) = qaqc::header_of<D, IS_V>(rows);
+        *reinterpret_cast<uint4*>(dst) = qaqc::header_of<D, IS_V>(rows, tw.y ? reinterpret_cast<const uint4*>(sm.old)->w >> 16 : 0u);
         // an open tile that is still the last thing in its pool gives back what it no longer needs:
         // appends continue right behind its bytes
         if (open && noff == tw.x && nb < tw.y && tw.x + tw.y == pool_end) ts.pool_end[bh] = noff + nb;

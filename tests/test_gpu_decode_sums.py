@@ -6,9 +6,10 @@ import math
 import pytest
 import torch
 
+import oracle
 from paper_2403_04643_b200 import qaq, synth
 
-from gpu_helpers import gpu_pipeline, make_inputs
+from gpu_helpers import assert_attention_close, gpu_pipeline, make_inputs, u16
 
 pytestmark = pytest.mark.gpu
 
@@ -142,3 +143,39 @@ def test_an_infinite_logit_gives_zeros_however_the_sequence_is_split(heads, toke
     qaq.qaq_quantize_append(cache, K.cuda(), V.cuda(), thr, bitsK=bits, bitsV=bits)
     out = qaq.qaq_decode_attention_multi(cache, torch.rand((heads, n_q, D), generator=g).half().cuda(), 1 / math.sqrt(D))
     assert (out[0] == 0).all() and torch.isfinite(out).all() and (out[1:] != 0).any(dim=2).all()
+
+
+@pytest.mark.parametrize("D", [32, 64, 128])
+@pytest.mark.parametrize("where", ["old", "new", "outlier", "none"])
+def test_the_largest_value_of_a_tile_that_is_built_in_steps(D, where):
+    # what decides between one and two words per outlier sum is kept with the tile: appended, lowered and raised, a tile gives what
+    # the oracle gives for the final cache, wherever its values beyond 128 are (a token of the first append, of the second, an outlier only)
+    wl = synth.scaled(synth.CONFIGS["C2"], heads=2, head_dim=D, tokens=150, alpha=0.05)
+    K, V, q, ring, nv = make_inputs(wl)
+    if where in ("old", "new"):
+        t = 130 if where == "old" else 145
+        K[:, :, t] *= 400; V[:, :, t] *= 400
+    if where == "outlier":
+        K[:, :, 133, 7] = 3000.0; V[:, :, 133, 9] = -3000.0
+    cfg = qaq.make_config(wl.batch, wl.heads, D, 192, 2, 8, wl.window, wl.alpha)
+    Kd, Vd, qd = K.cuda(), V.cuda(), q.cuda()
+    thr = qaq.qaq_outlier_thresholds(cfg, Kd[:, :, :129], Vd[:, :, :129])
+    cache = qaq.Cache(cfg)
+    high = torch.full((wl.bh, 150), 6, dtype=torch.uint8, device="cuda")
+    for a, b in ((0, 129), (129, 140), (140, 150)):
+        bits = high[:, a:b].contiguous()
+        qaq.qaq_quantize_append(cache, Kd[:, :, a:b], Vd[:, :, a:b], thr, bitsK=bits, bitsV=bits)
+    low = torch.where(torch.arange(150, device="cuda") % 3 == 0, 3, 6).to(torch.uint8).repeat(wl.bh, 1).contiguous()
+    qaq.qaq_requantize_down(cache, bitsK=low, bitsV=low)
+    th = thr.cpu().numpy()
+    u = lambda x: u16(x).reshape(wl.bh, 150, D)
+    for bits in (low, high):
+        if bits is high:
+            qaq.qaq_requantize(cache, Kd, Vd, thr, bitsK=high, bitsV=high)
+        out = qaq.qaq_decode_attention(cache, qd, 1 / math.sqrt(D)).cpu().numpy()
+        for bh in range(wl.bh):
+            b = bits[bh].cpu().numpy()
+            k = oracle.quantize(u(K)[bh], th[bh, 0], th[bh, 1], b)
+            v = oracle.quantize(u(V)[bh], th[bh, 2], th[bh, 3], b)
+            want, _ = oracle.decode(u16(q).reshape(wl.bh, D)[bh], k, v, 1 / math.sqrt(D))
+            assert_attention_close(out[bh], want)
