@@ -69,9 +69,9 @@ __device__ __forceinline__ uint32_t pool_take(uint32_t* pool, uint32_t amount, u
 // 128: 173 us for keys and values, against 323 us; one warp per tile 231 us (as many tiles in flight per SM, for their
 // shared memory); rounds unrolled by two 7 % slower, by four 20 % (the code of one round is what the instruction cache
 // holds); the window in batches of 16 loads 3 % slower, eleven CTAs per SM 3 %.  32 (b,h) of one tile 7.0 against 7.7 us, of 16 tiles 10.5 against 17.2 us.
-// A one-token append is a chain of memory latencies (token count; table and metadata; the tile) and of instructions: four
-// warps share the rounds of pass 2, and nothing but the tile itself waits for the table.  32 (b,h), a tile of 1 to 64
-// tokens: 6.3 us, against 8.4 us with two warps and the window read in two parts, as much as the kernel of 256 threads.
+// A one-token append is a chain of memory latencies (token count; table and metadata; the tile) and of instructions: eight
+// warps share pass 2, a round each, and nothing but the tile itself waits for the table.  32 (b,h), a tile of 1 to 64
+// tokens: 6.0 us, 6.3 with four warps, 8.4 with two and the window read in two parts.
 // The integer unit limits this kernel (compares, minima, byte shuffles and selects all run there, at half rate), so sums,
 // shifts and packing are put where the multipliers are.
 __device__ __forceinline__ uint64_t pair_of(float a, float b) {
@@ -164,7 +164,7 @@ __device__ __forceinline__ uint32_t prefix(uint32_t x, int lane, uint32_t& sum) 
     sum = __shfl_sync(0xFFFFFFFFu, inc, 31);
     return inc - x;
 }
-constexpr int OPEN_WARPS = 4;           // warps of a CTA with an open tile
+constexpr int OPEN_WARPS = 8;           // warps of a CTA with an open tile
 constexpr uint32_t STORED = 1u << 30;   // of a slot's last word: the token is taken from the stored tile
 
 // One tile of one tensor, by two warps: half of its tokens each until the widths are known, half of the slots each from there.
@@ -475,7 +475,7 @@ __device__ __forceinline__ void quantize_tile(const QuantArgs& a, TileScratch<D>
 
 // dynamic shared memory: the scratch, the tile as it is stored (OPEN), the warps' lists of outliers
 template <int D, bool OPEN>
-__global__ void __launch_bounds__(OPEN ? 32 * OPEN_WARPS : 64, OPEN ? 4 : (12)) quant_tiles_kernel(const QuantArgs a, uint32_t cap) {
+__global__ void __launch_bounds__(OPEN ? 32 * OPEN_WARPS : 64, OPEN ? 2 : (12)) quant_tiles_kernel(const QuantArgs a, uint32_t cap) {
     extern __shared__ __align__(64) unsigned char tiles_smem[];
     TileScratch<D>& sm = *reinterpret_cast<TileScratch<D>*>(tiles_smem);
     uint8_t* stored_tile = tiles_smem + sizeof(TileScratch<D>);
