@@ -235,9 +235,13 @@ struct DecSmem {
     alignas(16) uint32_t qw[2][2][32][D / 32];// operand words of q per lane: low nibbles of its words, high nibbles
     float qscale[2][NQ], qsum[2][NQ];
     // results of the warps; the warp that meets the (b,h) boundary leaves what it has of the first one in entry W
-    float cross[NQ][D];
+    union {
+        float cross[NQ][D];
+        float from_sum[8][D];                 // clusters, where no warp meets a boundary: what the CTAs send (see merge_cluster), and nothing else
+    };
     float mm[W + 1][NQ], ml[W + 1][NQ], cs[W + 1][NQ];
     int seg[W + 1];                           // which of the two (b,h) an entry belongs to, -1: none
+    float2 from_ml[NQ][8];                    // likewise
     int last[2];
 };
 
@@ -526,14 +530,17 @@ __device__ void merge_split(const DecArgs& a, DecSmem<D, NQ>& sm, int bh, int nt
     }
 }
 
-// The same for the CTAs of a cluster, which find each other's results in shared memory: query j is put together by CTA
-// j mod cluster; every CTA normalises its share of the scores.
+// The same for the CTAs of a cluster, which send their results to each other's shared memory before they meet at the cluster barrier:
+// query j is put together by CTA j mod cluster, which gets its sums; (max, sum of p) go to all.  After the barrier everything is local,
+// and a CTA can leave without waiting for the others.  (Results left in place, read by the peers after the barrier, a second barrier before anybody
+// leaves: 1 us more of a call.)  Every CTA normalises its share of the scores.
 __device__ __forceinline__ void cluster_arrive() { asm volatile("barrier.cluster.arrive.release.aligned;" ::: "memory"); }
 __device__ __forceinline__ void cluster_wait() { asm volatile("barrier.cluster.wait.acquire.aligned;" ::: "memory"); }
-__device__ __forceinline__ float peer_load(const float* p, int rank) {
-    float x;
-    asm volatile("{\n.reg .u32 a;\nmapa.shared::cluster.u32 a, %1, %2;\nld.shared::cluster.f32 %0, [a];\n}" : "=f"(x) : "r"(smem_addr(p)), "r"(rank) : "memory");
-    return x;
+__device__ __forceinline__ void peer_store(const float* p, int rank, float x) {
+    asm volatile("{\n.reg .u32 a;\nmapa.shared::cluster.u32 a, %0, %1;\nst.shared::cluster.f32 [a], %2;\n}" ::"r"(smem_addr(p)), "r"(rank), "f"(x) : "memory");
+}
+__device__ __forceinline__ void peer_store(const float2* p, int rank, float x, float y) {
+    asm volatile("{\n.reg .u32 a;\nmapa.shared::cluster.u32 a, %0, %1;\nst.shared::cluster.v2.f32 [a], {%2, %3};\n}" ::"r"(smem_addr(p)), "r"(rank), "f"(x), "f"(y) : "memory");
 }
 template <int D, int NQ>
 __device__ __forceinline__ void merge_cluster(const DecArgs& a, DecSmem<D, NQ>& sm, const Group<D, NQ>& gr, int bh, int rank, int T, bool kept) {
@@ -547,7 +554,7 @@ __device__ __forceinline__ void merge_cluster(const DecArgs& a, DecSmem<D, NQ>& 
     for (int j = 0; j < gr.nq; ++j) {
         if (j % ncl != rank && !(NQ == 1 && (a.scores || a.ml))) continue;
         float m = NEG, l = 0.f;
-        if (lane < ncl) { m = peer_load(&sm.mm[S::WARPS][j], lane); l = peer_load(&sm.ml[S::WARPS][j], lane); }
+        if (lane < ncl) { const float2 ml = sm.from_ml[j][lane]; m = ml.x; l = ml.y; }
         M = warp_max(m);
         const float w = m == NEG ? 0.f : __expf(m - M);
         L = warp_sum(w * l);
@@ -555,14 +562,13 @@ __device__ __forceinline__ void merge_cluster(const DecArgs& a, DecSmem<D, NQ>& 
             float x[8], sum = 0.f;
             const int d = tid < D ? tid : 0;
 #pragma unroll
-            for (int i = 0; i < 8; ++i) x[i] = i < ncl ? peer_load(&sm.cross[j][d], i) : 0.f;
+            for (int i = 0; i < 8; ++i) x[i] = i < ncl ? sm.from_sum[j / ncl * ncl + i][d] : 0.f;
 #pragma unroll
             for (int i = 0; i < 8; ++i) sum = fmaf(__shfl_sync(0xFFFFFFFFu, w, i), x[i], sum);
             if (tid < D) gr.out[(size_t)bh * a.out_stride + j * D + tid] = L > 0.f ? sum / L : 0.f;
             if (NQ == 1 && a.ml && tid == 0) { a.ml[2 * bh] = M; a.ml[2 * bh + 1] = L; }
         }
     }
-    cluster_arrive();                   // (its second half: nobody leaves while its results are being read)
     if (NQ == 1 && a.scores && !a.ml) {
         float* row = a.scores + (size_t)bh * a.scores_stride;
         const int t = (rank + ncl * (tid >> 5)) * QAQ_TILE + 2 * lane;
@@ -576,7 +582,6 @@ __device__ __forceinline__ void merge_cluster(const DecArgs& a, DecSmem<D, NQ>& 
             if (t + 1 < T) row[t + 1] = __expf(lg.y - M) * inv;
         }
     }
-    cluster_wait();
 }
 
 // A CTA's run meets one or two (b,h); it leaves one partial for each, or the result where a (b,h) is one CTA's alone.
@@ -629,6 +634,8 @@ __global__ void __launch_bounds__(Shape<NQ>::THREADS, Shape<NQ>::CTAS_PER_SM) de
             if (tid < D) a.out[(size_t)bh * a.out_stride + tid] = 0.f;
         return;
     }
+    __syncwarp();
+    if (CLUSTER) cluster_arrive();
     // this CTA's run of the flattened (b,h, tile) sequence: it begins in bh0 and may reach into bh0 + 1, which begins at f_bound;
     // in a cluster the CTA has one (b,h)
     const int ntiles = (T + QAQ_TILE - 1) / QAQ_TILE;
@@ -679,8 +686,9 @@ __global__ void __launch_bounds__(Shape<NQ>::THREADS, Shape<NQ>::CTAS_PER_SM) de
     if (!CLUSTER) { tk = fetch_tab(a.k.tile, f); tv = fetch_tab(a.v.tile, f); kt = fetch_toks(a.k, f); }
     // ---- queries of the run's (b,h), by all warps alike: four channels per lane of every query, and the four channels whose
     //      operand word the thread makes; all loads first
-    constexpr int WORDS = 64 * P, PER = (2 * WORDS + S::THREADS - 1) / S::THREADS;      // operand words of a (b,h); words per thread
-    uint2 qrow[2][NQ], qword[PER];
+    constexpr int SEGS = CLUSTER ? 1 : 2;
+    constexpr int WORDS = 64 * P, PER = (SEGS * WORDS + S::THREADS - 1) / S::THREADS;   // operand words of a (b,h); words per thread
+    uint2 qrow[SEGS][NQ], qword[PER];
     const bool q_aligned = ((uintptr_t)a.q & 7) == 0 && (a.q_stride & 3) == 0;
     auto load4 = [&](const __half* p) {
         if (q_aligned) return *reinterpret_cast<const uint2*>(p);
@@ -688,7 +696,7 @@ __global__ void __launch_bounds__(Shape<NQ>::THREADS, Shape<NQ>::CTAS_PER_SM) de
         return make_uint2(h[0] | (uint32_t)h[1] << 16, h[2] | (uint32_t)h[3] << 16);
     };
 #pragma unroll
-    for (int sg = 0; sg < 2; ++sg)
+    for (int sg = 0; sg < SEGS; ++sg)
 #pragma unroll
         for (int j = 0; j < NQ; ++j) {
             qrow[sg][j] = make_uint2(0u, 0u);
@@ -716,9 +724,9 @@ __global__ void __launch_bounds__(Shape<NQ>::THREADS, Shape<NQ>::CTAS_PER_SM) de
     }
     for (int i = 4 * lane; i < NQ * D; i += 128) *reinterpret_cast<float4*>(&ws.macc[0][0] + i) = make_float4(0.f, 0.f, 0.f, 0.f);
     auto half_at = [](const uint2& v, int i) { return __half2float(__ushort_as_half((unsigned short)((i < 2 ? v.x : v.y) >> (16 * (i & 1))))); };
-    float qsc[2][NQ];
+    float qsc[SEGS][NQ];
 #pragma unroll
-    for (int sg = 0; sg < 2; ++sg)
+    for (int sg = 0; sg < SEGS; ++sg)
 #pragma unroll
         for (int j = 0; j < NQ; ++j) {
             float qmax = 0.f, qs = 0.f;
@@ -745,7 +753,7 @@ __global__ void __launch_bounds__(Shape<NQ>::THREADS, Shape<NQ>::CTAS_PER_SM) de
         word_of(tid + k * S::THREADS, sg, ln, r, ch);
         float sc = 0.f;
 #pragma unroll
-        for (int j = 0; j < NQ; ++j) if ((ln >> 3) == j) sc = sg ? qsc[1][j] : qsc[0][j];
+        for (int j = 0; j < NQ; ++j) if ((ln >> 3) == j) sc = sg ? qsc[SEGS - 1][j] : qsc[0][j];
         const float qinv = sc > 0.f ? 1.0f / sc : 0.f;
         uint32_t v = 0;
 #pragma unroll
@@ -758,7 +766,8 @@ __global__ void __launch_bounds__(Shape<NQ>::THREADS, Shape<NQ>::CTAS_PER_SM) de
         if (sg < nseg) sm.qw[sg][r & 1][ln][r >> 1] = v;
     }
     if (tid == 0) sm.seg[S::WARPS] = -1;
-    for (int i = tid; i < NQ * D; i += S::THREADS) (&sm.cross[0][0])[i] = 0.f;
+    if (!CLUSTER)
+        for (int i = tid; i < NQ * D; i += S::THREADS) (&sm.cross[0][0])[i] = 0.f;
     __syncthreads();
 
     // digit rows of the value weights this lane feeds: columns 0..3 of the first query of a pair, 4..7 of the second
@@ -1122,6 +1131,7 @@ __global__ void __launch_bounds__(Shape<NQ>::THREADS, Shape<NQ>::CTAS_PER_SM) de
     __syncwarp();
     }
     __syncthreads();
+    if (CLUSTER) cluster_wait();         // (all CTAs of the cluster run: what follows writes to them)
     // ---- merge the warps (log-sum-exp) into the partials of the (b,h): lane i knows the weight of entry i
 #pragma unroll 1
     for (int seg = 0; seg < nseg; ++seg) {
@@ -1137,7 +1147,7 @@ __global__ void __launch_bounds__(Shape<NQ>::THREADS, Shape<NQ>::CTAS_PER_SM) de
             const int d = tid < D ? tid : 0;
 #pragma unroll
             for (int i = 0; i < S::WARPS; ++i) x = fmaf(__shfl_sync(0xFFFFFFFFu, wgt, i), sm.ws[i].macc[j][d], x);
-            x = fmaf(__shfl_sync(0xFFFFFFFFu, wgt, S::WARPS), sm.cross[j][d], x);
+            if (!CLUSTER) x = fmaf(__shfl_sync(0xFFFFFFFFu, wgt, S::WARPS), sm.cross[j][d], x);
             float* dst = gr.part + ((size_t)(2 * blockIdx.x + seg) * NQ + j) * (D + 4);
             if (alone) {
                 if (tid < D) gr.out[(size_t)bh * a.out_stride + j * D + tid] = L > 0.f ? x / L : 0.f;
@@ -1145,9 +1155,9 @@ __global__ void __launch_bounds__(Shape<NQ>::THREADS, Shape<NQ>::CTAS_PER_SM) de
                     if (a.ml && tid == 0) { a.ml[2 * bh] = M; a.ml[2 * bh + 1] = L; }
                     if (a.scores && !a.ml) normalise_scores<S::THREADS>(a.scores + (size_t)bh * a.scores_stride, T, M, L);
                 }
-            } else if (CLUSTER) {          // (entry W is free: no warp crosses into another (b,h))
-                if (tid < D) sm.cross[j][tid] = x;
-                if (tid == 0) { sm.mm[S::WARPS][j] = M; sm.ml[S::WARPS][j] = L; }
+            } else if (CLUSTER) {
+                if (tid < D) peer_store(&sm.from_sum[j / ncl * ncl + rank][tid], j % ncl, x);
+                if (tid < ncl) peer_store(&sm.from_ml[j][rank], tid, M, L);
             } else {
                 if (tid < D) __stcg(dst + tid, x);
                 if (tid == 0) __stcg(reinterpret_cast<float2*>(dst + D), make_float2(M, L));
