@@ -437,12 +437,15 @@ __global__ void __launch_bounds__(THREADS) thr_select_kernel(const ThrArgs a) {
 // A key among the k + 1 smallest is not above the (k + 1)-th smallest of the pieces' minima (a piece: eight keys), so the minima
 // and the maxima give a bin of 32 keys for either tail; the keys up to the one and from the other on are counted by bins, which
 // gives the bin of each rank, and a second count, of the keys inside these two bins, the keys themselves.  Nothing is guessed, there
-// is no other path to fall back to.  What bounds it: the latency of one load after the other step.  32 (b,h) of 100 tokens 13.2 us
-// with a sample, brackets from it and lists of candidates, 7.8 this way; 256 of 100 22.5 and 21.4; 64 of 400, head_dim 64, 15.5 and 10.9.  (The keys of a problem spread over a thread-block cluster, whose
-// counts meet in distributed shared memory: 32 (b,h) of 1000 tokens 25 to 36 us, the three kernels above 19.)
-constexpr int SHORT_THREADS = 512, SHORT_PIECES = 8;                             // pieces of a thread
-__global__ void __launch_bounds__(SHORT_THREADS, 2) thr_short_kernel(const ThrArgs a) {
+// is no other path to fall back to.  What bounds it: one step after the other, by 16 warps.  32 (b,h) of 100 tokens 13.2 us with a sample,
+// brackets from it and lists of candidates, 7.8 with every key tested against the bins in both counts, 6.0 with a mask of what lies in
+// them; 256 of 100 tokens 22.5, 21.4, 16.0; 64 of 400, head_dim 64, 15.5, 10.9, 7.3.  (The keys of a problem spread over a thread-block
+// cluster, whose counts meet in distributed shared memory: 32 (b,h) of 1000 tokens 25 to 36 us, the three kernels above 19.)
+constexpr int SHORT_THREADS = 512;
+template <int PIECES>                                                            // of a thread
+__global__ void __launch_bounds__(SHORT_THREADS, PIECES > 8 ? 1 : 2) thr_short_kernel(const ThrArgs a) {
     constexpr int THREADS = SHORT_THREADS;
+    static_assert(PIECES <= 16, "eight bits for each");
     constexpr int PER = 2048 / THREADS;                                          // bins of a thread
     __shared__ uint32_t s_lo[2048], s_hi[2048];                                  // counts by the upper 11 bits of the key: minima, maxima; then s_lo: keys
     __shared__ uint32_t s_fine[64], s_nan, s_part[2][32], s_found[4];            // counts by the lower 5 bits; NaNs
@@ -455,16 +458,16 @@ __global__ void __launch_bounds__(SHORT_THREADS, 2) thr_short_kernel(const ThrAr
     const int shift = 31 - __clz(a.D / 8);                                       // pieces of a token
     const uint32_t total = (uint32_t)a.T * (uint32_t)a.D, n8 = total / 8;
     const __half* X = (x ? a.X[1] : a.X[0]) + (size_t)(bh / a.H) * a.sb + (size_t)(bh % a.H) * a.sh;
-    uint4 raw[SHORT_PIECES];
+    uint4 raw[PIECES];
 #pragma unroll
-    for (int u = 0; u < SHORT_PIECES; ++u) {
+    for (int u = 0; u < PIECES; ++u) {
         const uint32_t i = tid + THREADS * u;
         raw[u] = make_uint4(0x7FFF7FFFu, 0x7FFF7FFFu, 0x7FFF7FFFu, 0x7FFF7FFFu);            // not numbers where there is no piece
         if (i < n8) raw[u] = *reinterpret_cast<const uint4*>(X + (size_t)(i >> shift) * a.st + ((i & ((1u << shift) - 1)) << 3));
     }
     uint32_t nan = 0;
 #pragma unroll
-    for (int u = 0; u < SHORT_PIECES; ++u) {
+    for (int u = 0; u < PIECES; ++u) {
         if (THREADS * u >= n8) break;
         const __half2 v0 = h2_of(raw[u].x), v1 = h2_of(raw[u].y), v2 = h2_of(raw[u].z), v3 = h2_of(raw[u].w);
         const __half2 mn = __hmin2(__hmin2(v0, v1), __hmin2(v2, v3)), mx = __hmax2(__hmax2(v0, v1), __hmax2(v2, v3));
@@ -473,11 +476,11 @@ __global__ void __launch_bounds__(SHORT_THREADS, 2) thr_short_kernel(const ThrAr
             atomicAdd(&s_lo[key_of(__half_as_ushort(m)) >> 5], 1u);
             atomicAdd(&s_hi[key_of(__half_as_ushort(M)) >> 5], 1u);
         }
-        uint32_t w[4] = {raw[u].x, raw[u].y, raw[u].z, raw[u].w}, nn = 0, neg = 0;
-#pragma unroll
-        for (int j = 0; j < 4; ++j) w[j] = keys_of(w[j], nn, neg);
-        if (tid + THREADS * u < n8) nan += nn;
-        raw[u] = make_uint4(w[0], w[1], w[2], w[3]);
+        const __half2 sum = __hmin2_nan(__hmin2_nan(v0, v1), __hmin2_nan(v2, v3));
+        if (!__hbeq2(sum, sum) && tid + THREADS * u < n8) {                      // a NaN among them
+            uint32_t neg = 0;
+            (void)keys_of(raw[u].x, nan, neg); (void)keys_of(raw[u].y, nan, neg); (void)keys_of(raw[u].z, nan, neg); (void)keys_of(raw[u].w, nan, neg);
+        }
     }
     nan = __reduce_add_sync(0xFFFFFFFFu, nan);
     if (lane == 0 && nan) atomicAdd(&s_nan, nan);
@@ -518,25 +521,42 @@ __global__ void __launch_bounds__(SHORT_THREADS, 2) thr_short_kernel(const ThrAr
     const uint32_t lo = s_found[0], hi = s_found[2];
     for (int i = tid; i < 2048; i += THREADS) s_lo[i] = 0;
     __syncthreads();
-    // (the keys of NaNs lie outside those of the infinities)
-    auto for_numbers = [&](auto each) {
+    // what lies in these bins or beyond, as values (NaNs compare false; a zero of the other sign may come along, which changes no rank)
+    const __half2 lo2 = __half2half2(__ushort_as_half(half_of_key(min((lo << 5) | 31u, KEY_PLUS_INF)))), hi2 = __half2half2(__ushort_as_half(half_of_key(max(hi << 5, KEY_MINUS_INF))));
+    uint32_t set[(PIECES + 3) / 4];                                              // eight bits a piece: bit 2j + h is half h of word j
 #pragma unroll
-        for (int u = 0; u < SHORT_PIECES; ++u) {
+    for (int i = 0; i < (PIECES + 3) / 4; ++i) set[i] = 0;
+#pragma unroll
+    for (int u = 0; u < PIECES; ++u) {
+        if (THREADS * u >= n8) break;
+        const uint32_t w[4] = {raw[u].x, raw[u].y, raw[u].z, raw[u].w};
+        uint32_t m = 0;
+#pragma unroll
+        for (int j = 0; j < 4; ++j) {
+            const uint32_t out = __hle2_mask(h2_of(w[j]), lo2) | __hge2_mask(h2_of(w[j]), hi2);
+            m |= (out & 0x00010001u) << (2 * j);
+        }
+        set[u >> 2] |= ((m | (m >> 15)) & 0xFFu) << (8 * (u & 3));
+    }
+    auto for_set = [&](auto each) {
+#pragma unroll
+        for (int u = 0; u < PIECES; ++u) {
             if (THREADS * u >= n8) break;
-            const uint32_t w[4] = {raw[u].x, raw[u].y, raw[u].z, raw[u].w};
-#pragma unroll
-            for (int j = 0; j < 8; ++j) {
-                const uint32_t k = (w[j >> 1] >> (16 * (j & 1))) & 0xFFFFu;
-                if (k >= KEY_MINUS_INF && k <= KEY_PLUS_INF) each(k);
+            uint32_t m = (set[u >> 2] >> (8 * (u & 3))) & 0xFFu;
+            while (m) {
+                const int bit = __ffs(m) - 1;
+                m &= m - 1;
+                const uint32_t a01 = (bit & 2) ? raw[u].y : raw[u].x, a23 = (bit & 2) ? raw[u].w : raw[u].z, w = (bit & 4) ? a23 : a01;
+                each(key_of((unsigned short)((bit & 1) ? w >> 16 : w & 0xFFFFu)));
             }
         }
     };
-    for_numbers([&](uint32_t k) { if ((k >> 5) <= lo || (k >> 5) >= hi) atomicAdd(&s_lo[k >> 5], 1u); });
+    for_set([&](uint32_t k) { atomicAdd(&s_lo[k >> 5], 1u); });
     __syncthreads();
     const uint32_t N = total - s_nan, k = (uint32_t)rank_k(a.alpha, N);
     bins_of(s_lo, s_lo, [&](uint32_t) { return k; }, [&](uint32_t all) { return all > k ? all - 1 - k : 0xFFFFFFFFu; });
     const uint32_t binA = s_found[0], binB = s_found[2];
-    for_numbers([&](uint32_t key) {
+    for_set([&](uint32_t key) {
         if ((key >> 5) == binA) atomicAdd(&s_fine[key & 31], 1u);
         if ((key >> 5) == binB) atomicAdd(&s_fine[32 + (key & 31)], 1u);
     });
@@ -616,9 +636,14 @@ extern "C" qaq_status qaq_outlier_thresholds(const qaq_config* cfg, const void* 
     a.thr = thr;
     a.scan_tokens = SCAN_TOKENS_MAX;
     const size_t keys = (size_t)n_tokens * cfg->head_dim;
-    // (with 1024 threads for twice as many keys 32 (b,h) of 333 tokens take 15.9 us, the kernels below 14.4; 256 of them 61 and 33)
-    if (keys <= SHORT_THREADS * SHORT_PIECES * 8) {
-        QAQ_CUDA_TRY(qaq_launch(thr_short_kernel, dim3(BH * 2), dim3(SHORT_THREADS), 0, s, a));
+    // 32768 keys, two CTAs to an SM; twice as many while every problem has an SM to itself (32 (b,h) of 333 tokens 10.4 us, 13.4 by the
+    // kernels below; 256 of them 38.7 and 31.0)
+    if (keys <= SHORT_THREADS * 8 * 8) {
+        QAQ_CUDA_TRY(qaq_launch(thr_short_kernel<8>, dim3(BH * 2), dim3(SHORT_THREADS), 0, s, a));
+        return QAQ_OK;
+    }
+    if (keys <= SHORT_THREADS * 16 * 8 && BH * 2 <= 148) {
+        QAQ_CUDA_TRY(qaq_launch(thr_short_kernel<16>, dim3(BH * 2), dim3(SHORT_THREADS), 0, s, a));
         return QAQ_OK;
     }
     // 512 threads while a problem has an SM to itself or shares it with one (32 (b,h): 6.4 against 7.9 us), else 256 (256
