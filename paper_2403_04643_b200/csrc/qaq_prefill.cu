@@ -42,6 +42,7 @@ struct PrefillArgs {
     float* qnorm2;       // [BH][n] or null
     float2* part;        // [BH][nchunk][n] (reference, sum of powers of two relative to it) of the visible logits of a chunk
     int nchunk, tiles;   // chunks of a (b,h); tiles of a chunk, or of a CTA of a cluster
+    int each_head, each_batch;   // 1, or 0 where all heads (batch elements) share their keys
 };
 
 // ONE_PASS: the CTAs of a cluster share a (b,h) and keep its logits in tensor memory until they have the statistics of its rows.
@@ -228,7 +229,7 @@ __global__ void __launch_bounds__(PW_THREADS, 1) window_kernel(const __grid_cons
 #pragma unroll
                     for (int r = 0; r < W::REGIONS; ++r) {
                         if (k == 0) bulk_rows(s_q + (it & 1) * W::QUERY_BYTES + r * (NC * W::ROW_BYTES), &queries, 64 * r, o.bh * a.n, bar);
-                        bulk_tile(base + st * W::TILE_BYTES + r * (PW_TILE * W::ROW_BYTES), &keys, 64 * r, (o.tile + k) * PW_TILE, o.bh % a.H, o.bh / a.H, bar);
+                        bulk_tile(base + st * W::TILE_BYTES + r * (PW_TILE * W::ROW_BYTES), &keys, 64 * r, (o.tile + k) * PW_TILE, o.bh % a.H * a.each_head, o.bh / a.H * a.each_batch, bar);
                     }
                 }
             }
@@ -506,7 +507,7 @@ __global__ void __launch_bounds__(128 * PS_TILES, 1) window_short_kernel(const P
         float v[CW];
         load_acc(acc + ((uint32_t)(32 * (warp & 3)) << 16) + group * NC + h, v);
 #pragma unroll
-        for (int c = 0; c < CW; ++c) x[h + c] = v[c] * sc;
+        for (int c = 0; c < CW; ++c) x[h + c] = v[c];
     }
     if (!ok)
 #pragma unroll
@@ -521,8 +522,8 @@ __global__ void __launch_bounds__(128 * PS_TILES, 1) window_short_kernel(const P
 #pragma unroll
         for (int c = 0; c < 8; ++c) {
             const bool seen = c0 + c >= hidden;
-            m[c] = warp_max(seen ? x[c0 + c] : NEG);
-            sum[c] = x[c0 + c] = seen ? pow2(x[c0 + c] - m[c]) : 0.f;
+            m[c] = warp_max(seen ? x[c0 + c] * sc : NEG);
+            sum[c] = x[c0 + c] = seen ? pow2(fmaf(x[c0 + c], sc, -m[c])) : 0.f;
         }
         if (lane == 0) {
             *reinterpret_cast<float4*>(&s_max[warp][c0]) = make_float4(m[0], m[1], m[2], m[3]);
@@ -606,7 +607,10 @@ qaq_status run_window(PrefillArgs a, const void* K, long sb, long sh, long st, i
     if (tiles <= PS_TILES) return run_short<D, NC>(a, K, sb, sh, st, tiles, 1, s);
     CUtensorMap keys, queries;
     const cuuint32_t inner = D >= 64 ? 64 : 32;
-    const cuuint64_t ksize[4] = {(cuuint64_t)D, (cuuint64_t)a.T, (cuuint64_t)a.H, (cuuint64_t)batch}, kstride[3] = {2ull * st, 2ull * sh, 2ull * sb};
+    // (a stride of zero is a dimension of one in the description; the stride of such a dimension is never used)
+    a.each_head = sh && a.H > 1; a.each_batch = sb && batch > 1;
+    const cuuint64_t ksize[4] = {(cuuint64_t)D, (cuuint64_t)a.T, (cuuint64_t)(a.each_head ? a.H : 1), (cuuint64_t)(a.each_batch ? batch : 1)};
+    const cuuint64_t kstride[3] = {2ull * st, 2ull * (a.each_head ? sh : st), 2ull * (a.each_batch ? sb : st)};
     const cuuint64_t qsize[2] = {(cuuint64_t)D, (cuuint64_t)a.BH * a.n}, qstride[1] = {2ull * D};
     const cuuint32_t kbox[4] = {inner, PW_TILE, 1, 1}, qbox[2] = {inner, NC};
     if (!describe(&keys, K, 4, ksize, kstride, kbox, D) || !describe(&queries, a.Q, 2, qsize, qstride, qbox, D)) return QAQ_ERR_CUDA;
