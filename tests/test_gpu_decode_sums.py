@@ -157,7 +157,7 @@ def test_the_largest_value_of_a_tile_that_is_built_in_steps(D, where):
         K[:, :, t] *= 400; V[:, :, t] *= 400
     if where == "outlier":
         K[:, :, 133, 7] = 3000.0; V[:, :, 133, 9] = -3000.0
-    cfg = qaq.make_config(wl.batch, wl.heads, D, 192, 2, 8, wl.window, wl.alpha)
+    cfg = qaq.make_config(wl.batch, wl.heads, D, 400, 2, 8, wl.window, wl.alpha)      # room for the tiles that grow again
     Kd, Vd, qd = K.cuda(), V.cuda(), q.cuda()
     thr = qaq.qaq_outlier_thresholds(cfg, Kd[:, :, :129], Vd[:, :, :129])
     cache = qaq.Cache(cfg)
@@ -173,6 +173,7 @@ def test_the_largest_value_of_a_tile_that_is_built_in_steps(D, where):
         if bits is high:
             qaq.qaq_requantize(cache, Kd, Vd, thr, bitsK=high, bitsV=high)
         out = qaq.qaq_decode_attention(cache, qd, 1 / math.sqrt(D)).cpu().numpy()
+        assert qaq.qaq_cache_stats(cache).device_status == 0
         for bh in range(wl.bh):
             b = bits[bh].cpu().numpy()
             k = oracle.quantize(u(K)[bh], th[bh, 0], th[bh, 1], b)
