@@ -410,7 +410,7 @@ def main():
                             "bytes_per_launch": ab["decode"]},
         "roofline_issue": {"quant_tiles_kernel": issue_roofline(instr("quant"), stage_ms["quant"] * 1e-3, clocks.get("sm_mhz")),
                            "decode_kernel": issue_roofline(instr("decode"), stage_ms["dec"] * 1e-3, clocks.get("sm_mhz"))},
-        "gpu_launches": args.steps * L * 5,   # thresholds 3 (sample, scan, select), quantize 1, decode 1
+        "gpu_launches": args.steps * L * 6,   # reset 1, thresholds 3 (sample, scan, select), quantize 1, decode 1
         "clocks": clocks,
     }
 

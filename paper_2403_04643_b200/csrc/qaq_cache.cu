@@ -61,7 +61,7 @@ extern "C" qaq_status qaq_cache_create(const qaq_config* cfg, qaq_cache** out) {
     auto carve = [&](size_t bytes) { size_t o = off; off = align_up(off + bytes, 256); return o; };
     size_t o_codes[2], o_bits[2], o_mnmx[2], o_tile[2], o_outl[2], o_pe[2], o_ope[2];
     // three regions: pools that need no initialisation; tables that start at zero; what qaq_cache_reset clears
-    // (one contiguous range, one memset)
+    // (one contiguous range)
     for (int x = 0; x < 2; ++x) {
         o_codes[x] = carve(BH * c->pool_bytes);
         o_outl[x] = carve(BH * (size_t)c->ocap * 4);
@@ -110,11 +110,18 @@ extern "C" qaq_status qaq_cache_destroy(qaq_cache* c) {
     return QAQ_OK;
 }
 
+// Clears the tables.  A kernel, not a memset: what follows it in the stream can then be launched while it runs (qaq_launch).
+static __global__ void __launch_bounds__(256) reset_kernel(uint4* at, size_t n) {
+    qaq_dependency();
+    for (size_t i = (size_t)blockIdx.x * 256 + threadIdx.x; i < n; i += (size_t)gridDim.x * 256) at[i] = make_uint4(0u, 0u, 0u, 0u);
+}
+
 extern "C" qaq_status qaq_cache_reset(qaq_cache* c, void* stream) {
     if (!c) return QAQ_ERR_INVALID_ARG;
     cudaStream_t s = (cudaStream_t)stream;
     // widths, tile lengths, outlier counts, pool ends and the status word: one contiguous range
-    QAQ_CUDA_TRY(cudaMemsetAsync((char*)c->slab + c->reset_off, 0, c->reset_bytes, s));
+    const size_t n = c->reset_bytes / sizeof(uint4), blocks = (n + 1023) / 1024;          // (both ends are multiples of 256 bytes)
+    QAQ_CUDA_TRY(qaq_launch(reset_kernel, dim3((unsigned)(blocks < 592 ? blocks : 592)), dim3(256), 0, s, (uint4*)((char*)c->slab + c->reset_off), n));
     c->tokens = 0;
     return QAQ_OK;
 }
