@@ -55,13 +55,12 @@ struct ThrArgs {
 // lanes of a warp to the same handful of counters; 11 bits spread them over 32 bins per octave.  In the first pass every
 // thread sums its bins and a CTA-wide prefix sum finds the bins holding the wanted ranks; in the second each rank has 32 bins,
 // one per lane of a warp.
-// NaNs sort below -inf (sign set) or above +inf.  SKIP_NAN: they do not count (AHEAD pieces of a thread are then on their way at
-// once: the data itself); else a caller whose ranks are meant among the non-NaN values adds the number of negative NaNs.
+// NaNs sort below -inf (sign set) or above +inf.  SKIP_NAN: they do not count (the data itself); else a caller whose ranks are meant among
+// the non-NaN values adds the number of negative NaNs.  AHEAD pieces of a thread are on their way at once.
 constexpr uint32_t KEY_MINUS_INF = 0x03FF, KEY_PLUS_INF = 0xFC00;
-template <int THREADS, bool SKIP_NAN, typename Load>
+template <int THREADS, bool SKIP_NAN, int AHEAD, typename Load>
 __device__ void cta_select(Load load, uint32_t n, uint32_t wantA, uint32_t wantB, uint32_t* hist, uint32_t* s_tmp, uint32_t& outA, uint32_t& outB) {
     constexpr int BINS = 2048 / THREADS;                     // of a thread
-    constexpr int AHEAD = SKIP_NAN ? 4 : 1;
     const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
     const uint32_t n8 = (n + 7) / 8;
     auto for_keys = [&](auto each) {
@@ -150,10 +149,10 @@ __device__ void cta_select(Load load, uint32_t n, uint32_t wantA, uint32_t wantB
     __syncthreads();
 }
 
-// keys that sit in shared or global memory (16-byte aligned)
-template <int THREADS>
+// keys that sit in shared memory (AHEAD 1) or global memory (16-byte aligned)
+template <int THREADS, int AHEAD = 1>
 __device__ __forceinline__ void cta_select_keys(const unsigned short* keys, uint32_t n, uint32_t wantA, uint32_t wantB, uint32_t* hist, uint32_t* s_tmp, uint32_t& outA, uint32_t& outB) {
-    cta_select<THREADS, false>([&](uint32_t i) { return reinterpret_cast<const uint4*>(keys)[i]; }, n, wantA, wantB, hist, s_tmp, outA, outB);
+    cta_select<THREADS, false, AHEAD>([&](uint32_t i) { return reinterpret_cast<const uint4*>(keys)[i]; }, n, wantA, wantB, hist, s_tmp, outA, outB);
 }
 
 __device__ __forceinline__ unsigned long long rank_k(double alpha, unsigned long long N) {
@@ -403,18 +402,18 @@ __global__ void __launch_bounds__(THREADS) thr_select_kernel(const ThrArgs a) {
         if (c0 > k && c1 > k && c <= a.cap) {
             // rank k from below and rank k from above
             const unsigned short* l = a.list + (size_t)bhx * a.cap;                // 16-byte aligned
-            const unsigned short* keys = l;
+            uint32_t lo, hi;
             if (c <= (uint32_t)SELECT_KEYS) {
-                // the usual case: the list fits in shared memory; bring it in with independent wide loads.  (A longer
-                // list is read twice where it lies, eight keys at a time; one at a time: 124 us for 640 lists of 52000
-                // keys, eight: 43 us)
+                // the usual case: the list fits in shared memory; bring it in with independent wide loads
                 for (uint32_t i = threadIdx.x; i < (c + 7) / 8; i += THREADS)
                     reinterpret_cast<uint4*>(s_keys)[i] = reinterpret_cast<const uint4*>(l)[i];
                 __syncthreads();
-                keys = s_keys;
+                cta_select_keys<THREADS>(s_keys, c, (uint32_t)k, (uint32_t)(c - 1 - k), hist, s_tmp, lo, hi);
+            } else {
+                // a longer list is read twice where it lies, four times eight keys at a time (160 (b,h) of 8192 tokens at 5 %, the whole
+                // search: eight 261 us, four times eight 258; one at a time the select alone took 124)
+                cta_select_keys<THREADS, 4>(l, c, (uint32_t)k, (uint32_t)(c - 1 - k), hist, s_tmp, lo, hi);
             }
-            uint32_t lo, hi;
-            cta_select_keys<THREADS>(keys, c, (uint32_t)k, (uint32_t)(c - 1 - k), hist, s_tmp, lo, hi);
             res[0] = float_of_key(lo); res[1] = float_of_key(hi);
         } else {
             // bracket too tight or list overflow: two-pass radix select over this problem's data, for both ranks at once, eight
@@ -426,7 +425,7 @@ __global__ void __launch_bounds__(THREADS) thr_select_kernel(const ThrArgs a) {
                 return make_uint4(keys_of(r.x), keys_of(r.y), keys_of(r.z), keys_of(r.w));
             };
             uint32_t lo, hi;
-            cta_select<THREADS, true>(load, (uint32_t)total, (uint32_t)k, (uint32_t)(N - 1 - k), hist, s_tmp, lo, hi);
+            cta_select<THREADS, true, 4>(load, (uint32_t)total, (uint32_t)k, (uint32_t)(N - 1 - k), hist, s_tmp, lo, hi);
             res[0] = float_of_key(lo); res[1] = float_of_key(hi);
         }
     }
@@ -654,7 +653,7 @@ extern "C" qaq_status qaq_outlier_thresholds(const qaq_config* cfg, const void* 
     dim3 grid((n_tokens + a.scan_tokens - 1) / a.scan_tokens, BH * 2);
     QAQ_CUDA_TRY(qaq_launch(thr_scan_kernel, grid, dim3(256), 0, s, a));
     // lists that stay in shared memory are a matter of latency (256 (b,h) of 4096 tokens, alpha = 1 %: 14.6 us with 256
-    // threads, 19.1 with 512), longer ones of throughput (160 of 8192 tokens, 5 %: 68.3 and 48.7 us)
+    // threads, 19.1 with 512), longer ones of throughput (160 of 8192 tokens, 5 %: 68.3 and 48.7 us, 46 with four loads ahead)
     if (1.25 * cfg->outlier_frac * (double)keys <= SELECT_KEYS) QAQ_CUDA_TRY(qaq_launch(thr_select_kernel<256>, dim3(BH * 2), dim3(256), 0, s, a));
     else QAQ_CUDA_TRY(qaq_launch(thr_select_kernel<512>, dim3(BH * 2), dim3(512), 0, s, a));
     return QAQ_OK;
