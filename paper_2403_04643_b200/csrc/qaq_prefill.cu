@@ -171,7 +171,8 @@ __device__ __forceinline__ void query_norm(const PrefillArgs& a, int bh, int i) 
 
 // One CTA per SM, which goes through its share of the work: a warp asks for the keys (tiles of 128 tokens, a ring of stages), a
 // warp multiplies them, sixteen look at the accumulators.  Row t of an accumulator is a token, a thread's; column i a query.
-// The reference of a row is a warp's largest logit of its first tile; it is raised where a later logit exceeds it by 2^64.
+// The reference of a row is a warp's largest logit of its first tile that has one above -inf (keys that are not finite); it is raised
+// where a later logit exceeds it by 2^64.
 // A wait that runs out of tries (a copy or a peer that never came) ends the waiting: the rows are then not numbers.
 // Where the accumulators of two (b,h) have room (up to 32 rows) half of the sixteen warps take the statistics of the next one while
 // the others write the rows of the last (256 (b,h) of 4096 tokens, 32 rows: 70 us, 82 with all of them at one job after the other, 78
@@ -286,6 +287,7 @@ __global__ void __launch_bounds__(PW_THREADS, 1) window_kernel(const __grid_cons
 #pragma unroll
                 for (int c = 0; c < CW; ++c) sum[c] = 0.f;
                 float* const ref = sm.ref[it & 1][w];
+                bool unset = false;                              // a row has no reference yet: its logits so far are -inf (0 stands in)
 #pragma unroll 1
                 for (int k = group; k < o.n; k += GROUPS) {
                     const uint32_t g = g0 + k;
@@ -300,8 +302,21 @@ __global__ void __launch_bounds__(PW_THREADS, 1) window_kernel(const __grid_cons
                         for (int c = 0; c < CW; c += 4) {
                             float m[4];
 #pragma unroll
-                            for (int j = 0; j < 4; ++j) { m[j] = warp_max(c + j < hidden ? NEG : x[c + j] * sc); m[j] = m[j] == NEG ? 0.f : m[j]; }
+                            for (int j = 0; j < 4; ++j) m[j] = warp_max(c + j < hidden ? NEG : x[c + j] * sc);
                             if (lane == 0) *reinterpret_cast<float4*>(ref + c) = make_float4(m[0], m[1], m[2], m[3]);
+                        }
+                        __syncwarp();
+                        const bool none = ref[lane % CW] == NEG;
+                        unset = __any_sync(0xFFFFFFFFu, none);
+                        if (unset) {
+                            if (none) ref[lane % CW] = 0.f;
+                            __syncwarp();
+                        }
+                    } else if (unset) {
+#pragma unroll
+                        for (int c = 0; c < CW; ++c) {
+                            const float m = warp_max(c < hidden ? NEG : x[c] * sc);
+                            if (m != NEG && !__any_sync(0xFFFFFFFFu, sum[c] != 0.f) && lane == 0) ref[c] = m;
                         }
                         __syncwarp();
                     }
@@ -464,7 +479,7 @@ template <int D, int NC>
 __global__ void __launch_bounds__(128 * PS_TILES, 1) window_short_kernel(const PrefillArgs a, const __half* K, long sb, long sh, long st) {
     using W = Window<D, NC, STATS>;
     constexpr int RB = W::ROW_BYTES, CW = NC < 32 ? NC : 32;
-    const float NEG = __int_as_float(0xff800000), sc = a.scale * 1.4426950408889634f;
+    const float NEG = __int_as_float(0xff800000), LOWEST = __int_as_float(0xff7fffff), sc = a.scale * 1.4426950408889634f;
     extern __shared__ unsigned char s_dyn[];
     __shared__ alignas(8) unsigned long long s_bar[PS_TILES];
     __shared__ uint32_t s_tmem;
@@ -523,7 +538,7 @@ __global__ void __launch_bounds__(128 * PS_TILES, 1) window_short_kernel(const P
         for (int c = 0; c < 8; ++c) {
             const bool seen = c0 + c >= hidden;
             m[c] = warp_max(seen ? x[c0 + c] * sc : NEG);
-            sum[c] = x[c0 + c] = seen ? pow2(fmaf(x[c0 + c], sc, -m[c])) : 0.f;
+            sum[c] = x[c0 + c] = seen ? pow2(fmaf(x[c0 + c], sc, -fmaxf(m[c], LOWEST))) : 0.f;      // (a maximum of -inf: zeros)
         }
         if (lane == 0) {
             *reinterpret_cast<float4*>(&s_max[warp][c0]) = make_float4(m[0], m[1], m[2], m[3]);

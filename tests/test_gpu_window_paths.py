@@ -74,3 +74,17 @@ def test_heads_that_share_keys_and_keys_that_are_not_numbers(T):
     assert torch.isnan(ring[:, :, T // 2]).all()
     ring[:, :, T // 2] = 0
     assert (ring == 0).all() and (shared.sum() > 0)
+
+
+@pytest.mark.parametrize("D", [32, 64, 128])
+@pytest.mark.parametrize("heads,T,n", [(2, 100, 5), (2, 700, 33), (300, 400, 16), (3, 1500, 16), (2, 3000, 32), (2, 4100, 64), (2, 9000, 64)])
+def test_logits_of_minus_infinity(D, heads, T, n):
+    # the first two thirds of the tokens have logits of -inf in every row, the others are far below zero: entries of 0, and rows that
+    # are normalised over the rest (logits of about -1000, whose binary32 sums are off by 2^-24 of 8000 a few times: 1e-3 of an entry)
+    K = keys(1, heads, T, D, token_major=False, seed=T)
+    K[..., 0] = -1000.0
+    K[:, :, :2 * T // 3, 0] = -math.inf
+    Q = torch.randn((heads, n, D), generator=torch.Generator().manual_seed(n)).half()
+    Q[..., 0] = math.sqrt(D)
+    ring = rows_match(K, Q, heads, {0, heads - 1})
+    assert torch.allclose(ring.sum(2), torch.ones(heads, n, device="cuda"), atol=1e-4)
