@@ -46,6 +46,11 @@ typedef struct {
     long max_outliers_per_bh;   /* per tensor; <= 0: derived from outlier_frac with slack */
 } qaq_config;
 
+/* What stands in place of every score of a token whose window could not be computed, as a binary32 pattern (a NaN that arithmetic
+ * does not give): a kernel of qaq_prefill_window waited in vain for its own copies or for its peers.  Where the first row of a token's
+ * window holds it and no other row a number, its value takes bits_max, and the device status of the cache becomes QAQ_ERR_CUDA. */
+#define QAQ_SCORE_LOST 0x7FC0105Eu
+
 /* Scalars of the bit-width rules (Section 4.1), see qaq_policy_from_hyper. */
 typedef struct {
     float cK; /* keys:   B = min{b : range       <= cK * 2^b} */
@@ -61,7 +66,7 @@ typedef struct {
     double cr_paper;          /* 16*2*T*D*BH / (code bits + 16 bits per outlier): memory
                                  "calculated by the quantized bit" (Sections 2.1, 5.2) */
     double cr_total;          /* fp16 bytes / resident_bytes */
-    int device_status;        /* sticky qaq_status raised on the device (capacity) */
+    int device_status;        /* sticky qaq_status raised on the device: capacity, lost copies or score windows */
 } qaq_stats;
 
 typedef struct qaq_cache qaq_cache; /* opaque; owns its device memory */
@@ -134,7 +139,8 @@ qaq_status qaq_select_bits(const qaq_config* cfg, const qaq_policy* policy, cons
  * qnorm2: NULL or binary32 [batch*heads][n] receiving sum_d (softmax_scale * q_d)^2 per query
  * (the caller takes the quantile it wants for qaq_policy_from_hyper); ws:
  * qaq_prefill_window_workspace_bytes bytes, 8-byte aligned.  Device pointers, asynchronous on
- * stream.  Errors: QAQ_ERR_INVALID_ARG, QAQ_ERR_UNSUPPORTED_SHAPE (window > 64), QAQ_ERR_WORKSPACE.
+ * stream.  Errors: QAQ_ERR_INVALID_ARG, QAQ_ERR_UNSUPPORTED_SHAPE (window > 64), QAQ_ERR_WORKSPACE; a wait of the kernels that
+ * runs out (nothing does in correct operation) leaves QAQ_SCORE_LOST in the rows it concerns, which the calls that take them report.
  */
 qaq_status qaq_prefill_window_workspace_bytes(const qaq_config* cfg, int n_tokens, size_t* host_out);
 qaq_status qaq_prefill_window(const qaq_config* cfg, const void* Q, const void* K, long stride_b, long stride_h,

@@ -65,7 +65,8 @@ struct Window {
         alignas(16) float ref[2][TEAM][CW], sum[2][TEAM][CW];      // of a warp: reference and sum of every row over its tokens
         alignas(16) float2 all[2][PW_CLUSTER][NC];           // the same of every CTA of the cluster, which all write here
         alignas(16) float2 row[2][NC];                        // what the rows are normalised with: reference, 1 / sum
-        uint32_t tmem;
+        uint32_t tmem, failed;                               // a wait ran out
+        int stopped;                                         // the first of the CTA's items whose statistics it has not taken, then; else -1
     };
     static constexpr int FIT = (PW_SMEM - 1024 - 2 * (int)QUERY_BYTES - (int)sizeof(Shared)) / (int)TILE_BYTES, STAGES = FIT < 8 ? FIT : 8;
     static_assert(STAGES >= 4, "stages");
@@ -169,11 +170,19 @@ __device__ __forceinline__ void query_norm(const PrefillArgs& a, int bh, int i) 
     a.qnorm2[(size_t)bh * a.n + i] = s;
 }
 
+// `tokens` entries of n rows, T apart, by a whole CTA
+__device__ __noinline__ void lose_rows(float* row, int n, int T, int tokens) {
+    for (; n > 0; --n, row += T)
+        for (int t = threadIdx.x; t < tokens; t += blockDim.x) row[t] = __uint_as_float(QAQ_SCORE_LOST);
+}
+
 // One CTA per SM, which goes through its share of the work: a warp asks for the keys (tiles of 128 tokens, a ring of stages), a
 // warp multiplies them, sixteen look at the accumulators.  Row t of an accumulator is a token, a thread's; column i a query.
 // The reference of a row is a warp's largest logit of its first tile that has one above -inf (keys that are not finite); it is raised
 // where a later logit exceeds it by 2^64.
-// A wait that runs out of tries (a copy or a peer that never came) ends the waiting: the rows are then not numbers.
+// A wait that runs out of tries (a copy or a peer that never came) ends the CTA's waiting.  It then sends no more statistics, so that the
+// other CTAs of the (b,h) run out of tries as well, or leaves a mark in place of those of its chunk, and in the end QAQ_SCORE_LOST
+// in all rows of its tokens.
 // Where the accumulators of two (b,h) have room (up to 32 rows) half of the sixteen warps take the statistics of the next one while
 // the others write the rows of the last (256 (b,h) of 4096 tokens, 32 rows: 70 us, 82 with all of them at one job after the other, 78
 // with eight warps); with 64 rows the tensor memory is full and the halves wait for each other (160 of 8192: 222 us, 152 together).
@@ -205,6 +214,7 @@ __global__ void __launch_bounds__(PW_THREADS, 1) window_kernel(const __grid_cons
         for (int i = 0; i < STAGES; ++i) { bar_init(full + 8 * i, 1); bar_init(empty + 8 * i, 1); }
         for (int i = 0; i < SLOTS; ++i) { bar_init(there + 8 * i, 1); bar_init(taken + 8 * i, 4 * W::PARTS); }
         for (int i = 0; i < 2; ++i) { bar_init(q_free + 8 * i, 1); bar_init(stats + 8 * i, 1); bar_init(used + 8 * i, ncta); }
+        sm.failed = 0; sm.stopped = -1;
         asm volatile("fence.mbarrier_init.release.cluster;\nfence.proxy.async.shared::cta;" ::: "memory");
     }
     qaq_dependency();
@@ -214,6 +224,7 @@ __global__ void __launch_bounds__(PW_THREADS, 1) window_kernel(const __grid_cons
     if (MODE == ONE_PASS) cluster_barrier(); else __syncthreads();
     tmem_after_sync();
     const uint32_t acc = *(volatile uint32_t*)&sm.tmem;
+    volatile uint32_t& failed = sm.failed;
     bool ok = true;
     if (warp == 0) {
         if (lane == 0) {
@@ -234,8 +245,9 @@ __global__ void __launch_bounds__(PW_THREADS, 1) window_kernel(const __grid_cons
                     }
                 }
             }
-            if (!ok)                   // what is on its way arrives before the CTA leaves
-                for (uint32_t j = g > STAGES ? g - STAGES : 0; j < g; ++j) bar_wait(full + 8 * (j % STAGES), (j / STAGES) & 1u);
+            if (!ok) failed = 1;
+            // what is on its way arrives before the CTA leaves (which takes no time but where something has failed)
+            for (uint32_t j = g > STAGES ? g - STAGES : 0; j < g; ++j) bar_wait(full + 8 * (j % STAGES), (j / STAGES) & 1u);
         }
     } else if (warp == 1) {
         if (lane == 0) {
@@ -254,6 +266,8 @@ __global__ void __launch_bounds__(PW_THREADS, 1) window_kernel(const __grid_cons
                 }
                 tensor_done(q_free + 8 * (it & 1));
             }
+            if (!ok) failed = 1;
+            if (it) bar_wait(q_free + 8 * ((it - 1) & 1), (uint32_t)((it - 1) >> 1) & 1u);              // likewise
         }
     } else {
         constexpr int CW = W::CW, GROUPS = W::GROUPS, TEAM = W::TEAM;
@@ -261,12 +275,6 @@ __global__ void __launch_bounds__(PW_THREADS, 1) window_kernel(const __grid_cons
         const int team = (warp - 2) / TEAM, w = (warp - 2) % TEAM, e = 32 * w + lane, quarter = warp & 3, group = (w >> 2) / W::PARTS, h = (w >> 2) % W::PARTS * CW;
         const float sc = a.scale * 1.4426950408889634f;
         const uint32_t lanes = acc + ((uint32_t)(32 * quarter) << 16) + h;
-        auto logits = [&](uint32_t slot, float (&x)[CW]) {
-            load_acc(lanes + slot * NC, x);
-            if (!ok)
-#pragma unroll
-                for (int c = 0; c < CW; ++c) x[c] = __int_as_float(0x7fffffff);
-        };
         auto wait_for = [&](uint32_t g) {
             ok = __all_sync(0xFFFFFFFFu, ok && bar_wait(there + 8 * (g % SLOTS), (g / SLOTS) & 1u));
             tmem_after_sync();
@@ -287,7 +295,8 @@ __global__ void __launch_bounds__(PW_THREADS, 1) window_kernel(const __grid_cons
 #pragma unroll
                 for (int c = 0; c < CW; ++c) sum[c] = 0.f;
                 float* const ref = sm.ref[it & 1][w];
-                bool unset = false;                              // a row has no reference yet: its logits so far are -inf (0 stands in)
+                float* const top = sm.sum[it & 1][w];            // (until the sums are there: largest logits)
+                bool none = true;                                // the row of the lane's column has no reference yet, 0 stands in: its logits are -inf
 #pragma unroll 1
                 for (int k = group; k < o.n; k += GROUPS) {
                     const uint32_t g = g0 + k;
@@ -295,28 +304,21 @@ __global__ void __launch_bounds__(PW_THREADS, 1) window_kernel(const __grid_cons
                     const int hidden = t0 + k * PW_TILE - (a.T - a.n) - h;
                     const bool part_hidden = hidden - lane + 31 > 0;
                     float x[CW];
-                    logits(g % SLOTS, x);
+                    load_acc(lanes + (g % SLOTS) * NC, x);
                     if (MODE == STATS) release(g);
-                    if (k == group) {
+                    if (__any_sync(0xFFFFFFFFu, none)) {
 #pragma unroll
                         for (int c = 0; c < CW; c += 4) {
                             float m[4];
 #pragma unroll
                             for (int j = 0; j < 4; ++j) m[j] = warp_max(c + j < hidden ? NEG : x[c + j] * sc);
-                            if (lane == 0) *reinterpret_cast<float4*>(ref + c) = make_float4(m[0], m[1], m[2], m[3]);
+                            if (lane == 0) *reinterpret_cast<float4*>(top + c) = make_float4(m[0], m[1], m[2], m[3]);
                         }
                         __syncwarp();
-                        const bool none = ref[lane % CW] == NEG;
-                        unset = __any_sync(0xFFFFFFFFu, none);
-                        if (unset) {
-                            if (none) ref[lane % CW] = 0.f;
-                            __syncwarp();
-                        }
-                    } else if (unset) {
-#pragma unroll
-                        for (int c = 0; c < CW; ++c) {
-                            const float m = warp_max(c < hidden ? NEG : x[c] * sc);
-                            if (m != NEG && !__any_sync(0xFFFFFFFFu, sum[c] != 0.f) && lane == 0) ref[c] = m;
+                        if (none) {
+                            const float m = top[lane % CW];
+                            none = m == NEG;
+                            ref[lane % CW] = none ? 0.f : m;
                         }
                         __syncwarp();
                     }
@@ -328,10 +330,10 @@ __global__ void __launch_bounds__(PW_THREADS, 1) window_kernel(const __grid_cons
                     if (part_hidden)
 #pragma unroll
                         for (int c = 0; c < CW; ++c) if (c < hidden) x[c] = NEG;
-                    float top = NEG;
+                    float most = NEG;
 #pragma unroll
-                    for (int c = 0; c < CW; c += 2) top = fmaxf(top, fmaxf(x[c], x[c + 1]));
-                    if (__any_sync(0xFFFFFFFFu, top > 64.0f)) {
+                    for (int c = 0; c < CW; c += 2) most = fmaxf(most, fmaxf(x[c], x[c + 1]));
+                    if (__any_sync(0xFFFFFFFFu, most > 64.0f)) {
                         __syncwarp();
 #pragma unroll
                         for (int c = 0; c < CW; ++c) {
@@ -354,7 +356,9 @@ __global__ void __launch_bounds__(PW_THREADS, 1) window_kernel(const __grid_cons
                     if ((lane & 3) == 0) sm.sum[it & 1][w][c0 + (lane >> 2)] = s;
                 }
                 if (group >= o.n && lane < CW) { ref[lane] = NEG; sm.sum[it & 1][w][lane] = 0.f; }      // no tile for the group
+                if (!ok) failed = 1;
                 team_sync<32 * TEAM>(0);
+                ok = !failed;              // whatever warp of the team has waited in vain so far
                 const int c = e % NC;
                 float2 st = make_float2(NEG, 0.f);
                 if (c < a.n)
@@ -364,18 +368,19 @@ __global__ void __launch_bounds__(PW_THREADS, 1) window_kernel(const __grid_cons
                         if (!(sm.sum[it & 1][from][c % CW] == 0.f)) fold_stats(st, make_float2(sm.ref[it & 1][from][c % CW], sm.sum[it & 1][from][c % CW]));
                     }
                 if (MODE == STATS) {
-                    if (e < a.n) a.part[((size_t)o.bh * a.nchunk + o.chunk) * a.n + e] = st;
+                    if (e < a.n) a.part[((size_t)o.bh * a.nchunk + o.chunk) * a.n + e] = ok ? st : make_float2(0.f, -1.0f);      // (no sum is negative)
                 } else {
                     // every CTA of the (b,h) gets the statistics of all of them, as soon as all have used those of two items before.
                     // (A launch without clusters knows no asynchronous stores to a CTA of the cluster, its own included.)
                     const uint32_t bar = stats + 8 * (it & 1);
                     // Only warps that send wait: one that does not could come so late that the phase is over, and the one after.
                     if ((e & ~31) < ncta * NC) ok = __all_sync(0xFFFFFFFFu, ok && bar_wait_cluster(used + 8 * (it & 1), ((uint32_t)(it >> 1) & 1u) ^ 1u));
+                    if (!ok) failed = 1;
                     if (ncta == 1) {
                         if (e < a.n) sm.all[it & 1][0][e] = st;
                         team_sync<32 * TEAM>(0);
-                        if (e == 0) bar_arrive(bar);
-                    } else {
+                        if (e == 0 && !failed) bar_arrive(bar);
+                    } else if (ok) {
                     if (e == 0) bar_expect(bar, (uint32_t)(ncta * a.n) * 8u);
                     if (c < a.n)
                         for (int r = e / NC; r < ncta; r += 32 * TEAM / NC)
@@ -397,7 +402,9 @@ __global__ void __launch_bounds__(PW_THREADS, 1) window_kernel(const __grid_cons
                         sm.row[buf][e] = make_float2(st.x, st.y > 0.f ? 1.0f / st.y : 0.f);
                     }
                     team_sync<32 * TEAM>(1);
-                    if (ncta == 1) {
+                    if (!ok) {
+                        if (e == 0 && sm.stopped < 0) sm.stopped = it;
+                    } else if (ncta == 1) {
                         if (e == 0) bar_arrive(used + 8 * buf);
                     } else if (e < ncta)
                         asm volatile("{\n.reg .u32 m;\nmapa.shared::cluster.u32 m, %0, %1;\nmbarrier.arrive.release.cluster.shared::cluster.b64 _, [m];\n}" ::"r"(used + 8 * buf), "r"(e) : "memory");
@@ -409,7 +416,11 @@ __global__ void __launch_bounds__(PW_THREADS, 1) window_kernel(const __grid_cons
                     static_assert(EACH <= PW_CLUSTER && EACH * NC <= 32 * TEAM, "parts");
                     if (e < EACH * NC) {
                         if (e % NC < a.n)
-                            for (int ch = e / NC; ch < a.nchunk; ch += EACH) fold_stats(st, a.part[((size_t)o.bh * a.nchunk + ch) * a.n + e % NC]);
+                            for (int ch = e / NC; ch < a.nchunk; ch += EACH) {
+                                const float2 p = a.part[((size_t)o.bh * a.nchunk + ch) * a.n + e % NC];
+                                if (p.y < 0.f) failed = 1;
+                                fold_stats(st, p);
+                            }
                         sm.all[buf][e / NC][e % NC] = st;
                     }
                     team_sync<32 * TEAM>(1);
@@ -428,7 +439,7 @@ __global__ void __launch_bounds__(PW_THREADS, 1) window_kernel(const __grid_cons
                     const bool part_hidden = hidden - lane + 31 > 0;
                     float* row = row0 + k * PW_TILE;
                     float x[CW];
-                    logits(g % SLOTS, x);
+                    load_acc(lanes + (g % SLOTS) * NC, x);
                     release(g);
 #pragma unroll
                     for (int c = 0; c < CW; c += 2) {
@@ -453,11 +464,23 @@ __global__ void __launch_bounds__(PW_THREADS, 1) window_kernel(const __grid_cons
             }
             g0 += o.n;
         }
+        if (!ok) failed = 1;
     }
     __syncwarp();
     tmem_before_sync();
     if (MODE == ONE_PASS) cluster_barrier(); else __syncthreads();       // nobody leaves while somebody may write to its shared memory
     if (warp == 1) { tmem_after_sync(); asm volatile("tcgen05.dealloc.cta_group::1.sync.aligned.b32 %0, 512;" ::"r"(acc) : "memory"); }
+    if (MODE != STATS && failed) {
+        // Statistics that are on their way arrive before the CTA leaves.  Those of an item are sent when all CTAs of the cluster have
+        // taken the ones of two items before, so they can only be those of the first item that this CTA has not taken, and of the next;
+        // all that will be sent has been sent before the barrier above.
+        if (MODE == ONE_PASS && ncta > 1 && tid == 0 && sm.stopped >= 0)
+            for (int it = sm.stopped; it < sm.stopped + 2 && blockIdx.x / ncta + it * step < items; ++it) bar_wait_cluster(stats + 8 * (it & 1), (uint32_t)(it >> 1) & 1u);
+        for (int i = blockIdx.x / ncta; i < items; i += step) {
+            const Item o = item_of(i);
+            lose_rows(a.ring + (size_t)o.bh * a.n * a.T + o.tile * PW_TILE, a.n, a.T, min(o.n * PW_TILE, a.T - o.tile * PW_TILE));
+        }
+    }
 }
 
 // ---- few tiles in all: a thread keeps the logits of its token in registers, a CTA is one tile to four (four warps each), and the CTAs
@@ -482,7 +505,7 @@ __global__ void __launch_bounds__(128 * PS_TILES, 1) window_short_kernel(const P
     const float NEG = __int_as_float(0xff800000), LOWEST = __int_as_float(0xff7fffff), sc = a.scale * 1.4426950408889634f;
     extern __shared__ unsigned char s_dyn[];
     __shared__ alignas(8) unsigned long long s_bar[PS_TILES];
-    __shared__ uint32_t s_tmem;
+    __shared__ uint32_t s_tmem, s_failed;                    // s_failed: a wait ran out
     __shared__ alignas(16) float s_max[4 * PS_TILES][NC], s_sum[4 * PS_TILES][NC];       // of a warp: reference and sum of every row over its tokens
     __shared__ float2 s_all[PW_CLUSTER][NC];                 // the same of every CTA of the cluster, which all write here
     const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31, group = warp >> 2, groups = blockDim.x >> 7, warps = 4 * groups;
@@ -491,6 +514,7 @@ __global__ void __launch_bounds__(128 * PS_TILES, 1) window_short_kernel(const P
     const uint32_t columns = max(32, 1 << (32 - __clz(groups * NC - 1)));                // (a power of two)
     if (tid == 0) {
         for (int i = 0; i < PS_TILES; ++i) bar_init(smem_addr(s_bar) + 8 * i, 1);
+        s_failed = 0;
         asm volatile("fence.proxy.async.shared::cta;" ::: "memory");
     }
     qaq_dependency();
@@ -514,7 +538,8 @@ __global__ void __launch_bounds__(128 * PS_TILES, 1) window_short_kernel(const P
         tensor_done(bar);
     }
     __syncwarp();
-    const bool ok = __all_sync(0xFFFFFFFFu, bar_wait(bar, 0u));
+    if (!bar_wait(bar, 0u)) s_failed = 1;
+    __syncwarp();
     tmem_after_sync();
     float x[NC];
 #pragma unroll
@@ -524,9 +549,6 @@ __global__ void __launch_bounds__(128 * PS_TILES, 1) window_short_kernel(const P
 #pragma unroll
         for (int c = 0; c < CW; ++c) x[h + c] = v[c];
     }
-    if (!ok)
-#pragma unroll
-        for (int c = 0; c < NC; ++c) x[c] = __int_as_float(0x7fffffff);
     // ---- per warp: maximum of every row over its tokens, the logits become powers of two relative to it (0 where the query cannot
     //      see the token), and their sum
     const int t = t_group + 32 * (warp & 3) + lane, hidden = t - (a.T - a.n);
@@ -550,11 +572,13 @@ __global__ void __launch_bounds__(128 * PS_TILES, 1) window_short_kernel(const P
     tmem_before_sync();
     __syncthreads();
     if (warp == 0) { tmem_after_sync(); asm volatile("tcgen05.dealloc.cta_group::1.sync.aligned.b32 %0, %1;" ::"r"(acc), "r"(columns) : "memory"); }
+    bool lost = *(volatile uint32_t*)&s_failed != 0;
     if (ncta > 1) {
         asm volatile("barrier.cluster.wait.acquire.aligned;" ::: "memory");              // second half of the barrier begun at the start
         if (const int c = tid % NC; c < a.n) {
             float2 own = make_float2(NEG, 0.f);
             for (int w = 0; w < warps; ++w) fold_stats(own, make_float2(s_max[w][c], s_sum[w][c]));
+            if (lost) own.y = -1.0f;                         // (no sum is negative)
             for (int r = tid / NC; r < ncta; r += blockDim.x / NC)
                 asm volatile("{\n.reg .u32 p;\nmapa.shared::cluster.u32 p, %0, %1;\nst.shared::cluster.v2.f32 [p], {%2, %3};\n}"
                              ::"r"(smem_addr(&s_all[rank][c])), "r"(r), "f"(own.x), "f"(own.y) : "memory");
@@ -570,19 +594,24 @@ __global__ void __launch_bounds__(128 * PS_TILES, 1) window_short_kernel(const P
         const int c = CW * h + lane % CW;
         float2 all = make_float2(NEG, 0.f);
         if (c < a.n) {
-            if (ncta > 1) for (int r = 0; r < ncta; ++r) fold_stats(all, s_all[r][c]);
+            if (ncta > 1) for (int r = 0; r < ncta; ++r) { lost = lost || s_all[r][c].y < 0.f; fold_stats(all, s_all[r][c]); }
             else for (int w = 0; w < warps; ++w) fold_stats(all, make_float2(s_max[w][c], s_sum[w][c]));
         }
         const float own = c < a.n ? s_max[warp][c] : NEG;
         f[h] = all.y > 0.f && own != NEG ? pow2(own - all.x) / all.y : 0.f;
     }
     float* row = a.ring + ((size_t)bh * a.n + (a.n - 1)) * a.T + t;
+    if (__any_sync(0xFFFFFFFFu, lost)) {                     // the tokens of the CTA, by all of its warps alike
+        for (int c = 0; c < a.n; ++c, row -= a.T)
+            if (t < a.T) *row = __uint_as_float(QAQ_SCORE_LOST);
+    } else {
 #pragma unroll
-    for (int c = 0; c < NC; ++c) {
-        if (c >= a.n) break;
-        const float y = x[c] * __shfl_sync(0xFFFFFFFFu, f[c / CW], c % CW);
-        if (t < a.T) *row = y;
-        row -= a.T;
+        for (int c = 0; c < NC; ++c) {
+            if (c >= a.n) break;
+            const float y = x[c] * __shfl_sync(0xFFFFFFFFu, f[c / CW], c % CW);
+            if (t < a.T) *row = y;
+            row -= a.T;
+        }
     }
     if (t < a.T) a.nvalid[(size_t)bh * a.T + t] = (uint8_t)min(a.n, a.T - t);
 }

@@ -220,6 +220,7 @@ __device__ __forceinline__ void quantize_tile(const QuantArgs& a, TileScratch<D>
         nv = min(nv, a.W);
         const float* scores = a.ring + (size_t)bh * a.W * a.n_new + col;
         shat = OPEN ? qaqc::window_max_one_loop<32>(scores, a.W, a.n_new, nv) : qaqc::window_max<32>(scores, a.W, a.n_new, nv);
+        if (qaqc::window_lost(scores, nv, shat)) { nv = 0; atomicMax(a.status, (int)QAQ_ERR_CUDA); }
     }
     if (OPEN) {                        // the tile as it is stored follows on its own: it is needed later
         asm volatile("cp.async.commit_group;" ::: "memory");
@@ -534,6 +535,7 @@ __global__ void __launch_bounds__(2 * D) select_kernel(const QuantArgs a) {
     }
 #pragma unroll
     for (int o = 1; o < P; o <<= 1) shat = fmaxf(shat, __shfl_xor_sync(0xFFFFFFFFu, shat, o));
+    if (qaqc::window_lost(a.ring + (size_t)bh * a.W * a.n_new + tn, nv, shat)) nv = 0;
 #pragma unroll
     for (int x = 0; x < 2; ++x) {
         const __half2 lo2 = __half2half2(__float2half_ru(thr[2 * x])), hi2 = __half2half2(__float2half_rd(thr[2 * x + 1]));

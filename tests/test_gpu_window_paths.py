@@ -8,9 +8,9 @@ import pytest
 import torch
 
 import oracle
-from paper_2403_04643_b200 import qaq
+from paper_2403_04643_b200 import qaq, synth
 
-from gpu_helpers import u16
+from gpu_helpers import make_inputs, u16
 
 pytestmark = pytest.mark.gpu
 
@@ -88,3 +88,50 @@ def test_logits_of_minus_infinity(D, heads, T, n):
     Q[..., 0] = math.sqrt(D)
     ring = rows_match(K, Q, heads, {0, heads - 1})
     assert torch.allclose(ring.sum(2), torch.ones(heads, n, device="cuda"), atol=1e-4)
+
+
+LOST = torch.tensor([0x7FC0105E], dtype=torch.int32).view(torch.float32)      # QAQ_SCORE_LOST
+
+
+@pytest.mark.parametrize("D", [32, 128])
+@pytest.mark.parametrize("W", [5, 40])
+@pytest.mark.parametrize("how", ["tiles", "open", "select", "lower", "raise"])
+def test_a_lost_window_is_reported_by_the_calls_that_take_it(D, W, how):
+    # what a window kernel whose wait ran out leaves in the rows of its tokens: their values take bits_max and the device status says so,
+    # nothing else changes; a window without a number for another reason is not reported
+    wl = synth.scaled(synth.CONFIGS["C2"], heads=2, head_dim=D, tokens=150, window=W)
+    K, V, q, ring, nv = (t.cuda() for t in make_inputs(wl))
+    nan, lost = ring.clone(), ring.clone()
+    nan[..., 70:90] = math.nan
+    lost[..., 70:90] = LOST.cuda()
+    if how == "open":
+        nan[..., 149] = math.nan
+        lost[..., 149] = LOST.cuda()
+    pol = qaq.qaq_policy_from_hyper(0.006, 0.03, 64.0, 150)
+    cfg = qaq.make_config(wl.batch, wl.heads, D, 400, 2, 8, W, wl.alpha)
+    thr = qaq.qaq_outlier_thresholds(cfg, K, V)
+
+    def widths(r):
+        if how == "select":
+            return *qaq.qaq_select_bits(cfg, pol, K, V, r, nv, thr), None
+        cache = qaq.Cache(cfg)
+        if how == "open":
+            for a, b in ((0, 149), (149, 150)):
+                qaq.qaq_quantize_append(cache, K[:, :, a:b], V[:, :, a:b], thr, policy=pol, ring=r[..., a:b].contiguous(), nvalid=nv[..., a:b].contiguous())
+        elif how == "tiles":
+            qaq.qaq_quantize_append(cache, K, V, thr, policy=pol, ring=r, nvalid=nv)
+        else:
+            bits = torch.full((wl.bh, 150), 8 if how == "lower" else 1, dtype=torch.uint8, device="cuda")
+            qaq.qaq_quantize_append(cache, K, V, thr, bitsK=bits, bitsV=bits)
+            if how == "lower":
+                qaq.qaq_requantize_down(cache, policy=pol, ring=r, nvalid=nv)
+            else:
+                qaq.qaq_requantize(cache, K, V, thr, policy=pol, ring=r, nvalid=nv)
+        return *(qaq.qaq_cache_export(cache, x)["bits"] for x in (0, 1)), qaq.qaq_cache_stats(cache).device_status
+
+    k0, v0, s0 = widths(nan)
+    k1, v1, s1 = widths(lost)
+    there = (lost == lost).all(dim=2).view(wl.bh, 150)
+    assert torch.equal(k0, k1) and torch.equal(v0[there], v1[there])
+    assert (v0[~there] == 2).all() and (v1[~there] == 8).all()
+    assert how == "select" or (s0, s1) == (qaq.QAQ_OK, 4)
