@@ -628,17 +628,20 @@ qaq_status run_short(const PrefillArgs& a, const void* K, long sb, long sh, long
 // Descriptions of K ([batch][head][token][channel] with the caller's strides) and of the queries for the copies of tiles.
 typedef CUresult (*EncodeTiled)(CUtensorMap*, CUtensorMapDataType, cuuint32_t, void*, const cuuint64_t*, const cuuint64_t*, const cuuint32_t*, const cuuint32_t*,
                                 CUtensorMapInterleave, CUtensorMapSwizzle, CUtensorMapL2promotion, CUtensorMapFloatOOBfill);
-bool describe(CUtensorMap* map, const void* at, int rank, const cuuint64_t* size, const cuuint64_t* stride, const cuuint32_t* box, int D) {
-    static const EncodeTiled encode = [] {
-        void* f = nullptr;
+cudaError_t describe(CUtensorMap* map, const void* at, int rank, const cuuint64_t* size, const cuuint64_t* stride, const cuuint32_t* box, int D) {
+    static std::atomic<void*> known;                         // once it is found
+    void* f = known.load(std::memory_order_acquire);
+    if (!f) {
         cudaDriverEntryPointQueryResult found;
         const cudaError_t e = cudaGetDriverEntryPointByVersion("cuTensorMapEncodeTiled", &f, 12000, cudaEnableDefault, &found);
-        if (e != cudaSuccess) (void)cudaGetLastError();
-        return e == cudaSuccess && found == cudaDriverEntryPointSuccess ? (EncodeTiled)f : (EncodeTiled) nullptr;
-    }();
+        if (e != cudaSuccess) return e;
+        if (found != cudaDriverEntryPointSuccess || !f) return cudaErrorSymbolNotFound;
+        known.store(f, std::memory_order_release);
+    }
     const cuuint32_t each[4] = {1, 1, 1, 1};
-    return encode && encode(map, CU_TENSOR_MAP_DATA_TYPE_FLOAT16, rank, const_cast<void*>(at), size, stride, box, each, CU_TENSOR_MAP_INTERLEAVE_NONE,
-                            D >= 64 ? CU_TENSOR_MAP_SWIZZLE_128B : CU_TENSOR_MAP_SWIZZLE_64B, CU_TENSOR_MAP_L2_PROMOTION_L2_256B, CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE) == CUDA_SUCCESS;
+    const CUresult r = ((EncodeTiled)f)(map, CU_TENSOR_MAP_DATA_TYPE_FLOAT16, rank, const_cast<void*>(at), size, stride, box, each, CU_TENSOR_MAP_INTERLEAVE_NONE,
+                                        D >= 64 ? CU_TENSOR_MAP_SWIZZLE_128B : CU_TENSOR_MAP_SWIZZLE_64B, CU_TENSOR_MAP_L2_PROMOTION_L2_256B, CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE);
+    return r == CUDA_SUCCESS ? cudaSuccess : r == CUDA_ERROR_INVALID_VALUE ? cudaErrorInvalidValue : cudaErrorUnknown;
 }
 
 template <int D, int NC>
@@ -657,7 +660,8 @@ qaq_status run_window(PrefillArgs a, const void* K, long sb, long sh, long st, i
     const cuuint64_t kstride[3] = {2ull * st, 2ull * (a.each_head ? sh : st), 2ull * (a.each_batch ? sb : st)};
     const cuuint64_t qsize[2] = {(cuuint64_t)D, (cuuint64_t)a.BH * a.n}, qstride[1] = {2ull * D};
     const cuuint32_t kbox[4] = {inner, PW_TILE, 1, 1}, qbox[2] = {inner, NC};
-    if (!describe(&keys, K, 4, ksize, kstride, kbox, D) || !describe(&queries, a.Q, 2, qsize, qstride, qbox, D)) return QAQ_ERR_CUDA;
+    QAQ_CUDA_TRY(describe(&keys, K, 4, ksize, kstride, kbox, D));
+    QAQ_CUDA_TRY(describe(&queries, a.Q, 2, qsize, qstride, qbox, D));
     static SmemSeen seen[3];
     static ClusterRoom room;
     QAQ_CUDA_TRY(qaq_allow_smem((const void*)window_kernel<D, NC, ONE_PASS>, PW_SMEM, seen[0]));

@@ -3,8 +3,11 @@ host-side argument checks answer before anything touches a device."""
 import ctypes as C
 import os
 import re
+import subprocess
+import sys
 
 import pytest
+import torch
 
 from paper_2403_04643_b200 import qaq
 
@@ -57,3 +60,23 @@ def test_bad_arguments_are_refused_on_the_host():
     assert L.qaq_select_bits(C.byref(cfg), C.byref(pol), None, None, 0, 0, 128, 4, None, None, None, None, None, None) == 1
     assert L.qaq_outlier_thresholds(C.byref(cfg), None, None, 0, 0, 128, 4, None, None, 0, None) == 1
     assert L.qaq_thresholds_workspace_bytes(C.byref(cfg), C.byref(n)) == 0 and n.value > 0
+
+
+@pytest.mark.skipif(torch.cuda.is_available(), reason="the pointers are not real: nothing may be launched")
+def test_the_reason_of_a_failed_description_is_kept():
+    # without a driver there is no description of the keys for the copies of tiles: the call says so, and why (in a process of its own:
+    # the reason is that of the most recent failure)
+    code = """
+import ctypes as C
+from paper_2403_04643_b200 import qaq
+cfg = qaq.make_config(1, 2, 64, 6000, 2, 8, 16, 0.01)
+L, n, p = qaq.lib(), C.c_size_t(), 1 << 20
+assert L.qaq_prefill_window_workspace_bytes(C.byref(cfg), 6000, C.byref(n)) == 0
+for _ in range(2):
+    assert L.qaq_last_cuda_error().decode() == "cudaSuccess" or _
+    assert L.qaq_prefill_window(C.byref(cfg), p, p, 2 * 6000 * 64, 6000 * 64, 64, 6000, 0.125, p, p, None, p, n.value, None) == 4
+    print(L.qaq_last_cuda_error().decode())
+"""
+    r = subprocess.run([sys.executable, "-c", code], capture_output=True, text=True, cwd=ROOT)
+    assert r.returncode == 0, r.stderr
+    assert len(r.stdout.split()) == 2 and "cudaSuccess" not in r.stdout.split()
