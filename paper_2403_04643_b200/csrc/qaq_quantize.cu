@@ -71,7 +71,8 @@ __device__ __forceinline__ uint32_t pool_take(uint32_t* pool, uint32_t amount, u
 // holds); the window in batches of 16 loads 3 % slower, eleven CTAs per SM 3 %.  32 (b,h) of one tile 7.0 against 7.7 us, of 16 tiles 10.5 against 17.2 us.
 // A one-token append is a chain of memory latencies (token count; table and metadata; the tile) and of instructions: eight
 // warps share pass 2, a round each, and nothing but the tile itself waits for the table.  32 (b,h), a tile of 1 to 64
-// tokens: 6.0 us, 6.3 with four warps, 8.4 with two and the window read in two parts.
+// tokens, captured: 5.5 us, 5.8 with four warps; where not all CTAs of eight warps run at once (96 registers: two to an SM) four are
+// better: 148 (b,h) 7.1 and 7.4, 160 9.6 and 7.5, 256 10.3 and 7.7, 512 18.8 and 12.0.
 // The integer unit limits this kernel (compares, minima, byte shuffles and selects all run there, at half rate), so sums,
 // shifts and packing are put where the multipliers are.
 __device__ __forceinline__ uint64_t pair_of(float a, float b) {
@@ -164,16 +165,15 @@ __device__ __forceinline__ uint32_t prefix(uint32_t x, int lane, uint32_t& sum) 
     sum = __shfl_sync(0xFFFFFFFFu, inc, 31);
     return inc - x;
 }
-constexpr int OPEN_WARPS = 8;           // warps of a CTA with an open tile
 constexpr uint32_t STORED = 1u << 30;   // of a slot's last word: the token is taken from the stored tile
 
 // One tile of one tensor, by two warps: half of its tokens each until the widths are known, half of the slots each from there.
-// OPEN: a tile that is begun, continued or closed, the only one of its (b,h) in the launch: its tokens up to s_lo are cached
-// already (and come from the tile as it is stored), those from s_lo to s_hi are new.
-template <int D, bool IS_V, bool OPEN>
+// OPEN (the number of warps; 0: whole tiles, two warps): a tile that is begun, continued or closed, the only one of its (b,h) in the
+// launch: its tokens up to s_lo are cached already (and come from the tile as it is stored), those from s_lo to s_hi are new.
+template <int D, bool IS_V, int OPEN>
 __device__ __forceinline__ void quantize_tile(const QuantArgs& a, TileScratch<D>& sm, uint8_t* stored_tile, uint32_t* list, const uint32_t cap) {
     constexpr int P = D / 32, TPI = 32 / P, IT = QAQ_TILE / 2 / TPI;  // lanes per token, tokens of a warp at a time, rounds
-    constexpr int PR = D / 8, NW = OPEN ? OPEN_WARPS : 2;             // 16-byte pieces of a row; warps
+    constexpr int PR = D / 8, NW = OPEN ? OPEN : 2;             // 16-byte pieces of a row; warps
     const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31, g = lane / P, p = lane % P;
     const bool counted = OPEN && a.d_count;
     const int t_old = counted ? *a.d_count : a.t_old;
@@ -475,8 +475,8 @@ __device__ __forceinline__ void quantize_tile(const QuantArgs& a, TileScratch<D>
 }
 
 // dynamic shared memory: the scratch, the tile as it is stored (OPEN), the warps' lists of outliers
-template <int D, bool OPEN>
-__global__ void __launch_bounds__(OPEN ? 32 * OPEN_WARPS : 64, OPEN ? 2 : (12)) quant_tiles_kernel(const QuantArgs a, uint32_t cap) {
+template <int D, int OPEN>
+__global__ void __launch_bounds__(OPEN ? 32 * OPEN : 64, OPEN == 0 ? 12 : OPEN == 4 ? 4 : 2) quant_tiles_kernel(const QuantArgs a, uint32_t cap) {
     extern __shared__ __align__(64) unsigned char tiles_smem[];
     TileScratch<D>& sm = *reinterpret_cast<TileScratch<D>*>(tiles_smem);
     uint8_t* stored_tile = tiles_smem + sizeof(TileScratch<D>);
@@ -487,16 +487,16 @@ __global__ void __launch_bounds__(OPEN ? 32 * OPEN_WARPS : 64, OPEN ? 2 : (12)) 
 }
 
 // tiles.x tiles of every (b,h), all whole, or one that is not (or may not be)
-template <int D, bool OPEN>
+template <int D, int OPEN>
 qaq_status launch_tiles(int tiles, int BH, const QuantArgs& a, double alpha, cudaStream_t s) {
     // the lists hold a tenth more than the share of outliers asked for gives a tile, and some (twelve CTAs per SM at 1 %)
     const uint32_t want = (uint32_t)(alpha * (QAQ_TILE * D) * 1.1) + 60, cap = (want < 2048 ? want : 2048) / 2;
     const size_t smem = sizeof(TileScratch<D>) + (OPEN ? qaqc::tile_bytes_max(D) + 16 : 0) + 2 * cap * sizeof(uint32_t);
     static_assert(sizeof(TileScratch<D>) + qaqc::tile_bytes_max(D) + 16 + 2048 * sizeof(uint32_t) <= 48 * 1024, "shared memory that needs no attribute");
-    QAQ_CUDA_TRY(qaq_launch(quant_tiles_kernel<D, OPEN>, dim3((unsigned)tiles, (unsigned)BH, 2), dim3(OPEN ? 32 * OPEN_WARPS : 64), smem, s, a, cap));
+    QAQ_CUDA_TRY(qaq_launch(quant_tiles_kernel<D, OPEN>, dim3((unsigned)tiles, (unsigned)BH, 2), dim3(OPEN ? 32 * OPEN : 64), smem, s, a, cap));
     return QAQ_OK;
 }
-template <bool OPEN>
+template <int OPEN>
 qaq_status launch(int D, int tiles, int BH, const QuantArgs& a, double alpha, cudaStream_t s) {
     switch (D) {
         case 32: return launch_tiles<32, OPEN>(tiles, BH, a, alpha, s);
@@ -504,6 +504,10 @@ qaq_status launch(int D, int tiles, int BH, const QuantArgs& a, double alpha, cu
         case 128: return launch_tiles<128, OPEN>(tiles, BH, a, alpha, s);
     }
     return QAQ_ERR_UNSUPPORTED_SHAPE;
+}
+// eight warps while all CTAs run at once, else four (figures at the top)
+qaq_status launch_open(int D, int BH, const QuantArgs& a, double alpha, cudaStream_t s) {
+    return 2 * BH <= 2 * 148 ? launch<8>(D, 1, BH, a, alpha, s) : launch<4>(D, 1, BH, a, alpha, s);
 }
 
 // Widths alone: one CTA = 64 tokens of one (b,h); P = D/32 lanes own a token, each lane 32 consecutive channels (64 bytes) of
@@ -598,18 +602,18 @@ qaq_status qaq_launch_append(qaq_cache* c, const void* K, const void* V, long sb
     if (cur % QAQ_TILE != 0) {  // head: finish (or extend) the open tile
         const int end = min(t1, (cur / QAQ_TILE + 1) * QAQ_TILE);
         a.tok_lo = cur - t0; a.tok_hi = end - t0; a.first_tile = cur / QAQ_TILE;
-        if ((stt = launch<true>(D, 1, BH, a, c->cfg.outlier_frac, s)) != QAQ_OK) return stt;
+        if ((stt = launch_open(D, BH, a, c->cfg.outlier_frac, s)) != QAQ_OK) return stt;
         cur = end;
     }
     const int full_end = t1 / QAQ_TILE * QAQ_TILE;
     if (cur < full_end) {       // body: whole tiles
         a.tok_lo = cur - t0; a.tok_hi = full_end - t0; a.first_tile = cur / QAQ_TILE;
-        if ((stt = launch<false>(D, (full_end - cur) / QAQ_TILE, BH, a, c->cfg.outlier_frac, s)) != QAQ_OK) return stt;
+        if ((stt = launch<0>(D, (full_end - cur) / QAQ_TILE, BH, a, c->cfg.outlier_frac, s)) != QAQ_OK) return stt;
         cur = full_end;
     }
     if (cur < t1) {             // tail: a new, partly filled tile
         a.tok_lo = cur - t0; a.tok_hi = t1 - t0; a.first_tile = cur / QAQ_TILE;
-        if ((stt = launch<true>(D, 1, BH, a, c->cfg.outlier_frac, s)) != QAQ_OK) return stt;
+        if ((stt = launch_open(D, BH, a, c->cfg.outlier_frac, s)) != QAQ_OK) return stt;
     }
     c->tokens = t1;
     return QAQ_OK;
@@ -664,5 +668,5 @@ extern "C" qaq_status qaq_stream_append(qaq_cache* c, const void* k_new, const v
     a.k = c->t[0]; a.v = c->t[1]; a.pool_bytes = c->pool_bytes; a.ocap = c->ocap;
     a.tmax_pad = c->tmax_pad; a.ntiles = c->ntiles; a.status = c->d_status;
     a.d_count = qaq_d_count(c); a.d_ticket = qaq_d_ticket(c); a.max_tokens = (int)c->cfg.max_tokens;
-    return launch<true>(D, 1, c->BH, a, c->cfg.outlier_frac, (cudaStream_t)stream);
+    return launch_open(D, c->BH, a, c->cfg.outlier_frac, (cudaStream_t)stream);
 }

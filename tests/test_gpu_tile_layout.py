@@ -235,3 +235,32 @@ def test_sequences_of_many_heads_whose_clusters_may_not_all_run_at_once(heads, t
     assert_attention_close(out.cpu().numpy(), ref.X)
     S = scores.cpu().numpy().astype(np.float64)
     assert np.all(np.abs(S - ref.S) <= 1e-6 + 1e-2 * ref.S) and np.allclose(S.sum(1), 1.0, atol=1e-3)
+
+
+@pytest.mark.parametrize("D", [32, 64, 128])
+@pytest.mark.parametrize("heads", [148, 149])
+def test_open_tiles_of_many_heads(D, heads):
+    # one-token and longer appends by CTAs of eight warps (148) and of four (149): the cache equals the oracle's, and one filled at once
+    T = 150
+    g = torch.Generator().manual_seed(heads + D)
+    K, V = (torch.randn((1, heads, T, D), generator=g).half() for _ in range(2))
+    bits = torch.randint(1, 9, (heads, T), generator=g).to(torch.uint8).cuda()
+    cfg = qaq.make_config(1, heads, D, T, 1, 8, 1, 0.02)
+    Kd, Vd = K.cuda(), V.cuda()
+    thr = qaq.qaq_outlier_thresholds(cfg, Kd, Vd)
+    caches = []
+    for cuts in ((0, T), (0, 20, 21, 63, 64, 65, 129, 130, T)):
+        cache = qaq.Cache(cfg)
+        for a, b in zip(cuts, cuts[1:]):
+            w = bits[:, a:b].contiguous()
+            qaq.qaq_quantize_append(cache, Kd[:, :, a:b], Vd[:, :, a:b], thr, bitsK=w, bitsV=w)
+        caches.append([qaq.qaq_cache_export(cache, x) for x in (0, 1)])
+    th = thr.cpu().numpy()
+    for x, X in enumerate((K, V)):
+        a, b = caches[0][x], caches[1][x]
+        assert b["stats"].device_status == 0
+        assert all(torch.equal(a[k], b[k]) for k in ("bits", "mn", "step", "off", "codes", "rowptr"))
+        for bh in (0, 77, heads - 1):
+            want = oracle.quantize(X[0, bh].numpy().view("uint16"), th[bh, 2 * x], th[bh, 2 * x + 1], bits[bh].cpu().numpy())
+            nb = int(want.off[T])
+            assert (b["codes"][bh, :nb].cpu().numpy() == want.stream).all() and (b["rowptr"][bh].cpu().numpy() == want.rowptr).all()
