@@ -133,10 +133,15 @@ static inline cudaError_t qaq_allow_smem(const void* kernel, size_t smem, SmemSe
 }
 // How many clusters of k CTAs of a kernel run at once: asked once per kernel, k and context (whose id goes with the answer).
 struct ClusterRoom { std::atomic<unsigned long long> known[9]; };
-template <class K>
-int clusters_at_once(K kernel, int threads, size_t smem, int k, ClusterRoom& room) {
+struct ContextName {                             // (who asks for several sizes looks it up once)
     unsigned long long id = 0;
-    const bool named = qaq_context_id(id);
+    bool named;
+    ContextName() { named = qaq_context_id(id); }
+};
+template <class K>
+int clusters_at_once(K kernel, int threads, size_t smem, int k, ClusterRoom& room, const ContextName& context = ContextName()) {
+    const unsigned long long id = context.id;
+    const bool named = context.named;
     const unsigned long long was = room.known[k].load(std::memory_order_acquire);
     if (named && (was >> 16) == id + 1) return (int)(was & 0xFFFFu);
     cudaLaunchAttribute at;

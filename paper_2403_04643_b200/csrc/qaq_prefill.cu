@@ -11,14 +11,14 @@
 // (tcgen05.mma, binary16 in, binary32 sums in tensor memory: a token a lane, a query a column), so neither the keys nor the
 // logits pass through registers on their way there, and a row's 32 consecutive tokens are one store of a warp.  What the keys
 // wait for in the meantime decides between three ways:
-//   window_short_kernel   few tiles in all: the logits in registers, many CTAs per SM.
+//   window_short_kernel   few tiles in all (64 of a (b,h) at most): the logits in registers, several CTAs per SM.
 //   window_kernel         one pass: resident CTAs, the logits of a (b,h) in the tensor memory of a cluster until the statistics of its
 //                         rows are known; K is read once and the rows written once.
-//                         Two passes, (b,h) longer than that (8192 tokens with 64 rows, 16384 with 32, 32768 with 16): statistics per
-//                         chunk of tokens, then the logits again and the rows.
+//                         Two passes, (b,h) longer than that (8192 tokens with 64 rows, 16384 with 32, 32768 with 16) or too few to keep
+//                         the SMs busy in clusters: statistics per chunk of tokens, then the logits again and the rows.
 // Before (mma.sync fragments from global memory, logits in shared memory; beyond 4096 tokens two passes), now: 256 (b,h) of 4096
 // tokens, 32 rows 129 and 70 us, with 64 rows 345 and 115; 160 of 8192, 64 rows 321 and 152; 32 of 32768, 32 rows 187 and 118; 32 of 333
-// 8.3 and 5.5; 256 of 300 11.9 and 9.2.
+// 8.3 and 5.5; 256 of 300 11.9 and 9.2; with head_dim 32 and 5 rows 64 of 2048 tokens 7.0 and 7.1, 192 of 600 (head_dim 64) 13.6 and 7.8.
 #include <cuda.h>
 
 #include "qaq_internal.cuh"
@@ -483,11 +483,12 @@ __global__ void __launch_bounds__(PW_THREADS, 1) window_kernel(const __grid_cons
     }
 }
 
-// ---- few tiles in all: a thread keeps the logits of its token in registers, a CTA is one tile to four (four warps each), and the CTAs
-// of a (b,h) form a cluster where it has more than one.  No warp waits for another's work but at barriers, several CTAs share an
+// ---- few tiles in all: a thread keeps the logits of its token (up to 16 rows: or of two) in registers, a CTA is one group of four warps to
+// four, a tile (or two) each, and the CTAs of a (b,h) form a cluster where it has more than one.  No warp waits for another's work but at barriers, several CTAs share an
 // SM, keys come by plain asynchronous copies.  Tensor memory is given back before the CTAs of a cluster wait for each other, so that
-// nobody waits for it who is waited for.  32 (b,h) of 333 tokens, 32 rows: 5.4 us, the kernel above 7.8 us.
-constexpr int PS_TILES = 4;            // tiles of a CTA at most
+// nobody waits for it who is waited for.  32 (b,h) of 333 tokens, 32 rows: 5.6 us, the kernel above 7.8 us; of 2048 tokens 10.7 and 12.8;
+// of 4096 tokens, head_dim 32, 5 rows 7.2 us with two tiles to a group, 10.2 with one, 11.7.
+constexpr int PS_GROUPS = 4;           // groups of four warps of a CTA at most
 template <int ROW_BYTES, int ROWS>     // rows of a [.][D] operand on their way to shared memory, by four warps; what lies beyond `rows` is not touched
 __device__ __forceinline__ void fetch_rows(uint32_t dst, const __half* src, long stride, int rows, int D, int thread) {
     const int PR = D / 8, row = thread / PR, c = thread % PR, step = 128 / PR;           // 16-byte pieces of a row; rows at a time, a multiple of 8
@@ -498,22 +499,24 @@ __device__ __forceinline__ void fetch_rows(uint32_t dst, const __half* src, long
     for (int r = row; r < ROWS; r += step, src += step * stride, dst += step * ROW_BYTES)
         if (r < rows) asm volatile("cp.async.cg.shared.global [%0], [%1], 16;" ::"r"(dst), "l"(src) : "memory");
 }
-template <int D, int NC>
-__global__ void __launch_bounds__(128 * PS_TILES, 1) window_short_kernel(const PrefillArgs a, const __half* K, long sb, long sh, long st) {
+// TP: tokens of a thread, tiles of a group of four warps.
+constexpr int short_ctas(int NC) { return NC <= 32 ? 2 : 1; }          // of PS_GROUPS groups to an SM, for their registers
+template <int D, int NC, int TP>
+__global__ void __launch_bounds__(128 * PS_GROUPS, short_ctas(NC)) window_short_kernel(const PrefillArgs a, const __half* K, long sb, long sh, long st) {
     using W = Window<D, NC, STATS>;
     constexpr int RB = W::ROW_BYTES, CW = NC < 32 ? NC : 32;
     const float NEG = __int_as_float(0xff800000), LOWEST = __int_as_float(0xff7fffff), sc = a.scale * 1.4426950408889634f;
     extern __shared__ unsigned char s_dyn[];
-    __shared__ alignas(8) unsigned long long s_bar[PS_TILES];
+    __shared__ alignas(8) unsigned long long s_bar[PS_GROUPS];
     __shared__ uint32_t s_tmem, s_failed;                    // s_failed: a wait ran out
-    __shared__ alignas(16) float s_max[4 * PS_TILES][NC], s_sum[4 * PS_TILES][NC];       // of a warp: reference and sum of every row over its tokens
+    __shared__ alignas(16) float s_max[4 * PS_GROUPS][NC], s_sum[4 * PS_GROUPS][NC];       // of a warp: reference and sum of every row over its tokens
     __shared__ float2 s_all[PW_CLUSTER][NC];                 // the same of every CTA of the cluster, which all write here
     const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31, group = warp >> 2, groups = blockDim.x >> 7, warps = 4 * groups;
     const int bh = blockIdx.y, rank = blockIdx.x, ncta = gridDim.x;
-    const uint32_t base = (smem_addr(s_dyn) + 1023u) & ~1023u, queries = base + groups * W::TILE_BYTES, bar = smem_addr(s_bar) + 8 * group;
-    const uint32_t columns = max(32, 1 << (32 - __clz(groups * NC - 1)));                // (a power of two)
+    const uint32_t base = (smem_addr(s_dyn) + 1023u) & ~1023u, tile = base + group * TP * W::TILE_BYTES, queries = base + groups * TP * W::TILE_BYTES, bar = smem_addr(s_bar) + 8 * group;
+    const uint32_t columns = max(32, 1 << (32 - __clz(groups * TP * NC - 1)));                // (a power of two)
     if (tid == 0) {
-        for (int i = 0; i < PS_TILES; ++i) bar_init(smem_addr(s_bar) + 8 * i, 1);
+        for (int i = 0; i < PS_GROUPS; ++i) bar_init(smem_addr(s_bar) + 8 * i, 1);
         s_failed = 0;
         asm volatile("fence.proxy.async.shared::cta;" ::: "memory");
     }
@@ -521,8 +524,12 @@ __global__ void __launch_bounds__(128 * PS_TILES, 1) window_short_kernel(const P
     // first half of a cluster barrier: by the time the row statistics are exchanged every CTA of the cluster is known
     // to be running (its shared memory may be written)
     if (ncta > 1) asm volatile("barrier.cluster.arrive.release.aligned;" ::: "memory");
-    const int t_group = (rank * groups + group) * PW_TILE;
-    fetch_rows<RB, PW_TILE>(base + group * W::TILE_BYTES, K + (size_t)(bh / a.H) * sb + (size_t)(bh % a.H) * sh + (ptrdiff_t)t_group * st, st, a.T - t_group, D, tid & 127);
+    const int t_group = (rank * groups + group) * TP * PW_TILE;
+#pragma unroll
+    for (int i = 0; i < TP; ++i) {
+        const int t0 = t_group + i * PW_TILE;
+        fetch_rows<RB, PW_TILE>(tile + i * W::TILE_BYTES, K + (size_t)(bh / a.H) * sb + (size_t)(bh % a.H) * sh + (ptrdiff_t)t0 * st, st, a.T - t0, D, tid & 127);
+    }
     if (group == 0) fetch_rows<RB, NC>(queries, a.Q + (size_t)bh * a.n * D, D, a.n, D, tid);      // (columns of rows that are not there are not looked at)
     asm volatile("cp.async.commit_group;" ::: "memory");
     if (warp == 0)
@@ -534,21 +541,24 @@ __global__ void __launch_bounds__(128 * PS_TILES, 1) window_short_kernel(const P
     tmem_after_sync();
     const uint32_t acc = *(volatile uint32_t*)&s_tmem;
     if ((tid & 127) == 0) {
-        multiply<D, NC>(acc + group * NC, base + group * W::TILE_BYTES, queries);
+#pragma unroll
+        for (int i = 0; i < TP; ++i) multiply<D, NC>(acc + (group * TP + i) * NC, tile + i * W::TILE_BYTES, queries);
         tensor_done(bar);
     }
     __syncwarp();
     if (!bar_wait(bar, 0u)) s_failed = 1;
     __syncwarp();
     tmem_after_sync();
-    float x[NC];
+    float x[TP][NC];
 #pragma unroll
-    for (int h = 0; h < NC; h += CW) {
-        float v[CW];
-        load_acc(acc + ((uint32_t)(32 * (warp & 3)) << 16) + group * NC + h, v);
+    for (int i = 0; i < TP; ++i)
 #pragma unroll
-        for (int c = 0; c < CW; ++c) x[h + c] = v[c];
-    }
+        for (int h = 0; h < NC; h += CW) {
+            float v[CW];
+            load_acc(acc + ((uint32_t)(32 * (warp & 3)) << 16) + (group * TP + i) * NC + h, v);
+#pragma unroll
+            for (int c = 0; c < CW; ++c) x[i][h + c] = v[c];
+        }
     // ---- per warp: maximum of every row over its tokens, the logits become powers of two relative to it (0 where the query cannot
     //      see the token), and their sum
     const int t = t_group + 32 * (warp & 3) + lane, hidden = t - (a.T - a.n);
@@ -558,9 +568,14 @@ __global__ void __launch_bounds__(128 * PS_TILES, 1) window_short_kernel(const P
         float m[8], sum[8];
 #pragma unroll
         for (int c = 0; c < 8; ++c) {
-            const bool seen = c0 + c >= hidden;
-            m[c] = warp_max(seen ? x[c0 + c] * sc : NEG);
-            sum[c] = x[c0 + c] = seen ? pow2(fmaf(x[c0 + c], sc, -fmaxf(m[c], LOWEST))) : 0.f;      // (a maximum of -inf: zeros)
+            float top = NEG;
+#pragma unroll
+            for (int i = 0; i < TP; ++i) top = fmaxf(top, c0 + c >= hidden + i * PW_TILE ? x[i][c0 + c] * sc : NEG);
+            m[c] = warp_max(top);
+            sum[c] = 0.f;
+#pragma unroll
+            for (int i = 0; i < TP; ++i)
+                sum[c] += x[i][c0 + c] = c0 + c >= hidden + i * PW_TILE ? pow2(fmaf(x[i][c0 + c], sc, -fmaxf(m[c], LOWEST))) : 0.f;      // (a maximum of -inf: zeros)
         }
         if (lane == 0) {
             *reinterpret_cast<float4*>(&s_max[warp][c0]) = make_float4(m[0], m[1], m[2], m[3]);
@@ -603,28 +618,23 @@ __global__ void __launch_bounds__(128 * PS_TILES, 1) window_short_kernel(const P
     float* row = a.ring + ((size_t)bh * a.n + (a.n - 1)) * a.T + t;
     if (__any_sync(0xFFFFFFFFu, lost)) {                     // the tokens of the CTA, by all of its warps alike
         for (int c = 0; c < a.n; ++c, row -= a.T)
-            if (t < a.T) *row = __uint_as_float(QAQ_SCORE_LOST);
+            for (int i = 0; i < TP; ++i)
+                if (t + i * PW_TILE < a.T) row[i * PW_TILE] = __uint_as_float(QAQ_SCORE_LOST);
     } else {
 #pragma unroll
         for (int c = 0; c < NC; ++c) {
             if (c >= a.n) break;
-            const float y = x[c] * __shfl_sync(0xFFFFFFFFu, f[c / CW], c % CW);
-            if (t < a.T) *row = y;
+            const float y = __shfl_sync(0xFFFFFFFFu, f[c / CW], c % CW);
+#pragma unroll
+            for (int i = 0; i < TP; ++i)
+                if (t + i * PW_TILE < a.T) row[i * PW_TILE] = x[i][c] * y;
             row -= a.T;
         }
     }
-    if (t < a.T) a.nvalid[(size_t)bh * a.T + t] = (uint8_t)min(a.n, a.T - t);
+#pragma unroll
+    for (int i = 0; i < TP; ++i)
+        if (t + i * PW_TILE < a.T) a.nvalid[(size_t)bh * a.T + t + i * PW_TILE] = (uint8_t)min(a.n, a.T - t - i * PW_TILE);
 }
-template <int D, int NC>
-qaq_status run_short(const PrefillArgs& a, const void* K, long sb, long sh, long st, int groups, int ncta, cudaStream_t s) {
-    using W = Window<D, NC, STATS>;
-    static SmemSeen seen;
-    QAQ_CUDA_TRY(qaq_allow_smem((const void*)window_short_kernel<D, NC>, 1024 + PS_TILES * W::TILE_BYTES + W::QUERY_BYTES, seen));
-    QAQ_CUDA_TRY(qaq_launch_cluster(window_short_kernel<D, NC>, dim3((unsigned)ncta, (unsigned)a.BH), dim3(128u * groups), ncta, 1024 + groups * W::TILE_BYTES + W::QUERY_BYTES, s,
-                                    a, (const __half*)K, sb, sh, st));
-    return QAQ_OK;
-}
-
 // Descriptions of K ([batch][head][token][channel] with the caller's strides) and of the queries for the copies of tiles.
 typedef CUresult (*EncodeTiled)(CUtensorMap*, CUtensorMapDataType, cuuint32_t, void*, const cuuint64_t*, const cuuint64_t*, const cuuint32_t*, const cuuint32_t*,
                                 CUtensorMapInterleave, CUtensorMapSwizzle, CUtensorMapL2promotion, CUtensorMapFloatOOBfill);
@@ -644,14 +654,80 @@ cudaError_t describe(CUtensorMap* map, const void* at, int rank, const cuuint64_
     return r == CUDA_SUCCESS ? cudaSuccess : r == CUDA_ERROR_INVALID_VALUE ? cudaErrorInvalidValue : cudaErrorUnknown;
 }
 
+// Which way: the one whose time, estimated from the work of the fullest SM, is the least.  The figures (us) are fitted to some 1300 sizes
+// from 4 to 320 (b,h), 100 to 8192 tokens, measured each way: off by 11, 8 and 7 % (window_short_kernel, by rows), 6, 5 and 4 % (one pass).
+struct Costs {
+    float start, cluster, cta, group[2], turn; // window_short_kernel: a launch, one of clusters, every CTA of an SM, every group of warps of them (of one tile, of
+                                               // two), every time that CTAs wait for others to end (for clusters 1 + D / 64 times that)
+    float resident, item, tile, bytes;         // window_kernel: a launch, every (b,h) of a CTA, every tile, its bytes with head_dim 128
+};
+constexpr Costs costs_of(int NC) {
+    return NC == 16 ? Costs{1.74f, 1.18f, 0.86f, {0.45f, 0.64f}, 3.f, 6.1f, 0.79f, 0.35f, 0.54f}
+         : NC == 32 ? Costs{2.53f, 1.13f, 0.87f, {0.79f, 0.f}, 2.5f, 6.25f, 1.06f, 0.49f, 0.52f}
+                    : Costs{4.2f, 1.22f, 0.82f, {1.14f, 0.f}, 5.f, 4.65f, 2.66f, 1.05f, 0.46f};
+}
+struct ShortPlan { float time; int tp, groups, ncta; };
+template <int D, int NC, int TP>
+constexpr int short_smem(int groups) { return 1024 + groups * TP * Window<D, NC, STATS>::TILE_BYTES + Window<D, NC, STATS>::QUERY_BYTES; }
+// The best plan with TP tiles to a group, if it is better than `best` (alone[k]: so many clusters of k CTAs have an SM for every CTA).
+template <int D, int NC, int TP>
+void plan_short(int BH, int tiles, const int* alone, ShortPlan& best) {
+    constexpr Costs cost = costs_of(NC);
+    for (int g = 1; g <= PS_GROUPS && (g - 1) * TP < tiles; ++g) {
+        const int k = (tiles + g * TP - 1) / (g * TP), smem = short_smem<D, NC, TP>(g) + NC * 200 + 1024;         // (200 bytes a row: the statistics)
+        if (k > PW_CLUSTER || alone[k] < 1 || smem > PW_SMEM) continue;
+        const int ctas = (BH + alone[k] - 1) / alone[k], at_once = min(short_ctas(NC) * PS_GROUPS / g, (PW_SMEM + 1024) / smem);
+        const float time = cost.start + (k > 1 ? cost.cluster : 0.f) + (float)ctas * (cost.cta + (float)g * cost.group[TP - 1]) +
+                           (float)((ctas - 1) / at_once) * (k > 1 ? 1.f + D / 64.f : 1.f) * cost.turn;
+        if (time < best.time) best = {time, TP, g, k};
+    }
+}
+template <int D, int NC, int TP>
+qaq_status run_short(const PrefillArgs& a, const void* K, long sb, long sh, long st, const ShortPlan& p, cudaStream_t s) {
+    constexpr int most = PW_SMEM - NC * 200 - 1024, all = short_smem<D, NC, TP>(PS_GROUPS);
+    static SmemSeen seen;
+    QAQ_CUDA_TRY(qaq_allow_smem((const void*)window_short_kernel<D, NC, TP>, all < most ? all : most, seen));
+    QAQ_CUDA_TRY(qaq_launch_cluster(window_short_kernel<D, NC, TP>, dim3((unsigned)p.ncta, (unsigned)a.BH), dim3(128u * p.groups), p.ncta, short_smem<D, NC, TP>(p.groups), s,
+                                    a, (const __half*)K, sb, sh, st));
+    return QAQ_OK;
+}
+
 template <int D, int NC>
 qaq_status run_window(PrefillArgs a, const void* K, long sb, long sh, long st, int batch, cudaStream_t s) {
     using W = Window<D, NC, ONE_PASS>;
+    constexpr Costs cost = costs_of(NC);
+    constexpr float per_tile = cost.tile + cost.bytes * D / 128.f;
     const int tiles = (a.T + PW_TILE - 1) / PW_TILE;
-    // few tiles: one-tile CTAs while all of them run at once (two to an SM: 32 (b,h) of 1000 tokens 9.2 us, 9.0 by the kernel below, of 333
-    // 6.0 and 7.8), else a (b,h) to a CTA (256 of 300 tokens 9.2 and 12.8)
-    if (tiles <= PW_CLUSTER && (long long)a.BH * tiles <= 2 * 148) return run_short<D, NC>(a, K, sb, sh, st, 1, tiles, s);
-    if (tiles <= PS_TILES) return run_short<D, NC>(a, K, sb, sh, st, tiles, 1, s);
+    static SmemSeen seen[3];
+    static ClusterRoom room;
+    const ContextName context;
+    QAQ_CUDA_TRY(qaq_allow_smem((const void*)window_kernel<D, NC, ONE_PASS>, PW_SMEM, seen[0]));
+    // two passes: chunks of at least PW_CHUNK tokens (the workspace's), as long as every SM gets eight
+    const int chunk = max(PW_CHUNK / PW_TILE, (int)((long long)tiles * a.BH / (8 * 148)));
+    const long long chunks = (long long)a.BH * ((tiles + chunk - 1) / chunk);
+    float least = cost.resident + 2.f * (float)((chunks + 147) / 148 * chunk) * per_tile;
+    // one pass: the size of the cluster; one that leaves no accumulators for a second (b,h) has to be that much better
+    int alone[PW_CLUSTER + 1] = {}, best = 0, each = 0;
+    float one_pass = 0.f;
+    for (int k = 1; k <= PW_CLUSTER && k <= tiles; ++k) {
+        const int n = (tiles + k - 1) / k;
+        alone[k] = clusters_at_once(window_kernel<D, NC, ONE_PASS>, PW_THREADS, PW_SMEM, k, room, context);
+        if (n > W::SLOTS || (tiles + n - 1) / n != k || alone[k] < 1) continue;
+        const int items = (a.BH + alone[k] - 1) / alone[k];
+        const float time = cost.resident + (float)items * cost.item + (float)items * (float)n * per_tile, chosen_by = time * (2 * n > W::SLOTS ? 1.08f : 1.f);
+        if (time < least && (!best || chosen_by < one_pass)) { best = k; one_pass = chosen_by; each = n; }
+    }
+    if (best) least = one_pass;
+    // few tiles
+    if (tiles <= PW_CLUSTER * PS_GROUPS * 2) {
+        ShortPlan plan = {least, 0, 0, 0};
+        plan_short<D, NC, 1>(a.BH, tiles, alone, plan);
+        if constexpr (NC == 16) {
+            plan_short<D, NC, 2>(a.BH, tiles, alone, plan);
+            if (plan.tp == 2) return run_short<D, NC, 2>(a, K, sb, sh, st, plan, s);
+        }
+        if (plan.tp == 1) return run_short<D, NC, 1>(a, K, sb, sh, st, plan, s);
+    }
     CUtensorMap keys, queries;
     const cuuint32_t inner = D >= 64 ? 64 : 32;
     // (a stride of zero is a dimension of one in the description; the stride of such a dimension is never used)
@@ -662,29 +738,15 @@ qaq_status run_window(PrefillArgs a, const void* K, long sb, long sh, long st, i
     const cuuint32_t kbox[4] = {inner, PW_TILE, 1, 1}, qbox[2] = {inner, NC};
     QAQ_CUDA_TRY(describe(&keys, K, 4, ksize, kstride, kbox, D));
     QAQ_CUDA_TRY(describe(&queries, a.Q, 2, qsize, qstride, qbox, D));
-    static SmemSeen seen[3];
-    static ClusterRoom room;
-    QAQ_CUDA_TRY(qaq_allow_smem((const void*)window_kernel<D, NC, ONE_PASS>, PW_SMEM, seen[0]));
-    // the size of the cluster: the fewest tiles one after the other, and where that is the same, accumulators of two (b,h) at a time
-    int best = 0, most = 0;
-    long long least = 0;
-    for (int k = 1; k <= PW_CLUSTER && k <= tiles; ++k) {
-        const int each = (tiles + k - 1) / k;
-        if (each > W::SLOTS || (tiles + each - 1) / each != k) continue;
-        const int n = clusters_at_once(window_kernel<D, NC, ONE_PASS>, PW_THREADS, PW_SMEM, k, room);
-        if (n < 1) continue;
-        const long long time = (long long)((a.BH + n - 1) / n) * each;
-        if (!best || time < least || (time == least && 2 * a.tiles > W::SLOTS)) { best = k; least = time; a.tiles = each; most = min(a.BH, n); }
-    }
     if (best) {
-        QAQ_CUDA_TRY(qaq_launch_cluster(window_kernel<D, NC, ONE_PASS>, dim3((unsigned)(most * best)), dim3(PW_THREADS), best, PW_SMEM, s, keys, queries, a));
+        a.tiles = each;
+        QAQ_CUDA_TRY(qaq_launch_cluster(window_kernel<D, NC, ONE_PASS>, dim3((unsigned)(min(a.BH, alone[best]) * best)), dim3(PW_THREADS), best, PW_SMEM, s, keys, queries, a));
         return QAQ_OK;
     }
-    // chunks of at least PW_CHUNK tokens (the workspace's), as long as every SM gets eight
     QAQ_CUDA_TRY(qaq_allow_smem((const void*)window_kernel<D, NC, STATS>, PW_SMEM, seen[1]));
     QAQ_CUDA_TRY(qaq_allow_smem((const void*)window_kernel<D, NC, ROWS>, PW_SMEM, seen[2]));
-    a.tiles = max(PW_CHUNK / PW_TILE, (int)((long long)tiles * a.BH / (8 * 148)));
-    a.nchunk = (tiles + a.tiles - 1) / a.tiles;
+    a.tiles = chunk;
+    a.nchunk = (tiles + chunk - 1) / chunk;
     const dim3 grid((unsigned)min(148, a.BH * a.nchunk));
     QAQ_CUDA_TRY(qaq_launch(window_kernel<D, NC, STATS>, grid, dim3(PW_THREADS), PW_SMEM, s, keys, queries, a));
     QAQ_CUDA_TRY(qaq_launch(window_kernel<D, NC, ROWS>, grid, dim3(PW_THREADS), PW_SMEM, s, keys, queries, a));

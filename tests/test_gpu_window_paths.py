@@ -38,16 +38,22 @@ def keys(B, H, T, D, token_major, seed):
 
 @pytest.mark.parametrize("D", [32, 64, 128])
 @pytest.mark.parametrize("heads,T,n", [
-    (2, 1, 1), (2, 127, 16), (2, 129, 17), (3, 1024, 33),           # a cluster of one-tile CTAs
-    (320, 128, 32), (110, 300, 5), (80, 512, 64),                   # up to four tiles in a CTA
-    (40, 1025, 64), (75, 513, 32), (9, 2048, 16), (5, 4097, 32), (3, 8191, 64),      # one pass, clusters of several sizes
-    (160, 640, 1),                                                  # more (b,h) than CTAs
-    (2, 8193, 64), (2, 16385, 32),                                  # two passes
+    (2, 1, 1), (2, 127, 16), (2, 129, 17), (3, 1024, 33),           # few tiles: clusters of one-tile CTAs
+    (320, 128, 32), (110, 300, 5), (160, 385, 64), (320, 512, 17),  # a (b,h) to a CTA, in turn too
+    (80, 512, 64), (32, 1025, 32), (24, 1793, 64), (12, 3969, 32),  # clusters of CTAs of two to four tiles, the last of them empty
+    (40, 600, 16), (24, 1281, 5), (64, 1921, 1), (32, 4097, 16), (9, 8190, 16),      # up to 16 rows: two tiles to a group of warps
+    (160, 640, 1), (300, 640, 33), (100, 1025, 64), (9, 2048, 16), (5, 4097, 32), (3, 8191, 64),   # one pass, clusters of several sizes
+    (256, 2000, 64), (160, 1700, 32), (70, 8100, 64), (96, 5000, 16),                # one pass, several (b,h) per cluster
+    (2, 8193, 64), (2, 16385, 32), (2, 33000, 16), (1, 9000, 5),    # two passes
+    (24, 8193, 64), (20, 16400, 17),                                # two passes, several chunks of a CTA
+    (96, 8193, 64),                                                 # two passes, chunks of more than four tiles
 ])
 def test_window_rows_of_every_way(D, heads, T, n):
     K = keys(1, heads, T, D, token_major=heads % 2 == 1, seed=D + T)
     Q = torch.randn((heads, n, D), generator=torch.Generator().manual_seed(n)).half()
-    rows_match(K, Q, heads, {0, heads // 2, heads - 1})
+    ring = rows_match(K, Q, heads, {0, heads // 2, heads - 1})
+    seen = min(n, T)                                                # queries that exist: their rows come first
+    assert torch.allclose(ring[:, :seen].sum(2), torch.ones(heads, seen, device="cuda"), atol=1e-4) and (ring[:, seen:] == 0).all()
 
 
 @pytest.mark.parametrize("T,n", [(700, 40), (4100, 32), (8200, 64)])
@@ -77,7 +83,7 @@ def test_heads_that_share_keys_and_keys_that_are_not_numbers(T):
 
 
 @pytest.mark.parametrize("D", [32, 64, 128])
-@pytest.mark.parametrize("heads,T,n", [(2, 100, 5), (2, 700, 33), (300, 400, 16), (3, 1500, 16), (2, 3000, 32), (2, 4100, 64), (2, 9000, 64)])
+@pytest.mark.parametrize("heads,T,n", [(2, 100, 5), (2, 700, 33), (300, 400, 16), (3, 1500, 16), (2, 3000, 32), (160, 1700, 32), (2, 4100, 64), (2, 9000, 64)])
 def test_logits_of_minus_infinity(D, heads, T, n):
     # the first two thirds of the tokens have logits of -inf in every row, the others are far below zero: entries of 0, and rows that
     # are normalised over the rest (logits of about -1000, whose binary32 sums are off by 2^-24 of 8000 a few times: 1e-3 of an entry)
