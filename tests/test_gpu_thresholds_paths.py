@@ -83,9 +83,10 @@ def test_tails_that_lie_in_one_part_of_the_sequence(alpha, part, factor):
     check(K, V, wl, alpha)
 
 
-@pytest.mark.parametrize("D,T,alpha", [(128, 4096, 0.01), (64, 2049, 0.3), (32, 700, 1.0), (128, 4097, 0.2)])
+@pytest.mark.parametrize("D,T,alpha", [(128, 4096, 0.01), (64, 2049, 0.3), (32, 700, 1.0), (32, 2500, 1.0), (128, 4097, 0.2)])
 def test_the_exact_select_over_the_data_passes_over_nans(D, T, alpha):
-    # sampled tokens all zero: lists overflow; NaNs of both signs, infinities, a problem of NaNs alone in its unsampled tokens
+    # sampled tokens all zero: lists overflow (700 tokens of 32 channels: the kernel of short sequences, which samples nothing); NaNs of
+    # both signs, infinities, a problem of NaNs alone in its unsampled tokens
     wl = synth.scaled(synth.CONFIGS["C2"], heads=3, head_dim=D, tokens=T)
     K, V = synth.make_kv(wl, 0)
     g = torch.Generator().manual_seed(D)
@@ -99,12 +100,13 @@ def test_the_exact_select_over_the_data_passes_over_nans(D, T, alpha):
     check(K, V, wl, alpha)
 
 
-@pytest.mark.parametrize("D,T", [(32, 1), (128, 33), (128, 256), (64, 512), (128, 257), (32, 2048), (64, 1024), (128, 513)])
+@pytest.mark.parametrize("D,T,heads", [(32, 1, 3), (128, 33, 3), (128, 256, 3), (64, 512, 3), (128, 257, 3), (32, 2048, 3), (64, 1024, 3), (128, 513, 3),
+                                       (32, 2049, 3), (64, 1025, 3), (32, 1024, 75), (32, 1025, 74), (32, 1025, 75), (128, 400, 75)])
 @pytest.mark.parametrize("alpha", [0.0, 0.01, 0.3, 1.0])
-def test_short_sequences(D, T, alpha):
-    # up to the keys that one CTA holds with 512 and with 1024 threads, and one token beyond; ranks beyond the number of pieces
-    # (0.3, 1.0); NaNs of both signs, infinities, both zeros, a tail of ties
-    wl = synth.scaled(synth.CONFIGS["C2"], heads=3, head_dim=D, tokens=T)
+def test_short_sequences(D, T, heads, alpha):
+    # up to the keys that one CTA holds with 8 and with 16 pieces to a thread (these only up to 74 (b,h)), and one token beyond; ranks
+    # beyond the number of pieces (0.3, 1.0); NaNs of both signs, infinities, both zeros, a tail of ties
+    wl = synth.scaled(synth.CONFIGS["C2"], heads=heads, head_dim=D, tokens=T)
     K, V = synth.make_kv(wl, 0)
     flat = V.view(-1)
     for i, x in enumerate((float("nan"), -float("nan"), float("inf"), -float("inf"), 0.0, -0.0)):

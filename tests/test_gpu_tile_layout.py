@@ -163,9 +163,9 @@ def test_query_rows_at_any_address():
     assert torch.equal(got, out)
 
 
-@pytest.mark.parametrize("D,window,tokens", [(128, 64, 4097), (64, 5, 4161), (32, 64, 4500)])
+@pytest.mark.parametrize("D,window,tokens", [(128, 64, 4097), (64, 5, 4161), (32, 64, 4500), (64, 64, 8257)])
 def test_long_windows_of_any_length_and_number_of_rows(D, window, tokens):
-    # above 4096 tokens the rows are made in two passes over the keys; 64 rows read a warp's keys once
+    # above 4096 tokens: one pass with the logits in tensor memory (64 rows), two tiles to a group of warps (5 rows), two passes (8257)
     wl = synth.scaled(synth.CONFIGS["C1"], batch=1, heads=2, head_dim=D, tokens=tokens, window=window, seed=D)
     K, _ = synth.make_kv(wl)
     Q = torch.randn((wl.bh, window, D), generator=torch.Generator().manual_seed(D)).to(torch.float16)

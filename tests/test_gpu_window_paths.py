@@ -141,3 +141,27 @@ def test_a_lost_window_is_reported_by_the_calls_that_take_it(D, W, how):
     assert torch.equal(k0, k1) and torch.equal(v0[there], v1[there])
     assert (v0[~there] == 2).all() and (v1[~there] == 8).all()
     assert how == "select" or (s0, s1) == (qaq.QAQ_OK, 4)
+
+
+def laid_out(X, how):
+    """The values of X [B,H,T,D] with other strides (elements; 16-byte aligned rows, as the calls ask for)."""
+    B, H, T, D = X.shape
+    big = {
+        "padded rows": lambda: torch.empty((B, H, T, D + 8), dtype=X.dtype, device=X.device)[..., :D],
+        "gap between heads": lambda: torch.empty((B, H, T * D + 24), dtype=X.dtype, device=X.device).as_strided((B, H, T, D), (H * (T * D + 24), T * D + 24, D, 1)),
+        "slice": lambda: torch.empty((B, H, T + 40, D), dtype=X.dtype, device=X.device)[:, :, 7:7 + T],
+        "some of many heads": lambda: torch.empty((B, T, H + 3, D), dtype=X.dtype, device=X.device)[:, :, 2:2 + H].transpose(1, 2),
+        "batch inside": lambda: torch.empty((H, T, B, D), dtype=X.dtype, device=X.device).permute(2, 0, 1, 3),
+    }[how]()
+    big.copy_(X)
+    return big
+
+
+@pytest.mark.parametrize("D", [32, 64, 128])
+@pytest.mark.parametrize("how", ["padded rows", "gap between heads", "slice", "some of many heads", "batch inside"])
+@pytest.mark.parametrize("T,n", [(300, 9), (3000, 16), (4100, 64), (9000, 64)])
+def test_keys_of_any_strides(D, how, T, n):
+    # few tiles with one and with several tiles to a CTA, one pass, two passes: the copies of tiles take the caller's strides
+    K = laid_out(keys(2, 2, T, D, token_major=False, seed=T), how)
+    Q = torch.randn((4, n, D), generator=torch.Generator().manual_seed(n)).half()
+    rows_match(K, Q, 2, range(4))
