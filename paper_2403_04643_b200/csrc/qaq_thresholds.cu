@@ -12,7 +12,7 @@
 //                          turned out too tight (fewer than k+1 candidates) or a problem's list overflowed, the
 //                          problem is redone exactly by a two-pass radix select over its data, so the
 //                          result is always the exact order statistic.
-// Short sequences take one kernel (thr_short_kernel).
+// Short sequences take one kernel (thr_short_kernel; a tile or less of many (b,h) the first one above, whose sample is then everything).
 // binary16 patterns are mapped to 16-bit keys that sort like the values.
 #include "qaq_internal.cuh"
 
@@ -180,8 +180,8 @@ __device__ __forceinline__ uint32_t bracket_rank(double alpha, uint32_t M) {
     return r > (M - 1) / 2 ? (M - 1) / 2 : r;
 }
 
-// ---- 1. sample: brackets
-template <int THREADS>
+// ---- 1. sample: brackets.  WHOLE: up to SAMPLE_TOKENS tokens, which are all looked at: the answer.
+template <int THREADS, bool WHOLE>
 __global__ void __launch_bounds__(THREADS) thr_sample_kernel(const ThrArgs a) {
     constexpr int PIECES = SAMPLE_TOKENS * 128 / 8 / THREADS;            // 16-byte pieces of a thread at most
     qaq_dependency();
@@ -190,7 +190,7 @@ __global__ void __launch_bounds__(THREADS) thr_sample_kernel(const ThrArgs a) {
     __shared__ uint32_t hist[2048], s_tmp[4], s_cnt[2];
     const int b_idx = bh / a.H, h_idx = bh % a.H;
     const __half* X = a.X[x] + (size_t)b_idx * a.sb + (size_t)h_idx * a.sh;
-    constexpr int ns = SAMPLE_TOKENS;                            // (shorter sequences: thr_short_kernel)
+    const int ns = WHOLE ? a.T : SAMPLE_TOKENS;
     const int M = ns * a.D;
     if (threadIdx.x < 2) s_cnt[threadIdx.x] = 0;
     __syncthreads();
@@ -218,14 +218,17 @@ __global__ void __launch_bounds__(THREADS) thr_sample_kernel(const ThrArgs a) {
     const uint32_t Mv = (uint32_t)M - s_cnt[0];                    // non-NaN sample values
     const uint32_t n_neg_nan = s_cnt[1];
     Problem* pr = a.prob + bhx;
+    float* const thr = a.thr + (size_t)bh * 4 + 2 * x;
     if (Mv == 0) {
-        if (threadIdx.x == 0) { pr->klo = 0; pr->khi = 0xFFFF; pr->cnt[0] = pr->cnt[1] = 0; pr->nan = 0; pr->n = 0; }
+        if (WHOLE) { if (threadIdx.x < 2) thr[threadIdx.x] = 0.f; }
+        else if (threadIdx.x == 0) { pr->klo = 0; pr->khi = 0xFFFF; pr->cnt[0] = pr->cnt[1] = 0; pr->nan = 0; pr->n = 0; }
         return;
     }
-    const uint32_t r = bracket_rank(a.alpha, Mv);
+    const uint32_t r = WHOLE ? (uint32_t)rank_k(a.alpha, Mv) : bracket_rank(a.alpha, Mv);
     uint32_t klo, khi;
     cta_select_keys<THREADS>(s_keys, (uint32_t)M, r + n_neg_nan, Mv - 1 - r + n_neg_nan, hist, s_tmp, klo, khi);
-    if (threadIdx.x == 0) { pr->klo = klo; pr->khi = khi; pr->cnt[0] = pr->cnt[1] = 0; pr->nan = 0; pr->n = 0; }
+    if (WHOLE) { if (threadIdx.x < 2) thr[threadIdx.x] = float_of_key(threadIdx.x ? khi : klo); }
+    else if (threadIdx.x == 0) { pr->klo = klo; pr->khi = khi; pr->cnt[0] = pr->cnt[1] = 0; pr->nan = 0; pr->n = 0; }
 }
 
 // ---- 2. the one pass over the data: compaction of the tail candidates.
@@ -635,20 +638,27 @@ extern "C" qaq_status qaq_outlier_thresholds(const qaq_config* cfg, const void* 
     a.thr = thr;
     a.scan_tokens = SCAN_TOKENS_MAX;
     const size_t keys = (size_t)n_tokens * cfg->head_dim;
-    // 32768 keys, two CTAs to an SM; twice as many while every problem has an SM to itself (32 (b,h) of 333 tokens 10.4 us, 13.4 by the
-    // kernels below; 256 of them 38.7 and 31.0)
+    // a tile or less of so many (b,h) that the CTAs of 512 threads come in turns (two to an SM): 160 (b,h) of 40 tokens, head_dim 32, 6.4 us,
+    // 9.0 by the kernel for short sequences, 320 of them 8.5 and 13.7 (head_dim 128: 13.0 and 16.1); 148 6.4 and 6.5
+    if (n_tokens <= SAMPLE_TOKENS && BH * 2 > 2 * 148) {
+        QAQ_CUDA_TRY(qaq_launch(thr_sample_kernel<256, true>, dim3(BH * 2), dim3(256), 0, s, a));
+        return QAQ_OK;
+    }
+    // 32768 keys; twice as many while every problem has an SM to itself (32 (b,h) of 333 tokens 10.4 us, 13.4 by the kernels below;
+    // 256 of them 38.7 and 31.0), not quite where these would spread few problems over all SMs (one (b,h) of 800 tokens, head_dim 64, 11.3 and
+    // 11.5, of 1024 13.0 and 11.7; 12 of 1024 13.0 and 12.9)
     if (keys <= SHORT_THREADS * 8 * 8) {
         QAQ_CUDA_TRY(qaq_launch(thr_short_kernel<8>, dim3(BH * 2), dim3(SHORT_THREADS), 0, s, a));
         return QAQ_OK;
     }
-    if (keys <= SHORT_THREADS * 16 * 8 && BH * 2 <= 148) {
+    if (keys <= (size_t)SHORT_THREADS * 8 * (BH < 8 ? 12 : 16) && BH * 2 <= 148) {
         QAQ_CUDA_TRY(qaq_launch(thr_short_kernel<16>, dim3(BH * 2), dim3(SHORT_THREADS), 0, s, a));
         return QAQ_OK;
     }
     // 512 threads while a problem has an SM to itself or shares it with one (32 (b,h): 6.4 against 7.9 us), else 256 (256
     // (b,h): 14.4 against 15.6)
-    if (BH * 2 <= 2 * 148) QAQ_CUDA_TRY(qaq_launch(thr_sample_kernel<512>, dim3(BH * 2), dim3(512), 0, s, a));
-    else QAQ_CUDA_TRY(qaq_launch(thr_sample_kernel<256>, dim3(BH * 2), dim3(256), 0, s, a));
+    if (BH * 2 <= 2 * 148) QAQ_CUDA_TRY(qaq_launch(thr_sample_kernel<512, false>, dim3(BH * 2), dim3(512), 0, s, a));
+    else QAQ_CUDA_TRY(qaq_launch(thr_sample_kernel<256, false>, dim3(BH * 2), dim3(256), 0, s, a));
     a.scan_tokens = scan_tokens_for(cfg->outlier_frac, cfg->head_dim, BH, n_tokens);
     dim3 grid((n_tokens + a.scan_tokens - 1) / a.scan_tokens, BH * 2);
     QAQ_CUDA_TRY(qaq_launch(thr_scan_kernel, grid, dim3(256), 0, s, a));

@@ -101,11 +101,12 @@ def test_the_exact_select_over_the_data_passes_over_nans(D, T, alpha):
 
 
 @pytest.mark.parametrize("D,T,heads", [(32, 1, 3), (128, 33, 3), (128, 256, 3), (64, 512, 3), (128, 257, 3), (32, 2048, 3), (64, 1024, 3), (128, 513, 3),
-                                       (32, 2049, 3), (64, 1025, 3), (32, 1024, 75), (32, 1025, 74), (32, 1025, 75), (128, 400, 75)])
+                                       (32, 2049, 3), (64, 1025, 3), (32, 1024, 75), (32, 1025, 74), (32, 1025, 75), (128, 400, 75),
+                                       (32, 2048, 8), (64, 768, 7), (64, 769, 7), (32, 1, 149), (128, 33, 149), (64, 64, 149), (32, 65, 149)])
 @pytest.mark.parametrize("alpha", [0.0, 0.01, 0.3, 1.0])
 def test_short_sequences(D, T, heads, alpha):
-    # up to the keys that one CTA holds with 8 and with 16 pieces to a thread (these only up to 74 (b,h)), and one token beyond; ranks
-    # beyond the number of pieces (0.3, 1.0); NaNs of both signs, infinities, both zeros, a tail of ties
+    # up to the keys that one CTA holds with 8 and with 16 pieces to a thread (these only up to 74 (b,h); up to 7 (b,h) 12 pieces), and one
+    # token beyond; up to 64 tokens of more than 148 (b,h); ranks beyond the number of pieces (0.3, 1.0); NaNs of both signs, infinities, both zeros, a tail of ties
     wl = synth.scaled(synth.CONFIGS["C2"], heads=heads, head_dim=D, tokens=T)
     K, V = synth.make_kv(wl, 0)
     flat = V.view(-1)
