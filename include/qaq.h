@@ -46,10 +46,10 @@ typedef struct {
     long max_outliers_per_bh;   /* per tensor; <= 0: derived from outlier_frac with slack */
 } qaq_config;
 
-/* What stands in place of every score of a token whose window could not be computed, as a binary32 pattern (a NaN that arithmetic
- * does not give): a kernel of qaq_prefill_window waited in vain for its own copies or for its peers.  Where the first row of a token's
- * window holds it and no other row a number, its value takes bits_max, and the device status of the cache becomes QAQ_ERR_CUDA. */
-#define QAQ_SCORE_LOST 0x7FC0105Eu
+/* What stands in place of every score of a token whose window could not be computed, as a binary32 pattern (3.4e38: a score is at most
+ * 1): a kernel of qaq_prefill_window waited in vain for its own copies or for its peers.  A value whose largest score it is takes
+ * bits_max, as the rule has it, and the device status of the cache becomes QAQ_ERR_CUDA. */
+#define QAQ_SCORE_LOST 0x7F7E105Eu
 
 /* Scalars of the bit-width rules (Section 4.1), see qaq_policy_from_hyper. */
 typedef struct {

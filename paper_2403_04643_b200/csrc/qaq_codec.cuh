@@ -314,10 +314,6 @@ __device__ __forceinline__ float window_max_one_loop(const float* r, int W, long
     }
     return m;
 }
-// The window of this token was lost (QAQ_SCORE_LOST): no row of the nv > 0 held a number, and the first one says why.
-__device__ __forceinline__ bool window_lost(const float* r, int nv, float max) {
-    return nv > 0 && max == __int_as_float(0xff800000) && __float_as_uint(*r) == QAQ_SCORE_LOST;
-}
 // The nibble words of one part (w bits, 1..4) of a lane's 32 channels of one token.  Keys: the unit at `at`; values: byte i of
 // units 4p .. 4p+3, which lie m units apart from `at` on.
 template <int W, bool IS_V>

@@ -168,12 +168,12 @@ __device__ __forceinline__ uint32_t prefix(uint32_t x, int lane, uint32_t& sum) 
 constexpr uint32_t STORED = 1u << 30;   // of a slot's last word: the token is taken from the stored tile
 
 // One tile of one tensor, by two warps: half of its tokens each until the widths are known, half of the slots each from there.
-// OPEN (the number of warps; 0: whole tiles, two warps): a tile that is begun, continued or closed, the only one of its (b,h) in the
+// By NW warps.  OPEN: a tile that is begun, continued or closed, the only one of its (b,h) in the
 // launch: its tokens up to s_lo are cached already (and come from the tile as it is stored), those from s_lo to s_hi are new.
-template <int D, bool IS_V, int OPEN>
+template <int D, bool IS_V, bool OPEN, int NW>
 __device__ __forceinline__ void quantize_tile(const QuantArgs& a, TileScratch<D>& sm, uint8_t* stored_tile, uint32_t* list, const uint32_t cap) {
     constexpr int P = D / 32, TPI = 32 / P, IT = QAQ_TILE / 2 / TPI;  // lanes per token, tokens of a warp at a time, rounds
-    constexpr int PR = D / 8, NW = OPEN ? OPEN : 2;             // 16-byte pieces of a row; warps
+    constexpr int PR = D / 8;                                         // 16-byte pieces of a row
     const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31, g = lane / P, p = lane % P;
     const bool counted = OPEN && a.d_count;
     const int t_old = counted ? *a.d_count : a.t_old;
@@ -220,7 +220,6 @@ __device__ __forceinline__ void quantize_tile(const QuantArgs& a, TileScratch<D>
         nv = min(nv, a.W);
         const float* scores = a.ring + (size_t)bh * a.W * a.n_new + col;
         shat = OPEN ? qaqc::window_max_one_loop<32>(scores, a.W, a.n_new, nv) : qaqc::window_max<32>(scores, a.W, a.n_new, nv);
-        if (qaqc::window_lost(scores, nv, shat)) { nv = 0; atomicMax(a.status, (int)QAQ_ERR_CUDA); }
     }
     if (OPEN) {                        // the tile as it is stored follows on its own: it is needed later
         asm volatile("cp.async.commit_group;" ::: "memory");
@@ -292,6 +291,7 @@ __device__ __forceinline__ void quantize_tile(const QuantArgs& a, TileScratch<D>
         if (given) b = b < 1 ? 1 : (b > 8 ? 8 : b);
         else if (!IS_V) b = ladder(r, a.cK, a.bmin, a.bmax);
         else b = nv == 0 ? a.bmax : ladder(__fmul_rn(r, shat), a.cV, a.bmin, a.bmax);
+        if (IS_V && __float_as_uint(shat) == QAQ_SCORE_LOST) atomicMax(a.status, (int)QAQ_ERR_CUDA);
         if (OPEN && !fresh) b = old ? min((int)(bs_old & 0xFFu), 8) : 0;
     }
     uint32_t alike = 0;
@@ -475,39 +475,39 @@ __device__ __forceinline__ void quantize_tile(const QuantArgs& a, TileScratch<D>
 }
 
 // dynamic shared memory: the scratch, the tile as it is stored (OPEN), the warps' lists of outliers
-template <int D, int OPEN>
-__global__ void __launch_bounds__(OPEN ? 32 * OPEN : 64, OPEN == 0 ? 12 : OPEN == 4 ? 4 : 2) quant_tiles_kernel(const QuantArgs a, uint32_t cap) {
+template <int D, bool OPEN, int NW>
+__global__ void __launch_bounds__(32 * NW, OPEN ? 16 / NW : 12) quant_tiles_kernel(const QuantArgs a, uint32_t cap) {
     extern __shared__ __align__(64) unsigned char tiles_smem[];
     TileScratch<D>& sm = *reinterpret_cast<TileScratch<D>*>(tiles_smem);
     uint8_t* stored_tile = tiles_smem + sizeof(TileScratch<D>);
     uint32_t* list = reinterpret_cast<uint32_t*>(stored_tile + (OPEN ? qaqc::tile_bytes_max(D) + 16 : 0));
     qaq_dependency();
-    if (blockIdx.z == 0) quantize_tile<D, false, OPEN>(a, sm, stored_tile, list, cap);
-    else quantize_tile<D, true, OPEN>(a, sm, stored_tile, list, cap);
+    if (blockIdx.z == 0) quantize_tile<D, false, OPEN, NW>(a, sm, stored_tile, list, cap);
+    else quantize_tile<D, true, OPEN, NW>(a, sm, stored_tile, list, cap);
 }
 
 // tiles.x tiles of every (b,h), all whole, or one that is not (or may not be)
-template <int D, int OPEN>
+template <int D, bool OPEN, int NW>
 qaq_status launch_tiles(int tiles, int BH, const QuantArgs& a, double alpha, cudaStream_t s) {
     // the lists hold a tenth more than the share of outliers asked for gives a tile, and some (twelve CTAs per SM at 1 %)
     const uint32_t want = (uint32_t)(alpha * (QAQ_TILE * D) * 1.1) + 60, cap = (want < 2048 ? want : 2048) / 2;
     const size_t smem = sizeof(TileScratch<D>) + (OPEN ? qaqc::tile_bytes_max(D) + 16 : 0) + 2 * cap * sizeof(uint32_t);
     static_assert(sizeof(TileScratch<D>) + qaqc::tile_bytes_max(D) + 16 + 2048 * sizeof(uint32_t) <= 48 * 1024, "shared memory that needs no attribute");
-    QAQ_CUDA_TRY(qaq_launch(quant_tiles_kernel<D, OPEN>, dim3((unsigned)tiles, (unsigned)BH, 2), dim3(OPEN ? 32 * OPEN : 64), smem, s, a, cap));
+    QAQ_CUDA_TRY(qaq_launch(quant_tiles_kernel<D, OPEN, NW>, dim3((unsigned)tiles, (unsigned)BH, 2), dim3(32 * NW), smem, s, a, cap));
     return QAQ_OK;
 }
-template <int OPEN>
+template <bool OPEN, int NW>
 qaq_status launch(int D, int tiles, int BH, const QuantArgs& a, double alpha, cudaStream_t s) {
     switch (D) {
-        case 32: return launch_tiles<32, OPEN>(tiles, BH, a, alpha, s);
-        case 64: return launch_tiles<64, OPEN>(tiles, BH, a, alpha, s);
-        case 128: return launch_tiles<128, OPEN>(tiles, BH, a, alpha, s);
+        case 32: return launch_tiles<32, OPEN, NW>(tiles, BH, a, alpha, s);
+        case 64: return launch_tiles<64, OPEN, NW>(tiles, BH, a, alpha, s);
+        case 128: return launch_tiles<128, OPEN, NW>(tiles, BH, a, alpha, s);
     }
     return QAQ_ERR_UNSUPPORTED_SHAPE;
 }
 // eight warps while all CTAs run at once, else four (figures at the top)
 qaq_status launch_open(int D, int BH, const QuantArgs& a, double alpha, cudaStream_t s) {
-    return 2 * BH <= 2 * 148 ? launch<8>(D, 1, BH, a, alpha, s) : launch<4>(D, 1, BH, a, alpha, s);
+    return 2 * BH <= 2 * 148 ? launch<true, 8>(D, 1, BH, a, alpha, s) : launch<true, 4>(D, 1, BH, a, alpha, s);
 }
 
 // Widths alone: one CTA = 64 tokens of one (b,h); P = D/32 lanes own a token, each lane 32 consecutive channels (64 bytes) of
@@ -539,7 +539,6 @@ __global__ void __launch_bounds__(2 * D) select_kernel(const QuantArgs a) {
     }
 #pragma unroll
     for (int o = 1; o < P; o <<= 1) shat = fmaxf(shat, __shfl_xor_sync(0xFFFFFFFFu, shat, o));
-    if (qaqc::window_lost(a.ring + (size_t)bh * a.W * a.n_new + tn, nv, shat)) nv = 0;
 #pragma unroll
     for (int x = 0; x < 2; ++x) {
         const __half2 lo2 = __half2half2(__float2half_ru(thr[2 * x])), hi2 = __half2half2(__float2half_rd(thr[2 * x + 1]));
@@ -608,7 +607,7 @@ qaq_status qaq_launch_append(qaq_cache* c, const void* K, const void* V, long sb
     const int full_end = t1 / QAQ_TILE * QAQ_TILE;
     if (cur < full_end) {       // body: whole tiles
         a.tok_lo = cur - t0; a.tok_hi = full_end - t0; a.first_tile = cur / QAQ_TILE;
-        if ((stt = launch<0>(D, (full_end - cur) / QAQ_TILE, BH, a, c->cfg.outlier_frac, s)) != QAQ_OK) return stt;
+        if ((stt = launch<false, 2>(D, (full_end - cur) / QAQ_TILE, BH, a, c->cfg.outlier_frac, s)) != QAQ_OK) return stt;
         cur = full_end;
     }
     if (cur < t1) {             // tail: a new, partly filled tile

@@ -127,10 +127,9 @@ __device__ __forceinline__ void requantize_tile(const RequantArgs& a, RequantScr
             B = ladder(rng, a.cK, a.bmin, a.bmax);
         } else {
             const long col = (long)min(tok, a.T - 1);           // whole warps read the window; columns beyond the last are not used
-            int nv = min((int)a.nvalid[(size_t)bh * a.ncols + col], a.W);
-            const float* scores = a.ring + (size_t)bh * a.W * a.ncols + col;
-            const float sh = qaqc::window_max<16, true>(scores, a.W, a.ncols, nv);
-            if (qaqc::window_lost(scores, nv, sh)) { nv = 0; atomicMax(a.status, (int)QAQ_ERR_CUDA); }
+            const int nv = min((int)a.nvalid[(size_t)bh * a.ncols + col], a.W);
+            const float sh = qaqc::window_max<16, true>(a.ring + (size_t)bh * a.W * a.ncols + col, a.W, a.ncols, nv);
+            if (__float_as_uint(sh) == QAQ_SCORE_LOST) atomicMax(a.status, (int)QAQ_ERR_CUDA);
             B = nv == 0 ? a.bmax : ladder(__fmul_rn(rng, sh), a.cV, a.bmin, a.bmax);
         }
         if (valid) Bn = (UP || B < Bo) ? B : Bo;

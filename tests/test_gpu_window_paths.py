@@ -96,7 +96,7 @@ def test_logits_of_minus_infinity(D, heads, T, n):
     assert torch.allclose(ring.sum(2), torch.ones(heads, n, device="cuda"), atol=1e-4)
 
 
-LOST = torch.tensor([0x7FC0105E], dtype=torch.int32).view(torch.float32)      # QAQ_SCORE_LOST
+LOST = torch.tensor([0x7F7E105E], dtype=torch.int32).view(torch.float32)      # QAQ_SCORE_LOST
 
 
 @pytest.mark.parametrize("D", [32, 128])
@@ -137,7 +137,7 @@ def test_a_lost_window_is_reported_by_the_calls_that_take_it(D, W, how):
 
     k0, v0, s0 = widths(nan)
     k1, v1, s1 = widths(lost)
-    there = (lost == lost).all(dim=2).view(wl.bh, 150)
+    there = (lost < 2).all(dim=2).view(wl.bh, 150)
     assert torch.equal(k0, k1) and torch.equal(v0[there], v1[there])
     assert (v0[~there] == 2).all() and (v1[~there] == 8).all()
     assert how == "select" or (s0, s1) == (qaq.QAQ_OK, 4)
