@@ -143,10 +143,11 @@ __device__ __forceinline__ float pow2(float x) {
     asm("ex2.approx.ftz.f32 %0, %1;" : "=f"(r) : "f"(x));
     return r;
 }
-// (reference, sum of 2^(logit - reference))
+// (reference, sum of 2^(logit - reference)); a sum of 0 says that there was nothing (a reference of -inf does not: it may be logits that
+// are no numbers, and a sum that is none)
 __device__ __forceinline__ void fold_stats(float2& to, const float2& p) {
-    const float NEG = __int_as_float(0xff800000), m = fmaxf(to.x, p.x);
-    to.y = (to.x == NEG ? 0.f : to.y * pow2(to.x - m)) + (p.x == NEG ? 0.f : p.y * pow2(p.x - m));
+    const float m = fmaxf(to.x, p.x);
+    to.y = (to.y == 0.f ? 0.f : to.y * pow2(to.x - m)) + (p.y == 0.f ? 0.f : p.y * pow2(p.x - m));
     to.x = m;
 }
 // Sums of eight columns over the lanes of the warp: lane 4k (and the three behind it) gets that of column k.
@@ -484,9 +485,9 @@ __global__ void __launch_bounds__(PW_THREADS, 1) window_kernel(const __grid_cons
 }
 
 // ---- few tiles in all: a thread keeps the logits of its token (up to 16 rows: or of two) in registers, a CTA is one group of four warps to
-// four, a tile (or two) each, and the CTAs of a (b,h) form a cluster where it has more than one.  No warp waits for another's work but at barriers, several CTAs share an
-// SM, keys come by plain asynchronous copies.  Tensor memory is given back before the CTAs of a cluster wait for each other, so that
-// nobody waits for it who is waited for.  32 (b,h) of 333 tokens, 32 rows: 5.6 us, the kernel above 7.8 us; of 2048 tokens 10.7 and 12.8;
+// four, a tile (or two) each, and the CTAs of a (b,h) form a cluster where it has more than one.  No warp waits for another's work but at
+// barriers, several CTAs share an SM, keys come by plain asynchronous copies.  Tensor memory is given back before the CTAs of a cluster
+// wait for each other, so that nobody waits for it who is waited for.  32 (b,h) of 333 tokens, 32 rows: 5.6 us, the kernel above 7.8 us; of 2048 tokens 10.7 and 12.8;
 // of 4096 tokens, head_dim 32, 5 rows 7.2 us with two tiles to a group, 10.2 with one, 11.7.
 constexpr int PS_GROUPS = 4;           // groups of four warps of a CTA at most
 template <int ROW_BYTES, int ROWS>     // rows of a [.][D] operand on their way to shared memory, by four warps; what lies beyond `rows` is not touched
@@ -499,8 +500,8 @@ __device__ __forceinline__ void fetch_rows(uint32_t dst, const __half* src, long
     for (int r = row; r < ROWS; r += step, src += step * stride, dst += step * ROW_BYTES)
         if (r < rows) asm volatile("cp.async.cg.shared.global [%0], [%1], 16;" ::"r"(dst), "l"(src) : "memory");
 }
-// TP: tokens of a thread, tiles of a group of four warps.
 constexpr int short_ctas(int NC) { return NC <= 32 ? 2 : 1; }          // of PS_GROUPS groups to an SM, for their registers
+// TP: tokens of a thread, tiles of a group of four warps.
 template <int D, int NC, int TP>
 __global__ void __launch_bounds__(128 * PS_GROUPS, short_ctas(NC)) window_short_kernel(const PrefillArgs a, const __half* K, long sb, long sh, long st) {
     using W = Window<D, NC, STATS>;
@@ -635,6 +636,7 @@ __global__ void __launch_bounds__(128 * PS_GROUPS, short_ctas(NC)) window_short_
     for (int i = 0; i < TP; ++i)
         if (t + i * PW_TILE < a.T) a.nvalid[(size_t)bh * a.T + t + i * PW_TILE] = (uint8_t)min(a.n, a.T - t - i * PW_TILE);
 }
+
 // Descriptions of K ([batch][head][token][channel] with the caller's strides) and of the queries for the copies of tiles.
 typedef CUresult (*EncodeTiled)(CUtensorMap*, CUtensorMapDataType, cuuint32_t, void*, const cuuint64_t*, const cuuint64_t*, const cuuint32_t*, const cuuint32_t*,
                                 CUtensorMapInterleave, CUtensorMapSwizzle, CUtensorMapL2promotion, CUtensorMapFloatOOBfill);

@@ -67,19 +67,23 @@ def test_a_reference_far_below_a_later_logit(T, n):
 
 
 @pytest.mark.parametrize("T", [100, 1500, 9000])
-def test_heads_that_share_keys_and_keys_that_are_not_numbers(T):
-    # one set of keys under several heads by a stride of zero; a NaN stays in its token and row, the other tokens of the row become 0
+@pytest.mark.parametrize("n", [8, 40])
+def test_heads_that_share_keys_and_keys_that_are_not_numbers(T, n):
+    # one set of keys under several heads by a stride of zero; NaNs stay in their tokens and rows, the other tokens of the rows become 0,
+    # whether one token is not a number or most of them, to the edge of a warp's 32
     K = keys(1, 1, T, 128, token_major=False, seed=T)
-    Q = torch.randn((3, 8, 128), generator=torch.Generator().manual_seed(1)).half()
+    Q = torch.randn((3, n, 128), generator=torch.Generator().manual_seed(1)).half()
     shared = rows_match(K.expand(1, 3, T, 128), Q, 3, range(3))
-    bad = K.clone()
-    bad[0, 0, T // 2, 5] = math.nan
-    cfg = qaq.make_config(1, 3, 128, T, 2, 8, 8, 0.01)
-    ring, _ = qaq.qaq_prefill_window(cfg, Q.cuda(), bad.expand(1, 3, T, 128), 1 / math.sqrt(128))
-    ring = ring.view(3, 8, T)
-    assert torch.isnan(ring[:, :, T // 2]).all()
-    ring[:, :, T // 2] = 0
-    assert (ring == 0).all() and (shared.sum() > 0)
+    assert shared.sum() > 0
+    cfg = qaq.make_config(1, 3, 128, T, 2, 8, n, 0.01)
+    for none in (slice(T // 2, T // 2 + 1), slice(0, T - n - 10), slice(0, (T - n - 1) // 32 * 32)):
+        bad = K.clone()
+        bad[0, 0, none, 5] = math.nan
+        ring, _ = qaq.qaq_prefill_window(cfg, Q.cuda(), bad.expand(1, 3, T, 128), 1 / math.sqrt(128))
+        ring = ring.view(3, n, T)
+        assert torch.isnan(ring[:, :, none]).all()
+        ring[:, :, none] = 0
+        assert (ring == 0).all()
 
 
 @pytest.mark.parametrize("D", [32, 64, 128])
