@@ -39,7 +39,7 @@ import hashlib
 COUNTERS_JSON = os.path.join(ROOT, "profiles", "counters_C3.json")
 CSRC = os.path.join(ROOT, "paper_2403_04643_b200", "csrc")
 ISSUE_SLOTS_PER_CLOCK = 148 * 4
-KERNEL_KEYS = {"quant": "quant_tiles_kernel<128, 0>", "decode": "decode_kernel<128, 1, 0, 0>", "thr_scan": "thr_scan_kernel"}
+KERNEL_KEYS = {"quant": "quant_tiles_kernel<128, 0, 2>", "decode": "decode_kernel<128, 1, 0, 0>", "thr_scan": "thr_scan_kernel"}
 
 
 def csrc_hash():
